@@ -57,6 +57,7 @@ struct dc_layer_rt {
                                     // channels per block (0 = default)
     void* weight_halo;              // conv, bf16: weights packed for the patch-reuse and column-slab kernels
     int halo_bn;                    // channels per block that packing is grouped by
+    float* weight_simt;             // conv on the register-blocked CUDA-core kernel: its packed weights (dc_conv_simt.cu)
     void* in_padded;                // conv, bf16, cin <= 8: input with channels padded to 8
     void* in_s2d;                   // conv, bf16, strided over few channels: the space-to-depth copy of the input the rewritten layer reads (dc_conv_s2d.cu)
     int s2d_s, s2d_py, s2d_px, s2d_cin, s2d_hi, s2d_wi;   // ... its block size (0: layer as declared), leading zero rows / columns, and the input as declared
@@ -160,6 +161,25 @@ struct dc_once_per_device {
     }
 };
 
+// Programmatic dependent launch: a kernel launched with dc_launch_pdl may become resident while the previous kernel of
+// the stream is still running.  dc_pdl_wait() returns once that kernel has completed and its writes are visible: nothing
+// another kernel produces is read, and nothing at all is written, before it, and every such kernel calls it.
+// dc_pdl_release() lets the next kernel do the same.
+__device__ __forceinline__ void dc_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dc_pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+static inline cudaError_t dc_launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // ---- kernels' host-side launchers (each returns DC_OK or DC_ERR_CUDA) ----
 int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst);
 int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key);   // both in key-frame layout
@@ -169,6 +189,12 @@ int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, co
                             const void* prev_out, void* out);
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                    const int32_t* tile_count, const uint32_t* masks, int max_tiles);
+// stride-1 layers and single output pixels on CUDA cores (dc_conv_simt.cu)
+bool dc_dense_ok(const dc_layer_rt& L);
+int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
+                        const int32_t* tile_count, const uint32_t* masks, int max_tiles);
+int dc_launch_dense(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
+int dc_pack_weights_simt(dc_cache* c, int layer);
 int dc_launch_input_map(dc_cache* c, const uint8_t* frame, size_t pitch);
 int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch);   // frame: 16-byte aligned rows
 int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);

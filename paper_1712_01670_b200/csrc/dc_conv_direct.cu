@@ -1,8 +1,9 @@
 // Partial convolution on CUDA cores (Section 5, "Reuse", third step: convolve only the
-// pixels that were not filled from the cache).
+// pixels that were not filled from the cache): the general kernel, and which kernel a layer runs on.
 //
-// Used for float32 networks, whose 1e-4 accuracy bound rules out tensor-core input formats,
-// for layer shapes the tensor-core kernel does not take, and for grouped convolutions.  One CTA of 128 threads owns one
+// float32 networks, whose 1e-4 accuracy bound rules out tensor-core input formats, and layer shapes that the
+// tensor-core kernels do not take run on dc_conv_simt.cu where they can, and here otherwise (strides, kernel sizes
+// other than 1, 3 and 5).  One CTA of 128 threads owns one
 // dirty 16x8 output tile and a group of 32 output channels; thread t owns pixel t and keeps 32
 // float accumulators.  Weights for one kernel row and 8 input channels are staged in shared
 // memory as floats [kx][ci][co] and read as broadcast float4; inputs come straight from the
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(DC_TILE_PX) k_conv_direct(ConvArgs a)
     }
 }
 
+
 template <typename T>
 __global__ void k_convert_weights(const float* src, size_t n, T* dst)
 {
@@ -112,6 +114,7 @@ __global__ void k_convert_weights(const float* src, size_t n, T* dst)
 }
 
 }  // namespace
+
 
 int dc_conv_bf16_supported(const dc_cache* c, int layer);
 int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
@@ -129,6 +132,8 @@ int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int3
     }
     if (c->cfg.dtype == DC_BF16 && dc_conv_bf16_supported(c, layer))
         return dc_launch_conv_bf16(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
+    if (dc_dense_ok(L)) return dc_launch_dense(c, layer, in, out, masks);
+    if (L.weight_simt) return dc_launch_conv_simt(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
     ConvArgs a;
     a.in = in; a.w = L.weight; a.bias = L.bias; a.out = out;
     a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;
@@ -170,7 +175,8 @@ int dc_pack_weights(dc_cache* c, int layer, const float* w_dev, const float* b_d
             const int rc = dc_s2d_rewrite(c, layer);
             if (rc != DC_OK) return rc;
         }
-        return dc_pack_weights_bf16(c, layer);
+        const int rc = dc_pack_weights_bf16(c, layer);
+        if (rc != DC_OK || dc_conv_bf16_supported(c, layer)) return rc;
     }
-    return DC_OK;
+    return dc_pack_weights_simt(c, layer);
 }

@@ -799,3 +799,65 @@ def test_lookahead_gives_identical_results():
         assert dc.status() == B.DC_OK
     finally:
         dc.close()
+
+
+@pytest.mark.parametrize("dtype,hi,wi,cin,cout,k,S,groups", [
+    (B.DC_FP32, 130, 200, 4, 64, 3, 3, 1),       # 8 x 8 sums per thread, 64-channel blocks, one short chunk
+    (B.DC_FP32, 140, 210, 7, 32, 3, 5, 1),       # 8 x 8 sums, 32-channel blocks, channels not a multiple of four
+    (B.DC_FP32, 90, 140, 24, 128, 1, 6, 1),      # 1 x 1, a last chunk that is half full
+    (B.DC_FP32, 19, 21, 10, 20, 5, 2, 1),         # 8 x 4 sums, a last block that is not full, 5 x 5 taps
+    (B.DC_FP32, 17, 9, 12, 24, 3, 2, 2),         # two channel groups
+    (B.DC_BF16, 33, 18, 24, 16, 3, 3, 1),        # bfloat16 with channel counts the tensor-core kernels do not take
+    (B.DC_BF16, 16, 8, 24, 40, 1, 2, 1),         # exactly one tile per stream
+    (B.DC_FP32, 7, 9, 7, 12, 0, 5, 1),           # one output pixel (k = 0: the kernel covers the map), odd reduction
+    (B.DC_BF16, 8, 10, 64, 48, 0, 9, 1),
+])
+def test_conv_on_cuda_cores(dtype, hi, wi, cin, cout, k, S, groups):
+    """The register-blocked kernel and the one for single output pixels: full and partial convolution against the
+    oracle at partial tiles, partial channel blocks and chunks, groups, every shape of a thread's sums."""
+    g = rng(hi * 5 + wi + cout)
+    bf16 = dtype == B.DC_BF16
+    quant = orc.QUANT_BF16 if bf16 else orc.QUANT_NONE
+    nb = nets.NetBuilder(hi, wi)
+    x0 = nb.conv(-1, 4 if cin % 4 else cin, 1, 1, 0)
+    while nb.shape(x0)[2] < cin:                                    # an odd channel count: the frame's three channels joined on
+        x0 = nb.concat(x0, -1)
+    if k:
+        nb.conv(x0, cout, k, 1, k // 2, 1, groups=groups)
+    else:
+        nb.fc(x0, cout, relu=1)
+    L = dict(nb.layers[-1], kind=0, sh=1, sw=1)
+    li = len(nb.layers) - 1
+    wts = g.normal(0, np.sqrt(2.0 / (L["kh"] * L["kw"] * cin / groups)), size=(cout, L["kh"], L["kw"], cin // groups)).astype(np.float32)
+    bias = g.normal(0, 0.1, size=cout).astype(np.float32)
+    ws = [np.zeros((l["cout"], 1, 1, 3), np.float32) if l["kind"] == 0 else None for l in nb.layers[:-1]] + [wts]
+    bs = [np.zeros(l["cout"], np.float32) if l["kind"] == 0 else None for l in nb.layers[:-1]] + [bias]
+    q = lambda shape: np.stack([orc.quant_array(g.normal(size=shape).astype(np.float32).astype(np.float64), quant) for _ in range(S)])
+    xq, pq = q((hi, wi, cin)), q((L["out_h"], L["out_w"], cout))
+    dc = DeepCache(wi, hi, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=dtype, max_regions=4)
+    try:
+        assert B.dc_cache_layer_conv_scheme(dc.handle, li) == 0
+        xin, pin = torch.from_numpy(xq).to(dc.tdtype).cuda(), torch.from_numpy(pq).to(dc.tdtype).cuda()
+        full = dc.conv_partial(li, xin)
+        regs = torch.zeros((S, dc.max_regions, 6), dtype=torch.int32)
+        counts = torch.zeros(S, dtype=torch.int32)
+        ow, oh = L["out_w"], L["out_h"]
+        if oh > 4:
+            regs[0, 0] = torch.tensor([1, 2, ow // 2, min(11, oh - 3), 2, 1], dtype=torch.int32)
+            counts[0] = 1
+        regs[1, 0] = torch.tensor([0, 0, ow, oh, 0, 0], dtype=torch.int32)       # a stream with nothing left to compute
+        counts[1] = 1
+        part = dc.conv_partial(li, xin, pin, regs.cuda(), counts.cuda())
+        wq = orc.quant_array(wts, quant)
+        for s_ in range(S):
+            r = np.zeros(1, orc.REGION_DTYPE)
+            r[0] = tuple(int(v) for v in regs[s_, 0])
+            want_full, _ = orc.conv_reuse(xq[s_], L, wq, bias, quant)
+            want, reused = orc.conv_reuse(xq[s_], L, wq, bias, quant, pq[s_], r[:int(counts[s_])])
+            U.assert_map_close(full[s_], want_full, bf16, f"full, stream {s_}")
+            U.assert_map_close(part[s_], want, bf16, f"partial, stream {s_}")
+            m = reused.astype(bool)
+            assert np.array_equal(part[s_].float().cpu().numpy().astype(np.float64)[m], want[m])
+        assert dc.status() == B.DC_OK
+    finally:
+        dc.close()
