@@ -1,10 +1,7 @@
 // Image block matching (Section 4, Steps 1-5) on the GPU.  Integer arithmetic only.
 //
-//   k_search   Step 2: one warp per block; the block of the current frame sits in shared
-//              memory, candidates of the previous frame are fetched as unaligned 32-bit words
-//              (two aligned loads + funnel shift), |a-b| per byte by vabsdiff4, squares summed
-//              by dp4a, warp-reduced.  Candidates are ordered by (SSE, |dx|+|dy|, dy, dx).
-//              Blocks that pass the PSNR bound add their vector to the Step 3 sums.
+//   dc_search_win.cu  Step 2 for other block sizes and for blocks clipped by the frame's edge.  Candidates are ordered
+//              by (SSE, |dx|+|dy|, dy, dx).  Blocks that pass the PSNR bound add their vector to the Step 3 sums.
 //   k_search_dsw  Step 2 for 16-pixel blocks with diamond search (the common case): one CTA per 8 x 2
 //              blocks, the previous frame's window staged once in shared memory as one word per pixel; one
 //              warp per block, lane 2r + h scoring every other pixel of block row r, so that loads are free of
@@ -18,6 +15,7 @@
 //   k_merge_runs, k_merge   Step 5: maximal horizontal runs per block row, merged vertically when the
 //              spans are identical, emitted in (y, x) order by a CTA-wide ordered compaction.
 #include "dc_common.cuh"
+#include "dc_search_win.cuh"
 
 namespace {
 
@@ -28,7 +26,6 @@ struct MatchArgs {
     const uint8_t* cur;  size_t cur_pitch;  size_t cur_stream;
     const uint8_t* prev; size_t prev_pitch; size_t prev_stream;
     int W, H, B, R, Gx, Gy, S, search, skip_k, region_mode;
-    int edge_only;                       // generic search: 1 = only blocks clipped by the frame edge, 2 = only blocks clipped in width (the rest has a fast kernel)
     uint32_t limit[4];
     int16_t* mv; uint32_t* sse; uint8_t* matched; int32_t* acc; int32_t* gmv;
     int32_t* status;                     // device status word: a walk ended by its step limit records DC_ERR_TIMEOUT
@@ -104,7 +101,6 @@ __device__ __forceinline__ bool load_block(const MatchArgs& a, uint32_t* sm, Blo
     c.lane = threadIdx.x & 31;
     c.x0 = bx * a.B; c.y0 = by * a.B;
     c.bw = min(a.B, a.W - c.x0); c.bh = min(a.B, a.H - c.y0);
-    if ((a.edge_only == 1 && c.bw == a.B && c.bh == a.B) || (a.edge_only == 2 && c.bw == a.B)) return false;
     c.W = a.W; c.H = a.H; c.R = a.R;
     c.prev = a.prev + (size_t)s * a.prev_stream; c.prev_pitch = a.prev_pitch;
     c.cur_sm = sm;
@@ -130,88 +126,6 @@ __device__ __forceinline__ bool load_block(const MatchArgs& a, uint32_t* sm, Blo
 __device__ __forceinline__ int limit_index(const MatchArgs& a, int bw, int bh)
 {
     return (bh < a.B ? 2 : 0) + (bw < a.B ? 1 : 0);
-}
-
-template <int ITERS>
-__global__ void __launch_bounds__(WARPS * 32) k_search(MatchArgs a)
-{
-    __shared__ uint32_t sm_all[WARPS][32 * MAX_ROW_WORDS];
-    BlockCtx<ITERS> c; int s, b;
-    if (!load_block<ITERS>(a, sm_all[threadIdx.x >> 5], c, s, b)) return;
-    if (a.skip_k > 1 && ((b % a.Gx) % a.skip_k != 0 || (b / a.Gx) % a.skip_k != 0)) {
-        // Section 4, k-skip: this block is not searched and takes no part in Step 3
-        if (c.lane == 0) {
-            size_t g = (size_t)s * a.Gx * a.Gy + b;
-            a.mv[2 * g] = 0; a.mv[2 * g + 1] = 0; a.sse[g] = 0xffffffffu;
-        }
-        return;
-    }
-
-    int bx_ = 0, by_ = 0;
-    uint32_t bs = c.sse(0, 0);                         // the zero vector is always a candidate
-    unsigned long long bk = cand_key(bs, 0, 0);
-    if (a.search == DC_SEARCH_EXHAUSTIVE) {
-        for (int dy = -a.R; dy <= a.R; ++dy)
-            for (int dx = -a.R; dx <= a.R; ++dx) {
-                if ((dx == 0 && dy == 0) || !c.valid(dx, dy)) continue;
-                uint32_t v = c.sse(dx, dy);
-                unsigned long long k = cand_key(v, dx, dy);
-                if (k < bk) { bk = k; bs = v; bx_ = dx; by_ = dy; }
-            }
-    } else if (a.search == DC_SEARCH_THREE_STEP) {
-        // nine-point passes with step S0, S0/2, ..., 1; S0 = largest power of two with 2 S0 - 1 <= R
-        int step = a.R < 1 ? 0 : 1;
-        while (4 * step - 1 <= a.R) step *= 2;
-        for (; step >= 1; step >>= 1) {
-            const int cx = bx_, cy = by_;
-#pragma unroll 1
-            for (int i = 0; i < 9; ++i) {
-                if (i == 4) continue;
-                const int dx = cx + (i % 3 - 1) * step, dy = cy + (i / 3 - 1) * step;
-                if (!c.valid(dx, dy)) continue;
-                uint32_t v = c.sse(dx, dy);
-                unsigned long long k = cand_key(v, dx, dy);
-                if (k < bk) { bk = k; bs = v; bx_ = dx; by_ = dy; }
-            }
-        }
-    } else {
-        // large diamond until its centre wins, then one small diamond
-        const int lx[8] = {0, -1, 1, -2, 2, -1, 1, 0}, ly[8] = {-2, -1, -1, 0, 0, 1, 1, 2};
-        const int sx[4] = {0, -1, 1, 0}, sy[4] = {-1, 0, 0, 1};
-        const int max_steps = (2 * a.R + 1) * (2 * a.R + 1);   // every move strictly lowers the key: never reached
-        bool settled = false;
-        for (int step = 0; step < max_steps && !settled; ++step) {
-            int cx = bx_, cy = by_;
-#pragma unroll 1
-            for (int i = 0; i < 8; ++i) {
-                int dx = cx + lx[i], dy = cy + ly[i];
-                if (!c.valid(dx, dy)) continue;
-                uint32_t v = c.sse(dx, dy);
-                unsigned long long k = cand_key(v, dx, dy);
-                if (k < bk) { bk = k; bs = v; bx_ = dx; by_ = dy; }
-            }
-            settled = bx_ == cx && by_ == cy;
-        }
-        if (!settled && c.lane == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);   // the limit ended the walk: result not valid
-        int cx = bx_, cy = by_;
-#pragma unroll 1
-        for (int i = 0; i < 4; ++i) {
-            int dx = cx + sx[i], dy = cy + sy[i];
-            if (!c.valid(dx, dy)) continue;
-            uint32_t v = c.sse(dx, dy);
-            unsigned long long k = cand_key(v, dx, dy);
-            if (k < bk) { bk = k; bs = v; bx_ = dx; by_ = dy; }
-        }
-    }
-    if (c.lane == 0) {
-        size_t g = (size_t)s * a.Gx * a.Gy + b;
-        a.mv[2 * g] = (int16_t)bx_; a.mv[2 * g + 1] = (int16_t)by_; a.sse[g] = bs;
-        if (bs <= a.limit[limit_index(a, c.bw, c.bh)]) {          // PSNR > T (Step 3's set S)
-            atomicAdd(&a.acc[4 * s + 0], bx_);
-            atomicAdd(&a.acc[4 * s + 1], by_);
-            atomicAdd(&a.acc[4 * s + 2], 1);
-        }
-    }
 }
 
 // mean of n values with sum `sum`, rounded to nearest, halves away from zero
@@ -1291,22 +1205,36 @@ __global__ void k_copy_frame(const uint8_t* src, size_t src_pitch, uint8_t* dst,
 }
 
 template <int ITERS>
-void launch_generic(dc_cache* c, MatchArgs& a, bool search)
+void launch_verify(dc_cache* c, MatchArgs& a)
 {
-    int warps = a.S * a.Gx * a.Gy;
-    int grid = dc_div_up(warps, WARPS);
-    if (search) { dc_prof_scope ps(c, DC_ST_SEARCH); k_search<ITERS><<<grid, WARPS * 32, 0, c->stream>>>(a); }
-    else { dc_prof_scope ps(c, DC_ST_VERIFY); k_verify<ITERS><<<grid, WARPS * 32, 0, c->stream>>>(a); }
+    dc_prof_scope ps(c, DC_ST_VERIFY);
+    k_verify<ITERS><<<dc_div_up(a.S * a.Gx * a.Gy, WARPS), WARPS * 32, 0, c->stream>>>(a);
 }
 
-void launch_by_block(dc_cache* c, MatchArgs& a, bool search)
+void launch_verify_by_block(dc_cache* c, MatchArgs& a)
 {
     int row_words = (a.B * 3 + 3) / 4, iters = dc_div_up(a.B * row_words, 32);
-    if (iters <= 2) launch_generic<2>(c, a, search);
-    else if (iters <= 3) launch_generic<3>(c, a, search);
-    else if (iters <= 6) launch_generic<6>(c, a, search);
-    else if (iters <= 12) launch_generic<12>(c, a, search);
-    else launch_generic<24>(c, a, search);
+    if (iters <= 2) launch_verify<2>(c, a);
+    else if (iters <= 3) launch_verify<3>(c, a);
+    else if (iters <= 6) launch_verify<6>(c, a);
+    else if (iters <= 12) launch_verify<12>(c, a);
+    else launch_verify<24>(c, a);
+}
+
+// Step 2 over staged windows: every block, or (only_clipped, see dc_win_args) those that the 16-pixel kernels leave out
+int search_win(dc_cache* c, const MatchArgs& a, int only_clipped)
+{
+    dc_win_args w;
+    const size_t bytes = c->key_pitch * (size_t)c->cfg.height * c->S + 256;      // the library's copies and their spare tail
+    w.cur = a.cur; w.cur_end = a.cur + bytes; w.cur_pitch = a.cur_pitch; w.cur_stream = a.cur_stream;
+    w.prev = a.prev; w.prev_end = a.prev + bytes; w.prev_pitch = a.prev_pitch; w.prev_stream = a.prev_stream;
+    w.W = a.W; w.H = a.H; w.B = a.B; w.R = a.R; w.Gx = a.Gx; w.Gy = a.Gy; w.S = a.S; w.search = a.search; w.skip_k = a.skip_k;
+    w.only_clipped = only_clipped;
+    for (int i = 0; i < 4; ++i) w.limit[i] = a.limit[i];
+    w.mv = a.mv; w.sse = a.sse; w.acc = a.acc; w.status = a.status;
+    dc_prof_scope ps(c, DC_ST_SEARCH);
+    c->launches += 1;
+    return dc_launch_search_win(w, c->num_sms, c->device, c->stream);
 }
 
 }  // namespace
@@ -1332,7 +1260,7 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
     a.cur = cur_key; a.cur_pitch = c->key_pitch; a.cur_stream = c->key_pitch * (size_t)c->cfg.height;
     a.prev = prev_key; a.prev_pitch = c->key_pitch; a.prev_stream = c->key_pitch * (size_t)c->cfg.height;
     a.W = c->cfg.width; a.H = c->cfg.height; a.B = c->cfg.block; a.R = c->cfg.range;
-    a.Gx = c->Gx; a.Gy = c->Gy; a.S = c->S; a.search = c->cfg.search; a.skip_k = c->cfg.skip_k; a.region_mode = c->cfg.region_mode; a.edge_only = 0;
+    a.Gx = c->Gx; a.Gy = c->Gy; a.S = c->S; a.search = c->cfg.search; a.skip_k = c->cfg.skip_k; a.region_mode = c->cfg.region_mode;
     for (int i = 0; i < 4; ++i) a.limit[i] = c->sse_limit[i];
     a.mv = c->blk_mv; a.sse = c->blk_sse; a.matched = c->matched; a.acc = c->mv_acc; a.gmv = c->gmv;
     a.status = c->status;
@@ -1353,10 +1281,8 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
             c->launches += 1;
         }
         if (a.W % 16 != 0) {                                        // blocks clipped by the right edge
-            a.edge_only = 2;
-            launch_by_block(c, a, true);
-            a.edge_only = 0;
-            c->launches += 1;
+            const int rc = search_win(c, a, 2);
+            if (rc != DC_OK) return rc;
         }
     } else if (a.B == 16 && a.search == DC_SEARCH_THREE_STEP && a.skip_k <= 1 && tss_window_bytes(a.R) <= 160 * 1024) {
         int s0 = a.R < 1 ? 0 : 1;                                   // first step: the largest power of two with 2 S0 - 1 <= R
@@ -1374,10 +1300,8 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
             k_search_tss16q<TSS_LPB, TSS_VS><<<ctas, TSS_LPB * 8 * TSS_VS, smem, c->stream>>>(a, s0, wr, words, pitch);
         }
         if (a.W % 16 != 0) {                                        // blocks clipped by the right edge
-            a.edge_only = 2;
-            launch_by_block(c, a, true);
-            a.edge_only = 0;
-            c->launches += 1;
+            const int rc = search_win(c, a, 2);
+            if (rc != DC_OK) return rc;
         }
     } else if (a.B == 16 && a.search == DC_SEARCH_EXHAUSTIVE && a.R <= E_MAXR && a.W >= 16 && a.H >= 16) {
         const int chunks = (2 * a.R + 1 + E_DY - 1) / E_DY;
@@ -1392,13 +1316,12 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
             k_search_es16<<<((a.Gx + 7) / 8) * a.Gy * a.S, 256, smem, c->stream>>>(a);
         }
         if (a.W % 16 != 0 || a.H % 16 != 0) {                   // blocks clipped by the right / bottom edge
-            a.edge_only = 1;
-            launch_by_block(c, a, true);
-            a.edge_only = 0;
-            c->launches += 1;
+            const int rc = search_win(c, a, 1);
+            if (rc != DC_OK) return rc;
         }
     } else {
-        launch_by_block(c, a, true);
+        const int rc = search_win(c, a, 0);
+        if (rc != DC_OK) return rc;
     }
     if (a.region_mode == DC_REGIONS_PER_BLOCK) {
         dc_prof_scope ps(c, DC_ST_VERIFY);
@@ -1410,7 +1333,7 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
         k_verify16_list<<<c->num_sms * 8, 256, 0, c->stream>>>(a, (const uint32_t*)c->long_list, todo_count);
         c->launches += 1;
     } else {
-        launch_by_block(c, a, false);
+        launch_verify_by_block(c, a);
     }
     {
         dc_prof_scope ps(c, DC_ST_MERGE);

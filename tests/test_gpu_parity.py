@@ -861,3 +861,17 @@ def test_conv_on_cuda_cores(dtype, hi, wi, cin, cout, k, S, groups):
         assert dc.status() == B.DC_OK
     finally:
         dc.close()
+
+
+@pytest.mark.parametrize("search", [B.DC_SEARCH_EXHAUSTIVE, B.DC_SEARCH_DIAMOND, B.DC_SEARCH_THREE_STEP])
+@pytest.mark.parametrize("block,R,shape", [(4, 12, (41, 67)), (13, 9, (70, 131)), (24, 64, (150, 170)), (32, 33, (64, 96)), (9, 7, (200, 181))])
+def test_match_staged_window_shapes(search, block, R, shape):
+    """Block sizes whose lanes own 1 to 32 pixels with a last one that is full or not, windows that shrink the tile (large
+    ranges), clipped right columns and bottom rows, k-skip."""
+    g = rng(block * 3 + R)
+    H, W = shape
+    prev = g.integers(0, 256, size=(H, W, 3), dtype=np.uint8)
+    smooth = np.repeat(np.repeat(g.integers(0, 256, size=(H // 8 + 1, W // 8 + 1, 3), dtype=np.uint8), 8, 0), 8, 1)[:H, :W]
+    pairs = [(prev, np.roll(prev, (min(R, 5), -min(R, 6)), axis=(0, 1))), (smooth, np.roll(smooth, (-3, 4), axis=(0, 1))), (prev, smooth)]
+    check_pairs(pairs, block, R, search)
+    check_pairs(pairs[1:2], block, R, search, skip_k=2)
