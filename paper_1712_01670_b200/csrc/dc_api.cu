@@ -10,6 +10,7 @@
 #include "dc_common.cuh"
 
 static thread_local char g_last_cuda_error[256];
+thread_local bool g_dc_pdl = true;
 
 void dc_note_cuda_error(cudaError_t e, const char* file, int line)
 {
@@ -35,18 +36,6 @@ bool dc_layer_cached(const dc_cache* c, int layer)
 }
 
 namespace {
-
-// nearest bfloat16 (ties to even) of a double, as its 16 bit pattern
-uint16_t bf16_bits_from_double(double v)
-{
-    if (v == 0.0) return 0;
-    int e = ilogb(v);
-    if (e < -126) e = -126;
-    double q = ldexp(nearbyint(ldexp(v, 7 - e)), e - 7);
-    float f = (float)q;                       // exact: q has at most 8 significant bits
-    uint32_t u; memcpy(&u, &f, 4);
-    return (uint16_t)(u >> 16);
-}
 
 template <typename T>
 int dev_alloc(dc_cache* c, T** p, size_t count)
@@ -165,10 +154,11 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     }
     dc_use_match_set(c, 0);
     DC_TRY(dev_alloc(c, &c->table, (size_t)n * S * c->max_regions));
-    DC_TRY(dev_alloc(c, &c->layers_dev, (size_t)n));
-    DC_TRY(dev_alloc(c, &c->in_hw_dev, (size_t)n * 2));
+    DC_TRY(dc_build_propagate_table(c, layers));
     DC_TRY(dev_alloc(c, &c->dirty_count, (size_t)n));
     DC_TRY(dev_alloc(c, &c->all_count, (size_t)n * 2));
+    DC_TRY(dev_alloc(c, &c->partial, (size_t)S + 2));
+    DC_CUDA(cudaMemsetAsync(c->partial, 0, sizeof(int32_t) * (S + 2), c->stream));
     DC_TRY(dev_alloc(c, &c->reuse_px, (size_t)n * S * 2));
     c->alive = c->reuse_px + (size_t)n * S;
     DC_TRY(dev_alloc(c, &c->status, (size_t)1));
@@ -176,7 +166,6 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     DC_CUDA(cudaMemsetAsync(c->reused_total, 0, sizeof(unsigned long long) * n, c->stream));
     DC_CUDA(cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream));
     DC_CUDA(cudaMemsetAsync(c->table, 0, sizeof(dc_region) * n * S * c->max_regions, c->stream));
-    DC_CUDA(cudaMemcpyAsync(c->layers_dev, layers, sizeof(dc_layer_desc) * n, cudaMemcpyHostToDevice, c->stream));
 
     // PSNR > T as an integer bound on the SSE, for the four block shapes of a clipped grid
     for (int i = 0; i < 4; ++i) {
@@ -186,20 +175,7 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
         double lim = ceil(q) - 1.0;
         c->sse_limit[i] = lim >= 4294967295.0 ? 4294967295u : (uint32_t)lim;
     }
-    // pixel -> map element table
-    if (cfg.dtype == DC_BF16) {
-        uint16_t lut[256];
-        for (int i = 0; i < 256; ++i) lut[i] = bf16_bits_from_double((double)i / 255.0);
-        DC_TRY(dev_alloc(c, (uint16_t**)&c->pix_lut, (size_t)256));
-        DC_CUDA(cudaMemcpy(c->pix_lut, lut, sizeof(lut), cudaMemcpyHostToDevice));
-    } else {
-        float lut[256];
-        for (int i = 0; i < 256; ++i) lut[i] = (float)((double)i / 255.0);
-        DC_TRY(dev_alloc(c, (float**)&c->pix_lut, (size_t)256));
-        DC_CUDA(cudaMemcpy(c->pix_lut, lut, sizeof(lut), cudaMemcpyHostToDevice));
-    }
-
-    int32_t in_hw[DC_MAX_LAYERS * 2], all_count[DC_MAX_LAYERS * 2];
+    int32_t all_count[DC_MAX_LAYERS * 2];
     size_t max_tiles = 1;
     bool need_input_map = false;
     for (int i = 0; i < n; ++i) {
@@ -210,7 +186,6 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
         if (L.d.kind == DC_FC && c->executable) { L.d.kind = DC_CONV; L.d.sh = L.d.sw = 1; L.d.ph = L.d.pw = 0; }
         L.in_h = L.d.in0 < 0 ? cfg.height : layers[L.d.in0].out_h;
         L.in_w = L.d.in0 < 0 ? cfg.width : layers[L.d.in0].out_w;
-        in_hw[2 * i] = L.in_h; in_hw[2 * i + 1] = L.in_w;
         all_count[i] = 0; all_count[n + i] = 0;
         if (!c->executable) continue;
         if (L.d.in0 < 0 && L.d.kind != DC_RESIZE_AREA) need_input_map = true;
@@ -245,7 +220,6 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
             DC_TRY(dc_pack_weights(c, i, (const float*)weights_dev[i], (const float*)bias_dev[i]));
         }
     }
-    DC_CUDA(cudaMemcpyAsync(c->in_hw_dev, in_hw, sizeof(int32_t) * 2 * n, cudaMemcpyHostToDevice, c->stream));
     DC_CUDA(cudaMemcpyAsync(c->all_count, all_count, sizeof(int32_t) * 2 * n, cudaMemcpyHostToDevice, c->stream));
     DC_TRY(dev_alloc(c, &c->zero_masks, max_tiles * 4));
     DC_CUDA(cudaMemsetAsync(c->zero_masks, 0, max_tiles * 4 * sizeof(uint32_t), c->stream));
@@ -253,13 +227,27 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
         DC_TRY(dev_alloc(c, (uint8_t**)&c->input_map, (size_t)S * cfg.height * cfg.width * 3 * c->elt));
     size_t stat_ints = (size_t)S * (3 + 4 + 1) + (size_t)n * S;
     if (cudaMallocHost(&c->stats_pinned, stat_ints * sizeof(int32_t)) != cudaSuccess) { cudaGetLastError(); return DC_ERR_ALLOC; }
-    DC_CUDA(cudaStreamSynchronize(c->stream));      // layers / in_hw / all_count live on this stack frame
+    DC_CUDA(cudaStreamSynchronize(c->stream));      // all_count lives on this stack frame
     for (int i = 0; i < n; ++i)
         if (c->executable && c->L[i].d.kind == DC_CONV) {
             const void* in = c->L[i].d.in0 < 0 ? c->input_map : c->L[c->L[i].d.in0].map[0];
             if (c->L[i].s2d_s) in = c->L[i].in_s2d;               // the kernels being timed read the block map
             DC_TRY(dc_conv_bf16_autotune(c, i, in));
         }
+    // who reads the frame as a map, and who reads the resized frame
+    c->fused_input = need_input_map; c->resize_feeds = -1;
+    int resize = -1, readers = 0;
+    for (int i = 0; i < n && c->executable; ++i) {
+        const dc_layer_desc& d = c->L[i].d;
+        if (d.kind == DC_RESIZE_AREA) { resize = i; continue; }
+        const bool two = d.kind == DC_ADD || d.kind == DC_CONCAT;
+        if ((two && d.in1 < 0) || (d.in0 < 0 && !dc_conv_takes_frame(c, i))) c->fused_input = false;
+    }
+    for (int i = 0; i < n && resize >= 0; ++i) {
+        const dc_layer_desc& d = c->L[i].d;
+        if (d.kind == DC_CONV && d.in0 == resize && dc_conv_takes_frame(c, i) && !c->L[i].s2d_s) { c->resize_feeds = i; ++readers; }
+    }
+    if (readers != 1) c->resize_feeds = -1;
     if (c->executable) DC_TRY(dc_build_classify_table(c));       // after the tuner: it decides each layer's tile geometry
     DC_CUDA(cudaStreamSynchronize(c->stream));
     return DC_OK;
@@ -279,8 +267,8 @@ void release(dc_cache* c)
         cudaFree(m.long_list); cudaFree(m.gmv); cudaFree(m.regions0); cudaFree(m.n_regions);
     }
     cudaFree(c->table); cudaFree(c->classify_table);
-    cudaFree(c->layers_dev); cudaFree(c->in_hw_dev); cudaFree(c->dirty_count); cudaFree(c->all_count);
-    cudaFree(c->reuse_px); cudaFree(c->zero_masks); cudaFree(c->status); cudaFree(c->input_map); cudaFree(c->pix_lut);
+    cudaFree(c->prop_table); cudaFree(c->dirty_count); cudaFree(c->partial); cudaFree(c->all_count);
+    cudaFree(c->reuse_px); cudaFree(c->zero_masks); cudaFree(c->status); cudaFree(c->input_map);
     if (c->stats_pinned) cudaFreeHost(c->stats_pinned);
     for (int i = 0; i < c->n_layers; ++i) {
         dc_layer_rt& L = c->L[i];
@@ -405,7 +393,7 @@ int dc_cache_set_key(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
 {
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
     DC_TRY(cancel_lookahead(c));
-    DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, c->key[c->key_cur]));
+    DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, c->key[c->key_cur], nullptr));
     c->key_valid = true;
     return DC_OK;
 }
@@ -418,16 +406,14 @@ int dc_match_blocks(dc_cache* c, const uint8_t* frame_dev, size_t pitch, int16_t
     if (!c->key_valid) return DC_ERR_STATE;
     DC_TRY(cancel_lookahead(c));
     uint8_t* scratch = c->key[(c->key_cur + 1) % 3];                             // scratch copy; the cache key stays
-    DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, scratch));
-    DC_TRY(dc_launch_match(c, scratch, c->key[c->key_cur]));
-    const size_t nblk = (size_t)c->S * c->Gx * c->Gy;
-    const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    if (block_mv_dev) DC_CUDA(cudaMemcpyAsync(block_mv_dev, c->blk_mv, nblk * 2 * sizeof(int16_t), k, c->stream));
-    if (block_sse_dev) DC_CUDA(cudaMemcpyAsync(block_sse_dev, c->blk_sse, nblk * sizeof(uint32_t), k, c->stream));
-    if (matched_dev) DC_CUDA(cudaMemcpyAsync(matched_dev, c->matched, nblk, k, c->stream));
-    if (global_mv_dev) DC_CUDA(cudaMemcpyAsync(global_mv_dev, c->gmv, sizeof(int32_t) * 3 * c->S, k, c->stream));
-    if (regions_dev) DC_CUDA(cudaMemcpyAsync(regions_dev, c->regions0, sizeof(dc_region) * c->S * c->max_regions, k, c->stream));
-    if (n_regions_dev) DC_CUDA(cudaMemcpyAsync(n_regions_dev, c->n_regions, sizeof(int32_t) * c->S, k, c->stream));
+    DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, scratch, c->mv_acc));
+    // the kernels write the caller's arrays themselves; vectors are read back as 32-bit words, so an oddly aligned array of
+    // vectors is filled by a copy instead
+    const bool direct_mv = block_mv_dev && (uintptr_t)block_mv_dev % 4 == 0;
+    const dc_match_out out = {direct_mv ? block_mv_dev : nullptr, block_sse_dev, matched_dev, global_mv_dev, regions_dev, n_regions_dev};
+    DC_TRY(dc_launch_match(c, scratch, c->key[c->key_cur], &out));
+    if (block_mv_dev && !direct_mv)
+        DC_CUDA(cudaMemcpyAsync(block_mv_dev, c->blk_mv, (size_t)c->S * c->Gx * c->Gy * 2 * sizeof(int16_t), cudaMemcpyDeviceToDevice, c->stream));
     return DC_OK;
 }
 
@@ -436,18 +422,7 @@ int dc_propagate_regions(dc_cache* c, const dc_region* in_dev, const int32_t* n_
 {
     if (!c || !in_dev || !n_in_dev || !out_dev) return DC_ERR_ARG;
     if (layer_begin < 0 || layer_end > c->n_layers || layer_begin >= layer_end) return DC_ERR_ARG;
-    const size_t per_layer = (size_t)c->S * c->max_regions;
-    // slots beyond n_in keep whatever an earlier call left: clear the table first
-    DC_CUDA(cudaMemsetAsync(c->table, 0, sizeof(dc_region) * per_layer * layer_end, c->stream));
-    DC_CUDA(cudaMemsetAsync(c->alive, 0, sizeof(int32_t) * c->n_layers * c->S, c->stream));
-    DC_TRY(dc_launch_propagate(c, in_dev, n_in_dev, layer_end));
-    DC_CUDA(cudaMemcpyAsync(out_dev, c->table + per_layer * layer_begin,
-                            sizeof(dc_region) * per_layer * (layer_end - layer_begin), cudaMemcpyDeviceToDevice, c->stream));
-    if (n_out_dev)
-        for (int l = 0; l < layer_end - layer_begin; ++l)
-            DC_CUDA(cudaMemcpyAsync(n_out_dev + (size_t)l * c->S, n_in_dev, sizeof(int32_t) * c->S,
-                                    cudaMemcpyDeviceToDevice, c->stream));
-    return DC_OK;
+    return dc_launch_propagate(c, in_dev, n_in_dev, layer_end, false, out_dev, layer_begin, n_out_dev);
 }
 
 int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* prev_out_dev,
@@ -459,15 +434,15 @@ int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* 
     const int tiles = dc_layer_tiles(c, L);
     if (regions_dev || n_regions_dev) {
         if (!regions_dev || !n_regions_dev || !prev_out_dev || prev_out_dev == out_map_dev) return DC_ERR_ARG;
-        DC_CUDA(cudaMemsetAsync(c->dirty_count + layer, 0, sizeof(int32_t), c->stream));
-        DC_CUDA(cudaMemsetAsync(c->reuse_px + (size_t)layer * c->S, 0, sizeof(int32_t) * c->S, c->stream));
-        DC_TRY(dc_launch_classify_copy(c, layer, regions_dev, n_regions_dev, prev_out_dev, out_map_dev));
-        return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.dirty_list, c->dirty_count + layer, L.masks, tiles);
+        int32_t* count = c->partial + c->partial_cur;
+        c->partial_cur ^= 1;
+        DC_TRY(dc_launch_classify_copy(c, layer, regions_dev, n_regions_dev, prev_out_dev, out_map_dev, count, c->partial + 2, c->partial + c->partial_cur));
+        return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.dirty_list, count, L.masks, tiles);
     }
     return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.all_list, dc_all_count(c, layer), c->zero_masks, tiles);
 }
 
-int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* out_map_dev, dc_frame_stats* stats)
+static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* out_map_dev, dc_frame_stats* stats)
 {
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
     if (!c->executable) return DC_ERR_STATE;
@@ -477,24 +452,25 @@ int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* ou
     // the library's own aligned copy of the frame: matched now, the cache key of the next frame (Section 3)
     uint8_t* frame_copy = c->key[(c->key_cur + 1) % 3];
     const bool looked_ahead = c->la_frame == frame_dev && c->la_pitch == pitch && c->key_valid;
-    c->overlap_mode = looked_ahead;                   // a caller that looks ahead keeps doing so: see ring_budget()
+    // a caller that looks ahead keeps doing so: where the matcher of the next frame is large (more blocks than the SMs hold
+    // warps, ten times over), the inference leaves it room (see ring_budget())
+    c->overlap_mode = looked_ahead && (long long)S * c->Gx * c->Gy > (long long)c->num_sms * 640;
+    g_dc_pdl = !c->overlap_mode;
     if (looked_ahead) {
         // dc_lookahead_frame already copied this frame in and (unless it is a full frame) matched it
         DC_CUDA(cudaStreamWaitEvent(c->stream, c->ev_match, 0));
         c->la_frame = nullptr;
     } else {
         DC_TRY(cancel_lookahead(c));
-        DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, frame_copy));
+        DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, frame_copy, c->mv_acc));
     }
     if (c->la_stream) DC_CUDA(cudaEventRecord(c->ev_key, c->stream));   // a later lookahead may start from here
     if (!refresh) {
-        DC_CUDA(cudaMemsetAsync(c->dirty_count, 0, sizeof(int32_t) * n, c->stream));
-        DC_CUDA(cudaMemsetAsync(c->reuse_px, 0, sizeof(int32_t) * n * S * 2, c->stream));     // and `alive` behind it
         if (looked_ahead && c->la_matched) dc_use_match_set(c, c->mset_cur ^ 1);              // results are waiting there
-        else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur]));
-        DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n));
+        else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur], nullptr));
+        DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n, true, nullptr, 0, nullptr));
     }
-    if (c->input_map) DC_TRY(dc_launch_input_map(c, frame_copy, c->key_pitch));
+    if (c->input_map && !c->fused_input) DC_TRY(dc_launch_input_map(c, frame_copy, c->key_pitch));
     const size_t per_layer = (size_t)S * c->max_regions;
     // bitmaps, reuse copies and dirty lists of every cached layer in one launch (they need only the rectangles and
     // each layer's own cached map); possible while all cached layers keep their newest map at the same index
@@ -512,8 +488,10 @@ int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* ou
         case DC_CONV: {
             const int tiles = dc_layer_tiles(c, L);
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
+            if (L.d.in0 < 0 && c->fused_input) { DC_TRY(dc_launch_frame_operand(c, i, frame_copy, c->key_pitch)); in = nullptr; }
+            else if (i == c->resize_feeds) in = nullptr;              // its operand copy is filled already
             if (!refresh) {
-                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out));
+                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
                 DC_TRY(dc_launch_conv(c, i, in, out, L.dirty_list, c->dirty_count + i, L.masks, tiles));
             } else {
                 DC_TRY(dc_launch_conv(c, i, in, out, L.all_list, dc_all_count(c, i), c->zero_masks, tiles));
@@ -525,7 +503,7 @@ int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* ou
             if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_maxpool(c, i, in, L.map[0], nullptr)); break; }
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
             if (!refresh) {           // Section 5's three steps on a pooling layer: copy, mark, compute the rest
-                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out));
+                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
                 DC_TRY(dc_launch_maxpool(c, i, in, out, L.masks));
             } else {
                 DC_TRY(dc_launch_maxpool(c, i, in, out, nullptr));
@@ -539,7 +517,7 @@ int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* ou
             if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_lrn(c, i, in, L.map[0], nullptr)); break; }
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
             if (!refresh) {
-                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out));
+                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
                 DC_TRY(dc_launch_lrn(c, i, in, out, L.masks));
             } else {
                 DC_TRY(dc_launch_lrn(c, i, in, out, nullptr));
@@ -562,9 +540,16 @@ int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* ou
     if (refresh) c->frames_full += 1; else c->frames_cached += 1;
     c->last_refreshed = refresh;
     if (out_map_dev)
-        DC_CUDA(cudaMemcpyAsync(out_map_dev, layer_input(c, n - 1), c->L[n - 1].map_bytes, cudaMemcpyDeviceToDevice, c->stream));
+        DC_TRY(dc_launch_copy_map(c, layer_input(c, n - 1), out_map_dev, c->L[n - 1].map_bytes));
     if (stats) return fill_stats(c, refresh, stats);
     return DC_OK;
+}
+
+int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* out_map_dev, dc_frame_stats* stats)
+{
+    const int rc = infer_frame(c, frame_dev, pitch, out_map_dev, stats);
+    g_dc_pdl = true;
+    return rc;
 }
 
 static int ensure_lookahead_stream(dc_cache* c)
@@ -595,10 +580,10 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     const int main_set = c->mset_cur;
     c->stream = c->la_stream;                                       // the launchers enqueue on c->stream
     uint8_t* next_copy = c->key[(c->key_cur + 1) % 3];
-    int rc = dc_launch_copy_frame(c, frame_dev, pitch, next_copy);
+    int rc = dc_launch_copy_frame(c, frame_dev, pitch, next_copy, c->mset[main_set ^ 1].mv_acc);
     if (rc == DC_OK && !next_is_full) {
         dc_use_match_set(c, main_set ^ 1);
-        rc = dc_launch_match(c, next_copy, c->key[c->key_cur]);
+        rc = dc_launch_match(c, next_copy, c->key[c->key_cur], nullptr);
         dc_use_match_set(c, main_set);
     }
     c->stream = main_stream;

@@ -118,16 +118,18 @@ struct dc_cache {
     dc_region* regions0;            // [S][max_regions] rectangles on the frame
     int32_t* n_regions;             // [S]
     dc_region* table;               // [n_layers][S][max_regions]
-    dc_layer_desc* layers_dev;      // [n_layers]
-    int32_t* in_hw_dev;             // [n_layers][2]
+    void* prop_table;               // [n_layers] the layer table as region propagation reads it (dc_regions.cu)
     int32_t* dirty_count;           // [n_layers]
+    int32_t* partial;               // dc_conv_partial: two dirty counters used in turn (each call zeroes the other), then [S] reused pixels (not read)
+    int partial_cur;
     int32_t* all_count;             // [n_layers]
     int32_t* reuse_px;              // [n_layers][S]
-    int32_t* alive;                 // [n_layers][S] rectangles not yet eroded away (directly behind reuse_px)
+    int32_t* alive;                 // [n_layers][S] rectangles not yet eroded away
     uint32_t* zero_masks;           // all-zero reuse bitmap shared by full frames
     int32_t* status;                // device status word
     void* input_map;                // frame / 255 as a map, [S][H][W][3]
-    void* pix_lut;                  // 256 entries: pixel value -> map element
+    bool fused_input;               // the frame goes straight into the operand copies of the convolutions that read it: no input map per frame
+    int resize_feeds;               // few-channel convolution whose padded operand the resize layer writes as well, or -1
     void* stats_pinned;             // host staging for statistics
     unsigned long long* reused_total; // [n_layers] reused output pixels summed over all frames so far
     int64_t frames_cached, frames_full;
@@ -168,6 +170,10 @@ struct dc_once_per_device {
 __device__ __forceinline__ void dc_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dc_pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Off while a large matcher runs beside the inference (dc_infer_frame): a kernel that waits for its turn holds room on
+// the SMs that the block search on the side stream could use.
+extern thread_local bool g_dc_pdl;
+
 template <typename... KArgs, typename... Args>
 static inline cudaError_t dc_launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args&&... args)
 {
@@ -176,17 +182,20 @@ static inline cudaError_t dc_launch_pdl(void (*kernel)(KArgs...), dim3 grid, int
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.attrs = attr; cfg.numAttrs = g_dc_pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 // ---- kernels' host-side launchers (each returns DC_OK or DC_ERR_CUDA) ----
-int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst);
-int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key);   // both in key-frame layout
+int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst, int32_t* zero);
+// arrays of a caller of dc_match_blocks that the kernels write themselves (NULL: not wanted)
+struct dc_match_out { int16_t* mv; uint32_t* sse; uint8_t* matched; int32_t* gmv; dc_region* regions; int32_t* n_regions; };
+int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key, const dc_match_out* out);   // both frames in key-frame layout
 void dc_use_match_set(dc_cache* c, int k);
-int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end);
+int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers);
+int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out);
 int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, const int32_t* n_regions,
-                            const void* prev_out, void* out);
+                            const void* prev_out, void* out, int32_t* count, int32_t* px, int32_t* zero_next);
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                    const int32_t* tile_count, const uint32_t* masks, int max_tiles);
 // stride-1 layers and single output pixels on CUDA cores (dc_conv_simt.cu)
@@ -196,6 +205,9 @@ int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const
 int dc_launch_dense(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
 int dc_pack_weights_simt(dc_cache* c, int layer);
 int dc_launch_input_map(dc_cache* c, const uint8_t* frame, size_t pitch);
+bool dc_conv_takes_frame(const dc_cache* c, int layer);      // the layer's operand copy can be filled from the frame itself
+int dc_launch_frame_operand(dc_cache* c, int layer, const uint8_t* frame, size_t pitch);
+int dc_launch_copy_map(dc_cache* c, const void* src, void* dst, size_t bytes);
 int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch);   // frame: 16-byte aligned rows
 int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
 int dc_launch_lrn(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);

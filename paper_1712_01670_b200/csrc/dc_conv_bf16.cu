@@ -68,14 +68,6 @@ __host__ __device__ constexpr size_t ctl_bytes(int epi_warps) { return sizeof(Sm
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Programmatic dependent launch: a convolution kernel is launched so that its CTAs may become resident while the
-// previous kernel of the stream is still running (on SMs that kernel has left).  Barrier set-up, tensor-memory
-// allocation and descriptor prefetch run there; pdl_wait() returns once the previous kernel has completed and its
-// writes are visible, and nothing that another kernel produces is read (or overwritten) before it.
-// pdl_release() lets the kernel after this one do the same.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 __device__ __forceinline__ void mbar_init(void* bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -383,8 +375,8 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    pdl_wait();                 // the previous kernel's output, the tile list and its count are read from here on
-    pdl_release();
+    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
+    dc_pdl_release();
     const int n_tiles = *a.tile_count;
     const int n_items = (n_tiles + MT - 1) / MT * a.NB;     // an item: MT tiles x one block of BN channels; none for this CTA: it only frees its tensor memory
 
@@ -552,8 +544,8 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    pdl_wait();                 // the previous kernel's output, the tile list and its count are read from here on
-    pdl_release();
+    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
+    dc_pdl_release();
     const int n_items = *a.tile_count;
 
     if (warp == 0) {
@@ -685,8 +677,8 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    pdl_wait();                 // the previous kernel's output, the tile list and its count are read from here on
-    pdl_release();
+    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
+    dc_pdl_release();
     const int n_tiles = *a.tile_count;
     const int n_items = (n_tiles + MT - 1) / MT * a.NB;
 
@@ -902,8 +894,8 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     cluster_sync_all();                                       // both CTAs' barriers exist before either is signalled from outside
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    pdl_wait();                 // the previous kernel's output, the tile list and its count are read from here on
-    pdl_release();
+    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
+    dc_pdl_release();
     const int n_tiles = *a.tile_count;
     const int n_items = (n_tiles + 1) / 2 * a.NB;
 
@@ -1023,6 +1015,8 @@ __global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin,
 // [S][H][W][C] -> [S][H][W][8] with zero padding, C <= 8
 __global__ void k_pad_channels8(const __nv_bfloat16* in, size_t pixels, int C, __nv_bfloat16* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < pixels; i += (size_t)gridDim.x * blockDim.x) {
         unsigned short v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         const unsigned short* p = (const unsigned short*)in + i * C;
@@ -1035,6 +1029,8 @@ __global__ void k_pad_channels8(const __nv_bfloat16* in, size_t pixels, int C, _
 // [S][H][W][C] -> [S][H][W][16] with zero padding, C < 16
 __global__ void k_pad_channels16(const __nv_bfloat16* in, size_t pixels, int C, __nv_bfloat16* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < pixels; i += (size_t)gridDim.x * blockDim.x) {
         unsigned short v[16];
 #pragma unroll
@@ -1121,25 +1117,6 @@ static uint32_t tmem_cols_for(int nbuf, int mt, int bn)
 // inference (dc_lookahead_frame): with 182 KB a convolution CTA leaves room for one CTA of the block search (32 KB) on
 // its SM, which then works in the tensor-core kernel's idle issue slots instead of waiting for a free SM.  Set per
 // launch from the cache's state.
-// Launch with programmatic stream serialization allowed (see pdl_wait): the kernel may start before the previous
-// kernel of the stream has ended.  Not while the block search of the next frame runs beside the inference: there the
-// search is the longer chain, and it is the gaps between convolution kernels that let more of its CTAs in.
-// DC_NO_PDL=1 (diagnostics) always launches the ordinary way.
-static thread_local bool t_pdl = true;
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_conv_kernel(void (*kernel)(KArgs...), int grid, int threads, size_t smem, cudaStream_t stream, Args&&... args)
-{
-    static const bool pdl_env = getenv("DC_NO_PDL") == nullptr;
-    const bool pdl = pdl_env && t_pdl;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 static thread_local int t_ring_kb = 200;
 static thread_local int t_epi_warps = 4;      // the layer's tuned epilogue width, honoured by launches with one CTA per SM
 static int epi_warps_for(int ctas) { return t_epi_warps == 8 && ctas != 2 ? 8 : 4; }
@@ -1261,6 +1238,16 @@ int dc_conv_bf16_supported(const dc_cache* c, int layer)
     return make_plan(c->L[layer].d, p) || smallc_ok(c->L[layer].d) || pad16_ok(c->L[layer].d);
 }
 
+// The first convolution of a bfloat16 cache reads a rearranged copy of its input: the block map (strided layers) or the
+// pixels with their channels padded to eight (few-channel kernel).
+bool dc_conv_takes_frame(const dc_cache* c, int layer)
+{
+    const dc_layer_rt& L = c->L[layer];
+    TcPlan p;
+    if (c->cfg.dtype != DC_BF16 || L.d.kind != DC_CONV || !dc_conv_bf16_supported(c, layer)) return false;
+    return L.s2d_s ? L.s2d_cin == 3 : n_groups(L.d) == 1 && L.d.cin == 3 && smallc_ok(L.d) && !make_plan(L.d, p) && L.in_padded != nullptr;
+}
+
 // Normal layers need no repacking ([cout][kh][kw][cin] is already K-major); few-channel layers
 // get their tap-major packed copy and a buffer for the channel-padded input.
 int dc_pack_weights_bf16(dc_cache* c, int layer)
@@ -1360,9 +1347,9 @@ static int launch_smallc(dc_cache* c, int layer, const void* in, void* out, cons
     int items = max_tiles < 1 ? 1 : max_tiles;
     int grid = items > c->num_sms * ctas ? c->num_sms * ctas : items;
     dc_prof_scope ps(c, DC_ST_CONV);
-    k_pad_channels8<<<grid_pad, 256, 0, c->stream>>>((const __nv_bfloat16*)in, pixels, d.cin, (__nv_bfloat16*)L.in_padded);
-    DC_CUDA(launch_conv_kernel(k_conv_tc_smallc, grid, threads_for(a.epi_warps), smem, c->stream, tmA, sa));
-    c->launches += 2;
+    if (in) DC_CUDA(dc_launch_pdl(k_pad_channels8, dim3((unsigned)grid_pad), 256, 0, c->stream, (const __nv_bfloat16*)in, pixels, (int)d.cin, (__nv_bfloat16*)L.in_padded));
+    DC_CUDA(dc_launch_pdl(k_conv_tc_smallc, dim3((unsigned)(grid)), threads_for(a.epi_warps), smem, c->stream, tmA, sa));
+    c->launches += in ? 2 : 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
@@ -1441,11 +1428,11 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     int grid = items > c->num_sms * ctas ? c->num_sms * ctas : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
     if (slab) {
-        if (mt == 2) DC_CUDA(launch_conv_kernel(k_conv_tc_halo<2, true>, grid, threads_for(a.epi_warps), smem, c->stream, tmA, ha));
-        else DC_CUDA(launch_conv_kernel(k_conv_tc_halo<1, true>, grid, threads_for(a.epi_warps), smem, c->stream, tmA, ha));
+        if (mt == 2) DC_CUDA(dc_launch_pdl(k_conv_tc_halo<2, true>, dim3((unsigned)(grid)), threads_for(a.epi_warps), smem, c->stream, tmA, ha));
+        else DC_CUDA(dc_launch_pdl(k_conv_tc_halo<1, true>, dim3((unsigned)(grid)), threads_for(a.epi_warps), smem, c->stream, tmA, ha));
     } else {
-        if (mt == 2) DC_CUDA(launch_conv_kernel(k_conv_tc_halo<2, false>, grid, threads_for(a.epi_warps), smem, c->stream, tmA, ha));
-        else DC_CUDA(launch_conv_kernel(k_conv_tc_halo<1, false>, grid, threads_for(a.epi_warps), smem, c->stream, tmA, ha));
+        if (mt == 2) DC_CUDA(dc_launch_pdl(k_conv_tc_halo<2, false>, dim3((unsigned)(grid)), threads_for(a.epi_warps), smem, c->stream, tmA, ha));
+        else DC_CUDA(dc_launch_pdl(k_conv_tc_halo<1, false>, dim3((unsigned)(grid)), threads_for(a.epi_warps), smem, c->stream, tmA, ha));
     }
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
@@ -1537,7 +1524,7 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     const int max_pairs = c->num_sms / 2;                        // one CTA per SM, a pair per TPC
     const int pairs = items > max_pairs ? max_pairs : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
-    DC_CUDA(launch_conv_kernel(k_conv_tc_pair, 2 * pairs, kThreads, smem, c->stream, *tmAp, *tmWp, ha));
+    DC_CUDA(dc_launch_pdl(k_conv_tc_pair, dim3((unsigned)(2 * pairs)), kThreads, smem, c->stream, *tmAp, *tmWp, ha));
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;
@@ -1551,7 +1538,6 @@ int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const
 {
     const int G = n_groups(c->L[layer].d);
     t_ring_kb = c->overlap_mode ? 182 : 200;
-    t_pdl = !c->overlap_mode;
     t_bias_bytes = bias_bytes_for(group_view(c->L[layer].d));
     // eight epilogue warps take the registers that the block search of the next frame needs to stay resident beside
     // this kernel: while that overlap is in use the CTA keeps to four
@@ -1584,7 +1570,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
         const size_t pixels = (size_t)c->S * L.in_h * L.in_w;
         int grid_pad = (int)((pixels + 255) / 256); if (grid_pad > c->num_sms * 8) grid_pad = c->num_sms * 8;
         dc_prof_scope ps(c, DC_ST_CONV);
-        k_pad_channels16<<<grid_pad, 256, 0, c->stream>>>((const __nv_bfloat16*)in, pixels, L.d.cin, (__nv_bfloat16*)L.in_padded);
+        DC_CUDA(dc_launch_pdl(k_pad_channels16, dim3((unsigned)grid_pad), 256, 0, c->stream, (const __nv_bfloat16*)in, pixels, (int)L.d.cin, (__nv_bfloat16*)L.in_padded));
         c->launches += 1;
         in = L.in_padded;
     }
@@ -1647,8 +1633,8 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     long long items = (long long)(((max_tiles < 1 ? 1 : max_tiles) + p.MT - 1) / p.MT) * p.NB;
     int grid = items > c->num_sms * ctas ? c->num_sms * ctas : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
-    if (p.MT == 2) DC_CUDA(launch_conv_kernel(k_conv_tc<2>, grid, threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
-    else DC_CUDA(launch_conv_kernel(k_conv_tc<1>, grid, threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
+    if (p.MT == 2) DC_CUDA(dc_launch_pdl(k_conv_tc<2>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
+    else DC_CUDA(dc_launch_pdl(k_conv_tc<1>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;

@@ -34,6 +34,8 @@ struct ConvArgs {
 template <typename T>
 __global__ void __launch_bounds__(DC_TILE_PX) k_conv_direct(ConvArgs a)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     __shared__ __align__(16) float wsm[MAX_KW * CI_T * CO_T];
     const T* in = (const T*)a.in; const T* wt = (const T*)a.w; T* out = (T*)a.out;
     const int tid = threadIdx.x, prow = tid / DC_TILE_W, pcol = tid % DC_TILE_W;
@@ -120,14 +122,17 @@ int dc_conv_bf16_supported(const dc_cache* c, int layer);
 int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                         const int32_t* tile_count, const uint32_t* masks, int max_tiles);
 
+// in == nullptr: the layer's operand copy (L.in_s2d or L.in_padded) has been filled already
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                    const int32_t* tile_count, const uint32_t* masks, int max_tiles)
 {
     dc_layer_rt& L = c->L[layer];
     if (L.s2d_s) {                                                // the rewritten layer reads the block map of its input
-        dc_prof_scope ps(c, DC_ST_CONV);
-        const int rc = dc_launch_s2d(c, layer, in);
-        if (rc != DC_OK) return rc;
+        if (in) {
+            dc_prof_scope ps(c, DC_ST_CONV);
+            const int rc = dc_launch_s2d(c, layer, in);
+            if (rc != DC_OK) return rc;
+        }
         in = L.in_s2d;
     }
     if (c->cfg.dtype == DC_BF16 && dc_conv_bf16_supported(c, layer))
@@ -148,8 +153,8 @@ int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int3
     if (gx > cap) gx = cap;
     dim3 grid(gx, co_groups);
     dc_prof_scope ps(c, DC_ST_CONV);
-    if (c->cfg.dtype == DC_BF16) k_conv_direct<__nv_bfloat16><<<grid, DC_TILE_PX, 0, c->stream>>>(a);
-    else k_conv_direct<float><<<grid, DC_TILE_PX, 0, c->stream>>>(a);
+    if (c->cfg.dtype == DC_BF16) DC_CUDA(dc_launch_pdl(k_conv_direct<__nv_bfloat16>, grid, DC_TILE_PX, 0, c->stream, a));
+    else DC_CUDA(dc_launch_pdl(k_conv_direct<float>, grid, DC_TILE_PX, 0, c->stream, a));
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;

@@ -31,6 +31,8 @@ struct S2dArgs {
 // One thread per 8 channels (16 bytes) of a block pixel.
 __global__ void k_space_to_depth(const S2dArgs a)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const int chunks = a.cs / 8;
     const size_t total = (size_t)a.S * a.Hs * a.Ws * chunks;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -130,8 +132,7 @@ int dc_launch_s2d(dc_cache* c, int layer, const void* in)
     a.Hs = L.in_h; a.Ws = L.in_w; a.cs = L.d.cin;
     const size_t total = (size_t)a.S * a.Hs * a.Ws * (a.cs / 8);
     int grid = (int)((total + 255) / 256); if (grid > c->num_sms * 16) grid = c->num_sms * 16;
-    k_space_to_depth<<<grid, 256, 0, c->stream>>>(a);
+    DC_CUDA(dc_launch_pdl(k_space_to_depth, dim3((unsigned)grid), 256, 0, c->stream, a));
     c->launches += 1;
-    DC_CUDA(cudaGetLastError());
     return DC_OK;
 }

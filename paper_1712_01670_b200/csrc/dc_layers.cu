@@ -12,57 +12,111 @@ template <typename T> __device__ __forceinline__ T from_f(float v);
 template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
-// round a double to bfloat16, nearest even, without passing through float
+// Round a double to bfloat16, nearest even: first to a float that keeps a trace of what was cut off in its last bit
+// (round to odd), so that the second rounding sees on which side of a tie the value lay.
 __device__ __forceinline__ __nv_bfloat16 double_to_bf16(double v)
 {
-    if (v == 0.0) return __float2bfloat16_rn(0.f);
-    int e = ilogb(v);
-    if (e < -126) e = -126;
-    double q = ldexp(rint(ldexp(v, 7 - e)), e - 7);   // exactly representable in bfloat16
-    return __float2bfloat16_rn((float)q);
+    float f = __double2float_rz(v);
+    if ((double)f != v) f = __uint_as_float(__float_as_uint(f) | 1u);
+    return __float2bfloat16_rn(f);
 }
 template <typename T> __device__ __forceinline__ T from_d(double v);
 template <> __device__ __forceinline__ float from_d<float>(double v) { return (float)v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_d<__nv_bfloat16>(double v) { return double_to_bf16(v); }
 
-// pixel value -> map element through a 256-entry table (pixel / 255 in the map's type)
+// pixel / 255 in the map's type.  bfloat16: the product with the float nearest to 1/255, rounded, is the correctly
+// rounded quotient for all 256 values; float: the division.
+template <typename T> __device__ __forceinline__ T from_pixel(uint32_t v);
+template <> __device__ __forceinline__ float from_pixel<float>(uint32_t v) { return __fdiv_rn((float)v, 255.f); }
+template <> __device__ __forceinline__ __nv_bfloat16 from_pixel<__nv_bfloat16>(uint32_t v) { return __float2bfloat16_rn((float)v * (1.f / 255.f)); }
+
+// Frame copy (rows 16-byte aligned) -> network input map: four values per thread, one aligned word of the row.
 template <typename T>
-__global__ void k_input_map(const uint8_t* frame, size_t pitch, int W, int H, int S, const T* lut, T* out)
+__global__ void __launch_bounds__(256) k_input_map(const uint8_t* frame, size_t pitch, int row_elems, int words, unsigned total, T* out)
 {
-    __shared__ T sl[256];
-    if (threadIdx.x < 256) sl[threadIdx.x] = lut[threadIdx.x];
-    __syncthreads();
-    const int row_elems = W * 3;
-    const size_t total = (size_t)S * H * row_elems;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        size_t row = i / row_elems; int x = (int)(i - row * row_elems);
-        out[i] = sl[frame[row * pitch + x]];
+    dc_pdl_wait();
+    dc_pdl_release();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned row = i / (unsigned)words, w = i - row * (unsigned)words;
+        const uint32_t v = __ldg((const uint32_t*)(frame + (size_t)row * pitch) + w);
+        T* o = out + (size_t)row * row_elems + 4 * w;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) if ((int)(4 * w) + k < row_elems) o[k] = from_pixel<T>((v >> (8 * k)) & 0xffu);
+    }
+}
+
+// Frame copy -> the first convolution's operand copies, without the input map in between (bfloat16 caches whose input
+// map nobody else reads).  k_frame_pad8: [S][H][W][8], three channels and five zeros, one pixel per thread.
+__global__ void __launch_bounds__(256) k_frame_pad8(const uint8_t* frame, size_t pitch, int W, unsigned total, uint4* out)
+{
+    dc_pdl_wait();
+    dc_pdl_release();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned row = i / (unsigned)W, x = i - row * (unsigned)W;
+        const uint32_t* q = (const uint32_t*)(frame + (size_t)row * pitch) + (3 * x >> 2);
+        const uint32_t v = __funnelshift_r(__ldg(q), __ldg(q + 1), (3 * x & 3) * 8);    // the copy's rows have spare bytes
+        const __nv_bfloat162 rg = __halves2bfloat162(from_pixel<__nv_bfloat16>(v & 0xffu), from_pixel<__nv_bfloat16>((v >> 8) & 0xffu));
+        const __nv_bfloat162 b0 = __halves2bfloat162(from_pixel<__nv_bfloat16>((v >> 16) & 0xffu), __float2bfloat16_rn(0.f));
+        out[i] = make_uint4(*(const uint32_t*)&rg, *(const uint32_t*)&b0, 0u, 0u);
+    }
+}
+// k_frame_s2d: the space-to-depth block map of dc_conv_s2d.cu.  Element e of a block pixel is byte e % (3 s) of the block's
+// row e / (3 s): within a block row the bytes are consecutive in the frame.  One thread per 8 elements.
+__global__ void __launch_bounds__(256) k_frame_s2d(const uint8_t* frame, size_t pitch, int W, int H, int bs, int Py, int Px, int Hs, int Ws, int chunks,
+                                                   unsigned total, uint4* out)
+{
+    dc_pdl_wait();
+    dc_pdl_release();
+    const int rb = 3 * bs;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned u = i / (unsigned)chunks, ch = i - u * (unsigned)chunks;
+        const unsigned r = u / (unsigned)Ws, bx = u - r * (unsigned)Ws, st = r / (unsigned)Hs, by = r - st * (unsigned)Hs;
+        const uint8_t* src = frame + (size_t)st * H * pitch;
+        const int x_byte = ((int)bx * bs - Px) * 3, y0 = (int)by * bs - Py;
+        __align__(16) __nv_bfloat16 v[8];
+        int dy = (int)(8 * ch) / rb, b = (int)(8 * ch) - dy * rb;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int iy = y0 + dy, xb = x_byte + b;
+            const bool on = dy < bs && iy >= 0 && iy < H && xb >= 0 && xb < 3 * W;
+            v[j] = on ? from_pixel<__nv_bfloat16>(__ldg(src + (size_t)iy * pitch + xb)) : __float2bfloat16_rn(0.f);
+            if (++b == rb) { b = 0; ++dy; }
+        }
+        out[i] = *(const uint4*)v;
     }
 }
 
 // Box average of the frame: output (oy, ox) is the mean over rows [floor(oy H / Ho),
 // ceil((oy + 1) H / Ho) - 1] and the like columns, divided by 255.  One CTA per output row:
 // pass 1 sums the span's source rows column-wise with coalesced 16-byte loads (row starts are
-// 16-byte aligned in the library's frame copy) into shared memory; pass 2 sums each output's
-// column span.  All sums are integers; the one division is done in double.
+// 16-byte aligned in the library's frame copy), six rows in flight, into shared memory; pass 2 sums each output
+// pixel's column span.  All sums are integers; the one division is done in double.  pad8 (or NULL): the pixel once more with
+// its channels padded to eight, for the few-channel convolution that follows.
 template <typename T>
 __global__ void __launch_bounds__(256) k_resize_area(const uint8_t* frame, size_t pitch, int W, int H, int S,
-                                                     int Wo, int Ho, T* out)
+                                                     int Wo, int Ho, T* out, uint4* pad8)
 {
     extern __shared__ uint16_t colsum[];                       // [ceil16(W * 3)]
+    dc_pdl_wait();
+    dc_pdl_release();
     const int oy = blockIdx.x % Ho, s = blockIdx.x / Ho;
     const int y0 = (int)((long long)oy * H / Ho), y1 = (int)(((long long)(oy + 1) * H + Ho - 1) / Ho) - 1;
-    const int row_bytes = W * 3, chunks = (row_bytes + 15) >> 4;
+    const int row_bytes = W * 3, chunks = (row_bytes + 15) >> 4, rows = y1 - y0 + 1;
     const uint8_t* base = frame + ((size_t)s * H + y0) * pitch;
     for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
         uint32_t acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};            // 16 byte columns as 8 pairs of 16-bit sums
-        for (int y = 0; y <= y1 - y0; ++y) {
-            const uint4 v = __ldg((const uint4*)(base + (size_t)y * pitch + c * 16));
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        for (int yb = 0; yb < rows; yb += 6) {
+            uint4 v[6];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                acc[2 * k] += __byte_perm(w[k], 0, 0x4140);    // bytes 0, 1 -> two 16-bit lanes
-                acc[2 * k + 1] += __byte_perm(w[k], 0, 0x4342);
+            for (int k = 0; k < 6; ++k) v[k] = yb + k < rows ? __ldg((const uint4*)(base + (size_t)(yb + k) * pitch + c * 16)) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[2 * j] += __byte_perm(w[j], 0, 0x4140);    // bytes 0, 1 -> two 16-bit lanes
+                    acc[2 * j + 1] += __byte_perm(w[j], 0, 0x4342);
+                }
             }
         }
         uint4* dst = (uint4*)(colsum + c * 16);
@@ -70,14 +124,21 @@ __global__ void __launch_bounds__(256) k_resize_area(const uint8_t* frame, size_
         dst[1] = make_uint4(acc[4], acc[5], acc[6], acc[7]);
     }
     __syncthreads();
-    const int rows = y1 - y0 + 1;
-    for (int t = threadIdx.x; t < Wo * 3; t += blockDim.x) {
-        const int ox = t / 3, ch = t - ox * 3;
+    for (int ox = threadIdx.x; ox < Wo; ox += blockDim.x) {
         const int x0 = (int)((long long)ox * W / Wo), x1 = (int)(((long long)(ox + 1) * W + Wo - 1) / Wo) - 1;
-        uint32_t sum = 0;
-        for (int x = x0; x <= x1; ++x) sum += colsum[x * 3 + ch];
-        const double mean = (double)sum / ((double)(rows * (x1 - x0 + 1)) * 255.0);
-        out[(((size_t)s * Ho + oy) * Wo + ox) * 3 + ch] = from_d<T>(mean);
+        uint32_t sum[3] = {0, 0, 0};
+        for (int x = x0; x <= x1; ++x) { sum[0] += colsum[x * 3]; sum[1] += colsum[x * 3 + 1]; sum[2] += colsum[x * 3 + 2]; }
+        const double div = (double)(rows * (x1 - x0 + 1)) * 255.0;
+        const size_t px = ((size_t)s * Ho + oy) * Wo + ox;
+        T v[3];
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) { v[ch] = from_d<T>((double)sum[ch] / div); out[px * 3 + ch] = v[ch]; }
+        if constexpr (sizeof(T) == 2) {
+            if (pad8) {
+                const __nv_bfloat162 rg = __halves2bfloat162(v[0], v[1]), b0 = __halves2bfloat162(v[2], __float2bfloat16_rn(0.f));
+                pad8[px] = make_uint4(*(const uint32_t*)&rg, *(const uint32_t*)&b0, 0u, 0u);
+            }
+        }
     }
 }
 
@@ -103,37 +164,54 @@ template <> struct Vec16<__nv_bfloat16> {
     static __device__ __forceinline__ uint4 vmax(uint4 a, uint4 b) { return make_uint4(m2(a.x, b.x), m2(a.y, b.y), m2(a.z, b.z), m2(a.w, b.w)); }
 };
 
-// masks (optional): the layer's per-tile reuse bitmaps; a pixel whose bit is set was filled from the cache
-template <typename T>
-__global__ void k_maxpool_vec(const T* in, int Hi, int Wi, int C, int S, dc_layer_desc L, T* out, const uint32_t* masks,
-                              int tiles_x, int tiles_y)
+// masks (optional): the layer's per-tile reuse bitmaps; a pixel whose bit is set was filled from the cache.
+// K x K windows with K known: the loads of an output vector are independent and travel together (a tap
+// outside the map is moved to the nearest row and column inside, whose tap is in the window too: the maximum is the same).  K = 0: any window, tap after tap.
+template <typename T, int K>
+__global__ void __launch_bounds__(256) k_maxpool_vec(const uint4* in, int Hi, int Wi, unsigned cv, dc_layer_desc L, unsigned total, uint4* out, const uint32_t* masks,
+                                                     int tiles_x, int tiles_y)
 {
-    constexpr int N = Vec16<T>::N;
-    const int cv = C / N;
-    const size_t total = (size_t)S * L.out_h * L.out_w * cv;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        int c = (int)(i % cv); size_t t = i / cv;
-        int ox = (int)(t % L.out_w); t /= L.out_w;
-        int oy = (int)(t % L.out_h); int s = (int)(t / L.out_h);
+    dc_pdl_wait();
+    dc_pdl_release();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned t = i / cv, c = i - t * cv, u = t / (unsigned)L.out_w;
+        const int ox = (int)(t - u * (unsigned)L.out_w);
+        const unsigned s = u / (unsigned)L.out_h;
+        const int oy = (int)(u - s * (unsigned)L.out_h);
         if (masks) {
             const size_t tile = ((size_t)s * tiles_y + oy / DC_TILE_H) * tiles_x + ox / DC_TILE_W;
             const int bit = DC_TILE_BIT(oy % DC_TILE_H, ox % DC_TILE_W);
             if ((masks[tile * 4 + (bit >> 5)] >> (bit & 31)) & 1u) continue;
         }
-        uint4 m = make_uint4(0, 0, 0, 0);
-        bool first = true;
-        for (int ky = 0; ky < L.kh; ++ky) {
-            int iy = oy * L.sh - L.ph + ky;
-            if (iy < 0 || iy >= Hi) continue;
-            for (int kx = 0; kx < L.kw; ++kx) {
-                int ix = ox * L.sw - L.pw + kx;
-                if (ix < 0 || ix >= Wi) continue;
-                uint4 v = __ldg((const uint4*)(in + (((size_t)s * Hi + iy) * Wi + ix) * C) + c);
-                m = first ? v : Vec16<T>::vmax(m, v);
-                first = false;
+        const int y0 = oy * L.sh - L.ph, x0 = ox * L.sw - L.pw;
+        const uint4* base = in + (size_t)s * Hi * Wi * cv + c;
+        uint4 m;
+        if constexpr (K > 0) {
+            uint4 v[K * K];
+#pragma unroll
+            for (int k = 0; k < K * K; ++k) {
+                const int y = min(max(y0 + k / K, max(y0, 0)), Hi - 1), x = min(max(x0 + k % K, max(x0, 0)), Wi - 1);
+                v[k] = __ldg(base + ((size_t)y * Wi + x) * cv);
+            }
+            m = v[0];
+#pragma unroll
+            for (int k = 1; k < K * K; ++k) m = Vec16<T>::vmax(m, v[k]);
+        } else {
+            bool first = true;
+            m = make_uint4(0, 0, 0, 0);
+            for (int ky = 0; ky < L.kh; ++ky) {
+                const int iy = y0 + ky;
+                if (iy < 0 || iy >= Hi) continue;
+                for (int kx = 0; kx < L.kw; ++kx) {
+                    const int ix = x0 + kx;
+                    if (ix < 0 || ix >= Wi) continue;
+                    const uint4 v = __ldg(base + ((size_t)iy * Wi + ix) * cv);
+                    m = first ? v : Vec16<T>::vmax(m, v);
+                    first = false;
+                }
             }
         }
-        *((uint4*)(out + i / cv * C) + c) = m;
+        out[i] = m;
     }
 }
 
@@ -142,6 +220,8 @@ __global__ void k_maxpool_vec(const T* in, int Hi, int Wi, int C, int S, dc_laye
 template <typename T>
 __global__ void k_maxpool2x2_vec(const uint4* in, int Hi, int Wi, int cv, int out_h, int out_w, unsigned total, uint4* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const unsigned c = i % cv, t = i / cv, ox = t % out_w, u = t / out_w, oy = u % out_h, s = u / out_h;
         const uint4* p = in + (((size_t)s * Hi + 2 * oy) * Wi + 2 * ox) * cv + c;
@@ -154,6 +234,8 @@ __global__ void k_maxpool2x2_vec(const uint4* in, int Hi, int Wi, int cv, int ou
 template <typename T>
 __global__ void k_maxpool(const T* in, int Hi, int Wi, int C, int S, dc_layer_desc L, T* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const size_t total = (size_t)S * L.out_h * L.out_w * C;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         int c = (int)(i % C); size_t t = i / C;
@@ -176,6 +258,8 @@ __global__ void k_maxpool(const T* in, int Hi, int Wi, int C, int S, dc_layer_de
 template <typename T>
 __global__ void k_add(const T* a, const T* b, size_t n, int relu, T* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         float v = to_f(a[i]) + to_f(b[i]);
         if (relu) v = fmaxf(v, 0.f);
@@ -186,6 +270,8 @@ __global__ void k_add(const T* a, const T* b, size_t n, int relu, T* out)
 template <typename T>
 __global__ void k_relu(const T* a, size_t n, T* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         out[i] = from_f<T>(fmaxf(to_f(a[i]), 0.f));
 }
@@ -221,6 +307,8 @@ template <> struct VecOps<__nv_bfloat16> {
 template <typename T>
 __global__ void k_add_vec(const uint4* a, const uint4* b, size_t nvec, int relu, uint4* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
         const uint4 va = __ldg(a + i), vb = b ? __ldg(b + i) : make_uint4(0, 0, 0, 0);
         out[i] = VecOps<T>::add(va, vb, relu);
@@ -233,6 +321,8 @@ template <typename T>
 __global__ void k_lrn(const T* in, int H, int W, int C, int S, int r, float alpha_n2, float beta, float kappa, T* out,
                       const uint32_t* masks, int tiles_x, int tiles_y)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const size_t total = (size_t)S * H * W * C;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int c = (int)(i % C); size_t t = i / C;
@@ -258,16 +348,108 @@ __global__ void k_lrn(const T* in, int H, int W, int C, int S, int r, float alph
     }
 }
 
+// The same for 16-byte vectors of channels, R known: the (2 R + 1)^2 loads of a vector are independent.  beta = 3/4 (the
+// default) takes two correctly rounded square roots and a division in place of powf, which dominated the kernel.
+template <typename T> struct Unpack;
+template <> struct Unpack<float> {
+    static __device__ __forceinline__ void get(uint4 v, float* f) { f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w); }
+    static __device__ __forceinline__ uint4 put(const float* f) { return make_uint4(__float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3])); }
+};
+template <> struct Unpack<__nv_bfloat16> {
+    static __device__ __forceinline__ void get(uint4 v, float* f)
+    {
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { f[2 * k] = __uint_as_float(w[k] << 16); f[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u); }
+    }
+    static __device__ __forceinline__ uint4 put(const float* f)
+    {
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { const __nv_bfloat162 p = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]); w[k] = *(const uint32_t*)&p; }
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+};
+
+template <typename T, int R>
+__global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, unsigned cv, float alpha_n2, float beta, float kappa, unsigned total, uint4* out,
+                                                 const uint32_t* masks, int tiles_x, int tiles_y)
+{
+    constexpr int N = Vec16<T>::N;
+    dc_pdl_wait();
+    dc_pdl_release();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned t = i / cv, c = i - t * cv, u = t / (unsigned)W, s = u / (unsigned)H;
+        const int x = (int)(t - u * (unsigned)W), y = (int)(u - s * (unsigned)H);
+        if (masks) {                                             // pixel filled from the cache
+            const size_t tile = ((size_t)s * tiles_y + y / DC_TILE_H) * tiles_x + x / DC_TILE_W;
+            const int bit = DC_TILE_BIT(y % DC_TILE_H, x % DC_TILE_W);
+            if ((masks[tile * 4 + (bit >> 5)] >> (bit & 31)) & 1u) continue;
+        }
+        const uint4* base = in + (size_t)s * H * W * cv + c;
+        float sum[N], mid[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) sum[k] = 0.f;
+#pragma unroll
+        for (int dy = -R; dy <= R; ++dy) {
+            uint4 v[2 * R + 1];
+#pragma unroll
+            for (int dx = -R; dx <= R; ++dx) {
+                const int yy = y + dy, xx = x + dx;
+                v[dx + R] = yy >= 0 && yy < H && xx >= 0 && xx < W ? __ldg(base + ((size_t)yy * W + xx) * cv) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int dx = 0; dx <= 2 * R; ++dx) {
+                float f[N];
+                Unpack<T>::get(v[dx], f);
+                if (dy == 0 && dx == R) {
+#pragma unroll
+                    for (int k = 0; k < N; ++k) mid[k] = f[k];
+                }
+#pragma unroll
+                for (int k = 0; k < N; ++k) sum[k] = fmaf(f[k], f[k], sum[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const float d = fmaf(alpha_n2, sum[k], kappa);
+            if (beta == 0.75f && d > 0.f) { const float r = __fsqrt_rn(d); mid[k] = __fdiv_rn(mid[k], r * __fsqrt_rn(r)); }
+            else mid[k] *= powf(d, -beta);
+        }
+        out[i] = Unpack<T>::put(mid);
+    }
+}
+
 // Channel concatenation of two NHWC maps
 template <typename T>
 __global__ void k_concat(const T* a, int Ca, const T* b, int Cb, size_t pixels, T* out)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const int C = Ca + Cb;
     const size_t total = pixels * C;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const int c = (int)(i % C); const size_t px = i / C;
         out[i] = c < Ca ? a[px * Ca + c] : b[px * Cb + (c - Ca)];
     }
+}
+// The same where both inputs' pixels are whole 16-byte vectors.
+__global__ void __launch_bounds__(256) k_concat_vec(const uint4* a, unsigned va, const uint4* b, unsigned vb, unsigned total, uint4* out)
+{
+    dc_pdl_wait();
+    dc_pdl_release();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned px = i / (va + vb), c = i - px * (va + vb);
+        out[i] = c < va ? __ldg(a + (size_t)px * va + c) : __ldg(b + (size_t)px * vb + (c - va));
+    }
+}
+
+// Plain copy of a map
+__global__ void __launch_bounds__(256) k_copy_vec(const uint4* a, unsigned total, uint4* out)
+{
+    dc_pdl_wait();
+    dc_pdl_release();
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) out[i] = __ldg(a + i);
 }
 
 inline int grid_for(const dc_cache* c, size_t n, int block)
@@ -280,134 +462,183 @@ inline int grid_for(const dc_cache* c, size_t n, int block)
 
 #define DISPATCH(c, expr_f32, expr_bf16) do { if ((c)->cfg.dtype == DC_BF16) { expr_bf16; } else { expr_f32; } } while (0)
 
+namespace {
+constexpr size_t k32Bit = 0x7fffffffull;                       // the vector kernels index with 32 bits
+}
+
 int dc_launch_input_map(dc_cache* c, const uint8_t* frame, size_t pitch)
 {
-    size_t n = (size_t)c->S * c->cfg.height * c->cfg.width * 3;
-    int W = c->cfg.width, H = c->cfg.height;
+    const int row = c->cfg.width * 3, words = (row + 3) / 4;
+    const size_t n = (size_t)c->S * c->cfg.height * words;
+    if (n > k32Bit) return DC_ERR_CONFIG;                       // 8 GB of pixels
+    const dim3 grid((unsigned)grid_for(c, n, 256));
     dc_prof_scope ps(c, DC_ST_INPUT);
     DISPATCH(c,
-        (k_input_map<float><<<grid_for(c, n, 256), 256, 0, c->stream>>>(frame, pitch, W, H, c->S, (const float*)c->pix_lut, (float*)c->input_map)),
-        (k_input_map<__nv_bfloat16><<<grid_for(c, n, 256), 256, 0, c->stream>>>(frame, pitch, W, H, c->S, (const __nv_bfloat16*)c->pix_lut, (__nv_bfloat16*)c->input_map)));
+        DC_CUDA(dc_launch_pdl(k_input_map<float>, grid, 256, 0, c->stream, frame, pitch, row, words, (unsigned)n, (float*)c->input_map)),
+        DC_CUDA(dc_launch_pdl(k_input_map<__nv_bfloat16>, grid, 256, 0, c->stream, frame, pitch, row, words, (unsigned)n, (__nv_bfloat16*)c->input_map)));
     c->launches += 1;
-    DC_CUDA(cudaGetLastError());
+    return DC_OK;
+}
+
+// The frame straight into the operand copy of convolution `layer` (dc_conv_takes_frame).
+int dc_launch_frame_operand(dc_cache* c, int layer, const uint8_t* frame, size_t pitch)
+{
+    dc_layer_rt& L = c->L[layer];
+    dc_prof_scope ps(c, DC_ST_INPUT);
+    if (L.s2d_s) {
+        const int chunks = L.d.cin / 8;
+        const size_t n = (size_t)c->S * L.in_h * L.in_w * chunks;
+        DC_CUDA(dc_launch_pdl(k_frame_s2d, dim3((unsigned)grid_for(c, n, 256)), 256, 0, c->stream, frame, pitch, L.s2d_wi, L.s2d_hi, L.s2d_s, L.s2d_py, L.s2d_px, L.in_h, L.in_w,
+                              chunks, (unsigned)n, (uint4*)L.in_s2d));
+    } else {
+        const size_t n = (size_t)c->S * L.in_h * L.in_w;
+        DC_CUDA(dc_launch_pdl(k_frame_pad8, dim3((unsigned)grid_for(c, n, 256)), 256, 0, c->stream, frame, pitch, L.in_w, (unsigned)n, (uint4*)L.in_padded));
+    }
+    c->launches += 1;
     return DC_OK;
 }
 
 int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch)
 {
     dc_layer_rt& L = c->L[layer];
-    int grid = c->S * L.d.out_h;
-    size_t smem = (size_t)((c->cfg.width * 3 + 15) / 16) * 16 * sizeof(uint16_t);
+    const dim3 grid((unsigned)(c->S * L.d.out_h));
+    const size_t smem = (size_t)((c->cfg.width * 3 + 15) / 16) * 16 * sizeof(uint16_t);
     if (smem > 48 * 1024 || (size_t)c->cfg.height > 255u * (size_t)L.d.out_h) return DC_ERR_CONFIG;   // 16-bit column sums
+    uint4* pad8 = c->resize_feeds >= 0 ? (uint4*)c->L[c->resize_feeds].in_padded : nullptr;
     dc_prof_scope ps(c, DC_ST_INPUT);
     DISPATCH(c,
-        (k_resize_area<float><<<grid, 256, smem, c->stream>>>(frame, pitch, c->cfg.width, c->cfg.height, c->S, L.d.out_w, L.d.out_h, (float*)L.map[0])),
-        (k_resize_area<__nv_bfloat16><<<grid, 256, smem, c->stream>>>(frame, pitch, c->cfg.width, c->cfg.height, c->S, L.d.out_w, L.d.out_h, (__nv_bfloat16*)L.map[0])));
+        DC_CUDA(dc_launch_pdl(k_resize_area<float>, grid, 256, smem, c->stream, frame, pitch, c->cfg.width, c->cfg.height, c->S, L.d.out_w, L.d.out_h, (float*)L.map[0], (uint4*)nullptr)),
+        DC_CUDA(dc_launch_pdl(k_resize_area<__nv_bfloat16>, grid, 256, smem, c->stream, frame, pitch, c->cfg.width, c->cfg.height, c->S, L.d.out_w, L.d.out_h, (__nv_bfloat16*)L.map[0], pad8)));
     c->launches += 1;
-    DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
 
 int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks)
 {
     dc_layer_rt& L = c->L[layer];
-    size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
+    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout, nv = n * c->elt / 16;
     dc_prof_scope ps(c, DC_ST_POINTWISE);
-    if ((L.d.cout * c->elt) % 16 == 0 && !masks && L.d.kh == 2 && L.d.kw == 2 && L.d.sh == 2 && L.d.sw == 2 && L.d.ph == 0 &&
-        L.d.pw == 0 && 2 * L.d.out_h <= L.in_h && 2 * L.d.out_w <= L.in_w && n * c->elt / 16 < 0x7fffffffull) {
-        const unsigned nv = (unsigned)(n * c->elt / 16);
+    c->launches += 1;
+    if ((L.d.cout * c->elt) % 16 == 0 && nv < k32Bit) {
         const int cv = L.d.cout * c->elt / 16;
-        DISPATCH(c,
-            (k_maxpool2x2_vec<float><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const uint4*)in, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, nv, (uint4*)out)),
-            (k_maxpool2x2_vec<__nv_bfloat16><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const uint4*)in, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, nv, (uint4*)out)));
-        c->launches += 1;
-        DC_CUDA(cudaGetLastError());
-        return DC_OK;
-    }
-    if ((L.d.cout * c->elt) % 16 == 0) {
-        size_t nv = n * c->elt / 16;
-        DISPATCH(c,
-            (k_maxpool_vec<float><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const float*)in, L.in_h, L.in_w, L.d.cout, c->S, L.d, (float*)out, masks, L.tiles_x, L.tiles_y)),
-            (k_maxpool_vec<__nv_bfloat16><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const __nv_bfloat16*)in, L.in_h, L.in_w, L.d.cout, c->S, L.d, (__nv_bfloat16*)out, masks, L.tiles_x, L.tiles_y)));
-        c->launches += 1;
-        DC_CUDA(cudaGetLastError());
+        const dim3 grid((unsigned)grid_for(c, nv, 256));
+        if (!masks && L.d.kh == 2 && L.d.kw == 2 && L.d.sh == 2 && L.d.sw == 2 && L.d.ph == 0 && L.d.pw == 0 && 2 * L.d.out_h <= L.in_h && 2 * L.d.out_w <= L.in_w) {
+            DISPATCH(c,
+                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<float>, grid, 256, 0, c->stream, (const uint4*)in, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, (uint4*)out)),
+                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)in, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, (uint4*)out)));
+            return DC_OK;
+        }
+#define DC_POOL(T, K) DC_CUDA(dc_launch_pdl(k_maxpool_vec<T, K>, grid, 256, 0, c->stream, (const uint4*)in, L.in_h, L.in_w, (unsigned)cv, L.d, (unsigned)nv, (uint4*)out, masks, L.tiles_x, L.tiles_y))
+        if (L.d.kh == 3 && L.d.kw == 3) DISPATCH(c, DC_POOL(float, 3), DC_POOL(__nv_bfloat16, 3));
+        else if (L.d.kh == 2 && L.d.kw == 2) DISPATCH(c, DC_POOL(float, 2), DC_POOL(__nv_bfloat16, 2));
+        else DISPATCH(c, DC_POOL(float, 0), DC_POOL(__nv_bfloat16, 0));
+#undef DC_POOL
         return DC_OK;
     }
     if (masks) return DC_ERR_STATE;                             // cached pooling needs 16-byte pixels (checked at creation)
+    const dim3 grid((unsigned)grid_for(c, n, 256));
     DISPATCH(c,
-        (k_maxpool<float><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const float*)in, L.in_h, L.in_w, L.d.cout, c->S, L.d, (float*)out)),
-        (k_maxpool<__nv_bfloat16><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const __nv_bfloat16*)in, L.in_h, L.in_w, L.d.cout, c->S, L.d, (__nv_bfloat16*)out)));
-    c->launches += 1;
-    DC_CUDA(cudaGetLastError());
+        DC_CUDA(dc_launch_pdl(k_maxpool<float>, grid, 256, 0, c->stream, (const float*)in, L.in_h, L.in_w, L.d.cout, c->S, L.d, (float*)out)),
+        DC_CUDA(dc_launch_pdl(k_maxpool<__nv_bfloat16>, grid, 256, 0, c->stream, (const __nv_bfloat16*)in, L.in_h, L.in_w, L.d.cout, c->S, L.d, (__nv_bfloat16*)out)));
     return DC_OK;
 }
 
 int dc_launch_add(dc_cache* c, int layer, const void* a, const void* b)
 {
     dc_layer_rt& L = c->L[layer];
-    size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
+    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
     dc_prof_scope ps(c, DC_ST_POINTWISE);
+    c->launches += 1;
     if ((n * c->elt) % 16 == 0) {                                 // maps come from cudaMalloc: 256-byte aligned
         const size_t nv = n * c->elt / 16;
+        const dim3 grid((unsigned)grid_for(c, nv, 256));
         DISPATCH(c,
-            (k_add_vec<float><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0])),
-            (k_add_vec<__nv_bfloat16><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0])));
+            DC_CUDA(dc_launch_pdl(k_add_vec<float>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0])),
+            DC_CUDA(dc_launch_pdl(k_add_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0])));
     } else {
+        const dim3 grid((unsigned)grid_for(c, n, 256));
         DISPATCH(c,
-            (k_add<float><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const float*)a, (const float*)b, n, L.d.relu, (float*)L.map[0])),
-            (k_add<__nv_bfloat16><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const __nv_bfloat16*)a, (const __nv_bfloat16*)b, n, L.d.relu, (__nv_bfloat16*)L.map[0])));
+            DC_CUDA(dc_launch_pdl(k_add<float>, grid, 256, 0, c->stream, (const float*)a, (const float*)b, n, L.d.relu, (float*)L.map[0])),
+            DC_CUDA(dc_launch_pdl(k_add<__nv_bfloat16>, grid, 256, 0, c->stream, (const __nv_bfloat16*)a, (const __nv_bfloat16*)b, n, L.d.relu, (__nv_bfloat16*)L.map[0])));
     }
-    c->launches += 1;
-    DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
 
 int dc_launch_relu(dc_cache* c, int layer, const void* a)
 {
     dc_layer_rt& L = c->L[layer];
-    size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
+    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
     dc_prof_scope ps(c, DC_ST_POINTWISE);
+    c->launches += 1;
     if ((n * c->elt) % 16 == 0) {
         const size_t nv = n * c->elt / 16;
+        const dim3 grid((unsigned)grid_for(c, nv, 256));
         DISPATCH(c,
-            (k_add_vec<float><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const uint4*)a, nullptr, nv, 1, (uint4*)L.map[0])),
-            (k_add_vec<__nv_bfloat16><<<grid_for(c, nv, 256), 256, 0, c->stream>>>((const uint4*)a, nullptr, nv, 1, (uint4*)L.map[0])));
+            DC_CUDA(dc_launch_pdl(k_add_vec<float>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)nullptr, nv, 1, (uint4*)L.map[0])),
+            DC_CUDA(dc_launch_pdl(k_add_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)nullptr, nv, 1, (uint4*)L.map[0])));
     } else {
+        const dim3 grid((unsigned)grid_for(c, n, 256));
         DISPATCH(c,
-            (k_relu<float><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const float*)a, n, (float*)L.map[0])),
-            (k_relu<__nv_bfloat16><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const __nv_bfloat16*)a, n, (__nv_bfloat16*)L.map[0])));
+            DC_CUDA(dc_launch_pdl(k_relu<float>, grid, 256, 0, c->stream, (const float*)a, n, (float*)L.map[0])),
+            DC_CUDA(dc_launch_pdl(k_relu<__nv_bfloat16>, grid, 256, 0, c->stream, (const __nv_bfloat16*)a, n, (__nv_bfloat16*)L.map[0])));
     }
-    c->launches += 1;
-    DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
 
 int dc_launch_lrn(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks)
 {
     dc_layer_rt& L = c->L[layer];
-    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
+    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout, nv = n * c->elt / 16;
     const int r = L.d.ph, win = 2 * r + 1;
     const bool defaults = c->cfg.lrn_alpha == 0.0 && c->cfg.lrn_beta == 0.0 && c->cfg.lrn_k == 0.0;
     const float alpha = (float)(defaults ? 1e-4 : c->cfg.lrn_alpha), beta = (float)(defaults ? 0.75 : c->cfg.lrn_beta);
-    const float kappa = (float)(defaults ? 1.0 : c->cfg.lrn_k);
+    const float kappa = (float)(defaults ? 1.0 : c->cfg.lrn_k), an = alpha / (win * win);
     dc_prof_scope ps(c, DC_ST_POINTWISE);
-    DISPATCH(c,
-        (k_lrn<float><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const float*)in, L.d.out_h, L.d.out_w, L.d.cout, c->S, r, alpha / (win * win), beta, kappa, (float*)out, masks, L.tiles_x, L.tiles_y)),
-        (k_lrn<__nv_bfloat16><<<grid_for(c, n, 256), 256, 0, c->stream>>>((const __nv_bfloat16*)in, L.d.out_h, L.d.out_w, L.d.cout, c->S, r, alpha / (win * win), beta, kappa, (__nv_bfloat16*)out, masks, L.tiles_x, L.tiles_y)));
     c->launches += 1;
-    DC_CUDA(cudaGetLastError());
+    if ((L.d.cout * c->elt) % 16 == 0 && nv < k32Bit && (r == 1 || r == 2)) {
+        const dim3 grid((unsigned)grid_for(c, nv, 256));
+        const unsigned cv = (unsigned)(L.d.cout * c->elt / 16);
+#define DC_LRN_VEC(T, R) DC_CUDA(dc_launch_pdl(k_lrn_vec<T, R>, grid, 256, 0, c->stream, (const uint4*)in, L.d.out_h, L.d.out_w, cv, an, beta, kappa, (unsigned)nv, (uint4*)out, masks, L.tiles_x, L.tiles_y))
+        if (r == 1) DISPATCH(c, DC_LRN_VEC(float, 1), DC_LRN_VEC(__nv_bfloat16, 1));
+        else DISPATCH(c, DC_LRN_VEC(float, 2), DC_LRN_VEC(__nv_bfloat16, 2));
+#undef DC_LRN_VEC
+        return DC_OK;
+    }
+    const dim3 grid((unsigned)grid_for(c, n, 256));
+    DISPATCH(c,
+        DC_CUDA(dc_launch_pdl(k_lrn<float>, grid, 256, 0, c->stream, (const float*)in, L.d.out_h, L.d.out_w, L.d.cout, c->S, r, an, beta, kappa, (float*)out, masks, L.tiles_x, L.tiles_y)),
+        DC_CUDA(dc_launch_pdl(k_lrn<__nv_bfloat16>, grid, 256, 0, c->stream, (const __nv_bfloat16*)in, L.d.out_h, L.d.out_w, L.d.cout, c->S, r, an, beta, kappa, (__nv_bfloat16*)out, masks, L.tiles_x, L.tiles_y)));
     return DC_OK;
 }
 
 int dc_launch_concat(dc_cache* c, int layer, const void* a, int ca, const void* b, int cb)
 {
     dc_layer_rt& L = c->L[layer];
-    const size_t pixels = (size_t)c->S * L.d.out_h * L.d.out_w;
+    const size_t pixels = (size_t)c->S * L.d.out_h * L.d.out_w, nv = pixels * L.d.cout * c->elt / 16;
     dc_prof_scope ps(c, DC_ST_POINTWISE);
-    DISPATCH(c,
-        (k_concat<float><<<grid_for(c, pixels * L.d.cout, 256), 256, 0, c->stream>>>((const float*)a, ca, (const float*)b, cb, pixels, (float*)L.map[0])),
-        (k_concat<__nv_bfloat16><<<grid_for(c, pixels * L.d.cout, 256), 256, 0, c->stream>>>((const __nv_bfloat16*)a, ca, (const __nv_bfloat16*)b, cb, pixels, (__nv_bfloat16*)L.map[0])));
     c->launches += 1;
-    DC_CUDA(cudaGetLastError());
+    if ((ca * c->elt) % 16 == 0 && (cb * c->elt) % 16 == 0 && nv < k32Bit) {
+        DC_CUDA(dc_launch_pdl(k_concat_vec, dim3((unsigned)grid_for(c, nv, 256)), 256, 0, c->stream, (const uint4*)a, (unsigned)(ca * c->elt / 16), (const uint4*)b,
+                              (unsigned)(cb * c->elt / 16), (unsigned)nv, (uint4*)L.map[0]));
+        return DC_OK;
+    }
+    const dim3 grid((unsigned)grid_for(c, pixels * L.d.cout, 256));
+    DISPATCH(c,
+        DC_CUDA(dc_launch_pdl(k_concat<float>, grid, 256, 0, c->stream, (const float*)a, ca, (const float*)b, cb, pixels, (float*)L.map[0])),
+        DC_CUDA(dc_launch_pdl(k_concat<__nv_bfloat16>, grid, 256, 0, c->stream, (const __nv_bfloat16*)a, ca, (const __nv_bfloat16*)b, cb, pixels, (__nv_bfloat16*)L.map[0])));
+    return DC_OK;
+}
+
+// A map into a caller's buffer: by a kernel where both are 16-byte aligned, so that it joins the chain of kernels before it
+// without the gap of a copy node.
+int dc_launch_copy_map(dc_cache* c, const void* src, void* dst, size_t bytes)
+{
+    if (bytes % 16 == 0 && (uintptr_t)dst % 16 == 0 && bytes / 16 < k32Bit) {
+        const size_t nv = bytes / 16;
+        DC_CUDA(dc_launch_pdl(k_copy_vec, dim3((unsigned)grid_for(c, nv, 256)), 256, 0, c->stream, (const uint4*)src, (unsigned)nv, (uint4*)dst));
+        c->launches += 1;
+        return DC_OK;
+    }
+    DC_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, c->stream));
     return DC_OK;
 }

@@ -12,7 +12,7 @@
 //              covers the whole reach of the search.
 //   k_verify   Steps 3-4: rounds the mean vector M, scores every block at M (reusing the Step 2
 //              score when the block's own best vector is M); k_verify16_prep / k_verify16_list for 16-pixel blocks.
-//   k_merge_runs, k_merge   Step 5: maximal horizontal runs per block row, merged vertically when the
+//   k_merge    Step 5: maximal horizontal runs per block row, merged vertically when the
 //              spans are identical, emitted in (y, x) order by a CTA-wide ordered compaction.
 #include "dc_common.cuh"
 #include "dc_search_win.cuh"
@@ -139,6 +139,8 @@ __device__ __forceinline__ int round_mean(int sum, int n)
 // the PSNR test of Step 2.  One thread per block.  The global vector is still reported.
 __global__ void k_accept_own(MatchArgs a)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const int per = a.Gx * a.Gy;
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= per * a.S) return;
@@ -159,6 +161,8 @@ __global__ void k_accept_own(MatchArgs a)
 template <int ITERS>
 __global__ void __launch_bounds__(WARPS * 32) k_verify(MatchArgs a)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     __shared__ uint32_t sm_all[WARPS][32 * MAX_ROW_WORDS];
     BlockCtx<ITERS> c; int s, b;
     if (!load_block<ITERS>(a, sm_all[threadIdx.x >> 5], c, s, b)) return;
@@ -180,56 +184,56 @@ __global__ void __launch_bounds__(WARPS * 32) k_verify(MatchArgs a)
     }
 }
 
-// Step 5, part 1: for every block that starts a maximal horizontal run of matched blocks, the column
-// where the run ends; 0 for every other block (an end is never 0).  One thread per block; the forward
-// scan of a run start stays inside one row of bytes (cache hits after the first touch).
-__global__ void k_merge_runs(const uint8_t* matched, const int16_t* mv, int Gx, int total, uint16_t* run_end)
+// Step 5: maximal horizontal runs of matched blocks per block row; a run continues the rectangle above it only when the
+// run directly above starts and ends at the same columns; every other run heads a rectangle that extends down while
+// that holds.  One CTA per stream; heads are emitted in (y, x) order by a CTA-wide ordered compaction.
+// In per-block mode (mv != nullptr) neighbours of a run, the run above and the runs below must also carry the same
+// vector, and the rectangle's source is displaced by that vector instead of the global one.
+// The end column of the run starting at each block (0 for every other block: an end is never 0), and the vectors, lie in
+// shared memory when they fit (else in run_end): the scans along a row and down a column are chains of dependent
+// loads, and they set the time (full-HD frames: 31 + 10 us with the runs in global memory and a launch of their own).
+__global__ void __launch_bounds__(1024) k_merge(const uint8_t* matched, const int16_t* mv, const int32_t* gmv, int W, int H, int B,
+                                                int Gx, int Gy, int max_regions, uint16_t* run_end, int in_smem, dc_region* regions,
+                                                int32_t* n_regions, int32_t* status, int32_t* gmv_out, int32_t* n_out, dc_region* regions_out)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= total) return;
-    const int c = b % Gx;
-    uint16_t e = 0;
-    if (mv == nullptr) {
-        if (matched[b] && (c == 0 || !matched[b - 1])) {
-            int j = c + 1;
-            while (j < Gx && matched[b - c + j]) ++j;
-            e = (uint16_t)j;
-        }
-    } else if (matched[b]) {
-        // per-block mode: a run also ends where the vector changes
-        const uint32_t* v = (const uint32_t*)mv;                  // (dx, dy) as one word
-        const uint32_t mine = v[b];
-        if (c == 0 || !matched[b - 1] || v[b - 1] != mine) {
-            int j = c + 1;
-            while (j < Gx && matched[b - c + j] && v[b - c + j] == mine) ++j;
-            e = (uint16_t)j;
-        }
-    }
-    run_end[b] = e;
-}
-
-// Step 5, part 2: a run continues the rectangle above it only when the run directly above starts and
-// ends at the same columns; every other run heads a rectangle that extends down while that holds.
-// One CTA per stream; heads are emitted in (y, x) order by a CTA-wide ordered compaction.
-// In per-block mode (mv != nullptr) the run above, and the runs below, must also carry the same vector,
-// and the rectangle's source is displaced by that vector instead of the global one.
-__global__ void __launch_bounds__(1024) k_merge(const uint16_t* run_end, const int16_t* mv, const int32_t* gmv, int W, int H, int B,
-                                                int Gx, int Gy, int max_regions, dc_region* regions,
-                                                int32_t* n_regions, int32_t* status)
-{
+    extern __shared__ __align__(16) uint8_t merge_smem[];
     __shared__ int warp_sums[32];
-    __shared__ int base;
-    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const uint16_t* e = run_end + (size_t)s * Gx * Gy;
-    const uint32_t* v = mv ? (const uint32_t*)mv + (size_t)s * Gx * Gy : nullptr;
-    dc_region* out = regions + (size_t)s * max_regions;
-    int Mx = gmv[3 * s], My = gmv[3 * s + 1];
-    if (tid == 0) base = 0;
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, n = Gx * Gy;
+    dc_pdl_wait();
+    dc_pdl_release();
+    const uint8_t* m = matched + (size_t)s * n;
+    const uint32_t* v = mv ? (const uint32_t*)mv + (size_t)s * n : nullptr;              // (dx, dy) as one word
+    uint16_t* e = in_smem ? (uint16_t*)(merge_smem + (mv ? (size_t)n * 4 : 0)) : run_end + (size_t)s * n;
+    if (in_smem) {
+        if (mv) {
+            uint32_t* vs = (uint32_t*)merge_smem;
+            for (int i = tid; i < n; i += 1024) vs[i] = v[i];
+            v = vs;
+        }
+        uint8_t* ms = (uint8_t*)(e + n);
+        for (int i = tid; i < n; i += 1024) ms[i] = m[i];
+        m = ms;
+        __syncthreads();
+    }
+    for (int b = tid; b < n; b += 1024) {
+        const int c = b % Gx;
+        int end = 0;
+        if (m[b] && (c == 0 || !m[b - 1] || (v && v[b - 1] != v[b]))) {
+            end = c + 1;
+            const uint8_t* row = m + (b - c);
+            while (end < Gx && row[end] && (!v || v[b - c + end] == v[b])) ++end;
+        }
+        e[b] = (uint16_t)end;
+    }
     __syncthreads();
-    for (int start = 0; start < Gx * Gy; start += 1024) {
+    dc_region* out = regions + (size_t)s * max_regions;
+    dc_region* user = regions_out ? regions_out + (size_t)s * max_regions : nullptr;
+    int Mx = gmv[3 * s], My = gmv[3 * s + 1];
+    int base = 0;                                                     // rectangles emitted so far, the same in all threads
+    for (int start = 0; start < n; start += 1024) {
         const int b = start + tid;
         int head = 0, c1 = 0, h = 0, r = 0, c0 = 0;
-        if (b < Gx * Gy) {
+        if (b < n) {
             r = b / Gx; c0 = b - r * Gx;
             c1 = e[b];
             if (c1 != 0 && !(r > 0 && e[b - Gx] == c1 && (!v || v[b - Gx] == v[b]))) {
@@ -242,25 +246,29 @@ __global__ void __launch_bounds__(1024) k_merge(const uint16_t* run_end, const i
         const int pre = __popc(bal & ((1u << lane) - 1u));
         if (lane == 0) warp_sums[wid] = __popc(bal);
         __syncthreads();
-        int woff = 0, total = 0;
-        for (int i = 0; i < 32; ++i) { const int v = warp_sums[i]; if (i < wid) woff += v; total += v; }
+        const int mine = warp_sums[lane];
+        const int woff = __reduce_add_sync(0xffffffffu, lane < wid ? mine : 0), total = __reduce_add_sync(0xffffffffu, mine);
         const int idx = base + woff + pre;
         if (head) {
             if (idx < max_regions) {
                 const int x = c0 * B, y = r * B;
                 const int x1 = min(c1 * B, W), y1 = min((r + h) * B, H);
-                if (mv) { Mx = mv[2 * ((size_t)s * Gx * Gy + b)]; My = mv[2 * ((size_t)s * Gx * Gy + b) + 1]; }
+                if (v) { const uint32_t own = v[b]; Mx = (int16_t)(own & 0xffffu); My = (int16_t)(own >> 16); }
                 dc_region g = { x, y, x1 - x, y1 - y, x + Mx, y + My };
                 out[idx] = g;
+                if (user) user[idx] = g;
             } else {
                 atomicExch(status, (int)DC_ERR_OVERFLOW);
             }
         }
-        __syncthreads();
-        if (tid == 0) base += total;
-        __syncthreads();
+        base += total;
+        __syncthreads();                                              // warp_sums is free again
     }
-    if (tid == 0) n_regions[s] = min(base, max_regions);
+    if (tid == 0) {
+        n_regions[s] = min(base, max_regions);
+        if (n_out) n_out[s] = min(base, max_regions);
+    }
+    if (gmv_out && tid < 3) gmv_out[3 * s + tid] = gmv[3 * s + tid];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -484,26 +492,7 @@ __device__ __forceinline__ uint32_t lds_at(uint32_t p)
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(p), "n"(OFF) : "memory");
     return v;
 }
-__device__ __forceinline__ uint32_t score_at(uint32_t p, const uint32_t (&cw)[8], bool row_on)
-{
-    const uint32_t w0 = lds_at<0>(p), w1 = lds_at<8>(p), w2 = lds_at<16>(p), w3 = lds_at<24>(p);
-    const uint32_t w4 = lds_at<32>(p), w5 = lds_at<40>(p), w6 = lds_at<48>(p), w7 = lds_at<56>(p);
-    uint32_t a0 = 0, a1 = 0, d;
-    d = __vabsdiffu4(cw[0], w0); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[1], w1); a1 = __dp4a(d, d, a1);
-    d = __vabsdiffu4(cw[2], w2); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[3], w3); a1 = __dp4a(d, d, a1);
-    d = __vabsdiffu4(cw[4], w4); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[5], w5); a1 = __dp4a(d, d, a1);
-    d = __vabsdiffu4(cw[6], w6); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[7], w7); a1 = __dp4a(d, d, a1);
-    const uint32_t mine = row_on ? a0 + a1 : 0u;
-    uint32_t sum;
-    asm volatile("redux.sync.add.u32 %0, %1, 0xffffffff;" : "=r"(sum) : "r"(mine));
-    return sum;
-}
-
-// The same with the candidate's offset from p known at compile time: the eight loads need no address arithmetic.
+// The candidate's offset from p is known at compile time: the eight loads need no address arithmetic.
 template <int OFF>
 __device__ __forceinline__ uint32_t score_at_fixed(uint32_t p, const uint32_t (&cw)[8], bool row_on)
 {
@@ -561,12 +550,33 @@ struct WalkW {
     int nx, ny; uint32_t ns;    // on return 2: the centre the walk has chosen and not yet moved to, and its SSE
 };
 
+// Three points of such a round at a time, their loads in flight together; n_px: how many of the lane's eight pixels lie
+// inside the frame (fewer than eight for the last block column of a width that is not a multiple of 16).
+struct Edge3 { uint32_t s[3]; };
+__device__ __forceinline__ Edge3 score3(const uint32_t (&p)[3], const uint32_t (&cw)[8], bool row_on, int n_px)
+{
+    uint32_t acc[3] = {0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            uint32_t w;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(p[k] + 8u * j) : "memory");
+            const uint32_t d = j < n_px ? __vabsdiffu4(cw[j], w) : 0u;
+            acc[k] = __dp4a(d, d, acc[k]);
+        }
+    Edge3 r;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r.s[k] = __reduce_add_sync(0xffffffffu, row_on ? acc[k] : 0u);
+    return r;
+}
+
 //   lane_base  shared-memory address of this lane's first word of the candidate at displacement (0, 0);
 //              (dx, dy) is at lane_base + (dy * PITCH + dx) * 4
 //   reach(x, y)  true when every point around centre (x, y) is staged
 // Returns 1 when the walk has finished (result: w.cx, w.cy, w.bs), 2 when the next centre is out of reach.
 template <int PITCH, typename Reach>
-__device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base, const uint32_t (&cw)[8], bool row_on,
+__device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base, const uint32_t (&cw)[8], bool row_on, int n_px, bool clipped,
                                          const WalkBounds& wb, WalkW& w, const Reach& reach)
 {
     static __constant__ int c_points[13] = DC_POINT_ROW(PITCH);
@@ -574,11 +584,11 @@ __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base,
     // all 13 points valid  <=>  cx in [dx_lo + 2, dx_hi - 2] and cy likewise: one unsigned compare per axis
     const int ix_lo = wb.dx_lo + 2, iy_lo = wb.dy_lo + 2;
     const unsigned ix_span = (unsigned)max(wb.dx_hi - 2 - ix_lo, -1), iy_span = (unsigned)max(wb.dy_hi - 2 - iy_lo, -1);
+    const bool roomy = !clipped && wb.dx_hi - 2 >= ix_lo && wb.dy_hi - 2 >= iy_lo;
     uint32_t pc = lane_base + (uint32_t)((w.cy * PITCH + w.cx) * 4);
 #pragma unroll 1
     for (int move = 0;; ++move) {
-        const bool interior = wb.dx_hi - 2 >= ix_lo && wb.dy_hi - 2 >= iy_lo &&
-                              (unsigned)(w.cx - ix_lo) <= ix_span && (unsigned)(w.cy - iy_lo) <= iy_span;
+        const bool interior = roomy && (unsigned)(w.cx - ix_lo) <= ix_span && (unsigned)(w.cy - iy_lo) <= iy_span;
         uint32_t ms = 0xffffffffu; int mi = 8; bool tie = !interior;
         if (interior) {
             switch (w.kind) {
@@ -600,18 +610,26 @@ __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base,
         if (!tie) {
             if (ms < w.bs) { ns = ms; nx = w.cx + c_point_x[mi]; ny = w.cy + c_point_y[mi]; }
         } else {
-            // the exact order, point by point
+            // the exact order
             uint32_t m = c_kind_mask[w.kind] & valid_points(w.cx, w.cy, wb);
             uint32_t bt = w.kind == KIND_FIRST ? 0xffffffffu : tie_key(w.cx, w.cy);
             const uint32_t kc = ((uint32_t)(w.cy + 128) << 8) | (uint32_t)(w.cx + 128);  // low half of the centre's tie key
 #pragma unroll 1
-            while (m) {                                           // one candidate per turn; m is the same in all lanes
-                const int i = __ffs(m) - 1;
-                m &= m - 1;
-                const int pw = c_points[i];
-                const uint32_t s = score_at(pc + (uint32_t)(pw >> 16), cw, row_on);
-                if (s <= ns) {
-                    const uint32_t lo = (kc + (uint32_t)pw) & 0xffffu;               // ((dy + 128) << 8) | (dx + 128)
+            while (m) {                                           // three candidates per turn; m is the same in all lanes
+                int pw[3]; uint32_t p[3]; bool on[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    on[k] = m != 0;
+                    pw[k] = on[k] ? c_points[__ffs(m) - 1] : 0;   // none left: the centre once more, ignored
+                    p[k] = pc + (uint32_t)(pw[k] >> 16);
+                    m &= m - 1;
+                }
+                const Edge3 e = score3(p, cw, row_on, n_px);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const uint32_t s = e.s[k];
+                    if (!on[k] || s > ns) continue;
+                    const uint32_t lo = (kc + (uint32_t)pw[k]) & 0xffffu;            // ((dy + 128) << 8) | (dx + 128)
                     const int dx = (int)(lo & 0xff) - 128, dy = (int)(lo >> 8) - 128;
                     const uint32_t kt = ((uint32_t)(abs(dx) + abs(dy)) << 16) | lo;
                     if (s < ns || kt < bt) { ns = s; bt = kt; nx = dx; ny = dy; }
@@ -632,11 +650,13 @@ __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base,
         w.cx = nx; w.cy = ny; w.bs = ns;
     }
 }
+// how many of a lane's pixels h, h + 2, ... of a block row of bw pixels exist
+__device__ __forceinline__ int lane_pixel_count(int bw, int h) { return (bw - h + 1) >> 1; }
 
 // Phase 1: one CTA per 8 x W_VS blocks, one warp per block.  The window reaches W_WRY rows above and below the tile
 // and 12 pixels to its left and right (its left edge stays a multiple of 4 pixels, so that 4 pixels are 12 aligned
-// bytes of the packed frame).  A walk whose next centre is out of reach is handed to phase 2.  Blocks clipped in
-// width are left to the generic kernel.  Launched without k-skip only (every block is searched).
+// bytes of the packed frame).  A walk whose next centre is out of reach is handed to phase 2.  Launched without k-skip
+// only (every block is searched).
 constexpr int W_VS = 2, W_WRY = 10, W_SIDE = 12;
 constexpr int W_COLS = 128 + 2 * W_SIDE;                    // staged pixels per window row
 constexpr int W_PITCH = 154;                                // words per window row
@@ -649,6 +669,8 @@ struct TileReach {
 
 __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, uint4* long_list, int32_t* long_count)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     constexpr int THREADS = W_VS * 8 * 32, GROUPS = W_COLS / 4;
     constexpr int ROWS_PER_PASS = THREADS / GROUPS, PASSES = (W_ROWS + ROWS_PER_PASS - 1) / ROWS_PER_PASS;
     __shared__ __align__(16) uint32_t win[W_ROWS * W_PITCH];
@@ -658,8 +680,8 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
     const int by = vg * W_VS + (warp >> 3), bx = strip * 8 + (warp & 7);
     const int x0 = bx * 16, y0 = by * 16;
-    const bool searched = bx < a.Gx && by < a.Gy && a.W - x0 >= 16;
-    const int bh = searched ? min(16, a.H - y0) : 0;
+    const bool searched = bx < a.Gx && by < a.Gy;
+    const int bh = searched ? min(16, a.H - y0) : 0, bw = min(16, a.W - x0);
     const bool row_on = r < bh;
     uint32_t cw[8];                                            // issued first: in flight while the window is staged
     load_lane_pixels(a.cur + (size_t)s * a.cur_stream + (size_t)(row_on ? y0 + r : 0) * a.cur_pitch + (size_t)(row_on ? x0 : 0) * 3,
@@ -689,15 +711,15 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
     __syncthreads();
     const size_t g = (size_t)s * a.Gx * a.Gy + (size_t)by * a.Gx + bx;
     if (searched) {
-        const WalkBounds wb = walk_bounds(a, x0, y0, 16, bh);
+        const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
         const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(win) +
                                    (uint32_t)((((warp >> 3) * 16 + r + W_WRY) * W_PITCH + (x0 - xs + W_SIDE) + h) * 4);
         WalkW w = {0, 0, KIND_FIRST, 0xffffffffu, 0, 0, 0u};
-        const int st = warp_walk<W_PITCH>(a, lane_base, cw, row_on, wb, w, TileReach());
+        const int st = warp_walk<W_PITCH>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, wb, w, TileReach());
         if (lane == 0) {
             if (st == 1) {
                 a.mv[2 * g] = (int16_t)w.cx; a.mv[2 * g + 1] = (int16_t)w.cy; a.sse[g] = w.bs;
-                if (w.bs <= a.limit[limit_index(a, 16, bh)]) {        // PSNR > T: member of Step 3's set S
+                if (w.bs <= a.limit[limit_index(a, bw, bh)]) {        // PSNR > T: member of Step 3's set S
                     atomicAdd(&sums[0], w.cx); atomicAdd(&sums[1], w.cy); atomicAdd(&sums[2], 1);
                 }
             } else {                                                  // block, chosen next centre, its SSE, centre it was found from
@@ -771,6 +793,8 @@ struct StackWinR {
 template <int LPB, int VS>
 __global__ void __launch_bounds__(LPB * 8 * VS) k_search_tss16q(MatchArgs a, int s0, int wr, int words, int pitch)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     extern __shared__ uint32_t tss_win[];
     constexpr int THREADS = LPB * 8 * VS;
     const int rows = 16 * VS + 2 * wr, cpr = words / 4, chunks = rows * cpr;
@@ -845,6 +869,8 @@ static size_t tss_window_bytes(int R)
 // Section 4, k-skip: blocks that are not searched report vector (0, 0) and SSE 2^32 - 1.  One thread per block.
 __global__ void k_mark_unsearched(MatchArgs a)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const int gi = blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= a.S * a.Gx * a.Gy) return;
     const int b = gi % (a.Gx * a.Gy), by = b / a.Gx, bx = b - by * a.Gx;
@@ -856,7 +882,7 @@ __global__ void k_mark_unsearched(MatchArgs a)
 // centre whenever that is out of reach.  A continued walk makes exactly the move it had chosen (new points only),
 // so the sequence of scored candidates is the uninterrupted walk's.
 // With k-skip (Section 4) the searched blocks lie k blocks apart and share no window: there is no phase 1 then,
-// and this kernel walks every searched full-width block from its start (long_list == nullptr; item i is the
+// and this kernel walks every searched block from its start (long_list == nullptr; item i is the
 // i-th searched block in stream / row / column order).
 constexpr int P_WARPS = 8;
 constexpr int P_REACH = 8;                                  // staged pixels above and left of the block at the window's centre
@@ -870,12 +896,14 @@ struct PrivateReach {
 
 __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a, const uint4* long_list, const int32_t* long_count, int32_t* cursor)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     __shared__ __align__(16) uint32_t win_all[P_WARPS][P_ROWS * P_PITCH];
     const int lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
     uint32_t* win = win_all[threadIdx.x >> 5];
     const int per = a.Gx * a.Gy;
     const bool direct = long_list == nullptr;
-    const int sgx = (a.W / 16 + a.skip_k - 1) / a.skip_k, sgy = (a.Gy + a.skip_k - 1) / a.skip_k;   // searched columns (full width only), rows
+    const int sgx = (a.Gx + a.skip_k - 1) / a.skip_k, sgy = (a.Gy + a.skip_k - 1) / a.skip_k;       // searched columns, rows
     const int n = direct ? a.S * sgx * sgy : *long_count;
     const int max_rounds = 4 * a.R + 8;                               // each re-staging moves the centre by more than 4 px
 #pragma unroll 1
@@ -897,12 +925,12 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
             w.kind = c_kind_of_move[((w.cy - oy + 2) * 5 + (w.cx - ox + 2)) >> 1];
         }
         const int s = (int)(g / per), b = (int)(g - (size_t)s * per), by = b / a.Gx, bx = b - by * a.Gx;
-        const int x0 = bx * 16, y0 = by * 16, bh = min(16, a.H - y0);
+        const int x0 = bx * 16, y0 = by * 16, bh = min(16, a.H - y0), bw = min(16, a.W - x0);
         const bool row_on = r < bh;
         uint32_t cw[8];
         load_lane_pixels(a.cur + (size_t)s * a.cur_stream + (size_t)(row_on ? y0 + r : y0) * a.cur_pitch + (size_t)x0 * 3, h, row_on, cw);
         const uint8_t* prev = a.prev + (size_t)s * a.prev_stream;
-        const WalkBounds wb = walk_bounds(a, x0, y0, 16, bh);
+        const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
 #pragma unroll 1
         for (int round = 0;; ++round) {
             // the window around the centre that is scored next
@@ -937,7 +965,7 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
             // this lane's first word at displacement (0, 0): frame row y0 + r, pixel x0 + h, relative to the window's
             // origin (it may lie outside the window; only displacements near the centre are ever addressed)
             const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)(((r + y0 - wy0) * P_PITCH + (x0 - wx0) + h) * 4);
-            const int st = warp_walk<P_PITCH>(a, lane_base, cw, row_on, wb, w, reach);
+            const int st = warp_walk<P_PITCH>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, wb, w, reach);
             if (st == 1) break;
             if (round >= max_rounds) {                                   // never reached; a walk cut here is not valid
                 if (lane == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
@@ -948,7 +976,7 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
             w.cx = w.nx; w.cy = w.ny; w.bs = w.ns;
             __syncwarp();                                                // every lane has finished reading the old window
         }
-        if (lane == 0) publish_block(a, s, g, 16, bh, ((unsigned long long)w.bs << 32) | tie_key(w.cx, w.cy));
+        if (lane == 0) publish_block(a, s, g, bw, bh, ((unsigned long long)w.bs << 32) | tie_key(w.cx, w.cy));
     }
 }
 
@@ -959,6 +987,8 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
 // half-warp per block and one lane per block row, so that no warp idles on blocks that were settled.
 __global__ void __launch_bounds__(256) k_verify16_prep(MatchArgs a, uint32_t* list, int32_t* list_count)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const int lane = threadIdx.x & 31;
     const int per = a.Gx * a.Gy;
     const unsigned gi = blockIdx.x * 256u + threadIdx.x;                          // S * Gx * Gy < 2^31
@@ -999,6 +1029,8 @@ __global__ void __launch_bounds__(256) k_verify16_prep(MatchArgs a, uint32_t* li
 
 __global__ void __launch_bounds__(256) k_verify16_list(MatchArgs a, const uint32_t* list, const int32_t* list_count)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     const int lane = threadIdx.x & 31, r = lane & 15, half = lane >> 4;
     const int per = a.Gx * a.Gy, n = *list_count;
     const int stride = gridDim.x * 16;
@@ -1068,6 +1100,8 @@ constexpr int E_MAXROWS = 16 + 2 * E_MAXR + E_DY - 1;   // plus rows only touche
 
 __global__ void __launch_bounds__(256, 3) k_search_es16(MatchArgs a)
 {
+    dc_pdl_wait();
+    dc_pdl_release();
     extern __shared__ uint32_t es_sm[];
     const int R = a.R, n_d = 2 * R + 1;
     const int chunks = (n_d + E_DY - 1) / E_DY;
@@ -1180,27 +1214,40 @@ __global__ void __launch_bounds__(256, 3) k_search_es16(MatchArgs a)
     if (lane == 0) publish_block(a, s, g, 16, 16, bk);            // the zero vector is always valid, so bk is set
 }
 
-// Frame -> the library's aligned copy.  16-byte vectors when the source rows are aligned.
-__global__ void k_copy_frame(const uint8_t* src, size_t src_pitch, uint8_t* dst, size_t dst_pitch, int row_bytes,
-                             int rows, int vec)
+// Frame -> the library's aligned copy, one 16-byte vector of a row per thread.  Rows of any alignment are read as aligned
+// 32-bit words and shifted; bytes beyond a row's end become zeros; the last words of the caller's buffer are read byte
+// by byte.  Also zeroes the Step 3 sums and list counters of the search that follows (zero: n_zero words, or NULL).
+__global__ void __launch_bounds__(256) k_copy_frame(const uint8_t* src, const uint8_t* src_end, size_t src_pitch, uint8_t* dst, size_t dst_pitch, int row_bytes,
+                                                    unsigned total, int chunks, int32_t* zero, int n_zero)
 {
-    if (vec) {
-        const int chunks = (row_bytes + 15) >> 4;             // the last chunk may read source padding? no: see below
-        const size_t total = (size_t)rows * chunks;
-        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-            const size_t row = i / chunks; const int c = (int)(i - row * chunks);
-            if (c * 16 + 16 <= row_bytes) {
-                *(uint4*)(dst + row * dst_pitch + c * 16) = __ldg((const uint4*)(src + row * src_pitch + c * 16));
-            } else {                                          // ragged tail of the row: byte by byte
-                for (int k = c * 16; k < row_bytes; ++k) dst[row * dst_pitch + k] = src[row * src_pitch + k];
-            }
+    dc_pdl_wait();
+    dc_pdl_release();
+    if (zero && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const unsigned row = i / (unsigned)chunks, c = i - row * (unsigned)chunks;
+        const uint8_t* p = src + (size_t)row * src_pitch + c * 16u;
+        const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u;
+        const int left = row_bytes - (int)c * 16;                     // bytes of the row from here on
+        uint4 v;
+        if (((uintptr_t)p & 15u) == 0 && p + 16 <= src_end) {
+            v = __ldg((const uint4*)p);
+        } else if (p + 20 <= src_end) {
+            const uint32_t* q = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
+            const uint32_t w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = __ldg(q + 3), w4 = sh ? __ldg(q + 4) : 0u;
+            v = make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh), __funnelshift_r(w3, w4, sh));
+        } else {
+            uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int k = 0; k < 16; ++k) if (k < left) w[k >> 2] |= (uint32_t)__ldg(p + k) << (8 * (k & 3));
+            v = make_uint4(w[0], w[1], w[2], w[3]);
         }
-    } else {
-        const size_t total = (size_t)rows * row_bytes;
-        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-            const size_t row = i / row_bytes; const int k = (int)(i - row * row_bytes);
-            dst[row * dst_pitch + k] = src[row * src_pitch + k];
+        if (left < 16) {
+            const uint32_t keep[4] = {left >= 4 ? ~0u : (1u << (8 * left)) - 1u, left >= 8 ? ~0u : left <= 4 ? 0u : (1u << (8 * (left - 4))) - 1u,
+                                      left >= 12 ? ~0u : left <= 8 ? 0u : (1u << (8 * (left - 8))) - 1u, left <= 12 ? 0u : (1u << (8 * (left - 12))) - 1u};
+            v.x &= keep[0]; v.y &= keep[1]; v.z &= keep[2]; v.w &= keep[3];
         }
+        *(uint4*)(dst + (size_t)row * dst_pitch + c * 16u) = v;
     }
 }
 
@@ -1208,7 +1255,7 @@ template <int ITERS>
 void launch_verify(dc_cache* c, MatchArgs& a)
 {
     dc_prof_scope ps(c, DC_ST_VERIFY);
-    k_verify<ITERS><<<dc_div_up(a.S * a.Gx * a.Gy, WARPS), WARPS * 32, 0, c->stream>>>(a);
+    dc_launch_pdl(k_verify<ITERS>, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, WARPS)), WARPS * 32, 0, c->stream, a);    // errors: cudaGetLastError below
 }
 
 void launch_verify_by_block(dc_cache* c, MatchArgs& a)
@@ -1239,22 +1286,23 @@ int search_win(dc_cache* c, const MatchArgs& a, int only_clipped)
 
 }  // namespace
 
-int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst)
+// zero: the Step 3 sums of the match set that the search after this copy will use, or NULL
+int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst, int32_t* zero)
 {
-    const int row_bytes = c->cfg.width * 3, rows = c->cfg.height * c->S;
-    const int vec = ((uintptr_t)frame % 16 == 0) && (pitch % 16 == 0);
-    size_t work = vec ? (size_t)rows * ((row_bytes + 15) / 16) : (size_t)rows * row_bytes;
-    int grid = (int)((work + 255) / 256);
-    if (grid > c->num_sms * 16) grid = c->num_sms * 16;
-    if (grid < 1) grid = 1;
+    const int row_bytes = c->cfg.width * 3, rows = c->cfg.height * c->S, chunks = (row_bytes + 15) / 16;
+    const uint8_t* end = frame + pitch * (size_t)(rows - 1) + row_bytes;
+    const size_t work = (size_t)rows * chunks;
+    if (work > 0xffffffffull) return DC_ERR_CONFIG;                   // 64 GB of pixels
+    size_t grid = (work + 255) / 256;
+    if (grid > (size_t)c->num_sms * 32) grid = (size_t)c->num_sms * 32;
     dc_prof_scope ps(c, DC_ST_KEY_UPDATE);
-    k_copy_frame<<<grid, 256, 0, c->stream>>>(frame, pitch, dst, c->key_pitch, row_bytes, rows, vec);
+    DC_CUDA(dc_launch_pdl(k_copy_frame, dim3((unsigned)grid), 256, 0, c->stream, frame, end, pitch, dst, c->key_pitch, row_bytes, (unsigned)work, chunks,
+                          zero, 4 * c->S + 4));
     c->launches += 1;
-    DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
 
-int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key)
+int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key, const dc_match_out* out)
 {
     MatchArgs a;
     a.cur = cur_key; a.cur_pitch = c->key_pitch; a.cur_stream = c->key_pitch * (size_t)c->cfg.height;
@@ -1262,27 +1310,26 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
     a.W = c->cfg.width; a.H = c->cfg.height; a.B = c->cfg.block; a.R = c->cfg.range;
     a.Gx = c->Gx; a.Gy = c->Gy; a.S = c->S; a.search = c->cfg.search; a.skip_k = c->cfg.skip_k; a.region_mode = c->cfg.region_mode;
     for (int i = 0; i < 4; ++i) a.limit[i] = c->sse_limit[i];
-    a.mv = c->blk_mv; a.sse = c->blk_sse; a.matched = c->matched; a.acc = c->mv_acc; a.gmv = c->gmv;
+    // the caller's arrays, where given, take the place of the library's
+    a.mv = out && out->mv ? out->mv : c->blk_mv; a.sse = out && out->sse ? out->sse : c->blk_sse;
+    a.matched = out && out->matched ? out->matched : c->matched; a.acc = c->mv_acc; a.gmv = c->gmv;
     a.status = c->status;
-    // Step 3 sums and, behind them, the counter of walks handed to the second search phase
-    DC_CUDA(cudaMemsetAsync(c->mv_acc, 0, sizeof(int32_t) * (4 * c->S + 4), c->stream));
+    // Step 3 sums and, behind them, the counter of walks handed to the second search phase: zeroed by the frame copy
     int32_t* long_count = c->mv_acc + 4 * c->S;
+    // walks that phase 2 may get: no more warps than blocks
+    const dim3 long_grid((unsigned)min(c->num_sms * 5, dc_div_up(a.S * a.Gx * a.Gy, P_WARPS)));
     if (a.B == 16 && a.search == DC_SEARCH_DIAMOND) {
         {
             dc_prof_scope ps(c, DC_ST_SEARCH);
             if (a.skip_k <= 1) {
                 const dim3 tiles((a.Gx + 7) / 8, (a.Gy + W_VS - 1) / W_VS, a.S);
-                k_search_dsw<<<tiles, W_VS * 8 * 32, 0, c->stream>>>(a, c->long_list, long_count);
-                k_search_dsw_long<<<c->num_sms * 5, P_WARPS * 32, 0, c->stream>>>(a, c->long_list, long_count, long_count + 1);
+                DC_CUDA(dc_launch_pdl(k_search_dsw, tiles, W_VS * 8 * 32, 0, c->stream, a, c->long_list, long_count));
+                DC_CUDA(dc_launch_pdl(k_search_dsw_long, long_grid, P_WARPS * 32, 0, c->stream, a, (const uint4*)c->long_list, (const int32_t*)long_count, long_count + 1));
             } else {
-                k_mark_unsearched<<<dc_div_up(a.S * a.Gx * a.Gy, 256), 256, 0, c->stream>>>(a);
-                k_search_dsw_long<<<c->num_sms * 5, P_WARPS * 32, 0, c->stream>>>(a, nullptr, long_count, long_count + 1);
+                DC_CUDA(dc_launch_pdl(k_mark_unsearched, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a));
+                DC_CUDA(dc_launch_pdl(k_search_dsw_long, long_grid, P_WARPS * 32, 0, c->stream, a, (const uint4*)nullptr, (const int32_t*)long_count, long_count + 1));
             }
             c->launches += 1;
-        }
-        if (a.W % 16 != 0) {                                        // blocks clipped by the right edge
-            const int rc = search_win(c, a, 2);
-            if (rc != DC_OK) return rc;
         }
     } else if (a.B == 16 && a.search == DC_SEARCH_THREE_STEP && a.skip_k <= 1 && tss_window_bytes(a.R) <= 160 * 1024) {
         int s0 = a.R < 1 ? 0 : 1;                                   // first step: the largest power of two with 2 S0 - 1 <= R
@@ -1297,7 +1344,7 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
         {
             dc_prof_scope ps(c, DC_ST_SEARCH);
             const int ctas = ((a.Gx + 7) / 8) * ((a.Gy + TSS_VS - 1) / TSS_VS) * a.S;
-            k_search_tss16q<TSS_LPB, TSS_VS><<<ctas, TSS_LPB * 8 * TSS_VS, smem, c->stream>>>(a, s0, wr, words, pitch);
+            DC_CUDA(dc_launch_pdl(k_search_tss16q<TSS_LPB, TSS_VS>, dim3((unsigned)ctas), TSS_LPB * 8 * TSS_VS, smem, c->stream, a, s0, wr, words, pitch));
         }
         if (a.W % 16 != 0) {                                        // blocks clipped by the right edge
             const int rc = search_win(c, a, 2);
@@ -1313,7 +1360,7 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
         }
         {
             dc_prof_scope ps(c, DC_ST_SEARCH);
-            k_search_es16<<<((a.Gx + 7) / 8) * a.Gy * a.S, 256, smem, c->stream>>>(a);
+            DC_CUDA(dc_launch_pdl(k_search_es16, dim3((unsigned)(((a.Gx + 7) / 8) * a.Gy * a.S)), 256, smem, c->stream, a));
         }
         if (a.W % 16 != 0 || a.H % 16 != 0) {                   // blocks clipped by the right / bottom edge
             const int rc = search_win(c, a, 1);
@@ -1325,24 +1372,30 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
     }
     if (a.region_mode == DC_REGIONS_PER_BLOCK) {
         dc_prof_scope ps(c, DC_ST_VERIFY);
-        k_accept_own<<<dc_div_up(a.S * a.Gx * a.Gy, 256), 256, 0, c->stream>>>(a);
+        DC_CUDA(dc_launch_pdl(k_accept_own, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a));
     } else if (a.B == 16) {
         dc_prof_scope ps(c, DC_ST_VERIFY);
         int32_t* todo_count = long_count + 2;                       // zeroed with the Step 3 sums; the walk list is free again
-        k_verify16_prep<<<dc_div_up(a.S * a.Gx * a.Gy, 256), 256, 0, c->stream>>>(a, (uint32_t*)c->long_list, todo_count);
-        k_verify16_list<<<c->num_sms * 8, 256, 0, c->stream>>>(a, (const uint32_t*)c->long_list, todo_count);
+        DC_CUDA(dc_launch_pdl(k_verify16_prep, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a, (uint32_t*)c->long_list, todo_count));
+        DC_CUDA(dc_launch_pdl(k_verify16_list, dim3((unsigned)min(c->num_sms * 8, dc_div_up(a.S * a.Gx * a.Gy, 16))), 256, 0, c->stream, a,
+                              (const uint32_t*)c->long_list, (const int32_t*)todo_count));
         c->launches += 1;
     } else {
         launch_verify_by_block(c, a);
     }
     {
         dc_prof_scope ps(c, DC_ST_MERGE);
-        const int16_t* own = a.region_mode == DC_REGIONS_PER_BLOCK ? c->blk_mv : nullptr;
-        k_merge_runs<<<dc_div_up(c->S * a.Gx * a.Gy, 256), 256, 0, c->stream>>>(c->matched, own, a.Gx, c->S * a.Gx * a.Gy, c->run_end);
-        k_merge<<<c->S, 1024, 0, c->stream>>>(c->run_end, own, c->gmv, a.W, a.H, a.B, a.Gx, a.Gy, c->max_regions,
-                                              c->regions0, c->n_regions, c->status);
+        const bool own = a.region_mode == DC_REGIONS_PER_BLOCK;
+        const int n = a.Gx * a.Gy;
+        const size_t need = (size_t)n * (own ? 7 : 3);              // runs, matched flags and vectors of a stream
+        const bool fits = need <= 160 * 1024;
+        static dc_once_per_device attr_set;
+        if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+        DC_CUDA(dc_launch_pdl(k_merge, dim3((unsigned)c->S), 1024, fits ? need : 0, c->stream, (const uint8_t*)a.matched, (const int16_t*)(own ? a.mv : nullptr),
+                              (const int32_t*)c->gmv, a.W, a.H, a.B, a.Gx, a.Gy, c->max_regions, c->run_end, fits ? 1 : 0, c->regions0, c->n_regions, c->status,
+                              out ? out->gmv : nullptr, out ? out->n_regions : nullptr, out ? out->regions : nullptr));
     }
-    c->launches += 4;
+    c->launches += 3;
     DC_CUDA(cudaGetLastError());
     return DC_OK;
 }

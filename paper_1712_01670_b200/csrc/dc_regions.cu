@@ -2,8 +2,7 @@
 // (Section 5, "Reuse": copy cached regions, build the bitmap, list what is left to compute).
 //
 //   k_propagate      one thread per (stream, rectangle slot) walks the layer table in order and
-//                    writes the rectangle's image after every layer.  Slots are independent,
-//                    so no synchronisation is needed; a vanished rectangle is all zeros.
+//                    writes the rectangle's image after every layer; a vanished rectangle is all zeros.
 //   k_classify_copy  one warp per 16x8 output tile: lanes test the stream's rectangles against
 //                    the tile, OR their coverage into a 128-bit bitmap, the warp copies each
 //                    covered row span from the cached map with bulk copies (global -> shared ->
@@ -24,6 +23,7 @@ __device__ __forceinline__ int ceil_div(int a, int b) { return -floor_div(-a, b)
 // inside [x, x + w).  First = ceil((x + p) / s) as printed in Table 2; last = floor((x + w - k + p) / s).
 __device__ __forceinline__ void erode_axis(int x, int w, int k, int s, int p, int& xo, int& wo)
 {
+    if (s == 1) { xo = x + p; wo = w - k + 1; return; }
     int first = ceil_div(x + p, s), last = floor_div(x + w - k + p, s);
     xo = first; wo = last - first + 1;
 }
@@ -37,7 +37,13 @@ __device__ __forceinline__ void resize_axis(int x, int w, int n_in, int n_out, i
 
 __device__ __forceinline__ dc_region empty_region() { dc_region e = {0, 0, 0, 0, 0, 0}; return e; }
 
-__device__ dc_region apply_layer(const dc_layer_desc& L, int in_h, int in_w, dc_region a, dc_region b)
+// A layer as propagation sees it.  from0 / from1: where the input's rectangle is: kFrame, kPrevious (the layer before, still in
+// registers), kTable (the table in global memory), or one of the kSlots places of the thread in shared memory; keep: the
+// place that this layer's own rectangle takes, or -1.
+constexpr int kSlots = 6, kFrame = -1, kPrevious = -2, kTable = -3;
+struct PropLayer { int kind, kh, kw, sh, sw, ph, pw, in_h, in_w, out_h, out_w, in0, in1, from0, from1, keep; };
+
+__device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
 {
     if (a.w <= 0 || a.h <= 0) return empty_region();
     switch (L.kind) {
@@ -45,8 +51,8 @@ __device__ dc_region apply_layer(const dc_layer_desc& L, int in_h, int in_w, dc_
         // D_t on the current rectangle and, independently, on the cached one; smaller size wins
         int dx, dw, dy, dh, qx, qw, qy, qh;
         if (L.kind == DC_RESIZE_AREA) {
-            resize_axis(a.x, a.w, in_w, L.out_w, dx, dw);  resize_axis(a.y, a.h, in_h, L.out_h, dy, dh);
-            resize_axis(a.sx, a.w, in_w, L.out_w, qx, qw); resize_axis(a.sy, a.h, in_h, L.out_h, qy, qh);
+            resize_axis(a.x, a.w, L.in_w, L.out_w, dx, dw);  resize_axis(a.y, a.h, L.in_h, L.out_h, dy, dh);
+            resize_axis(a.sx, a.w, L.in_w, L.out_w, qx, qw); resize_axis(a.sy, a.h, L.in_h, L.out_h, qy, qh);
         } else {
             erode_axis(a.x, a.w, L.kw, L.sw, L.pw, dx, dw);  erode_axis(a.y, a.h, L.kh, L.sh, L.ph, dy, dh);
             erode_axis(a.sx, a.w, L.kw, L.sw, L.pw, qx, qw); erode_axis(a.sy, a.h, L.kh, L.sh, L.ph, qy, qh);
@@ -79,23 +85,63 @@ __device__ dc_region apply_layer(const dc_layer_desc& L, int in_h, int in_w, dc_
     }
 }
 
-__global__ void k_propagate(const dc_layer_desc* layers, const int32_t* in_hw, int layer_end, int S, int max_regions,
-                            const dc_region* in, const int32_t* n_in, dc_region* table, int32_t* alive)
+// One CTA per stream, a thread one rectangle at a time.  Rectangles that a later layer than the next one needs (residual
+// branches) wait in shared memory, and so does the layer table: the walk is a chain of a few dozen arithmetic steps per
+// layer (through a table in global memory it was a chain of memory round trips: 48 us for the 71 layers of ResNet-50).
+// out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): rectangles still
+// alive per layer and stream; with it the counters of the reuse step are zeroed.
+__global__ void __launch_bounds__(256) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions,
+                                                   const dc_region* in, const int32_t* n_in, dc_region* table, int32_t* alive, int32_t* reuse_px,
+                                                   int32_t* dirty_count, dc_region* out, int out_begin, int32_t* n_out)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int s = blockIdx.y;
-    if (i >= max_regions || i >= n_in[s]) return;          // a caller's count beyond the table is cut, never written
-    const size_t slot = (size_t)s * max_regions + i;
+    __shared__ PropLayer sl[DC_MAX_LAYERS];
+    __shared__ int32_t keep[kSlots * 6][256];
+    __shared__ int32_t count[DC_MAX_LAYERS];
+    const int s = blockIdx.x, tid = threadIdx.x;
+    for (int i = tid; i < layer_end * (int)(sizeof(PropLayer) / 4); i += 256) ((int*)sl)[i] = __ldg((const int*)layers + i);
+    if (tid < DC_MAX_LAYERS) count[tid] = 0;
+    dc_pdl_wait();
+    dc_pdl_release();
+    __syncthreads();
     const size_t layer_stride = (size_t)S * max_regions;
-    const dc_region r0 = in[slot];
-    for (int l = 0; l < layer_end; ++l) {
-        const dc_layer_desc L = layers[l];
-        dc_region a = L.in0 < 0 ? r0 : table[L.in0 * layer_stride + slot];
-        dc_region b = a;
-        if (L.kind == DC_ADD || L.kind == DC_CONCAT) b = L.in1 < 0 ? r0 : table[L.in1 * layer_stride + slot];
-        const dc_region o = apply_layer(L, in_hw[2 * l], in_hw[2 * l + 1], a, b);
-        table[l * layer_stride + slot] = o;
-        if (o.w > 0 && alive) atomicAdd(&alive[l * S + s], 1);     // rectangles still alive at this layer
+    const int n = min(n_in[s], max_regions);              // a caller's count beyond the table is cut, never written
+    // a caller's list has zeros behind its rectangles
+    const int rows = out ? max_regions : n;
+    for (int i = tid; i < rows; i += 256) {
+        const size_t slot = (size_t)s * max_regions + i;
+        const bool on = i < n;
+        const dc_region r0 = on ? in[slot] : empty_region();
+        dc_region prev = r0;
+        auto fetch = [&](int from, int layer) -> dc_region {
+            if (from == kFrame) return r0;
+            if (from == kPrevious) return prev;
+            if (from == kTable) return on ? table[layer * layer_stride + slot] : empty_region();
+            dc_region r = {keep[from * 6][tid], keep[from * 6 + 1][tid], keep[from * 6 + 2][tid], keep[from * 6 + 3][tid], keep[from * 6 + 4][tid], keep[from * 6 + 5][tid]};
+            return r;
+        };
+        for (int l = 0; l < layer_end; ++l) {
+            const PropLayer& L = sl[l];
+            const dc_region a = fetch(L.from0, L.in0);
+            const dc_region b = L.kind == DC_ADD || L.kind == DC_CONCAT ? fetch(L.from1, L.in1) : a;
+            const dc_region o = apply_layer(L, a, b);
+            if (L.keep >= 0) {
+                int32_t (*k)[256] = &keep[L.keep * 6];
+                k[0][tid] = o.x; k[1][tid] = o.y; k[2][tid] = o.w; k[3][tid] = o.h; k[4][tid] = o.sx; k[5][tid] = o.sy;
+            }
+            table[l * layer_stride + slot] = o;
+            if (out && l >= out_begin) out[(l - out_begin) * layer_stride + slot] = o;
+            if (o.w > 0 && alive) atomicAdd(&count[l], 1);
+            prev = o;
+        }
+    }
+    if (n_out) for (int l = out_begin + tid; l < layer_end; l += 256) n_out[(l - out_begin) * S + s] = n_in[s];
+    if (alive) {
+        __syncthreads();
+        for (int l = tid; l < n_layers; l += 256) {
+            alive[l * S + s] = l < layer_end ? count[l] : 0;
+            reuse_px[l * S + s] = 0;
+            if (s == 0) dirty_count[l] = 0;
+        }
     }
 }
 
@@ -171,9 +217,11 @@ struct ClassifyArgs {
     const int32_t* alive;                        // per stream: rectangles alive at this layer, or NULL (unknown)
     unsigned long long* reused_total;
     int32_t* status;                             // device status word
+    int parts;                                   // warps that share a tile's copies (each tests the rectangles, the first one records the outcome)
+    int32_t* zero_next;                          // a counter that this launch zeroes for a later one, or NULL
 };
 
-__device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int tile, const int lane, CopyLane& cl)
+__device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int tile, const int part, const int lane, CopyLane& cl)
 {
     const int per = a.tiles_x * a.tiles_y;
     const int s = tile / per, t = tile - s * per, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
@@ -211,50 +259,58 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
                 switch (bit >> 5) { case 0: m0 |= v; break; case 1: m1 |= v; break; case 2: m2 |= v; break; default: m3 |= v; }
             }
         }
-        // the warp copies every hit span together: rows of (ix1 - ix0) pixels, px_bytes each
+        // Section 5 "Reuse", step 1.  Inside the tile a rectangle is (iy1 - iy0) row spans, each contiguous in both maps
+        // (all channels of ix1 - ix0 pixels).  Spans are cut into segments of kSeg bytes, and the segments of all the
+        // rectangles that hit are numbered through: per round every lane moves one of them, a bulk copy into the warp's
+        // staging, then a bulk copy out to the new map, so that a tile with several small rectangles costs one round
+        // trip and not one per rectangle.  Addresses and sizes are multiples of 16 bytes (px_bytes is).
         unsigned hits = __ballot_sync(0xffffffffu, hit);
-        while (hits) {
-            int src_lane = __ffs(hits) - 1; hits &= hits - 1;
-            int rx = __shfl_sync(0xffffffffu, r.x, src_lane), ry = __shfl_sync(0xffffffffu, r.y, src_lane);
-            int rsx = __shfl_sync(0xffffffffu, r.sx, src_lane), rsy = __shfl_sync(0xffffffffu, r.sy, src_lane);
-            int cx0 = __shfl_sync(0xffffffffu, ix0, src_lane), cx1 = __shfl_sync(0xffffffffu, ix1, src_lane);
-            int cy0 = __shfl_sync(0xffffffffu, iy0, src_lane), cy1 = __shfl_sync(0xffffffffu, iy1, src_lane);
-            // Section 5 "Reuse", step 1.  Inside the tile the rectangle is (cy1 - cy0) row spans, each contiguous in both
-            // maps (all channels of cx1 - cx0 pixels).  Spans are cut into segments of kSeg bytes; per round every lane
-            // moves one segment: a bulk copy into the warp's staging, then a bulk copy out to the new map.  Addresses
-            // and sizes are multiples of 16 bytes (px_bytes is).
-            const int span_bytes = (cx1 - cx0) * a.px_bytes;
-            const int segs = (span_bytes + kSeg - 1) / kSeg, items = (cy1 - cy0) * segs;
-            const uint8_t* src0 = a.prev + map_base + ((size_t)(cy0 - ry + rsy) * a.Wo + (cx0 - rx + rsx)) * a.px_bytes;
-            uint8_t* dst0 = a.out + map_base + ((size_t)cy0 * a.Wo + cx0) * a.px_bytes;
-            const size_t row_pitch = (size_t)a.Wo * a.px_bytes;
-            for (int i0 = 0; i0 < items && !cl.dead; i0 += 32) {
-                const int it = i0 + lane;
-                const bool on = it < items;
-                const int row = on ? it / segs : 0, sg = it - row * segs;
-                const uint32_t bytes = on ? (uint32_t)min(kSeg, span_bytes - sg * kSeg) : 0u;
-                const size_t off = (size_t)row * row_pitch + (size_t)sg * kSeg;
-                const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
-                if (lane == 0) rs_expect(cl.bar, total);
-                __syncwarp();
-                if (on) rs_load(cl.stage + lane * kSeg, src0 + off, bytes, cl.bar);
-                const bool landed = rs_wait(cl.bar, cl.phase);
-                if (!__all_sync(0xffffffffu, landed)) {                     // never seen; leave rather than spin for ever
-                    if (lane == 0 && a.status) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
-                    cl.dead = true;
-                    break;
-                }
-                cl.phase ^= 1u;
-                if (on) rs_store(dst0 + off, cl.stage + lane * kSeg, bytes);
-                rs_commit();
-                rs_wait_read();                                             // staging may be overwritten by the next round
-                __syncwarp();
+        if (hits == 0) continue;
+        const int span_bytes = hit ? (ix1 - ix0) * a.px_bytes : 0;
+        const int segs = (span_bytes + kSeg - 1) / kSeg, mine = hit ? (iy1 - iy0) * segs : 0;
+        int first = mine;                                               // inclusive sum over the lanes, then this lane's start
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, first, o); if (lane >= o) first += v; }
+        const int items = __shfl_sync(0xffffffffu, first, 31);
+        first -= mine;
+        const int src_y = iy0 - r.y + r.sy, src_x = ix0 - r.x + r.sx;   // cached position of (ix0, iy0)
+        for (int i0 = part * 32; i0 < items && !cl.dead; i0 += 32 * a.parts) {
+            const int it = i0 + lane;
+            const bool on = it < items;
+            int owner = 0;                                              // the lane whose rectangle segment `it` belongs to
+            for (unsigned h = hits; h; h &= h - 1) {
+                const int k = __ffs(h) - 1;
+                if (it >= __shfl_sync(0xffffffffu, first, k)) owner = k;
             }
+            const int o_first = __shfl_sync(0xffffffffu, first, owner), o_segs = max(1, __shfl_sync(0xffffffffu, segs, owner));
+            const int o_span = __shfl_sync(0xffffffffu, span_bytes, owner);
+            const int o_x = __shfl_sync(0xffffffffu, ix0, owner), o_y = __shfl_sync(0xffffffffu, iy0, owner);
+            const int o_sx = __shfl_sync(0xffffffffu, src_x, owner), o_sy = __shfl_sync(0xffffffffu, src_y, owner);
+            const int loc = it - o_first, row = loc / o_segs, sg = loc - row * o_segs;
+            const uint32_t bytes = on ? (uint32_t)min(kSeg, o_span - sg * kSeg) : 0u;
+            const size_t seg_off = (size_t)sg * kSeg;
+            const uint8_t* src = a.prev + map_base + ((size_t)(o_sy + row) * a.Wo + o_sx) * a.px_bytes + seg_off;
+            uint8_t* dst = a.out + map_base + ((size_t)(o_y + row) * a.Wo + o_x) * a.px_bytes + seg_off;
+            const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+            if (lane == 0) rs_expect(cl.bar, total);
+            __syncwarp();
+            if (on) rs_load(cl.stage + lane * kSeg, src, bytes, cl.bar);
+            const bool landed = rs_wait(cl.bar, cl.phase);
+            if (!__all_sync(0xffffffffu, landed)) {                     // never seen; leave rather than spin for ever
+                if (lane == 0 && a.status) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
+                cl.dead = true;
+                break;
+            }
+            cl.phase ^= 1u;
+            if (on) rs_store(dst, cl.stage + lane * kSeg, bytes);
+            rs_commit();
+            rs_wait_read();                                             // staging may be overwritten by the next round
+            __syncwarp();
         }
     }
     m0 = __reduce_or_sync(0xffffffffu, m0); m1 = __reduce_or_sync(0xffffffffu, m1);
     m2 = __reduce_or_sync(0xffffffffu, m2); m3 = __reduce_or_sync(0xffffffffu, m3);
-    if (lane == 0) {
+    if (lane == 0 && part == 0) {
         uint32_t* mk = a.masks + (size_t)tile * 4;
         mk[0] = m0; mk[1] = m1; mk[2] = m2; mk[3] = m3;
         int covered = __popc(m0) + __popc(m1) + __popc(m2) + __popc(m3);
@@ -271,7 +327,7 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
 // The same for a layer with flat tiles: row i of the tile's bitmap is group tile * 16 + i, a group being 8 pixels of
 // one image row, numbered (stream * Ho + y) * gpr + column group.  A tile may hold groups of several streams (small
 // maps); each stream's rectangles are tested against that stream's groups only.
-__device__ __forceinline__ void classify_tile_flat(const ClassifyArgs& a, const int tile, const int lane, CopyLane& cl)
+__device__ __forceinline__ void classify_tile_flat(const ClassifyArgs& a, const int tile, const int part, const int lane, CopyLane& cl)
 {
     const int gps = a.Ho * a.gpr;                                  // groups per stream
     const int G0 = tile * DC_TILE_H, G1 = min(G0 + DC_TILE_H, a.S * gps);
@@ -325,7 +381,7 @@ __device__ __forceinline__ void classify_tile_flat(const ClassifyArgs& a, const 
                 const int rw = __shfl_sync(0xffffffffu, r.w, src_lane);
                 const int rsx = __shfl_sync(0xffffffffu, r.sx, src_lane), rsy = __shfl_sync(0xffffffffu, r.sy, src_lane);
                 const uint32_t h16 = __shfl_sync(0xffffffffu, hit16, src_lane);
-                for (int i0 = 0; i0 < DC_TILE_H * segs_max && !cl.dead; i0 += 32) {
+                for (int i0 = part * 32; i0 < DC_TILE_H * segs_max && !cl.dead; i0 += 32 * a.parts) {
                     const int it = i0 + lane, row = it / segs_max, sg = it - row * segs_max;
                     uint32_t bytes = 0;
                     size_t src_off = 0, dst_off = 0;
@@ -361,10 +417,10 @@ __device__ __forceinline__ void classify_tile_flat(const ClassifyArgs& a, const 
         s0 = __reduce_or_sync(0xffffffffu, s0); s1 = __reduce_or_sync(0xffffffffu, s1);
         s2 = __reduce_or_sync(0xffffffffu, s2); s3 = __reduce_or_sync(0xffffffffu, s3);
         const int covered_s = __popc(s0) + __popc(s1) + __popc(s2) + __popc(s3);
-        if (lane == 0 && covered_s) { atomicAdd(&a.reuse_px[s], covered_s); atomicAdd(a.reused_total, (unsigned long long)covered_s); }
+        if (lane == 0 && part == 0 && covered_s) { atomicAdd(&a.reuse_px[s], covered_s); atomicAdd(a.reused_total, (unsigned long long)covered_s); }
         m0 |= s0; m1 |= s1; m2 |= s2; m3 |= s3;
     }
-    if (lane == 0) {
+    if (lane == 0 && part == 0) {
         uint32_t* mk = a.masks + (size_t)tile * 4;
         mk[0] = m0; mk[1] = m1; mk[2] = m2; mk[3] = m3;
         if (__popc(m0) + __popc(m1) + __popc(m2) + __popc(m3) < in_tile) {
@@ -392,10 +448,13 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy(ClassifyArgs 
 {
     extern __shared__ uint8_t copy_smem[];
     CopyLane cl = copy_lane_setup(copy_smem);
-    const int tile = blockIdx.x * kCopyWarps + (threadIdx.x >> 5);
+    dc_pdl_wait();
+    dc_pdl_release();
+    if (a.zero_next && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_next = 0;
+    const int w = blockIdx.x * kCopyWarps + (threadIdx.x >> 5), tile = w / a.parts, part = w - tile * a.parts;
     if (tile < a.n_tiles) {
-        if (a.gpr > 0) classify_tile_flat(a, tile, threadIdx.x & 31, cl);
-        else classify_tile(a, tile, threadIdx.x & 31, cl);
+        if (a.gpr > 0) classify_tile_flat(a, tile, part, threadIdx.x & 31, cl);
+        else classify_tile(a, tile, part, threadIdx.x & 31, cl);
     }
     rs_wait_all();
 }
@@ -405,7 +464,7 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy(ClassifyArgs 
 // Warps are numbered through all layers' tiles; first_warp is the running sum.
 struct ClassifyLayer {
     const dc_region* regions; uint8_t* map[2];
-    int Ho, Wo, px_bytes, tiles_x, tiles_y, first_warp, gpr;
+    int Ho, Wo, px_bytes, tiles_x, tiles_y, first_warp, gpr, parts;
     uint32_t* masks; int32_t* dirty_list; int32_t* dirty_count; int32_t* reuse_px;
     const int32_t* alive; unsigned long long* reused_total; int32_t* status;
 };
@@ -415,6 +474,8 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
 {
     extern __shared__ uint8_t copy_smem[];
     CopyLane cl = copy_lane_setup(copy_smem);
+    dc_pdl_wait();
+    dc_pdl_release();
     const int w = blockIdx.x * kCopyWarps + (threadIdx.x >> 5);
     if (w >= total_warps) return;                       // no copy was issued by this warp
     int lo = 0, hi = n_cached - 1;
@@ -430,12 +491,24 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
     a.gpr = L.gpr; a.n_tiles = 0;
     a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = L.dirty_count; a.reuse_px = L.reuse_px;
     a.alive = L.alive; a.reused_total = L.reused_total; a.status = L.status;
-    if (a.gpr > 0) classify_tile_flat(a, w - L.first_warp, threadIdx.x & 31, cl);
-    else classify_tile(a, w - L.first_warp, threadIdx.x & 31, cl);
+    a.parts = L.parts; a.zero_next = nullptr;
+    const int u = w - L.first_warp, tile = u / a.parts, part = u - tile * a.parts;
+    if (a.gpr > 0) classify_tile_flat(a, tile, part, threadIdx.x & 31, cl);
+    else classify_tile(a, tile, part, threadIdx.x & 31, cl);
     rs_wait_all();
 }
 
 }  // namespace
+
+// Warps per tile of a layer: one where there are tiles enough to fill the machine (24 warps per SM, twice over); otherwise
+// the copies of a tile, up to 128 pixels of px_bytes in rounds of 32 segments, are dealt to as many as have a round to do.
+static int copy_parts(const dc_cache* c, long long tiles_in_launch, int px_bytes)
+{
+    const int rounds = dc_div_up(DC_TILE_H * dc_div_up(DC_TILE_W * px_bytes, kSeg), 32);
+    long long room = (long long)c->num_sms * 48 / (tiles_in_launch > 0 ? tiles_in_launch : 1);
+    if (room > rounds) room = rounds;
+    return room < 1 ? 1 : room > 8 ? 8 : (int)room;
+}
 
 // Builds the device table for k_classify_copy_all (once, after every map is allocated).
 int dc_build_classify_table(dc_cache* c)
@@ -444,6 +517,8 @@ int dc_build_classify_table(dc_cache* c)
     ClassifyLayer* h = (ClassifyLayer*)malloc(sizeof(ClassifyLayer) * (n > 0 ? n : 1));
     if (!h) return DC_ERR_ALLOC;
     int k = 0, warps = 0;
+    long long tiles = 0;
+    for (int i = 0; i < n; ++i) if (dc_layer_cached(c, i)) tiles += dc_layer_tiles(c, c->L[i]);
     for (int i = 0; i < n; ++i) {
         if (!dc_layer_cached(c, i)) continue;
         dc_layer_rt& L = c->L[i];
@@ -457,7 +532,8 @@ int dc_build_classify_table(dc_cache* c)
         e.reuse_px = c->reuse_px + (size_t)i * c->S; e.alive = c->alive + (size_t)i * c->S;
         e.reused_total = c->reused_total + i;
         e.status = c->status;
-        warps += dc_layer_tiles(c, L);
+        e.parts = copy_parts(c, tiles, e.px_bytes);
+        warps += dc_layer_tiles(c, L) * e.parts;
     }
     c->n_cached = k; c->classify_warps = warps;
     int rc = DC_OK;
@@ -471,7 +547,7 @@ int dc_build_classify_table(dc_cache* c)
 }
 
 // All cached layers at once; `cur` is the index of the map that holds the cached values (the same for every layer:
-// they all flip once per frame).  The caller has zeroed the dirty counts and the reuse counters on the stream.
+// they all flip once per frame).  Region propagation has zeroed the dirty counts and the reuse counters.
 int dc_launch_classify_all(dc_cache* c, int cur)
 {
     if (c->n_cached <= 0) return DC_OK;
@@ -480,29 +556,63 @@ int dc_launch_classify_all(dc_cache* c, int cur)
         static dc_once_per_device attr_set;
         if (attr_set.first(c->device))
             DC_CUDA(cudaFuncSetAttribute(k_classify_copy_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCopySmem));
-        k_classify_copy_all<<<dc_div_up(c->classify_warps, kCopyWarps), kCopyWarps * 32, kCopySmem, c->stream>>>(
-            (const ClassifyLayer*)c->classify_table, c->n_cached, c->classify_warps, c->n_regions, c->max_regions, c->S, cur);
+        DC_CUDA(dc_launch_pdl(k_classify_copy_all, dim3((unsigned)dc_div_up(c->classify_warps, kCopyWarps)), kCopyWarps * 32, kCopySmem, c->stream,
+                              (const ClassifyLayer*)c->classify_table, c->n_cached, c->classify_warps, (const int32_t*)c->n_regions, c->max_regions, c->S, cur));
     }
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
 
-int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end)
+// The layer table as k_propagate reads it.
+int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
 {
-    dim3 grid(dc_div_up(c->max_regions, 128), c->S);
-    {
-        dc_prof_scope ps(c, DC_ST_PROPAGATE);
-        k_propagate<<<grid, 128, 0, c->stream>>>(c->layers_dev, c->in_hw_dev, layer_end, c->S, c->max_regions,
-                                                 in, n_in, c->table, c->alive);
+    const int n = c->n_layers;
+    PropLayer t[DC_MAX_LAYERS];
+    int last_use[DC_MAX_LAYERS];                           // last layer that needs l's rectangle other than as "the layer before"
+    for (int l = 0; l < n; ++l) last_use[l] = -1;
+    for (int l = 0; l < n; ++l) {
+        const dc_layer_desc& d = layers[l];
+        if (d.in0 >= 0 && d.in0 != l - 1) last_use[d.in0] = l;
+        if ((d.kind == DC_ADD || d.kind == DC_CONCAT) && d.in1 >= 0 && d.in1 != l - 1) last_use[d.in1] = l;
     }
-    c->launches += 1;
-    DC_CUDA(cudaGetLastError());
+    int owner[kSlots];
+    for (int k = 0; k < kSlots; ++k) owner[k] = -1;
+    auto from = [&](int l, int in) {
+        if (in < 0) return kFrame;
+        if (in == l - 1) return kPrevious;
+        for (int k = 0; k < kSlots; ++k) if (owner[k] == in) return k;
+        return kTable;
+    };
+    for (int l = 0; l < n; ++l) {
+        const dc_layer_desc& d = layers[l];
+        const int ih = d.in0 < 0 ? c->cfg.height : layers[d.in0].out_h, iw = d.in0 < 0 ? c->cfg.width : layers[d.in0].out_w;
+        t[l] = {d.kind, d.kh, d.kw, d.sh, d.sw, d.ph, d.pw, ih, iw, d.out_h, d.out_w, d.in0, d.in1, from(l, d.in0), from(l, d.in1), -1};
+        for (int k = 0; k < kSlots; ++k) if (owner[k] >= 0 && last_use[owner[k]] <= l) owner[k] = -1;
+        if (last_use[l] > l)
+            for (int k = 0; k < kSlots; ++k) if (owner[k] < 0) { owner[k] = l; t[l].keep = k; break; }
+    }
+    if (cudaMalloc(&c->prop_table, sizeof(PropLayer) * n) != cudaSuccess) { cudaGetLastError(); return DC_ERR_ALLOC; }
+    c->bytes += sizeof(PropLayer) * n;
+    DC_CUDA(cudaMemcpy(c->prop_table, t, sizeof(PropLayer) * n, cudaMemcpyHostToDevice));
     return DC_OK;
 }
 
+// for_frame: the rectangles of the frame being inferred (counts what is alive, zeroes the reuse step's counters);
+// otherwise a caller's, returned in out / n_out for layers out_begin .. layer_end - 1.
+int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out)
+{
+    dc_prof_scope ps(c, DC_ST_PROPAGATE);
+    DC_CUDA(dc_launch_pdl(k_propagate, dim3((unsigned)c->S), 256, 0, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, in, n_in,
+                          c->table, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
+    c->launches += 1;
+    return DC_OK;
+}
+
+// count, px: where the dirty tiles and the reused pixels per stream are counted; count is zero when the kernel starts.
+// zero_next: a counter that the kernel zeroes, or NULL.
 int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, const int32_t* n_regions,
-                            const void* prev_out, void* out)
+                            const void* prev_out, void* out, int32_t* count, int32_t* px, int32_t* zero_next)
 {
     dc_layer_rt& L = c->L[layer];
     ClassifyArgs a;
@@ -511,17 +621,17 @@ int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, co
     a.Ho = L.d.out_h; a.Wo = L.d.out_w; a.px_bytes = L.d.cout * c->elt;
     a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y; a.S = c->S;
     a.gpr = L.flat ? L.gpr : 0; a.n_tiles = dc_layer_tiles(c, L);
-    a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = c->dirty_count + layer;
-    a.reuse_px = c->reuse_px + (size_t)layer * c->S;
+    a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = count;
+    a.reuse_px = px;
+    a.zero_next = zero_next; a.parts = copy_parts(c, dc_layer_tiles(c, L), a.px_bytes);
     a.reused_total = c->reused_total + layer;
     a.status = c->status;
     a.alive = (regions == c->table + (size_t)layer * c->S * c->max_regions) ? c->alive + (size_t)layer * c->S : nullptr;
-    // the caller has zeroed dirty_count[layer] and reuse_px[layer][*] on the stream
-    int tiles = dc_layer_tiles(c, L);
+    const int warps = dc_layer_tiles(c, L) * a.parts;
     static dc_once_per_device attr_set;
     if (attr_set.first(c->device))
         DC_CUDA(cudaFuncSetAttribute(k_classify_copy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCopySmem));
-    { dc_prof_scope ps(c, DC_ST_CLASSIFY_COPY); k_classify_copy<<<dc_div_up(tiles, kCopyWarps), kCopyWarps * 32, kCopySmem, c->stream>>>(a); }
+    { dc_prof_scope ps(c, DC_ST_CLASSIFY_COPY); DC_CUDA(dc_launch_pdl(k_classify_copy, dim3((unsigned)dc_div_up(warps, kCopyWarps)), kCopyWarps * 32, kCopySmem, c->stream, a)); }
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;
