@@ -181,6 +181,7 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     for (int i = 0; i < n; ++i) {
         dc_layer_rt& L = c->L[i];
         L.d = layers[i];
+        L.fuse_add = -1;
         // an executable fully-connected layer runs as the convolution that covers its input map; the device copy of the
         // layer table keeps DC_FC, so Table 2 still marks nothing of its output reusable and every tile is computed
         if (L.d.kind == DC_FC && c->executable) { L.d.kind = DC_CONV; L.d.sh = L.d.sw = 1; L.d.ph = L.d.pw = 0; }
@@ -234,6 +235,13 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
             if (c->L[i].s2d_s) in = c->L[i].in_s2d;               // the kernels being timed read the block map
             DC_TRY(dc_conv_bf16_autotune(c, i, in));
         }
+    // element-wise adds whose later operand is a convolution on the cluster kernel are done by that kernel
+    for (int j = 0; j < n && c->executable && cfg.dtype == DC_BF16; ++j) {
+        const dc_layer_desc& d = c->L[j].d;
+        if (d.kind != DC_ADD || d.in0 < 0 || d.in1 < 0 || d.in0 == d.in1) continue;
+        dc_layer_rt& P = c->L[d.in0 > d.in1 ? d.in0 : d.in1];
+        if (P.d.kind == DC_CONV && P.tc_cs > 0 && P.fuse_add < 0) P.fuse_add = j;
+    }
     // who reads the frame as a map, and who reads the resized frame
     c->fused_input = need_input_map; c->resize_feeds = -1;
     int resize = -1, readers = 0;
@@ -490,8 +498,15 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
             if (L.d.in0 < 0 && c->fused_input) { DC_TRY(dc_launch_frame_operand(c, i, frame_copy, c->key_pitch)); in = nullptr; }
             else if (i == c->resize_feeds) in = nullptr;              // its operand copy is filled already
-            if (!refresh) {
-                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
+            if (!refresh && !classified)
+                DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
+            if (L.fuse_add >= 0) {                                    // every tile: the add is due for reused pixels too
+                dc_layer_rt& A = c->L[L.fuse_add];
+                c->add_in = layer_input(c, A.d.in0 == i ? A.d.in1 : A.d.in0); c->add_out = A.map[0]; c->add_relu = A.d.relu;
+                const int rc = dc_launch_conv(c, i, in, out, L.all_list, dc_all_count(c, i), refresh ? c->zero_masks : L.masks, tiles);
+                c->add_out = nullptr;
+                if (rc != DC_OK) return rc;
+            } else if (!refresh) {
                 DC_TRY(dc_launch_conv(c, i, in, out, L.dirty_list, c->dirty_count + i, L.masks, tiles));
             } else {
                 DC_TRY(dc_launch_conv(c, i, in, out, L.all_list, dc_all_count(c, i), c->zero_masks, tiles));
@@ -511,7 +526,12 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             L.cur ^= 1;
             break;
         }
-        case DC_ADD: DC_TRY(dc_launch_add(c, i, in, layer_input(c, L.d.in1))); break;
+        case DC_ADD: {
+            const int later = L.d.in0 > L.d.in1 ? L.d.in0 : L.d.in1;
+            if (later >= 0 && c->L[later].fuse_add == i) break;       // done by that convolution
+            DC_TRY(dc_launch_add(c, i, in, layer_input(c, L.d.in1)));
+            break;
+        }
         case DC_RELU: DC_TRY(dc_launch_relu(c, i, in)); break;
         case DC_LRN: {
             if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_lrn(c, i, in, L.map[0], nullptr)); break; }
@@ -674,7 +694,7 @@ int dc_cache_layer_conv_scheme(const dc_cache* c, int layer, int32_t* scheme)
     const dc_layer_rt& L = c->L[layer];
     if (L.d.kind != DC_CONV || !c->executable) { *scheme = -1; return DC_OK; }
     if (!dc_conv_bf16_supported(c, layer)) { *scheme = 0; return DC_OK; }
-    *scheme = (L.tc_mt > 0 ? L.tc_mt : 1) + (L.flat ? 7 : 0);
+    *scheme = L.tc_cs > 0 ? 10 : (L.tc_mt > 0 ? L.tc_mt : 1) + (L.flat ? 7 : 0);
     return DC_OK;
 }
 

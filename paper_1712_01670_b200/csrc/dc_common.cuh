@@ -51,6 +51,8 @@ struct dc_layer_rt {
     float* bias;                    // conv: [cout]
     void* weight_packed;            // conv, bf16: K-major tensor-core layout (see dc_conv_bf16.cu)
     int k_packed;                   // padded reduction length of weight_packed
+    int tc_cs;                      // conv, bf16: > 0: few tiles, a cluster of this many CTAs per tile and channel block (dc_conv_cluster.cu)
+    int fuse_add;                   // conv, bf16: the element-wise add layer that this layer's kernel does as well, or -1
     int tc_ctas;                    // conv, bf16: CTAs per SM the tuned launch uses (1 or 2)
     int tc_ew;                      // conv, bf16: epilogue warps per CTA (4, or 8 with one CTA per SM); 0 = 4
     int tc_mt, tc_bn;               // conv, bf16: tuned tiles per work item (3, 4: patch-reuse kernel with 1, 2; 5, 6: column-slab kernel) and
@@ -128,6 +130,7 @@ struct dc_cache {
     uint32_t* zero_masks;           // all-zero reuse bitmap shared by full frames
     int32_t* status;                // device status word
     void* input_map;                // frame / 255 as a map, [S][H][W][3]
+    const void* add_in; void* add_out; int add_relu;   // operands of the add that the next convolution launch does as well (NULL: none)
     bool fused_input;               // the frame goes straight into the operand copies of the convolutions that read it: no input map per frame
     int resize_feeds;               // few-channel convolution whose padded operand the resize layer writes as well, or -1
     void* stats_pinned;             // host staging for statistics

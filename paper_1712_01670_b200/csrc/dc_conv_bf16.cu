@@ -23,6 +23,8 @@
 #include <stdlib.h>
 
 #include "dc_common.cuh"
+#include "dc_conv_cluster.cuh"
+#include "dc_tcgen05.cuh"
 
 namespace {
 
@@ -66,44 +68,6 @@ constexpr int kStageBytes = 32 * 80;
 // Shared memory the control block takes with `epi_warps` epilogue warps (4 or 8).
 __host__ __device__ constexpr size_t ctl_bytes(int epi_warps) { return sizeof(SmemCtl) - (size_t)(8 - epi_warps) * kStageBytes; }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(void* bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(void* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(void* bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// Arrival that orders nothing but the barrier itself: used to hand a TMEM accumulator back (its reads are
-// ordered by tcgen05.wait::ld + tcgen05.fence), so the arrival need not wait for the epilogue's global stores.
-__device__ __forceinline__ void mbar_arrive_relaxed(void* bar)
-{
-    asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// Arrival on a barrier in the other CTA of a pair (addr: shared::cluster address from mapa).
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(void* bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ unsigned long long now_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
 // Bounded wait.  Returns false (and raises the abort flag + status word) when the limit passes
 // or another role has already given up.
 __device__ __forceinline__ bool mbar_wait(void* bar, uint32_t parity, SmemCtl* ctl, int32_t* status)
@@ -121,86 +85,6 @@ __device__ __forceinline__ bool mbar_wait(void* bar, uint32_t parity, SmemCtl* c
             }
         }
     }
-}
-
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, void* bar)
-{
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int c0, int c1, void* bar)
-{
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1) : "memory");
-}
-
-// K-major operand tile in shared memory.  Swizzled layouts: rows of BK bf16, 8-row groups `sbo`
-// bytes apart (lbo unused, 16).  Unswizzled layout (layout_type 0): 8-row x 16-byte core matrices,
-// `sbo` bytes apart along M/N and `lbo` bytes apart along K.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t sbo, uint32_t layout_type, uint32_t lbo = 16)
-{
-    uint32_t lo = ((saddr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);   // start address, LBO
-    uint32_t hi = ((sbo >> 4) & 0x3FFFu) | (1u << 14) | (layout_type << 29);   // SBO, descriptor version 1, swizzle
-    return ((uint64_t)hi << 32) | lo;
-}
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit(void* bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r)
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-                 "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
-{
-    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&v);
-}
-// 16-byte accesses to the epilogue's staging by shared-space address: through a generic pointer they would be
-// generic loads and stores, which resolve the address space first and wait on the long-latency scoreboard.
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-// (acc0 + b0, acc1 + b1) in fp32 (one packed add), then round to nearest even into two bf16; RELU clamps negative
-// results to zero in the same conversion (rounding is monotonic, so clamping before or after it gives the same value).
-template <bool RELU>
-__device__ __forceinline__ uint32_t bias_pack_bf16(uint32_t acc0, uint32_t acc1, float b0, float b1)
-{
-    uint32_t out;
-    if (RELU)
-        asm("{\n\t.reg .b64 a, b, d;\n\t.reg .f32 x, y;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
-            "add.rn.f32x2 d, a, b;\n\tmov.b64 {x, y}, d;\n\tcvt.rn.relu.bf16x2.f32 %0, y, x;\n\t}"
-            : "=r"(out) : "r"(acc0), "r"(acc1), "f"(b0), "f"(b1));
-    else
-        asm("{\n\t.reg .b64 a, b, d;\n\t.reg .f32 x, y;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
-            "add.rn.f32x2 d, a, b;\n\tmov.b64 {x, y}, d;\n\tcvt.rn.bf16x2.f32 %0, y, x;\n\t}"
-            : "=r"(out) : "r"(acc0), "r"(acc1), "f"(b0), "f"(b1));
-    return out;
 }
 
 // Copies the launch's bias values behind the control block (all threads; before the set-up's __syncthreads).  The
@@ -815,23 +699,6 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
 // thread is the only consumer.  Barriers: full / a_full / tmem_empty live in the leader and collect both CTAs;
 // empty / a_empty / tmem_full exist in each CTA and are signalled in both by the leader's tcgen05.commit.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t map_to_cta(const void* p, uint32_t rank)      // shared::cluster address of p in CTA `rank`
-{
-    uint32_t out;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(smem_u32(p)), "r"(rank));
-    return out;
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // loads into this CTA's shared memory whose bytes are counted on the barrier at shared::cluster address `bar` (the leader's)
 __device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, uint32_t bar)
 {
@@ -1553,35 +1420,10 @@ int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const
     return DC_OK;
 }
 
-static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* out, const int32_t* tile_list,
-                        const int32_t* tile_count, const uint32_t* masks, int max_tiles)
+// Tensor maps of the tap-by-tap kernels: the input (16 x 8 windows, or single row pieces for flat tiles) and the weights.
+static int generic_maps(dc_cache* c, dc_layer_rt& L, const dc_layer_desc& d, const TcPlan& p, const void* in, const void* weights, int cin_all, int cout_all,
+                        CUtensorMap** map_a, CUtensorMap** map_b)
 {
-    dc_layer_rt& L = c->L[layer];
-    if (L.flat && L.tc_mt > 2) return DC_ERR_CONFIG;              // flat tiles exist in the tap-by-tap kernel only
-    if (L.tc_mt == 7) return launch_pair(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
-    if (L.tc_mt >= 5) return launch_halo(c, layer, grp, L.tc_mt - 4, true, in, out, tile_list, tile_count, masks, max_tiles);
-    if (L.tc_mt >= 3) return launch_halo(c, layer, grp, L.tc_mt - 2, false, in, out, tile_list, tile_count, masks, max_tiles);
-    const bool grouped = n_groups(L.d) > 1;
-    const bool pad16 = !grouped && pad16_ok(L.d) && L.weight_packed && L.in_padded;
-    const dc_layer_desc d = pad16 ? padded16(L.d) : group_view(L.d);
-    const int cin_all = pad16 ? 16 : L.d.cin, cout_all = L.d.cout;
-    const void* weights = pad16 ? L.weight_packed : L.weight;
-    if (pad16) {
-        const size_t pixels = (size_t)c->S * L.in_h * L.in_w;
-        int grid_pad = (int)((pixels + 255) / 256); if (grid_pad > c->num_sms * 8) grid_pad = c->num_sms * 8;
-        dc_prof_scope ps(c, DC_ST_CONV);
-        DC_CUDA(dc_launch_pdl(k_pad_channels16, dim3((unsigned)grid_pad), 256, 0, c->stream, (const __nv_bfloat16*)in, pixels, (int)L.d.cin, (__nv_bfloat16*)L.in_padded));
-        c->launches += 1;
-        in = L.in_padded;
-    }
-    in = (const uint8_t*)in + (size_t)grp * d.cin * 2;            // the group's first input channel (grp = 0 when ungrouped)
-    TcPlan p;
-    int ctas = L.tc_ctas == 2 ? 2 : 1;
-    if (ctas == 2 && !make_plan(d, p, L.tc_mt, L.tc_bn, 2)) ctas = 1;
-    if (!make_plan(d, p, L.tc_mt, L.tc_bn, ctas)) {
-        if (smallc_ok(d)) return launch_smallc(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
-        return DC_ERR_CONFIG;
-    }
     EncodeTiledFn enc = encode_fn();
     if (!enc) return DC_ERR_CUDA;
     bool hit_a, hit_b;
@@ -1609,6 +1451,87 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
                 CU_TENSOR_MAP_INTERLEAVE_NONE, p.swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) { tm_drop(&L.tm_b, 1, tmBp); return DC_ERR_CUDA; }
     }
+    *map_a = tmAp; *map_b = tmBp;
+    return DC_OK;
+}
+
+// Few tiles: one cluster of L.tc_cs CTAs per tile and block of L.tc_bn channels.
+static bool cluster_plan(const dc_layer_desc& d, int bn, int cs, TcPlan& p)
+{
+    if (bn != 32 && bn != 64) return false;
+    t_ring_kb = 200; t_epi_warps = 4; t_bias_bytes = 0;
+    if (!make_plan(d, p, 1, bn, 1)) return false;
+    const int kiters = d.kh * d.kw * (d.cin / p.BK);
+    if (kiters < cs) return false;
+    const int most = dc_div_up(kiters, cs);
+    p.stages = most < kClusterStages ? most : kClusterStages;
+    while (p.stages > 1 && dc_cluster_smem(p.stages, p.a_bytes, p.b_bytes, p.BN) > 227 * 1024) --p.stages;
+    return p.stages >= 2 || most == 1;
+}
+
+static int launch_cluster(dc_cache* c, int layer, int grp, const void* in, void* out, const int32_t* tile_list,
+                          const int32_t* tile_count, const uint32_t* masks, int max_tiles)
+{
+    dc_layer_rt& L = c->L[layer];
+    const dc_layer_desc d = group_view(L.d);
+    TcPlan p;
+    if (!cluster_plan(d, L.tc_bn, L.tc_cs, p)) return DC_ERR_CONFIG;
+    in = (const uint8_t*)in + (size_t)grp * d.cin * 2;
+    CUtensorMap *tmAp, *tmBp;
+    const int rc = generic_maps(c, L, d, p, in, L.weight, L.d.cin, L.d.cout, &tmAp, &tmBp);
+    if (rc != DC_OK) return rc;
+    dc_cluster_args a;
+    a.bias = L.bias; a.out = (__nv_bfloat16*)out; a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;
+    a.Ho = d.out_h; a.Wo = d.out_w; a.Co = L.d.cout; a.Ci = d.cin; a.kh = d.kh; a.kw = d.kw; a.sh = d.sh; a.sw = d.sw;
+    a.ph = d.ph; a.pw = d.pw; a.relu = d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
+    a.BN = p.BN; a.NB = p.NB; a.BK = p.BK; a.kchunks = d.cin / p.BK; a.stages = p.stages; a.a_bytes = p.a_bytes; a.b_bytes = p.b_bytes;
+    a.nb_off = grp * p.NB; a.CS = L.tc_cs;
+    a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    a.sbo = p.sbo; a.layout_type = p.layout_type; a.tmem_cols = tmem_cols_for(1, 1, p.BN);
+    a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr;
+    a.status = c->status;
+    TcArgs w;
+    set_wait_limit(c, w);
+    a.wait_ns = w.wait_ns; a.skip_loads = w.skip_loads;
+    a.add_in = (const __nv_bfloat16*)c->add_in; a.add_out = (__nv_bfloat16*)c->add_out; a.add_relu = c->add_relu;
+    dc_prof_scope ps(c, DC_ST_CONV);
+    c->launches += 1;
+    return dc_launch_cluster_kernel(c, *tmAp, *tmBp, a, max_tiles);
+}
+
+static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* out, const int32_t* tile_list,
+                        const int32_t* tile_count, const uint32_t* masks, int max_tiles)
+{
+    dc_layer_rt& L = c->L[layer];
+    if (L.tc_cs > 0) return launch_cluster(c, layer, grp, in, out, tile_list, tile_count, masks, max_tiles);
+    if (L.flat && L.tc_mt > 2) return DC_ERR_CONFIG;              // flat tiles exist in the tap-by-tap kernel only
+    if (L.tc_mt == 7) return launch_pair(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
+    if (L.tc_mt >= 5) return launch_halo(c, layer, grp, L.tc_mt - 4, true, in, out, tile_list, tile_count, masks, max_tiles);
+    if (L.tc_mt >= 3) return launch_halo(c, layer, grp, L.tc_mt - 2, false, in, out, tile_list, tile_count, masks, max_tiles);
+    const bool grouped = n_groups(L.d) > 1;
+    const bool pad16 = !grouped && pad16_ok(L.d) && L.weight_packed && L.in_padded;
+    const dc_layer_desc d = pad16 ? padded16(L.d) : group_view(L.d);
+    const int cin_all = pad16 ? 16 : L.d.cin, cout_all = L.d.cout;
+    const void* weights = pad16 ? L.weight_packed : L.weight;
+    if (pad16) {
+        const size_t pixels = (size_t)c->S * L.in_h * L.in_w;
+        int grid_pad = (int)((pixels + 255) / 256); if (grid_pad > c->num_sms * 8) grid_pad = c->num_sms * 8;
+        dc_prof_scope ps(c, DC_ST_CONV);
+        DC_CUDA(dc_launch_pdl(k_pad_channels16, dim3((unsigned)grid_pad), 256, 0, c->stream, (const __nv_bfloat16*)in, pixels, (int)L.d.cin, (__nv_bfloat16*)L.in_padded));
+        c->launches += 1;
+        in = L.in_padded;
+    }
+    in = (const uint8_t*)in + (size_t)grp * d.cin * 2;            // the group's first input channel (grp = 0 when ungrouped)
+    TcPlan p;
+    int ctas = L.tc_ctas == 2 ? 2 : 1;
+    if (ctas == 2 && !make_plan(d, p, L.tc_mt, L.tc_bn, 2)) ctas = 1;
+    if (!make_plan(d, p, L.tc_mt, L.tc_bn, ctas)) {
+        if (smallc_ok(d)) return launch_smallc(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
+        return DC_ERR_CONFIG;
+    }
+    CUtensorMap *tmAp, *tmBp;
+    const int rc = generic_maps(c, L, d, p, in, weights, cin_all, cout_all, &tmAp, &tmBp);
+    if (rc != DC_OK) return rc;
     const CUtensorMap& tmA = *tmAp;
     const CUtensorMap& tmB = *tmBp;
     TcArgs a;
@@ -1659,7 +1582,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     cudaEvent_t e0, e1;
     DC_CUDA(cudaEventCreate(&e0));
     DC_CUDA(cudaEventCreate(&e1));
-    float best = 1e30f; int best_mt = L.tc_mt, best_bn = L.tc_bn, best_ctas = 1, best_flat = 0, best_ew = 4;
+    float best = 1e30f; int best_mt = L.tc_mt, best_bn = L.tc_bn, best_ctas = 1, best_flat = 0, best_ew = 4, best_cs = 0;
     constexpr int kTuneReps = 6;                                      // timed launches per candidate, after one untimed
     // the GPU may have been idle: bring the clocks up before the first candidate is timed
     for (int rep = 0; rep < 12; ++rep)
@@ -1668,10 +1591,10 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     // times the launch the current L.tc_* fields select; keeps it when it is the fastest so far
     // DC_CONV_SCHEME=<code> (diagnostics, tests): only candidates of that operand scheme are timed, so the scheme runs
     // wherever it can (1, 2 tap by tap; 3, 4 patch; 5, 6 column slabs; the second of each pair with two tiles per item;
-    // 7 column slabs on CTA pairs; 8, 9 tap by tap on flat tiles)
+    // 7 column slabs on CTA pairs; 8, 9 tap by tap on flat tiles; 10 tap by tap on clusters)
     const int only = getenv("DC_CONV_SCHEME") ? atoi(getenv("DC_CONV_SCHEME")) : 0;
     auto trial = [&](const char* what) {
-        if (only > 0 && generic && (L.flat ? L.tc_mt + 7 : L.tc_mt) != only) return;
+        if (only > 0 && generic && (L.tc_cs > 0 ? 10 : L.flat ? L.tc_mt + 7 : L.tc_mt) != only) return;
         int rc = DC_OK;
         for (int rep = 0; rep < kTuneReps + 1 && rc == DC_OK; ++rep) {
             if (rep == 1) cudaEventRecord(e0, c->stream);
@@ -1681,9 +1604,9 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
         if (rc != DC_OK || cudaEventSynchronize(e1) != cudaSuccess) { cudaGetLastError(); return; }
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        if (verbose) fprintf(stderr, "libdeepcache: layer %d: %s, tiles/item code %d, %d channels per block, %d CTA(s) per SM, %d epilogue warps: %.3f ms\n",
-                             layer, what, L.flat ? L.tc_mt + 7 : L.tc_mt, L.tc_bn, L.tc_ctas, L.tc_ew, ms / kTuneReps);
-        if (ms < best) { best = ms; best_mt = L.tc_mt; best_bn = L.tc_bn; best_ctas = L.tc_ctas; best_flat = L.flat; best_ew = L.tc_ew; }
+        if (verbose) fprintf(stderr, "libdeepcache: layer %d: %s, tiles/item code %d, %d channels per block, %d CTA(s) per SM, %d epilogue warps, clusters of %d: %.4f ms\n",
+                             layer, what, L.flat ? L.tc_mt + 7 : L.tc_mt, L.tc_bn, L.tc_ctas, L.tc_ew, L.tc_cs, ms / kTuneReps);
+        if (ms < best) { best = ms; best_mt = L.tc_mt; best_bn = L.tc_bn; best_ctas = L.tc_ctas; best_flat = L.flat; best_ew = L.tc_ew; best_cs = L.tc_cs; }
     };
     // one CTA per SM with four or eight epilogue warps, or two CTAs per SM with four each
     for (int shape = 0; shape < 3; ++shape) {
@@ -1734,11 +1657,28 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
             trial("CTA-pair kernel");
         }
     }
-    L.tc_mt = best_mt; L.tc_bn = best_bn; L.tc_ctas = best_ctas; L.flat = best_flat; L.tc_ew = best_ew;
+    // few tiles: the reduction split over clusters of CTAs, while that gives no more than three CTAs per SM
+    if (generic && !(de.cin < 16) && L.d.cin == de.cin * n_groups(L.d)) {
+        L.tc_mt = 1; L.tc_ctas = 1; L.tc_ew = 4;
+        for (int flat = 0; flat < 2; ++flat) {
+            if (flat && L.tiles_flat * 20 > L.tiles_x * L.tiles_y * c->S * 19) continue;
+            L.flat = flat;
+            for (int bn = 32; bn <= 64; bn += 32)
+                for (int cs = 2; cs <= 8; cs *= 2) {
+                    TcPlan q;
+                    if (de.cout % bn != 0 || !cluster_plan(de, bn, cs, q)) continue;
+                    if ((long long)dc_layer_tiles(c, L) * (de.cout / bn) * cs > 3LL * c->num_sms && only != 10) continue;
+                    L.tc_bn = bn; L.tc_cs = cs;
+                    trial("cluster kernel");
+                }
+        }
+        L.tc_cs = 0; L.flat = 0;
+    }
+    L.tc_mt = best_mt; L.tc_bn = best_bn; L.tc_ctas = best_ctas; L.flat = best_flat; L.tc_ew = best_ew; L.tc_cs = best_cs;
     cudaEventDestroy(e0); cudaEventDestroy(e1);
     c->launches = 0;
-    if (verbose) fprintf(stderr, "libdeepcache: layer %d: chose code %d, %d channels per block, %d CTA(s) per SM, %d epilogue warps (%.3f ms)\n",
-                         layer, best_flat ? best_mt + 7 : best_mt, best_bn, best_ctas, best_ew, best / kTuneReps);
+    if (verbose) fprintf(stderr, "libdeepcache: layer %d: chose code %d, %d channels per block, %d CTA(s) per SM, %d epilogue warps, clusters of %d (%.4f ms)\n",
+                         layer, best_flat ? best_mt + 7 : best_mt, best_bn, best_ctas, best_ew, best_cs, best / kTuneReps);
     return DC_OK;
 }
 

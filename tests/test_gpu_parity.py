@@ -604,6 +604,19 @@ def test_conv_wide_layers_on_cta_pairs(scheme, hi, wi, cin, cout, k, p, monkeypa
     _one_layer_full_and_partial(hi, wi, cin, cout, k, 1, p, 3, scheme)
 
 
+@pytest.mark.parametrize("hi,wi,cin,cout,k,st,p,S", [
+    (7, 7, 512, 64, 3, 1, 1, 1),         # one tile, more steps per CTA than ring slots
+    (7, 7, 128, 256, 1, 1, 0, 5),        # two steps in all: clusters of two
+    (14, 14, 64, 96, 3, 2, 1, 3),        # strided, 32-channel blocks, 7 x 7 output
+    (13, 21, 48, 64, 3, 1, 1, 2),        # 16-channel steps, 32-byte operand rows
+    (17, 9, 32, 32, 5, 1, 2, 2),         # 64-byte operand rows, partial tiles
+])
+def test_conv_on_clusters(hi, wi, cin, cout, k, st, p, S, monkeypatch):
+    """Few tiles: the reduction split over a cluster of CTAs, full and partial convolution (scheme 10)."""
+    monkeypatch.setenv("DC_CONV_SCHEME", "10")
+    _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, 10)
+
+
 @pytest.mark.parametrize("scheme", [8, 9])
 @pytest.mark.parametrize("hi,wi,cin,cout,k,st,p,S", [
     (7, 7, 128, 256, 3, 1, 1, 5),        # 7 pieces per stream: every tile holds pieces of two or three streams
