@@ -4,15 +4,15 @@
 // dc_conv_bf16.cu then run on a handful of SMs, each walking all taps and channels alone (512 -> 512, 3x3 at 7x7: 4 CTAs,
 // 72 steps, 32 us).  Here a work item - one tile, a narrow block of BN = 32 or 64 output channels - belongs to a cluster of
 // CS = 2, 4 or 8 CTAs.  Each takes 1 / CS of the (tap, channel chunk) steps, operands and MMA as in the tap-by-tap kernel;
-// the partial sums meet through distributed shared memory: every CTA leaves its 128 x BN floats in its own shared
-// memory, and after a cluster barrier finishes 128 / CS of the pixels from all CS copies, in rank order.  The weights do not
-// depend on any kernel before, so their loads start before the wait for the previous layer.
-// What bounds it: the chain of latencies of one item (tile list, one TMA round trip, the cluster barrier, the remote
-// reads), about 4 us, and no longer the length of the reduction.
+// the partial sums meet through distributed shared memory: CTA r finishes pixels r * 128 / CS ..., and every CTA writes its
+// sums of those pixels into r's shared memory; after one cluster barrier each CTA adds its CS copies in rank order,
+// without touching the others again.  The weights do not depend on any kernel before, so their loads start before the
+// wait for the previous layer.
+// What bounds it: the chain of latencies of one item (tile list, one TMA round trip, the cluster barrier), and no longer
+// the length of the reduction.
 //
 // An element-wise add that follows (a residual block's end) can be done in the same pass over the tile: reused pixels
-// are read back from the output map, where the reuse copy has put them.  Such a launch visits every tile; a tile without
-// a pixel to compute skips its loads and MMAs.
+// are read back from the output map, where the reuse copy has put them.  Such a launch visits every tile.
 #include "dc_conv_cluster.cuh"
 #include "dc_tcgen05.cuh"
 
@@ -44,11 +44,9 @@ __device__ __forceinline__ bool cl_wait(void* bar, uint32_t parity, CtlCl* ctl, 
         }
     }
 }
-__device__ __forceinline__ float4 ld_remote(uint32_t addr)
+__device__ __forceinline__ void st_remote(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
 }
 // padded row of partial sums: 16-byte accesses of neighbouring lanes fall in different banks
 __host__ __device__ constexpr int red_pitch(int BN) { return BN + 4; }
@@ -58,7 +56,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     extern __shared__ uint8_t smem_raw[];
     uint8_t* ring = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int stage_bytes = a.a_bytes + a.b_bytes;
-    float* red = (float*)(ring + (size_t)a.stages * stage_bytes);            // [128][BN + 4]
+    float* red = (float*)(ring + (size_t)a.stages * stage_bytes);            // [CS][128 / CS][BN + 4]: this CTA's pixels, from every CTA
     CtlCl* ctl = (CtlCl*)(red + 128 * red_pitch(a.BN));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank(), item = blockIdx.x / a.CS, nb = item % a.NB, idx = item / a.NB;
@@ -80,6 +78,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     }
     tc_fence_before();
     __syncthreads();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");    // waited for before another CTA's shared memory is written
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
     auto load_weights = [&](int it) {
@@ -113,20 +112,29 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         s = ts; y = ty * DC_TILE_H + row; x0 = tx * DC_TILE_W;
         return y < a.Ho;
     };
-    // which pixels of a tile row have to be computed
-    auto todo_of = [&](int row) -> uint32_t {
-        int s, y, x0;
-        if (!locate(row, s, y, x0)) return 0u;
-        uint32_t m = ~(a.masks[(size_t)tile * 4 + (row >> 2)] >> (8 * (row & 3))) & 0xffu;
-        if (a.Wo - x0 < DC_TILE_W) m &= (1u << (a.Wo - x0)) - 1u;
-        return m;
+    // What thread u finishes: 8 channels of one of this CTA's pixels.  The first unit's operands are fetched now, beside
+    // the loads and MMAs.
+    const int rows = 128 / a.CS, per_px = a.BN / 8, units = present ? rows * per_px : 0;
+    struct Unit { size_t at; uint4 other; float4 b0, b1; bool in_map, active; };
+    auto unit_of = [&](int u) -> Unit {
+        Unit n;
+        const int pr = u / per_px, c8 = u - pr * per_px, m = rank * rows + pr, row = m / DC_TILE_W, col = m % DC_TILE_W;
+        int s = 0, y = 0, x0 = 0;
+        n.in_map = locate(row, s, y, x0) && x0 + col < a.Wo;
+        n.active = n.in_map && !((a.masks[(size_t)tile * 4 + (row >> 2)] >> (8 * (row & 3) + col)) & 1u);
+        const int ch = (nb + a.nb_off) * a.BN + c8 * 8;
+        n.at = (((size_t)s * a.Ho + y) * a.Wo + x0 + col) * a.Co + ch;
+        n.b0 = __ldg((const float4*)(a.bias + ch)); n.b1 = __ldg((const float4*)(a.bias + ch + 4));
+        n.other = n.in_map && a.add_out ? *(const uint4*)(a.add_in + n.at) : make_uint4(0, 0, 0, 0);
+        return n;
     };
-    const bool work = present && __any_sync(0xffffffffu, todo_of(lane & 15) != 0);    // the same in all warps of the cluster
+    Unit mine = {};
+    if ((int)threadIdx.x < units) mine = unit_of(threadIdx.x);
 
     if (warp == 0) {
         // ---------------- producer ----------------
         bool ok = true;
-        if (!work) {
+        if (!present) {
             // the weights are on their way: let them land before this CTA's shared memory is given up
             if (lane == 0 && !a.skip_loads)
                 for (int it = 0; it < early && ok; ++it) { mbar_arrive(&ctl->full[it]); ok = cl_wait(&ctl->full[it], 0, ctl, a.status); }
@@ -161,7 +169,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0 && work) {
+        if (lane == 0 && present) {
             const uint64_t dconst = umma_desc(0, a.sbo, a.layout_type);
             const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
             const int ksteps = a.BK / 16;
@@ -178,57 +186,46 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
             if (ok) umma_commit(&ctl->done);
         }
         __syncwarp();
-    } else if (work) {
-        // ---------------- partial sums to shared memory ----------------
+    } else if (present) {
+        // ---------------- partial sums to the CTA that finishes the pixel ----------------
         const int q = warp & 3, m = q * 32 + lane;                   // tensor-memory lane quadrant of this warp, its pixel
-        const bool ok = cl_wait(&ctl->done, 0, ctl, a.status);
-        if (__all_sync(0xffffffffu, ok)) {
+        const int owner = m / rows;
+        const uint32_t dst = map_to_cta(red + (rank * rows + m - owner * rows) * red_pitch(a.BN), (uint32_t)owner);
+        bool ok = cl_wait(&ctl->done, 0, ctl, a.status);
+        ok = __all_sync(0xffffffffu, ok);
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (ok) {
             tc_fence_after();
-            const uint32_t dst = smem_u32(red + m * red_pitch(a.BN));
             for (int c = 0; c < a.BN / 32; ++c) {
                 uint32_t r[32];
                 tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + c * 32, r);
                 tmem_ld_wait();
 #pragma unroll
-                for (int v = 0; v < 8; ++v) sts128(dst + c * 128 + v * 16, r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+                for (int v = 0; v < 8; ++v) st_remote(dst + c * 128 + v * 16, r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
             }
         }
         tc_fence_before();
     }
-    cluster_sync_all();                      // every CTA's sums are in its shared memory
+    if (warp < 2 || !present) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // (the accumulator warps have waited)
+    cluster_sync_all();                      // this CTA's pixels have arrived from every CTA
     const bool dead = ctl->abort_flag != 0;  // an aborted launch's sums are not valid: nothing is stored
-    if (present && !dead && (work || a.add_out)) {
-        // ---------------- this CTA's pixels: sums of all ranks, bias, ReLU, bf16, store ----------------
-        const int rows = 128 / a.CS, per_px = a.BN / 8;
-        uint32_t base[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) base[r] = map_to_cta(red, (uint32_t)(r < a.CS ? r : 0));
-        for (int u = threadIdx.x; u < rows * per_px; u += kThreadsCl) {
-            const int pr = u / per_px, c8 = u - pr * per_px, m = rank * rows + pr, row = m / DC_TILE_W, col = m % DC_TILE_W;
-            int s, y, x0;
-            if (!locate(row, s, y, x0) || x0 + col >= a.Wo) continue;
-            const bool active = (todo_of(row) >> col) & 1u;
-            if (!active && !a.add_out) continue;
-            const int ch = (nb + a.nb_off) * a.BN + c8 * 8;
-            const size_t at = (((size_t)s * a.Ho + y) * a.Wo + x0 + col) * a.Co + ch;
+    if (!dead) {
+        // ---------------- this CTA's pixels: sums from all ranks, bias, ReLU, bf16, store ----------------
+        for (int u = threadIdx.x; u < units; u += kThreadsCl) {
+            if (u != (int)threadIdx.x) mine = unit_of(u);
+            if (!mine.in_map || (!mine.active && !a.add_out)) continue;
             uint4 o;
-            if (active) {
-                float v[8];
-                const float4 b0 = __ldg((const float4*)(a.bias + ch)), b1 = __ldg((const float4*)(a.bias + ch + 4));
-                float4 p0[8], p1[8];
-                const uint32_t off = (uint32_t)(m * red_pitch(a.BN) + c8 * 8) * 4u;
-#pragma unroll
-                for (int r = 0; r < 8; ++r)
-                    if (r < a.CS) { p0[r] = ld_remote(base[r] + off); p1[r] = ld_remote(base[r] + off + 16); }
-                float4 s0 = p0[0], s1 = p1[0];
-#pragma unroll
-                for (int r = 1; r < 8; ++r)
-                    if (r < a.CS) {
-                        s0.x += p0[r].x; s0.y += p0[r].y; s0.z += p0[r].z; s0.w += p0[r].w;
-                        s1.x += p1[r].x; s1.y += p1[r].y; s1.z += p1[r].z; s1.w += p1[r].w;
-                    }
-                v[0] = s0.x + b0.x; v[1] = s0.y + b0.y; v[2] = s0.z + b0.z; v[3] = s0.w + b0.w;
-                v[4] = s1.x + b1.x; v[5] = s1.y + b1.y; v[6] = s1.z + b1.z; v[7] = s1.w + b1.w;
+            if (mine.active) {
+                const float* p = red + (u / per_px) * red_pitch(a.BN) + (u % per_px) * 8;
+                float4 s0 = *(const float4*)p, s1 = *(const float4*)(p + 4);
+                for (int r = 1; r < a.CS; ++r) {
+                    p += rows * red_pitch(a.BN);
+                    const float4 p0 = *(const float4*)p, p1 = *(const float4*)(p + 4);
+                    s0.x += p0.x; s0.y += p0.y; s0.z += p0.z; s0.w += p0.w;
+                    s1.x += p1.x; s1.y += p1.y; s1.z += p1.z; s1.w += p1.w;
+                }
+                float v[8] = {s0.x + mine.b0.x, s0.y + mine.b0.y, s0.z + mine.b0.z, s0.w + mine.b0.w,
+                              s1.x + mine.b1.x, s1.y + mine.b1.y, s1.z + mine.b1.z, s1.w + mine.b1.w};
                 if (a.relu) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k) v[k] = fmaxf(v[k], 0.f);
@@ -237,27 +234,13 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
 #pragma unroll
                 for (int k = 0; k < 4; ++k) h[k] = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
                 o = *(const uint4*)h;
-                *(uint4*)(a.out + at) = o;
+                *(uint4*)(a.out + mine.at) = o;
             } else {
-                o = *(const uint4*)(a.out + at);                     // filled from the cache
+                o = *(const uint4*)(a.out + mine.at);                // filled from the cache
             }
-            if (a.add_out) {
-                const uint4 w = *(const uint4*)(a.add_in + at);
-                const uint32_t x[4] = {o.x, o.y, o.z, o.w}, z[4] = {w.x, w.y, w.z, w.w};
-                uint32_t r[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {                        // fp32 sum, one rounding to bf16 (as the add layer's own kernel)
-                    float lo = __uint_as_float(x[k] << 16) + __uint_as_float(z[k] << 16);
-                    float hi = __uint_as_float(x[k] & 0xffff0000u) + __uint_as_float(z[k] & 0xffff0000u);
-                    if (a.add_relu) { lo = fmaxf(lo, 0.f); hi = fmaxf(hi, 0.f); }
-                    const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
-                    r[k] = *(const uint32_t*)&t;
-                }
-                *(uint4*)(a.add_out + at) = make_uint4(r[0], r[1], r[2], r[3]);
-            }
+            if (a.add_out) *(uint4*)(a.add_out + mine.at) = add_bf16x8(o, mine.other, a.add_relu);
         }
     }
-    cluster_sync_all();                      // nobody leaves while its sums may still be read
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(a.tmem_cols) : "memory");

@@ -120,6 +120,22 @@ __device__ __forceinline__ uint32_t bias_pack_bf16(uint32_t acc0, uint32_t acc1,
     return out;
 }
 
+// a + b (+ ReLU) of eight bf16: fp32 sums, each rounded once (as the add layer's own kernel)
+__device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b, int relu)
+{
+    const uint32_t x[4] = {a.x, a.y, a.z, a.w}, z[4] = {b.x, b.y, b.z, b.w};
+    uint32_t r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float lo = __uint_as_float(x[k] << 16) + __uint_as_float(z[k] << 16);
+        float hi = __uint_as_float(x[k] & 0xffff0000u) + __uint_as_float(z[k] & 0xffff0000u);
+        if (relu) { lo = fmaxf(lo, 0.f); hi = fmaxf(hi, 0.f); }
+        const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+        r[k] = *(const uint32_t*)&t;
+    }
+    return make_uint4(r[0], r[1], r[2], r[3]);
+}
+
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;
