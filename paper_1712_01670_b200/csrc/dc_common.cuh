@@ -62,6 +62,7 @@ struct dc_layer_rt {
     float* weight_simt;             // conv on the register-blocked CUDA-core kernel: its packed weights (dc_conv_simt.cu)
     void* in_padded;                // conv, bf16, cin <= 8: input with channels padded to 8
     void* in_s2d;                   // conv, bf16, strided over few channels: the space-to-depth copy of the input the rewritten layer reads (dc_conv_s2d.cu)
+    int s2d_ws, s2d_cs;             // ... columns of the block map and channels of its pixels
     int s2d_s, s2d_py, s2d_px, s2d_cin, s2d_hi, s2d_wi;   // ... its block size (0: layer as declared), leading zero rows / columns, and the input as declared
     uint32_t* masks;                // conv: [S][tiles_y][tiles_x][4] reuse bitmap of each tile
     int32_t* dirty_list;            // conv: compacted tiles needing computation
@@ -120,6 +121,7 @@ struct dc_cache {
     dc_region* regions0;            // [S][max_regions] rectangles on the frame
     int32_t* n_regions;             // [S]
     dc_region* table;               // [n_layers][S][max_regions]
+    int prop_slots;                 // rectangles a thread of region propagation keeps for later layers
     void* prop_table;               // [n_layers] the layer table as region propagation reads it (dc_regions.cu)
     int32_t* dirty_count;           // [n_layers]
     int32_t* partial;               // dc_conv_partial: two dirty counters used in turn (each call zeroes the other), then [S] reused pixels (not read)

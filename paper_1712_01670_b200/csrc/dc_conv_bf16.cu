@@ -498,7 +498,7 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Input-patch reuse ("halo") variant for stride-1 k x k convolutions with cin a multiple of 64.
+// Input-patch reuse ("halo") variant for stride-1 k x k convolutions with cin a multiple of 16.
 // k_conv_tc fetches the 16x8 input window once per kernel tap (9 x 16 KB for 3x3); here the
 // (16 + kh - 1) x (8 + kw - 1) patch is fetched ONCE per 64-channel chunk and every tap reads it
 // in place.  That needs an operand layout whose rows may start at any patch pixel: the
@@ -513,6 +513,7 @@ struct TcHaloArgs {
     TcArgs t;
     const __nv_bfloat16* wpacked;    // [NB][taps][kchunks][8][BN][8]
     int PW, PH, plane_bytes, patch_bytes, a_stages;
+    int k_last;                      // K steps of 16 channels in the last chunk (4 unless the channels are no multiple of 64)
 };
 
 __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32_t bytes, void* bar)
@@ -640,6 +641,7 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
+                    const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < (SLAB ? a.kw : 1) && ok; ++ax) {     // A stages of this chunk: one patch, or kw slabs
                         ok = mbar_wait(&ctl->a_full[sa], pa, ctl, a.status);
                         const uint64_t apatch = aconst + (aring_lo + (uint32_t)sa * a_slot_lo);
@@ -656,8 +658,8 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                                 const uint64_t adesc = apatch + j * patch_lo + tap_lo;
                                 uint32_t acc_j = accumulate;
 #pragma unroll
-                                for (int kk = 0; kk < 4; ++kk) {        // K = 16 per instruction, 64 channels per chunk
-                                    umma_f16(d_tmem + j * a.BN, adesc + kk * a_kstep, bdesc + kk * b_kstep, a.idesc, acc_j);
+                                for (int kk = 0; kk < 4; ++kk) {        // K = 16 per instruction, up to 64 channels per chunk
+                                    if (kk < n_kk) umma_f16(d_tmem + j * a.BN, adesc + kk * a_kstep, bdesc + kk * b_kstep, a.idesc, acc_j);
                                     acc_j = 1;
                                 }
                             }
@@ -823,6 +825,7 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
+                    const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < a.kw && ok; ++ax) {
                         ok = mbar_wait(&ctl->a_full[sa], pa, ctl, a.status);
                         const uint64_t aslab = aconst + (aring_lo + (uint32_t)sa * a_slot_lo);
@@ -833,8 +836,8 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             const uint64_t bdesc = bconst + (bring_lo + (uint32_t)sb * b_lo);
                             const uint64_t adesc = aslab + (uint32_t)t * 64u;
 #pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {                 // K = 16 per instruction, 64 channels per chunk
-                                umma_f16_pair(d_tmem, adesc + kk * 2u, bdesc + kk * b_kstep, a.idesc, accumulate);
+                            for (int kk = 0; kk < 4; ++kk) {                 // K = 16 per instruction, up to 64 channels per chunk
+                                if (kk < n_kk) umma_f16_pair(d_tmem, adesc + kk * 2u, bdesc + kk * b_kstep, a.idesc, accumulate);
                                 accumulate = 1;
                             }
                             umma_commit_pair(&ctl->empty[sb]);
@@ -863,11 +866,11 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
 }
 
-// weights [cout][taps][cin] -> [NB][taps][kchunks][8][BN][8]
+// weights [cout][taps][cin] -> [NB][taps][kchunks][8][BN][8], zeros beyond the last channel
 __global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin, int BN, __nv_bfloat16* out)
 {
-    const int kchunks = cin / 64;
-    const size_t total = (size_t)cout * taps * cin;
+    const int kchunks = (cin + 63) / 64;
+    const size_t total = (size_t)cout * taps * kchunks * 64;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         size_t r = i;
         const int e = (int)(r & 7); r >>= 3;
@@ -875,7 +878,8 @@ __global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin,
         const int k8 = (int)(r & 7); r >>= 3;
         const int cc = (int)(r % kchunks); r /= kchunks;
         const int tap = (int)(r % taps); const int nb = (int)(r / taps);
-        out[i] = w[((size_t)(nb * BN + n) * taps + tap) * cin + cc * 64 + k8 * 8 + e];
+        const int ch = cc * 64 + k8 * 8 + e;
+        out[i] = ch < cin ? w[((size_t)(nb * BN + n) * taps + tap) * cin + ch] : __float2bfloat16(0.f);
     }
 }
 
@@ -1021,6 +1025,16 @@ static dc_layer_desc group_view(const dc_layer_desc& d)
     return g;
 }
 
+// Elements from one input pixel, and one input row, to the next.  A block map whose kernel columns were merged into channels
+// (dc_conv_s2d.cu) has windows of several pixels as its pixels: they overlap.
+struct InPitch { cuuint64_t px, row; };
+static InPitch in_pitch(const dc_layer_rt& L, int cin)
+{
+    InPitch p = {(cuuint64_t)cin, (cuuint64_t)L.in_w * cin};
+    if (L.s2d_s) { p.px = (cuuint64_t)L.s2d_cs; p.row = (cuuint64_t)L.s2d_ws * L.s2d_cs; }
+    return p;
+}
+
 struct TcPlan { int BK, BN, NB, MT, nbuf, stages, a_bytes, b_bytes; CUtensorMapSwizzle swz; uint32_t layout_type, sbo; size_t smem; };
 
 bool make_plan(const dc_layer_desc& d, TcPlan& p, int want_mt = 0, int want_bn = 0, int ctas = 1)
@@ -1055,11 +1069,13 @@ bool make_plan(const dc_layer_desc& d, TcPlan& p, int want_mt = 0, int want_bn =
     return true;
 }
 
-struct HaloPlan { int BN, NB, PW, PH, plane_bytes, patch_bytes, b_bytes; };
+// Channels that are no multiple of 64 (AlexNet's 96, or 48 per group): the last chunk's missing channels are zero-filled by
+// the loads, the packed weights have zeros there, and the chunk's K steps without a channel are left out.
+struct HaloPlan { int BN, NB, PW, PH, plane_bytes, patch_bytes, b_bytes, kchunks, k_last; };
 
 bool halo_ok(const dc_layer_desc& d, HaloPlan& h, int want_bn = 0)
 {
-    if (d.kind != DC_CONV || d.sh != 1 || d.sw != 1 || d.cin % 64 != 0 || d.kh * d.kw < 2 || d.kh > 5 || d.kw > 5) return false;
+    if (d.kind != DC_CONV || d.sh != 1 || d.sw != 1 || d.cin % 16 != 0 || d.kh * d.kw < 2 || d.kh > 5 || d.kw > 5) return false;
     h.BN = 0;
     for (int bn = 256; bn >= 32; bn -= 32) if (d.cout % bn == 0) { h.BN = bn; break; }
     if (!h.BN) return false;
@@ -1072,6 +1088,7 @@ bool halo_ok(const dc_layer_desc& d, HaloPlan& h, int want_bn = 0)
     h.plane_bytes = (h.PW * h.PH * 16 + 127) & ~127;       // TMA destinations are 128-byte aligned
     h.patch_bytes = 8 * h.plane_bytes;
     h.b_bytes = h.BN * 128;
+    h.kchunks = (d.cin + 63) / 64; h.k_last = (d.cin - (h.kchunks - 1) * 64 + 15) / 16;
     return true;
 }
 
@@ -1125,7 +1142,7 @@ int dc_pack_weights_bf16(dc_cache* c, int layer)
     const dc_layer_desc dg = group_view(L.d);                     // the layer itself when it is not grouped
     if (halo_ok(dg, h)) {
         // [cout][taps][cin / groups]: channel blocks never straddle a group (BN divides cout / groups)
-        const size_t n = (size_t)L.d.cout * L.d.kh * L.d.kw * dg.cin;
+        const size_t n = (size_t)L.d.cout * L.d.kh * L.d.kw * h.kchunks * 64;
         DC_CUDA(cudaMalloc(&L.weight_halo, n * 2));
         c->bytes += n * 2;
         int grid = (int)((n + 255) / 256); if (grid > c->num_sms * 8) grid = c->num_sms * 8;
@@ -1233,7 +1250,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     if (L.halo_bn != h.BN) {
         // the packed weights are grouped by channel block: another block width needs another packing (same size).
         // Happens while the tuner tries widths and once more for its final choice, never in steady state.
-        const size_t n = (size_t)cout_all * d.kh * d.kw * d.cin;
+        const size_t n = (size_t)cout_all * d.kh * d.kw * h.kchunks * 64;
         int pgrid = (int)((n + 255) / 256); if (pgrid > c->num_sms * 8) pgrid = c->num_sms * 8;
         k_pack_halo<<<pgrid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, cout_all, d.kh * d.kw, d.cin, h.BN,
                                                   (__nv_bfloat16*)L.weight_halo);
@@ -1244,7 +1261,8 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, slab ? 5 : 3, 0, &hit);
     if (!hit) {
         cuuint64_t dims[4] = {(cuuint64_t)d.cin, (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
-        cuuint64_t strides[3] = {(cuuint64_t)cin_all * 2, (cuuint64_t)L.in_w * cin_all * 2, (cuuint64_t)L.in_h * L.in_w * cin_all * 2};
+        const InPitch ip = in_pitch(L, cin_all);
+        cuuint64_t strides[3] = {ip.px * 2, ip.row * 2, (cuuint64_t)L.in_h * ip.row * 2};
         cuuint32_t box[4] = {8, (cuuint32_t)h.PW, (cuuint32_t)h.PH, 1};
         if (slab) { box[0] = 64; box[1] = DC_TILE_W; }            // a column slab: 64 channels x 8 pixels x PH rows
         cuuint32_t estr[4] = {1, 1, 1, 1};
@@ -1261,12 +1279,13 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     a.bias = L.bias; a.out = (__nv_bfloat16*)out; a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;
     a.Ho = d.out_h; a.Wo = d.out_w; a.Co = cout_all; a.Ci = d.cin; a.kh = d.kh; a.kw = d.kw; a.sh = 1; a.sw = 1;
     a.ph = d.ph; a.pw = d.pw; a.relu = d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
-    a.BN = h.BN; a.NB = h.NB; a.nb_off = grp * h.NB; a.BK = 64; a.kchunks = d.cin / 64; a.MT = mt; a.nbuf = mt * h.BN * 2 <= 512 ? 2 : 1;
+    a.BN = h.BN; a.NB = h.NB; a.nb_off = grp * h.NB; a.BK = 64; a.kchunks = h.kchunks; a.MT = mt; a.nbuf = mt * h.BN * 2 <= 512 ? 2 : 1;
     a.a_bytes = 0; a.b_bytes = h.b_bytes; a.sbo = 128; a.layout_type = 0;
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(h.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.status = c->status;
     set_wait_limit(c, a);
     ha.wpacked = (const __nv_bfloat16*)L.weight_halo;
+    ha.k_last = h.k_last;
     ha.PW = h.PW; ha.PH = h.PH; ha.plane_bytes = h.plane_bytes;
     ha.patch_bytes = slab ? h.PH * DC_TILE_W * 128 : h.patch_bytes;
     // patch ring: as deep as leaves at least 3 weight stages (a small-K item is one patch, so depth = items in flight)
@@ -1306,7 +1325,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     return DC_OK;
 }
 
-// The CTA-pair kernel takes stride-1 layers with cin a multiple of 64 (the column-slab conditions) whose output
+// The CTA-pair kernel takes stride-1 layers with cin a multiple of 16 (the column-slab conditions) whose output
 // channels divide into blocks of 256 or 128 (half a block per CTA).
 static bool pair_ok(const dc_layer_desc& d, int& bn)
 {
@@ -1323,10 +1342,11 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     const dc_layer_desc& d = L.d;
     EncodeTiledFn enc = encode_fn();
     int bn = 0;
-    if (!enc || !L.weight_halo || !pair_ok(d, bn)) return DC_ERR_CONFIG;
-    const int half = bn / 2, taps = d.kh * d.kw, kchunks = d.cin / 64;
+    HaloPlan h;
+    if (!enc || !L.weight_halo || !pair_ok(d, bn) || !halo_ok(d, h)) return DC_ERR_CONFIG;
+    const int half = bn / 2, taps = d.kh * d.kw, kchunks = h.kchunks;
     if (L.halo_bn != half) {                                     // weights grouped by half blocks: [2 NB][taps][kchunks][8][half][8]
-        const size_t n = (size_t)d.cout * taps * d.cin;
+        const size_t n = (size_t)d.cout * taps * kchunks * 64;
         int pgrid = (int)((n + 255) / 256); if (pgrid > c->num_sms * 8) pgrid = c->num_sms * 8;
         k_pack_halo<<<pgrid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, d.cout, taps, d.cin, half, (__nv_bfloat16*)L.weight_halo);
         L.halo_bn = half;
@@ -1336,7 +1356,8 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, 5, 0, &hit_a);     // the column-slab map of the single-CTA kernel
     if (!hit_a) {
         cuuint64_t dims[4] = {(cuuint64_t)d.cin, (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
-        cuuint64_t strides[3] = {(cuuint64_t)d.cin * 2, (cuuint64_t)L.in_w * d.cin * 2, (cuuint64_t)L.in_h * L.in_w * d.cin * 2};
+        const InPitch ip = in_pitch(L, d.cin);
+        cuuint64_t strides[3] = {ip.px * 2, ip.row * 2, (cuuint64_t)L.in_h * ip.row * 2};
         cuuint32_t box[4] = {64, DC_TILE_W, (cuuint32_t)PH, 1};
         cuuint32_t estr[4] = {1, 1, 1, 1};
         if (enc(tmAp, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(in), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1348,7 +1369,7 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     const int b_bytes = half * 128;                              // one CTA's weight tile: half rows of 64 channels
     CUtensorMap* tmWp = tm_find(&L.tm_b, 1, nullptr, L.weight_halo, 7, half, &hit_b);
     if (!hit_b) {                                                // the packed weights as rows of 128 bytes; a box is one tile
-        const cuuint64_t rows = (cuuint64_t)d.cout * taps * d.cin * 2 / 128;
+        const cuuint64_t rows = (cuuint64_t)d.cout * taps * kchunks;
         cuuint64_t dims[2] = {64, rows};
         cuuint64_t strides[1] = {128};
         cuuint32_t box[2] = {64, (cuuint32_t)(b_bytes / 128)};
@@ -1372,6 +1393,7 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     set_wait_limit(c, a);
     a.tmem_cols = tmem_cols_for(2, 1, bn);
     ha.wpacked = (const __nv_bfloat16*)L.weight_halo;
+    ha.k_last = h.k_last;
     ha.PW = DC_TILE_W; ha.PH = PH; ha.plane_bytes = 0;
     ha.patch_bytes = PH * DC_TILE_W * 128;                       // one slab
     const int budget = ring_budget(1);
@@ -1431,7 +1453,8 @@ static int generic_maps(dc_cache* c, dc_layer_rt& L, const dc_layer_desc& d, con
     CUtensorMap* tmBp = tm_find(&L.tm_b, 1, nullptr, weights, 1, p.BN, &hit_b);
     if (!hit_a) {   // input map [S][Hi][Wi][Ci] bf16; box = BK channels x 16 columns x 8 rows x 1 stream
         cuuint64_t dims[4] = {(cuuint64_t)d.cin, (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
-        cuuint64_t strides[3] = {(cuuint64_t)cin_all * 2, (cuuint64_t)L.in_w * cin_all * 2, (cuuint64_t)L.in_h * L.in_w * cin_all * 2};
+        const InPitch ip = in_pitch(L, cin_all);
+        cuuint64_t strides[3] = {ip.px * 2, ip.row * 2, (cuuint64_t)L.in_h * ip.row * 2};
         // a strided convolution reads every sw-th column / sh-th row: the box spans TW * sw x TH * sh input
         // pixels and the traversal strides pick TW x TH of them
         // (flat tiles: one image row of 8 pixels per box)

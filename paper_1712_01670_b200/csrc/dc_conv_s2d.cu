@@ -13,7 +13,7 @@
 // rectangles (Table 2 works on the layer as declared) and its tiles do not change.
 //
 // The rewritten layer (channels padded to 16, 32 or 64) runs on the ordinary kernels: AlexNet's first layer becomes a
-// 3 x 3 convolution over 64 channels (column slabs), ResNet's stem a 4 x 4 convolution over 16.  (The same rewrite with
+// 3 x 3 convolution over 64 channels (column slabs), ResNet's stem a 4 x 4 convolution over 16, run as 4 x 1 over 64.  (The same rewrite with
 // 1 x 1 blocks, padding a stride-1 layer's 96 channels to 128 so that it leaves the tap-by-tap kernel, was measured on
 // AlexNet's second layer: faster alone, slower in the trunk with the copy it needs: not kept.)
 #include "dc_common.cuh"
@@ -97,8 +97,7 @@ int dc_s2d_rewrite(dc_cache* c, int layer)
     const int Py = (d.ph + s - 1) / s * s, Px = (d.pw + s - 1) / s * s;
     const int offy = Py - d.ph, offx = Px - d.pw;
     const int Ty = (d.kh + offy + s - 1) / s, Tx = (d.kw + offx + s - 1) / s;
-    // block pixels padded to 16, 32 or 64 channels, whichever holds them (always 64, so that the stem of ResNet could run
-    // on column slabs, was measured: the same 0.21 ms for the layer, and a block map four times the size)
+    // block pixels padded to 16, 32 or 64 channels, whichever holds them
     const int cb = d.cin * s * s, cs = cb <= 16 ? 16 : cb <= 32 ? 32 : 64;
     const int Hs = d.out_h + Ty - 1, Ws = d.out_w + Tx - 1;
     const size_t wn = (size_t)d.cout * Ty * Tx * cs, mn = (size_t)c->S * Hs * Ws * cs;
@@ -117,8 +116,14 @@ int dc_s2d_rewrite(dc_cache* c, int layer)
     c->bytes -= old_bytes;
     L.weight = w2;
     L.s2d_s = s; L.s2d_py = Py; L.s2d_px = Px; L.s2d_cin = d.cin; L.s2d_hi = L.in_h; L.s2d_wi = L.in_w;
+    L.s2d_ws = Ws; L.s2d_cs = cs;
     L.d.kh = Ty; L.d.kw = Tx; L.d.sh = L.d.sw = 1; L.d.ph = L.d.pw = 0; L.d.cin = cs;
     L.in_h = Hs; L.in_w = Ws;
+    // Narrow block pixels: the Tx pixels of a kernel row are consecutive in memory, so they are the channels of one pixel of an
+    // overlapping view of the map (pixels Tx * cs channels wide, cs apart), and the kernel becomes Ty x 1 over them.  The
+    // weights [cout][Ty][Tx][cs] need no change.  ResNet's stem: 4 x 4 taps of 16 channels, one 32-byte row per pixel
+    // and tap to fetch, become one column slab of 128-byte rows for all 4 x 1 taps of 64.
+    if (cs < 64 && Tx > 1 && (Tx * cs) % 64 == 0) { L.d.kw = 1; L.d.cin = Tx * cs; L.in_w = Ws - Tx + 1; }
     return DC_OK;
 }
 
@@ -129,7 +134,7 @@ int dc_launch_s2d(dc_cache* c, int layer, const void* in)
     S2dArgs a;
     a.in = (const __nv_bfloat16*)in; a.out = (__nv_bfloat16*)L.in_s2d;
     a.S = c->S; a.Hi = L.s2d_hi; a.Wi = L.s2d_wi; a.cin = L.s2d_cin; a.s = L.s2d_s; a.Py = L.s2d_py; a.Px = L.s2d_px;
-    a.Hs = L.in_h; a.Ws = L.in_w; a.cs = L.d.cin;
+    a.Hs = L.in_h; a.Ws = L.s2d_ws; a.cs = L.s2d_cs;
     const size_t total = (size_t)a.S * a.Hs * a.Ws * (a.cs / 8);
     int grid = (int)((total + 255) / 256); if (grid > c->num_sms * 16) grid = c->num_sms * 16;
     DC_CUDA(dc_launch_pdl(k_space_to_depth, dim3((unsigned)grid), 256, 0, c->stream, a));

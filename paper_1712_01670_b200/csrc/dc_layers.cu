@@ -486,9 +486,9 @@ int dc_launch_frame_operand(dc_cache* c, int layer, const uint8_t* frame, size_t
     dc_layer_rt& L = c->L[layer];
     dc_prof_scope ps(c, DC_ST_INPUT);
     if (L.s2d_s) {
-        const int chunks = L.d.cin / 8;
-        const size_t n = (size_t)c->S * L.in_h * L.in_w * chunks;
-        DC_CUDA(dc_launch_pdl(k_frame_s2d, dim3((unsigned)grid_for(c, n, 256)), 256, 0, c->stream, frame, pitch, L.s2d_wi, L.s2d_hi, L.s2d_s, L.s2d_py, L.s2d_px, L.in_h, L.in_w,
+        const int chunks = L.s2d_cs / 8;
+        const size_t n = (size_t)c->S * L.in_h * L.s2d_ws * chunks;
+        DC_CUDA(dc_launch_pdl(k_frame_s2d, dim3((unsigned)grid_for(c, n, 256)), 256, 0, c->stream, frame, pitch, L.s2d_wi, L.s2d_hi, L.s2d_s, L.s2d_py, L.s2d_px, L.in_h, L.s2d_ws,
                               chunks, (unsigned)n, (uint4*)L.in_s2d));
     } else {
         const size_t n = (size_t)c->S * L.in_h * L.in_w;

@@ -85,20 +85,20 @@ __device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
     }
 }
 
-// One CTA per stream, a thread one rectangle at a time.  Rectangles that a later layer than the next one needs (residual
+// One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a later layer than the next one needs (residual
 // branches) wait in shared memory, and so does the layer table: the walk is a chain of a few dozen arithmetic steps per
 // layer (through a table in global memory it was a chain of memory round trips: 48 us for the 71 layers of ResNet-50).
 // out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): rectangles still
 // alive per layer and stream; with it the counters of the reuse step are zeroed.
-__global__ void __launch_bounds__(256) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions,
+__global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions,
                                                    const dc_region* in, const int32_t* n_in, dc_region* table, int32_t* alive, int32_t* reuse_px,
                                                    int32_t* dirty_count, dc_region* out, int out_begin, int32_t* n_out)
 {
     __shared__ PropLayer sl[DC_MAX_LAYERS];
-    __shared__ int32_t keep[kSlots * 6][256];
+    extern __shared__ int32_t keep[];                      // [places in use][6][threads]
     __shared__ int32_t count[DC_MAX_LAYERS];
-    const int s = blockIdx.x, tid = threadIdx.x;
-    for (int i = tid; i < layer_end * (int)(sizeof(PropLayer) / 4); i += 256) ((int*)sl)[i] = __ldg((const int*)layers + i);
+    const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    for (int i = tid; i < layer_end * (int)(sizeof(PropLayer) / 4); i += nt) ((int*)sl)[i] = __ldg((const int*)layers + i);
     if (tid < DC_MAX_LAYERS) count[tid] = 0;
     dc_pdl_wait();
     dc_pdl_release();
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(256) k_propagate(const PropLayer* layers, int 
     const int n = min(n_in[s], max_regions);              // a caller's count beyond the table is cut, never written
     // a caller's list has zeros behind its rectangles
     const int rows = out ? max_regions : n;
-    for (int i = tid; i < rows; i += 256) {
+    for (int i = blockIdx.y * nt + tid; i < rows; i += gridDim.y * nt) {
         const size_t slot = (size_t)s * max_regions + i;
         const bool on = i < n;
         const dc_region r0 = on ? in[slot] : empty_region();
@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(256) k_propagate(const PropLayer* layers, int 
             if (from == kFrame) return r0;
             if (from == kPrevious) return prev;
             if (from == kTable) return on ? table[layer * layer_stride + slot] : empty_region();
-            dc_region r = {keep[from * 6][tid], keep[from * 6 + 1][tid], keep[from * 6 + 2][tid], keep[from * 6 + 3][tid], keep[from * 6 + 4][tid], keep[from * 6 + 5][tid]};
+            const int32_t* k = keep + from * 6 * nt + tid;
+            dc_region r = {k[0], k[nt], k[2 * nt], k[3 * nt], k[4 * nt], k[5 * nt]};
             return r;
         };
         for (int l = 0; l < layer_end; ++l) {
@@ -125,8 +126,8 @@ __global__ void __launch_bounds__(256) k_propagate(const PropLayer* layers, int 
             const dc_region b = L.kind == DC_ADD || L.kind == DC_CONCAT ? fetch(L.from1, L.in1) : a;
             const dc_region o = apply_layer(L, a, b);
             if (L.keep >= 0) {
-                int32_t (*k)[256] = &keep[L.keep * 6];
-                k[0][tid] = o.x; k[1][tid] = o.y; k[2][tid] = o.w; k[3][tid] = o.h; k[4][tid] = o.sx; k[5][tid] = o.sy;
+                int32_t* k = keep + L.keep * 6 * nt + tid;
+                k[0] = o.x; k[nt] = o.y; k[2 * nt] = o.w; k[3 * nt] = o.h; k[4 * nt] = o.sx; k[5 * nt] = o.sy;
             }
             table[l * layer_stride + slot] = o;
             if (out && l >= out_begin) out[(l - out_begin) * layer_stride + slot] = o;
@@ -134,10 +135,10 @@ __global__ void __launch_bounds__(256) k_propagate(const PropLayer* layers, int 
             prev = o;
         }
     }
-    if (n_out) for (int l = out_begin + tid; l < layer_end; l += 256) n_out[(l - out_begin) * S + s] = n_in[s];
+    if (n_out && blockIdx.y == 0) for (int l = out_begin + tid; l < layer_end; l += nt) n_out[(l - out_begin) * S + s] = n_in[s];
     if (alive) {
         __syncthreads();
-        for (int l = tid; l < n_layers; l += 256) {
+        for (int l = tid; l < n_layers; l += nt) {
             alive[l * S + s] = l < layer_end ? count[l] : 0;
             reuse_px[l * S + s] = 0;
             if (s == 0) dirty_count[l] = 0;
@@ -590,7 +591,7 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
         t[l] = {d.kind, d.kh, d.kw, d.sh, d.sw, d.ph, d.pw, ih, iw, d.out_h, d.out_w, d.in0, d.in1, from(l, d.in0), from(l, d.in1), -1};
         for (int k = 0; k < kSlots; ++k) if (owner[k] >= 0 && last_use[owner[k]] <= l) owner[k] = -1;
         if (last_use[l] > l)
-            for (int k = 0; k < kSlots; ++k) if (owner[k] < 0) { owner[k] = l; t[l].keep = k; break; }
+            for (int k = 0; k < kSlots; ++k) if (owner[k] < 0) { owner[k] = l; t[l].keep = k; if (k >= c->prop_slots) c->prop_slots = k + 1; break; }
     }
     if (cudaMalloc(&c->prop_table, sizeof(PropLayer) * n) != cudaSuccess) { cudaGetLastError(); return DC_ERR_ALLOC; }
     c->bytes += sizeof(PropLayer) * n;
@@ -603,7 +604,13 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
 int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out)
 {
     dc_prof_scope ps(c, DC_ST_PROPAGATE);
-    DC_CUDA(dc_launch_pdl(k_propagate, dim3((unsigned)c->S), 256, 0, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, in, n_in,
+    // a thread per rectangle where the frame can have many
+    const int threads = c->max_regions > 512 ? 1024 : 256;
+    const size_t smem = (size_t)c->prop_slots * 6 * threads * sizeof(int32_t);
+    static dc_once_per_device attr_set;
+    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_propagate, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlots * 6 * 1024 * (int)sizeof(int32_t)));
+    const dim3 grid((unsigned)c->S, for_frame ? 1u : (unsigned)dc_div_up(c->max_regions, threads));
+    DC_CUDA(dc_launch_pdl(k_propagate, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, in, n_in,
                           c->table, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
     c->launches += 1;
     return DC_OK;
