@@ -237,7 +237,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     uint8_t* ring = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int stage_bytes = MT * a.a_bytes + a.b_bytes;
     SmemCtl* ctl = (SmemCtl*)(ring + (size_t)a.stages * stage_bytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int per_stream = a.tiles_x * a.tiles_y;
     const int taps = a.kh * a.kw, kiters = taps * a.kchunks;
 
@@ -296,9 +296,10 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             for (int tap = 0; tap < taps && ok; ++tap) {
                 const int ky = tap / a.kw, kx = tap - ky * a.kw;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
-                    if (lane == 0) {
-                        ok = mbar_wait(&ctl->empty[st], ph ^ 1u, ctl, a.status);
-                        if (ok && !a.skip_loads) {
+                    ok = mbar_wait(&ctl->empty[st], ph ^ 1u, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (ok && !a.skip_loads) {
+                        if (elect_one()) {
                             uint8_t* sa = ring + (size_t)st * stage_bytes;
                             mbar_expect_tx(&ctl->full[st], a.flat ? flat_tx : (uint32_t)stage_bytes);
                             if (!a.flat) {
@@ -308,8 +309,8 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                             }
                             tma_load_2d(sa + MT * a.a_bytes, &tmB, tap * a.Ci + cc * a.BK, (nb + a.nb_off) * a.BN, &ctl->full[st]);
                         }
+                        __syncwarp();
                     }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
                     // the slot is free and its byte count announced (lane 0, above): every lane brings its own group
                     if (a.flat && ok && !a.skip_loads && fon)
                         tma_load_4d(ring + (size_t)st * stage_bytes + (size_t)lane * (a.a_bytes / DC_TILE_H), &tmA, cc * a.BK, fx + kx, fy + ky, fs,
@@ -325,9 +326,9 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        // Only lane 0 works; descriptors differ from slot to slot in their address bits alone, so the
+        // One elected lane issues; descriptors differ from slot to slot in their address bits alone, so the
         // constant upper half is built once and the loop adds (address >> 4).
-        if (lane == 0) {
+        {
             const uint64_t dconst = umma_desc(0, a.sbo, a.layout_type);
             const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
             const int ksteps = a.BK / 16;
@@ -336,27 +337,34 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)(MT * a.BN);
                 ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int k = 0; k < kiters && ok; ++k) {
                     ok = mbar_wait(&ctl->full[st], ph, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t adesc0 = dconst + (ring_lo + (uint32_t)st * stage_lo);
                     const uint64_t bdesc = adesc0 + MT * a_lo;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int j = 0; j < MT; ++j) {
-                        uint32_t acc_j = accumulate;
-                        for (int kk = 0; kk < ksteps; ++kk) {          // 16 bf16 = 32 bytes = 2 descriptor units
-                            umma_f16(d_tmem + j * a.BN, adesc0 + j * a_lo + 2 * kk, bdesc + 2 * kk, a.idesc, acc_j);
-                            acc_j = 1;
+                        for (int j = 0; j < MT; ++j) {
+                            uint32_t acc_j = accumulate;
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk) {           // 16 bf16 = 32 bytes = 2 descriptor units
+                                if (kk < ksteps) umma_f16(d_tmem + j * a.BN, adesc0 + j * a_lo + 2 * kk, bdesc + 2 * kk, a.idesc, acc_j);
+                                acc_j = 1;
+                            }
                         }
+                        umma_commit(&ctl->empty[st]);                  // frees the slot when these MMAs retire
                     }
+                    __syncwarp();
                     accumulate = 1;
-                    umma_commit(&ctl->empty[st]);                      // frees the slot when these MMAs retire
                     if (++st == a.stages) { st = 0; ph ^= 1u; }
                 }
-                if (ok) umma_commit(&ctl->tmem_full[acc]);
+                if (ok && elect_one()) umma_commit(&ctl->tmem_full[acc]);
+                __syncwarp();
                 if (++acc == (uint32_t)a.nbuf) { acc = 0; acc_ph ^= 1u; }
             }
         }
@@ -400,7 +408,7 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
     uint8_t* wsm = base;                                        // packed weights
     uint8_t* ring = wsm + ((sa.w_bytes + 127) & ~127);
     SmemCtl* ctl = (SmemCtl*)(ring + (size_t)a.stages * sa.stage_bytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int per_stream = a.tiles_x * a.tiles_y;
     const int taps = a.kh * a.kw;
 
@@ -433,7 +441,7 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
     const int n_items = *a.tile_count;
 
     if (warp == 0) {
-        if (lane == 0) {                                        // producer: one patch per item
+        {                                                       // producer: one patch per item
             int st = 0; uint32_t ph = 0;
             bool ok = true;
             int tile_next = a.tile_list[blockIdx.x];            // fetched one item ahead: off the critical path
@@ -441,19 +449,20 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
                 const int tile = tile_next;
                 if (item + (int)gridDim.x < n_items) tile_next = a.tile_list[item + gridDim.x];
                 const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-                ok = mbar_wait(&ctl->empty[st], ph ^ 1u, ctl, a.status);
+                ok = __all_sync(0xffffffffu, mbar_wait(&ctl->empty[st], ph ^ 1u, ctl, a.status));
                 if (!ok) break;
-                if (!a.skip_loads) {
+                if (!a.skip_loads && elect_one()) {
                     mbar_expect_tx(&ctl->full[st], (uint32_t)(sa.PW * sa.PH * 16));
                     tma_load_4d(ring + (size_t)st * sa.stage_bytes, &tmA, 0, tx * DC_TILE_W - a.pw, ty * DC_TILE_H - a.ph, s, &ctl->full[st]);
                 }
+                __syncwarp();
                 if (++st == a.stages) { st = 0; ph ^= 1u; }
             }
-            if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
+            if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {                                        // MMA issuer
+        {                                                       // MMA issuer
             const uint32_t b_lbo = (uint32_t)a.Co * 16u;
             const uint64_t bconst = umma_desc(smem_u32(wsm), 128, 0, b_lbo);
             const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)sa.stage_bytes >> 4;
@@ -461,26 +470,29 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
             int st = 0; uint32_t ph = 0, acc = 0, acc_ph = 0;
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
-                if (ok) ok = mbar_wait(&ctl->full[st], ph, ctl, a.status);
+                ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status) && mbar_wait(&ctl->full[st], ph, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)a.BN;
                 const uint32_t patch_lo = ring_lo + (uint32_t)st * stage_lo;
                 // K step kk covers taps 2kk and 2kk+1: two 16-byte pixel columns of the patch, `lbo` apart
                 int tap = 0, ky = 0, kx = 0;
-                for (int kk = 0; kk < sa.kblocks / 2; ++kk) {
-                    const uint32_t off0 = (uint32_t)(ky * sa.PW + kx);
-                    if (++kx == a.kw) { kx = 0; ++ky; }
-                    ++tap;
-                    uint32_t off1 = off0 + 1;                      // past the last tap: any finite data (its weights are zero)
-                    if (tap < taps) { off1 = (uint32_t)(ky * sa.PW + kx); if (++kx == a.kw) { kx = 0; ++ky; } }
-                    ++tap;
-                    const uint64_t adesc = hi + (patch_lo + off0) + ((uint64_t)(off1 - off0) << 16);
-                    umma_f16(d_tmem, adesc, bconst + (uint64_t)(kk * ((2 * b_lbo) >> 4)), a.idesc, kk != 0);
+                if (elect_one()) {
+                    for (int kk = 0; kk < sa.kblocks / 2; ++kk) {
+                        const uint32_t off0 = (uint32_t)(ky * sa.PW + kx);
+                        if (++kx == a.kw) { kx = 0; ++ky; }
+                        ++tap;
+                        uint32_t off1 = off0 + 1;                      // past the last tap: any finite data (its weights are zero)
+                        if (tap < taps) { off1 = (uint32_t)(ky * sa.PW + kx); if (++kx == a.kw) { kx = 0; ++ky; } }
+                        ++tap;
+                        const uint64_t adesc = hi + (patch_lo + off0) + ((uint64_t)(off1 - off0) << 16);
+                        umma_f16(d_tmem, adesc, bconst + (uint64_t)(kk * ((2 * b_lbo) >> 4)), a.idesc, kk != 0);
+                    }
+                    umma_commit(&ctl->empty[st]);
+                    umma_commit(&ctl->tmem_full[acc]);
                 }
-                umma_commit(&ctl->empty[st]);
-                umma_commit(&ctl->tmem_full[acc]);
+                __syncwarp();
                 if (++st == a.stages) { st = 0; ph ^= 1u; }
                 if (++acc == 2u) { acc = 0; acc_ph ^= 1u; }
             }
@@ -506,12 +518,12 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
 // bytes) of [patch row][patch column] pixels.  A tile is 8 pixels wide, so the 8 rows of one
 // operand group are the 8 consecutive pixels of one image row, and groups are one patch row
 // (PW x 16 bytes) apart: SBO = PW * 16, LBO = plane size, start = plane + (ky * PW + kx) * 16.
-// Weights are pre-packed per (channel block, tap, chunk) as [k/8][BN][8] and arrive with one
-// plain bulk copy each.
+// Weights are pre-packed per (channel block, tap, chunk) as the MMA reads them (k_pack_halo) and
+// arrive with one plain bulk copy each.
 // ---------------------------------------------------------------------------------------------
 struct TcHaloArgs {
     TcArgs t;
-    const __nv_bfloat16* wpacked;    // [NB][taps][kchunks][8][BN][8]
+    const __nv_bfloat16* wpacked;    // [NB][taps][kchunks][BN][64], swizzled (k_pack_halo)
     int PW, PH, plane_bytes, patch_bytes, a_stages;
     int k_last;                      // K steps of 16 channels in the last chunk (4 unless the channels are no multiple of 64)
 };
@@ -535,12 +547,12 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
 {
     extern __shared__ uint8_t smem_raw[];
     const TcArgs& a = ha.t;
-    constexpr uintptr_t kAlign = SLAB ? 1023 : 127;           // swizzle atoms start on 1024-byte boundaries
+    constexpr uintptr_t kAlign = 1023;                        // swizzle atoms start on 1024-byte boundaries
     uint8_t* aring = (uint8_t*)(((uintptr_t)smem_raw + kAlign) & ~kAlign);
     const int a_slot = MT * ha.patch_bytes;
     uint8_t* bring = aring + (size_t)ha.a_stages * a_slot;
     SmemCtl* ctl = (SmemCtl*)(bring + (size_t)a.stages * a.b_bytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int per_stream = a.tiles_x * a.tiles_y;
     const int taps = a.kh * a.kw;
 
@@ -583,9 +595,10 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
             }
             for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                 for (int kx = 0; kx < (SLAB ? a.kw : 1) && ok; ++kx) {
-                    if (lane == 0) {
-                        ok = mbar_wait(&ctl->a_empty[sa], pa ^ 1u, ctl, a.status);
-                        if (ok && !a.skip_loads) {
+                    ok = mbar_wait(&ctl->a_empty[sa], pa ^ 1u, ctl, a.status);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (ok && !a.skip_loads) {
+                        if (elect_one()) {
                             if (SLAB) {
                                 mbar_expect_tx(&ctl->a_full[sa], (uint32_t)(MT * ha.patch_bytes));
 #pragma unroll
@@ -601,21 +614,22 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                                                     cc * 64 + g * 8, xb[j], yb[j], sN[j], &ctl->a_full[sa]);
                             }
                         }
+                        __syncwarp();
                     }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
                     if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
                     // the weight tiles that go with this A stage: all taps (patch), or the taps of column kx (slab)
                     for (int t = 0; t < (SLAB ? a.kh : taps) && ok; ++t) {
                         const int tap = SLAB ? t * a.kw + kx : t;
-                        if (lane == 0) {
-                            ok = mbar_wait(&ctl->empty[sb], pb ^ 1u, ctl, a.status);
-                            if (ok && !a.skip_loads) {
+                        ok = mbar_wait(&ctl->empty[sb], pb ^ 1u, ctl, a.status);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (ok && !a.skip_loads) {
+                            if (elect_one()) {
                                 mbar_expect_tx(&ctl->full[sb], (uint32_t)a.b_bytes);
                                 const uint8_t* src = (const uint8_t*)ha.wpacked + ((size_t)((nb + a.nb_off) * taps + tap) * a.kchunks + cc) * a.b_bytes;
                                 bulk_copy_g2s(bring + (size_t)sb * a.b_bytes, src, (uint32_t)a.b_bytes, &ctl->full[sb]);
                             }
+                            __syncwarp();
                         }
-                        ok = __shfl_sync(0xffffffffu, ok, 0);
                         if (++sb == a.stages) { sb = 0; pb ^= 1u; }
                     }
                 }
@@ -623,55 +637,60 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
         }
         if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
     } else if (warp == 1) {
-        // ---------------- MMA issuer (lane 0 only) ----------------
-        if (lane == 0) {
-            const uint32_t b_lbo = (uint32_t)a.BN * 16u;
+        // ---------------- MMA issuer (one elected lane) ----------------
+        {
             // A: patch planes (rows PW * 16 bytes apart, planes along K), or a 128-byte swizzled K-major slab
             const uint64_t aconst = SLAB ? umma_desc(0, 1024, 2) : umma_desc(0, (uint32_t)ha.PW * 16u, 0, (uint32_t)ha.plane_bytes);
-            const uint64_t bconst = umma_desc(0, 128, 0, b_lbo);
+            const uint64_t bconst = umma_desc(0, 1024, 2);                               // weights: 128-byte swizzled, K-major
             const uint32_t aring_lo = smem_u32(aring) >> 4, bring_lo = smem_u32(bring) >> 4;
             const uint32_t a_slot_lo = (uint32_t)a_slot >> 4, patch_lo = (uint32_t)ha.patch_bytes >> 4;
             const uint32_t a_kstep = SLAB ? 2u : (uint32_t)(2 * ha.plane_bytes) >> 4;    // 16 channels further along K
-            const uint32_t b_kstep = (2 * b_lbo) >> 4, b_lo = (uint32_t)a.b_bytes >> 4;
+            const uint32_t b_kstep = 2u, b_lo = (uint32_t)a.b_bytes >> 4;
             int sa = 0, sb = 0; uint32_t pa = 0, pb = 0, acc = 0, acc_ph = 0;
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)(MT * a.BN);
                 ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
+                ok = __all_sync(0xffffffffu, ok);
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                     const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < (SLAB ? a.kw : 1) && ok; ++ax) {     // A stages of this chunk: one patch, or kw slabs
-                        ok = mbar_wait(&ctl->a_full[sa], pa, ctl, a.status);
+                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->a_full[sa], pa, ctl, a.status));
                         const uint64_t apatch = aconst + (aring_lo + (uint32_t)sa * a_slot_lo);
                         // patch: taps in (ky, kx) order at (ky * PW + kx) * 16 bytes; slab ax: taps (ky, ax) at ky atoms of 1024 bytes
                         const int n_t = SLAB ? a.kh : taps;
                         for (int t = 0; t < n_t && ok; ++t) {
                             const uint32_t tap_lo = SLAB ? (uint32_t)t * 64u : (uint32_t)((t / a.kw) * ha.PW + t % a.kw);
-                            ok = mbar_wait(&ctl->full[sb], pb, ctl, a.status);
+                            ok = __all_sync(0xffffffffu, mbar_wait(&ctl->full[sb], pb, ctl, a.status));
                             if (!ok) break;
                             tc_fence_after();
                             const uint64_t bdesc = bconst + (bring_lo + (uint32_t)sb * b_lo);
+                            if (elect_one()) {
 #pragma unroll
-                            for (int j = 0; j < MT; ++j) {
-                                const uint64_t adesc = apatch + j * patch_lo + tap_lo;
-                                uint32_t acc_j = accumulate;
+                                for (int j = 0; j < MT; ++j) {
+                                    const uint64_t adesc = apatch + j * patch_lo + tap_lo;
+                                    uint32_t acc_j = accumulate;
 #pragma unroll
-                                for (int kk = 0; kk < 4; ++kk) {        // K = 16 per instruction, up to 64 channels per chunk
-                                    if (kk < n_kk) umma_f16(d_tmem + j * a.BN, adesc + kk * a_kstep, bdesc + kk * b_kstep, a.idesc, acc_j);
-                                    acc_j = 1;
+                                    for (int kk = 0; kk < 4; ++kk) {    // K = 16 per instruction, up to 64 channels per chunk
+                                        if (kk < n_kk) umma_f16(d_tmem + j * a.BN, adesc + kk * a_kstep, bdesc + kk * b_kstep, a.idesc, acc_j);
+                                        acc_j = 1;
+                                    }
                                 }
+                                umma_commit(&ctl->empty[sb]);
                             }
+                            __syncwarp();
                             accumulate = 1;
-                            umma_commit(&ctl->empty[sb]);
                             if (++sb == a.stages) { sb = 0; pb ^= 1u; }
                         }
-                        if (ok) umma_commit(&ctl->a_empty[sa]);         // the A stage is free once its taps retire
+                        if (ok && elect_one()) umma_commit(&ctl->a_empty[sa]);   // the A stage is free once its taps retire
+                        __syncwarp();
                         if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
                     }
                 }
-                if (ok) umma_commit(&ctl->tmem_full[acc]);
+                if (ok && elect_one()) umma_commit(&ctl->tmem_full[acc]);
+                __syncwarp();
                 if (++acc == (uint32_t)a.nbuf) { acc = 0; acc_ph ^= 1u; }
             }
         }
@@ -726,7 +745,7 @@ __device__ __forceinline__ void umma_commit_pair(void* bar)
 }
 
 // ha.t.BN: output channels per item (both CTAs together); ha.t.b_bytes: one CTA's weight tile (BN / 2 rows of 128 bytes);
-// tmW: the packed weights [2 NB][taps][kchunks][8][BN / 2][8] seen as rows of 128 bytes.
+// tmW: the packed weights [2 NB][taps][kchunks][BN / 2][64] seen as rows of 128 bytes.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const TcHaloArgs ha)
 {
@@ -739,7 +758,7 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int a_slot = ha.patch_bytes;                        // one slab
     uint8_t* bring = aring + (size_t)ha.a_stages * a_slot;
     SmemCtl* ctl = (SmemCtl*)(bring + (size_t)a.stages * a.b_bytes);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int per_stream = a.tiles_x * a.tiles_y;
     const int taps = a.kh * a.kw;
 
@@ -782,26 +801,26 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const int xb = tx * DC_TILE_W - a.pw, yb = ty * DC_TILE_H - a.ph;
             for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                 for (int kx = 0; kx < a.kw && ok; ++kx) {
-                    if (lane == 0) {
-                        ok = mbar_wait(&ctl->a_empty[sa], pa ^ 1u, ctl, a.status);
-                        if (ok && !a.skip_loads) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->a_empty[sa], pa ^ 1u, ctl, a.status));
+                    if (ok && !a.skip_loads) {
+                        if (elect_one()) {
                             if (leader) mbar_expect_tx(&ctl->a_full[sa], (uint32_t)(2 * ha.patch_bytes));
                             tma_load_4d_pair(aring + (size_t)sa * a_slot, &tmA, cc * 64, xb + kx, yb, s, a_full0 + (uint32_t)sa * 8u);
                         }
+                        __syncwarp();
                     }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
                     if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
                     for (int t2 = 0; t2 < a.kh && ok; ++t2) {
                         const int tap = t2 * a.kw + kx;
-                        if (lane == 0) {
-                            ok = mbar_wait(&ctl->empty[sb], pb ^ 1u, ctl, a.status);
-                            if (ok && !a.skip_loads) {
+                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->empty[sb], pb ^ 1u, ctl, a.status));
+                        if (ok && !a.skip_loads) {
+                            if (elect_one()) {
                                 if (leader) mbar_expect_tx(&ctl->full[sb], (uint32_t)(2 * a.b_bytes));
                                 const int row = (((nb * 2 + (int)rank) * taps + tap) * a.kchunks + cc) * rows_per_tile;
                                 tma_load_2d_pair(bring + (size_t)sb * a.b_bytes, &tmW, 0, row, full0 + (uint32_t)sb * 8u);
                             }
+                            __syncwarp();
                         }
-                        ok = __shfl_sync(0xffffffffu, ok, 0);
                         if (++sb == a.stages) { sb = 0; pb ^= 1u; }
                     }
                 }
@@ -809,45 +828,51 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
     } else if (warp == 1) {
-        // ---------------- MMA issuer: the leader's lane 0 issues for both CTAs ----------------
-        if (leader && lane == 0) {
-            const uint32_t b_lbo = (uint32_t)(a.BN / 2) * 16u;
+        // ---------------- MMA issuer: an elected lane of the leader issues for both CTAs ----------------
+        if (leader) {
             const uint64_t aconst = umma_desc(0, 1024, 2);
-            const uint64_t bconst = umma_desc(0, 128, 0, b_lbo);
+            const uint64_t bconst = umma_desc(0, 1024, 2);                               // weights: 128-byte swizzled, K-major
             const uint32_t aring_lo = smem_u32(aring) >> 4, bring_lo = smem_u32(bring) >> 4;
             const uint32_t a_slot_lo = (uint32_t)a_slot >> 4;
-            const uint32_t b_kstep = (2 * b_lbo) >> 4, b_lo = (uint32_t)a.b_bytes >> 4;
+            const uint32_t b_kstep = 2u, b_lo = (uint32_t)a.b_bytes >> 4;
             int sa = 0, sb = 0; uint32_t pa = 0, pb = 0, acc = 0, acc_ph = 0;
             bool ok = true;
             for (int item = pair; item < n_items && ok; item += n_pairs) {
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)a.BN;
-                ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
+                ok = __all_sync(0xffffffffu, mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status));
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                     const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < a.kw && ok; ++ax) {
-                        ok = mbar_wait(&ctl->a_full[sa], pa, ctl, a.status);
+                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->a_full[sa], pa, ctl, a.status));
                         const uint64_t aslab = aconst + (aring_lo + (uint32_t)sa * a_slot_lo);
                         for (int t = 0; t < a.kh && ok; ++t) {               // tap (t, ax): the slab from swizzle atom t on
-                            ok = mbar_wait(&ctl->full[sb], pb, ctl, a.status);
+                            ok = __all_sync(0xffffffffu, mbar_wait(&ctl->full[sb], pb, ctl, a.status));
                             if (!ok) break;
                             tc_fence_after();
                             const uint64_t bdesc = bconst + (bring_lo + (uint32_t)sb * b_lo);
                             const uint64_t adesc = aslab + (uint32_t)t * 64u;
+                            if (elect_one()) {
+                                uint32_t acc_k = accumulate;
 #pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {                 // K = 16 per instruction, up to 64 channels per chunk
-                                if (kk < n_kk) umma_f16_pair(d_tmem, adesc + kk * 2u, bdesc + kk * b_kstep, a.idesc, accumulate);
-                                accumulate = 1;
+                                for (int kk = 0; kk < 4; ++kk) {             // K = 16 per instruction, up to 64 channels per chunk
+                                    if (kk < n_kk) umma_f16_pair(d_tmem, adesc + kk * 2u, bdesc + kk * b_kstep, a.idesc, acc_k);
+                                    acc_k = 1;
+                                }
+                                umma_commit_pair(&ctl->empty[sb]);
                             }
-                            umma_commit_pair(&ctl->empty[sb]);
+                            __syncwarp();
+                            accumulate = 1;
                             if (++sb == a.stages) { sb = 0; pb ^= 1u; }
                         }
-                        if (ok) umma_commit_pair(&ctl->a_empty[sa]);
+                        if (ok && elect_one()) umma_commit_pair(&ctl->a_empty[sa]);
+                        __syncwarp();
                         if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
                     }
                 }
-                if (ok) umma_commit_pair(&ctl->tmem_full[acc]);
+                if (ok && elect_one()) umma_commit_pair(&ctl->tmem_full[acc]);
+                __syncwarp();
                 if (++acc == 2u) { acc = 0; acc_ph ^= 1u; }
             }
         }
@@ -866,7 +891,10 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
 }
 
-// weights [cout][taps][cin] -> [NB][taps][kchunks][8][BN][8], zeros beyond the last channel
+// weights [cout][taps][cin] -> [NB][taps][kchunks] tiles of BN rows (output channels) x 64 channels, zeros beyond the last
+// channel.  A tile lies in memory as the MMA reads it from shared memory, K-major with 128-byte swizzle: the 16-byte piece
+// k8 of row n is at piece k8 ^ (n & 7) of that row, so that a plain bulk copy brings it in place.  (Unswizzled core
+// matrices, the layout before, cost the MMAs shared-memory time.)
 __global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin, int BN, __nv_bfloat16* out)
 {
     const int kchunks = (cin + 63) / 64;
@@ -874,11 +902,11 @@ __global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin,
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         size_t r = i;
         const int e = (int)(r & 7); r >>= 3;
+        const int piece = (int)(r & 7); r >>= 3;
         const int n = (int)(r % BN); r /= BN;
-        const int k8 = (int)(r & 7); r >>= 3;
         const int cc = (int)(r % kchunks); r /= kchunks;
         const int tap = (int)(r % taps); const int nb = (int)(r / taps);
-        const int ch = cc * 64 + k8 * 8 + e;
+        const int ch = cc * 64 + (piece ^ (n & 7)) * 8 + e;
         out[i] = ch < cin ? w[((size_t)(nb * BN + n) * taps + tap) * cin + ch] : __float2bfloat16(0.f);
     }
 }
@@ -1301,7 +1329,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     if (a.stages < 2) return DC_ERR_CONFIG;
     a.epi_warps = epi_warps_for(ctas);
     a.bias_smem = t_bias_bytes ? d.cout : 0;
-    const size_t smem = (size_t)a_total + (size_t)a.stages * h.b_bytes + ctl_bytes(a.epi_warps) + t_bias_bytes + (slab ? 1280 : 256);
+    const size_t smem = (size_t)a_total + (size_t)a.stages * h.b_bytes + ctl_bytes(a.epi_warps) + t_bias_bytes + 1280;
     if (smem > 227 * 1024) return DC_ERR_CONFIG;
     static dc_once_per_device attr_set;
     if (attr_set.first(c->device)) {
@@ -1345,7 +1373,7 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     HaloPlan h;
     if (!enc || !L.weight_halo || !pair_ok(d, bn) || !halo_ok(d, h)) return DC_ERR_CONFIG;
     const int half = bn / 2, taps = d.kh * d.kw, kchunks = h.kchunks;
-    if (L.halo_bn != half) {                                     // weights grouped by half blocks: [2 NB][taps][kchunks][8][half][8]
+    if (L.halo_bn != half) {                                     // weights grouped by half blocks: [2 NB][taps][kchunks][half][64]
         const size_t n = (size_t)d.cout * taps * kchunks * 64;
         int pgrid = (int)((n + 255) / 256); if (pgrid > c->num_sms * 8) pgrid = c->num_sms * 8;
         k_pack_halo<<<pgrid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, d.cout, taps, d.cin, half, (__nv_bfloat16*)L.weight_halo);

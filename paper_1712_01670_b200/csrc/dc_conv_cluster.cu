@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     const int stage_bytes = a.a_bytes + a.b_bytes;
     float* red = (float*)(ring + (size_t)a.stages * stage_bytes);            // [CS][128 / CS][BN + 4]: this CTA's pixels, from every CTA
     CtlCl* ctl = (CtlCl*)(red + 128 * red_pitch(a.BN));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank(), item = blockIdx.x / a.CS, nb = item % a.NB, idx = item / a.NB;
     const int kiters = a.kh * a.kw * a.kchunks;
     const int k0 = rank * kiters / a.CS, nk = (rank + 1) * kiters / a.CS - k0;
@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         tma_load_2d(ring + (size_t)st * stage_bytes + a.a_bytes, &tmB, tap * a.Ci + cc * a.BK, (nb + a.nb_off) * a.BN, &ctl->full[st]);
     };
     const int early = nk < a.stages ? nk : a.stages;
-    if (warp == 0 && lane == 0 && !a.skip_loads)
-        for (int it = 0; it < early; ++it) load_weights(it);
+    if (warp == 0 && !a.skip_loads)
+        for (int it = 0; it < early; ++it) { if (elect_one()) load_weights(it); __syncwarp(); }
     dc_pdl_wait();                           // the previous kernel's output, the tile list and its count are read from here on
     dc_pdl_release();
     const int n_tiles = *a.tile_count;
@@ -139,9 +139,9 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
             if (lane == 0 && !a.skip_loads)
                 for (int it = 0; it < early && ok; ++it) { mbar_arrive(&ctl->full[it]); ok = cl_wait(&ctl->full[it], 0, ctl, a.status); }
         } else if (!a.skip_loads) {
-            // 16 x 8 tile: lane 0 brings the window of a tap; flat tiles: lane l brings row piece l
+            // 16 x 8 tile: an elected lane brings the window of a tap; flat tiles: lane l brings row piece l
             int fs = 0, fx = 0, fy = 0;
-            bool fon = !a.flat && lane == 0;
+            bool fon = false;
             if (a.flat) {
                 int y, x0;
                 fon = lane < DC_TILE_H && locate(lane, fs, y, x0);
@@ -153,15 +153,16 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
             const uint32_t a_tx = a.flat ? (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * (uint32_t)piece : (uint32_t)a.a_bytes;
             for (int it = 0; it < nk && ok; ++it) {
                 const int st = it % a.stages, tap = (k0 + it) / a.kchunks, cc = (k0 + it) - tap * a.kchunks, ky = tap / a.kw, kx = tap - ky * a.kw;
-                if (lane == 0) {
-                    if (it >= a.stages) {
-                        ok = cl_wait(&ctl->empty[st], (uint32_t)(it / a.stages - 1) & 1u, ctl, a.status);
-                        if (ok) load_weights(it);
-                    }
-                    if (ok) mbar_expect_tx(&ctl->full[st], a_tx);
+                if (it >= a.stages) ok = __all_sync(0xffffffffu, cl_wait(&ctl->empty[st], (uint32_t)(it / a.stages - 1) & 1u, ctl, a.status));
+                if (!ok) break;
+                if (elect_one()) {
+                    if (it >= a.stages) load_weights(it);
+                    mbar_expect_tx(&ctl->full[st], a_tx);
+                    if (!a.flat) tma_load_4d(ring + (size_t)st * stage_bytes, &tmA, cc * a.BK, fx + kx, fy + ky, fs, &ctl->full[st]);
                 }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (ok && fon) tma_load_4d(ring + (size_t)st * stage_bytes + (size_t)lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, &ctl->full[st]);
+                __syncwarp();
+                if (a.flat && fon) tma_load_4d(ring + (size_t)st * stage_bytes + (size_t)lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, &ctl->full[st]);
+                __syncwarp();
             }
         }
         // on an abort: give the copies already issued a bounded chance to land before the CTA exits
@@ -169,21 +170,26 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0 && present) {
+        if (present) {
             const uint64_t dconst = umma_desc(0, a.sbo, a.layout_type);
             const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
             const int ksteps = a.BK / 16;
             bool ok = true;
             for (int it = 0; it < nk && ok; ++it) {
                 const int st = it % a.stages;
-                ok = cl_wait(&ctl->full[st], (uint32_t)(it / a.stages) & 1u, ctl, a.status);
+                ok = __all_sync(0xffffffffu, cl_wait(&ctl->full[st], (uint32_t)(it / a.stages) & 1u, ctl, a.status));
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t adesc = dconst + (ring_lo + (uint32_t)st * stage_lo), bdesc = adesc + a_lo;
-                for (int kk = 0; kk < ksteps; ++kk) umma_f16(tmem_base, adesc + 2 * kk, bdesc + 2 * kk, a.idesc, (uint32_t)((it | kk) != 0));
-                if (it + a.stages < nk) umma_commit(&ctl->empty[st]);
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        if (kk < ksteps) umma_f16(tmem_base, adesc + 2 * kk, bdesc + 2 * kk, a.idesc, (uint32_t)((it | kk) != 0));
+                    if (it + a.stages < nk) umma_commit(&ctl->empty[st]);
+                    if (it + 1 == nk) umma_commit(&ctl->done);
+                }
+                __syncwarp();
             }
-            if (ok) umma_commit(&ctl->done);
         }
         __syncwarp();
     } else if (present) {
