@@ -154,6 +154,7 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     }
     dc_use_match_set(c, 0);
     DC_TRY(dev_alloc(c, &c->table, (size_t)n * S * c->max_regions));
+    DC_TRY(dev_alloc(c, &c->live, (size_t)n * S * c->max_regions));
     DC_TRY(dc_build_propagate_table(c, layers));
     DC_TRY(dev_alloc(c, &c->dirty_count, (size_t)n));
     DC_TRY(dev_alloc(c, &c->all_count, (size_t)n * 2));
@@ -274,7 +275,7 @@ void release(dc_cache* c)
         cudaFree(m.blk_mv); cudaFree(m.blk_sse); cudaFree(m.matched); cudaFree(m.run_end); cudaFree(m.mv_acc);
         cudaFree(m.long_list); cudaFree(m.gmv); cudaFree(m.regions0); cudaFree(m.n_regions);
     }
-    cudaFree(c->table); cudaFree(c->classify_table);
+    cudaFree(c->table); cudaFree(c->live); cudaFree(c->classify_table);
     cudaFree(c->prop_table); cudaFree(c->dirty_count); cudaFree(c->partial); cudaFree(c->all_count);
     cudaFree(c->reuse_px); cudaFree(c->zero_masks); cudaFree(c->status); cudaFree(c->input_map);
     if (c->stats_pinned) cudaFreeHost(c->stats_pinned);
@@ -450,6 +451,9 @@ int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* 
     return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.all_list, dc_all_count(c, layer), c->zero_masks, tiles);
 }
 
+// More blocks than the SMs hold warps, ten times over: matching a frame then takes about as long as a trunk's inference.
+static bool matcher_is_large(const dc_cache* c) { return (long long)c->S * c->Gx * c->Gy > (long long)c->num_sms * 640; }
+
 static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* out_map_dev, dc_frame_stats* stats)
 {
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
@@ -460,9 +464,9 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
     // the library's own aligned copy of the frame: matched now, the cache key of the next frame (Section 3)
     uint8_t* frame_copy = c->key[(c->key_cur + 1) % 3];
     const bool looked_ahead = c->la_frame == frame_dev && c->la_pitch == pitch && c->key_valid;
-    // a caller that looks ahead keeps doing so: where the matcher of the next frame is large (more blocks than the SMs hold
-    // warps, ten times over), the inference leaves it room (see ring_budget())
-    c->overlap_mode = looked_ahead && (long long)S * c->Gx * c->Gy > (long long)c->num_sms * 640;
+    // a caller that looks ahead keeps doing so: where the matcher of the next frame is large, the inference leaves it room
+    // (see ring_budget())
+    c->overlap_mode = looked_ahead && matcher_is_large(c);
     g_dc_pdl = !c->overlap_mode;
     if (looked_ahead) {
         // dc_lookahead_frame already copied this frame in and (unless it is a full frame) matched it
@@ -600,6 +604,7 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     const int main_set = c->mset_cur;
     c->stream = c->la_stream;                                       // the launchers enqueue on c->stream
     uint8_t* next_copy = c->key[(c->key_cur + 1) % 3];
+    g_dc_pdl = !matcher_is_large(c);                                // as in the inference it runs beside
     int rc = dc_launch_copy_frame(c, frame_dev, pitch, next_copy, c->mset[main_set ^ 1].mv_acc);
     if (rc == DC_OK && !next_is_full) {
         dc_use_match_set(c, main_set ^ 1);
@@ -607,6 +612,7 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
         dc_use_match_set(c, main_set);
     }
     c->stream = main_stream;
+    g_dc_pdl = true;
     if (rc != DC_OK) return rc;
     DC_CUDA(cudaEventRecord(c->ev_match, c->la_stream));
     c->la_frame = frame_dev; c->la_pitch = pitch; c->la_matched = !next_is_full;

@@ -88,10 +88,12 @@ __device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
 // One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a later layer than the next one needs (residual
 // branches) wait in shared memory, and so does the layer table: the walk is a chain of a few dozen arithmetic steps per
 // layer (through a table in global memory it was a chain of memory round trips: 48 us for the 71 layers of ResNet-50).
+// alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most
+// of a frame's erode within a few layers, and the reuse step tests every tile against all it is given.
 // out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): rectangles still
 // alive per layer and stream; with it the counters of the reuse step are zeroed.
 __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions,
-                                                   const dc_region* in, const int32_t* n_in, dc_region* table, int32_t* alive, int32_t* reuse_px,
+                                                   const dc_region* in, const int32_t* n_in, dc_region* table, dc_region* live, int32_t* alive, int32_t* reuse_px,
                                                    int32_t* dirty_count, dc_region* out, int out_begin, int32_t* n_out)
 {
     __shared__ PropLayer sl[DC_MAX_LAYERS];
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
             }
             table[l * layer_stride + slot] = o;
             if (out && l >= out_begin) out[(l - out_begin) * layer_stride + slot] = o;
-            if (o.w > 0 && alive) atomicAdd(&count[l], 1);
+            if (o.w > 0 && alive) live[l * layer_stride + (size_t)s * max_regions + atomicAdd(&count[l], 1)] = o;
             prev = o;
         }
     }
@@ -471,7 +473,7 @@ struct ClassifyLayer {
 };
 
 __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const ClassifyLayer* layers, int n_cached, int total_warps,
-                                                                       const int32_t* n_regions, int max_regions, int S, int cur)
+                                                                       int max_regions, int S, int cur)
 {
     extern __shared__ uint8_t copy_smem[];
     CopyLane cl = copy_lane_setup(copy_smem);
@@ -486,7 +488,7 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
     }
     const ClassifyLayer& L = layers[lo];
     ClassifyArgs a;
-    a.regions = L.regions; a.n_regions = n_regions; a.max_regions = max_regions;
+    a.regions = L.regions; a.n_regions = L.alive; a.max_regions = max_regions;     // the rectangles left at this layer
     a.prev = L.map[cur]; a.out = L.map[cur ^ 1];
     a.Ho = L.Ho; a.Wo = L.Wo; a.px_bytes = L.px_bytes; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y; a.S = S;
     a.gpr = L.gpr; a.n_tiles = 0;
@@ -524,7 +526,7 @@ int dc_build_classify_table(dc_cache* c)
         if (!dc_layer_cached(c, i)) continue;
         dc_layer_rt& L = c->L[i];
         ClassifyLayer& e = h[k++];
-        e.regions = c->table + (size_t)i * c->S * c->max_regions;
+        e.regions = c->live + (size_t)i * c->S * c->max_regions;
         e.map[0] = (uint8_t*)L.map[0]; e.map[1] = (uint8_t*)L.map[1];
         e.Ho = L.d.out_h; e.Wo = L.d.out_w; e.px_bytes = L.d.cout * c->elt;
         e.tiles_x = L.tiles_x; e.tiles_y = L.tiles_y; e.first_warp = warps;
@@ -558,7 +560,7 @@ int dc_launch_classify_all(dc_cache* c, int cur)
         if (attr_set.first(c->device))
             DC_CUDA(cudaFuncSetAttribute(k_classify_copy_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCopySmem));
         DC_CUDA(dc_launch_pdl(k_classify_copy_all, dim3((unsigned)dc_div_up(c->classify_warps, kCopyWarps)), kCopyWarps * 32, kCopySmem, c->stream,
-                              (const ClassifyLayer*)c->classify_table, c->n_cached, c->classify_warps, (const int32_t*)c->n_regions, c->max_regions, c->S, cur));
+                              (const ClassifyLayer*)c->classify_table, c->n_cached, c->classify_warps, c->max_regions, c->S, cur));
     }
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
@@ -611,7 +613,7 @@ int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, i
     if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_propagate, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlots * 6 * 1024 * (int)sizeof(int32_t)));
     const dim3 grid((unsigned)c->S, for_frame ? 1u : (unsigned)dc_div_up(c->max_regions, threads));
     DC_CUDA(dc_launch_pdl(k_propagate, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, in, n_in,
-                          c->table, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
+                          c->table, c->live, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
     c->launches += 1;
     return DC_OK;
 }
