@@ -72,19 +72,11 @@ __host__ __device__ constexpr size_t ctl_bytes(int epi_warps) { return sizeof(Sm
 // or another role has already given up.
 __device__ __forceinline__ bool mbar_wait(void* bar, uint32_t parity, SmemCtl* ctl, int32_t* status)
 {
-    if (mbar_try(bar, parity)) return true;
-    const unsigned long long t0 = now_ns();
-    for (uint32_t spin = 1;; ++spin) {
-        if (mbar_try(bar, parity)) return true;
-        if ((spin & 255u) == 0) {
-            if (ctl->abort_flag) return false;
-            if (now_ns() - t0 > ctl->wait_ns) {
-                ctl->abort_flag = 1;
-                atomicExch(status, (int)DC_ERR_TIMEOUT);
-                return false;
-            }
-        }
-    }
+    return mbar_wait_at(smem_u32(bar), parity, &ctl->abort_flag, &ctl->wait_ns, status);
+}
+__device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, SmemCtl* ctl, int32_t* status)
+{
+    return mbar_wait_at(bar, parity, &ctl->abort_flag, &ctl->wait_ns, status);
 }
 
 // Copies the launch's bias values behind the control block (all threads; before the set-up's __syncthreads).  The
@@ -264,16 +256,19 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     const int n_tiles = *a.tile_count;
     const int n_items = (n_tiles + MT - 1) / MT * a.NB;     // an item: MT tiles x one block of BN channels; none for this CTA: it only frees its tensor memory
 
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        int st = 0; uint32_t ph = 0;                              // ring slot and its phase
+        RingPos r;
+        r.start(smem_u32(ring), (uint32_t)a.stages);
+        const uint32_t r0 = r.data, b_at = (uint32_t)(MT * a.a_bytes);
         bool ok = true;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-            const int group = item / a.NB, nb = item % a.NB;
-            int sN[MT], xb[MT], yb[MT];
+        if (a.flat) {
             // flat tiles: lane l fetches group (l & 15) of tile (l >> 4), one box of 8 pixels per tap and chunk
-            int fs = 0, fx = 0, fy = 0; bool fon = false; uint32_t flat_tx = 0;
-            if (a.flat) {
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+                const int group = item / a.NB, nb = item % a.NB;
+                const int row0 = (nb + a.nb_off) * a.BN;
+                int fs = 0, fx = 0, fy = 0; bool fon = false;
                 const int j = lane >> 4, idx = group * MT + j;
                 if (j < MT) {
                     const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
@@ -283,88 +278,89 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     const int loc = g - fs * gps, y = loc / a.gpr;
                     fx = (loc - y * a.gpr) * DC_TILE_W * a.sw - a.pw; fy = y * a.sh - a.ph;
                 }
-                flat_tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * (uint32_t)(a.a_bytes / DC_TILE_H) + (uint32_t)a.b_bytes;
-            } else {
+                const uint32_t piece = (uint32_t)(a.a_bytes / DC_TILE_H);
+                const uint32_t tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * piece + (uint32_t)a.b_bytes;
+                for (int tap = 0; tap < taps && ok; ++tap) {
+                    const int ky = tap / a.kw, kx = tap - ky * a.kw;
+                    for (int cc = 0; cc < a.kchunks && ok; ++cc) {
+                        ok = __all_sync(0xffffffffu, mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status));
+                        if (ok && !a.skip_loads) {
+                            if (elect_one()) {
+                                mbar_expect_tx(full0 + r.off, tx);
+                                tma_load_2d(r.data + b_at, &tmB, tap * a.Ci + cc * a.BK, row0, full0 + r.off);
+                            }
+                            __syncwarp();                               // the slot is free and its byte count announced: every lane brings its own group
+                            if (fon) tma_load_4d(r.data + lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, full0 + r.off);
+                        }
+                        r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
+                    }
+                }
+            }
+        } else if (elect_one()) {
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+                const int group = item / a.NB, nb = item % a.NB;
+                const int row0 = (nb + a.nb_off) * a.BN;
+                const uint32_t tx = b_at + (uint32_t)a.b_bytes;
+                int sN[MT], xb[MT], yb[MT];
 #pragma unroll
                 for (int j = 0; j < MT; ++j) {                      // an absent second tile repeats the first (never stored)
                     const int idx = group * MT + j;
                     const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
-                    const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-                    sN[j] = s; xb[j] = tx * DC_TILE_W * a.sw - a.pw; yb[j] = ty * DC_TILE_H * a.sh - a.ph;
+                    const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx_ = t - ty * a.tiles_x;
+                    sN[j] = s; xb[j] = tx_ * DC_TILE_W * a.sw - a.pw; yb[j] = ty * DC_TILE_H * a.sh - a.ph;
                 }
-            }
-            for (int tap = 0; tap < taps && ok; ++tap) {
-                const int ky = tap / a.kw, kx = tap - ky * a.kw;
-                for (int cc = 0; cc < a.kchunks && ok; ++cc) {
-                    ok = mbar_wait(&ctl->empty[st], ph ^ 1u, ctl, a.status);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (ok && !a.skip_loads) {
-                        if (elect_one()) {
-                            uint8_t* sa = ring + (size_t)st * stage_bytes;
-                            mbar_expect_tx(&ctl->full[st], a.flat ? flat_tx : (uint32_t)stage_bytes);
-                            if (!a.flat) {
+                int w_col = 0;                                      // column of the weight matrix: taps, then channels
+                for (int ky = 0; ky < a.kh && ok; ++ky)
+                    for (int kx = 0; kx < a.kw && ok; ++kx)
+                        for (int c0 = 0; c0 < a.Ci; c0 += a.BK, w_col += a.BK) {
+                            ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
+                            if (!ok) break;
+                            if (!a.skip_loads) {
+                                mbar_expect_tx(full0 + r.off, tx);
 #pragma unroll
                                 for (int j = 0; j < MT; ++j)
-                                    tma_load_4d(sa + j * a.a_bytes, &tmA, cc * a.BK, xb[j] + kx, yb[j] + ky, sN[j], &ctl->full[st]);
+                                    tma_load_4d(r.data + j * a.a_bytes, &tmA, c0, xb[j] + kx, yb[j] + ky, sN[j], full0 + r.off);
+                                tma_load_2d(r.data + b_at, &tmB, w_col, row0, full0 + r.off);
                             }
-                            tma_load_2d(sa + MT * a.a_bytes, &tmB, tap * a.Ci + cc * a.BK, (nb + a.nb_off) * a.BN, &ctl->full[st]);
+                            r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
                         }
-                        __syncwarp();
-                    }
-                    // the slot is free and its byte count announced (lane 0, above): every lane brings its own group
-                    if (a.flat && ok && !a.skip_loads && fon)
-                        tma_load_4d(ring + (size_t)st * stage_bytes + (size_t)lane * (a.a_bytes / DC_TILE_H), &tmA, cc * a.BK, fx + kx, fy + ky, fs,
-                                    &ctl->full[st]);
-                    if (++st == a.stages) { st = 0; ph ^= 1u; }
-                }
             }
         }
+        __syncwarp();
         // on an abort: give the copies already issued a bounded chance to land before the CTA exits
-        if (!ok && lane == 0) {
+        if (__any_sync(0xffffffffu, !ok)) {
             const unsigned long long t0 = now_ns();
             while (now_ns() - t0 < 2000000ull) { }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        // One elected lane issues; descriptors differ from slot to slot in their address bits alone, so the
-        // constant upper half is built once and the loop adds (address >> 4).
-        {
+        // Descriptors differ from slot to slot in their address bits alone.
+        if (elect_one()) {
             const uint64_t dconst = umma_desc(0, a.sbo, a.layout_type);
-            const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
-            const int ksteps = a.BK / 16;
-            int st = 0; uint32_t ph = 0, acc = 0, acc_ph = 0;
+            const uint32_t d_hi = (uint32_t)(dconst >> 32), r0 = (uint32_t)dconst + (smem_u32(ring) >> 4);
+            const uint32_t stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
+            const int ksteps = a.BK / 16;                           // 16 bf16 = 32 bytes = 2 descriptor units
+            RingPos r;
+            r.start(r0, (uint32_t)a.stages);
+            uint32_t acc = 0, acc_ph = 0;
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)(MT * a.BN);
                 ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
-                ok = __all_sync(0xffffffffu, ok);
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int k = 0; k < kiters && ok; ++k) {
-                    ok = mbar_wait(&ctl->full[st], ph, ctl, a.status);
-                    ok = __all_sync(0xffffffffu, ok);
+                    ok = mbar_wait_a(full0 + r.off, r.phase, ctl, a.status);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint64_t adesc0 = dconst + (ring_lo + (uint32_t)st * stage_lo);
-                    const uint64_t bdesc = adesc0 + MT * a_lo;
-                    if (elect_one()) {
 #pragma unroll
-                        for (int j = 0; j < MT; ++j) {
-                            uint32_t acc_j = accumulate;
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk) {           // 16 bf16 = 32 bytes = 2 descriptor units
-                                if (kk < ksteps) umma_f16(d_tmem + j * a.BN, adesc0 + j * a_lo + 2 * kk, bdesc + 2 * kk, a.idesc, acc_j);
-                                acc_j = 1;
-                            }
-                        }
-                        umma_commit(&ctl->empty[st]);                  // frees the slot when these MMAs retire
-                    }
-                    __syncwarp();
+                    for (int j = 0; j < MT; ++j)
+                        umma_chunk(d_tmem + j * a.BN, r.data + j * a_lo, d_hi, 2u, r.data + MT * a_lo, d_hi, 2u, a.idesc, accumulate, ksteps);
                     accumulate = 1;
-                    if (++st == a.stages) { st = 0; ph ^= 1u; }
+                    umma_commit_at(empty0 + r.off);                    // frees the slot when these MMAs retire
+                    r.next(r0, (uint32_t)a.stages, stage_lo);
                 }
-                if (ok && elect_one()) umma_commit(&ctl->tmem_full[acc]);
-                __syncwarp();
+                if (ok) umma_commit(&ctl->tmem_full[acc]);
                 if (++acc == (uint32_t)a.nbuf) { acc = 0; acc_ph ^= 1u; }
             }
         }
@@ -441,59 +437,55 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
     const int n_items = *a.tile_count;
 
     if (warp == 0) {
-        {                                                       // producer: one patch per item
-            int st = 0; uint32_t ph = 0;
+        if (elect_one()) {                                      // producer: one patch per item
+            RingPos r;
+            r.start(smem_u32(ring), (uint32_t)a.stages);
+            const uint32_t r0 = r.data, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
             bool ok = true;
             int tile_next = a.tile_list[blockIdx.x];            // fetched one item ahead: off the critical path
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+            for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
                 const int tile = tile_next;
                 if (item + (int)gridDim.x < n_items) tile_next = a.tile_list[item + gridDim.x];
                 const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-                ok = __all_sync(0xffffffffu, mbar_wait(&ctl->empty[st], ph ^ 1u, ctl, a.status));
+                ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
                 if (!ok) break;
-                if (!a.skip_loads && elect_one()) {
-                    mbar_expect_tx(&ctl->full[st], (uint32_t)(sa.PW * sa.PH * 16));
-                    tma_load_4d(ring + (size_t)st * sa.stage_bytes, &tmA, 0, tx * DC_TILE_W - a.pw, ty * DC_TILE_H - a.ph, s, &ctl->full[st]);
+                if (!a.skip_loads) {
+                    mbar_expect_tx(full0 + r.off, (uint32_t)(sa.PW * sa.PH * 16));
+                    tma_load_4d(r.data, &tmA, 0, tx * DC_TILE_W - a.pw, ty * DC_TILE_H - a.ph, s, full0 + r.off);
                 }
-                __syncwarp();
-                if (++st == a.stages) { st = 0; ph ^= 1u; }
+                r.next(r0, (uint32_t)a.stages, (uint32_t)sa.stage_bytes);
             }
-            if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
+            if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
         }
         __syncwarp();
     } else if (warp == 1) {
-        {                                                       // MMA issuer
+        if (elect_one()) {                                      // MMA issuer
             const uint32_t b_lbo = (uint32_t)a.Co * 16u;
             const uint64_t bconst = umma_desc(smem_u32(wsm), 128, 0, b_lbo);
-            const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)sa.stage_bytes >> 4;
             const uint64_t hi = umma_desc(0, (uint32_t)sa.PW * 16u, 0, 0);     // SBO = one patch row; LBO added per K step
-            int st = 0; uint32_t ph = 0, acc = 0, acc_ph = 0;
-            bool ok = true;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status) && mbar_wait(&ctl->full[st], ph, ctl, a.status);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+            RingPos r;
+            r.start(smem_u32(ring) >> 4, (uint32_t)a.stages);
+            const uint32_t r0 = r.data, stage_lo = (uint32_t)sa.stage_bytes >> 4, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+            uint32_t acc = 0, acc_ph = 0;
+            for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+                if (!(mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status) && mbar_wait_a(full0 + r.off, r.phase, ctl, a.status))) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)a.BN;
-                const uint32_t patch_lo = ring_lo + (uint32_t)st * stage_lo;
                 // K step kk covers taps 2kk and 2kk+1: two 16-byte pixel columns of the patch, `lbo` apart
                 int tap = 0, ky = 0, kx = 0;
-                if (elect_one()) {
-                    for (int kk = 0; kk < sa.kblocks / 2; ++kk) {
-                        const uint32_t off0 = (uint32_t)(ky * sa.PW + kx);
-                        if (++kx == a.kw) { kx = 0; ++ky; }
-                        ++tap;
-                        uint32_t off1 = off0 + 1;                      // past the last tap: any finite data (its weights are zero)
-                        if (tap < taps) { off1 = (uint32_t)(ky * sa.PW + kx); if (++kx == a.kw) { kx = 0; ++ky; } }
-                        ++tap;
-                        const uint64_t adesc = hi + (patch_lo + off0) + ((uint64_t)(off1 - off0) << 16);
-                        umma_f16(d_tmem, adesc, bconst + (uint64_t)(kk * ((2 * b_lbo) >> 4)), a.idesc, kk != 0);
-                    }
-                    umma_commit(&ctl->empty[st]);
-                    umma_commit(&ctl->tmem_full[acc]);
+                for (int kk = 0; kk < sa.kblocks / 2; ++kk) {
+                    const uint32_t off0 = (uint32_t)(ky * sa.PW + kx);
+                    if (++kx == a.kw) { kx = 0; ++ky; }
+                    ++tap;
+                    uint32_t off1 = off0 + 1;                      // past the last tap: any finite data (its weights are zero)
+                    if (tap < taps) { off1 = (uint32_t)(ky * sa.PW + kx); if (++kx == a.kw) { kx = 0; ++ky; } }
+                    ++tap;
+                    const uint64_t adesc = hi + (r.data + off0) + ((uint64_t)(off1 - off0) << 16);
+                    umma_f16(d_tmem, adesc, bconst + (uint64_t)(kk * ((2 * b_lbo) >> 4)), a.idesc, kk != 0);
                 }
-                __syncwarp();
-                if (++st == a.stages) { st = 0; ph ^= 1u; }
+                umma_commit_at(empty0 + r.off);
+                umma_commit(&ctl->tmem_full[acc]);
+                r.next(r0, (uint32_t)a.stages, stage_lo);
                 if (++acc == 2u) { acc = 0; acc_ph ^= 1u; }
             }
         }
@@ -527,12 +519,6 @@ struct TcHaloArgs {
     int PW, PH, plane_bytes, patch_bytes, a_stages;
     int k_last;                      // K steps of 16 channels in the last chunk (4 unless the channels are no multiple of 64)
 };
-
-__device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32_t bytes, void* bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
 
 // SLAB = false: the A side of a 64-channel chunk is one (16 + kh - 1) x (8 + kw - 1) patch in eight 16-byte planes
 //               (unswizzled core matrices), read in place by every tap.
@@ -579,118 +565,111 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
     const int n_tiles = *a.tile_count;
     const int n_items = (n_tiles + MT - 1) / MT * a.NB;
 
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
     if (warp == 0) {
         // ---------------- producer: patches by TMA, weights by bulk copy ----------------
-        int sa = 0, sb = 0; uint32_t pa = 0, pb = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-            const int group = item / a.NB, nb = item % a.NB;
-            int sN[MT], xb[MT], yb[MT];
+        if (elect_one()) {
+            RingPos ra, rb;
+            ra.start(smem_u32(aring), (uint32_t)ha.a_stages); rb.start(smem_u32(bring), (uint32_t)a.stages);
+            const uint32_t a0 = ra.data, b0 = rb.data;
+            const size_t tap_stride = (size_t)a.kchunks * a.b_bytes;             // packed weights: one tap further
+            bool ok = true;
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+                const int group = item / a.NB, nb = item % a.NB;
+                int sN[MT], xb[MT], yb[MT];
 #pragma unroll
-            for (int j = 0; j < MT; ++j) {
-                const int idx = group * MT + j;
-                const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
-                const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-                sN[j] = s; xb[j] = tx * DC_TILE_W - a.pw; yb[j] = ty * DC_TILE_H - a.ph;
-            }
-            for (int cc = 0; cc < a.kchunks && ok; ++cc) {
-                for (int kx = 0; kx < (SLAB ? a.kw : 1) && ok; ++kx) {
-                    ok = mbar_wait(&ctl->a_empty[sa], pa ^ 1u, ctl, a.status);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (ok && !a.skip_loads) {
-                        if (elect_one()) {
+                for (int j = 0; j < MT; ++j) {
+                    const int idx = group * MT + j;
+                    const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
+                    const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
+                    sN[j] = s; xb[j] = tx * DC_TILE_W - a.pw; yb[j] = ty * DC_TILE_H - a.ph;
+                }
+                const uint8_t* w_item = (const uint8_t*)ha.wpacked + (size_t)(nb + a.nb_off) * taps * tap_stride;
+                for (int cc = 0; cc < a.kchunks && ok; ++cc) {
+                    for (int kx = 0; kx < (SLAB ? a.kw : 1) && ok; ++kx) {
+                        ok = mbar_wait_a(a_empty0 + ra.off, ra.phase ^ 1u, ctl, a.status);
+                        if (!ok) break;
+                        if (!a.skip_loads) {
                             if (SLAB) {
-                                mbar_expect_tx(&ctl->a_full[sa], (uint32_t)(MT * ha.patch_bytes));
+                                mbar_expect_tx(a_full0 + ra.off, (uint32_t)(MT * ha.patch_bytes));
 #pragma unroll
                                 for (int j = 0; j < MT; ++j)
-                                    tma_load_4d(aring + (size_t)sa * a_slot + j * ha.patch_bytes, &tmA, cc * 64, xb[j] + kx, yb[j], sN[j],
-                                                &ctl->a_full[sa]);
+                                    tma_load_4d(ra.data + j * ha.patch_bytes, &tmA, cc * 64, xb[j] + kx, yb[j], sN[j], a_full0 + ra.off);
                             } else {
-                                mbar_expect_tx(&ctl->a_full[sa], (uint32_t)(MT * 8 * ha.PW * ha.PH * 16));
+                                mbar_expect_tx(a_full0 + ra.off, (uint32_t)(MT * 8 * ha.PW * ha.PH * 16));
 #pragma unroll
                                 for (int j = 0; j < MT; ++j)
                                     for (int g = 0; g < 8; ++g)
-                                        tma_load_4d(aring + (size_t)sa * a_slot + j * ha.patch_bytes + g * ha.plane_bytes, &tmA,
-                                                    cc * 64 + g * 8, xb[j], yb[j], sN[j], &ctl->a_full[sa]);
+                                        tma_load_4d(ra.data + j * ha.patch_bytes + g * ha.plane_bytes, &tmA, cc * 64 + g * 8, xb[j], yb[j], sN[j], a_full0 + ra.off);
                             }
                         }
-                        __syncwarp();
-                    }
-                    if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
-                    // the weight tiles that go with this A stage: all taps (patch), or the taps of column kx (slab)
-                    for (int t = 0; t < (SLAB ? a.kh : taps) && ok; ++t) {
-                        const int tap = SLAB ? t * a.kw + kx : t;
-                        ok = mbar_wait(&ctl->empty[sb], pb ^ 1u, ctl, a.status);
-                        ok = __all_sync(0xffffffffu, ok);
-                        if (ok && !a.skip_loads) {
-                            if (elect_one()) {
-                                mbar_expect_tx(&ctl->full[sb], (uint32_t)a.b_bytes);
-                                const uint8_t* src = (const uint8_t*)ha.wpacked + ((size_t)((nb + a.nb_off) * taps + tap) * a.kchunks + cc) * a.b_bytes;
-                                bulk_copy_g2s(bring + (size_t)sb * a.b_bytes, src, (uint32_t)a.b_bytes, &ctl->full[sb]);
+                        ra.next(a0, (uint32_t)ha.a_stages, (uint32_t)a_slot);
+                        // the weight tiles that go with this A stage: all taps (patch), or the taps of column kx (slab)
+                        const uint8_t* w = w_item + kx * tap_stride + (size_t)cc * a.b_bytes;
+                        const size_t w_step = SLAB ? a.kw * tap_stride : tap_stride;
+                        const int n_t = SLAB ? a.kh : taps;
+                        for (int t = 0; t < n_t; ++t) {
+                            ok = mbar_wait_a(empty0 + rb.off, rb.phase ^ 1u, ctl, a.status);
+                            if (!ok) break;
+                            if (!a.skip_loads) {
+                                mbar_expect_tx(full0 + rb.off, (uint32_t)a.b_bytes);
+                                bulk_copy(rb.data, w, (uint32_t)a.b_bytes, full0 + rb.off);
                             }
-                            __syncwarp();
+                            w += w_step;
+                            rb.next(b0, (uint32_t)a.stages, (uint32_t)a.b_bytes);
                         }
-                        if (++sb == a.stages) { sb = 0; pb ^= 1u; }
                     }
                 }
             }
+            if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
         }
-        if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
+        __syncwarp();
     } else if (warp == 1) {
-        // ---------------- MMA issuer (one elected lane) ----------------
-        {
-            // A: patch planes (rows PW * 16 bytes apart, planes along K), or a 128-byte swizzled K-major slab
+        // ---------------- MMA issuer ----------------
+        if (elect_one()) {
+            // A: patch planes (rows PW * 16 bytes apart, planes along K), or a 128-byte swizzled K-major slab; weights: 128-byte
+            // swizzled, K-major.  Descriptors differ from slot to slot in their lower halves alone.
             const uint64_t aconst = SLAB ? umma_desc(0, 1024, 2) : umma_desc(0, (uint32_t)ha.PW * 16u, 0, (uint32_t)ha.plane_bytes);
-            const uint64_t bconst = umma_desc(0, 1024, 2);                               // weights: 128-byte swizzled, K-major
-            const uint32_t aring_lo = smem_u32(aring) >> 4, bring_lo = smem_u32(bring) >> 4;
-            const uint32_t a_slot_lo = (uint32_t)a_slot >> 4, patch_lo = (uint32_t)ha.patch_bytes >> 4;
+            const uint64_t bconst = umma_desc(0, 1024, 2);
+            const uint32_t a_hi = (uint32_t)(aconst >> 32), b_hi = (uint32_t)(bconst >> 32);
+            const uint32_t a0 = (uint32_t)aconst + (smem_u32(aring) >> 4), b0 = (uint32_t)bconst + (smem_u32(bring) >> 4);
+            const uint32_t a_slot_lo = (uint32_t)a_slot >> 4, patch_lo = (uint32_t)ha.patch_bytes >> 4, b_lo = (uint32_t)a.b_bytes >> 4;
             const uint32_t a_kstep = SLAB ? 2u : (uint32_t)(2 * ha.plane_bytes) >> 4;    // 16 channels further along K
-            const uint32_t b_kstep = 2u, b_lo = (uint32_t)a.b_bytes >> 4;
-            int sa = 0, sb = 0; uint32_t pa = 0, pb = 0, acc = 0, acc_ph = 0;
+            RingPos ra, rb;
+            ra.start(a0, (uint32_t)ha.a_stages); rb.start(b0, (uint32_t)a.stages);
+            uint32_t acc = 0, acc_ph = 0;
             bool ok = true;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)(MT * a.BN);
                 ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
-                ok = __all_sync(0xffffffffu, ok);
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                     const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < (SLAB ? a.kw : 1) && ok; ++ax) {     // A stages of this chunk: one patch, or kw slabs
-                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->a_full[sa], pa, ctl, a.status));
-                        const uint64_t apatch = aconst + (aring_lo + (uint32_t)sa * a_slot_lo);
+                        ok = mbar_wait_a(a_full0 + ra.off, ra.phase, ctl, a.status);
                         // patch: taps in (ky, kx) order at (ky * PW + kx) * 16 bytes; slab ax: taps (ky, ax) at ky atoms of 1024 bytes
+                        uint32_t at = ra.data;
+                        int col = 0;
                         const int n_t = SLAB ? a.kh : taps;
                         for (int t = 0; t < n_t && ok; ++t) {
-                            const uint32_t tap_lo = SLAB ? (uint32_t)t * 64u : (uint32_t)((t / a.kw) * ha.PW + t % a.kw);
-                            ok = __all_sync(0xffffffffu, mbar_wait(&ctl->full[sb], pb, ctl, a.status));
+                            ok = mbar_wait_a(full0 + rb.off, rb.phase, ctl, a.status);
                             if (!ok) break;
                             tc_fence_after();
-                            const uint64_t bdesc = bconst + (bring_lo + (uint32_t)sb * b_lo);
-                            if (elect_one()) {
 #pragma unroll
-                                for (int j = 0; j < MT; ++j) {
-                                    const uint64_t adesc = apatch + j * patch_lo + tap_lo;
-                                    uint32_t acc_j = accumulate;
-#pragma unroll
-                                    for (int kk = 0; kk < 4; ++kk) {    // K = 16 per instruction, up to 64 channels per chunk
-                                        if (kk < n_kk) umma_f16(d_tmem + j * a.BN, adesc + kk * a_kstep, bdesc + kk * b_kstep, a.idesc, acc_j);
-                                        acc_j = 1;
-                                    }
-                                }
-                                umma_commit(&ctl->empty[sb]);
-                            }
-                            __syncwarp();
+                            for (int j = 0; j < MT; ++j)
+                                umma_chunk(d_tmem + j * a.BN, at + j * patch_lo, a_hi, a_kstep, rb.data, b_hi, 2u, a.idesc, accumulate, n_kk);
                             accumulate = 1;
-                            if (++sb == a.stages) { sb = 0; pb ^= 1u; }
+                            umma_commit_at(empty0 + rb.off);
+                            rb.next(b0, (uint32_t)a.stages, b_lo);
+                            if (SLAB) at += 64u;
+                            else if (++col == a.kw) { col = 0; at += (uint32_t)(ha.PW - a.kw + 1); } else at += 1u;
                         }
-                        if (ok && elect_one()) umma_commit(&ctl->a_empty[sa]);   // the A stage is free once its taps retire
-                        __syncwarp();
-                        if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
+                        if (ok) umma_commit_at(a_empty0 + ra.off);             // the A stage is free once its taps retire
+                        ra.next(a0, (uint32_t)ha.a_stages, a_slot_lo);
                     }
                 }
-                if (ok && elect_one()) umma_commit(&ctl->tmem_full[acc]);
-                __syncwarp();
+                if (ok) umma_commit(&ctl->tmem_full[acc]);
                 if (++acc == (uint32_t)a.nbuf) { acc = 0; acc_ph ^= 1u; }
             }
         }
@@ -721,27 +700,21 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
 // empty / a_empty / tmem_full exist in each CTA and are signalled in both by the leader's tcgen05.commit.
 // ---------------------------------------------------------------------------------------------
 // loads into this CTA's shared memory whose bytes are counted on the barrier at shared::cluster address `bar` (the leader's)
-__device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, uint32_t bar)
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, uint32_t bar)
 {
     asm volatile("cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+                 ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar)
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar)
 {
     asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tm), "r"(bar), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+                 ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
 // arrives, once the MMAs issued so far have retired, on the barrier at this offset in both CTAs of the pair
-__device__ __forceinline__ void umma_commit_pair(void* bar)
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+                 ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
 
 // ha.t.BN: output channels per item (both CTAs together); ha.t.b_bytes: one CTA's weight tile (BN / 2 rows of 128 bytes);
@@ -787,92 +760,81 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int n_tiles = *a.tile_count;
     const int n_items = (n_tiles + 1) / 2 * a.NB;
 
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
     if (warp == 0) {
         // ---------------- producer: this CTA's slab and its half of the weights ----------------
-        const uint32_t a_full0 = map_to_cta(&ctl->a_full[0], 0), full0 = map_to_cta(&ctl->full[0], 0);   // the leader's barriers
-        int sa = 0, sb = 0; uint32_t pa = 0, pb = 0;
-        bool ok = true;
-        const int rows_per_tile = a.b_bytes >> 7;             // weight rows of 128 bytes in one CTA's tile
-        for (int item = pair; item < n_items && ok; item += n_pairs) {
-            const int group = item / a.NB, nb = item % a.NB;
-            const int idx = group * 2 + (int)rank;
-            const int tile = a.tile_list[idx < n_tiles ? idx : group * 2];      // an absent second tile repeats the first (never stored)
-            const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
-            const int xb = tx * DC_TILE_W - a.pw, yb = ty * DC_TILE_H - a.ph;
-            for (int cc = 0; cc < a.kchunks && ok; ++cc) {
-                for (int kx = 0; kx < a.kw && ok; ++kx) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&ctl->a_empty[sa], pa ^ 1u, ctl, a.status));
-                    if (ok && !a.skip_loads) {
-                        if (elect_one()) {
-                            if (leader) mbar_expect_tx(&ctl->a_full[sa], (uint32_t)(2 * ha.patch_bytes));
-                            tma_load_4d_pair(aring + (size_t)sa * a_slot, &tmA, cc * 64, xb + kx, yb, s, a_full0 + (uint32_t)sa * 8u);
+        if (elect_one()) {
+            const uint32_t lead_a_full = map_to_cta(&ctl->a_full[0], 0), lead_full = map_to_cta(&ctl->full[0], 0);   // the leader's barriers
+            RingPos ra, rb;
+            ra.start(smem_u32(aring), (uint32_t)ha.a_stages); rb.start(smem_u32(bring), (uint32_t)a.stages);
+            const uint32_t a0 = ra.data, b0 = rb.data;
+            const int rows_per_tile = a.b_bytes >> 7;             // weight rows of 128 bytes in one CTA's tile
+            bool ok = true;
+            for (int item = pair; item < n_items && ok; item += n_pairs) {
+                const int group = item / a.NB, nb = item % a.NB;
+                const int idx = group * 2 + (int)rank;
+                const int tile = a.tile_list[idx < n_tiles ? idx : group * 2];      // an absent second tile repeats the first (never stored)
+                const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
+                const int xb = tx * DC_TILE_W - a.pw, yb = ty * DC_TILE_H - a.ph;
+                const int row_step = a.kw * a.kchunks * rows_per_tile;              // packed weights: one kernel row further
+                for (int cc = 0; cc < a.kchunks && ok; ++cc) {
+                    for (int kx = 0; kx < a.kw && ok; ++kx) {
+                        ok = mbar_wait_a(a_empty0 + ra.off, ra.phase ^ 1u, ctl, a.status);
+                        if (!ok) break;
+                        if (!a.skip_loads) {
+                            if (leader) mbar_expect_tx(a_full0 + ra.off, (uint32_t)(2 * ha.patch_bytes));
+                            tma_load_4d_pair(ra.data, &tmA, cc * 64, xb + kx, yb, s, lead_a_full + ra.off);
                         }
-                        __syncwarp();
-                    }
-                    if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
-                    for (int t2 = 0; t2 < a.kh && ok; ++t2) {
-                        const int tap = t2 * a.kw + kx;
-                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->empty[sb], pb ^ 1u, ctl, a.status));
-                        if (ok && !a.skip_loads) {
-                            if (elect_one()) {
-                                if (leader) mbar_expect_tx(&ctl->full[sb], (uint32_t)(2 * a.b_bytes));
-                                const int row = (((nb * 2 + (int)rank) * taps + tap) * a.kchunks + cc) * rows_per_tile;
-                                tma_load_2d_pair(bring + (size_t)sb * a.b_bytes, &tmW, 0, row, full0 + (uint32_t)sb * 8u);
+                        ra.next(a0, (uint32_t)ha.a_stages, (uint32_t)a_slot);
+                        int row = (((nb * 2 + (int)rank) * taps + kx) * a.kchunks + cc) * rows_per_tile;
+                        for (int t2 = 0; t2 < a.kh; ++t2, row += row_step) {
+                            ok = mbar_wait_a(empty0 + rb.off, rb.phase ^ 1u, ctl, a.status);
+                            if (!ok) break;
+                            if (!a.skip_loads) {
+                                if (leader) mbar_expect_tx(full0 + rb.off, (uint32_t)(2 * a.b_bytes));
+                                tma_load_2d_pair(rb.data, &tmW, 0, row, lead_full + rb.off);
                             }
-                            __syncwarp();
+                            rb.next(b0, (uint32_t)a.stages, (uint32_t)a.b_bytes);
                         }
-                        if (++sb == a.stages) { sb = 0; pb ^= 1u; }
                     }
                 }
             }
+            if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
         }
-        if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
+        __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer: an elected lane of the leader issues for both CTAs ----------------
-        if (leader) {
-            const uint64_t aconst = umma_desc(0, 1024, 2);
-            const uint64_t bconst = umma_desc(0, 1024, 2);                               // weights: 128-byte swizzled, K-major
-            const uint32_t aring_lo = smem_u32(aring) >> 4, bring_lo = smem_u32(bring) >> 4;
-            const uint32_t a_slot_lo = (uint32_t)a_slot >> 4;
-            const uint32_t b_kstep = 2u, b_lo = (uint32_t)a.b_bytes >> 4;
-            int sa = 0, sb = 0; uint32_t pa = 0, pb = 0, acc = 0, acc_ph = 0;
+        if (leader && elect_one()) {
+            const uint64_t dconst = umma_desc(0, 1024, 2);            // slabs and weights: 128-byte swizzled, K-major
+            const uint32_t d_hi = (uint32_t)(dconst >> 32), a0 = (uint32_t)dconst + (smem_u32(aring) >> 4), b0 = (uint32_t)dconst + (smem_u32(bring) >> 4);
+            const uint32_t a_slot_lo = (uint32_t)a_slot >> 4, b_lo = (uint32_t)a.b_bytes >> 4;
+            RingPos ra, rb;
+            ra.start(a0, (uint32_t)ha.a_stages); rb.start(b0, (uint32_t)a.stages);
+            uint32_t acc = 0, acc_ph = 0;
             bool ok = true;
             for (int item = pair; item < n_items && ok; item += n_pairs) {
                 const uint32_t d_tmem = tmem_base + acc * (uint32_t)a.BN;
-                ok = __all_sync(0xffffffffu, mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status));
+                ok = mbar_wait(&ctl->tmem_empty[acc], acc_ph ^ 1u, ctl, a.status);
                 tc_fence_after();
                 uint32_t accumulate = 0;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                     const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < a.kw && ok; ++ax) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(&ctl->a_full[sa], pa, ctl, a.status));
-                        const uint64_t aslab = aconst + (aring_lo + (uint32_t)sa * a_slot_lo);
+                        ok = mbar_wait_a(a_full0 + ra.off, ra.phase, ctl, a.status);
                         for (int t = 0; t < a.kh && ok; ++t) {               // tap (t, ax): the slab from swizzle atom t on
-                            ok = __all_sync(0xffffffffu, mbar_wait(&ctl->full[sb], pb, ctl, a.status));
+                            ok = mbar_wait_a(full0 + rb.off, rb.phase, ctl, a.status);
                             if (!ok) break;
                             tc_fence_after();
-                            const uint64_t bdesc = bconst + (bring_lo + (uint32_t)sb * b_lo);
-                            const uint64_t adesc = aslab + (uint32_t)t * 64u;
-                            if (elect_one()) {
-                                uint32_t acc_k = accumulate;
-#pragma unroll
-                                for (int kk = 0; kk < 4; ++kk) {             // K = 16 per instruction, up to 64 channels per chunk
-                                    if (kk < n_kk) umma_f16_pair(d_tmem, adesc + kk * 2u, bdesc + kk * b_kstep, a.idesc, acc_k);
-                                    acc_k = 1;
-                                }
-                                umma_commit_pair(&ctl->empty[sb]);
-                            }
-                            __syncwarp();
+                            umma_chunk_pair(d_tmem, ra.data + (uint32_t)t * 64u, d_hi, 2u, rb.data, d_hi, 2u, a.idesc, accumulate, n_kk);
                             accumulate = 1;
-                            if (++sb == a.stages) { sb = 0; pb ^= 1u; }
+                            umma_commit_pair(empty0 + rb.off);
+                            rb.next(b0, (uint32_t)a.stages, b_lo);
                         }
-                        if (ok && elect_one()) umma_commit_pair(&ctl->a_empty[sa]);
-                        __syncwarp();
-                        if (++sa == ha.a_stages) { sa = 0; pa ^= 1u; }
+                        if (ok) umma_commit_pair(a_empty0 + ra.off);
+                        ra.next(a0, (uint32_t)ha.a_stages, a_slot_lo);
                     }
                 }
-                if (ok && elect_one()) umma_commit_pair(&ctl->tmem_full[acc]);
-                __syncwarp();
+                if (ok) umma_commit_pair(smem_u32(&ctl->tmem_full[acc]));
                 if (++acc == 2u) { acc = 0; acc_ph ^= 1u; }
             }
         }

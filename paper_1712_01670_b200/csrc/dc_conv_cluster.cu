@@ -27,22 +27,9 @@ struct CtlCl {
     unsigned long long wait_ns;
 };
 
-// Bounded wait, as in dc_conv_bf16.cu.
-__device__ __forceinline__ bool cl_wait(void* bar, uint32_t parity, CtlCl* ctl, int32_t* status)
+__device__ __forceinline__ bool cl_wait(uint32_t bar, uint32_t parity, CtlCl* ctl, int32_t* status)
 {
-    if (mbar_try(bar, parity)) return true;
-    const unsigned long long t0 = now_ns();
-    for (uint32_t spin = 1;; ++spin) {
-        if (mbar_try(bar, parity)) return true;
-        if ((spin & 255u) == 0) {
-            if (ctl->abort_flag) return false;
-            if (now_ns() - t0 > ctl->wait_ns) {
-                ctl->abort_flag = 1;
-                atomicExch(status, (int)DC_ERR_TIMEOUT);
-                return false;
-            }
-        }
-    }
+    return mbar_wait_at(bar, parity, &ctl->abort_flag, &ctl->wait_ns, status);
 }
 __device__ __forceinline__ void st_remote(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
@@ -81,14 +68,21 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");    // waited for before another CTA's shared memory is written
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    auto load_weights = [&](int it) {
-        const int st = it % a.stages, tap = (k0 + it) / a.kchunks, cc = (k0 + it) - tap * a.kchunks;
-        mbar_expect_tx(&ctl->full[st], (uint32_t)a.b_bytes);
-        tma_load_2d(ring + (size_t)st * stage_bytes + a.a_bytes, &tmB, tap * a.Ci + cc * a.BK, (nb + a.nb_off) * a.BN, &ctl->full[st]);
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), ring0 = smem_u32(ring);
+    const int tap0 = k0 / a.kchunks, cc0 = k0 - tap0 * a.kchunks;
+    const int w_row = (nb + a.nb_off) * a.BN, early = nk < a.stages ? nk : a.stages;
+    auto load_weights = [&](int tap, int cc, uint32_t off, uint32_t slot) {
+        mbar_expect_tx(full0 + off, (uint32_t)a.b_bytes);
+        tma_load_2d(slot + a.a_bytes, &tmB, tap * a.Ci + cc * a.BK, w_row, full0 + off);
     };
-    const int early = nk < a.stages ? nk : a.stages;
-    if (warp == 0 && !a.skip_loads)
-        for (int it = 0; it < early; ++it) { if (elect_one()) load_weights(it); __syncwarp(); }
+    if (warp == 0 && !a.skip_loads && elect_one()) {
+        int tap = tap0, cc = cc0;
+        for (int it = 0; it < early; ++it) {
+            load_weights(tap, cc, 8u * it, ring0 + it * stage_bytes);
+            if (++cc == a.kchunks) { cc = 0; ++tap; }
+        }
+    }
+    __syncwarp();
     dc_pdl_wait();                           // the previous kernel's output, the tile list and its count are read from here on
     dc_pdl_release();
     const int n_tiles = *a.tile_count;
@@ -137,7 +131,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         if (!present) {
             // the weights are on their way: let them land before this CTA's shared memory is given up
             if (lane == 0 && !a.skip_loads)
-                for (int it = 0; it < early && ok; ++it) { mbar_arrive(&ctl->full[it]); ok = cl_wait(&ctl->full[it], 0, ctl, a.status); }
+                for (int it = 0; it < early && ok; ++it) { mbar_arrive(&ctl->full[it]); ok = cl_wait(full0 + 8u * it, 0, ctl, a.status); }
         } else if (!a.skip_loads) {
             // 16 x 8 tile: an elected lane brings the window of a tap; flat tiles: lane l brings row piece l
             int fs = 0, fx = 0, fy = 0;
@@ -149,46 +143,59 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
             } else {
                 fs = ts; fx = tx * DC_TILE_W * a.sw - a.pw; fy = ty * DC_TILE_H * a.sh - a.ph;
             }
-            const int piece = a.flat ? a.a_bytes / DC_TILE_H : 0;
-            const uint32_t a_tx = a.flat ? (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * (uint32_t)piece : (uint32_t)a.a_bytes;
-            for (int it = 0; it < nk && ok; ++it) {
-                const int st = it % a.stages, tap = (k0 + it) / a.kchunks, cc = (k0 + it) - tap * a.kchunks, ky = tap / a.kw, kx = tap - ky * a.kw;
-                if (it >= a.stages) ok = __all_sync(0xffffffffu, cl_wait(&ctl->empty[st], (uint32_t)(it / a.stages - 1) & 1u, ctl, a.status));
-                if (!ok) break;
-                if (elect_one()) {
-                    if (it >= a.stages) load_weights(it);
-                    mbar_expect_tx(&ctl->full[st], a_tx);
-                    if (!a.flat) tma_load_4d(ring + (size_t)st * stage_bytes, &tmA, cc * a.BK, fx + kx, fy + ky, fs, &ctl->full[st]);
+            RingPos r;
+            r.start(ring0, (uint32_t)a.stages);
+            int cc = cc0, ky = tap0 / a.kw, kx = tap0 - ky * a.kw;
+            auto advance = [&]() {
+                if (++cc == a.kchunks) { cc = 0; if (++kx == a.kw) { kx = 0; ++ky; } }
+                r.next(ring0, (uint32_t)a.stages, (uint32_t)stage_bytes);
+            };
+            if (a.flat) {
+                const uint32_t piece = (uint32_t)(a.a_bytes / DC_TILE_H), a_tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * piece;
+                for (int it = 0; it < nk; ++it) {
+                    if (it >= a.stages) ok = __all_sync(0xffffffffu, cl_wait(empty0 + r.off, r.phase ^ 1u, ctl, a.status));
+                    if (!ok) break;
+                    if (elect_one()) {
+                        if (it >= a.stages) load_weights(ky * a.kw + kx, cc, r.off, r.data);
+                        mbar_expect_tx(full0 + r.off, a_tx);
+                    }
+                    __syncwarp();
+                    if (fon) tma_load_4d(r.data + lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, full0 + r.off);
+                    __syncwarp();
+                    advance();
                 }
-                __syncwarp();
-                if (a.flat && fon) tma_load_4d(ring + (size_t)st * stage_bytes + (size_t)lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, &ctl->full[st]);
-                __syncwarp();
+            } else if (elect_one()) {
+                for (int it = 0; it < nk; ++it) {
+                    if (it >= a.stages) {
+                        ok = cl_wait(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
+                        if (!ok) break;
+                        load_weights(ky * a.kw + kx, cc, r.off, r.data);
+                    }
+                    mbar_expect_tx(full0 + r.off, (uint32_t)a.a_bytes);
+                    tma_load_4d(r.data, &tmA, cc * a.BK, fx + kx, fy + ky, fs, full0 + r.off);
+                    advance();
+                }
             }
         }
         // on an abort: give the copies already issued a bounded chance to land before the CTA exits
-        if (!ok && lane == 0) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
+        if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (present) {
+        if (present && elect_one()) {
             const uint64_t dconst = umma_desc(0, a.sbo, a.layout_type);
-            const uint32_t ring_lo = smem_u32(ring) >> 4, stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
+            const uint32_t d_hi = (uint32_t)(dconst >> 32), r0 = (uint32_t)dconst + (ring0 >> 4);
+            const uint32_t stage_lo = (uint32_t)stage_bytes >> 4, a_lo = (uint32_t)a.a_bytes >> 4;
             const int ksteps = a.BK / 16;
-            bool ok = true;
-            for (int it = 0; it < nk && ok; ++it) {
-                const int st = it % a.stages;
-                ok = __all_sync(0xffffffffu, cl_wait(&ctl->full[st], (uint32_t)(it / a.stages) & 1u, ctl, a.status));
-                if (!ok) break;
+            RingPos r;
+            r.start(r0, (uint32_t)a.stages);
+            for (int it = 0; it < nk; ++it) {
+                if (!cl_wait(full0 + r.off, r.phase, ctl, a.status)) break;
                 tc_fence_after();
-                const uint64_t adesc = dconst + (ring_lo + (uint32_t)st * stage_lo), bdesc = adesc + a_lo;
-                if (elect_one()) {
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        if (kk < ksteps) umma_f16(tmem_base, adesc + 2 * kk, bdesc + 2 * kk, a.idesc, (uint32_t)((it | kk) != 0));
-                    if (it + a.stages < nk) umma_commit(&ctl->empty[st]);
-                    if (it + 1 == nk) umma_commit(&ctl->done);
-                }
-                __syncwarp();
+                umma_chunk(tmem_base, r.data, d_hi, 2u, r.data + a_lo, d_hi, 2u, a.idesc, (uint32_t)(it != 0), ksteps);
+                if (it + a.stages < nk) umma_commit_at(empty0 + r.off);
+                if (it + 1 == nk) umma_commit(&ctl->done);
+                r.next(r0, (uint32_t)a.stages, stage_lo);
             }
         }
         __syncwarp();
@@ -197,7 +204,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         const int q = warp & 3, m = q * 32 + lane;                   // tensor-memory lane quadrant of this warp, its pixel
         const int owner = m / rows;
         const uint32_t dst = map_to_cta(red + (rank * rows + m - owner * rows) * red_pitch(a.BN), (uint32_t)owner);
-        bool ok = cl_wait(&ctl->done, 0, ctl, a.status);
+        bool ok = cl_wait(smem_u32(&ctl->done), 0, ctl, a.status);
         ok = __all_sync(0xffffffffu, ok);
         asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         if (ok) {

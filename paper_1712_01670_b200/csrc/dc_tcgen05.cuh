@@ -9,8 +9,9 @@ namespace {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// One lane of a converged warp, chosen by the hardware.  Loops around TMA, MMA and commit instructions run in the whole
-// warp and only the instruction itself is guarded by this: the compiler then knows the warp is converged there.
+// One lane of a converged warp, chosen by the hardware.  The producer and MMA roles run inside `if (elect_one())`: behind
+// elect.sync the compiler knows that a single lane of a converged warp is active and issues TMA, MMA and commit
+// instructions directly; behind `lane == 0` it does not, and a step of a role's loop (64 channels) took up to twice as long.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
@@ -20,10 +21,6 @@ __device__ __forceinline__ bool elect_one()
 __device__ __forceinline__ void mbar_init(void* bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(void* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(void* bar)
 {
@@ -40,29 +37,88 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t addr)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-__device__ __forceinline__ bool mbar_try(void* bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
 __device__ __forceinline__ unsigned long long now_ns()
 {
     unsigned long long t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, void* bar)
+// Barriers and destinations of loads as 32-bit shared-memory addresses: what bounds a role's loop is the instructions that
+// one lane can issue, so the loops keep addresses in registers and advance them (RingPos).
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Bounded wait: false (with the abort flag and the status word set) when `limit` nanoseconds have passed or another role
+// has given up.
+__device__ __forceinline__ bool mbar_wait_at(uint32_t bar, uint32_t parity, volatile int* abort_flag, const unsigned long long* limit, int32_t* status)
+{
+    if (mbar_try(bar, parity)) return true;
+    const unsigned long long t0 = now_ns();
+    for (uint32_t spin = 1;; ++spin) {
+        if (mbar_try(bar, parity)) return true;
+        if ((spin & 255u) == 0) {
+            if (*abort_flag) return false;
+            if (now_ns() - t0 > *limit) {
+                *abort_flag = 1;
+                atomicExch(status, (int)DC_ERR_TIMEOUT);
+                return false;
+            }
+        }
+    }
+}
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, uint32_t bar)
 {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+                 ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int c0, int c1, void* bar)
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar)
 {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1) : "memory");
+                 ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void umma_commit_at(uint32_t bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// n (1 to 4) MMAs of K = 16 along a chunk; descriptors as constant upper and running lower halves, astep / bstep per MMA;
+// accumulate = 0: the first one overwrites the accumulator.
+#define DC_UMMA_CHUNK(name, group)                                                                                                              \
+    __device__ __forceinline__ void name(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t a_step, uint32_t b_lo, uint32_t b_hi, uint32_t b_step, \
+                                         uint32_t idesc, uint32_t accumulate, int n)                                                            \
+    {                                                                                                                                           \
+        _Pragma("unroll") for (int k = 0; k < 4; ++k)                                                                                           \
+            if (k < n)                                                                                                                          \
+                asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %6, 0;\n\tmov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t" \
+                             "tcgen05.mma." group ".kind::f16 [%0], da, db, %5, p;\n\t}"                                                        \
+                             ::"r"(d), "r"(a_lo + k * a_step), "r"(a_hi), "r"(b_lo + k * b_step), "r"(b_hi), "r"(idesc),                        \
+                               "r"(k == 0 ? accumulate : 1u) : "memory");                                                                       \
+    }
+DC_UMMA_CHUNK(umma_chunk, "cta_group::1")
+DC_UMMA_CHUNK(umma_chunk_pair, "cta_group::2")
+#undef DC_UMMA_CHUNK
+// A ring's running slot: its barrier and its data, advanced by fixed strides and wrapped with the phase.
+struct RingPos {
+    uint32_t off, data, left, phase;      // barrier offset (8 bytes a slot), data position, slots until the wrap, phase parity
+    __device__ __forceinline__ void start(uint32_t data0, uint32_t slots) { off = 0; data = data0; left = slots; phase = 0; }
+    __device__ __forceinline__ void next(uint32_t data0, uint32_t slots, uint32_t stride)
+    {
+        off += 8; data += stride;
+        if (--left == 0) { off = 0; data = data0; left = slots; phase ^= 1u; }
+    }
+};
 
 // K-major operand tile in shared memory.  Swizzled layouts: rows of BK bf16, 8-row groups `sbo`
 // bytes apart (lbo unused, 16).  Unswizzled layout (layout_type 0): 8-row x 16-byte core matrices,
