@@ -304,14 +304,18 @@ template <> struct VecOps<__nv_bfloat16> {
 };
 
 // out = a + b (+ ReLU); with b == nullptr: out = ReLU(a) (a + 0 is exact)
+// Bound by memory.  It walks from the end: what the convolution before it wrote last is still in L2, and the convolution
+// after it starts on what this kernel wrote last.  Its operands are not read again in this frame (streaming loads), so
+// they do not push those lines out.  ResNet-50 trunk, 128 streams: 3230 -> 3130 us for the whole pass.
 template <typename T>
 __global__ void k_add_vec(const uint4* a, const uint4* b, size_t nvec, int relu, uint4* out)
 {
     dc_pdl_wait();
     dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-        const uint4 va = __ldg(a + i), vb = b ? __ldg(b + i) : make_uint4(0, 0, 0, 0);
-        out[i] = VecOps<T>::add(va, vb, relu);
+        const size_t k = nvec - 1 - i;
+        const uint4 va = __ldcs(a + k), vb = b ? __ldcs(b + k) : make_uint4(0, 0, 0, 0);
+        out[k] = VecOps<T>::add(va, vb, relu);
     }
 }
 
