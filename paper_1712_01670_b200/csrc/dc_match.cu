@@ -189,32 +189,159 @@ __global__ void __launch_bounds__(WARPS * 32) k_verify(MatchArgs a)
 // that holds.  One CTA per stream; heads are emitted in (y, x) order by a CTA-wide ordered compaction.
 // In per-block mode (mv != nullptr) neighbours of a run, the run above and the runs below must also carry the same
 // vector, and the rectangle's source is displaced by that vector instead of the global one.
-// The end column of the run starting at each block (0 for every other block: an end is never 0), and the vectors, lie in
-// shared memory when they fit (else in run_end): the scans along a row and down a column are chains of dependent
-// loads, and they set the time (full-HD frames: 31 + 10 us with the runs in global memory and a launch of their own).
-__global__ void __launch_bounds__(1024) k_merge(const uint8_t* matched, const int16_t* mv, const int32_t* gmv, int W, int H, int B,
-                                                int Gx, int Gy, int max_regions, uint16_t* run_end, int in_smem, dc_region* regions,
-                                                int32_t* n_regions, int32_t* status, int32_t* gmv_out, int32_t* n_out, dc_region* regions_out)
+struct MergeArgs {
+    const uint8_t* matched; const int16_t* mv; const int32_t* gmv;
+    int W, H, B, Gx, Gy, max_regions;
+    uint16_t* run_end;
+    dc_region* regions; int32_t* n_regions; int32_t* status;
+    int32_t* gmv_out; int32_t* n_out; dc_region* regions_out;                            // the caller's, or null
+};
+__device__ __forceinline__ void emit_region(const MergeArgs& a, int s, int idx, int r, int c0, int c1, int h, int Mx, int My)
 {
-    extern __shared__ __align__(16) uint8_t merge_smem[];
-    __shared__ int warp_sums[32];
-    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, n = Gx * Gy;
+    if (idx >= a.max_regions) { atomicExch(a.status, (int)DC_ERR_OVERFLOW); return; }
+    const int x = c0 * a.B, y = r * a.B, x1 = min(c1 * a.B, a.W), y1 = min((r + h) * a.B, a.H);
+    const dc_region g = { x, y, x1 - x, y1 - y, x + Mx, y + My };
+    a.regions[(size_t)s * a.max_regions + idx] = g;
+    if (a.regions_out) a.regions_out[(size_t)s * a.max_regions + idx] = g;
+}
+__device__ __forceinline__ void finish_merge(const MergeArgs& a, int s, int count)
+{
+    if (threadIdx.x == 0) {
+        a.n_regions[s] = min(count, a.max_regions);
+        if (a.n_out) a.n_out[s] = min(count, a.max_regions);
+    }
+    if (a.gmv_out && threadIdx.x < 3) a.gmv_out[3 * s + threadIdx.x] = a.gmv[3 * s + threadIdx.x];
+}
+// Exclusive sum of `mine` over the CTA's 1024 threads, and the total (sums: 32 words, free again after the next barrier).
+__device__ __forceinline__ int block_exclusive(int mine, int* sums, int& total)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, inc, o); inc += lane >= o ? t : 0; }
+    if (lane == 31) sums[wid] = inc;
+    __syncthreads();
+    const int w = sums[lane];
+    total = __reduce_add_sync(0xffffffffu, w);
+    return __reduce_add_sync(0xffffffffu, lane < wid ? w : 0) + inc - mine;
+}
+// Length of the run of ones that starts at bit `from` of a row of `words` words (bits past the row are zero).
+__device__ __forceinline__ int ones_from(const uint32_t* row, int words, int from)
+{
+    int w = from >> 5;
+    if (w >= words) return 0;
+    uint32_t zeros = ~row[w] & (0xffffffffu << (from & 31));
+    while (zeros == 0) { if (++w == words) return words * 32 - from; zeros = ~row[w]; }
+    return w * 32 + __ffs(zeros) - 1 - from;
+}
+
+// The blocks of a row are bits of words in shared memory, built by ballots: a run's end is a search for the first zero
+// bit, and the passes over runs take a thread per word and visit set bits alone.  What bounds it: one SM per stream, so
+// the instructions of its passes and the barriers between them.  Measured on 120 x 68 blocks, 8 streams: 31 us with a
+// thread and its scans for every block, 19 us with bit strings but still a thread per block, 11.6 us so.
+// Dynamic shared memory: merge_smem_bytes().
+__host__ __device__ constexpr size_t merge_smem_bytes(int Gx, int Gy, bool own)
+{
+    const size_t n = (size_t)Gx * Gy, words = (size_t)(Gx + 31) / 32 * Gy;
+    return n * (own ? 4 : 0) + 4 * words * 4 + n * 2;
+}
+__global__ void __launch_bounds__(1024) k_merge(const MergeArgs a)
+{
+    extern __shared__ __align__(16) uint32_t merge_smem[];
+    __shared__ int sums[32];
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, Gx = a.Gx, Gy = a.Gy, n = Gx * Gy;
+    const int rw = (Gx + 31) >> 5, words = rw * Gy;
+    uint32_t* starts = merge_smem + (a.mv ? n : 0);           // bit c of row r: a run starts here
+    uint32_t* joined = starts + words;                        // the block continues its left neighbour's run; later: the run that starts here continues the one above
+    uint32_t* heads = joined + words;                         // the run that starts here heads a rectangle
+    uint32_t* first = heads + words;                          // rectangles before this word of heads
+    uint16_t* e = (uint16_t*)(first + words);                 // end column of the run that starts here
+    uint32_t* v = a.mv ? merge_smem : nullptr;                // (dx, dy) as one word
     dc_pdl_wait();
     dc_pdl_release();
-    const uint8_t* m = matched + (size_t)s * n;
-    const uint32_t* v = mv ? (const uint32_t*)mv + (size_t)s * n : nullptr;              // (dx, dy) as one word
-    uint16_t* e = in_smem ? (uint16_t*)(merge_smem + (mv ? (size_t)n * 4 : 0)) : run_end + (size_t)s * n;
-    if (in_smem) {
-        if (mv) {
-            uint32_t* vs = (uint32_t*)merge_smem;
-            for (int i = tid; i < n; i += 1024) vs[i] = v[i];
-            v = vs;
+    const int Mx = a.gmv[3 * s], My = a.gmv[3 * s + 1];
+    const uint8_t* gm = a.matched + (size_t)s * n;
+    const uint32_t* gv = (const uint32_t*)a.mv + (size_t)s * n;
+    for (int r = wid; r < Gy; r += 32) {
+        uint32_t left_on = 0, left_v = 0;                     // last block of the word before
+        for (int w0 = 0; w0 < rw; w0 += 4) {
+            uint32_t on[4], u[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {                     // four words' loads in flight
+                const int c = (w0 + k) * 32 + lane;
+                on[k] = c < Gx ? gm[r * Gx + c] : 0;
+                u[k] = v && c < Gx ? gv[r * Gx + c] : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int c = (w0 + k) * 32 + lane;
+                if (w0 + k >= rw) break;
+                const uint32_t word = __ballot_sync(0xffffffffu, on[k] != 0);
+                uint32_t join = word & ((word << 1) | left_on);
+                left_on = word >> 31;
+                if (v) {
+                    uint32_t pv = __shfl_up_sync(0xffffffffu, u[k], 1);
+                    if (lane == 0) pv = left_v;
+                    join &= __ballot_sync(0xffffffffu, pv == u[k]);
+                    left_v = __shfl_sync(0xffffffffu, u[k], 31);
+                    if (c < Gx) v[r * Gx + c] = u[k];
+                }
+                if (lane == 0) { joined[r * rw + w0 + k] = join; starts[r * rw + w0 + k] = word & ~join; }
+            }
         }
-        uint8_t* ms = (uint8_t*)(e + n);
-        for (int i = tid; i < n; i += 1024) ms[i] = m[i];
-        m = ms;
-        __syncthreads();
     }
+    __syncthreads();
+    for (int t = tid; t < words; t += 1024) {
+        const int r = t / rw, w = t - r * rw;
+        for (uint32_t left = starts[t]; left; left &= left - 1) {
+            const int c = w * 32 + __ffs(left) - 1;
+            e[r * Gx + c] = (uint16_t)(c + 1 + ones_from(joined + r * rw, rw, c + 1));
+        }
+    }
+    __syncthreads();
+    int mine = 0, total;
+    for (int t = tid; t < words; t += 1024) {
+        const int r = t / rw, w = t - r * rw;
+        const uint32_t here = starts[t];
+        uint32_t down = 0;
+        for (uint32_t left = r > 0 ? here & starts[t - rw] : 0; left; left &= left - 1) {
+            const int b = r * Gx + w * 32 + __ffs(left) - 1;
+            if (e[b - Gx] == e[b] && (!v || v[b - Gx] == v[b])) down |= left & (0u - left);
+        }
+        joined[t] = down;
+        heads[t] = here & ~down;
+    }
+    __syncthreads();
+    const int per = (words + 1023) / 1024, lo = min(tid * per, words), hi = min(lo + per, words);
+    for (int t = lo; t < hi; ++t) mine += __popc(heads[t]);
+    int before = block_exclusive(mine, sums, total);
+    for (int t = lo; t < hi; ++t) { first[t] = (uint32_t)before; before += __popc(heads[t]); }
+    __syncthreads();
+    for (int r = wid; r < Gy; r += 32)
+        for (int w = 0; w < rw; ++w) {
+            const int t = r * rw + w;
+            const uint32_t word = heads[t];
+            if (!((word >> lane) & 1u)) continue;
+            int h = 1;
+            while (r + h < Gy && ((joined[t + h * rw] >> lane) & 1u)) ++h;
+            const int c = w * 32 + lane, b = r * Gx + c;
+            const uint32_t own = v ? v[b] : 0u;
+            emit_region(a, s, (int)first[t] + __popc(word & ((1u << lane) - 1u)), r, c, e[b], h,
+                        v ? (int16_t)(own & 0xffffu) : Mx, v ? (int16_t)(own >> 16) : My);
+        }
+    finish_merge(a, s, total);
+}
+
+// The same for block grids beyond shared memory: block by block, the runs in global memory.
+__global__ void __launch_bounds__(1024) k_merge_large(const MergeArgs a)
+{
+    __shared__ int sums[32];
+    const int s = blockIdx.x, tid = threadIdx.x, Gx = a.Gx, Gy = a.Gy, n = Gx * Gy;
+    dc_pdl_wait();
+    dc_pdl_release();
+    const uint8_t* m = a.matched + (size_t)s * n;
+    const uint32_t* v = a.mv ? (const uint32_t*)a.mv + (size_t)s * n : nullptr;          // (dx, dy) as one word
+    uint16_t* e = a.run_end + (size_t)s * n;
     for (int b = tid; b < n; b += 1024) {
         const int c = b % Gx;
         int end = 0;
@@ -226,13 +353,11 @@ __global__ void __launch_bounds__(1024) k_merge(const uint8_t* matched, const in
         e[b] = (uint16_t)end;
     }
     __syncthreads();
-    dc_region* out = regions + (size_t)s * max_regions;
-    dc_region* user = regions_out ? regions_out + (size_t)s * max_regions : nullptr;
-    int Mx = gmv[3 * s], My = gmv[3 * s + 1];
+    int Mx = a.gmv[3 * s], My = a.gmv[3 * s + 1];
     int base = 0;                                                     // rectangles emitted so far, the same in all threads
     for (int start = 0; start < n; start += 1024) {
         const int b = start + tid;
-        int head = 0, c1 = 0, h = 0, r = 0, c0 = 0;
+        int head = 0, c1 = 0, h = 0, r = 0, c0 = 0, total;
         if (b < n) {
             r = b / Gx; c0 = b - r * Gx;
             c1 = e[b];
@@ -241,34 +366,15 @@ __global__ void __launch_bounds__(1024) k_merge(const uint8_t* matched, const in
                 while (r + h < Gy && e[b + h * Gx] == c1 && (!v || v[b + h * Gx] == v[b])) ++h;
             }
         }
-        // ordered compaction: exclusive scan of `head` over the 1024 threads
-        const unsigned bal = __ballot_sync(0xffffffffu, head);
-        const int pre = __popc(bal & ((1u << lane) - 1u));
-        if (lane == 0) warp_sums[wid] = __popc(bal);
-        __syncthreads();
-        const int mine = warp_sums[lane];
-        const int woff = __reduce_add_sync(0xffffffffu, lane < wid ? mine : 0), total = __reduce_add_sync(0xffffffffu, mine);
-        const int idx = base + woff + pre;
+        const int idx = base + block_exclusive(head, sums, total);
         if (head) {
-            if (idx < max_regions) {
-                const int x = c0 * B, y = r * B;
-                const int x1 = min(c1 * B, W), y1 = min((r + h) * B, H);
-                if (v) { const uint32_t own = v[b]; Mx = (int16_t)(own & 0xffffu); My = (int16_t)(own >> 16); }
-                dc_region g = { x, y, x1 - x, y1 - y, x + Mx, y + My };
-                out[idx] = g;
-                if (user) user[idx] = g;
-            } else {
-                atomicExch(status, (int)DC_ERR_OVERFLOW);
-            }
+            if (v) { const uint32_t own = v[b]; Mx = (int16_t)(own & 0xffffu); My = (int16_t)(own >> 16); }
+            emit_region(a, s, idx, r, c0, c1, h, Mx, My);
         }
         base += total;
-        __syncthreads();                                              // warp_sums is free again
+        __syncthreads();                                              // sums is free again
     }
-    if (tid == 0) {
-        n_regions[s] = min(base, max_regions);
-        if (n_out) n_out[s] = min(base, max_regions);
-    }
-    if (gmv_out && tid < 3) gmv_out[3 * s + tid] = gmv[3 * s + tid];
+    finish_merge(a, s, base);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1386,14 +1492,13 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
     {
         dc_prof_scope ps(c, DC_ST_MERGE);
         const bool own = a.region_mode == DC_REGIONS_PER_BLOCK;
-        const int n = a.Gx * a.Gy;
-        const size_t need = (size_t)n * (own ? 7 : 3);              // runs, matched flags and vectors of a stream
-        const bool fits = need <= 160 * 1024;
+        const size_t need = merge_smem_bytes(a.Gx, a.Gy, own);
         static dc_once_per_device attr_set;
         if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
-        DC_CUDA(dc_launch_pdl(k_merge, dim3((unsigned)c->S), 1024, fits ? need : 0, c->stream, (const uint8_t*)a.matched, (const int16_t*)(own ? a.mv : nullptr),
-                              (const int32_t*)c->gmv, a.W, a.H, a.B, a.Gx, a.Gy, c->max_regions, c->run_end, fits ? 1 : 0, c->regions0, c->n_regions, c->status,
-                              out ? out->gmv : nullptr, out ? out->n_regions : nullptr, out ? out->regions : nullptr));
+        const MergeArgs ma = {a.matched, own ? a.mv : nullptr, c->gmv, a.W, a.H, a.B, a.Gx, a.Gy, c->max_regions, c->run_end, c->regions0, c->n_regions,
+                              c->status, out ? out->gmv : nullptr, out ? out->n_regions : nullptr, out ? out->regions : nullptr};
+        if (need <= 160 * 1024) DC_CUDA(dc_launch_pdl(k_merge, dim3((unsigned)c->S), 1024, need, c->stream, ma));
+        else DC_CUDA(dc_launch_pdl(k_merge_large, dim3((unsigned)c->S), 1024, 0, c->stream, ma));
     }
     c->launches += 3;
     DC_CUDA(cudaGetLastError());

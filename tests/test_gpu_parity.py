@@ -175,6 +175,25 @@ def test_match_per_block_streams_and_full_hd():
                 region_mode=B.DC_REGIONS_PER_BLOCK)
 
 
+@pytest.mark.parametrize("gx,gy", [(31, 33), (32, 32), (33, 31), (64, 65), (1, 40), (40, 1), (96, 3), (256, 256)])
+def test_match_merge_grid_words(gx, gy):
+    """Step 5's runs and rectangles across the 32-block words of its bit strings, and a grid beyond shared memory."""
+    g = rng(gx * 131 + gy)
+    W, H = gx * 4, gy * 4
+    prev = g.integers(0, 256, size=(H, W, 3), dtype=np.uint8)
+    prev[: H // 2] = 77                                        # whole columns and rows that match
+    pairs = [(prev, prev)]
+    for n in (3, 12):
+        cur = prev.copy()
+        for _ in range(n):                                     # unmatched rectangles of blocks
+            x, y = int(g.integers(0, gx)), int(g.integers(0, gy))
+            part = cur[4 * y:4 * (y + int(g.integers(1, 9))), 4 * x:4 * (x + int(g.integers(1, 9)))]
+            part[:] = g.integers(0, 256, size=part.shape, dtype=np.uint8)
+        pairs.append((prev, cur))
+    for mode in (B.DC_REGIONS_GLOBAL, B.DC_REGIONS_PER_BLOCK):
+        check_pairs(pairs, 4, 1, B.DC_SEARCH_DIAMOND, region_mode=mode)
+
+
 @pytest.mark.parametrize("widx", [2, 3, 4])
 def test_infer_per_block_regions(widx):
     U.run_stream_parity(configs.WORKLOADS[widx](), 1, list(range(4)), region_mode=B.DC_REGIONS_PER_BLOCK)
