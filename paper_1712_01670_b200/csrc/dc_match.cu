@@ -8,7 +8,7 @@
 //              bank conflicts and of byte realignment; points already scored by the previous diamond are
 //              skipped (they cannot win).  Walks that leave the window continue in k_search_dsw_long with
 //              private windows.
-//   k_search_tss16q  Step 2 for 16-pixel blocks with three step search: the same lane layout, one window that
+//   k_search_tss16  Step 2 for 16-pixel blocks with three step search: the same lane layout, one window that
 //              covers the whole reach of the search.
 //   k_verify   Steps 3-4: rounds the mean vector M, scores every block at M (reusing the Step 2
 //              score when the block's own best vector is M); k_verify16_prep / k_verify16_list for 16-pixel blocks.
@@ -496,15 +496,6 @@ constexpr unsigned long long pack_moves(int first)
 }
 constexpr unsigned long long kMovesLo = pack_moves(0), kMovesHi = pack_moves(8);
 
-// st: 0 walking, 1 finished, 2 the walk left the staged window (resume elsewhere), 3 no block
-struct WalkState { int cx, cy, phase, st; uint32_t mask, bs, bt; };
-
-__device__ __forceinline__ void walk_begin(WalkState& w, bool on)
-{
-    w.cx = 0; w.cy = 0; w.phase = 0; w.st = on ? 0 : 3;
-    w.mask = on ? 0x1ffu : 0u;                                    // the centre (0, 0) and its large diamond
-    w.bs = 0xffffffffu; w.bt = 0xffffffffu;
-}
 // points of the large diamond around a new centre that the diamond around the old one did not contain:
 // the others lost to the new centre already and cannot win (mx, my: the move, one of the 8 diamond offsets)
 __device__ __forceinline__ uint32_t new_points(int mx, int my)
@@ -843,133 +834,150 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
 }
 
 // ---------------------------------------------------------------------------------------------
-// Step 2 for 16-pixel blocks, three step search (Section 7.5), several blocks per warp
+// Step 2 for 16-pixel blocks, three step search (Section 7.5): one warp per block
 // ---------------------------------------------------------------------------------------------
-// Same lane layout as the diamond kernel.  Every block scores the same number of points (the centre, then
-// eight per step), so the blocks of a warp stay in step without loss.  WalkState: phase = current step size,
-// mask = points of the 3 x 3 grid still to score (bit 4 = its centre).
-template <int LPB, typename Win>
-__device__ __forceinline__ void lockstep_tss(const MatchArgs& a, const RowCtx<16 / LPB>& rc, const Win& win, int q,
-                                             int dx_lo, unsigned dx_span, int dy_lo, unsigned dy_span, WalkState& w)
+// Layout of the diamond kernel: one word per pixel, lane 2 r + h scores every other pixel of block row r, no bank
+// conflicts.  The window reaches `side` pixels (2 S0 - 1, rounded up to four) to the left and right and wr = 2 S0 - 1
+// rows up and down, so every point of the search is staged.  A step scores its eight points in two batches of four,
+// 32 loads in flight each, and decides by SSE alone; when two of the scores that matter are equal the exact order
+// (SSE, |dx| + |dy|, dy, dx) picks from the same scores.
+// What bounds it: issue slots - 8 loads, 8 differences, 8 multiply-adds and a warp sum per point and block.  Measured
+// on 8 full-HD frames, range 16: 140 us with 4 lanes per block and byte-aligned rows (a bank conflict and a realignment
+// per word), 126 us so.
+constexpr int TSS_VS = 2;
+struct TssShape { int s0, wr, side, pitch; };
+static TssShape tss_shape(int R)
 {
-    constexpr int NR = 16 / LPB;
-#pragma unroll 1
-    for (int pass = 0; pass < 9 * 8; ++pass) {                   // at most 1 + 8 * log2(2 S0) points, S0 <= 64
-        if (w.st == 0 && w.mask == 0) {
-            w.phase >>= 1;                                        // next, halved step around the best point so far
-            if (w.phase == 0) w.st = 1;
-            else { w.cx = (int)(w.bt & 0xff) - 128; w.cy = (int)((w.bt >> 8) & 0xff) - 128; w.mask = 0x1efu; }
-        }
-        if (!__any_sync(0xffffffffu, w.st == 0)) break;
-        const bool run = w.st == 0;
-        const int i = run ? __ffs(w.mask) - 1 : 4;
-        w.mask &= w.mask - 1;
-        const int dx = w.cx + (i % 3 - 1) * w.phase, dy = w.cy + (i / 3 - 1) * w.phase;
-        const bool ok = run && (unsigned)(dx - dx_lo) <= dx_span && (unsigned)(dy - dy_lo) <= dy_span;
-        uint32_t ks = 0;
-        if (ok) {
-            uint32_t sh;
+    TssShape t;
+    t.s0 = R < 1 ? 0 : 1;                                       // first step: the largest power of two with 2 S0 - 1 <= R
+    while (t.s0 > 0 && 4 * t.s0 - 1 <= R) t.s0 *= 2;
+    t.wr = t.s0 > 0 ? 2 * t.s0 - 1 : 0;
+    t.side = (t.wr + 3) & ~3;
+    t.pitch = 128 + 2 * t.side + 2;                             // 2 modulo 4: conflict-free
+    return t;
+}
+static size_t tss_window_bytes(const TssShape& t) { return (size_t)(16 * TSS_VS + 2 * t.wr) * t.pitch * sizeof(uint32_t); }
+
+// SSE of N candidates over this lane's pixels, summed over the warp (n_px: the lane's pixels inside the frame)
+template <bool CLIP, int N>
+__device__ __forceinline__ void score_n(const uint32_t (&p)[N], const uint32_t (&cw)[8], bool row_on, int n_px, uint32_t* out)
+{
+    uint32_t w[N][8];
 #pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                const uint32_t* p = win.row(q + k * LPB, dx, dy, sh);
-                const uint32_t v = rc.template sse<false>(k, p, sh);
-                ks += rc.row_on[k] ? v : 0u;
-            }
-        }
+    for (int k = 0; k < N; ++k) {
+        w[k][0] = lds_at<0>(p[k]); w[k][1] = lds_at<8>(p[k]); w[k][2] = lds_at<16>(p[k]); w[k][3] = lds_at<24>(p[k]);
+        w[k][4] = lds_at<32>(p[k]); w[k][5] = lds_at<40>(p[k]); w[k][6] = lds_at<48>(p[k]); w[k][7] = lds_at<56>(p[k]);
+    }
 #pragma unroll
-        for (int off = LPB / 2; off > 0; off >>= 1) ks += __shfl_xor_sync(0xffffffffu, ks, off);
-        const uint32_t kt = ((uint32_t)(abs(dx) + abs(dy)) << 16) | ((uint32_t)(dy + 128) << 8) | (uint32_t)(dx + 128);
-        if (ok && (ks < w.bs || (ks == w.bs && kt < w.bt))) { w.bs = ks; w.bt = kt; }
+    for (int k = 0; k < N; ++k) {
+        uint32_t a0 = 0, a1 = 0;
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+            uint32_t d = !CLIP || j < n_px ? __vabsdiffu4(cw[j], w[k][j]) : 0u; a0 = __dp4a(d, d, a0);
+            d = !CLIP || j + 1 < n_px ? __vabsdiffu4(cw[j + 1], w[k][j + 1]) : 0u; a1 = __dp4a(d, d, a1);
+        }
+        out[k] = __reduce_add_sync(0xffffffffu, row_on ? a0 + a1 : 0u);
     }
 }
 
-// Window of a CTA's 8 x VS blocks whose reach is known at launch only (three step search: 2 S0 - 1 pixels).
-struct StackWinR {
-    const uint32_t* win; int x0, wx0, row0, wr, pitch;
-    __device__ __forceinline__ const uint32_t* row(int r, int dx, int dy, uint32_t& sh) const
-    {
-        const int off = (x0 + dx) * 3 - wx0;
-        sh = (off & 3) * 8;
-        return win + (row0 + r + dy + wr) * pitch + (off >> 2);
+// Lane g < 9 settles point g of the 3 x 3 grid (4: its centre, the best so far): its displacement, validity and tie key
+// are computed once per step and not point by point.
+template <bool CLIP>
+__device__ __forceinline__ void tss_walk(uint32_t lane_base, int pitch, int s0, const uint32_t (&cw)[8], bool row_on, int n_px,
+                                         const WalkBounds& wb, int& cx, int& cy, uint32_t& bs)
+{
+    const int lane = threadIdx.x & 31, gx = lane % 3 - 1, gy = lane / 3 - 1;
+    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4, centre = lane == 4;
+    {   // the zero vector
+        const uint32_t p[1] = {lane_base};
+        score_n<CLIP, 1>(p, cw, row_on, n_px, &bs);
     }
-};
+    cx = cy = 0;
+    uint32_t pc = lane_base;
+#pragma unroll 1
+    for (int step = s0; step > 0; step >>= 1) {
+        const uint32_t ox = (uint32_t)step * 4u, oy = (uint32_t)(step * pitch) * 4u;
+        uint32_t sc[8];
+        const uint32_t up[4] = {pc - oy - ox, pc - oy, pc - oy + ox, pc - ox}, dn[4] = {pc + ox, pc + oy - ox, pc + oy, pc + oy + ox};
+        score_n<CLIP, 4>(up, cw, row_on, n_px, sc);
+        score_n<CLIP, 4>(dn, cw, row_on, n_px, sc + 4);
+        // sc[0..3]: points 0 to 3, sc[4..7]: points 5 to 8
+        const uint32_t q0 = b0 ? sc[1] : sc[0], q1 = b0 ? sc[3] : sc[2], q2 = b0 ? sc[4] : bs, q3 = b0 ? sc[6] : sc[5];
+        uint32_t mine = b2 ? (b1 ? q3 : q2) : (b1 ? q1 : q0);
+        if (lane == 8) mine = sc[7];
+        const int dx = cx + gx * step, dy = cy + gy * step;
+        if (lane > 8 || (!centre && (dx < wb.dx_lo || dx > wb.dx_hi || dy < wb.dy_lo || dy > wb.dy_hi))) mine = 0xffffffffu;
+        bs = __reduce_min_sync(0xffffffffu, mine);
+        unsigned best = __ballot_sync(0xffffffffu, mine == bs);
+        if (best & (best - 1)) {                                  // equal scores: the exact order among them
+            const uint32_t kt = tie_key(dx, dy), kb = __reduce_min_sync(0xffffffffu, mine == bs ? kt : 0xffffffffu);
+            best = __ballot_sync(0xffffffffu, mine == bs && kt == kb);
+        }
+        const int g = __ffs(best) - 1, my = g / 3 - 1, mx = g - 3 * (my + 1) - 1;
+        cx += mx * step; cy += my * step;
+        pc += (uint32_t)((my * pitch + mx) * step * 4);
+    }
+}
 
-// One CTA per 8 x VS blocks; the window (dynamic shared memory) reaches wr = 2 S0 - 1 pixels around the tile, which
-// covers every point the search can visit.  Blocks clipped in width are left to the generic kernel.
-template <int LPB, int VS>
-__global__ void __launch_bounds__(LPB * 8 * VS) k_search_tss16q(MatchArgs a, int s0, int wr, int words, int pitch)
+__global__ void __launch_bounds__(TSS_VS * 8 * 32, 2) k_search_tss16(MatchArgs a, TssShape t)
 {
     dc_pdl_wait();
     dc_pdl_release();
-    extern __shared__ uint32_t tss_win[];
-    constexpr int THREADS = LPB * 8 * VS;
-    const int rows = 16 * VS + 2 * wr, cpr = words / 4, chunks = rows * cpr;
-    const int strips = (a.Gx + 7) >> 3, vgroups = (a.Gy + VS - 1) / VS;
-    const int strip = blockIdx.x % strips, vg = (blockIdx.x / strips) % vgroups, s = blockIdx.x / (strips * vgroups);
-    const int xs = strip * 128, yb = vg * 16 * VS;
-    const int wx0 = ((xs - wr) * 3) & ~15;                    // byte column of the window origin (may be < 0)
-    const int lane = threadIdx.x & 31, q = lane % LPB;
-    const int blk = threadIdx.x / LPB, by = vg * VS + (blk >> 3), bx = strip * 8 + (blk & 7);
-    const bool in_grid = bx < a.Gx && by < a.Gy;
+    extern __shared__ __align__(16) uint32_t tss_win[];
+    __shared__ int32_t sums[3];
+    constexpr int THREADS = TSS_VS * 8 * 32;
+    const int strip = blockIdx.x, vg = blockIdx.y, s = blockIdx.z;
+    const int xs = strip * 128, yb = vg * 16 * TSS_VS;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
+    const int by = vg * TSS_VS + (warp >> 3), bx = strip * 8 + (warp & 7);
     const int x0 = bx * 16, y0 = by * 16;
-    const bool searched = in_grid && a.W - x0 >= 16;
-    const int bw = searched ? 16 : 0, bh = searched ? min(16, a.H - y0) : 0;
-    RowCtx<16 / LPB> rc;                                      // issued first: in flight while the window is staged
-    rc.load_block(a.cur + (size_t)s * a.cur_stream + (size_t)(searched ? y0 : 0) * a.cur_pitch + (size_t)(searched ? x0 : 0) * 3,
-                  a.cur_pitch, q, LPB, bw, bh);
+    const bool searched = bx < a.Gx && by < a.Gy;
+    const int bh = searched ? min(16, a.H - y0) : 0, bw = min(16, a.W - x0);
+    const bool row_on = r < bh;
+    uint32_t cw[8];                                            // issued first: in flight while the window is staged
+    load_lane_pixels(a.cur + (size_t)s * a.cur_stream + (size_t)(row_on ? y0 + r : 0) * a.cur_pitch + (size_t)(row_on ? x0 : 0) * 3,
+                     h, row_on, cw);
+    if (threadIdx.x < 3) sums[threadIdx.x] = 0;
     const uint8_t* prev = a.prev + (size_t)s * a.prev_stream;
-    constexpr int UNR = 4;                                    // 16-byte chunks; wx0 and the pitch are 16-byte multiples
-    for (int i0 = threadIdx.x; i0 < chunks; i0 += THREADS * UNR) {
-        uint4 v[UNR];
+    // groups of 4 pixels, five in flight per thread; a thread's next group is THREADS further: rows and columns by addition
+    const int groups = (128 + 2 * t.side) / 4, rows = 16 * TSS_VS + 2 * t.wr, row_add = THREADS / groups, col_add = THREADS - row_add * groups;
+    constexpr int UNR = 5;
+    for (int row = threadIdx.x / groups, gq = threadIdx.x - row * groups; row < rows;) {
+        uint32_t pa[UNR], pb[UNR], pc[UNR];
+        uint32_t* dst[UNR];
 #pragma unroll
         for (int u = 0; u < UNR; ++u) {
-            const int i = i0 + u * THREADS, row = i / cpr, ci = i - row * cpr;
-            const int gy = yb - wr + row, gb = wx0 + ci * 16;
-            v[u] = make_uint4(0, 0, 0, 0);
-            if (i < chunks && gy >= 0 && gy < a.H && gb >= 0 && gb + 16 <= (int)a.prev_pitch)
-                v[u] = __ldg((const uint4*)(prev + (size_t)gy * a.prev_pitch + gb));
+            load_pixels4(prev, a.prev_pitch, a.H, yb - t.wr + row, xs - t.side + 4 * gq, pa[u], pb[u], pc[u]);
+            dst[u] = row < rows ? tss_win + row * t.pitch + 4 * gq : nullptr;
+            row += row_add; gq += col_add;
+            if (gq >= groups) { gq -= groups; ++row; }
         }
 #pragma unroll
-        for (int u = 0; u < UNR; ++u) {
-            const int i = i0 + u * THREADS, row = i / cpr, ci = i - row * cpr;
-            if (i < chunks) {
-                uint32_t* d = tss_win + row * pitch + ci * 4;
-                d[0] = v[u].x; d[1] = v[u].y; d[2] = v[u].z; d[3] = v[u].w;
+        for (int u = 0; u < UNR; ++u)
+            if (dst[u]) store_pixels4(dst[u], pa[u], pb[u], pc[u]);
+    }
+    __syncthreads();
+    if (searched) {
+        const size_t g = (size_t)s * a.Gx * a.Gy + (size_t)by * a.Gx + bx;
+        const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
+        const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(tss_win) +
+                                   (uint32_t)((((warp >> 3) * 16 + r + t.wr) * t.pitch + (x0 - xs + t.side) + h) * 4);
+        int cx, cy; uint32_t bs;
+        if (bw == 16) tss_walk<false>(lane_base, t.pitch, t.s0, cw, row_on, 8, wb, cx, cy, bs);
+        else tss_walk<true>(lane_base, t.pitch, t.s0, cw, row_on, lane_pixel_count(bw, h), wb, cx, cy, bs);
+        if (lane == 0) {
+            a.mv[2 * g] = (int16_t)cx; a.mv[2 * g + 1] = (int16_t)cy; a.sse[g] = bs;
+            if (bs <= a.limit[limit_index(a, bw, bh)]) {          // PSNR > T: member of Step 3's set S
+                atomicAdd(&sums[0], cx); atomicAdd(&sums[1], cy); atomicAdd(&sums[2], 1);
             }
         }
     }
     __syncthreads();
-    const size_t g = (size_t)s * a.Gx * a.Gy + (size_t)by * a.Gx + bx;
-    const int dx_lo = max(-a.R, -x0), dy_lo = max(-a.R, -y0);
-    const unsigned dx_span = (unsigned)(min(a.R, a.W - bw - x0) - dx_lo), dy_span = (unsigned)(min(a.R, a.H - bh - y0) - dy_lo);
-    const StackWinR sw = {tss_win, x0, wx0, (blk >> 3) * 16, wr, pitch};
-    WalkState w;
-    walk_begin(w, searched);
-    w.phase = s0;                                             // first pass: the centre and its eight neighbours at step S0
-    if (searched && s0 == 0) w.mask = 0x010u;                 // range 0: the zero vector alone
-    lockstep_tss<LPB>(a, rc, sw, q, dx_lo, dx_span, dy_lo, dy_span, w);
-    const int fx = (int)(w.bt & 0xff) - 128, fy = (int)((w.bt >> 8) & 0xff) - 128;
-    const bool fin = searched && q == 0;
-    if (fin) { a.mv[2 * g] = (int16_t)fx; a.mv[2 * g + 1] = (int16_t)fy; a.sse[g] = w.bs; }
-    const bool pass = fin && w.bs <= a.limit[limit_index(a, bw, bh)];     // PSNR > T: member of Step 3's set S
-    const int n_pass = __popc(__ballot_sync(0xffffffffu, pass));
-    const int sum_x = __reduce_add_sync(0xffffffffu, pass ? fx : 0), sum_y = __reduce_add_sync(0xffffffffu, pass ? fy : 0);
-    if (lane == 0 && n_pass) {
-        atomicAdd(&a.acc[4 * s + 0], sum_x);
-        atomicAdd(&a.acc[4 * s + 1], sum_y);
-        atomicAdd(&a.acc[4 * s + 2], n_pass);
+    if (threadIdx.x == 0 && sums[2]) {                            // Step 3's sums once per CTA (one stream per CTA)
+        atomicAdd(&a.acc[4 * s + 0], sums[0]);
+        atomicAdd(&a.acc[4 * s + 1], sums[1]);
+        atomicAdd(&a.acc[4 * s + 2], sums[2]);
     }
-}
-
-constexpr int TSS_LPB = 4, TSS_VS = 4;
-// shared memory of one k_search_tss16q CTA for search range R
-static size_t tss_window_bytes(int R)
-{
-    int s0 = R < 1 ? 0 : 1;
-    while (s0 > 0 && 4 * s0 - 1 <= R) s0 *= 2;
-    const int wr = s0 > 0 ? 2 * s0 - 1 : 1;
-    const int words = ((((112 + 2 * wr) * 3 + 15) >> 2) + 13 + 3) & ~3;
-    return (size_t)(16 * TSS_VS + 2 * wr) * (words | 1) * sizeof(uint32_t);
 }
 
 // Section 4, k-skip: blocks that are not searched report vector (0, 0) and SSE 2^32 - 1.  One thread per block.
@@ -1437,25 +1445,13 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
             }
             c->launches += 1;
         }
-    } else if (a.B == 16 && a.search == DC_SEARCH_THREE_STEP && a.skip_k <= 1 && tss_window_bytes(a.R) <= 160 * 1024) {
-        int s0 = a.R < 1 ? 0 : 1;                                   // first step: the largest power of two with 2 S0 - 1 <= R
-        while (s0 > 0 && 4 * s0 - 1 <= a.R) s0 *= 2;
-        const int wr = s0 > 0 ? 2 * s0 - 1 : 1;
-        const int words = ((((112 + 2 * wr) * 3 + 15) >> 2) + 13 + 3) & ~3, pitch = words | 1;
-        const size_t smem = tss_window_bytes(a.R);
+    } else if (a.B == 16 && a.search == DC_SEARCH_THREE_STEP && a.skip_k <= 1) {
+        const TssShape t = tss_shape(a.R);
         static dc_once_per_device attr_set;
-        if (attr_set.first(c->device)) {
-            DC_CUDA(cudaFuncSetAttribute(k_search_tss16q<TSS_LPB, TSS_VS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
-        }
-        {
-            dc_prof_scope ps(c, DC_ST_SEARCH);
-            const int ctas = ((a.Gx + 7) / 8) * ((a.Gy + TSS_VS - 1) / TSS_VS) * a.S;
-            DC_CUDA(dc_launch_pdl(k_search_tss16q<TSS_LPB, TSS_VS>, dim3((unsigned)ctas), TSS_LPB * 8 * TSS_VS, smem, c->stream, a, s0, wr, words, pitch));
-        }
-        if (a.W % 16 != 0) {                                        // blocks clipped by the right edge
-            const int rc = search_win(c, a, 2);
-            if (rc != DC_OK) return rc;
-        }
+        if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_search_tss16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tss_window_bytes(tss_shape(64))));
+        dc_prof_scope ps(c, DC_ST_SEARCH);
+        DC_CUDA(dc_launch_pdl(k_search_tss16, dim3((unsigned)((a.Gx + 7) / 8), (unsigned)((a.Gy + TSS_VS - 1) / TSS_VS), (unsigned)a.S), TSS_VS * 8 * 32,
+                              tss_window_bytes(t), c->stream, a, t));
     } else if (a.B == 16 && a.search == DC_SEARCH_EXHAUSTIVE && a.R <= E_MAXR && a.W >= 16 && a.H >= 16) {
         const int chunks = (2 * a.R + 1 + E_DY - 1) / E_DY;
         const size_t smem = ((size_t)(16 + chunks * E_DY - 1) * E_PITCH + 8 * 192) * sizeof(uint32_t);

@@ -47,7 +47,7 @@ __device__ __forceinline__ Tile tile_of(const dc_win_args& a)
     Tile t;
     const int tx = blockIdx.x % a.tiles_x, u = blockIdx.x / a.tiles_x;
     t.s = u / a.tiles_y;
-    t.bx0 = a.bx_first + tx * a.TX; t.by0 = (u - t.s * a.tiles_y) * a.TY;
+    t.bx0 = tx * a.TX; t.by0 = (u - t.s * a.tiles_y) * a.TY;
     t.nbx = min(a.TX, a.Gx - t.bx0); t.nby = min(a.TY, a.Gy - t.by0);
     return t;
 }
@@ -58,13 +58,13 @@ __device__ __forceinline__ bool searched(const dc_win_args& a, int bx, int by)
 // blocks this launch is about: all, or those that the frame's edge clips
 __device__ __forceinline__ bool mine(const dc_win_args& a, int bx, int by)
 {
-    return a.only_clipped == 0 || a.W - bx * a.B < a.B || (a.only_clipped == 1 && a.H - by * a.B < a.B);
+    return a.only_clipped == 0 || a.W - bx * a.B < a.B || a.H - by * a.B < a.B;
 }
 
 __device__ __forceinline__ bool any_mine(const dc_win_args& a, const Tile& t)
 {
     const bool right = t.bx0 + t.nbx == a.Gx && a.W % a.B != 0, bottom = t.by0 + t.nby == a.Gy && a.H % a.B != 0;
-    return a.only_clipped == 0 || right || (a.only_clipped == 1 && bottom);
+    return a.only_clipped == 0 || right || bottom;
 }
 
 // The window, rows warp by warp, a lane four pixels: the 12 bytes come as four aligned words, whatever the row's
@@ -476,13 +476,10 @@ int launch(K kernel, const dc_win_args& a, int threads, size_t smem, int device,
 int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t stream)
 {
     const bool all = a.search == DC_SEARCH_EXHAUSTIVE;
-    // clipped in width: the last block column alone
-    a.bx_first = a.only_clipped == 2 ? a.Gx - 1 : 0;
-    const int nx = a.Gx - a.bx_first;
     size_t smem = 0;
     auto shape = [&](int TX, int TY) {
         a.TX = TX; a.TY = TY;
-        a.tiles_x = dc_div_up(nx, TX); a.tiles_y = dc_div_up(a.Gy, TY);
+        a.tiles_x = dc_div_up(a.Gx, TX); a.tiles_y = dc_div_up(a.Gy, TY);
         a.win_cols = (TX * a.B + 2 * a.R + 3) & ~3;                   // staged in groups of four
         a.win_rows = TY * a.B + 2 * a.R + (all ? E_ROWS - 1 : 0);     // rows only touched by displacements beyond R (scored, never compared)
         a.win_pitch = a.win_cols + ((a.B - a.win_cols) % 32 + 32) % 32;   // = B modulo 32
@@ -490,7 +487,7 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     };
     // Wide tiles stage fewer window pixels per block; they shrink while the window is too large for three CTAs per SM, and
     // while the frames have fewer tiles than the machine has SMs (down to two blocks, one for the exhaustive search).
-    int TX = nx < 8 ? nx : 8, TY = TX < 4 ? 4 : 2;
+    int TX = a.Gx < 8 ? a.Gx : 8, TY = TX < 4 ? 4 : 2;
     if (TY > a.Gy) TY = a.Gy;
     shape(TX, TY);
     while (TX * TY > 1 && (smem > 200 * 1024 || (TX * TY > 2 && smem > 72 * 1024) ||

@@ -7,12 +7,12 @@ struct dc_win_args {
     const uint8_t* cur; const uint8_t* cur_end; size_t cur_pitch, cur_stream;
     const uint8_t* prev; const uint8_t* prev_end; size_t prev_pitch, prev_stream;
     int W, H, B, R, Gx, Gy, S, search, skip_k;
-    int only_clipped;                    // 0: every block; 1: blocks clipped by the frame's edge; 2: blocks clipped in width
+    int only_clipped;                    // 0: every block; 1: blocks clipped by the frame's edge
     uint32_t limit[4];                   // PSNR test as an SSE bound, index = 2 * (clipped in height) + (clipped in width)
     int16_t* mv; uint32_t* sse; int32_t* acc;   // acc: [S][4], zeroed: sums of Step 3
     int32_t* status;                     // device status word, or NULL
     // set by dc_launch_search_win
-    int bx_first, TX, TY, tiles_x, tiles_y, win_rows, win_cols, win_pitch;
+    int TX, TY, tiles_x, tiles_y, win_rows, win_cols, win_pitch;
 };
 
 // Enqueues the search; fails only with DC_ERR_CUDA.

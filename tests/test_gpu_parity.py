@@ -194,6 +194,19 @@ def test_match_merge_grid_words(gx, gy):
         check_pairs(pairs, 4, 1, B.DC_SEARCH_DIAMOND, region_mode=mode)
 
 
+@pytest.mark.parametrize("R", [0, 1, 2, 3, 7, 15, 63, 64])
+@pytest.mark.parametrize("shape", [(16, 16), (33, 129), (47, 143), (100, 260)])
+def test_match_three_step_16_windows(R, shape):
+    """The staged three step search: every first step, strips and blocks clipped on either side, ties."""
+    g = rng(R * 37 + shape[1])
+    H, W = shape
+    prev = g.integers(0, 256, size=(H, W, 3), dtype=np.uint8)
+    far = np.roll(prev, (-min(R, H // 3), min(R, W // 3)), axis=(0, 1))
+    const = np.full_like(prev, 50)
+    smooth = np.repeat((np.arange(W) // 4 % 3 * 40).astype(np.uint8)[None, :, None], H, 0).repeat(3, 2)
+    check_pairs([(prev, far), (const, const), (smooth, np.roll(smooth, 2, axis=1)), (prev, smooth)], 16, R, B.DC_SEARCH_THREE_STEP)
+
+
 @pytest.mark.parametrize("widx", [2, 3, 4])
 def test_infer_per_block_regions(widx):
     U.run_stream_parity(configs.WORKLOADS[widx](), 1, list(range(4)), region_mode=B.DC_REGIONS_PER_BLOCK)
