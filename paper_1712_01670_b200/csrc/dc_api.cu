@@ -346,6 +346,7 @@ int dc_cache_create(const dc_config* cfg, const dc_layer_desc* layers, int n_lay
     dc_cache* c = new (std::nothrow) dc_cache();
     if (!c) return DC_ERR_ALLOC;
     memset((void*)c, 0, sizeof(*c));
+    c->list_mark = DC_LISTS_FRESH;
     c->cfg = *cfg; c->n_layers = n_layers; c->stream = (cudaStream_t)cuda_stream;
     c->S = cfg->n_streams;
     c->Gx = dc_div_up(cfg->width, cfg->block); c->Gy = dc_div_up(cfg->height, cfg->block);
@@ -493,6 +494,7 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             if (dc_layer_cached(c, i)) { if (cur < 0) cur = c->L[i].cur; else if (c->L[i].cur != cur) same = false; }
         if (same) { DC_TRY(dc_launch_classify_all(c, cur)); classified = true; }
     }
+    c->list_mark = refresh ? -1 : classified ? c->launches : DC_LISTS_FRESH;      // a full frame's lists are constant
     for (int i = 0; i < n; ++i) {
         dc_layer_rt& L = c->L[i];
         const void* in = layer_input(c, L.d.in0);
@@ -573,6 +575,7 @@ int dc_infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* ou
 {
     const int rc = infer_frame(c, frame_dev, pitch, out_map_dev, stats);
     g_dc_pdl = true;
+    if (c) c->list_mark = DC_LISTS_FRESH;
     return rc;
 }
 

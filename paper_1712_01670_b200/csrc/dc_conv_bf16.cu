@@ -50,6 +50,7 @@ struct TcArgs {
     // image row, numbered (stream * Ho + y) * gpr + column group; n_groups_all = S * Ho * gpr.  0: 16 x 8 blocks.
     int flat = 0, gpr = 0, n_groups_all = 0;
     int epi_warps = 4;            // epilogue warps of the CTA: 4 (192 threads) or 8 (320 threads)
+    int early = 0;                // tile list, count and bitmaps are older than the kernel before this one (dc_lists_settled): read before the wait for it
     int bias_smem = 0;            // > 0: that many bias values (the launch's NB * BN, from channel block nb_off on) are staged in shared memory behind the control block
 };
 
@@ -78,6 +79,9 @@ __device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, SmemC
 {
     return mbar_wait_at(bar, parity, &ctl->abort_flag, &ctl->wait_ns, status);
 }
+
+// From here on the previous kernel's output is read and this kernel's is written.
+__device__ __forceinline__ void enter() { dc_pdl_wait(); dc_pdl_release(); }
 
 // Copies the launch's bias values behind the control block (all threads; before the set-up's __syncthreads).  The
 // epilogue reads 32 of them per step and lane: from shared memory that is eight short broadcast loads, through the
@@ -119,12 +123,13 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
     auto fetch = [&](int item) {
         if (item >= n_items) return;
         const int idx = (item / a.NB) * tiles_per_group + tile_sub;
-        tile_n0 = idx < n_tiles ? a.tile_list[idx] : -1;                           // a pair's second CTA may have no tile in the last group
-        mask_n0 = tile_n0 >= 0 ? a.masks[(size_t)tile_n0 * 4 + mword_i] : 0u;
-        tile_n1 = (a.MT > 1 && idx + 1 < n_tiles) ? a.tile_list[idx + 1] : -1;     // odd tile count: the last item has one tile
-        mask_n1 = tile_n1 >= 0 ? a.masks[(size_t)tile_n1 * 4 + mword_i] : 0u;
+        tile_n0 = idx < n_tiles ? __ldcg(a.tile_list + idx) : -1;                  // a pair's second CTA may have no tile in the last group
+        mask_n0 = tile_n0 >= 0 ? __ldcg(a.masks + (size_t)tile_n0 * 4 + mword_i) : 0u;
+        tile_n1 = (a.MT > 1 && idx + 1 < n_tiles) ? __ldcg(a.tile_list + idx + 1) : -1;   // odd tile count: the last item has one tile
+        mask_n1 = tile_n1 >= 0 ? __ldcg(a.masks + (size_t)tile_n1 * 4 + mword_i) : 0u;
     };
     fetch(first_item);
+    if (a.early) enter();
     for (int item = first_item; item < n_items && ok; item += item_stride) {
         const int nb = item % a.NB;
         const int tile_c0 = tile_n0, tile_c1 = tile_n1;
@@ -251,9 +256,8 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
-    dc_pdl_release();
-    const int n_tiles = *a.tile_count;
+    if (!a.early) enter();      // else each role enters once it has its first tile
+    const int n_tiles = __ldcg(a.tile_count);
     const int n_items = (n_tiles + MT - 1) / MT * a.NB;     // an item: MT tiles x one block of BN channels; none for this CTA: it only frees its tensor memory
 
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
@@ -263,15 +267,32 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         r.start(smem_u32(ring), (uint32_t)a.stages);
         const uint32_t r0 = r.data, b_at = (uint32_t)(MT * a.a_bytes);
         bool ok = true;
+        int ahead = 0;                                              // steps whose weights are on their way already
+        // the weights are nobody's output: those of the first item's first steps travel while the previous kernel ends
+        auto weights_ahead = [&](uint32_t tx, int row0) -> int {
+            if (a.skip_loads) return 0;
+            const int n = min(a.stages, kiters);
+            for (int k = 0; k < n; ++k) {
+                mbar_expect_tx(full0 + 8u * k, tx);
+                tma_load_2d(r0 + k * stage_bytes + b_at, &tmB, k * a.BK, row0, full0 + 8u * k);
+            }
+            return n;
+        };
         if (a.flat) {
             // flat tiles: lane l fetches group (l & 15) of tile (l >> 4), one box of 8 pixels per tap and chunk
+            const int j = lane >> 4;
+            int next = 0;                                       // this lane's tile of the item to come
+            auto peek = [&](int item) {
+                const int first = item / a.NB * MT;
+                if (item < n_items && j < MT) next = __ldcg(a.tile_list + (first + j < n_tiles ? first + j : first));
+            };
+            peek(blockIdx.x);
+            bool entered = !a.early;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int group = item / a.NB, nb = item % a.NB;
-                const int row0 = (nb + a.nb_off) * a.BN;
+                const int row0 = (item % a.NB + a.nb_off) * a.BN, tile = next;
+                peek(item + gridDim.x);
                 int fs = 0, fx = 0, fy = 0; bool fon = false;
-                const int j = lane >> 4, idx = group * MT + j;
                 if (j < MT) {
-                    const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
                     const int gps = a.Ho * a.gpr, g = tile * DC_TILE_H + (lane & 15);
                     fon = g < a.n_groups_all;                   // the last tile may have fewer groups: their rows stay as they are (never stored)
                     fs = g / gps;
@@ -280,12 +301,19 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 }
                 const uint32_t piece = (uint32_t)(a.a_bytes / DC_TILE_H);
                 const uint32_t tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * piece + (uint32_t)a.b_bytes;
+                if (!entered) {
+                    if (elect_one()) ahead = weights_ahead(tx, row0);
+                    ahead = __reduce_max_sync(0xffffffffu, ahead);
+                    enter();
+                    entered = true;
+                }
                 for (int tap = 0; tap < taps && ok; ++tap) {
                     const int ky = tap / a.kw, kx = tap - ky * a.kw;
                     for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                         ok = __all_sync(0xffffffffu, mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status));
                         if (ok && !a.skip_loads) {
-                            if (elect_one()) {
+                            if (ahead > 0) --ahead;
+                            else if (elect_one()) {
                                 mbar_expect_tx(full0 + r.off, tx);
                                 tma_load_2d(r.data + b_at, &tmB, tap * a.Ci + cc * a.BK, row0, full0 + r.off);
                             }
@@ -296,19 +324,31 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     }
                 }
             }
+            if (!entered) enter();
         } else if (elect_one()) {
+            int next[MT];                                           // tiles of the item to come
+            auto peek = [&](int item) {
+                const int first = item / a.NB * MT;
+#pragma unroll
+                for (int j = 0; j < MT; ++j)                        // an absent second tile repeats the first (never stored)
+                    if (item < n_items) next[j] = __ldcg(a.tile_list + (first + j < n_tiles ? first + j : first));
+            };
+            peek(blockIdx.x);
+            const uint32_t tx = b_at + (uint32_t)a.b_bytes;
+            if (a.early) {
+                if ((int)blockIdx.x < n_items) ahead = weights_ahead(tx, ((int)blockIdx.x % a.NB + a.nb_off) * a.BN);
+                enter();
+            }
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int group = item / a.NB, nb = item % a.NB;
-                const int row0 = (nb + a.nb_off) * a.BN;
-                const uint32_t tx = b_at + (uint32_t)a.b_bytes;
+                const int row0 = (item % a.NB + a.nb_off) * a.BN;
                 int sN[MT], xb[MT], yb[MT];
 #pragma unroll
-                for (int j = 0; j < MT; ++j) {                      // an absent second tile repeats the first (never stored)
-                    const int idx = group * MT + j;
-                    const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
+                for (int j = 0; j < MT; ++j) {
+                    const int tile = next[j];
                     const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx_ = t - ty * a.tiles_x;
                     sN[j] = s; xb[j] = tx_ * DC_TILE_W * a.sw - a.pw; yb[j] = ty * DC_TILE_H * a.sh - a.ph;
                 }
+                peek(item + gridDim.x);
                 int w_col = 0;                                      // column of the weight matrix: taps, then channels
                 for (int ky = 0; ky < a.kh && ok; ++ky)
                     for (int kx = 0; kx < a.kw && ok; ++kx)
@@ -316,11 +356,14 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                             ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
                             if (!ok) break;
                             if (!a.skip_loads) {
-                                mbar_expect_tx(full0 + r.off, tx);
+                                if (ahead > 0) --ahead;
+                                else {
+                                    mbar_expect_tx(full0 + r.off, tx);
+                                    tma_load_2d(r.data + b_at, &tmB, w_col, row0, full0 + r.off);
+                                }
 #pragma unroll
                                 for (int j = 0; j < MT; ++j)
                                     tma_load_4d(r.data + j * a.a_bytes, &tmA, c0, xb[j] + kx, yb[j] + ky, sN[j], full0 + r.off);
-                                tma_load_2d(r.data + b_at, &tmB, w_col, row0, full0 + r.off);
                             }
                             r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
                         }
@@ -334,6 +377,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
+        if (a.early) enter();
         // Descriptors differ from slot to slot in their address bits alone.
         if (elect_one()) {
             const uint64_t dconst = umma_desc(0, a.sbo, a.layout_type);
@@ -432,9 +476,8 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
-    dc_pdl_release();
-    const int n_items = *a.tile_count;
+    if (!a.early) enter();      // else each role enters once it has its first tile
+    const int n_items = __ldcg(a.tile_count);
 
     if (warp == 0) {
         if (elect_one()) {                                      // producer: one patch per item
@@ -442,10 +485,11 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
             r.start(smem_u32(ring), (uint32_t)a.stages);
             const uint32_t r0 = r.data, full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
             bool ok = true;
-            int tile_next = a.tile_list[blockIdx.x];            // fetched one item ahead: off the critical path
+            int tile_next = __ldcg(a.tile_list + blockIdx.x);   // fetched one item ahead: off the critical path
+            if (a.early) enter();
             for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
                 const int tile = tile_next;
-                if (item + (int)gridDim.x < n_items) tile_next = a.tile_list[item + gridDim.x];
+                if (item + (int)gridDim.x < n_items) tile_next = __ldcg(a.tile_list + item + gridDim.x);
                 const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
                 ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
                 if (!ok) break;
@@ -459,6 +503,7 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
         }
         __syncwarp();
     } else if (warp == 1) {
+        if (a.early) enter();
         if (elect_one()) {                                      // MMA issuer
             const uint32_t b_lbo = (uint32_t)a.Co * 16u;
             const uint64_t bconst = umma_desc(smem_u32(wsm), 128, 0, b_lbo);
@@ -560,9 +605,8 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
-    dc_pdl_release();
-    const int n_tiles = *a.tile_count;
+    if (!a.early) enter();      // else each role enters once it has its first tile
+    const int n_tiles = __ldcg(a.tile_count);
     const int n_items = (n_tiles + MT - 1) / MT * a.NB;
 
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
@@ -574,16 +618,38 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
             const uint32_t a0 = ra.data, b0 = rb.data;
             const size_t tap_stride = (size_t)a.kchunks * a.b_bytes;             // packed weights: one tap further
             bool ok = true;
+            int next[MT];                                                        // tiles of the item to come
+            auto peek = [&](int item) {
+                const int first = item / a.NB * MT;
+#pragma unroll
+                for (int j = 0; j < MT; ++j)                                     // an absent second tile repeats the first (never stored)
+                    if (item < n_items) next[j] = __ldcg(a.tile_list + (first + j < n_tiles ? first + j : first));
+            };
+            peek(blockIdx.x);
+            int ahead = 0;                                                       // weight tiles on their way already
+            if (a.early) {
+                // the weights are nobody's output: the first item's first tiles travel while the previous kernel ends
+                if ((int)blockIdx.x < n_items && !a.skip_loads) {
+                    const uint8_t* w = (const uint8_t*)ha.wpacked + (size_t)((int)blockIdx.x % a.NB + a.nb_off) * taps * tap_stride;
+                    const int n_ax = SLAB ? a.kw : 1, n_t = SLAB ? a.kh : taps, n = min(a.stages, a.kchunks * taps);
+                    for (int cc = 0, ax = 0, t = 0; ahead < n; ++ahead) {
+                        mbar_expect_tx(full0 + 8u * ahead, (uint32_t)a.b_bytes);
+                        bulk_copy(b0 + ahead * a.b_bytes, w + (SLAB ? t * a.kw + ax : t) * tap_stride + (size_t)cc * a.b_bytes, (uint32_t)a.b_bytes, full0 + 8u * ahead);
+                        if (++t == n_t) { t = 0; if (++ax == n_ax) { ax = 0; ++cc; } }
+                    }
+                }
+                enter();
+            }
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int group = item / a.NB, nb = item % a.NB;
+                const int nb = item % a.NB;
                 int sN[MT], xb[MT], yb[MT];
 #pragma unroll
                 for (int j = 0; j < MT; ++j) {
-                    const int idx = group * MT + j;
-                    const int tile = a.tile_list[idx < n_tiles ? idx : group * MT];
+                    const int tile = next[j];
                     const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
                     sN[j] = s; xb[j] = tx * DC_TILE_W - a.pw; yb[j] = ty * DC_TILE_H - a.ph;
                 }
+                peek(item + gridDim.x);
                 const uint8_t* w_item = (const uint8_t*)ha.wpacked + (size_t)(nb + a.nb_off) * taps * tap_stride;
                 for (int cc = 0; cc < a.kchunks && ok; ++cc) {
                     for (int kx = 0; kx < (SLAB ? a.kw : 1) && ok; ++kx) {
@@ -609,11 +675,15 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                         const size_t w_step = SLAB ? a.kw * tap_stride : tap_stride;
                         const int n_t = SLAB ? a.kh : taps;
                         for (int t = 0; t < n_t; ++t) {
-                            ok = mbar_wait_a(empty0 + rb.off, rb.phase ^ 1u, ctl, a.status);
-                            if (!ok) break;
-                            if (!a.skip_loads) {
-                                mbar_expect_tx(full0 + rb.off, (uint32_t)a.b_bytes);
-                                bulk_copy(rb.data, w, (uint32_t)a.b_bytes, full0 + rb.off);
+                            // a tile sent ahead: its slot was free, and may have been used and freed again by now (no wait for it)
+                            if (ahead > 0) --ahead;
+                            else {
+                                ok = mbar_wait_a(empty0 + rb.off, rb.phase ^ 1u, ctl, a.status);
+                                if (!ok) break;
+                                if (!a.skip_loads) {
+                                    mbar_expect_tx(full0 + rb.off, (uint32_t)a.b_bytes);
+                                    bulk_copy(rb.data, w, (uint32_t)a.b_bytes, full0 + rb.off);
+                                }
                             }
                             w += w_step;
                             rb.next(b0, (uint32_t)a.stages, (uint32_t)a.b_bytes);
@@ -626,6 +696,7 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
+        if (a.early) enter();
         if (elect_one()) {
             // A: patch planes (rows PW * 16 bytes apart, planes along K), or a 128-byte swizzled K-major slab; weights: 128-byte
             // swizzled, K-major.  Descriptors differ from slot to slot in their lower halves alone.
@@ -755,9 +826,8 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     cluster_sync_all();                                       // both CTAs' barriers exist before either is signalled from outside
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    dc_pdl_wait();              // the previous kernel's output, the tile list and its count are read from here on
-    dc_pdl_release();
-    const int n_tiles = *a.tile_count;
+    if (!a.early) enter();      // else each role enters once it has its first tile
+    const int n_tiles = __ldcg(a.tile_count);
     const int n_items = (n_tiles + 1) / 2 * a.NB;
 
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
@@ -770,10 +840,16 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t a0 = ra.data, b0 = rb.data;
             const int rows_per_tile = a.b_bytes >> 7;             // weight rows of 128 bytes in one CTA's tile
             bool ok = true;
+            int next = 0;                                         // the tile of the item to come
+            auto peek = [&](int item) {
+                const int first = item / a.NB * 2, idx = first + (int)rank;
+                if (item < n_items) next = __ldcg(a.tile_list + (idx < n_tiles ? idx : first));   // an absent second tile repeats the first (never stored)
+            };
+            peek(pair);
+            if (a.early) enter();
             for (int item = pair; item < n_items && ok; item += n_pairs) {
-                const int group = item / a.NB, nb = item % a.NB;
-                const int idx = group * 2 + (int)rank;
-                const int tile = a.tile_list[idx < n_tiles ? idx : group * 2];      // an absent second tile repeats the first (never stored)
+                const int nb = item % a.NB, tile = next;
+                peek(item + n_pairs);
                 const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
                 const int xb = tx * DC_TILE_W - a.pw, yb = ty * DC_TILE_H - a.ph;
                 const int row_step = a.kw * a.kchunks * rows_per_tile;              // packed weights: one kernel row further
@@ -804,6 +880,7 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         __syncwarp();
     } else if (warp == 1) {
         // ---------------- MMA issuer: an elected lane of the leader issues for both CTAs ----------------
+        if (a.early) enter();
         if (leader && elect_one()) {
             const uint64_t dconst = umma_desc(0, 1024, 2);            // slabs and weights: 128-byte swizzled, K-major
             const uint32_t d_hi = (uint32_t)(dconst >> 32), a0 = (uint32_t)dconst + (smem_u32(aring) >> 4), b0 = (uint32_t)dconst + (smem_u32(bring) >> 4);
@@ -1198,6 +1275,7 @@ static int launch_smallc(dc_cache* c, int layer, const void* in, void* out, cons
     a.BN = d.cout; a.NB = 1; a.nb_off = 0; a.MT = 1; a.nbuf = 2; a.BK = 16; a.kchunks = 1; a.a_bytes = 0; a.b_bytes = 0; a.sbo = 128; a.layout_type = 0;
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(d.cout >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.status = c->status;
+    a.early = dc_lists_settled(c);
     set_wait_limit(c, a);
     sa.wpacked = (const __nv_bfloat16*)L.weight_packed;
     sa.kblocks = L.k_packed / 8;
@@ -1273,6 +1351,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     a.a_bytes = 0; a.b_bytes = h.b_bytes; a.sbo = 128; a.layout_type = 0;
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(h.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.status = c->status;
+    a.early = dc_lists_settled(c);
     set_wait_limit(c, a);
     ha.wpacked = (const __nv_bfloat16*)L.weight_halo;
     ha.k_last = h.k_last;
@@ -1380,6 +1459,7 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     // instruction descriptor: D = f32, A = B = bf16, both K-major, N = bn, M = 256 (128 rows in each CTA)
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
     a.status = c->status;
+    a.early = dc_lists_settled(c);
     set_wait_limit(c, a);
     a.tmem_cols = tmem_cols_for(2, 1, bn);
     ha.wpacked = (const __nv_bfloat16*)L.weight_halo;
@@ -1505,7 +1585,7 @@ static int launch_cluster(dc_cache* c, int layer, int grp, const void* in, void*
     a.status = c->status;
     TcArgs w;
     set_wait_limit(c, w);
-    a.wait_ns = w.wait_ns; a.skip_loads = w.skip_loads;
+    a.wait_ns = w.wait_ns; a.skip_loads = w.skip_loads; a.early = dc_lists_settled(c);
     a.add_in = (const __nv_bfloat16*)c->add_in; a.add_out = (__nv_bfloat16*)c->add_out; a.add_relu = c->add_relu;
     dc_prof_scope ps(c, DC_ST_CONV);
     c->launches += 1;
@@ -1560,6 +1640,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr;
     a.epi_warps = epi_warps_for(ctas);
     a.bias_smem = t_bias_bytes ? d.cout : 0;
+    a.early = dc_lists_settled(c);
     set_wait_limit(c, a);
     static dc_once_per_device attr_set;
     if (attr_set.first(c->device)) {
@@ -1596,6 +1677,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     DC_CUDA(cudaEventCreate(&e0));
     DC_CUDA(cudaEventCreate(&e1));
     float best = 1e30f; int best_mt = L.tc_mt, best_bn = L.tc_bn, best_ctas = 1, best_flat = 0, best_ew = 4, best_cs = 0;
+    c->list_mark = -1;                                                // the list of all tiles
     constexpr int kTuneReps = 6;                                      // timed launches per candidate, after one untimed
     // the GPU may have been idle: bring the clocks up before the first candidate is timed
     for (int rep = 0; rep < 12; ++rep)
@@ -1689,7 +1771,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     }
     L.tc_mt = best_mt; L.tc_bn = best_bn; L.tc_ctas = best_ctas; L.flat = best_flat; L.tc_ew = best_ew; L.tc_cs = best_cs;
     cudaEventDestroy(e0); cudaEventDestroy(e1);
-    c->launches = 0;
+    c->launches = 0; c->list_mark = DC_LISTS_FRESH;
     if (verbose) fprintf(stderr, "libdeepcache: layer %d: chose code %d, %d channels per block, %d CTA(s) per SM, %d epilogue warps, clusters of %d (%.4f ms)\n",
                          layer, best_flat ? best_mt + 7 : best_mt, best_bn, best_ctas, best_ew, best_cs, best / kTuneReps);
     return DC_OK;

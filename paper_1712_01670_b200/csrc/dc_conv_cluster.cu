@@ -83,10 +83,11 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         }
     }
     __syncwarp();
-    dc_pdl_wait();                           // the previous kernel's output, the tile list and its count are read from here on
-    dc_pdl_release();
-    const int n_tiles = *a.tile_count;
-    const int listed = a.tile_list[idx];     // inside the list's length whatever the count
+    // the previous kernel's output is read, and this one's written, only after the wait; the tile list and the bitmaps too,
+    // unless they are older than that kernel
+    if (!a.early) { dc_pdl_wait(); dc_pdl_release(); }
+    const int n_tiles = __ldcg(a.tile_count);
+    const int listed = __ldcg(a.tile_list + idx);     // inside the list's length whatever the count
     const bool present = idx < n_tiles;
     const int tile = present ? listed : 0;
 
@@ -115,15 +116,17 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         const int pr = u / per_px, c8 = u - pr * per_px, m = rank * rows + pr, row = m / DC_TILE_W, col = m % DC_TILE_W;
         int s = 0, y = 0, x0 = 0;
         n.in_map = locate(row, s, y, x0) && x0 + col < a.Wo;
-        n.active = n.in_map && !((a.masks[(size_t)tile * 4 + (row >> 2)] >> (8 * (row & 3) + col)) & 1u);
+        n.active = n.in_map && !((__ldcg(a.masks + (size_t)tile * 4 + (row >> 2)) >> (8 * (row & 3) + col)) & 1u);
         const int ch = (nb + a.nb_off) * a.BN + c8 * 8;
         n.at = (((size_t)s * a.Ho + y) * a.Wo + x0 + col) * a.Co + ch;
         n.b0 = __ldg((const float4*)(a.bias + ch)); n.b1 = __ldg((const float4*)(a.bias + ch + 4));
-        n.other = n.in_map && a.add_out ? *(const uint4*)(a.add_in + n.at) : make_uint4(0, 0, 0, 0);
         return n;
     };
+    auto fetch_other = [&](Unit& n) { if (n.in_map && a.add_out) n.other = *(const uint4*)(a.add_in + n.at); };
     Unit mine = {};
     if ((int)threadIdx.x < units) mine = unit_of(threadIdx.x);
+    if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
+    fetch_other(mine);
 
     if (warp == 0) {
         // ---------------- producer ----------------
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     if (!dead) {
         // ---------------- this CTA's pixels: sums from all ranks, bias, ReLU, bf16, store ----------------
         for (int u = threadIdx.x; u < units; u += kThreadsCl) {
-            if (u != (int)threadIdx.x) mine = unit_of(u);
+            if (u != (int)threadIdx.x) { mine = unit_of(u); fetch_other(mine); }
             if (!mine.in_map || (!mine.active && !a.add_out)) continue;
             uint4 o;
             if (mine.active) {

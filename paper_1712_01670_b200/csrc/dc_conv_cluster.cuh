@@ -16,6 +16,7 @@ struct dc_cluster_args {
     int32_t* status;
     unsigned long long wait_ns;
     int skip_loads;
+    int early;                               // tile list, count and bitmaps are older than the kernel before this one (dc_lists_settled)
     // element-wise add of a later layer done here: add_out = (this layer's output) + add_in (+ ReLU), or NULL
     const __nv_bfloat16* add_in; __nv_bfloat16* add_out; int add_relu;
 };

@@ -46,6 +46,7 @@ struct SimtArgs {
     const int32_t* tile_list; const int32_t* tile_count; const uint32_t* masks;
     int Hi, Wi, Ci, Ho, Wo, Co, p, relu, tiles_x, tiles_y;
     int Cig, Cog, nb_g, NB, chunks;                                   // channels per group, blocks per group, blocks in all
+    int early;                                                        // dc_lists_settled()
 };
 
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi)
@@ -123,18 +124,20 @@ __global__ void __launch_bounds__(KS * simt_threads(BN, TC)) k_conv_simt(const S
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     if (ks < a.chunks) fetch_weights(ks, 0);                                              // the weights are nobody's output: before the wait
-    dc_pdl_wait();
-    dc_pdl_release();
-    if (ti >= *a.tile_count) { asm volatile("cp.async.wait_all;" ::: "memory"); return; }
-    const int tile = a.tile_list[ti];
+    // the previous kernel's output is read only after the wait; the tile list and the bitmaps too, unless they are older than it
+    if (!a.early) { dc_pdl_wait(); dc_pdl_release(); }
+    const bool present = ti < __ldcg(a.tile_count);
+    const int tile = present ? __ldcg(a.tile_list + ti) : 0;
     const int per = a.tiles_x * a.tiles_y, s = tile / per, t = tile - s * per, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
     const int grp = nb / a.nb_g, cb = (nb - grp * a.nb_g) * BN;       // group, first channel of the block inside it
     const int oy = ty * DC_TILE_H + prow, ox0 = tx * DC_TILE_W;
     // the row's pixels that this item has to write: inside the map and not reused
-    uint32_t todo = ~(a.masks[(size_t)tile * 4 + (prow >> 2)] >> (8 * (prow & 3))) & 0xffu;
+    uint32_t todo = ~(__ldcg(a.masks + (size_t)tile * 4 + (prow >> 2)) >> (8 * (prow & 3))) & 0xffu;
     if (a.Wo - ox0 < DC_TILE_W) todo &= (1u << (a.Wo - ox0)) - 1u;
     if (oy >= a.Ho) todo = 0;
     const bool busy = __any_sync(0xffffffffu, todo != 0);
+    if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
+    if (!present) { asm volatile("cp.async.wait_all;" ::: "memory"); return; }
 
     const T* in = (const T*)a.in + (size_t)s * a.Hi * a.Wi * a.Ci + grp * a.Cig;
     const bool vec = a.Ci % 4 == 0 && a.Cig % 4 == 0;
@@ -401,7 +404,7 @@ int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const
     const int G = L.d.groups > 1 ? L.d.groups : 1;
     SimtArgs a;
     a.in = in; a.w = L.weight_simt; a.bias = L.bias; a.out = out;
-    a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;
+    a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks; a.early = dc_lists_settled(c);
     a.Hi = L.in_h; a.Wi = L.in_w; a.Ci = L.d.cin; a.Ho = L.d.out_h; a.Wo = L.d.out_w; a.Co = L.d.cout; a.p = L.d.ph; a.relu = L.d.relu;
     a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
     a.Cig = L.d.cin / G; a.Cog = L.d.cout / G; a.nb_g = dc_div_up(a.Cog, sh.BN); a.NB = G * a.nb_g; a.chunks = dc_div_up(a.Cig, sh.CI);

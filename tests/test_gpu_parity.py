@@ -207,6 +207,29 @@ def test_match_three_step_16_windows(R, shape):
     check_pairs([(prev, far), (const, const), (smooth, np.roll(smooth, 2, axis=1)), (prev, smooth)], 16, R, B.DC_SEARCH_THREE_STEP)
 
 
+@pytest.mark.parametrize("hw,S", [((64, 64), 1), ((160, 128), 16)])
+def test_infer_back_to_back_frames(hw, S):
+    """Frames without a pause: tile lists and first weights are read before a kernel's turn (narrow layers whose weight
+    tiles fit the ring whole).  No wait may run out, and the maps are those of frames run one by one."""
+    g = rng(S)
+    net = nets.inception_lrn_net(*hw)
+    ws, bs = nets.random_weights(net, 3)
+    frames = [torch.from_numpy(g.integers(0, 256, size=(S, hw[0], hw[1], 3), dtype=np.uint8)).cuda() for _ in range(2)]
+    for f in frames[1:]:
+        f[:, :, : hw[1] // 2] = frames[0][:, :, : hw[1] // 2]
+    maps = []
+    for pause in (False, True):
+        dc = DeepCache(hw[1], hw[0], net, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_BF16, cache_pool=True)
+        for i in range(300):
+            dc.infer_frame(frames[i % 2], want_out=False)
+            if pause:
+                torch.cuda.synchronize()
+        assert dc.status() == B.DC_OK
+        maps.append(dc.layer_map(len(net) - 1).float().clone())
+        dc.close()
+    torch.testing.assert_close(maps[0], maps[1], rtol=0.05, atol=0.05 * float(maps[1].abs().max()))
+
+
 @pytest.mark.parametrize("widx", [2, 3, 4])
 def test_infer_per_block_regions(widx):
     U.run_stream_parity(configs.WORKLOADS[widx](), 1, list(range(4)), region_mode=B.DC_REGIONS_PER_BLOCK)
