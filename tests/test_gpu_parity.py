@@ -207,6 +207,23 @@ def test_match_three_step_16_windows(R, shape):
     check_pairs([(prev, far), (const, const), (smooth, np.roll(smooth, 2, axis=1)), (prev, smooth)], 16, R, B.DC_SEARCH_THREE_STEP)
 
 
+@pytest.mark.parametrize("h,w,k,st,p", [(33, 41, 3, 2, 1), (32, 32, 7, 2, 3), (47, 35, 5, 3, 2), (30, 31, 7, 3, 0), (39, 227, 11, 4, 0), (41, 43, 11, 4, 5)])
+def test_frame_into_block_map(h, w, k, st, p):
+    """A frame goes straight into a strided first layer's block map: blocks of 2, 3 and 4, padding on every side, rows that
+    end inside a word.  The same values as the block map of the frame's own input map, so the same output."""
+    S = 3
+    g = rng(h * w)
+    nb = nets.NetBuilder(h, w)
+    nb.conv(-1, 32, k, st, p, 1)
+    ws, bs = nets.random_weights(nb.layers, 5)
+    frame = torch.from_numpy(g.integers(0, 256, size=(S, h, w, 3), dtype=np.uint8)).cuda()
+    dc = DeepCache(w, h, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_BF16)
+    out = dc.infer_frame(frame)
+    want = dc.conv_partial(0, (frame.float() * (1.0 / 255.0)).to(torch.bfloat16))
+    assert torch.equal(out.view(want.shape), want)
+    dc.close()
+
+
 @pytest.mark.parametrize("hw,S", [((64, 64), 1), ((160, 128), 16)])
 def test_infer_back_to_back_frames(hw, S):
     """Frames without a pause: tile lists and first weights are read before a kernel's turn (narrow layers whose weight
