@@ -486,25 +486,7 @@ __host__ __device__ constexpr int point_y(int i)
     constexpr int t[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1};
     return t[i];
 }
-constexpr int kNP[25] = {0, 0, 31, 0, 0, 0, 11, 0, 21, 0, 171, 0, 0, 0, 213, 0, 168, 0, 208, 0, 0, 0, 248, 0, 0};
-// new-point masks of the 8 possible moves; a move's table index (my + 2) * 5 + (mx + 2) is always even
-constexpr unsigned long long pack_moves(int first)
-{
-    unsigned long long r = 0;
-    for (int h = first; h < first + 8 && 2 * h < 25; ++h) r |= (unsigned long long)kNP[2 * h] << (8 * (h - first));
-    return r;
-}
-constexpr unsigned long long kMovesLo = pack_moves(0), kMovesHi = pack_moves(8);
-
-// points of the large diamond around a new centre that the diamond around the old one did not contain:
-// the others lost to the new centre already and cannot win (mx, my: the move, one of the 8 diamond offsets)
-__device__ __forceinline__ uint32_t new_points(int mx, int my)
-{
-    const int h = ((my + 2) * 5 + (mx + 2)) >> 1;
-    return (uint32_t)((h < 8 ? kMovesLo >> (8 * h) : kMovesHi >> (8 * (h - 8))) & 0xffu);
-}
-
-// The same points for look-ups with a run-time index (the same in all lanes of a warp: one constant-cache access).
+// The points for look-ups with a run-time index (the same in all lanes of a warp: one constant-cache access).
 __constant__ int c_point_x[13] = {0, -1, 1, -2, 2, -1, 1, 0, 0, 0, -1, 1, 0};
 __constant__ int c_point_y[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1};
 // Per point and window pitch: byte offset of the point's candidate from the centre's, << 16, | the low 16 bits of the
