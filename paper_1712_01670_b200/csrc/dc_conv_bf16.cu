@@ -51,6 +51,7 @@ struct TcArgs {
     int flat = 0, gpr = 0, n_groups_all = 0;
     int epi_warps = 4;            // epilogue warps of the CTA: 4 (192 threads) or 8 (320 threads)
     int early = 0;                // tile list, count and bitmaps are older than the kernel before this one (dc_lists_settled): read before the wait for it
+    int slab_order = 0;           // tap-by-tap kernel: the steps in the column-slab kernels' order (see StepOrder)
     int bias_smem = 0;            // > 0: that many bias values (the launch's NB * BN, from channel block nb_off on) are staged in shared memory behind the control block
 };
 
@@ -82,6 +83,55 @@ __device__ __forceinline__ bool mbar_wait_a(uint32_t bar, uint32_t parity, SmemC
 
 // From here on the previous kernel's output is read and this kernel's is written.
 __device__ __forceinline__ void enter() { dc_pdl_wait(); dc_pdl_release(); }
+
+// The order in which a layer's products are summed.  Every kernel that a layer could be timed with sums in the same one, so that
+// the tuner's choice never shows in an output: two caches of one configuration give the same bits.  Layers that the
+// column-slab kernels take: 64 channels at a time, kernel columns, kernel rows (a slab holds one column's pixels for all
+// rows), 16 channels.  The others: kernel rows, kernel columns, channels.  (What a cluster sums in parts is decided by sizes
+// alone: cluster_rule.)
+//
+// The loop nest of a tap-by-tap producer: the innermost axis is the longest run in which only the channel, the input row and
+// the weights' column move, by constants (the producer is one lane: each nested loop's turn costs it).
+struct StepOrder {
+    int n0, n1, n2, n3, n3_last;                               // turns of the four axes, n3_last in the last turn of the outermost
+    int c0, c1, c3;                                            // what a turn adds to the first channel,
+    int x1, x2, y1, y2, y3;                                    // to (kx, ky)
+    int w0, w1, w2, w3;                                        // and to the column of the weight matrix (taps, then channels)
+    __device__ __forceinline__ explicit StepOrder(const TcArgs& a)
+    {
+        n0 = 1; c0 = c1 = c3 = 0; x1 = x2 = y1 = y2 = y3 = 0; w0 = 0;
+        const int row = a.kw * a.Ci;
+        if (!a.slab_order) {                                   // kernel rows, kernel columns, channels
+            n1 = a.kh; y1 = 1; w1 = row;
+            n2 = a.kw; x2 = 1; w2 = a.Ci;
+            n3 = n3_last = a.kchunks; c3 = w3 = a.BK;
+        } else if (a.BK == 64) {                               // channels, kernel columns, kernel rows
+            n1 = a.kchunks; c1 = w1 = 64;
+            n2 = a.kw; x2 = 1; w2 = a.Ci;
+            n3 = n3_last = a.kh; y3 = 1; w3 = row;
+        } else {                                               // 64 channels, kernel columns, kernel rows, channels
+            n0 = (a.Ci + 63) / 64; c0 = w0 = 64;
+            n1 = a.kw; x1 = 1; w1 = a.Ci;
+            n2 = a.kh; y2 = 1; w2 = row;
+            n3 = 64 / a.BK; n3_last = (a.Ci - (n0 - 1) * 64) / a.BK; c3 = w3 = a.BK;
+        }
+    }
+    // step(c, kx, ky, w) for every step until it returns false
+    template <typename F>
+    __device__ __forceinline__ void walk(F&& step) const
+    {
+        for (int i0 = 0; i0 < n0; ++i0) {
+            const int n = i0 + 1 < n0 ? n3 : n3_last;
+            for (int i1 = 0; i1 < n1; ++i1)
+                for (int i2 = 0; i2 < n2; ++i2) {
+                    const int x = i1 * x1 + i2 * x2;
+                    int c = i0 * c0 + i1 * c1, y = i1 * y1 + i2 * y2, w = i0 * w0 + i1 * w1 + i2 * w2;
+                    for (int i3 = 0; i3 < n; ++i3, c += c3, y += y3, w += w3)
+                        if (!step(c, x, y, w)) return;
+                }
+        }
+    }
+};
 
 // Copies the launch's bias values behind the control block (all threads; before the set-up's __syncthreads).  The
 // epilogue reads 32 of them per step and lane: from shared memory that is eight short broadcast loads, through the
@@ -236,7 +286,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     SmemCtl* ctl = (SmemCtl*)(ring + (size_t)a.stages * stage_bytes);
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int per_stream = a.tiles_x * a.tiles_y;
-    const int taps = a.kh * a.kw, kiters = taps * a.kchunks;
+    const int kiters = a.kh * a.kw * a.kchunks;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < a.stages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
@@ -266,16 +316,21 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         RingPos r;
         r.start(smem_u32(ring), (uint32_t)a.stages);
         const uint32_t r0 = r.data, b_at = (uint32_t)(MT * a.a_bytes);
+        const StepOrder order(a);
         bool ok = true;
         int ahead = 0;                                              // steps whose weights are on their way already
         // the weights are nobody's output: those of the first item's first steps travel while the previous kernel ends
         auto weights_ahead = [&](uint32_t tx, int row0) -> int {
             if (a.skip_loads) return 0;
             const int n = min(a.stages, kiters);
-            for (int k = 0; k < n; ++k) {
+            int k = 0;
+            order.walk([&](int, int, int, int w) {
+                if (k == n) return false;
                 mbar_expect_tx(full0 + 8u * k, tx);
-                tma_load_2d(r0 + k * stage_bytes + b_at, &tmB, k * a.BK, row0, full0 + 8u * k);
-            }
+                tma_load_2d(r0 + k * stage_bytes + b_at, &tmB, w, row0, full0 + 8u * k);
+                ++k;
+                return true;
+            });
             return n;
         };
         if (a.flat) {
@@ -307,22 +362,21 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     enter();
                     entered = true;
                 }
-                for (int tap = 0; tap < taps && ok; ++tap) {
-                    const int ky = tap / a.kw, kx = tap - ky * a.kw;
-                    for (int cc = 0; cc < a.kchunks && ok; ++cc) {
-                        ok = __all_sync(0xffffffffu, mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status));
-                        if (ok && !a.skip_loads) {
-                            if (ahead > 0) --ahead;
-                            else if (elect_one()) {
-                                mbar_expect_tx(full0 + r.off, tx);
-                                tma_load_2d(r.data + b_at, &tmB, tap * a.Ci + cc * a.BK, row0, full0 + r.off);
-                            }
-                            __syncwarp();                               // the slot is free and its byte count announced: every lane brings its own group
-                            if (fon) tma_load_4d(r.data + lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, full0 + r.off);
+                order.walk([&](int c, int kx, int ky, int w) {
+                    ok = __all_sync(0xffffffffu, mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status));
+                    if (!ok) return false;
+                    if (!a.skip_loads) {
+                        if (ahead > 0) --ahead;
+                        else if (elect_one()) {
+                            mbar_expect_tx(full0 + r.off, tx);
+                            tma_load_2d(r.data + b_at, &tmB, w, row0, full0 + r.off);
                         }
-                        r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
+                        __syncwarp();                                   // the slot is free and its byte count announced: every lane brings its own group
+                        if (fon) tma_load_4d(r.data + lane * piece, &tmA, c, fx + kx, fy + ky, fs, full0 + r.off);
                     }
-                }
+                    r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
+                    return true;
+                });
             }
             if (!entered) enter();
         } else if (elect_one()) {
@@ -349,24 +403,22 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     sN[j] = s; xb[j] = tx_ * DC_TILE_W * a.sw - a.pw; yb[j] = ty * DC_TILE_H * a.sh - a.ph;
                 }
                 peek(item + gridDim.x);
-                int w_col = 0;                                      // column of the weight matrix: taps, then channels
-                for (int ky = 0; ky < a.kh && ok; ++ky)
-                    for (int kx = 0; kx < a.kw && ok; ++kx)
-                        for (int c0 = 0; c0 < a.Ci; c0 += a.BK, w_col += a.BK) {
-                            ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
-                            if (!ok) break;
-                            if (!a.skip_loads) {
-                                if (ahead > 0) --ahead;
-                                else {
-                                    mbar_expect_tx(full0 + r.off, tx);
-                                    tma_load_2d(r.data + b_at, &tmB, w_col, row0, full0 + r.off);
-                                }
-#pragma unroll
-                                for (int j = 0; j < MT; ++j)
-                                    tma_load_4d(r.data + j * a.a_bytes, &tmA, c0, xb[j] + kx, yb[j] + ky, sN[j], full0 + r.off);
-                            }
-                            r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
+                order.walk([&](int c, int kx, int ky, int w) {
+                    ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
+                    if (!ok) return false;
+                    if (!a.skip_loads) {
+                        if (ahead > 0) --ahead;
+                        else {
+                            mbar_expect_tx(full0 + r.off, tx);
+                            tma_load_2d(r.data + b_at, &tmB, w, row0, full0 + r.off);
                         }
+#pragma unroll
+                        for (int j = 0; j < MT; ++j)
+                            tma_load_4d(r.data + j * a.a_bytes, &tmA, c, xb[j] + kx, yb[j] + ky, sN[j], full0 + r.off);
+                    }
+                    r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
+                    return true;
+                });
             }
         }
         __syncwarp();
@@ -631,11 +683,11 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                 // the weights are nobody's output: the first item's first tiles travel while the previous kernel ends
                 if ((int)blockIdx.x < n_items && !a.skip_loads) {
                     const uint8_t* w = (const uint8_t*)ha.wpacked + (size_t)((int)blockIdx.x % a.NB + a.nb_off) * taps * tap_stride;
-                    const int n_ax = SLAB ? a.kw : 1, n_t = SLAB ? a.kh : taps, n = min(a.stages, a.kchunks * taps);
-                    for (int cc = 0, ax = 0, t = 0; ahead < n; ++ahead) {
+                    const int n = min(a.stages, a.kchunks * taps);
+                    for (int cc = 0, kx = 0, ky = 0; ahead < n; ++ahead) {
                         mbar_expect_tx(full0 + 8u * ahead, (uint32_t)a.b_bytes);
-                        bulk_copy(b0 + ahead * a.b_bytes, w + (SLAB ? t * a.kw + ax : t) * tap_stride + (size_t)cc * a.b_bytes, (uint32_t)a.b_bytes, full0 + 8u * ahead);
-                        if (++t == n_t) { t = 0; if (++ax == n_ax) { ax = 0; ++cc; } }
+                        bulk_copy(b0 + ahead * a.b_bytes, w + (ky * a.kw + kx) * tap_stride + (size_t)cc * a.b_bytes, (uint32_t)a.b_bytes, full0 + 8u * ahead);
+                        if (++ky == a.kh) { ky = 0; if (++kx == a.kw) { kx = 0; ++cc; } }
                     }
                 }
                 enter();
@@ -670,11 +722,11 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                             }
                         }
                         ra.next(a0, (uint32_t)ha.a_stages, (uint32_t)a_slot);
-                        // the weight tiles that go with this A stage: all taps (patch), or the taps of column kx (slab)
+                        // the weight tiles that go with this A stage: all taps, column by column (patch), or the taps of column kx (slab)
                         const uint8_t* w = w_item + kx * tap_stride + (size_t)cc * a.b_bytes;
-                        const size_t w_step = SLAB ? a.kw * tap_stride : tap_stride;
+                        const size_t w_step = a.kw * tap_stride;
                         const int n_t = SLAB ? a.kh : taps;
-                        for (int t = 0; t < n_t; ++t) {
+                        for (int t = 0, ky = 0; t < n_t; ++t) {
                             // a tile sent ahead: its slot was free, and may have been used and freed again by now (no wait for it)
                             if (ahead > 0) --ahead;
                             else {
@@ -686,6 +738,7 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                                 }
                             }
                             w += w_step;
+                            if (!SLAB && ++ky == a.kh) { ky = 0; w -= a.kh * w_step - tap_stride; }      // the next column's first row
                             rb.next(b0, (uint32_t)a.stages, (uint32_t)a.b_bytes);
                         }
                     }
@@ -719,9 +772,9 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                     const int n_kk = cc + 1 < a.kchunks ? 4 : ha.k_last;
                     for (int ax = 0; ax < (SLAB ? a.kw : 1) && ok; ++ax) {     // A stages of this chunk: one patch, or kw slabs
                         ok = mbar_wait_a(a_full0 + ra.off, ra.phase, ctl, a.status);
-                        // patch: taps in (ky, kx) order at (ky * PW + kx) * 16 bytes; slab ax: taps (ky, ax) at ky atoms of 1024 bytes
+                        // patch: taps column by column at (ky * PW + kx) * 16 bytes; slab ax: taps (ky, ax) at ky atoms of 1024 bytes
                         uint32_t at = ra.data;
-                        int col = 0;
+                        int ky = 0;
                         const int n_t = SLAB ? a.kh : taps;
                         for (int t = 0; t < n_t && ok; ++t) {
                             ok = mbar_wait_a(full0 + rb.off, rb.phase, ctl, a.status);
@@ -734,7 +787,7 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                             umma_commit_at(empty0 + rb.off);
                             rb.next(b0, (uint32_t)a.stages, b_lo);
                             if (SLAB) at += 64u;
-                            else if (++col == a.kw) { col = 0; at += (uint32_t)(ha.PW - a.kw + 1); } else at += 1u;
+                            else if (++ky == a.kh) { ky = 0; at += 1u - (uint32_t)((a.kh - 1) * ha.PW); } else at += (uint32_t)ha.PW;
                         }
                         if (ok) umma_commit_at(a_empty0 + ra.off);             // the A stage is free once its taps retire
                         ra.next(a0, (uint32_t)ha.a_stages, a_slot_lo);
@@ -1562,6 +1615,31 @@ static bool cluster_plan(const dc_layer_desc& d, int bn, int cs, TcPlan& p)
     return p.stages >= 2 || most == 1;
 }
 
+// Do the clusters of a layer with every tile dirty run at the same time?
+static bool cluster_fits(const dc_cache* c, const dc_layer_rt& L, const dc_layer_desc& d, int bn, int cs)
+{
+    TcPlan p;
+    if (d.cout % bn != 0 || !cluster_plan(d, bn, cs, p)) return false;
+    const long long clusters = (long long)L.tiles_x * L.tiles_y * c->S * (d.cout / bn);
+    return clusters <= dc_cluster_wave(c->device, cs, dc_cluster_smem(p.stages, p.a_bytes, p.b_bytes, p.BN));
+}
+
+// How many CTAs a layer's clusters have, 0: it stays on the other kernels.  By sizes alone: a cluster sums in parts, so a choice
+// by timing would show in the outputs.  Measured with `steps` of 64 channels, the fastest other kernel against clusters of 2 /
+// 4 / 8 (us a launch): 72 steps, 1 tile 18.9 against 13.4 / 8.8 / 8.2; 36 steps, 2 tiles 12.4, 9.4 / 6.8 / 7.3; 16 steps 7.9, 7.0 / 5.8 /
+// 6.1; 9 steps 6.5, 7.1 / 7.2 / 9.2; 4 steps 5.0, 6.1.  They pay while one wave holds them (54 steps in twos: 72 clusters 14.2
+// against 16.1, 96 clusters 25.7 against 16.5); twos, the last resort, need a longer reduction (27 steps 19.8 against 20.4, 18
+// steps 9.4 against 8.5, 25 steps 25.9 against 18.6).  Over the layers of the trunks at 1 to 128 streams the rule's choice takes
+// 0.3 % longer than the fastest one of each layer.
+static int cluster_rule(const dc_cache* c, const dc_layer_rt& L, const dc_layer_desc& d)
+{
+    const int steps = d.kh * d.kw * ((d.cin + 63) / 64);
+    const struct { int cs, steps; } take[3] = {{8, 48}, {4, 16}, {2, 26}};
+    for (const auto& t : take)
+        if (steps >= t.steps && (cluster_fits(c, L, d, 32, t.cs) || cluster_fits(c, L, d, 64, t.cs))) return t.cs;
+    return 0;
+}
+
 static int launch_cluster(dc_cache* c, int layer, int grp, const void* in, void* out, const int32_t* tile_list,
                           const int32_t* tile_count, const uint32_t* masks, int max_tiles)
 {
@@ -1581,7 +1659,6 @@ static int launch_cluster(dc_cache* c, int layer, int grp, const void* in, void*
     a.nb_off = grp * p.NB; a.CS = L.tc_cs;
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.sbo = p.sbo; a.layout_type = p.layout_type; a.tmem_cols = tmem_cols_for(1, 1, p.BN);
-    a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr;
     a.status = c->status;
     TcArgs w;
     set_wait_limit(c, w);
@@ -1640,6 +1717,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr;
     a.epi_warps = epi_warps_for(ctas);
     a.bias_smem = t_bias_bytes ? d.cout : 0;
+    a.slab_order = L.weight_halo != nullptr;
     a.early = dc_lists_settled(c);
     set_wait_limit(c, a);
     static dc_once_per_device attr_set;
@@ -1658,10 +1736,9 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
 }
 
 // Picks, per convolution layer, the operand scheme and the work-item shape (tiles per item x channels per block)
-// by timing the candidates once on the layer's own buffers with every tile dirty.  Within one scheme the choice
-// changes only how the work is cut.  Between schemes the order in which the taps are accumulated in fp32 differs
-// (the column-slab kernel goes column by column), so two choices can differ in the last bits of a bf16 output; every
-// choice stays within the parity bound.  Called by dc_cache_create (which may synchronise).
+// by timing the candidates once on the layer's own buffers with every tile dirty.  All candidates of a layer sum in the same
+// order (StepOrder; cluster_rule decides whether a layer's candidates are the clusters of one size or the other kernels), so
+// the choice changes no bit of an output.  Called by dc_cache_create (which may synchronise).
 int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
 {
     dc_layer_rt& L = c->L[layer];
@@ -1703,8 +1780,11 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
                              layer, what, L.flat ? L.tc_mt + 7 : L.tc_mt, L.tc_bn, L.tc_ctas, L.tc_ew, L.tc_cs, ms / kTuneReps);
         if (ms < best) { best = ms; best_mt = L.tc_mt; best_bn = L.tc_bn; best_ctas = L.tc_ctas; best_flat = L.flat; best_ew = L.tc_ew; best_cs = L.tc_cs; }
     };
+    // clusters of CTAs sum in parts, so their size follows from the layer's sizes; the other kernels are then not timed
+    const bool may_cluster = generic && !(de.cin < 16) && L.d.cin == de.cin * n_groups(L.d);
+    const int cs = may_cluster && (only == 0 || only == 10) ? cluster_rule(c, L, de) : 0;
     // one CTA per SM with four or eight epilogue warps, or two CTAs per SM with four each
-    for (int shape = 0; shape < 3; ++shape) {
+    for (int shape = 0; shape < 3 && cs == 0; ++shape) {
         const int ctas = shape == 2 ? 2 : 1;
         L.tc_ctas = ctas; L.tc_ew = shape == 1 ? 8 : 4;
         t_epi_warps = L.tc_ew;                                        // make_plan below sizes the rings for it
@@ -1715,7 +1795,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
             continue;
         }
         const int default_bn = p.BN;
-        for (int bn = default_bn; bn >= 64 && bn >= default_bn / 2; bn -= 32) {
+        for (int bn = default_bn; (bn >= 64 || bn == default_bn) && bn >= default_bn / 2; bn -= 32) {
             if (de.cout % bn != 0) continue;
             for (int mt = 1; mt <= 2; ++mt) {
                 TcPlan q;
@@ -1732,7 +1812,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
         }
         HaloPlan h0;
         if (L.weight_halo && halo_ok(de, h0)) {
-            for (int bn = h0.BN; bn >= 64 && bn >= h0.BN / 2; bn -= 32) {
+            for (int bn = h0.BN; (bn >= 64 || bn == h0.BN) && bn >= h0.BN / 2; bn -= 32) {
                 HaloPlan h;
                 if (!halo_ok(de, h, bn)) continue;
                 for (int mt = 1; mt <= 2; ++mt) {                      // tc_mt 3 / 4: patch-reuse kernel with 1 / 2 tiles per item
@@ -1747,27 +1827,21 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     }
     {
         int pbn = 0;
-        if (generic && L.weight_halo && pair_ok(L.d, pbn)) {          // tc_mt 7: a CTA pair per two tiles (cta_group::2)
+        if (cs == 0 && generic && L.weight_halo && pair_ok(L.d, pbn)) {   // tc_mt 7: a CTA pair per two tiles (cta_group::2)
             L.tc_mt = 7; L.tc_bn = pbn; L.tc_ctas = 1; L.tc_ew = 4;
             trial("CTA-pair kernel");
         }
     }
-    // few tiles: the reduction split over clusters of CTAs, while that gives no more than three CTAs per SM
-    if (generic && !(de.cin < 16) && L.d.cin == de.cin * n_groups(L.d)) {
+    if (cs > 0 || (may_cluster && only == 10)) {                      // asked for where the rule has none: any size (diagnostics)
         L.tc_mt = 1; L.tc_ctas = 1; L.tc_ew = 4;
-        for (int flat = 0; flat < 2; ++flat) {
-            if (flat && L.tiles_flat * 20 > L.tiles_x * L.tiles_y * c->S * 19) continue;
-            L.flat = flat;
-            for (int bn = 32; bn <= 64; bn += 32)
-                for (int cs = 2; cs <= 8; cs *= 2) {
-                    TcPlan q;
-                    if (de.cout % bn != 0 || !cluster_plan(de, bn, cs, q)) continue;
-                    if ((long long)dc_layer_tiles(c, L) * (de.cout / bn) * cs > 3LL * c->num_sms && only != 10) continue;
-                    L.tc_bn = bn; L.tc_cs = cs;
-                    trial("cluster kernel");
-                }
-        }
-        L.tc_cs = 0; L.flat = 0;
+        for (int bn = 32; bn <= 64; bn += 32)
+            for (int k = cs > 0 ? cs : 2; k <= (cs > 0 ? cs : 8); k *= 2) {
+                TcPlan q;
+                if (de.cout % bn != 0 || !cluster_plan(de, bn, k, q) || (cs > 0 && !cluster_fits(c, L, de, bn, k))) continue;
+                L.tc_bn = bn; L.tc_cs = k;
+                trial("cluster kernel");
+            }
+        L.tc_cs = 0;
     }
     L.tc_mt = best_mt; L.tc_bn = best_bn; L.tc_ctas = best_ctas; L.flat = best_flat; L.tc_ew = best_ew; L.tc_cs = best_cs;
     cudaEventDestroy(e0); cudaEventDestroy(e1);

@@ -92,21 +92,8 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     const int tile = present ? listed : 0;
 
     // this tile's pixels: pixel m is column m % 8 of tile row m / 8
-    const int gps = a.Ho * a.gpr, per_stream = a.tiles_x * a.tiles_y;
-    int ts = 0, ty = 0, tx = 0;
-    if (!a.flat) { ts = tile / per_stream; const int t = tile - ts * per_stream; ty = t / a.tiles_x; tx = t - ty * a.tiles_x; }
-    auto locate = [&](int row, int& s, int& y, int& x0) -> bool {             // tile row -> stream, map row, first column
-        if (a.flat) {
-            const int g = tile * DC_TILE_H + row;
-            if (g >= a.n_groups_all) return false;
-            s = g / gps;
-            const int loc = g - s * gps;
-            y = loc / a.gpr; x0 = (loc - y * a.gpr) * DC_TILE_W;
-            return true;
-        }
-        s = ts; y = ty * DC_TILE_H + row; x0 = tx * DC_TILE_W;
-        return y < a.Ho;
-    };
+    const int per_stream = a.tiles_x * a.tiles_y;
+    const int ts = tile / per_stream, t_in = tile - ts * per_stream, ty = t_in / a.tiles_x, tx = t_in - ty * a.tiles_x;
     // What thread u finishes: 8 channels of one of this CTA's pixels.  The first unit's operands are fetched now, beside
     // the loads and MMAs.
     const int rows = 128 / a.CS, per_px = a.BN / 8, units = present ? rows * per_px : 0;
@@ -114,11 +101,11 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     auto unit_of = [&](int u) -> Unit {
         Unit n;
         const int pr = u / per_px, c8 = u - pr * per_px, m = rank * rows + pr, row = m / DC_TILE_W, col = m % DC_TILE_W;
-        int s = 0, y = 0, x0 = 0;
-        n.in_map = locate(row, s, y, x0) && x0 + col < a.Wo;
+        const int y = ty * DC_TILE_H + row, x = tx * DC_TILE_W + col;
+        n.in_map = y < a.Ho && x < a.Wo;
         n.active = n.in_map && !((__ldcg(a.masks + (size_t)tile * 4 + (row >> 2)) >> (8 * (row & 3) + col)) & 1u);
         const int ch = (nb + a.nb_off) * a.BN + c8 * 8;
-        n.at = (((size_t)s * a.Ho + y) * a.Wo + x0 + col) * a.Co + ch;
+        n.at = (((size_t)ts * a.Ho + y) * a.Wo + x) * a.Co + ch;
         n.b0 = __ldg((const float4*)(a.bias + ch)); n.b1 = __ldg((const float4*)(a.bias + ch + 4));
         return n;
     };
@@ -136,38 +123,11 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
             if (lane == 0 && !a.skip_loads)
                 for (int it = 0; it < early && ok; ++it) { mbar_arrive(&ctl->full[it]); ok = cl_wait(full0 + 8u * it, 0, ctl, a.status); }
         } else if (!a.skip_loads) {
-            // 16 x 8 tile: an elected lane brings the window of a tap; flat tiles: lane l brings row piece l
-            int fs = 0, fx = 0, fy = 0;
-            bool fon = false;
-            if (a.flat) {
-                int y, x0;
-                fon = lane < DC_TILE_H && locate(lane, fs, y, x0);
-                if (fon) { fx = x0 * a.sw - a.pw; fy = y * a.sh - a.ph; }
-            } else {
-                fs = ts; fx = tx * DC_TILE_W * a.sw - a.pw; fy = ty * DC_TILE_H * a.sh - a.ph;
-            }
-            RingPos r;
-            r.start(ring0, (uint32_t)a.stages);
-            int cc = cc0, ky = tap0 / a.kw, kx = tap0 - ky * a.kw;
-            auto advance = [&]() {
-                if (++cc == a.kchunks) { cc = 0; if (++kx == a.kw) { kx = 0; ++ky; } }
-                r.next(ring0, (uint32_t)a.stages, (uint32_t)stage_bytes);
-            };
-            if (a.flat) {
-                const uint32_t piece = (uint32_t)(a.a_bytes / DC_TILE_H), a_tx = (uint32_t)__popc(__ballot_sync(0xffffffffu, fon)) * piece;
-                for (int it = 0; it < nk; ++it) {
-                    if (it >= a.stages) ok = __all_sync(0xffffffffu, cl_wait(empty0 + r.off, r.phase ^ 1u, ctl, a.status));
-                    if (!ok) break;
-                    if (elect_one()) {
-                        if (it >= a.stages) load_weights(ky * a.kw + kx, cc, r.off, r.data);
-                        mbar_expect_tx(full0 + r.off, a_tx);
-                    }
-                    __syncwarp();
-                    if (fon) tma_load_4d(r.data + lane * piece, &tmA, cc * a.BK, fx + kx, fy + ky, fs, full0 + r.off);
-                    __syncwarp();
-                    advance();
-                }
-            } else if (elect_one()) {
+            if (elect_one()) {
+                const int fx = tx * DC_TILE_W * a.sw - a.pw, fy = ty * DC_TILE_H * a.sh - a.ph;
+                RingPos r;
+                r.start(ring0, (uint32_t)a.stages);
+                int cc = cc0, ky = tap0 / a.kw, kx = tap0 - ky * a.kw;
                 for (int it = 0; it < nk; ++it) {
                     if (it >= a.stages) {
                         ok = cl_wait(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
@@ -175,8 +135,9 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
                         load_weights(ky * a.kw + kx, cc, r.off, r.data);
                     }
                     mbar_expect_tx(full0 + r.off, (uint32_t)a.a_bytes);
-                    tma_load_4d(r.data, &tmA, cc * a.BK, fx + kx, fy + ky, fs, full0 + r.off);
-                    advance();
+                    tma_load_4d(r.data, &tmA, cc * a.BK, fx + kx, fy + ky, ts, full0 + r.off);
+                    if (++cc == a.kchunks) { cc = 0; if (++kx == a.kw) { kx = 0; ++ky; } }
+                    r.next(ring0, (uint32_t)a.stages, (uint32_t)stage_bytes);
                 }
             }
         }
@@ -270,19 +231,39 @@ size_t dc_cluster_smem(int stages, int a_bytes, int b_bytes, int BN)
     return (size_t)stages * (a_bytes + b_bytes) + (size_t)128 * red_pitch(BN) * 4 + sizeof(CtlCl) + 1024;
 }
 
-int dc_launch_cluster_kernel(dc_cache* c, const CUtensorMap& tmA, const CUtensorMap& tmB, const dc_cluster_args& a, int tiles)
+static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int ctas, int cs, size_t smem, cudaStream_t stream)
 {
-    static dc_once_per_device attr_set;
-    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_conv_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((tiles < 1 ? 1 : tiles) * a.NB * a.CS)); cfg.blockDim = dim3(kThreadsCl); cfg.stream = c->stream;
-    cfg.dynamicSmemBytes = dc_cluster_smem(a.stages, a.a_bytes, a.b_bytes, a.BN);
-    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)a.CS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = (unsigned)cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = g_dc_pdl ? 2 : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3(kThreadsCl); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cfg;
+}
+
+static cudaError_t cluster_smem_opt_in(int device)
+{
+    static dc_once_per_device attr_set;
+    return attr_set.first(device) ? cudaFuncSetAttribute(k_conv_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) : cudaSuccess;
+}
+
+int dc_cluster_wave(int device, int cs, size_t smem)
+{
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(attr, cs, cs, smem, nullptr);
+    int n = 0;
+    if (cluster_smem_opt_in(device) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, k_conv_cluster, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return n;
+}
+
+int dc_launch_cluster_kernel(dc_cache* c, const CUtensorMap& tmA, const CUtensorMap& tmB, const dc_cluster_args& a, int tiles)
+{
+    DC_CUDA(cluster_smem_opt_in(c->device));
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(attr, (tiles < 1 ? 1 : tiles) * a.NB * a.CS, a.CS, dc_cluster_smem(a.stages, a.a_bytes, a.b_bytes, a.BN), c->stream);
+    cfg.numAttrs = g_dc_pdl ? 2 : 1;
     DC_CUDA(cudaLaunchKernelEx(&cfg, k_conv_cluster, tmA, tmB, a));
     return DC_OK;
 }

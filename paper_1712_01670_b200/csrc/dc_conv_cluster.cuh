@@ -12,7 +12,6 @@ struct dc_cluster_args {
     int Ho, Wo, Co, Ci, kh, kw, sh, sw, ph, pw, relu, tiles_x, tiles_y;
     int BN, NB, BK, kchunks, stages, a_bytes, b_bytes, nb_off, CS;
     uint32_t idesc, sbo, layout_type, tmem_cols;
-    int flat, gpr, n_groups_all;              // flat tiles, see dc_conv_bf16.cu
     int32_t* status;
     unsigned long long wait_ns;
     int skip_loads;
@@ -22,5 +21,7 @@ struct dc_cluster_args {
 };
 
 size_t dc_cluster_smem(int stages, int a_bytes, int b_bytes, int BN);
+// clusters of cs CTAs with that much shared memory that the device runs at the same time
+int dc_cluster_wave(int device, int cs, size_t smem);
 // tiles: length of the tile list (upper bound of the count on the device)
 int dc_launch_cluster_kernel(dc_cache* c, const CUtensorMap& tmA, const CUtensorMap& tmB, const dc_cluster_args& a, int tiles);

@@ -705,6 +705,51 @@ def test_conv_flat_tiles_across_rows_and_streams(scheme, hi, wi, cin, cout, k, s
     _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, scheme)
 
 
+@pytest.mark.parametrize("hi,wi,cin,cout,k,S,groups", [
+    (28, 28, 128, 256, 3, 2, 1),         # two chunks of 64 channels, CTA pairs too
+    (13, 13, 96, 64, 5, 3, 1),           # 32-channel steps, a half-empty last chunk
+    (17, 23, 96, 128, 5, 1, 2),          # 48 channels per group: 16-channel steps
+    (9, 40, 192, 32, 3, 1, 1),           # the narrowest channel block
+])
+def test_conv_schemes_agree_bit_for_bit(hi, wi, cin, cout, k, S, groups, monkeypatch):
+    """What a layer was timed with must not show in its output: all operand schemes but the clusters sum in one order."""
+    g = rng(hi + cin + k)
+    nb = nets.NetBuilder(hi, wi)
+    nb.conv(nb.conv(-1, cin, 1, 1, 0), cout, k, 1, k // 2, 1, groups=groups)
+    ws, bs = nets.random_weights(nb.layers, 7)
+    x = torch.from_numpy(g.normal(size=(S, hi, wi, cin)).astype(np.float32)).to(torch.bfloat16).cuda()
+    want, taken = None, set()
+    for scheme in range(1, 10):
+        monkeypatch.setenv("DC_CONV_SCHEME", str(scheme))
+        dc = DeepCache(wi, hi, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_BF16)
+        out = dc.conv_partial(1, x)
+        taken.add(B.dc_cache_layer_conv_scheme(dc.handle, 1))
+        want = out if want is None else want
+        assert torch.equal(out, want), f"scheme {scheme}"
+        dc.close()
+    assert len(taken) >= 6
+
+
+@pytest.mark.parametrize("net,S", [("resnet50", 1), ("resnet50", 4), ("alexnet", 1), ("alexnet_grouped", 3)])
+def test_caches_of_one_configuration_repeat_themselves(net, S):
+    """Three caches, each timing its kernels anew: the same maps at every layer, bit for bit."""
+    layers = nets.resnet50_trunk(224, 224) if net == "resnet50" else nets.alexnet_trunk(227, 227, grouped=net == "alexnet_grouped")
+    W = layers[0]["out_w"] * 2 if net == "resnet50" else 227
+    ws, bs = nets.random_weights(layers, 4)
+    g = rng(S)
+    frames = [torch.from_numpy(g.integers(0, 256, size=(S, W, W, 3), dtype=np.uint8)).cuda() for _ in range(2)]
+    frames[1][:, : W // 2] = frames[0][:, : W // 2]
+    maps = None
+    for _ in range(3):
+        dc = DeepCache(W, W, layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_BF16)
+        for f in frames:
+            dc.infer_frame(f)
+        got = [dc.layer_map(i) for i in range(len(layers))]
+        maps = maps or got
+        assert all(torch.equal(a, b) for a, b in zip(got, maps))
+        dc.close()
+
+
 def _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, scheme):
     g = rng(hi * 7 + cout)
     nb = nets.NetBuilder(hi, wi)
