@@ -528,7 +528,8 @@ int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch)
     const dim3 grid((unsigned)(c->S * L.d.out_h));
     const size_t smem = (size_t)((c->cfg.width * 3 + 15) / 16) * 16 * sizeof(uint16_t);
     if (smem > 48 * 1024 || (size_t)c->cfg.height > 255u * (size_t)L.d.out_h) return DC_ERR_CONFIG;   // 16-bit column sums
-    uint4* pad8 = c->resize_feeds >= 0 ? (uint4*)c->L[c->resize_feeds].in_padded : nullptr;
+    // the operand copy of the convolution that reads this resized frame (a table may hold resizes to other sizes too)
+    uint4* pad8 = c->resize_feeds >= 0 && c->L[c->resize_feeds].d.in0 == layer ? (uint4*)c->L[c->resize_feeds].in_padded : nullptr;
     dc_prof_scope ps(c, DC_ST_INPUT);
     DISPATCH(c,
         DC_CUDA(dc_launch_pdl(k_resize_area<float>, grid, 256, smem, c->stream, frame, pitch, c->cfg.width, c->cfg.height, c->S, L.d.out_w, L.d.out_h, (float*)L.map[0], (uint4*)nullptr)),

@@ -519,6 +519,20 @@ def test_conv_schemes_forced(scheme, monkeypatch):
 
 
 # ------------------------------------------------------------------ dc_infer_frame
+@pytest.mark.parametrize("first,second", [((60, 70), (24, 30)), ((24, 30), (60, 70))])
+def test_infer_with_two_resized_inputs(first, second):
+    """Two area resizes to different sizes, each read by a convolution over three channels: a resize fills the operand
+    copy of its own reader only."""
+    b = nets.NetBuilder(80, 96)
+    for h, w in (first, second):
+        b.conv(b.resize_area(-1, h, w), 64, 3, 1, 1)
+    w = configs.small_cnn_stream()
+    w.layers, w.dtype, w.width, w.height = b.layers, configs.DTYPE_BF16, 96, 80
+    inner = w.make_streams
+    w.make_streams = lambda s, f, first=0: _cropped(inner(s, f), 80, 96)
+    U.run_stream_parity(w, 2, [0, 1, 2])
+
+
 def test_infer_workload_1():
     U.run_stream_parity(configs.WORKLOADS[1](), 1, [0, 1])
 
