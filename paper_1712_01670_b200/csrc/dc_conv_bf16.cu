@@ -1252,6 +1252,22 @@ bool dc_conv_takes_frame(const dc_cache* c, int layer)
     return L.s2d_s ? L.s2d_cin == 3 : n_groups(L.d) == 1 && L.d.cin == 3 && smallc_ok(L.d) && !make_plan(L.d, p) && L.in_padded != nullptr;
 }
 
+// The weights of the patch, slab and pair kernels are packed by channel blocks, so another block width needs another packing
+// (of the same size).  Happens while the tuner tries widths, and once more for its final choice before the cache is ready; a
+// launch that finds the packing changed under it (`changed`) must not read the weights ahead of its turn.
+static int pack_halo(dc_cache* c, dc_layer_rt& L, int bn, bool* changed)
+{
+    *changed = L.halo_bn != bn;
+    if (!*changed) return DC_OK;
+    const int taps = L.d.kh * L.d.kw, cin = L.d.cin / n_groups(L.d);
+    const size_t n = (size_t)L.d.cout * taps * ((cin + 63) / 64) * 64;
+    int grid = (int)((n + 255) / 256); if (grid > c->num_sms * 8) grid = c->num_sms * 8;
+    k_pack_halo<<<grid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, L.d.cout, taps, cin, bn, (__nv_bfloat16*)L.weight_halo);
+    DC_CUDA(cudaGetLastError());
+    L.halo_bn = bn;
+    return DC_OK;
+}
+
 // Normal layers need no repacking ([cout][kh][kw][cin] is already K-major); few-channel layers
 // get their tap-major packed copy and a buffer for the channel-padded input.
 int dc_pack_weights_bf16(dc_cache* c, int layer)
@@ -1265,11 +1281,9 @@ int dc_pack_weights_bf16(dc_cache* c, int layer)
         const size_t n = (size_t)L.d.cout * L.d.kh * L.d.kw * h.kchunks * 64;
         DC_CUDA(cudaMalloc(&L.weight_halo, n * 2));
         c->bytes += n * 2;
-        int grid = (int)((n + 255) / 256); if (grid > c->num_sms * 8) grid = c->num_sms * 8;
-        k_pack_halo<<<grid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, L.d.cout, L.d.kh * L.d.kw, dg.cin, h.BN,
-                                                 (__nv_bfloat16*)L.weight_halo);
-        L.halo_bn = h.BN;
-        DC_CUDA(cudaGetLastError());
+        bool changed;
+        const int rc = pack_halo(c, L, h.BN, &changed);
+        if (rc != DC_OK) return rc;
     }
     if (n_groups(L.d) > 1) return DC_OK;                          // grouped layers use the kernels above only
     if (pad16_ok(L.d)) {
@@ -1368,15 +1382,9 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     HaloPlan h;
     EncodeTiledFn enc = encode_fn();
     if (!enc || !L.weight_halo || !halo_ok(d, h, L.tc_bn)) return DC_ERR_CONFIG;
-    if (L.halo_bn != h.BN) {
-        // the packed weights are grouped by channel block: another block width needs another packing (same size).
-        // Happens while the tuner tries widths and once more for its final choice, never in steady state.
-        const size_t n = (size_t)cout_all * d.kh * d.kw * h.kchunks * 64;
-        int pgrid = (int)((n + 255) / 256); if (pgrid > c->num_sms * 8) pgrid = c->num_sms * 8;
-        k_pack_halo<<<pgrid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, cout_all, d.kh * d.kw, d.cin, h.BN,
-                                                  (__nv_bfloat16*)L.weight_halo);
-        L.halo_bn = h.BN;
-    }
+    bool repacked;
+    const int prc = pack_halo(c, L, h.BN, &repacked);
+    if (prc != DC_OK) return prc;
     in = (const uint8_t*)in + (size_t)grp * d.cin * 2;            // the group's first input channel
     bool hit;
     CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, slab ? 5 : 3, 0, &hit);
@@ -1404,7 +1412,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     a.a_bytes = 0; a.b_bytes = h.b_bytes; a.sbo = 128; a.layout_type = 0;
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(h.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.status = c->status;
-    a.early = dc_lists_settled(c);
+    a.early = repacked ? 0 : dc_lists_settled(c);                  // the producer sends for its first weights early
     set_wait_limit(c, a);
     ha.wpacked = (const __nv_bfloat16*)L.weight_halo;
     ha.k_last = h.k_last;
@@ -1467,12 +1475,9 @@ static int launch_pair(dc_cache* c, int layer, const void* in, void* out, const 
     HaloPlan h;
     if (!enc || !L.weight_halo || !pair_ok(d, bn) || !halo_ok(d, h)) return DC_ERR_CONFIG;
     const int half = bn / 2, taps = d.kh * d.kw, kchunks = h.kchunks;
-    if (L.halo_bn != half) {                                     // weights grouped by half blocks: [2 NB][taps][kchunks][half][64]
-        const size_t n = (size_t)d.cout * taps * kchunks * 64;
-        int pgrid = (int)((n + 255) / 256); if (pgrid > c->num_sms * 8) pgrid = c->num_sms * 8;
-        k_pack_halo<<<pgrid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, d.cout, taps, d.cin, half, (__nv_bfloat16*)L.weight_halo);
-        L.halo_bn = half;
-    }
+    bool repacked;                                               // weights grouped by half blocks: [2 NB][taps][kchunks][half][64], read after the wait
+    const int prc = pack_halo(c, L, half, &repacked);
+    if (prc != DC_OK) return prc;
     const int PH = DC_TILE_H + d.kh - 1;
     bool hit_a, hit_b;
     CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, 5, 0, &hit_a);     // the column-slab map of the single-CTA kernel
@@ -1845,6 +1850,11 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     }
     L.tc_mt = best_mt; L.tc_bn = best_bn; L.tc_ctas = best_ctas; L.flat = best_flat; L.tc_ew = best_ew; L.tc_cs = best_cs;
     cudaEventDestroy(e0); cudaEventDestroy(e1);
+    if (L.tc_mt >= 3 && L.tc_cs == 0) {                               // packed for the choice before any frame is launched
+        bool changed;
+        const int rc = pack_halo(c, L, L.tc_mt == 7 ? L.tc_bn / 2 : L.tc_bn, &changed);
+        if (rc != DC_OK) return rc;
+    }
     c->launches = 0; c->list_mark = DC_LISTS_FRESH;
     if (verbose) fprintf(stderr, "libdeepcache: layer %d: chose code %d, %d channels per block, %d CTA(s) per SM, %d epilogue warps, clusters of %d (%.4f ms)\n",
                          layer, best_flat ? best_mt + 7 : best_mt, best_bn, best_ctas, best_ew, best_cs, best / kTuneReps);

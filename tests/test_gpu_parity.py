@@ -764,6 +764,25 @@ def test_caches_of_one_configuration_repeat_themselves(net, S):
         dc.close()
 
 
+def test_first_frame_of_a_cache_reads_the_weights_of_its_choice():
+    """The tuner packs weights for the widths it tries; the first frame, launched at once, must find the final packing: the
+    same maps as the same frame given to the warm cache."""
+    b = nets.NetBuilder(57, 57)
+    x = b.conv(-1, 64, 3, 1, 1)
+    for cout in (128, 128, 256, 256):
+        x = b.conv(x, cout, 3, 1, 1)
+    ws, bs = nets.random_weights(b.layers, 12)
+    f = torch.from_numpy(rng(8).integers(0, 256, size=(16, 57, 57, 3), dtype=np.uint8)).cuda()
+    for _ in range(8):
+        dc = DeepCache(57, 57, b.layers, ws, bs, n_streams=16, block=16, search_range=4, dtype=B.DC_BF16)
+        dc.infer_frame(f, want_out=False)
+        first = [dc.layer_map(i) for i in range(len(b.layers))]
+        dc.reset()
+        dc.infer_frame(f, want_out=False)
+        assert all(torch.equal(a, dc.layer_map(i)) for i, a in enumerate(first))
+        dc.close()
+
+
 def _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, scheme):
     g = rng(hi * 7 + cout)
     nb = nets.NetBuilder(hi, wi)
