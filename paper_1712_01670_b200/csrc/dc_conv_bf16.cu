@@ -1865,6 +1865,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
 // tensor-core convolution launch of this cache issues none of its operand copies and bounds its waits by wait_ms
 // instead of 2 s: the MMA and epilogue roles find nothing arriving, give up, record DC_ERR_TIMEOUT in the status
 // word, free their tensor memory and the kernel returns normally.  No copy and no MMA is in flight when they leave.
+// (Cluster kernel: one CTA of each cluster issues none; the others finish their part and store nothing.)
 // The launch after it is an ordinary one.
 extern "C" int dc_debug_stall_next_conv(dc_cache* c, int wait_ms)
 {

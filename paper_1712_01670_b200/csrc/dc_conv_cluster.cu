@@ -31,6 +31,12 @@ __device__ __forceinline__ bool cl_wait(uint32_t bar, uint32_t parity, CtlCl* ct
 {
     return mbar_wait_at(bar, parity, &ctl->abort_flag, &ctl->wait_ns, status);
 }
+// Leaves word of an abort in every CTA of the cluster (after the first cluster barrier, before the second).
+__device__ __forceinline__ void abort_cluster(const CtlCl* ctl, int cs)
+{
+    for (int r = 0; r < cs; ++r)
+        asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(map_to_cta((const void*)&ctl->abort_flag, (uint32_t)r)), "r"(1) : "memory");
+}
 __device__ __forceinline__ void st_remote(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
@@ -49,6 +55,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
     const int rank = (int)cluster_rank(), item = blockIdx.x / a.CS, nb = item % a.NB, idx = item / a.NB;
     const int kiters = a.kh * a.kw * a.kchunks;
     const int k0 = rank * kiters / a.CS, nk = (rank + 1) * kiters / a.CS - k0;
+    const bool skip_loads = a.skip_loads && rank == 0;           // failure-detection tests: one CTA of the cluster gets no operands
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < a.stages; ++i) { mbar_init(&ctl->full[i], 2); mbar_init(&ctl->empty[i], 1); }   // weights and pixels arrive apart
@@ -75,7 +82,7 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         mbar_expect_tx(full0 + off, (uint32_t)a.b_bytes);
         tma_load_2d(slot + a.a_bytes, &tmB, tap * a.Ci + cc * a.BK, w_row, full0 + off);
     };
-    if (warp == 0 && !a.skip_loads && elect_one()) {
+    if (warp == 0 && !skip_loads && elect_one()) {
         int tap = tap0, cc = cc0;
         for (int it = 0; it < early; ++it) {
             load_weights(tap, cc, 8u * it, ring0 + it * stage_bytes);
@@ -120,9 +127,9 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         bool ok = true;
         if (!present) {
             // the weights are on their way: let them land before this CTA's shared memory is given up
-            if (lane == 0 && !a.skip_loads)
+            if (lane == 0 && !skip_loads)
                 for (int it = 0; it < early && ok; ++it) { mbar_arrive(&ctl->full[it]); ok = cl_wait(full0 + 8u * it, 0, ctl, a.status); }
-        } else if (!a.skip_loads) {
+        } else if (!skip_loads) {
             if (elect_one()) {
                 const int fx = tx * DC_TILE_W * a.sw - a.pw, fy = ty * DC_TILE_H * a.sh - a.ph;
                 RingPos r;
@@ -184,8 +191,10 @@ __global__ void __launch_bounds__(kThreadsCl, 1) k_conv_cluster(const __grid_con
         tc_fence_before();
     }
     if (warp < 2 || !present) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // (the accumulator warps have waited)
+    // a CTA that gave up has not sent its sums: no CTA of the cluster stores anything then
+    if (ctl->abort_flag != 0) abort_cluster(ctl, a.CS);
     cluster_sync_all();                      // this CTA's pixels have arrived from every CTA
-    const bool dead = ctl->abort_flag != 0;  // an aborted launch's sums are not valid: nothing is stored
+    const bool dead = ctl->abort_flag != 0;
     if (!dead) {
         // ---------------- this CTA's pixels: sums from all ranks, bias, ReLU, bf16, store ----------------
         for (int u = threadIdx.x; u < units; u += kThreadsCl) {

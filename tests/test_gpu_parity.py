@@ -925,6 +925,32 @@ def test_bounded_device_waits_run_out_and_the_cache_stays_usable(cin, k, monkeyp
         dc.close()
 
 
+def test_a_cluster_with_one_stalled_cta_stores_nothing(monkeypatch):
+    """One CTA of every cluster gets no operands and gives up: the others have only a part of the sums and must not store
+    it.  The next launch is correct."""
+    import ctypes
+    monkeypatch.setenv("DC_CONV_SCHEME", "10")
+    g = rng(17)
+    nb = nets.NetBuilder(13, 13)
+    nb.conv(nb.conv(-1, 256, 1, 1, 0), 128, 3, 1, 1, 1)
+    ws, bs = nets.random_weights(nb.layers, 3)
+    x = torch.from_numpy(g.normal(size=(2, 13, 13, 256)).astype(np.float32)).to(torch.bfloat16).cuda()
+    dc = DeepCache(13, 13, nb.layers, ws, bs, n_streams=2, block=16, search_range=4, dtype=B.DC_BF16)
+    try:
+        assert B.dc_cache_layer_conv_scheme(dc.handle, 1) == 10
+        stall = B.load().dc_debug_stall_next_conv
+        stall.restype, stall.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]
+        want = dc.conv_partial(1, x)
+        assert want.any()
+        assert stall(dc.handle, 5) == B.DC_OK
+        out = dc.conv_partial(1, x)                                # into a map of zeros
+        assert dc.status() == B.DC_ERR_TIMEOUT and not out.any()
+        dc.reset()
+        assert torch.equal(dc.conv_partial(1, x), want) and dc.status() == B.DC_OK
+    finally:
+        dc.close()
+
+
 def test_lookahead_gives_identical_results():
     """dc_lookahead_frame moves the matching of frame t+1 beside the inference of frame t; outputs, motion
     vectors and rectangles must not change.  Also: a lookahead for a frame that is then not used.
