@@ -158,8 +158,8 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     DC_TRY(dc_build_propagate_table(c, layers));
     DC_TRY(dev_alloc(c, &c->dirty_count, (size_t)n));
     DC_TRY(dev_alloc(c, &c->all_count, (size_t)n * 2));
-    DC_TRY(dev_alloc(c, &c->partial, (size_t)S + 2));
-    DC_CUDA(cudaMemsetAsync(c->partial, 0, sizeof(int32_t) * (S + 2), c->stream));
+    DC_TRY(dev_alloc(c, &c->partial, (size_t)S + 3));
+    DC_CUDA(cudaMemsetAsync(c->partial, 0, sizeof(int32_t) * (S + 3), c->stream));
     DC_TRY(dev_alloc(c, &c->reuse_px, (size_t)n * S * 2));
     c->alive = c->reuse_px + (size_t)n * S;
     DC_TRY(dev_alloc(c, &c->status, (size_t)1));
@@ -444,10 +444,9 @@ int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* 
     const int tiles = dc_layer_tiles(c, L);
     if (regions_dev || n_regions_dev) {
         if (!regions_dev || !n_regions_dev || !prev_out_dev || prev_out_dev == out_map_dev) return DC_ERR_ARG;
-        int32_t* count = c->partial + c->partial_cur;
-        c->partial_cur ^= 1;
-        DC_TRY(dc_launch_classify_copy(c, layer, regions_dev, n_regions_dev, prev_out_dev, out_map_dev, count, c->partial + 2, c->partial + c->partial_cur));
-        return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.dirty_list, count, L.masks, tiles);
+        DC_TRY(dc_launch_classify_copy(c, layer, regions_dev, n_regions_dev, prev_out_dev, out_map_dev, c->partial + 2, c->partial + 3,
+                                       (unsigned long long*)c->partial));
+        return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.dirty_list, c->partial + 2, L.masks, tiles);
     }
     return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.all_list, dc_all_count(c, layer), c->zero_masks, tiles);
 }

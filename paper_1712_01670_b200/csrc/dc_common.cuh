@@ -126,8 +126,7 @@ struct dc_cache {
     int prop_slots;                 // rectangles a thread of region propagation keeps for later layers
     void* prop_table;               // [n_layers] the layer table as region propagation reads it (dc_regions.cu)
     int32_t* dirty_count;           // [n_layers]
-    int32_t* partial;               // dc_conv_partial: two dirty counters used in turn (each call zeroes the other), then [S] reused pixels (not read)
-    int partial_cur;
+    int32_t* partial;               // dc_conv_partial: a running 64-bit counter (zero between launches), dirty tiles, [S] reused pixels (not read)
     int32_t* all_count;             // [n_layers]
     int32_t* reuse_px;              // [n_layers][S]
     int32_t* alive;                 // [n_layers][S] rectangles not yet eroded away
@@ -210,7 +209,7 @@ void dc_use_match_set(dc_cache* c, int k);
 int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers);
 int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out);
 int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, const int32_t* n_regions,
-                            const void* prev_out, void* out, int32_t* count, int32_t* px, int32_t* zero_next);
+                            const void* prev_out, void* out, int32_t* count, int32_t* px, unsigned long long* running);
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                    const int32_t* tile_count, const uint32_t* masks, int max_tiles);
 // stride-1 layers and single output pixels on CUDA cores (dc_conv_simt.cu)

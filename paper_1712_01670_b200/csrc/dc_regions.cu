@@ -221,8 +221,24 @@ struct ClassifyArgs {
     unsigned long long* reused_total;
     int32_t* status;                             // device status word
     int parts;                                   // warps that share a tile's copies (each tests the rectangles, the first one records the outcome)
-    int32_t* zero_next;                          // a counter that this launch zeroes for a later one, or NULL
+    // A caller's launch counts by itself, whatever ran before it (it may be a node of a graph that is launched many times): the
+    // running counter holds finished tiles above dirty ones, the last tile moves the sum to dirty_count and leaves zero.  (A
+    // ticket per CTA in an atomic of its own behind the count: 2 us longer.)  Else NULL: dirty_count was zeroed by the frame's
+    // region propagation and counts directly.
+    unsigned long long* running;
 };
+
+__device__ __forceinline__ void record_tile(const ClassifyArgs& a, int tile, bool dirty)
+{
+    if (!a.running) {
+        if (dirty) a.dirty_list[atomicAdd(a.dirty_count, 1)] = tile;
+        return;
+    }
+    const unsigned long long before = atomicAdd(a.running, (1ull << 32) | (dirty ? 1u : 0u));
+    const int slot = (int)(uint32_t)before;
+    if (dirty) a.dirty_list[slot] = tile;
+    if ((int)(before >> 32) == a.n_tiles - 1) { *a.dirty_count = slot + (dirty ? 1 : 0); *a.running = 0; }
+}
 
 __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int tile, const int part, const int lane, CopyLane& cl)
 {
@@ -319,10 +335,7 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
         int covered = __popc(m0) + __popc(m1) + __popc(m2) + __popc(m3);
         int in_tile = (X1 - X0) * (Y1 - Y0);
         if (covered) { atomicAdd(&a.reuse_px[s], covered); atomicAdd(a.reused_total, (unsigned long long)covered); }
-        if (covered < in_tile) {
-            int slot = atomicAdd(a.dirty_count, 1);
-            a.dirty_list[slot] = tile;
-        }
+        record_tile(a, tile, covered < in_tile);
     }
 }
 
@@ -426,10 +439,7 @@ __device__ __forceinline__ void classify_tile_flat(const ClassifyArgs& a, const 
     if (lane == 0 && part == 0) {
         uint32_t* mk = a.masks + (size_t)tile * 4;
         mk[0] = m0; mk[1] = m1; mk[2] = m2; mk[3] = m3;
-        if (__popc(m0) + __popc(m1) + __popc(m2) + __popc(m3) < in_tile) {
-            const int slot = atomicAdd(a.dirty_count, 1);
-            a.dirty_list[slot] = tile;
-        }
+        record_tile(a, tile, __popc(m0) + __popc(m1) + __popc(m2) + __popc(m3) < in_tile);
     }
 }
 
@@ -453,7 +463,6 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy(ClassifyArgs 
     CopyLane cl = copy_lane_setup(copy_smem);
     dc_pdl_wait();
     dc_pdl_release();
-    if (a.zero_next && blockIdx.x == 0 && threadIdx.x == 0) *a.zero_next = 0;
     const int w = blockIdx.x * kCopyWarps + (threadIdx.x >> 5), tile = w / a.parts, part = w - tile * a.parts;
     if (tile < a.n_tiles) {
         if (a.gpr > 0) classify_tile_flat(a, tile, part, threadIdx.x & 31, cl);
@@ -494,7 +503,7 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
     a.gpr = L.gpr; a.n_tiles = 0;
     a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = L.dirty_count; a.reuse_px = L.reuse_px;
     a.alive = L.alive; a.reused_total = L.reused_total; a.status = L.status;
-    a.parts = L.parts; a.zero_next = nullptr;
+    a.parts = L.parts; a.running = nullptr;
     const int u = w - L.first_warp, tile = u / a.parts, part = u - tile * a.parts;
     if (a.gpr > 0) classify_tile_flat(a, tile, part, threadIdx.x & 31, cl);
     else classify_tile(a, tile, part, threadIdx.x & 31, cl);
@@ -618,10 +627,10 @@ int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, i
     return DC_OK;
 }
 
-// count, px: where the dirty tiles and the reused pixels per stream are counted; count is zero when the kernel starts.
-// zero_next: a counter that the kernel zeroes, or NULL.
+// count, px: where the dirty tiles and the reused pixels per stream are counted.  running: a counter that is zero between
+// launches, or NULL: count is zero when the kernel starts.
 int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, const int32_t* n_regions,
-                            const void* prev_out, void* out, int32_t* count, int32_t* px, int32_t* zero_next)
+                            const void* prev_out, void* out, int32_t* count, int32_t* px, unsigned long long* running)
 {
     dc_layer_rt& L = c->L[layer];
     ClassifyArgs a;
@@ -632,7 +641,7 @@ int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, co
     a.gpr = L.flat ? L.gpr : 0; a.n_tiles = dc_layer_tiles(c, L);
     a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = count;
     a.reuse_px = px;
-    a.zero_next = zero_next; a.parts = copy_parts(c, dc_layer_tiles(c, L), a.px_bytes);
+    a.running = running; a.parts = copy_parts(c, dc_layer_tiles(c, L), a.px_bytes);
     a.reused_total = c->reused_total + layer;
     a.status = c->status;
     a.alive = (regions == c->table + (size_t)layer * c->S * c->max_regions) ? c->alive + (size_t)layer * c->S : nullptr;

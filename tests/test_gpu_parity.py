@@ -498,6 +498,38 @@ def test_conv_partial_ignores_rectangles_outside_the_map():
         dc.close()
 
 
+@pytest.mark.parametrize("dtype", [B.DC_FP32, B.DC_BF16])
+def test_conv_partial_in_a_graph_launched_again(dtype):
+    """One dc_conv_partial captured and launched several times, other calls between: every launch counts its tiles from zero."""
+    S, hi, wi = 2, 50, 70
+    nb = nets.NetBuilder(hi, wi)
+    nb.conv(nb.conv(-1, 64, 1, 1, 0), 64, 3, 1, 1)
+    ws, bs = nets.random_weights(nb.layers, 9)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        dc = DeepCache(wi, hi, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=dtype, max_regions=4)
+        g = rng(31)
+        x, prev = (torch.from_numpy(g.normal(size=(S, hi, wi, 64)).astype(np.float32)).to(dc.tdtype).cuda() for _ in range(2))
+        regs = torch.tensor([[[3, 4, 40, 33, 5, 6]] + [[0] * 6] * 3, [[0, 0, 70, 50, 0, 0]] + [[0] * 6] * 3], dtype=torch.int32).cuda()
+        n = torch.tensor([1, 1], dtype=torch.int32).cuda()
+        want, other = dc.conv_partial(1, x, prev, regs, n), dc.conv_partial(1, prev, x, regs, n)
+        out = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        B.dc_conv_partial(dc.handle, 1, x, prev, regs, n, out)
+    with torch.cuda.stream(stream):
+        for k in range(5):
+            out.zero_()
+            graph.replay()
+            stream.synchronize()
+            assert torch.equal(out, want), f"launch {k}"
+            if k == 2:
+                assert torch.equal(dc.conv_partial(1, prev, x, regs, n), other)
+        assert dc.status() == B.DC_OK
+        dc.close()
+
+
 @pytest.mark.parametrize("scheme", [1, 2, 3, 4, 5, 6, 7, 8, 9])
 def test_conv_schemes_forced(scheme, monkeypatch):
     """Every operand scheme of the tensor-core convolution (tap by tap, patch, column slabs; one or two tiles per
