@@ -644,7 +644,7 @@ int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, co
     a.running = running; a.parts = copy_parts(c, dc_layer_tiles(c, L), a.px_bytes);
     a.reused_total = c->reused_total + layer;
     a.status = c->status;
-    a.alive = (regions == c->table + (size_t)layer * c->S * c->max_regions) ? c->alive + (size_t)layer * c->S : nullptr;
+    a.alive = running ? nullptr : c->alive + (size_t)layer * c->S;      // counted for the frame's rectangles alone, not for a caller's in the same table
     const int warps = dc_layer_tiles(c, L) * a.parts;
     static dc_once_per_device attr_set;
     if (attr_set.first(c->device))

@@ -9,7 +9,7 @@ import torch
 
 from oracle import deepcache_oracle as orc
 from paper_1712_01670_b200 import binding as B
-from paper_1712_01670_b200.engine import DeepCache
+from paper_1712_01670_b200.engine import DeepCache, device_view
 from paper_1712_01670_b200.synth import configs, nets
 
 import parity_util as U
@@ -494,6 +494,32 @@ def test_conv_partial_ignores_rectangles_outside_the_map():
         assert dc.status() == B.DC_ERR_ARG
         dc.reset()
         assert dc.status() == B.DC_OK
+    finally:
+        dc.close()
+
+
+def test_conv_partial_with_rectangles_where_propagation_left_them():
+    """dc_propagate_regions leaves a caller's rectangles in the cache's table (dc_cache_layer_regions): a convolution given
+    that table reuses them, although no rectangle of the last frame was left at the layer."""
+    S, hi, wi = 2, 48, 64
+    nb = nets.NetBuilder(hi, wi)
+    nb.conv(nb.conv(-1, 32, 3, 1, 1), 64, 3, 1, 1)
+    ws, bs = nets.random_weights(nb.layers, 9)
+    g = rng(41)
+    dc = DeepCache(wi, hi, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_FP32, max_regions=4)
+    try:
+        for _ in range(2):                                          # two frames of noise: nothing matches
+            _, st = dc.infer_frame(g.integers(0, 256, size=(S, hi, wi, 3), dtype=np.uint8), want_stats=True)
+        assert not st[0].refreshed and st[0].n_regions == 0
+        regs = torch.tensor([[[4, 4, 40, 33, 5, 6]] + [[0] * 6] * 3, [[0, 0, 64, 48, 0, 0]] + [[0] * 6] * 3], dtype=torch.int32).cuda()
+        n = torch.tensor([1, 1], dtype=torch.int32).cuda()
+        out, _ = dc.propagate_regions(regs, n)
+        x = torch.from_numpy(g.normal(size=(S, hi, wi, 32)).astype(np.float32)).cuda()
+        prev = torch.from_numpy(g.normal(size=(S, hi, wi, 64)).astype(np.float32)).cuda()
+        ptr, _ = B.dc_cache_layer_regions(dc.handle, 1)
+        table = device_view(ptr, (S, dc.max_regions, 6), torch.int32, dc.device)
+        assert torch.equal(table, out[1])
+        assert torch.equal(dc.conv_partial(1, x, prev, table, n), dc.conv_partial(1, x, prev, out[1].contiguous(), n))
     finally:
         dc.close()
 
