@@ -442,8 +442,13 @@ int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* 
     if (!c->executable || c->L[layer].d.kind != DC_CONV) return DC_ERR_CONFIG;
     dc_layer_rt& L = c->L[layer];
     const int tiles = dc_layer_tiles(c, L);
+    const uintptr_t in_at = (uintptr_t)in_map_dev, out_at = (uintptr_t)out_map_dev;
+    if (in_at % c->elt || out_at % c->elt) return DC_ERR_ARG;
+    // the tensor-core kernels store vectors, and their loads take the map from a 16-byte boundary (copies of few-channel maps: from any)
+    if (dc_conv_bf16_supported(c, layer) && (out_at % 16 || (in_at % 16 && L.d.cin % 16 == 0 && !L.s2d_s))) return DC_ERR_ARG;
     if (regions_dev || n_regions_dev) {
         if (!regions_dev || !n_regions_dev || !prev_out_dev || prev_out_dev == out_map_dev) return DC_ERR_ARG;
+        if ((uintptr_t)prev_out_dev % 16 || out_at % 16) return DC_ERR_ARG;      // the reuse copy is a bulk copy
         DC_TRY(dc_launch_classify_copy(c, layer, regions_dev, n_regions_dev, prev_out_dev, out_map_dev, c->partial + 2, c->partial + 3,
                                        (unsigned long long*)c->partial));
         return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.dirty_list, c->partial + 2, L.masks, tiles);

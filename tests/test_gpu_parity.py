@@ -498,6 +498,44 @@ def test_conv_partial_ignores_rectangles_outside_the_map():
         dc.close()
 
 
+@pytest.mark.parametrize("dtype,cin,cout,k", [(B.DC_FP32, 16, 32, 3), (B.DC_FP32, 8, 12, 1), (B.DC_FP32, 8, 20, 0), (B.DC_BF16, 24, 16, 3), (B.DC_BF16, 64, 64, 3)])
+def test_conv_partial_takes_maps_at_any_element(dtype, cin, cout, k):
+    """A caller's maps that start one element past an aligned address: the kernels that move vectors leave them to the one
+    that does not; where only those exist, and for the reuse copy, the call is refused before any launch."""
+    S, hi, wi = 2, 9, 11
+    nb = nets.NetBuilder(hi, wi)
+    a = nb.conv(-1, cin, 1, 1, 0)
+    nb.conv(a, cout, k, 1, k // 2, 1) if k else nb.fc(a, cout, relu=1)
+    ws, bs = nets.random_weights(nb.layers, 5)
+    dc = DeepCache(wi, hi, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=dtype, max_regions=4)
+    try:
+        shape = dc.out_shape(1)
+        x = torch.from_numpy(rng(cin).normal(size=(S, hi, wi, cin)).astype(np.float32)).to(dc.tdtype).cuda()
+        want = dc.conv_partial(1, x)
+        xs = torch.zeros(x.numel() + 8, dtype=dc.tdtype, device="cuda")[1:1 + x.numel()].view(x.shape)
+        xs.copy_(x)
+        out = torch.zeros(want.numel() + 8, dtype=dc.tdtype, device="cuda")[1:1 + want.numel()].view(shape)
+        regs, n = torch.zeros((S, 4, 6), dtype=torch.int32, device="cuda"), torch.zeros(S, dtype=torch.int32, device="cuda")
+        ok = torch.zeros_like(want)
+        if B.dc_cache_layer_conv_scheme(dc.handle, 1) > 0:
+            for i, o in ((x, out), (xs, ok)):
+                with pytest.raises(B.DeepCacheError) as e:
+                    B.dc_conv_partial(dc.handle, 1, i, None, None, None, o)
+                assert e.value.status == B.DC_ERR_ARG
+        else:
+            for i, o in ((xs, ok), (x, out), (xs, out)):
+                o.zero_()
+                B.dc_conv_partial(dc.handle, 1, i, None, None, None, o)
+                U.assert_map_close(o, want.float().cpu().numpy().astype(np.float64), dtype == B.DC_BF16, "unaligned")
+        for p_, o in ((want, out), (out, ok)):
+            with pytest.raises(B.DeepCacheError) as e:
+                B.dc_conv_partial(dc.handle, 1, x, p_, regs, n, o)
+            assert e.value.status == B.DC_ERR_ARG
+        assert dc.status() == B.DC_OK
+    finally:
+        dc.close()
+
+
 def test_conv_partial_with_rectangles_where_propagation_left_them():
     """dc_propagate_regions leaves a caller's rectangles in the cache's table (dc_cache_layer_regions): a convolution given
     that table reuses them, although no rectangle of the last frame was left at the layer."""
