@@ -347,6 +347,7 @@ int dc_cache_create(const dc_config* cfg, const dc_layer_desc* layers, int n_lay
     if (!c) return DC_ERR_ALLOC;
     memset((void*)c, 0, sizeof(*c));
     c->list_mark = DC_LISTS_FRESH;
+    c->piece = 0x7fffffff;
     c->cfg = *cfg; c->n_layers = n_layers; c->stream = (cudaStream_t)cuda_stream;
     c->S = cfg->n_streams;
     c->Gx = dc_div_up(cfg->width, cfg->block); c->Gy = dc_div_up(cfg->height, cfg->block);
@@ -735,6 +736,15 @@ int dc_get_status(dc_cache* c, int32_t* status_host)
     if (!c || !status_host) return DC_ERR_ARG;
     DC_CUDA(cudaStreamSynchronize(c->stream));
     DC_CUDA(cudaMemcpy(status_host, c->status, sizeof(int32_t), cudaMemcpyDeviceToHost));
+    return DC_OK;
+}
+
+// Not part of the public header: tests declare it themselves.  Launches of this cache take at most `items` items, so that the
+// pieces of maps beyond 2^31 items run on small ones.
+int dc_debug_piece(dc_cache* c, int items)
+{
+    if (!c || items < 1) return DC_ERR_ARG;
+    c->piece = (size_t)items;
     return DC_OK;
 }
 

@@ -105,6 +105,7 @@ struct dc_cache {
     size_t key_pitch;
     int num_sms;
     int device;                     // ordinal of the device the cache lives on
+    size_t piece;                   // most items of a launch whose kernel indexes with 32 bits: larger maps are launched in pieces (tests lower it)
     int debug_stall_ms;             // > 0: the next tensor-core convolution launch is made to time out (tests)
     uint8_t* staging[2];            // device copies of host frames for dc_infer_frame_host (one in use, one prefetching)
     cudaStream_t copy_stream;       // dc_prefetch_frame_host copies on its own stream

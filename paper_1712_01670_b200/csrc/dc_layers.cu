@@ -486,21 +486,24 @@ inline int grid_for(const dc_cache* c, size_t n, int block)
 
 #define DISPATCH(c, expr_f32, expr_bf16) do { if ((c)->cfg.dtype == DC_BF16) { expr_bf16; } else { expr_f32; } } while (0)
 
-namespace {
-constexpr size_t k32Bit = 0x7fffffffull;                       // the vector kernels index with 32 bits
-}
+// The vector kernels index with 32 bits: a launch takes at most c->piece items (2^31 - 1), and a larger map several launches, cut
+// between `units` (rows or streams) of `each` items.  units_per_piece: 0 when a single unit is too large.
+static size_t units_per_piece(const dc_cache* c, size_t each) { return c->piece / (each ? each : 1); }
 
 int dc_launch_input_map(dc_cache* c, const uint8_t* frame, size_t pitch)
 {
     const int row = c->cfg.width * 3, words = (row + 3) / 4;
-    const size_t n = (size_t)c->S * c->cfg.height * words;
-    if (n > k32Bit) return DC_ERR_CONFIG;                       // 8 GB of pixels
-    const dim3 grid((unsigned)grid_for(c, n, 256));
+    const size_t rows = (size_t)c->S * c->cfg.height, per = units_per_piece(c, words);
+    if (per == 0) return DC_ERR_CONFIG;                          // one row of 8 GB
     dc_prof_scope ps(c, DC_ST_INPUT);
-    DISPATCH(c,
-        DC_CUDA(dc_launch_pdl(k_input_map<float>, grid, 256, 0, c->stream, frame, pitch, row, words, (unsigned)n, (float*)c->input_map)),
-        DC_CUDA(dc_launch_pdl(k_input_map<__nv_bfloat16>, grid, 256, 0, c->stream, frame, pitch, row, words, (unsigned)n, (__nv_bfloat16*)c->input_map)));
-    c->launches += 1;
+    for (size_t r = 0; r < rows; r += per) {
+        const size_t n = (rows - r < per ? rows - r : per) * words;
+        const dim3 grid((unsigned)grid_for(c, n, 256));
+        DISPATCH(c,
+            DC_CUDA(dc_launch_pdl(k_input_map<float>, grid, 256, 0, c->stream, frame + r * pitch, pitch, row, words, (unsigned)n, (float*)c->input_map + r * row)),
+            DC_CUDA(dc_launch_pdl(k_input_map<__nv_bfloat16>, grid, 256, 0, c->stream, frame + r * pitch, pitch, row, words, (unsigned)n, (__nv_bfloat16*)c->input_map + r * row)));
+        c->launches += 1;
+    }
     return DC_OK;
 }
 
@@ -514,11 +517,17 @@ int dc_launch_frame_operand(dc_cache* c, int layer, const uint8_t* frame, size_t
         const int rows = c->S * L.in_h, parts = dc_div_up(L.s2d_ws * chunks, 128), most = dc_div_up(c->num_sms * 16, parts);
         DC_CUDA(dc_launch_pdl(k_frame_s2d, dim3((unsigned)(rows < most ? rows : most), (unsigned)parts), 128, 0, c->stream, frame, pitch, L.s2d_wi, L.s2d_hi, L.s2d_s, L.s2d_py, L.s2d_px, L.in_h, L.s2d_ws,
                               chunks, rows, (uint4*)L.in_s2d));
+        c->launches += 1;
     } else {
-        const size_t n = (size_t)c->S * L.in_h * L.in_w;
-        DC_CUDA(dc_launch_pdl(k_frame_pad8, dim3((unsigned)grid_for(c, n, 256)), 256, 0, c->stream, frame, pitch, L.in_w, (unsigned)n, (uint4*)L.in_padded));
+        const size_t rows = (size_t)c->S * L.in_h, per = units_per_piece(c, L.in_w);
+        if (per == 0) return DC_ERR_CONFIG;
+        for (size_t r = 0; r < rows; r += per) {
+            const size_t n = (rows - r < per ? rows - r : per) * L.in_w;
+            DC_CUDA(dc_launch_pdl(k_frame_pad8, dim3((unsigned)grid_for(c, n, 256)), 256, 0, c->stream, frame + r * pitch, pitch, L.in_w, (unsigned)n,
+                                  (uint4*)L.in_padded + r * L.in_w));
+            c->launches += 1;
+        }
     }
-    c->launches += 1;
     return DC_OK;
 }
 
@@ -541,25 +550,32 @@ int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch)
 int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks)
 {
     dc_layer_rt& L = c->L[layer];
-    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout, nv = n * c->elt / 16;
+    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
+    const bool vec = (L.d.cout * c->elt) % 16 == 0;
+    const int cv = L.d.cout * c->elt / 16;
+    const size_t out1 = (size_t)L.d.out_h * L.d.out_w * cv, in1 = (size_t)L.in_h * L.in_w * cv, per = vec ? units_per_piece(c, out1) : 0;   // of one stream
     dc_prof_scope ps(c, DC_ST_POINTWISE);
-    c->launches += 1;
-    if ((L.d.cout * c->elt) % 16 == 0 && nv < k32Bit) {
-        const int cv = L.d.cout * c->elt / 16;
+    for (size_t s0 = 0; per > 0; s0 += per) {
+        const size_t nv = ((size_t)c->S - s0 < per ? (size_t)c->S - s0 : per) * out1;
+        const uint4* from = (const uint4*)in + s0 * in1;
+        uint4* to = (uint4*)out + s0 * out1;
+        const uint32_t* bits = masks ? masks + s0 * L.tiles_x * L.tiles_y * 4 : nullptr;
         const dim3 grid((unsigned)grid_for(c, nv, 256));
         if (!masks && L.d.kh == 2 && L.d.kw == 2 && L.d.sh == 2 && L.d.sw == 2 && L.d.ph == 0 && L.d.pw == 0 && 2 * L.d.out_h <= L.in_h && 2 * L.d.out_w <= L.in_w) {
             DISPATCH(c,
-                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<float>, grid, 256, 0, c->stream, (const uint4*)in, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, (uint4*)out)),
-                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)in, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, (uint4*)out)));
-            return DC_OK;
-        }
-#define DC_POOL(T, K) DC_CUDA(dc_launch_pdl(k_maxpool_vec<T, K>, grid, 256, 0, c->stream, (const uint4*)in, L.in_h, L.in_w, (unsigned)cv, L.d, (unsigned)nv, (uint4*)out, masks, L.tiles_x, L.tiles_y))
-        if (L.d.kh == 3 && L.d.kw == 3) DISPATCH(c, DC_POOL(float, 3), DC_POOL(__nv_bfloat16, 3));
-        else if (L.d.kh == 2 && L.d.kw == 2) DISPATCH(c, DC_POOL(float, 2), DC_POOL(__nv_bfloat16, 2));
-        else DISPATCH(c, DC_POOL(float, 0), DC_POOL(__nv_bfloat16, 0));
+                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<float>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, to)),
+                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<__nv_bfloat16>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, to)));
+        } else {
+#define DC_POOL(T, K) DC_CUDA(dc_launch_pdl(k_maxpool_vec<T, K>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, (unsigned)cv, L.d, (unsigned)nv, to, bits, L.tiles_x, L.tiles_y))
+            if (L.d.kh == 3 && L.d.kw == 3) DISPATCH(c, DC_POOL(float, 3), DC_POOL(__nv_bfloat16, 3));
+            else if (L.d.kh == 2 && L.d.kw == 2) DISPATCH(c, DC_POOL(float, 2), DC_POOL(__nv_bfloat16, 2));
+            else DISPATCH(c, DC_POOL(float, 0), DC_POOL(__nv_bfloat16, 0));
 #undef DC_POOL
-        return DC_OK;
+        }
+        c->launches += 1;
+        if (s0 + per >= (size_t)c->S) return DC_OK;
     }
+    c->launches += 1;
     if (masks) return DC_ERR_STATE;                             // cached pooling needs 16-byte pixels (checked at creation)
     const dim3 grid((unsigned)grid_for(c, n, 256));
     DISPATCH(c,
@@ -613,22 +629,27 @@ int dc_launch_relu(dc_cache* c, int layer, const void* a)
 int dc_launch_lrn(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks)
 {
     dc_layer_rt& L = c->L[layer];
-    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout, nv = n * c->elt / 16;
+    const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
     const int r = L.d.ph, win = 2 * r + 1;
     const bool defaults = c->cfg.lrn_alpha == 0.0 && c->cfg.lrn_beta == 0.0 && c->cfg.lrn_k == 0.0;
     const float alpha = (float)(defaults ? 1e-4 : c->cfg.lrn_alpha), beta = (float)(defaults ? 0.75 : c->cfg.lrn_beta);
     const float kappa = (float)(defaults ? 1.0 : c->cfg.lrn_k), an = alpha / (win * win);
     dc_prof_scope ps(c, DC_ST_POINTWISE);
-    c->launches += 1;
-    if ((L.d.cout * c->elt) % 16 == 0 && nv < k32Bit && (r == 1 || r == 2)) {
+    const unsigned cv = (unsigned)(L.d.cout * c->elt / 16);
+    const size_t each = (size_t)L.d.out_h * L.d.out_w * cv;                  // of one stream
+    const size_t per = (L.d.cout * c->elt) % 16 == 0 && (r == 1 || r == 2) ? units_per_piece(c, each) : 0;
+    for (size_t s0 = 0; per > 0; s0 += per) {
+        const size_t nv = ((size_t)c->S - s0 < per ? (size_t)c->S - s0 : per) * each;
         const dim3 grid((unsigned)grid_for(c, nv, 256));
-        const unsigned cv = (unsigned)(L.d.cout * c->elt / 16);
-#define DC_LRN_VEC(T, R) DC_CUDA(dc_launch_pdl(k_lrn_vec<T, R>, grid, 256, 0, c->stream, (const uint4*)in, L.d.out_h, L.d.out_w, cv, an, beta, kappa, (unsigned)nv, (uint4*)out, masks, L.tiles_x, L.tiles_y))
+        const uint32_t* bits = masks ? masks + s0 * L.tiles_x * L.tiles_y * 4 : nullptr;
+#define DC_LRN_VEC(T, R) DC_CUDA(dc_launch_pdl(k_lrn_vec<T, R>, grid, 256, 0, c->stream, (const uint4*)in + s0 * each, L.d.out_h, L.d.out_w, cv, an, beta, kappa, (unsigned)nv, (uint4*)out + s0 * each, bits, L.tiles_x, L.tiles_y))
         if (r == 1) DISPATCH(c, DC_LRN_VEC(float, 1), DC_LRN_VEC(__nv_bfloat16, 1));
         else DISPATCH(c, DC_LRN_VEC(float, 2), DC_LRN_VEC(__nv_bfloat16, 2));
 #undef DC_LRN_VEC
-        return DC_OK;
+        c->launches += 1;
+        if (s0 + per >= (size_t)c->S) return DC_OK;
     }
+    c->launches += 1;
     const dim3 grid((unsigned)grid_for(c, n, 256));
     DISPATCH(c,
         DC_CUDA(dc_launch_pdl(k_lrn<float>, grid, 256, 0, c->stream, (const float*)in, L.d.out_h, L.d.out_w, L.d.cout, c->S, r, an, beta, kappa, (float*)out, masks, L.tiles_x, L.tiles_y)),
@@ -642,7 +663,7 @@ int dc_launch_concat(dc_cache* c, int layer, const void* a, int ca, const void* 
     const size_t pixels = (size_t)c->S * L.d.out_h * L.d.out_w, nv = pixels * L.d.cout * c->elt / 16;
     dc_prof_scope ps(c, DC_ST_POINTWISE);
     c->launches += 1;
-    if ((ca * c->elt) % 16 == 0 && (cb * c->elt) % 16 == 0 && nv < k32Bit) {
+    if ((ca * c->elt) % 16 == 0 && (cb * c->elt) % 16 == 0 && nv <= c->piece) {
         DC_CUDA(dc_launch_pdl(k_concat_vec, dim3((unsigned)grid_for(c, nv, 256)), 256, 0, c->stream, (const uint4*)a, (unsigned)(ca * c->elt / 16), (const uint4*)b,
                               (unsigned)(cb * c->elt / 16), (unsigned)nv, (uint4*)L.map[0]));
         return DC_OK;
@@ -658,7 +679,7 @@ int dc_launch_concat(dc_cache* c, int layer, const void* a, int ca, const void* 
 // without the gap of a copy node.
 int dc_launch_copy_map(dc_cache* c, const void* src, void* dst, size_t bytes)
 {
-    if (bytes % 16 == 0 && (uintptr_t)dst % 16 == 0 && bytes / 16 < k32Bit) {
+    if (bytes % 16 == 0 && (uintptr_t)dst % 16 == 0 && bytes / 16 <= c->piece) {
         const size_t nv = bytes / 16;
         DC_CUDA(dc_launch_pdl(k_copy_vec, dim3((unsigned)grid_for(c, nv, 256)), 256, 0, c->stream, (const uint4*)src, (unsigned)nv, (uint4*)dst));
         c->launches += 1;

@@ -286,6 +286,46 @@ def test_infer_graph_with_every_layer_kind(dtype):
     U.run_stream_parity(w, 1, list(range(3)), cache_pool=True, region_mode=B.DC_REGIONS_PER_BLOCK)
 
 
+@pytest.mark.parametrize("dtype", [B.DC_FP32, B.DC_BF16])
+def test_large_maps_are_launched_in_pieces(dtype):
+    """Launches whose kernels index with 32 bits are cut between rows or streams.  With the limit lowered to a few thousand
+    items the maps of every layer are the same, for the frame's own map, the padded operand copy, pooling of every window
+    and LRN, cached or not, and for a limit below one stream (the general kernels; cached layers stay whole)."""
+    import ctypes
+    S, hi, wi = 5, 45, 53
+    b = nets.NetBuilder(hi, wi)
+    x = b.conv(-1, 32, 3, 1, 1)
+    p2, p3, p5 = b.maxpool(x, 2, 2), b.maxpool(x, 3, 2, 1), b.maxpool(x, 5, 3, 2)
+    b.conv(p2, 32, 3, 1, 1)
+    b.lrn(p3, 2)
+    b.lrn(x, 1)
+    b.conv(p5, 32, 1, 1, 0)
+    if dtype == B.DC_FP32:
+        b.maxpool(-1, 2, 2)                                        # reads the frame's map
+    ws, bs = nets.random_weights(b.layers, 2)
+    g = rng(6)
+    frames = [torch.from_numpy(g.integers(0, 256, size=(S, hi, wi, 3), dtype=np.uint8)).cuda() for _ in range(2)]
+    frames[1][:, :, : wi // 2] = frames[0][:, :, : wi // 2]
+    limit = B.load().dc_debug_piece
+    limit.restype, limit.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]
+    for pool in (False, True):
+        want = None
+        for items in ((0, 25000, 9600) if pool else (0, 25000, 9600, 700)):
+            dc = DeepCache(wi, hi, b.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=dtype, cache_pool=pool)
+            assert items == 0 or limit(dc.handle, items) == B.DC_OK
+            for f in frames:
+                dc.infer_frame(f)
+            got = [dc.layer_map(i).float() for i in range(len(b.layers))]
+            want = want or got
+            for i, (m, w_) in enumerate(zip(got, want)):
+                if b.layers[i]["kind"] == B.DC_LRN and 0 < items < 20000:
+                    torch.testing.assert_close(m, w_, rtol=0.01, atol=1e-5)       # the general kernel's own power function
+                else:
+                    assert torch.equal(m, w_), (items, i)
+            assert dc.status() == B.DC_OK
+            dc.close()
+
+
 class _cropped:
     """A stream batch cut to the top-left h x w pixels of every frame."""
 
