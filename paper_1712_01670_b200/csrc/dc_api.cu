@@ -400,13 +400,21 @@ int dc_cache_launches(const dc_cache* c, int64_t* launches)
     return DC_OK;
 }
 
+// A later lookahead starts from here (once one has been made): the side stream writes the key buffer behind the current one
+// and reads the current one.
+static int mark_key(dc_cache* c)
+{
+    if (c->la_stream) DC_CUDA(cudaEventRecord(c->ev_key, c->stream));
+    return DC_OK;
+}
+
 int dc_cache_set_key(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
 {
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
     DC_TRY(cancel_lookahead(c));
     DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, c->key[c->key_cur], nullptr));
     c->key_valid = true;
-    return DC_OK;
+    return mark_key(c);                                             // the key itself has changed
 }
 
 int dc_match_blocks(dc_cache* c, const uint8_t* frame_dev, size_t pitch, int16_t* block_mv_dev,
@@ -425,7 +433,7 @@ int dc_match_blocks(dc_cache* c, const uint8_t* frame_dev, size_t pitch, int16_t
     DC_TRY(dc_launch_match(c, scratch, c->key[c->key_cur], &out));
     if (block_mv_dev && !direct_mv)
         DC_CUDA(cudaMemcpyAsync(block_mv_dev, c->blk_mv, (size_t)c->S * c->Gx * c->Gy * 2 * sizeof(int16_t), cudaMemcpyDeviceToDevice, c->stream));
-    return DC_OK;
+    return mark_key(c);                                             // the scratch copy has been read
 }
 
 int dc_propagate_regions(dc_cache* c, const dc_region* in_dev, const int32_t* n_in_dev, int layer_begin,
@@ -482,7 +490,7 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
         DC_TRY(cancel_lookahead(c));
         DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, frame_copy, c->mv_acc));
     }
-    if (c->la_stream) DC_CUDA(cudaEventRecord(c->ev_key, c->stream));   // a later lookahead may start from here
+    DC_TRY(mark_key(c));
     if (!refresh) {
         if (looked_ahead && c->la_matched) dc_use_match_set(c, c->mset_cur ^ 1);              // results are waiting there
         else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur], nullptr));
@@ -603,7 +611,7 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     DC_TRY(ensure_lookahead_stream(c));
     DC_TRY(cancel_lookahead(c));
     // Everything the side stream touches is free once the main stream has passed the frame copy of the last
-    // dc_infer_frame (where ev_key was recorded): the third key buffer was last read two frames ago, and the
+    // dc_infer_frame, dc_match_blocks or dc_cache_set_key (mark_key): the third key buffer was last read two frames ago, and the
     // match set that the current inference does not read was last read by the frame before it.  Waiting for
     // that point only -- not for the end of the current inference -- is what lets the two overlap.
     DC_CUDA(cudaStreamWaitEvent(c->la_stream, c->ev_key, 0));

@@ -1126,6 +1126,45 @@ def test_lookahead_gives_identical_results():
         dc.close()
 
 
+def test_lookahead_waits_for_the_calls_between():
+    """dc_lookahead_frame right behind dc_match_blocks (whose frame lies where the announced one goes) and behind
+    dc_cache_set_key (which changes the key that it is matched against)."""
+    W, H, S = 1280, 720, 4
+    g = rng(12)
+    base = np.repeat(np.repeat(g.integers(0, 256, size=(S, H // 8, W // 8, 3), dtype=np.uint8), 8, 1), 8, 2)
+    f = [torch.from_numpy(np.roll(base, (3 * k, -2 * k), axis=(1, 2))).cuda() for k in range(4)]
+    layers = nets.vgg16_trunk(224, 224, H, W)[:3]
+    ws, bs = nets.random_weights(layers, 2)
+    rec = []
+    for early in (False, True):
+        dc = DeepCache(W, H, layers, ws, bs, n_streams=S, block=16, search_range=16, dtype=B.DC_BF16)
+        out = [torch.zeros(s_, dtype=t, device="cuda") for s_, t in (((S, dc.Gy, dc.Gx, 2), torch.int16), ((S, dc.Gy, dc.Gx), torch.int32), ((S, 3), torch.int32))]
+
+        def pause():
+            if not early:
+                torch.cuda.synchronize()
+
+        dc.infer_frame(f[0])
+        B.dc_lookahead_frame(dc.handle, f[1], W * 3)
+        dc.infer_frame(f[1])
+        pause()
+        B.dc_match_blocks(dc.handle, f[3], W * 3, out[0], out[1], None, out[2], None, None)
+        pause()
+        B.dc_lookahead_frame(dc.handle, f[2], W * 3)
+        pause()
+        a = dc.infer_frame(f[2])
+        pause()
+        B.dc_cache_set_key(dc.handle, f[0], W * 3)
+        pause()
+        B.dc_lookahead_frame(dc.handle, f[3], W * 3)
+        pause()
+        _, st = dc.infer_frame(f[3], want_stats=True)
+        rec.append((*[o.clone() for o in out], a, torch.tensor([[s_.mvx, s_.mvy, s_.k_passed, s_.n_matched] for s_ in st])))
+        assert dc.status() == B.DC_OK
+        dc.close()
+    assert all(torch.equal(x, y) for x, y in zip(*rec))
+
+
 @pytest.mark.parametrize("dtype,hi,wi,cin,cout,k,S,groups", [
     (B.DC_FP32, 130, 200, 4, 64, 3, 3, 1),       # 8 x 8 sums per thread, 64-channel blocks, one short chunk
     (B.DC_FP32, 140, 210, 7, 32, 3, 5, 1),       # 8 x 8 sums, 32-channel blocks, channels not a multiple of four
