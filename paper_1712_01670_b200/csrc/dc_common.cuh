@@ -177,6 +177,12 @@ struct dc_once_per_device {
 __device__ __forceinline__ void dc_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dc_pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A load of what another kernel (or a caller's) writes.  __ldg states that the data does not change while this kernel runs, and
+// the compiler may place it ahead of dc_pdl_wait(): a dependent kernel is resident while the writer still runs.  __ldg is left to
+// weights, biases and tables that were complete when the cache was created.
+template <typename T>
+__device__ __forceinline__ T dc_ld(const T* p) { return *p; }
+
 // A kernel that has passed dc_pdl_wait() proves everything before its predecessor complete, and a kernel starts only after
 // all CTAs of its predecessor have passed theirs (they release after it).  So what is older than the predecessor may be
 // read before the wait, through L2: a convolution fetches its tile list, the count and the bitmaps there when at least one

@@ -18,7 +18,7 @@ constexpr int CI_T = 8;      // input channels per staging step
 constexpr int MAX_KW = 11;
 
 template <typename T> __device__ __forceinline__ float ld_f(const T* p);
-template <> __device__ __forceinline__ float ld_f<float>(const float* p) { return __ldg(p); }
+template <> __device__ __forceinline__ float ld_f<float>(const float* p) { return dc_ld(p); }
 template <> __device__ __forceinline__ float ld_f<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 template <typename T> __device__ __forceinline__ T st_f(float v);
 template <> __device__ __forceinline__ float st_f<float>(float v) { return v; }

@@ -73,18 +73,18 @@ __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src)
 // four channels of one pixel as floats; n < 4: the channels that exist
 __device__ __forceinline__ float4 ld_quad(const float* p, int n, bool vec)
 {
-    if (vec) return __ldg((const float4*)p);
+    if (vec) return dc_ld((const float4*)p);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (n > 0) v.x = __ldg(p);
-    if (n > 1) v.y = __ldg(p + 1);
-    if (n > 2) v.z = __ldg(p + 2);
-    if (n > 3) v.w = __ldg(p + 3);
+    if (n > 0) v.x = dc_ld(p);
+    if (n > 1) v.y = dc_ld(p + 1);
+    if (n > 2) v.z = dc_ld(p + 2);
+    if (n > 3) v.w = dc_ld(p + 3);
     return v;
 }
 __device__ __forceinline__ float4 ld_quad(const __nv_bfloat16* p, int n, bool vec)
 {
     if (vec) {
-        const uint2 u = __ldg((const uint2*)p);
+        const uint2 u = dc_ld((const uint2*)p);
         return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
     }
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(256) k_input_map(const uint8_t* frame, size_t 
     dc_pdl_release();
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const unsigned row = i / (unsigned)words, w = i - row * (unsigned)words;
-        const uint32_t v = __ldg((const uint32_t*)(frame + (size_t)row * pitch) + w);
+        const uint32_t v = dc_ld((const uint32_t*)(frame + (size_t)row * pitch) + w);
         T* o = out + (size_t)row * row_elems + 4 * w;
 #pragma unroll
         for (int k = 0; k < 4; ++k) if ((int)(4 * w) + k < row_elems) o[k] = from_pixel<T>((v >> (8 * k)) & 0xffu);
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256) k_frame_pad8(const uint8_t* frame, size_t
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const unsigned row = i / (unsigned)W, x = i - row * (unsigned)W;
         const uint32_t* q = (const uint32_t*)(frame + (size_t)row * pitch) + (3 * x >> 2);
-        const uint32_t v = __funnelshift_r(__ldg(q), __ldg(q + 1), (3 * x & 3) * 8);    // the copy's rows have spare bytes
+        const uint32_t v = __funnelshift_r(dc_ld(q), dc_ld(q + 1), (3 * x & 3) * 8);    // the copy's rows have spare bytes
         const __nv_bfloat162 rg = __halves2bfloat162(from_pixel<__nv_bfloat16>(v & 0xffu), from_pixel<__nv_bfloat16>((v >> 8) & 0xffu));
         const __nv_bfloat162 b0 = __halves2bfloat162(from_pixel<__nv_bfloat16>((v >> 16) & 0xffu), __float2bfloat16_rn(0.f));
         out[i] = make_uint4(*(const uint32_t*)&rg, *(const uint32_t*)&b0, 0u, 0u);
@@ -71,7 +71,7 @@ __device__ __forceinline__ unsigned long long fetch_bytes8(const uint8_t* row, i
     const int from = byte > 0 ? byte : 0, left = row_bytes - from;
     if (left <= 0 || byte <= -8) return 0;
     const uint32_t* q = (const uint32_t*)row + (from >> 2);           // the copy's rows have spare bytes
-    const uint32_t w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2);
+    const uint32_t w0 = dc_ld(q), w1 = dc_ld(q + 1), w2 = dc_ld(q + 2);
     const int sh = (from & 3) * 8;
     unsigned long long v = (unsigned long long)__funnelshift_r(w1, w2, sh) << 32 | __funnelshift_r(w0, w1, sh);
     if (left < 8) v &= (1ull << (8 * left)) - 1ull;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(256) k_resize_area(const uint8_t* frame, size_
         for (int yb = 0; yb < rows; yb += 6) {
             uint4 v[6];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) v[k] = yb + k < rows ? __ldg((const uint4*)(base + (size_t)(yb + k) * pitch + c * 16)) : make_uint4(0, 0, 0, 0);
+            for (int k = 0; k < 6; ++k) v[k] = yb + k < rows ? dc_ld((const uint4*)(base + (size_t)(yb + k) * pitch + c * 16)) : make_uint4(0, 0, 0, 0);
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
                 const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_maxpool_vec(const uint4* in, int Hi, in
 #pragma unroll
             for (int k = 0; k < K * K; ++k) {
                 const int y = min(max(y0 + k / K, max(y0, 0)), Hi - 1), x = min(max(x0 + k % K, max(x0, 0)), Wi - 1);
-                v[k] = __ldg(base + ((size_t)y * Wi + x) * cv);
+                v[k] = dc_ld(base + ((size_t)y * Wi + x) * cv);
             }
             m = v[0];
 #pragma unroll
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(256) k_maxpool_vec(const uint4* in, int Hi, in
                 for (int kx = 0; kx < L.kw; ++kx) {
                     const int ix = x0 + kx;
                     if (ix < 0 || ix >= Wi) continue;
-                    const uint4 v = __ldg(base + ((size_t)iy * Wi + ix) * cv);
+                    const uint4 v = dc_ld(base + ((size_t)iy * Wi + ix) * cv);
                     m = first ? v : Vec16<T>::vmax(m, v);
                     first = false;
                 }
@@ -246,7 +246,7 @@ __global__ void k_maxpool2x2_vec(const uint4* in, int Hi, int Wi, int cv, int ou
         const unsigned c = i % cv, t = i / cv, ox = t % out_w, u = t / out_w, oy = u % out_h, s = u / out_h;
         const uint4* p = in + (((size_t)s * Hi + 2 * oy) * Wi + 2 * ox) * cv + c;
         const size_t row = (size_t)Wi * cv;
-        const uint4 v00 = __ldg(p), v01 = __ldg(p + cv), v10 = __ldg(p + row), v11 = __ldg(p + row + cv);
+        const uint4 v00 = dc_ld(p), v01 = dc_ld(p + cv), v10 = dc_ld(p + row), v11 = dc_ld(p + row + cv);
         out[i] = Vec16<T>::vmax(Vec16<T>::vmax(v00, v01), Vec16<T>::vmax(v10, v11));
     }
 }
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, 
 #pragma unroll
             for (int dx = -R; dx <= R; ++dx) {
                 const int yy = y + dy, xx = x + dx;
-                v[dx + R] = yy >= 0 && yy < H && xx >= 0 && xx < W ? __ldg(base + ((size_t)yy * W + xx) * cv) : make_uint4(0, 0, 0, 0);
+                v[dx + R] = yy >= 0 && yy < H && xx >= 0 && xx < W ? dc_ld(base + ((size_t)yy * W + xx) * cv) : make_uint4(0, 0, 0, 0);
             }
 #pragma unroll
             for (int dx = 0; dx <= 2 * R; ++dx) {
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(256) k_concat_vec(const uint4* a, unsigned va,
     dc_pdl_release();
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const unsigned px = i / (va + vb), c = i - px * (va + vb);
-        out[i] = c < va ? __ldg(a + (size_t)px * va + c) : __ldg(b + (size_t)px * vb + (c - va));
+        out[i] = c < va ? dc_ld(a + (size_t)px * va + c) : dc_ld(b + (size_t)px * vb + (c - va));
     }
 }
 
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(256) k_copy_vec(const uint4* a, unsigned total
 {
     dc_pdl_wait();
     dc_pdl_release();
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) out[i] = __ldg(a + i);
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) out[i] = dc_ld(a + i);
 }
 
 inline int grid_for(const dc_cache* c, size_t n, int block)

@@ -80,7 +80,7 @@ struct BlockCtx {
                 uintptr_t a = (uintptr_t)p;
                 const uint32_t* q = (const uint32_t*)(a & ~(uintptr_t)3);
                 uint32_t sh = ((uint32_t)a & 3u) * 8u;
-                uint32_t lo = __ldg(q), hi = __ldg(q + 1);
+                uint32_t lo = dc_ld(q), hi = dc_ld(q + 1);
                 uint32_t pv = __funnelshift_r(lo, hi, sh) & msk[it];
                 uint32_t d = __vabsdiffu4(cur_sm[smi[it]], pv);
                 acc = __dp4a(d, d, acc);
@@ -115,7 +115,7 @@ __device__ __forceinline__ bool load_block(const MatchArgs& a, uint32_t* sm, Blo
             const uint8_t* p = cur + (size_t)row * a.cur_pitch + wi * 4;
             uint32_t v = 0;
             for (int k = 0; k < 4; ++k)
-                if (wi * 4 + k < row_bytes) v |= (uint32_t)__ldg(p + k) << (8 * k);
+                if (wi * 4 + k < row_bytes) v |= (uint32_t)dc_ld(p + k) << (8 * k);
             sm[c.smi[it]] = v;
         }
     }
@@ -403,7 +403,7 @@ struct RowCtx {
             row_on[k] = on[k];
             const uint4* p = (const uint4*)cur_rows[k];
             uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0, v2 = v0;
-            if (on[k]) { v0 = __ldg(p); v1 = __ldg(p + 1); v2 = __ldg(p + 2); }
+            if (on[k]) { v0 = dc_ld(p); v1 = dc_ld(p + 1); v2 = dc_ld(p + 2); }
             cw[k][0] = v0.x; cw[k][1] = v0.y; cw[k][2] = v0.z; cw[k][3] = v0.w; cw[k][4] = v1.x; cw[k][5] = v1.y;
             cw[k][6] = v1.z; cw[k][7] = v1.w; cw[k][8] = v2.x; cw[k][9] = v2.y; cw[k][10] = v2.z; cw[k][11] = v2.w;
             if (clipped) {
@@ -530,7 +530,7 @@ __device__ __forceinline__ void load_lane_pixels(const uint8_t* row, int h, bool
     uint32_t w[12];
     const uint4* p = (const uint4*)row;
     uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0, v2 = v0;
-    if (on) { v0 = __ldg(p); v1 = __ldg(p + 1); v2 = __ldg(p + 2); }
+    if (on) { v0 = dc_ld(p); v1 = dc_ld(p + 1); v2 = dc_ld(p + 2); }
     w[0] = v0.x; w[1] = v0.y; w[2] = v0.z; w[3] = v0.w; w[4] = v1.x; w[5] = v1.y; w[6] = v1.z; w[7] = v1.w;
     w[8] = v2.x; w[9] = v2.y; w[10] = v2.z; w[11] = v2.w;
 #pragma unroll
@@ -558,7 +558,7 @@ __device__ __forceinline__ void load_pixels4(const uint8_t* prev, size_t pitch, 
     a = b = c = 0;
     if (gy >= 0 && gy < H && px0 >= 0 && (size_t)px0 * 3 + 12 <= pitch) {
         const uint32_t* q = (const uint32_t*)(prev + (size_t)gy * pitch + (size_t)px0 * 3);     // px0 * 3 is a multiple of 12
-        a = __ldg(q); b = __ldg(q + 1); c = __ldg(q + 2);
+        a = dc_ld(q); b = dc_ld(q + 1); c = dc_ld(q + 2);
     }
 }
 
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
             pa[k] = pb[k] = pc[k] = 0;
             if (col_ok && row < W_ROWS && gy >= 0 && gy < a.H) {
                 const uint32_t* q = (const uint32_t*)(src + (size_t)gy * a.prev_pitch);
-                pa[k] = __ldg(q); pb[k] = __ldg(q + 1); pc[k] = __ldg(q + 2);
+                pa[k] = dc_ld(q); pb[k] = dc_ld(q + 1); pc[k] = dc_ld(q + 2);
             }
         }
         if (row0 < ROWS_PER_PASS) {
@@ -1047,7 +1047,7 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
                         pa[k] = pb[k] = pc[k] = 0;
                         if (col_ok && row < P_ROWS && gy >= 0 && gy < a.H) {
                             const uint32_t* q = (const uint32_t*)(src + (size_t)gy * a.prev_pitch);
-                            pa[k] = __ldg(q); pb[k] = __ldg(q + 1); pc[k] = __ldg(q + 2);
+                            pa[k] = dc_ld(q); pb[k] = dc_ld(q + 1); pc[k] = dc_ld(q + 2);
                         }
                     }
 #pragma unroll
@@ -1146,7 +1146,7 @@ __global__ void __launch_bounds__(256) k_verify16_list(MatchArgs a, const uint32
             // four wide loads instead of thirteen narrow ones, then a word offset that is the same for a whole stream
             const uint8_t* p = a.prev + (size_t)s * a.prev_stream + (size_t)(y0 + My + r) * a.prev_pitch + (size_t)(x0 + Mx) * 3;
             const uint4* p16 = (const uint4*)((uintptr_t)p & ~(uintptr_t)15);
-            const uint4 c0 = __ldg(p16), c1 = __ldg(p16 + 1), c2 = __ldg(p16 + 2), c3 = __ldg(p16 + 3);
+            const uint4 c0 = dc_ld(p16), c1 = dc_ld(p16 + 1), c2 = dc_ld(p16 + 2), c3 = dc_ld(p16 + 3);
             const uint32_t ww[16] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w, c2.x, c2.y, c2.z, c2.w, c3.x, c3.y, c3.z, c3.w};
             const uint32_t boff = (uint32_t)(uintptr_t)p & 15u, sh = (boff & 3u) * 8u;
             uint32_t w[13];
@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(256, 3) k_search_es16(MatchArgs a)
         const int gy = y0 - R + row, gb = wx0 + ci * 16;
         uint4 v = make_uint4(0, 0, 0, 0);
         if (gy >= 0 && gy < a.H && gb >= 0 && gb + 16 <= (int)a.prev_pitch)
-            v = __ldg((const uint4*)(prev + (size_t)gy * a.prev_pitch + gb));
+            v = dc_ld((const uint4*)(prev + (size_t)gy * a.prev_pitch + gb));
         *(uint4*)(win + row * E_PITCH + ci * 4) = v;
     }
     const int bx = strip * 8 + warp, x0 = bx * 16;
@@ -1227,7 +1227,7 @@ __global__ void __launch_bounds__(256, 3) k_search_es16(MatchArgs a)
         const uint8_t* cb = a.cur + (size_t)s * a.cur_stream + (size_t)y0 * a.cur_pitch + (size_t)x0 * 3;
         for (int i = lane; i < 16 * 3; i += 32) {
             const int r = i / 3, q = i - r * 3;
-            *(uint4*)(curw + r * 12 + q * 4) = __ldg((const uint4*)(cb + (size_t)r * a.cur_pitch) + q);
+            *(uint4*)(curw + r * 12 + q * 4) = dc_ld((const uint4*)(cb + (size_t)r * a.cur_pitch) + q);
         }
     }
     __syncthreads();
@@ -1327,15 +1327,15 @@ __global__ void __launch_bounds__(256) k_copy_frame(const uint8_t* src, const ui
         const int left = row_bytes - (int)c * 16;                     // bytes of the row from here on
         uint4 v;
         if (((uintptr_t)p & 15u) == 0 && p + 16 <= src_end) {
-            v = __ldg((const uint4*)p);
+            v = dc_ld((const uint4*)p);
         } else if (p + 20 <= src_end) {
             const uint32_t* q = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
-            const uint32_t w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = __ldg(q + 3), w4 = sh ? __ldg(q + 4) : 0u;
+            const uint32_t w0 = dc_ld(q), w1 = dc_ld(q + 1), w2 = dc_ld(q + 2), w3 = dc_ld(q + 3), w4 = sh ? dc_ld(q + 4) : 0u;
             v = make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh), __funnelshift_r(w3, w4, sh));
         } else {
             uint32_t w[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int k = 0; k < 16; ++k) if (k < left) w[k >> 2] |= (uint32_t)__ldg(p + k) << (8 * (k & 3));
+            for (int k = 0; k < 16; ++k) if (k < left) w[k >> 2] |= (uint32_t)dc_ld(p + k) << (8 * (k & 3));
             v = make_uint4(w[0], w[1], w[2], w[3]);
         }
         if (left < 16) {

@@ -34,10 +34,10 @@ __device__ __forceinline__ uint32_t load_pixel(const uint8_t* p, const uint8_t* 
     const uint32_t* q = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
     const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u;
     if ((const uint8_t*)q >= lo && (const uint8_t*)(q + 2) <= hi) {
-        const uint32_t a = __ldg(q), b = sh > 8 ? __ldg(q + 1) : 0u;
+        const uint32_t a = dc_ld(q), b = sh > 8 ? dc_ld(q + 1) : 0u;
         return __funnelshift_r(a, b, sh) & 0x00ffffffu;
     }
-    return (uint32_t)__ldg(p) | ((uint32_t)__ldg(p + 1) << 8) | ((uint32_t)__ldg(p + 2) << 16);
+    return (uint32_t)dc_ld(p) | ((uint32_t)dc_ld(p + 1) << 8) | ((uint32_t)dc_ld(p + 2) << 16);
 }
 
 struct Tile { int s, bx0, by0, nbx, nby; };       // stream, first block, blocks of the tile that exist
@@ -91,7 +91,7 @@ __device__ __forceinline__ void stage_window(const dc_win_args& a, const Tile& t
                 const uint8_t* p = row + (size_t)x * 3;
                 const uint32_t* q = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
                 const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u, m = 0x00ffffffu;
-                const uint32_t w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = sh ? __ldg(q + 3) : 0u;
+                const uint32_t w0 = dc_ld(q), w1 = dc_ld(q + 1), w2 = dc_ld(q + 2), w3 = sh ? dc_ld(q + 3) : 0u;
                 const uint32_t b0 = __funnelshift_r(w0, w1, sh), b1 = __funnelshift_r(w1, w2, sh), b2 = __funnelshift_r(w2, w3, sh);
                 dst[c] = b0 & m; dst[c + 1] = __funnelshift_r(b0, b1, 24) & m; dst[c + 2] = __funnelshift_r(b1, b2, 16) & m; dst[c + 3] = b2 >> 8;
             } else {
