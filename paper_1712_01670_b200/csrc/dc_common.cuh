@@ -223,6 +223,7 @@ int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int3
 bool dc_dense_ok(const dc_layer_rt& L);
 int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                         const int32_t* tile_count, const uint32_t* masks, int max_tiles);
+bool dc_conv_simt_stores(const dc_cache* c, const void* out);   // out lies where dc_launch_conv_simt can store
 int dc_launch_dense(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
 int dc_pack_weights_simt(dc_cache* c, int layer);
 int dc_launch_input_map(dc_cache* c, const uint8_t* frame, size_t pitch);

@@ -137,10 +137,9 @@ int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int3
     }
     if (c->cfg.dtype == DC_BF16 && dc_conv_bf16_supported(c, layer))
         return dc_launch_conv_bf16(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
-    // these two read and write vectors of up to 16 bytes; a caller's maps that lie otherwise take the kernel below
-    const bool aligned = (((uintptr_t)in | (uintptr_t)out) & 15u) == 0;
-    if (aligned && dc_dense_ok(L)) return dc_launch_dense(c, layer, in, out, masks);
-    if (aligned && L.weight_simt) return dc_launch_conv_simt(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
+    if (dc_dense_ok(L)) return dc_launch_dense(c, layer, in, out, masks);
+    // (an output map that it could not store vectors to takes the kernel below)
+    if (L.weight_simt && dc_conv_simt_stores(c, out)) return dc_launch_conv_simt(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
     ConvArgs a;
     a.in = in; a.w = L.weight; a.bias = L.bias; a.out = out;
     a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;

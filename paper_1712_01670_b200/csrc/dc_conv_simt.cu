@@ -47,6 +47,7 @@ struct SimtArgs {
     int Hi, Wi, Ci, Ho, Wo, Co, p, relu, tiles_x, tiles_y;
     int Cig, Cog, nb_g, NB, chunks;                                   // channels per group, blocks per group, blocks in all
     int early;                                                        // dc_lists_settled()
+    int vec;                                                          // four channels of a pixel are one aligned load
 };
 
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi)
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(KS * simt_threads(BN, TC)) k_conv_simt(const S
     if (!present) { asm volatile("cp.async.wait_all;" ::: "memory"); return; }
 
     const T* in = (const T*)a.in + (size_t)s * a.Hi * a.Wi * a.Ci + grp * a.Cig;
-    const bool vec = a.Ci % 4 == 0 && a.Cig % 4 == 0;
+    const bool vec = a.vec != 0;
     float4 stage[QPT];
     auto load_patch = [&](int chunk) {
 #pragma unroll
@@ -280,7 +281,7 @@ __global__ void k_pack_simt(const T* w, int taps, int Cig, int Cog, int nb_g, in
 // kernels would hold one useful pixel of 128 and walk K alone).
 constexpr int DN_S = 4, DN_N = 4, DN_WARPS = 8;
 
-struct DenseArgs { const void* in; const void* w; const float* bias; void* out; const uint32_t* masks; int S, N, K, relu; };
+struct DenseArgs { const void* in; const void* w; const float* bias; void* out; const uint32_t* masks; int S, N, K, relu, vec; };
 
 template <typename T>
 __global__ void __launch_bounds__(DN_WARPS * 32) k_dense(const DenseArgs a)
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(DN_WARPS * 32) k_dense(const DenseArgs a)
     dc_pdl_wait();
     dc_pdl_release();
     const int nv = (a.K + 3) / 4, per = (nv + DN_WARPS - 1) / DN_WARPS, lo = warp * per, hi = min(nv, lo + per);
-    const bool vec = a.K % 4 == 0;
+    const bool vec = a.vec != 0;
     float acc[DN_S * DN_N];
 #pragma unroll
     for (int i = 0; i < DN_S * DN_N; ++i) acc[i] = 0.f;
@@ -396,6 +397,10 @@ static int launch_simt_kw(dc_cache* c, const SimtArgs& a, int kw, const SimtShap
     return launch_simt_shape<T, 3, simt_ci(3, false)>(c, a, s, max_tiles);
 }
 
+// A caller's map may start at any element: four of them are one load or store only where they lie on a boundary of four.
+static bool quads(const dc_cache* c, const void* map) { return (uintptr_t)map % (4u * (unsigned)c->elt) == 0; }
+bool dc_conv_simt_stores(const dc_cache* c, const void* out) { return quads(c, out); }
+
 int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list, const int32_t* tile_count,
                         const uint32_t* masks, int max_tiles)
 {
@@ -408,6 +413,7 @@ int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const
     a.Hi = L.in_h; a.Wi = L.in_w; a.Ci = L.d.cin; a.Ho = L.d.out_h; a.Wo = L.d.out_w; a.Co = L.d.cout; a.p = L.d.ph; a.relu = L.d.relu;
     a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
     a.Cig = L.d.cin / G; a.Cog = L.d.cout / G; a.nb_g = dc_div_up(a.Cog, sh.BN); a.NB = G * a.nb_g; a.chunks = dc_div_up(a.Cig, sh.CI);
+    a.vec = a.Ci % 4 == 0 && a.Cig % 4 == 0 && quads(c, in);
     dc_prof_scope ps(c, DC_ST_CONV);
     c->launches += 1;
     return c->cfg.dtype == DC_BF16 ? launch_simt_kw<__nv_bfloat16>(c, a, L.d.kw, sh, max_tiles) : launch_simt_kw<float>(c, a, L.d.kw, sh, max_tiles);
@@ -416,7 +422,8 @@ int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const
 int dc_launch_dense(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks)
 {
     dc_layer_rt& L = c->L[layer];
-    DenseArgs a = {in, L.weight, L.bias, out, masks, c->S, L.d.cout, L.d.kh * L.d.kw * L.d.cin, L.d.relu};
+    DenseArgs a = {in, L.weight, L.bias, out, masks, c->S, L.d.cout, L.d.kh * L.d.kw * L.d.cin, L.d.relu, 0};
+    a.vec = a.K % 4 == 0 && quads(c, in);
     const dim3 grid(dc_div_up(a.N, DN_N), dc_div_up(a.S, DN_S));
     dc_prof_scope ps(c, DC_ST_CONV);
     if (c->cfg.dtype == DC_BF16) DC_CUDA(dc_launch_pdl(k_dense<__nv_bfloat16>, grid, DN_WARPS * 32, 0, c->stream, a));
