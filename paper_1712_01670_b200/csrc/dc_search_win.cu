@@ -4,7 +4,8 @@
 //
 // One CTA per tile of TX x TY blocks.  The part of the previous frame that any candidate of the tile can touch (the tile
 // and R pixels around it) is staged once in shared memory, one 32-bit word per pixel (R, G, B, 0), so a candidate starts
-// at a word whatever its displacement and whatever the alignment of the caller's rows, and no walk leaves the window.
+// at a word whatever its displacement and whatever the alignment of the caller's rows.  Walks with a range beyond
+// kWalkReach may stage that much and fetch the rare candidate outside from global memory.
 //   k_win_walk  diamond and three step search: one warp per block, lane l owns pixels l, l + 32, ... of the block.  The
 //               window's row pitch is congruent to the block edge modulo 32, so the lanes of a load fall in 32
 //               different banks.  The points of a round are scored as straight-line code, their loads all in flight.
@@ -22,6 +23,9 @@ namespace {
 
 constexpr int E_ROWS = 8;                 // vertical displacements a lane scores together
 constexpr int kMaxWarps = 16;
+// Pixels around the tile that walks over a longer range stage at least.  A walk visits a few dozen candidates near its start;
+// staging 64 pixels on every side of a few small blocks cost more than all of them (see dc_launch_search_win).
+constexpr int kWalkReach = 32;
 
 __device__ __forceinline__ uint32_t tie_of(int dx, int dy)
 {
@@ -73,7 +77,7 @@ __device__ __forceinline__ bool any_mine(const dc_win_args& a, const Tile& t)
 __device__ __forceinline__ void stage_window(const dc_win_args& a, const Tile& t, uint32_t* win)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    const int x0 = t.bx0 * a.B - a.R, y0 = t.by0 * a.B - a.R;
+    const int x0 = t.bx0 * a.B - a.Rw, y0 = t.by0 * a.B - a.Rw;
     const uint8_t* prev = a.prev + (size_t)t.s * a.prev_stream;
     const int y_lo = max(y0, 0), y_hi = min(y0 + a.win_rows, a.H) - 1;
     const uint8_t* first = prev + (size_t)y_lo * a.prev_pitch + (size_t)max(x0, 0) * 3;
@@ -156,23 +160,72 @@ __device__ __forceinline__ uint32_t lds_off(uint32_t p)
     return v;
 }
 
-template <int ITERS>
+// FAR: the window holds fewer than R pixels around the tile.
+template <int ITERS, bool FAR>
 struct Walk {
     uint32_t base;                  // shared-memory byte address of displacement (0, 0)
     int pitch4;                     // window row in bytes
     int dx_lo, dx_hi, dy_lo, dy_hi; // displacements that keep the block inside the frame and the range
+    const dc_win_args* args;        // FAR: where candidates outside the window come from:
+    const uint8_t* home;            // the block's position in the previous frame
     uint32_t cw[ITERS], off[ITERS]; // this lane's pixels and their byte offsets in the window
     uint32_t on;                    // which of them exist
     bool whole;                     // the block is not clipped: the first FULL exist in every lane
     static constexpr int FULL = ITERS <= 8 ? ITERS - 1 : ITERS / 2;
     int bx, by; uint32_t bs;        // best point so far and its SSE
 
+    __device__ __forceinline__ bool staged(int cx, int cy, int reach) const
+    {
+        return !FAR || (abs(cx) + reach <= kWalkReach && abs(cy) + reach <= kWalkReach);
+    }
     __device__ __forceinline__ bool inside(int cx, int cy, int reach) const
     {
-        return cx - reach >= dx_lo && cx + reach <= dx_hi && cy - reach >= dy_lo && cy + reach <= dy_hi;
+        return cx - reach >= dx_lo && cx + reach <= dx_hi && cy - reach >= dy_lo && cy + reach <= dy_hi && staged(cx, cy, reach);
+    }
+    // A candidate outside the window, from global memory: eight of the lane's pixels in flight.
+    __device__ uint32_t far(int dx, int dy) const
+    {
+        const uint8_t* p0 = home + (ptrdiff_t)dy * (ptrdiff_t)args->prev_pitch + dx * 3;
+        const int B = args->B, inv = (65536 + B - 1) / B;                        // p / B for p < 1024: p * inv >> 16
+        // two aligned words around any pixel of the block lie inside the buffer (the same in all lanes)
+        const bool words = p0 - 3 >= args->prev && p0 + (size_t)(B - 1) * args->prev_pitch + (size_t)B * 3 + 8 <= args->prev_end;
+        uint32_t acc = 0;
+#pragma unroll
+        for (int i0 = 0; i0 < ITERS; i0 += 8) {
+            if (i0 * 32 >= B * B) break;
+            uint32_t px[8];
+            if (words) {
+                uint32_t lo[8], hi[8], sh[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = i0 + j, q = i * 32 + (int)(threadIdx.x & 31), r = q * inv >> 16, c = q - r * B;
+                    const bool there = i < ITERS && ((on >> (i & 31)) & 1u);     // else the block's first pixel, masked
+                    const uint8_t* p = there ? p0 + (size_t)r * args->prev_pitch + c * 3 : p0;
+                    const uint32_t* w = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
+                    sh[j] = ((uint32_t)(uintptr_t)p & 3u) * 8u;
+                    lo[j] = dc_ld(w); hi[j] = dc_ld(w + 1);
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) px[j] = __funnelshift_r(lo[j], hi[j], sh[j]) & 0x00ffffffu;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = i0 + j, q = i * 32 + (int)(threadIdx.x & 31), r = q * inv >> 16, c = q - r * B;
+                    px[j] = i < ITERS && ((on >> (i & 31)) & 1u) ? load_pixel(p0 + (size_t)r * args->prev_pitch + c * 3, args->prev, args->prev_end) : 0u;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (i0 + j >= ITERS) break;
+                const uint32_t d = ((on >> (i0 + j)) & 1u) ? __vabsdiffu4(cw[i0 + j], px[j]) : 0u;
+                acc = __dp4a(d, d, acc);
+            }
+        }
+        return __reduce_add_sync(0xffffffffu, acc);
     }
     __device__ __forceinline__ uint32_t score(int dx, int dy) const
     {
+        if (FAR && !staged(dx, dy, 0)) return far(dx, dy);
         const uint32_t p = base + (uint32_t)(dy * pitch4 + dx * 4);
         uint32_t acc = 0;
 #pragma unroll
@@ -323,8 +376,8 @@ struct Walk {
 
 // three CTAs per SM where the lane's pixels leave the registers for it (10-pixel blocks, 720p, 4 streams: 78 us, 90 with
 // two; 16-pixel blocks with three: twice as slow)
-template <int ITERS>
-__global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 ? 3 : ITERS <= 8 ? 2 : 1) k_win_walk(const dc_win_args a)
+template <int ITERS, bool FAR>
+__global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 && !FAR ? 3 : ITERS <= 8 ? 2 : 1) k_win_walk(const __grid_constant__ dc_win_args a)
 {
     extern __shared__ __align__(16) uint32_t win[];
     __shared__ int32_t sums[4];
@@ -335,7 +388,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 ? 3 : ITERS <= 8 ? 
     if (!any_mine(a, t)) return;
     const int ly = warp / a.TX, lx = warp - ly * a.TX, bx = t.bx0 + lx, by = t.by0 + ly;
     const bool block = ly < a.TY && lx < t.nbx && ly < t.nby && mine(a, bx, by), walk = block && searched(a, bx, by);
-    Walk<ITERS> w;
+    Walk<ITERS, FAR> w;
     const int x0 = bx * a.B, y0 = by * a.B, bw = min(a.B, a.W - x0), bh = min(a.B, a.H - y0);
     w.on = 0;
 #pragma unroll
@@ -352,7 +405,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 ? 3 : ITERS <= 8 ? 
     stage_window(a, t, win);
     __syncthreads();
     if (walk) {
-        w.base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)((ly * a.B + a.R) * a.win_pitch + lx * a.B + a.R) * 4u;
+        w.base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)((ly * a.B + a.Rw) * a.win_pitch + lx * a.B + a.Rw) * 4u;
+        if (FAR) { w.args = &a; w.home = a.prev + (size_t)t.s * a.prev_stream + (size_t)y0 * a.prev_pitch + (size_t)x0 * 3; }
         w.pitch4 = a.win_pitch * 4;
         w.dx_lo = max(-a.R, -x0); w.dx_hi = min(a.R, a.W - bw - x0); w.dy_lo = max(-a.R, -y0); w.dy_hi = min(a.R, a.H - bh - y0);
         w.whole = bw == a.B && bh == a.B;
@@ -480,28 +534,40 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     auto shape = [&](int TX, int TY) {
         a.TX = TX; a.TY = TY;
         a.tiles_x = dc_div_up(a.Gx, TX); a.tiles_y = dc_div_up(a.Gy, TY);
-        a.win_cols = (TX * a.B + 2 * a.R + 3) & ~3;                   // staged in groups of four
-        a.win_rows = TY * a.B + 2 * a.R + (all ? E_ROWS - 1 : 0);     // rows only touched by displacements beyond R (scored, never compared)
+        a.win_cols = (TX * a.B + 2 * a.Rw + 3) & ~3;                  // staged in groups of four
+        a.win_rows = TY * a.B + 2 * a.Rw + (all ? E_ROWS - 1 : 0);    // rows only touched by displacements beyond R (scored, never compared)
         a.win_pitch = a.win_cols + ((a.B - a.win_cols) % 32 + 32) % 32;   // = B modulo 32
         smem = (size_t)a.win_rows * a.win_pitch * 4 + (all ? (size_t)TX * TY * a.B * a.B * 4 : 0);
     };
     // Wide tiles stage fewer window pixels per block; they shrink while the window is too large for three CTAs per SM, and
     // while the frames have fewer tiles than the machine has SMs (down to two blocks, one for the exhaustive search).
-    int TX = a.Gx < 8 ? a.Gx : 8, TY = TX < 4 ? 4 : 2;
-    if (TY > a.Gy) TY = a.Gy;
-    shape(TX, TY);
-    while (TX * TY > 1 && (smem > 200 * 1024 || (TX * TY > 2 && smem > 72 * 1024) ||
-                           ((long long)a.tiles_x * a.tiles_y * a.S < num_sms && TX * TY > (all ? 1 : 2)))) {
-        if (TY > 1 && (TY > TX || smem <= 72 * 1024)) TY = (TY + 1) / 2; else if (TX > 1) TX = (TX + 1) / 2; else TY = (TY + 1) / 2;
+    int TX = 0, TY = 0;
+    auto fit = [&](int Rw) {                                          // returns the window pixels staged per block
+        a.Rw = Rw;
+        TX = a.Gx < 8 ? a.Gx : 8; TY = TX < 4 ? 4 : 2;
+        if (TY > a.Gy) TY = a.Gy;
         shape(TX, TY);
-    }
+        while (TX * TY > 1 && (smem > 200 * 1024 || (TX * TY > 2 && smem > 72 * 1024) ||
+                               ((long long)a.tiles_x * a.tiles_y * a.S < num_sms && TX * TY > (all ? 1 : 2)))) {
+            if (TY > 1 && (TY > TX || smem <= 72 * 1024)) TY = (TY + 1) / 2; else if (TX > 1) TX = (TX + 1) / 2; else TY = (TY + 1) / 2;
+            shape(TX, TY);
+        }
+        return a.win_rows * a.win_cols / (TX * TY);
+    };
+    // Walks over a long range: a window of kWalkReach where that stages less than a fifth per block.  (Match calls with the whole
+    // window and with the capped one, range 64, diamond: 1080p, 16 streams, 8-pixel blocks, 13 times the pixels: 13456 and 1610 us;
+    // 20 pixels, 6.6 times: 4145 and 2184; 227 x 227, 24 pixels, 2.7 times: 72 and 125.  Range 40, 1.4 to 1.8 times: 513 and 571.)
+    const int whole = fit(a.R);
+    bool far = !all && a.R > kWalkReach;
+    if (far && whole <= 5 * fit(kWalkReach)) { far = false; fit(a.R); }
     // exhaustive: as many warps as there are groups of 32 items, up to 16
     const int n_d = 2 * a.R + 1, groups = (n_d * dc_div_up(n_d, E_ROWS) + 31) / 32;
     int warps = TX * TY < 8 ? 8 : TX * TY;                            // walks: a warp per block; spare ones help to stage the window
     if (all) { const long long units = (long long)TX * TY * groups; warps = units < 4 ? 4 : units > kMaxWarps ? kMaxWarps : (int)units; }
     if (all) { static dc_once_per_device set; return launch(k_win_all, a, warps * 32, smem, device, set, stream); }
     // one instance per number of pixels a lane owns, up to 16-pixel blocks
-#define DC_WALK(n) { static dc_once_per_device set; return launch(k_win_walk<n>, a, warps * 32, smem, device, set, stream); }
+#define DC_WALK_(n, f) { static dc_once_per_device set; return launch(k_win_walk<n, f>, a, warps * 32, smem, device, set, stream); }
+#define DC_WALK(n) { if (far) DC_WALK_(n, true) DC_WALK_(n, false) }
     switch (dc_div_up(a.B * a.B, 32)) {
     case 1: DC_WALK(1)
     case 2: DC_WALK(2)
@@ -514,4 +580,5 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     default: if (a.B * a.B <= 512) DC_WALK(16) DC_WALK(32)
     }
 #undef DC_WALK
+#undef DC_WALK_
 }

@@ -1239,3 +1239,24 @@ def test_match_staged_window_shapes(search, block, R, shape):
     pairs = [(prev, np.roll(prev, (min(R, 5), -min(R, 6)), axis=(0, 1))), (smooth, np.roll(smooth, (-3, 4), axis=(0, 1))), (prev, smooth)]
     check_pairs(pairs, block, R, search)
     check_pairs(pairs[1:2], block, R, search, skip_k=2)
+
+
+@pytest.mark.parametrize("search", [B.DC_SEARCH_DIAMOND, B.DC_SEARCH_THREE_STEP])
+@pytest.mark.parametrize("block,R", [(4, 64), (6, 33), (8, 64), (10, 40), (14, 64), (20, 64), (32, 64)])
+def test_match_walks_leave_the_staged_window(search, block, R):
+    """Ranges beyond what the walks stage: a smooth texture moved by up to 60 pixels leads the walks out of the window, at its
+    edge, across the frame's edges and past the range."""
+    g = rng(block * 5 + R)
+    H, W = 190, 230
+    lat = g.uniform(0, 255, size=(H // 24 + 4, W // 24 + 4, 3))
+    y, x = np.arange(H + 80) / 30.0, np.arange(W + 80) / 30.0
+    iy, ix = y.astype(int) % lat.shape[0], x.astype(int) % lat.shape[1]
+    fy, fx = (y - y.astype(int))[:, None, None], (x - x.astype(int))[None, :, None]
+    rows = lat[iy] * (1 - fy) + lat[(iy + 1) % lat.shape[0]] * fy
+    tex = (rows[:, ix] * (1 - fx) + rows[:, (ix + 1) % lat.shape[1]] * fx).astype(np.uint8)
+    cut = lambda dy, dx: np.ascontiguousarray(tex[40 + dy:40 + dy + H, 40 + dx:40 + dx + W])
+    pairs = [(cut(0, 0), cut(dy, dx)) for dy, dx in ((33, -31), (-38, 36), (2, 39), (0, 1))]
+    far = [orc.match_blocks(c, p, block, R, search, 20.0, 1, 0)["mv"] for p, c in pairs]
+    assert max(np.abs(m).max() for m in far) > (32 if search == B.DC_SEARCH_DIAMOND or R >= 63 else 28)     # three steps reach 31 or 63
+    check_pairs(pairs, block, R, search)
+    check_pairs(pairs[:1], block, R, search, skip_k=2)
