@@ -193,6 +193,8 @@ int dc_propagate_regions(dc_cache* cache, const dc_region* in_dev, const int32_t
  *   out_map_dev   [S][Ho][Wo][cout]  (top blob); must not alias prev_out_dev
  * Alignment: prev_out_dev and out_map_dev 16 bytes where rectangles are given; on the tensor-core kernels
  * (dc_cache_layer_conv_scheme > 0) out_map_dev 16 bytes, and in_map_dev too where cin is a multiple of 16; else an element.
+ * The rectangles of a stream are disjoint (those of dc_match_blocks and dc_propagate_regions are); which of two overlapping
+ * ones a pixel is copied by is not defined.
  * A count above max_regions is cut to max_regions.  A rectangle that does not lie inside the Ho x Wo map on
  * both sides (current and cached) is not reused -- its pixels are convolved like any other -- and the device
  * status word is set to DC_ERR_ARG (dc_get_status); no map is ever addressed outside its bounds.
