@@ -162,6 +162,7 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     DC_CUDA(cudaMemsetAsync(c->partial, 0, sizeof(int32_t) * (S + 3), c->stream));
     DC_TRY(dev_alloc(c, &c->reuse_px, (size_t)n * S * 2));
     c->alive = c->reuse_px + (size_t)n * S;
+    DC_CUDA(cudaMemsetAsync(c->reuse_px, 0, sizeof(int32_t) * n * S * 2, c->stream));
     DC_TRY(dev_alloc(c, &c->status, (size_t)1));
     DC_TRY(dev_alloc(c, &c->reused_total, (size_t)n));
     DC_CUDA(cudaMemsetAsync(c->reused_total, 0, sizeof(unsigned long long) * n, c->stream));
@@ -230,6 +231,7 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     size_t stat_ints = (size_t)S * (3 + 4 + 1) + (size_t)n * S;
     if (cudaMallocHost(&c->stats_pinned, stat_ints * sizeof(int32_t)) != cudaSuccess) { cudaGetLastError(); return DC_ERR_ALLOC; }
     DC_CUDA(cudaStreamSynchronize(c->stream));      // all_count lives on this stack frame
+    DC_TRY(dc_settle_weights_f32(c));
     for (int i = 0; i < n; ++i)
         if (c->executable && c->L[i].d.kind == DC_CONV) {
             const void* in = c->L[i].d.in0 < 0 ? c->input_map : c->L[c->L[i].d.in0].map[0];
@@ -281,7 +283,7 @@ void release(dc_cache* c)
     if (c->stats_pinned) cudaFreeHost(c->stats_pinned);
     for (int i = 0; i < c->n_layers; ++i) {
         dc_layer_rt& L = c->L[i];
-        cudaFree(L.map[0]); cudaFree(L.map[1]); cudaFree(L.weight); cudaFree(L.bias); cudaFree(L.weight_packed); cudaFree(L.weight_simt); cudaFree(L.in_padded); cudaFree(L.in_s2d); cudaFree(L.weight_halo);
+        cudaFree(L.map[0]); cudaFree(L.map[1]); cudaFree(L.weight); cudaFree(L.bias); cudaFree(L.weight_packed); cudaFree(L.weight_simt); cudaFree(L.weight_f32); cudaFree(L.in_padded); cudaFree(L.in_s2d); cudaFree(L.weight_halo);
         cudaFree(L.masks); cudaFree(L.dirty_list); cudaFree(L.all_list);
     }
     cudaGetLastError();

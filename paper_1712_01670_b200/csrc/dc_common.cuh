@@ -60,6 +60,7 @@ struct dc_layer_rt {
     void* weight_halo;              // conv, bf16: weights packed for the patch-reuse and column-slab kernels
     int halo_bn;                    // channels per block that packing is grouped by
     float* weight_simt;             // conv on the register-blocked CUDA-core kernel: its packed weights (dc_conv_simt.cu)
+    void* weight_f32;               // conv, fp32, on the tensor cores: weights split into bf16 pieces (dc_conv_f32.cu)
     void* in_padded;                // conv, bf16, cin <= 8: input with channels padded to 8
     void* in_s2d;                   // conv, bf16, strided over few channels: the space-to-depth copy of the input the rewritten layer reads (dc_conv_s2d.cu)
     int s2d_ws, s2d_cs;             // ... columns of the block map and channels of its pixels
@@ -226,6 +227,11 @@ int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const
 bool dc_conv_simt_stores(const dc_cache* c, const void* out);   // out lies where dc_launch_conv_simt can store
 int dc_launch_dense(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
 int dc_pack_weights_simt(dc_cache* c, int layer);
+// float32 stride-1 layers on the tensor cores (dc_conv_f32.cu)
+int dc_launch_conv_f32(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
+                       const int32_t* tile_count, const uint32_t* masks, int max_tiles);
+int dc_pack_weights_f32(dc_cache* c, int layer);                 // sets L.weight_f32 for the layers that run there
+int dc_settle_weights_f32(dc_cache* c);                          // ... unless a weight stands against it
 int dc_launch_input_map(dc_cache* c, const uint8_t* frame, size_t pitch);
 bool dc_conv_takes_frame(const dc_cache* c, int layer);      // the layer's operand copy can be filled from the frame itself
 int dc_launch_frame_operand(dc_cache* c, int layer, const uint8_t* frame, size_t pitch);

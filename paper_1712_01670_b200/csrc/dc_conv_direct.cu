@@ -139,6 +139,7 @@ int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int3
         return dc_launch_conv_bf16(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
     if (dc_dense_ok(L)) return dc_launch_dense(c, layer, in, out, masks);
     // (an output map that it could not store vectors to takes the kernel below)
+    if (L.weight_f32 && dc_conv_simt_stores(c, out)) return dc_launch_conv_f32(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
     if (L.weight_simt && dc_conv_simt_stores(c, out)) return dc_launch_conv_simt(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
     ConvArgs a;
     a.in = in; a.w = L.weight; a.bias = L.bias; a.out = out;
@@ -184,5 +185,6 @@ int dc_pack_weights(dc_cache* c, int layer, const float* w_dev, const float* b_d
         const int rc = dc_pack_weights_bf16(c, layer);
         if (rc != DC_OK || dc_conv_bf16_supported(c, layer)) return rc;
     }
-    return dc_pack_weights_simt(c, layer);
+    const int rc = dc_pack_weights_f32(c, layer);
+    return rc != DC_OK || L.weight_f32 ? rc : dc_pack_weights_simt(c, layer);
 }

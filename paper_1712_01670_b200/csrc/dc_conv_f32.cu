@@ -1,0 +1,548 @@
+// Partial convolution of float32 maps on the 5th-generation tensor cores, without giving up float32 accuracy.
+//
+// A float has 24 significant bits, a bf16 eight: every operand is the exact sum of three bf16 pieces, x = x0 + x1 + x2 (each the
+// nearest bf16 of what is left).  The product of two operands is then six tensor-core products of pieces,
+//     x0 w0  +  (x0 w1 + x1 w0)  +  (x0 w2 + x1 w1 + x2 w0),
+// whose remainder (x1 w2 and smaller) is below 2^-26 of the product.  Products of bf16 are exact in fp32; what rounds is the sum,
+// and there the tensor core is kept on a short leash: it adds up one kernel row of 32 channels (terms of each of the three sizes in
+// an accumulator of its own), then the sums move to registers and are added there, rounded to nearest, in a fixed order.
+// Measured against 64-bit sums (2-norm, pixel inputs through five layers): 0.6 of the error of the chain of fp32 FMAs.
+//
+// One instruction takes several products: the weight pieces lie behind one another along N, so A = x0 times [w0 w1 w2] fills three
+// blocks of BN columns, x1 times [w0 w1] adds to the last two, x2 times [w0] to the last.  A block of BN = 64 channels so costs
+// 192 + 128 + 64 columns per 16 input channels, and the pixels are read from shared memory three times, not six.
+//
+// Work item: one dirty 16 x 8 tile (128 pixels = M) times BN channels; persistent CTAs, one per SM.  16 warps:
+//   0      weights: one bulk copy per (32 channels, kernel row), packed as the MMA reads them
+//   1      MMA issue
+//   2-9    the sums: tensor memory -> registers after every kernel row; bias, ReLU, store of the pixels not reused (a warp: 32 pixels,
+//          half of the channels)
+//   10-15  input: the (16 + kh - 1) x (8 + kw - 1) patch of 32 channels, split into pieces on its way to shared memory (planes of
+//          8 channels, 16 bytes a pixel: every tap is a shifted view of it, as in the patch scheme of the bf16 kernels)
+// What bounds it: the tensor pipe (see f32_bn), and beside it the sums' way out: without MMAs 0.8 of the time, without the stores 0.9.
+// Measured, 24 streams, all tiles, us (CUDA cores, here): 32 -> 32 at 227 x 227 451, 203; 32 -> 64 at 113 x 113 246, 80; 64 -> 64 461, 134;
+// 64 -> 128 at 56 x 56 213, 71.  One stream: 29.4, 14.6; 19.8, 8.9; 32.5, 13.1; 17.3, 11.0.
+//
+// Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf).  A tile that holds one is marked by the warps
+// that split it and its pixels are computed once more with FMAs from the float weights; weights like that keep the layer
+// on the CUDA cores.
+#include "dc_common.cuh"
+#include "dc_tcgen05.cuh"
+
+namespace {
+
+constexpr int kSumWarps = 8, kSplitWarps = 6, kThreadsF = 32 * (2 + kSumWarps + kSplitWarps);
+constexpr int kStagesF = 8;                       // weight stages at most
+constexpr int kChF = 32;                          // input channels per patch
+constexpr int kRowsPerDrain1 = 3;                 // 1 x 1 kernels: patches between two drains (6 steps of 16 channels, as a row of a 3 x 3 kernel)
+constexpr int kTileFlags = 8;                     // more than the items between the splitting warps and the epilogue (at most 5)
+constexpr unsigned long long kWaitLimitF = 2000000000ull;
+
+struct F32Args {
+    const float* in; const float* w; const uint8_t* wp; const float* bias; float* out;   // wp: [groups * nb_g][chunks][taps][4][3 BN][8] bf16
+    const int32_t* tile_list; const int32_t* tile_count; const uint32_t* masks;
+    int Hi, Wi, Ci, Ho, Wo, Co, p, relu, tiles_x, tiles_y;
+    int Cig, Cog, nb_g, NB, chunks, ks_last;      // channels per group; blocks per group and in all; patches; steps of 16 channels in the last
+    int stages;
+    int vec;                                      // four input channels are one aligned load
+    int early;
+    int32_t* status;
+    unsigned long long wait_ns;
+    int skip_loads;
+};
+
+// Channels of the output's staging (32 pixels for each warp): a warp's half, or as many as fit.
+__host__ __device__ constexpr int f32_stage_ch(int BN, int KW) { return BN == 32 ? 16 : KW == 5 ? 8 : 32; }
+
+struct __align__(16) CtlF {
+    unsigned long long full[kStagesF], empty[kStagesF], a_full[2], a_empty[2], t_full[2], t_empty[2];
+    uint32_t tmem_base;
+    volatile int abort_flag;
+    unsigned long long wait_ns;
+    volatile int odd[kTileFlags];                 // item that holds a value that does not split (its number + 1)
+};
+
+__device__ __forceinline__ bool f_wait(uint32_t bar, uint32_t parity, CtlF* ctl, int32_t* status)
+{
+    return mbar_wait_at(bar, parity, &ctl->abort_flag, &ctl->wait_ns, status);
+}
+// A whole warp's wait: one lane asks, so that a waiting warp takes one turn at the barrier and not 32.
+__device__ __forceinline__ bool f_wait_warp(uint32_t bar, uint32_t parity, int lane, CtlF* ctl, int32_t* status)
+{
+    bool ok = true;
+    if (lane == 0) ok = f_wait(bar, parity, ctl, status);
+    return __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+}
+// N columns, 128 rows, bf16 operands, fp32 sums
+__device__ __forceinline__ uint32_t f_idesc(int n) { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (8u << 24); }
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// Two floats into three pairs of pieces; `odd` becomes NaN if one of them does not split.
+__device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2, float& odd)
+{
+    p0 = bf16_pair(a, b);
+    a -= __uint_as_float(p0 << 16); b -= __uint_as_float(p0 & 0xffff0000u);
+    p1 = bf16_pair(a, b);
+    a -= __uint_as_float(p1 << 16); b -= __uint_as_float(p1 & 0xffff0000u);
+    p2 = bf16_pair(a, b);
+    odd = fmaf(a, 0.f, odd); odd = fmaf(b, 0.f, odd);
+}
+
+template <int BN, int KW>
+__global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
+{
+    constexpr int PW = DC_TILE_W + KW - 1, PX = PW * (DC_TILE_H + KW - 1), PLANE = PX * 16, PIECE = 4 * PLANE, A_SLOT = 3 * PIECE;
+    constexpr int TAP = 4 * 3 * BN * 16, B_STAGE = KW * TAP;              // weights of a tap, of a kernel row
+    constexpr int UNITS = (4 * PX + 32 * kSplitWarps - 1) / (32 * kSplitWarps);   // 8-channel pixels that a splitting thread holds
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+    uint8_t* bring = base + 2 * A_SLOT;
+    CtlF* ctl = (CtlF*)(bring + (size_t)a.stages * B_STAGE);
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int per_stream = a.tiles_x * a.tiles_y;
+    constexpr uint32_t kSet = 3 * BN, kCols = BN == 32 ? 256 : 512;
+    constexpr int STAGE_CH = f32_stage_ch(BN, KW), STAGE_PITCH = (STAGE_CH + 4) * 4;   // bank-conflict free for both sides
+    constexpr int kRows = KW > 1 ? 1 : kRowsPerDrain1;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < a.stages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&ctl->a_full[i], kSplitWarps); mbar_init(&ctl->a_empty[i], 1);
+            mbar_init(&ctl->t_full[i], 1); mbar_init(&ctl->t_empty[i], kSumWarps);
+        }
+        for (int i = 0; i < kTileFlags; ++i) ctl->odd[i] = 0;
+        ctl->abort_flag = 0;
+        ctl->wait_ns = a.wait_ns;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)), "r"(kCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    if (!a.early) { dc_pdl_wait(); dc_pdl_release(); }
+    const int n_items = __ldcg(a.tile_count) * a.NB;
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
+    const uint32_t t_full0 = smem_u32(&ctl->t_full[0]), t_empty0 = smem_u32(&ctl->t_empty[0]);
+    auto k_steps = [&](int cc) { return cc + 1 < a.chunks ? kChF / 16 : a.ks_last; };
+
+    if (warp == 0) {
+        // ---------------- weights ----------------
+        if (elect_one()) {
+            RingPos r;
+            r.start(smem_u32(bring), (uint32_t)a.stages);
+            const uint32_t r0 = r.data;
+            const size_t block = (size_t)a.chunks * KW * B_STAGE;
+            // a last patch of one step needs the first half of each tap alone
+            auto send = [&](uint32_t off, uint32_t dst, const uint8_t* src, int cc) {
+                const int half = k_steps(cc) == 1;
+                mbar_expect_tx(full0 + off, (uint32_t)(half ? B_STAGE / 2 : B_STAGE));
+                if (!half) bulk_copy(dst, src, B_STAGE, full0 + off);
+                else for (int t = 0; t < KW; ++t) bulk_copy(dst + t * TAP, src + t * TAP, TAP / 2, full0 + off);
+            };
+            bool ok = true;
+            int ahead = 0;
+            if (a.early) {
+                // the weights are nobody's output: the first stages travel while the previous kernel ends
+                if ((int)blockIdx.x < n_items && !a.skip_loads) {
+                    const uint8_t* w = a.wp + (size_t)(blockIdx.x % a.NB) * block;
+                    const int n = min(a.stages, a.chunks * KW);
+                    for (int cc = 0, t = 0; ahead < n; ++ahead) {
+                        send(8u * ahead, r0 + ahead * B_STAGE, w + (size_t)ahead * B_STAGE, cc);
+                        if (++t == KW) { t = 0; ++cc; }
+                    }
+                }
+                dc_pdl_wait(); dc_pdl_release();
+            }
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+                const uint8_t* w = a.wp + (size_t)(item % a.NB) * block;
+                for (int cc = 0; cc < a.chunks && ok; ++cc)
+                    for (int t = 0; t < KW; ++t, w += B_STAGE) {
+                        if (ahead > 0) --ahead;
+                        else {
+                            ok = f_wait(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
+                            if (!ok) break;
+                            if (!a.skip_loads) send(r.off, r.data, w, cc);
+                        }
+                        r.next(r0, (uint32_t)a.stages, (uint32_t)B_STAGE);
+                    }
+            }
+            // on an abort: give the copies already issued a bounded chance to land before the CTA exits
+            if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------- MMA issuer ----------------
+        if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
+        if (elect_one()) {
+            const uint64_t ac = umma_desc(0, PW * 16, 0, PLANE), bc = umma_desc(0, 128, 0, 3 * BN * 16);
+            const uint32_t a_hi = (uint32_t)(ac >> 32), b_hi = (uint32_t)(bc >> 32);
+            const uint32_t a0 = (uint32_t)ac + (smem_u32(base) >> 4), b0 = (uint32_t)bc + (smem_u32(bring) >> 4);
+            const uint32_t i3 = f_idesc(3 * BN), i2 = f_idesc(2 * BN), i1 = f_idesc(BN);
+            RingPos rb, ra;
+            rb.start(b0, (uint32_t)a.stages); ra.start(a0, 2);
+            uint32_t set = 0, set_ph = 0;
+            bool ok = true;
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+                int rows = 0;                                              // kernel rows in the accumulator set
+                for (int cc = 0; cc < a.chunks && ok; ++cc) {
+                    ok = f_wait(a_full0 + ra.off, ra.phase, ctl, a.status);
+                    const bool two = k_steps(cc) == 2;
+                    for (int ky = 0; ky < KW && ok; ++ky) {
+                        if (rows == 0) ok = f_wait(t_empty0 + 8u * set, set_ph ^ 1u, ctl, a.status);
+                        ok = ok && f_wait(full0 + rb.off, rb.phase, ctl, a.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t d = tmem_base + set * kSet, at = ra.data + (uint32_t)(ky * PW);
+                        // a kernel row's MMAs in one go: what one lane can issue is the limit here, not the tensor pipe
+#pragma unroll
+                        for (int kx = 0; kx < KW; ++kx)
+#pragma unroll
+                            for (int k = 0; k < kChF / 16; ++k)
+                                if (k == 0 || two) {
+                                    const uint32_t al = at + kx + k * (PLANE >> 3), bl = rb.data + ((kx * TAP + k * (2 * 3 * BN * 16)) >> 4);
+                                    umma_chunk(d, al, a_hi, 0, bl, b_hi, 0, i3, kx + k == 0 ? (uint32_t)rows : 1u, 1);
+                                    umma_chunk(d + BN, al + (PIECE >> 4), a_hi, 0, bl, b_hi, 0, i2, 1u, 1);
+                                    umma_chunk(d + 2 * BN, al + 2 * (PIECE >> 4), a_hi, 0, bl, b_hi, 0, i1, 1u, 1);
+                                }
+                        umma_commit_at(empty0 + rb.off);
+                        rb.next(b0, (uint32_t)a.stages, (uint32_t)B_STAGE >> 4);
+                        if (++rows == kRows || (cc + 1 == a.chunks && ky + 1 == KW)) {
+                            umma_commit_at(t_full0 + 8u * set);
+                            rows = 0;
+                            set ^= 1u;
+                            if (set == 0) set_ph ^= 1u;
+                        }
+                    }
+                    if (ok) umma_commit_at(a_empty0 + ra.off);
+                    ra.next(a0, 2, (uint32_t)A_SLOT >> 4);
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp < 2 + kSumWarps) {
+        // ---------------- sums, bias, ReLU, store ----------------
+        constexpr int CH = BN / 2;                                        // channels of this thread's pixel
+        const int q = warp & 3, half = (warp - 2) >> 2, m = q * 32 + lane, row = m / DC_TILE_W, col = m % DC_TILE_W;
+        const uint32_t lanes = (uint32_t)(q * 32) << 16;
+        const int drains = (a.chunks * KW + kRows - 1) / kRows;
+        auto tile_of = [&](int item) { return item < n_items ? __ldcg(a.tile_list + item / a.NB) : 0; };
+        int next = tile_of(blockIdx.x);
+        if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
+        const uint32_t stage = smem_u32(ctl + 1) + (warp - 2) * 32 * STAGE_PITCH;
+        uint32_t set = 0, set_ph = 0;
+        int seq = 0;
+        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++seq) {
+            const int tile = next;
+            next = tile_of(item + gridDim.x);
+            const uint32_t word = __ldcg(a.masks + (size_t)tile * 4 + (row >> 2));
+            float sum[CH];
+#pragma unroll
+            for (int j = 0; j < CH; ++j) sum[j] = 0.f;
+            bool ok = true;
+            for (int u = 0; u < drains; ++u) {
+                ok = f_wait_warp(t_full0 + 8u * set, set_ph, lane, ctl, a.status);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d = tmem_base + lanes + set * kSet + half * CH;
+#pragma unroll
+                for (int h = 0; h < CH; h += 16) {                         // the small terms first
+                    uint32_t x[16], y[16];
+                    tmem_ld16(d + 2 * BN + h, x);
+                    tmem_ld16(d + BN + h, y);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) x[j] = __float_as_uint(__uint_as_float(x[j]) + __uint_as_float(y[j]));
+                    tmem_ld16(d + h, y);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sum[h + j] += __uint_as_float(y[j]) + __uint_as_float(x[j]);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&ctl->t_empty[set]);
+                set ^= 1u;
+                if (set == 0) set_ph ^= 1u;
+            }
+            if (!ok) break;
+            const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
+            const int y = ty * DC_TILE_H + row, x = tx * DC_TILE_W + col;
+            const bool active = y < a.Ho && x < a.Wo && !((word >> (8 * (row & 3) + col)) & 1u);
+            const int nb = item % a.NB, grp = nb / a.nb_g, c0 = (nb - grp * a.nb_g) * BN + half * CH, n = min(CH, a.Cog - c0);
+            float* const tile_out = a.out + (((size_t)s * a.Ho + ty * DC_TILE_H) * a.Wo + tx * DC_TILE_W) * a.Co + grp * a.Cog + c0;
+            const float* bias = a.bias + grp * a.Cog + c0;
+            if (ctl->odd[seq % kTileFlags] == seq + 1) {
+                // a value of the patch does not split: this pixel once more, by FMAs
+                float* o = tile_out + ((size_t)row * a.Wo + col) * a.Co;
+                const float* w = a.w + (size_t)(grp * a.Cog + c0) * KW * KW * a.Cig;
+#pragma unroll 1
+                for (int j = 0; j < (active ? n : 0); ++j) {
+                    float v = 0.f;
+#pragma unroll 1
+                    for (int t = 0; t < KW * KW; ++t) {
+                        const int iy = y - a.p + t / KW, ix = x - a.p + t % KW;
+                        if (iy < 0 || iy >= a.Hi || ix < 0 || ix >= a.Wi) continue;
+                        const float* p = a.in + (((size_t)s * a.Hi + iy) * a.Wi + ix) * a.Ci + grp * a.Cig;
+                        const float* k = w + ((size_t)j * KW * KW + t) * a.Cig;
+#pragma unroll 1
+                        for (int c = 0; c < a.Cig; ++c) v = fmaf(dc_ld(p + c), __ldg(k + c), v);
+                    }
+                    v += __ldg(bias + j);
+                    o[j] = a.relu ? fmaxf(v, 0.f) : v;
+                }
+                continue;
+            }
+            // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
+            // warp touched 32 lines, and the stores took as long as the MMAs)
+            const uint32_t todo = __ballot_sync(0xffffffffu, active);
+            const int part = lane % (STAGE_CH / 4);
+#pragma unroll
+            for (int c = 0; c < CH; c += STAGE_CH) {
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < STAGE_CH; j += 4)
+                    sts128(stage + lane * STAGE_PITCH + j * 4, __float_as_uint(sum[c + j]), __float_as_uint(sum[c + j + 1]), __float_as_uint(sum[c + j + 2]), __float_as_uint(sum[c + j + 3]));
+                __syncwarp();
+                if (c + 4 * part >= n) continue;                           // channels come in fours
+                const float* pb = bias + c + 4 * part;
+                const float b0 = __ldg(pb), b1 = __ldg(pb + 1), b2 = __ldg(pb + 2), b3 = __ldg(pb + 3);
+#pragma unroll
+                for (int i = 0; i < STAGE_CH / 4; ++i) {
+                    const int p = i * (128 / STAGE_CH) + lane / (STAGE_CH / 4);
+                    const uint4 w = lds128(stage + p * STAGE_PITCH + part * 16);
+                    float4 v = make_float4(__uint_as_float(w.x) + b0, __uint_as_float(w.y) + b1, __uint_as_float(w.z) + b2, __uint_as_float(w.w) + b3);
+                    if (a.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+                    if ((todo >> p) & 1u) *(float4*)(tile_out + ((size_t)(q * 4 + p / 8) * a.Wo + p % 8) * a.Co + c + 4 * part) = v;
+                }
+            }
+        }
+    } else {
+        // ---------------- input patches, split into pieces ----------------
+        const int tid = threadIdx.x - (2 + kSumWarps) * 32;
+        int py[UNITS], px[UNITS], so[UNITS], cg[UNITS];                    // unit: pixel of the patch, its place, its channels; eight lanes, eight pixels
+#pragma unroll
+        for (int i = 0; i < UNITS; ++i) {
+            const int u = tid + i * 32 * kSplitWarps, p = (u >> 5) * 8 + (u & 7), g = (u >> 3) & 3;
+            py[i] = p / PW; px[i] = p - py[i] * PW; cg[i] = 8 * g;
+            so[i] = p < PX ? g * PLANE + p * 16 : -1;
+        }
+        // the patches in order, their loads one patch ahead of the splitting
+        struct Patch { int cc, seq; };                                     // cc < 0: none left
+        int item = blockIdx.x, cc = 0, seq = 0;
+        auto tile_of = [&](int i) { return i < n_items ? __ldcg(a.tile_list + i / a.NB) : 0; };
+        int tile = tile_of(item), y0 = 0, x0 = 0;
+        const float* in = a.in;
+        auto place = [&]() {
+            const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
+            y0 = ty * DC_TILE_H - a.p; x0 = tx * DC_TILE_W - a.p;
+            in = a.in + (size_t)s * a.Hi * a.Wi * a.Ci + item % a.NB / a.nb_g * a.Cig;
+            tile = tile_of(item + gridDim.x);
+        };
+        place();
+        auto load = [&](float4 (&v)[UNITS][2]) -> Patch {
+            if (item >= n_items) return {-1, 0};
+#pragma unroll
+            for (int i = 0; i < UNITS; ++i) {
+                v[i][0] = v[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const int y = y0 + py[i], x = x0 + px[i], left = a.Cig - (cc * kChF + cg[i]);
+                if (so[i] < 0 || left <= 0 || (unsigned)y >= (unsigned)a.Hi || (unsigned)x >= (unsigned)a.Wi) continue;
+                const float* p = in + ((size_t)y * a.Wi + x) * a.Ci + cc * kChF + cg[i];
+                if (a.vec) {
+                    v[i][0] = dc_ld((const float4*)p);
+                    if (left > 4) v[i][1] = dc_ld((const float4*)p + 1);
+                } else {
+                    float e[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) e[k] = k < left ? dc_ld(p + k) : 0.f;
+                    v[i][0] = make_float4(e[0], e[1], e[2], e[3]); v[i][1] = make_float4(e[4], e[5], e[6], e[7]);
+                }
+            }
+            const Patch now = {cc, seq};
+            if (++cc == a.chunks) { cc = 0; ++seq; item += gridDim.x; place(); }
+            return now;
+        };
+        const uint32_t a0 = smem_u32(base);
+        uint32_t slot = 0, phase = 0;
+        auto split = [&](const float4 (&v)[UNITS][2], Patch b) -> bool {
+            const int c_end = 16 * k_steps(b.cc);                          // channels of this patch that the MMAs read
+            if (!f_wait_warp(a_empty0 + 8u * slot, phase ^ 1u, lane, ctl, a.status)) return false;
+            float odd = 0.f;
+#pragma unroll
+            for (int i = 0; i < UNITS; ++i) {
+                if (so[i] < 0 || cg[i] >= c_end) continue;
+                uint32_t p0[4], p1[4], p2[4];
+                split2(v[i][0].x, v[i][0].y, p0[0], p1[0], p2[0], odd);
+                split2(v[i][0].z, v[i][0].w, p0[1], p1[1], p2[1], odd);
+                split2(v[i][1].x, v[i][1].y, p0[2], p1[2], p2[2], odd);
+                split2(v[i][1].z, v[i][1].w, p0[3], p1[3], p2[3], odd);
+                const uint32_t at = a0 + slot * A_SLOT + so[i];
+                sts128(at, p0[0], p0[1], p0[2], p0[3]);
+                sts128(at + PIECE, p1[0], p1[1], p1[2], p1[3]);
+                sts128(at + 2 * PIECE, p2[0], p2[1], p2[2], p2[3]);
+            }
+            if (odd != odd) ctl->odd[b.seq % kTileFlags] = b.seq + 1;
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ctl->a_full[slot]);
+            slot ^= 1u;
+            if (slot == 0) phase ^= 1u;
+            return true;
+        };
+        if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
+        float4 v0[UNITS][2], v1[UNITS][2];
+        Patch b0 = load(v0);
+        while (b0.cc >= 0) {
+            const Patch b1 = load(v1);
+            if (!split(v0, b0) || b1.cc < 0) break;
+            b0 = load(v0);
+            if (!split(v1, b1)) break;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
+    }
+}
+
+// weights [cout][taps][Cig] -> [groups * nb_g][chunks][taps][4][3 BN][8]: plane g of a stage holds channels 8 g ... of its 32, row p * BN + n
+// piece p of output channel n.  `odd` is set by a weight that does not split.
+__global__ void k_pack_f32(const float* w, int taps, int Cig, int Cog, int nb_g, int NB, int chunks, int BN, __nv_bfloat16* out, int32_t* odd)
+{
+    const size_t total = (size_t)NB * chunks * taps * 4 * BN * 8;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        size_t r = i;
+        const int e = (int)(r % 8); r /= 8;
+        const int n = (int)(r % BN); r /= BN;
+        const int g = (int)(r % 4); r /= 4;
+        const size_t stage = r;
+        const int t = (int)(r % taps); r /= taps;
+        const int cc = (int)(r % chunks), nb = (int)(r / chunks);
+        const int grp = nb / nb_g, co = (nb - grp * nb_g) * BN + n, c = cc * kChF + 8 * g + e;
+        float v = co < Cog && c < Cig ? w[((size_t)(grp * Cog + co) * taps + t) * Cig + c] : 0.f;
+        __nv_bfloat16* o = out + ((stage * 4 + g) * 3 * BN + n) * 8 + e;
+        for (int p = 0; p < 3; ++p) {
+            const __nv_bfloat16 b = __float2bfloat16_rn(v);
+            o[(size_t)p * BN * 8] = b;
+            v -= __bfloat162float(b);
+        }
+        if (!(v - v == 0.f)) *odd = 1;
+    }
+}
+
+// An MMA takes some 40 clocks for its pixels whatever its width: a step of 16 channels measured 240 clocks for 32 output channels and 310 for
+// 64.  Wide blocks, then, unless they leave SMs without an item: whichever takes fewer clocks with every tile dirty.
+int f32_bn(const dc_cache* c, const dc_layer_rt& L)
+{
+    const int G = L.d.groups > 1 ? L.d.groups : 1, cog = L.d.cout / G;
+    const long long tiles = (long long)L.tiles_x * L.tiles_y * c->S * G, sms = c->num_sms;
+    const long long narrow = (tiles * dc_div_up(cog, 32) + sms - 1) / sms * 240, wide = (tiles * dc_div_up(cog, 64) + sms - 1) / sms * 310;
+    return narrow < wide ? 32 : 64;
+}
+
+}  // namespace
+
+// Few channels on either side fill a small part of an MMA's 16 by 32; such layers stay on the CUDA cores.
+static bool f32_ok(const dc_cache* c, const dc_layer_desc& d)
+{
+    const int G = d.groups > 1 ? d.groups : 1;
+    return c->cfg.dtype == DC_FP32 && d.kind == DC_CONV && d.sh == 1 && d.sw == 1 && d.kh == d.kw && d.ph == d.pw &&
+           (d.kw == 1 || d.kw == 3 || d.kw == 5) && d.cin / G >= 16 && d.cout / G >= 32 && (d.cout / G) % 4 == 0;
+}
+
+static size_t f32_weight_bytes(const dc_cache* c, const dc_layer_rt& L)
+{
+    const int G = L.d.groups > 1 ? L.d.groups : 1, BN = f32_bn(c, L);
+    return (size_t)G * dc_div_up(L.d.cout / G, BN) * dc_div_up(L.d.cin / G, kChF) * L.d.kh * L.d.kw * 4 * 3 * BN * 16;
+}
+
+int dc_pack_weights_f32(dc_cache* c, int layer)
+{
+    dc_layer_rt& L = c->L[layer];
+    if (!f32_ok(c, L.d) || dc_dense_ok(L) || getenv("DC_NO_TENSOR_CORES")) return DC_OK;
+    const int G = L.d.groups > 1 ? L.d.groups : 1, cig = L.d.cin / G, cog = L.d.cout / G, taps = L.d.kh * L.d.kw;
+    const int BN = f32_bn(c, L), nb_g = dc_div_up(cog, BN), chunks = dc_div_up(cig, kChF);
+    const size_t bytes = f32_weight_bytes(c, L);
+    DC_CUDA(cudaMalloc(&L.weight_f32, bytes));
+    c->bytes += bytes;
+    int grid = (int)((bytes / 6 + 255) / 256); if (grid > c->num_sms * 8) grid = c->num_sms * 8;
+    k_pack_f32<<<grid, 256, 0, c->stream>>>((const float*)L.weight, taps, cig, cog, nb_g, G * nb_g, chunks, BN, (__nv_bfloat16*)L.weight_f32, c->reuse_px + layer);
+    DC_CUDA(cudaGetLastError());
+    return DC_OK;
+}
+
+// Layers with a weight that does not split go to the CUDA cores after all.  dc_pack_weights_f32 has left word in the first n_layers
+// counters of the reuse step (zeroed before); one wait for all layers.
+int dc_settle_weights_f32(dc_cache* c)
+{
+    int32_t odd[DC_MAX_LAYERS];
+    bool any = false;
+    for (int i = 0; i < c->n_layers; ++i) any = any || c->L[i].weight_f32;
+    if (!any) return DC_OK;
+    DC_CUDA(cudaMemcpyAsync(odd, c->reuse_px, sizeof(int32_t) * c->n_layers, cudaMemcpyDeviceToHost, c->stream));
+    DC_CUDA(cudaStreamSynchronize(c->stream));
+    for (int i = 0; i < c->n_layers; ++i) {
+        dc_layer_rt& L = c->L[i];
+        if (!L.weight_f32 || !odd[i]) continue;
+        cudaFree(L.weight_f32);
+        L.weight_f32 = nullptr;
+        c->bytes -= f32_weight_bytes(c, L);
+        const int rc = dc_pack_weights_simt(c, i);
+        if (rc != DC_OK) return rc;
+    }
+    return DC_OK;
+}
+
+template <int BN, int KW>
+static int launch_f32(dc_cache* c, F32Args& a, int grid)
+{
+    constexpr int a_total = 2 * 3 * 4 * 16 * (DC_TILE_W + KW - 1) * (DC_TILE_H + KW - 1), stage = KW * 4 * 3 * BN * 16, staging = kSumWarps * 32 * (f32_stage_ch(BN, KW) + 4) * 4;
+    constexpr int room = (226 * 1024 - (int)sizeof(CtlF) - staging - a_total) / stage;
+    static_assert(room >= 2, "two kernel rows of weights fit");
+    a.stages = room > kStagesF ? kStagesF : room;
+    const size_t smem = (size_t)a_total + (size_t)a.stages * stage + sizeof(CtlF) + staging + 128;
+    static dc_once_per_device attr_set;
+    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_conv_f32<BN, KW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    DC_CUDA(dc_launch_pdl(k_conv_f32<BN, KW>, dim3((unsigned)grid), kThreadsF, smem, c->stream, a));
+    return DC_OK;
+}
+
+int dc_launch_conv_f32(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list, const int32_t* tile_count,
+                       const uint32_t* masks, int max_tiles)
+{
+    dc_layer_rt& L = c->L[layer];
+    const int G = L.d.groups > 1 ? L.d.groups : 1, BN = f32_bn(c, L);
+    F32Args a;
+    a.in = (const float*)in; a.w = (const float*)L.weight; a.wp = (const uint8_t*)L.weight_f32; a.bias = L.bias; a.out = (float*)out;
+    a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks; a.early = dc_lists_settled(c);
+    a.Hi = L.in_h; a.Wi = L.in_w; a.Ci = L.d.cin; a.Ho = L.d.out_h; a.Wo = L.d.out_w; a.Co = L.d.cout;
+    a.p = L.d.ph; a.relu = L.d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
+    a.Cig = L.d.cin / G; a.Cog = L.d.cout / G; a.nb_g = dc_div_up(a.Cog, BN); a.NB = G * a.nb_g; a.chunks = dc_div_up(a.Cig, kChF);
+    a.ks_last = (a.Cig - (a.chunks - 1) * kChF + 15) / 16;
+    a.vec = a.Ci % 4 == 0 && a.Cig % 4 == 0 && (uintptr_t)in % 16 == 0;
+    a.status = c->status; a.wait_ns = kWaitLimitF; a.skip_loads = 0;
+    if (c->debug_stall_ms > 0) { a.wait_ns = (unsigned long long)c->debug_stall_ms * 1000000ull; a.skip_loads = 1; c->debug_stall_ms = 0; }
+    const long long items = (long long)(max_tiles < 1 ? 1 : max_tiles) * a.NB;
+    const int grid = items > c->num_sms ? c->num_sms : (int)items;
+    dc_prof_scope ps(c, DC_ST_CONV);
+    c->launches += 1;
+    if (L.d.kw == 1) return BN == 64 ? launch_f32<64, 1>(c, a, grid) : launch_f32<32, 1>(c, a, grid);
+    if (L.d.kw == 3) return BN == 64 ? launch_f32<64, 3>(c, a, grid) : launch_f32<32, 3>(c, a, grid);
+    return BN == 64 ? launch_f32<64, 5>(c, a, grid) : launch_f32<32, 5>(c, a, grid);
+}

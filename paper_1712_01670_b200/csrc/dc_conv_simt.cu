@@ -1,5 +1,5 @@
-// Partial convolution on CUDA cores for stride-1 1x1, 3x3 and 5x5 layers (float32 caches, and bfloat16 channel counts
-// that the tensor-core kernels do not take), grouped ones included, and for layers with one output pixel per stream.
+// Partial convolution on CUDA cores for stride-1 1x1, 3x3 and 5x5 layers (float32 and bfloat16 channel counts that the
+// tensor-core kernels do not take), grouped ones included, and for layers with one output pixel per stream.
 //   k_conv_simt  register-blocked, packed fp32 FMAs
 //   k_dense      fully-connected layers: one warp per slice of the reduction
 // Only pixels whose bit in the tile's reuse bitmap is clear are written.

@@ -1102,6 +1102,7 @@ def test_bounded_waits_run_out_in_every_scheme(scheme, monkeypatch):
     try:
         assert B.dc_cache_layer_conv_scheme(dc.handle, 1) == scheme
         stall = B.load().dc_debug_stall_next_conv
+        import ctypes
         stall.restype, stall.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]
         want = dc.conv_partial(1, x)
         assert stall(dc.handle, 5) == B.DC_OK
@@ -1127,6 +1128,7 @@ def test_a_cluster_with_one_stalled_cta_stores_nothing(monkeypatch):
     try:
         assert B.dc_cache_layer_conv_scheme(dc.handle, 1) == 10
         stall = B.load().dc_debug_stall_next_conv
+        import ctypes
         stall.restype, stall.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]
         want = dc.conv_partial(1, x)
         assert want.any()
@@ -1312,3 +1314,111 @@ def test_match_walks_leave_the_staged_window(search, block, R):
     assert max(np.abs(m).max() for m in far) > (32 if search == B.DC_SEARCH_DIAMOND or R >= 63 else 28)     # three steps reach 31 or 63
     check_pairs(pairs, block, R, search)
     check_pairs(pairs[:1], block, R, search, skip_k=2)
+
+
+@pytest.mark.parametrize("hi,wi,cin,cout,k,S,groups", [
+    (17, 9, 16, 32, 3, 2, 1),           # one step of 16 channels, tiles cut on both sides
+    (64, 72, 32, 64, 3, 4, 1),          # one whole patch of 32 channels, 64 output channels
+    (113, 113, 64, 64, 3, 6, 1),        # wide blocks, several items per CTA
+    (30, 22, 80, 128, 3, 3, 1),         # a last patch of one step
+    (33, 21, 20, 36, 3, 2, 1),          # channels beyond the last of a step and of a block
+    (40, 30, 48, 64, 5, 3, 1),          # 5 x 5: the largest patch
+    (90, 140, 24, 128, 1, 6, 1),        # 1 x 1
+    (16, 8, 200, 96, 1, 2, 1),          # several 1 x 1 patches to a drain, the last drain not full
+    (24, 20, 40, 72, 3, 2, 2),          # two channel groups
+    (19, 25, 19, 40, 3, 2, 1),          # pixels that no vector load takes
+])
+def test_conv_fp32_on_tensor_cores(hi, wi, cin, cout, k, S, groups):
+    """float32 layers whose operands are split into bf16 pieces: full and partial, against 64-bit sums.  Every product is within
+    2^-25 of the float one; a sum in the tensor core (steps = 2 k of 16 channels and three products, at most 12 for 1 x 1) may
+    be cut by 2^-23 of the terms' magnitudes per step, a sum in registers rounds by 2^-24."""
+    g = rng(hi * 7 + wi + cout)
+    nb = nets.NetBuilder(hi, wi)
+    x0 = nb.conv(-1, cin - 3 if cin % 4 else cin, 1, 1, 0)
+    if nb.shape(x0)[2] < cin:
+        x0 = nb.concat(x0, -1)                                      # an odd channel count: the frame's three channels joined on
+    nb.conv(x0, cout, k, 1, k // 2, 1, groups=groups)
+    li, L = len(nb.layers) - 1, nb.layers[-1]
+    wts = g.normal(0, np.sqrt(2.0 / (k * k * cin / groups)), size=(cout, k, k, cin // groups)).astype(np.float32)
+    bias = g.normal(0, 0.1, size=cout).astype(np.float32)
+    ws = [np.zeros((l["cout"], 1, 1, 3), np.float32) if l["kind"] == 0 else None for l in nb.layers[:-1]] + [wts]
+    bs = [np.zeros(l["cout"], np.float32) if l["kind"] == 0 else None for l in nb.layers[:-1]] + [bias]
+    dc = DeepCache(wi, hi, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_FP32, max_regions=4)
+    try:
+        xin = torch.from_numpy(g.normal(size=(S, hi, wi, cin)).astype(np.float32)).cuda()
+        prev = torch.from_numpy(g.normal(size=(S, hi, wi, cout)).astype(np.float32)).cuda()
+        conv = lambda x, w, b: torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), w, b, padding=k // 2, groups=groups).permute(0, 2, 3, 1)
+        w64 = torch.from_numpy(wts).cuda().double().permute(0, 3, 1, 2)
+        want = conv(xin, w64, torch.from_numpy(bias).cuda().double()).relu()
+        drains = -(-(-(-cin // groups // 32) * k) // (1 if k > 1 else 3))
+        bound = (36 * 2.0 ** -23 + (drains + 4) * 2.0 ** -24) * (conv(xin.abs(), w64.abs(), None) + 1.0)
+        full = dc.conv_partial(li, xin)
+        assert ((full.double() - want).abs() <= bound).all()
+        regs, counts = torch.zeros((S, 4, 6), dtype=torch.int32, device="cuda"), torch.zeros(S, dtype=torch.int32, device="cuda")
+        regs[0, 0] = torch.tensor([1, 2, wi // 2, hi - 5, 2, 1], dtype=torch.int32)
+        regs[1, 0] = torch.tensor([0, 0, wi, hi, 0, 0], dtype=torch.int32)          # a stream with nothing left to compute
+        counts[:2] = 1
+        part = dc.conv_partial(li, xin, prev, regs, counts)
+        made = full.clone()                                         # what is computed does not depend on what is reused
+        made[1] = prev[1]
+        made[0, 2:hi - 3, 1:1 + wi // 2] = prev[0, 1:hi - 4, 2:2 + wi // 2]
+        assert torch.equal(part, made) and dc.status() == B.DC_OK
+        stall = B.load().dc_debug_stall_next_conv
+        import ctypes
+        stall.restype, stall.argtypes = ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]
+        assert stall(dc.handle, 5) == B.DC_OK
+        dc.conv_partial(li, xin)                                    # returns normally; its output is not valid
+        assert dc.status() == B.DC_ERR_TIMEOUT
+        dc.reset()
+        assert torch.equal(dc.conv_partial(li, xin), full) and dc.status() == B.DC_OK
+    finally:
+        dc.close()
+
+
+def test_conv_fp32_on_tensor_cores_with_values_that_do_not_split():
+    """Infinities, NaN and the largest floats come out as from a chain of FMAs; tiles without them are not touched."""
+    g = rng(77)
+    nb = nets.NetBuilder(48, 40)
+    nb.conv(nb.conv(-1, 32, 1, 1, 0), 64, 3, 1, 1, 0)
+    wts = g.normal(0, 0.1, size=(64, 3, 3, 32)).astype(np.float32)
+    wts[5] = 0.5                                                   # exact in one piece: the others are zero
+    zero = np.zeros(64, np.float32)
+    dc = DeepCache(40, 48, nb.layers, [np.zeros((32, 1, 1, 3), np.float32), wts], [zero[:32], zero], n_streams=1, block=16, search_range=4,
+                   dtype=B.DC_FP32, max_regions=4)
+    try:
+        x = torch.from_numpy(g.normal(size=(1, 48, 40, 32)).astype(np.float32)).cuda()
+        clean = dc.conv_partial(1, x)
+        x[0, 3, 3, 7], x[0, 20, 12, 1], x[0, 37, 30, 31], x[0, 37, 12, 4] = float("inf"), float("-inf"), float("nan"), 3.402e38
+        got = dc.conv_partial(1, x)
+        want = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), torch.from_numpy(wts).cuda().double().permute(0, 3, 1, 2), padding=1).permute(0, 2, 3, 1).float()
+        odd = ~torch.isfinite(want) | (want.abs() > 1e30)
+        assert odd.sum() >= 4 * 9 * 63
+        assert torch.equal(torch.isnan(got), torch.isnan(want))
+        assert torch.equal(got[torch.isinf(want)], want[torch.isinf(want)])
+        big = odd & torch.isfinite(want)
+        assert torch.allclose(got[big], want[big], rtol=1e-6)
+        assert (got[~odd] - clean[~odd]).abs().max() < 1e-4
+        far = torch.ones((48, 40), dtype=torch.bool, device="cuda")
+        for y, xx in ((3, 3), (20, 12), (37, 30), (37, 12)):       # whole tiles whose patch holds one of them
+            far[max(0, (y - 1) // 16 * 16):(y + 1) // 16 * 16 + 16, max(0, (xx - 1) // 8 * 8):(xx + 1) // 8 * 8 + 8] = False
+        assert far.sum() > 500 and torch.equal(got[0][far], clean[0][far])
+    finally:
+        dc.close()
+
+
+def test_conv_fp32_weights_that_do_not_split(monkeypatch):
+    g = rng(78)
+    nb = nets.NetBuilder(24, 40)
+    nb.conv(nb.conv(-1, 16, 1, 1, 0), 32, 3, 1, 1, 0)
+    wts = g.normal(0, 0.1, size=(32, 3, 3, 16)).astype(np.float32)
+    wts[3, 1, 1, 2] = 3.402e38
+    x = torch.from_numpy(g.uniform(-0.2, 0.2, size=(1, 24, 40, 16)).astype(np.float32)).cuda()
+    out = []
+    for cores in (False, True):
+        if cores:
+            monkeypatch.setenv("DC_NO_TENSOR_CORES", "1")
+        dc = DeepCache(40, 24, nb.layers, [np.zeros((16, 1, 1, 3), np.float32), wts], [np.zeros(16, np.float32), np.zeros(32, np.float32)], n_streams=1,
+                       block=16, search_range=4, dtype=B.DC_FP32, max_regions=4)
+        out.append(dc.conv_partial(1, x))
+        dc.close()
+    assert torch.isfinite(out[0]).all() and torch.equal(*out)
