@@ -372,8 +372,10 @@ __global__ void k_lrn(const T* in, int H, int W, int C, int S, int r, float alph
     }
 }
 
-// The same for 16-byte vectors of channels, R known: the (2 R + 1)^2 loads of a vector are independent.  beta = 3/4 (the
-// default) takes two correctly rounded square roots and a division in place of powf, which dominated the kernel.
+// The same for 16-byte vectors of channels, R known.  A thread takes Y rows of one column, so that the squares of a row are summed along x
+// once for all the outputs above and below it, and beta = 3/4 (the default) takes two reciprocal square roots (inverse_3_4).
+// What bounds it: instructions (some 200 per vector of eight channels) and the loads behind them.  16 streams, 32 channels at 128 x 160, R = 1: 43 us (a thread per output, two correctly
+// rounded square roots and a division), 24 now; 64 channels at 32 x 40, R = 2, Y = 1: 14, 10.
 template <typename T> struct Unpack;
 template <> struct Unpack<float> {
     static __device__ __forceinline__ void get(uint4 v, float* f) { f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w); }
@@ -395,52 +397,94 @@ template <> struct Unpack<__nv_bfloat16> {
     }
 };
 
-template <typename T, int R>
-__global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, unsigned cv, float alpha_n2, float beta, float kappa, unsigned total, uint4* out,
+// d^(-3/4): d^(-1/2) and then (d^(1/2))^(-1/2), each with one Newton step (relative error below 2^-23 together, as the two rounded square
+// roots and the division that they replace).
+__device__ __forceinline__ float rsqrt_step(float d)
+{
+    const float y = rsqrtf(d), e = fmaf(-d * y, y, 1.f);
+    return fmaf(0.5f * y, e, y);
+}
+__device__ __forceinline__ float inverse_3_4(float d)
+{
+    const float y = rsqrt_step(d);
+    return y * rsqrt_step(d * y);
+}
+
+template <typename T, int R, int Y>
+__global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, unsigned cv, float alpha_n2, float beta, float kappa, unsigned strips, unsigned total, uint4* out,
                                                  const uint32_t* masks, int tiles_x, int tiles_y)
 {
     constexpr int N = Vec16<T>::N;
     dc_pdl_wait();
     dc_pdl_release();
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const unsigned t = i / cv, c = i - t * cv, u = t / (unsigned)W, s = u / (unsigned)H;
-        const int x = (int)(t - u * (unsigned)W), y = (int)(u - s * (unsigned)H);
-        if (masks) {                                             // pixel filled from the cache
-            const size_t tile = ((size_t)s * tiles_y + y / DC_TILE_H) * tiles_x + x / DC_TILE_W;
-            const int bit = DC_TILE_BIT(y % DC_TILE_H, x % DC_TILE_W);
-            if ((masks[tile * 4 + (bit >> 5)] >> (bit & 31)) & 1u) continue;
-        }
-        const uint4* base = in + (size_t)s * H * W * cv + c;
-        float sum[N], mid[N];
+        const unsigned t = i / cv, c = i - t * cv, u = t / (unsigned)W, s = u / strips;
+        const int x = (int)(t - u * (unsigned)W), y0 = (int)(u - s * strips) * Y;
+        uint32_t todo = 0;                                       // rows to write: inside the map and not filled from the cache
 #pragma unroll
-        for (int k = 0; k < N; ++k) sum[k] = 0.f;
+        for (int k = 0; k < Y; ++k)
+            if (y0 + k < H) todo |= 1u << k;
+        if (masks) {
+            const size_t col = (size_t)s * tiles_y * tiles_x + x / DC_TILE_W;
 #pragma unroll
-        for (int dy = -R; dy <= R; ++dy) {
-            uint4 v[2 * R + 1];
-#pragma unroll
-            for (int dx = -R; dx <= R; ++dx) {
-                const int yy = y + dy, xx = x + dx;
-                v[dx + R] = yy >= 0 && yy < H && xx >= 0 && xx < W ? dc_ld(base + ((size_t)yy * W + xx) * cv) : make_uint4(0, 0, 0, 0);
+            for (int k = 0; k < Y; ++k) {
+                const int y = min(y0 + k, H - 1), bit = DC_TILE_BIT(y % DC_TILE_H, x % DC_TILE_W);
+                if ((masks[(col + (size_t)(y / DC_TILE_H) * tiles_x) * 4 + (bit >> 5)] >> (bit & 31)) & 1u) todo &= ~(1u << k);
             }
+        }
+        if (todo == 0) continue;
+        const size_t at = ((size_t)s * H + y0) * W + x;
+        const uint4* base = in + at * cv + c;
+        float sum[Y][N];
+#pragma unroll
+        for (int k = 0; k < Y; ++k)
+#pragma unroll
+            for (int j = 0; j < N; ++j) sum[k][j] = 0.f;
+        uint4 v[Y + 2 * R][2 * R + 1], mid[Y];                   // the strip's input: all loads at once
+#pragma unroll
+        for (int r = 0; r < Y + 2 * R; ++r)
+#pragma unroll
+            for (int dx = 0; dx <= 2 * R; ++dx) {
+                const bool in_map = y0 + r - R >= 0 && y0 + r - R < H && x + dx - R >= 0 && x + dx - R < W;
+                v[r][dx] = in_map ? dc_ld(base + ((ptrdiff_t)(r - R) * W + (dx - R)) * cv) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+        for (int r = 0; r < Y + 2 * R; ++r) {
+            float row[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) row[j] = 0.f;
 #pragma unroll
             for (int dx = 0; dx <= 2 * R; ++dx) {
                 float f[N];
-                Unpack<T>::get(v[dx], f);
-                if (dy == 0 && dx == R) {
+                Unpack<T>::get(v[r][dx], f);
 #pragma unroll
-                    for (int k = 0; k < N; ++k) mid[k] = f[k];
-                }
-#pragma unroll
-                for (int k = 0; k < N; ++k) sum[k] = fmaf(f[k], f[k], sum[k]);
+                for (int j = 0; j < N; ++j) row[j] = fmaf(f[j], f[j], row[j]);
             }
+            if (r >= R && r < Y + R) mid[r - R] = v[r][R];
+#pragma unroll
+            for (int k = 0; k < Y; ++k)
+                if (r - R - k >= -R && r - R - k <= R) {
+#pragma unroll
+                    for (int j = 0; j < N; ++j) sum[k][j] += row[j];
+                }
         }
 #pragma unroll
-        for (int k = 0; k < N; ++k) {
-            const float d = fmaf(alpha_n2, sum[k], kappa);
-            if (beta == 0.75f && d > 0.f) { const float r = __fsqrt_rn(d); mid[k] = __fdiv_rn(mid[k], r * __fsqrt_rn(r)); }
-            else mid[k] *= powf(d, -beta);
+        for (int k = 0; k < Y; ++k) {
+            if (!((todo >> k) & 1u)) continue;
+            float f[N];
+            Unpack<T>::get(mid[k], f);
+            bool plain = beta == 0.75f;
+#pragma unroll
+            for (int j = 0; j < N; ++j) { sum[k][j] = fmaf(alpha_n2, sum[k][j], kappa); plain = plain && sum[k][j] > 1e-30f && sum[k][j] < 1e30f; }
+            if (plain) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) f[j] *= inverse_3_4(sum[k][j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < N; ++j) f[j] *= powf(sum[k][j], -beta);
+            }
+            out[(at + (size_t)k * W) * cv + c] = Unpack<T>::put(f);
         }
-        out[i] = Unpack<T>::put(mid);
     }
 }
 
@@ -639,12 +683,18 @@ int dc_launch_lrn(dc_cache* c, int layer, const void* in, void* out, const uint3
     const size_t each = (size_t)L.d.out_h * L.d.out_w * cv;                  // of one stream
     const size_t per = (L.d.cout * c->elt) % 16 == 0 && (r == 1 || r == 2) ? units_per_piece(c, each) : 0;
     for (size_t s0 = 0; per > 0; s0 += per) {
-        const size_t nv = ((size_t)c->S - s0 < per ? (size_t)c->S - s0 : per) * each;
+        const size_t streams = (size_t)c->S - s0 < per ? (size_t)c->S - s0 : per;
+        // strips of two rows where they leave a wave of threads
+        const int Y = streams * each >= (size_t)c->num_sms * 2048 * 2 ? 2 : 1;
+        const unsigned strips = (unsigned)dc_div_up(L.d.out_h, Y);
+        const size_t nv = streams * strips * L.d.out_w * cv;
         const dim3 grid((unsigned)grid_for(c, nv, 256));
         const uint32_t* bits = masks ? masks + s0 * L.tiles_x * L.tiles_y * 4 : nullptr;
-#define DC_LRN_VEC(T, R) DC_CUDA(dc_launch_pdl(k_lrn_vec<T, R>, grid, 256, 0, c->stream, (const uint4*)in + s0 * each, L.d.out_h, L.d.out_w, cv, an, beta, kappa, (unsigned)nv, (uint4*)out + s0 * each, bits, L.tiles_x, L.tiles_y))
-        if (r == 1) DISPATCH(c, DC_LRN_VEC(float, 1), DC_LRN_VEC(__nv_bfloat16, 1));
-        else DISPATCH(c, DC_LRN_VEC(float, 2), DC_LRN_VEC(__nv_bfloat16, 2));
+#define DC_LRN_VEC(T, R, Y) DC_CUDA(dc_launch_pdl(k_lrn_vec<T, R, Y>, grid, 256, 0, c->stream, (const uint4*)in + s0 * each, L.d.out_h, L.d.out_w, cv, an, beta, kappa, strips, (unsigned)nv, (uint4*)out + s0 * each, bits, L.tiles_x, L.tiles_y))
+        if (r == 1 && Y == 2) DISPATCH(c, DC_LRN_VEC(float, 1, 2), DC_LRN_VEC(__nv_bfloat16, 1, 2));
+        else if (r == 1) DISPATCH(c, DC_LRN_VEC(float, 1, 1), DC_LRN_VEC(__nv_bfloat16, 1, 1));
+        else if (Y == 2) DISPATCH(c, DC_LRN_VEC(float, 2, 2), DC_LRN_VEC(__nv_bfloat16, 2, 2));
+        else DISPATCH(c, DC_LRN_VEC(float, 2, 1), DC_LRN_VEC(__nv_bfloat16, 2, 1));
 #undef DC_LRN_VEC
         c->launches += 1;
         if (s0 + per >= (size_t)c->S) return DC_OK;
