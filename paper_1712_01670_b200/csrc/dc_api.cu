@@ -456,7 +456,7 @@ int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* 
     const uintptr_t in_at = (uintptr_t)in_map_dev, out_at = (uintptr_t)out_map_dev;
     if (in_at % c->elt || out_at % c->elt) return DC_ERR_ARG;
     // the tensor-core kernels store vectors, and their loads take the map from a 16-byte boundary (copies of few-channel maps: from any)
-    if (dc_conv_bf16_supported(c, layer) && (out_at % 16 || (in_at % 16 && L.d.cin % 16 == 0 && !L.s2d_s))) return DC_ERR_ARG;
+    if (dc_conv_bf16_supported(c, layer) && !dc_conv_any_element(c, layer, in_map_dev, out_map_dev) && (out_at % 16 || (in_at % 16 && L.d.cin % 16 == 0 && !L.s2d_s))) return DC_ERR_ARG;
     if (regions_dev || n_regions_dev) {
         if (!regions_dev || !n_regions_dev || !prev_out_dev || prev_out_dev == out_map_dev) return DC_ERR_ARG;
         if ((uintptr_t)prev_out_dev % 16 || out_at % 16) return DC_ERR_ARG;      // the reuse copy is a bulk copy

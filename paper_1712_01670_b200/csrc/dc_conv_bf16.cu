@@ -140,7 +140,7 @@ __device__ __forceinline__ void stage_bias(const TcArgs& a, SmemCtl* ctl, int ep
 {
     float* dst = (float*)((uint8_t*)ctl + ctl_bytes(epi_warps));
     const float* src = a.bias + (size_t)a.nb_off * a.BN;
-    for (int i = threadIdx.x; i < a.bias_smem; i += blockDim.x) dst[i] = __ldg(src + i);
+    for (int i = threadIdx.x; i < a.bias_smem; i += blockDim.x) dst[i] = a.nb_off * a.BN + i < a.Co ? __ldg(src + i) : 0.f;
 }
 
 // Epilogue warps (4 warps = 128 TMEM lanes = the 128 pixels of a tile): for every work item wait
@@ -259,9 +259,10 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
                                bias_pack_bf16<false>(r[v * 8 + 6], r[v * 8 + 7], bv[2 * v + 1].z, bv[2 * v + 1].w));
                 }
                 __syncwarp();
+                const unsigned store = (int)ch_off + c * 32 < a.Co ? act_mask : 0u;     // (a last block that is filled up)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    if ((act_mask >> ((lane >> 2) + 8 * k)) & 1u)
+                    if ((store >> ((lane >> 2) + 8 * k)) & 1u)
                         *(uint4*)(a.out + wb_off[k] + c * 32) = lds128(rd + k * (8 * 80));
                 }
                 __syncwarp();
@@ -987,10 +988,11 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // channel.  A tile lies in memory as the MMA reads it from shared memory, K-major with 128-byte swizzle: the 16-byte piece
 // k8 of row n is at piece k8 ^ (n & 7) of that row, so that a plain bulk copy brings it in place.  (Unswizzled core
 // matrices, the layout before, cost the MMAs shared-memory time.)
-__global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin, int BN, __nv_bfloat16* out)
+// rows: output channels filled up to whole blocks.
+__global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int rows, int taps, int cin, int BN, __nv_bfloat16* out)
 {
     const int kchunks = (cin + 63) / 64;
-    const size_t total = (size_t)cout * taps * kchunks * 64;
+    const size_t total = (size_t)rows * taps * kchunks * 64;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         size_t r = i;
         const int e = (int)(r & 7); r >>= 3;
@@ -999,7 +1001,7 @@ __global__ void k_pack_halo(const __nv_bfloat16* w, int cout, int taps, int cin,
         const int cc = (int)(r % kchunks); r /= kchunks;
         const int tap = (int)(r % taps); const int nb = (int)(r / taps);
         const int ch = cc * 64 + (piece ^ (n & 7)) * 8 + e;
-        out[i] = ch < cin ? w[((size_t)(nb * BN + n) * taps + tap) * cin + ch] : __float2bfloat16(0.f);
+        out[i] = ch < cin && nb * BN + n < cout ? w[((size_t)(nb * BN + n) * taps + tap) * cin + ch] : __float2bfloat16(0.f);
     }
 }
 
@@ -1138,10 +1140,14 @@ static void set_wait_limit(dc_cache* c, TcArgs& a)
 // [cout][kh][kw][cin / groups] need no slicing, and the kernel adds the group's first channel block (nb_off) to the
 // channel blocks it reads weights for and writes.  This is the layer as one group sees it.
 static int n_groups(const dc_layer_desc& d) { return d.groups > 1 ? d.groups : 1; }
+// Output channels come in blocks of 32.  An ungrouped layer whose channels do not is seen with them filled up (weight rows beyond the last
+// are zeros, by the loads or by k_pack_halo; the epilogue stores what exists): 32 -> 16 channels at 64 x 80, 16 streams, 27 us on
+// the CUDA cores, 7 here.  Single output pixels stay with k_dense, and with more than 4096 channels the bias is not staged.
 static dc_layer_desc group_view(const dc_layer_desc& d)
 {
     dc_layer_desc g = d;
     g.cin = d.cin / n_groups(d); g.cout = d.cout / n_groups(d); g.groups = 1;
+    if (n_groups(d) == 1 && d.cout % 32 != 0 && d.cout % 8 == 0 && d.cout <= 4096 && d.out_h * d.out_w > 1) g.cout = dc_div_up(d.cout, 32) * 32;
     return g;
 }
 
@@ -1239,7 +1245,7 @@ int dc_conv_bf16_supported(const dc_cache* c, int layer)
         const dc_layer_desc g = group_view(c->L[layer].d);
         return make_plan(g, p) && (g.cin * 2) % 16 == 0;          // a group's first channel must be 16-byte aligned for its tensor map
     }
-    return make_plan(c->L[layer].d, p) || smallc_ok(c->L[layer].d) || pad16_ok(c->L[layer].d);
+    return make_plan(group_view(c->L[layer].d), p) || smallc_ok(c->L[layer].d) || pad16_ok(c->L[layer].d);
 }
 
 // The first convolution of a bfloat16 cache reads a rearranged copy of its input: the block map (strided layers) or the
@@ -1259,10 +1265,10 @@ static int pack_halo(dc_cache* c, dc_layer_rt& L, int bn, bool* changed)
 {
     *changed = L.halo_bn != bn;
     if (!*changed) return DC_OK;
-    const int taps = L.d.kh * L.d.kw, cin = L.d.cin / n_groups(L.d);
-    const size_t n = (size_t)L.d.cout * taps * ((cin + 63) / 64) * 64;
+    const int taps = L.d.kh * L.d.kw, cin = L.d.cin / n_groups(L.d), rows = group_view(L.d).cout * n_groups(L.d);
+    const size_t n = (size_t)rows * taps * ((cin + 63) / 64) * 64;
     int grid = (int)((n + 255) / 256); if (grid > c->num_sms * 8) grid = c->num_sms * 8;
-    k_pack_halo<<<grid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, L.d.cout, taps, cin, bn, (__nv_bfloat16*)L.weight_halo);
+    k_pack_halo<<<grid, 256, 0, c->stream>>>((const __nv_bfloat16*)L.weight, L.d.cout, rows, taps, cin, bn, (__nv_bfloat16*)L.weight_halo);
     DC_CUDA(cudaGetLastError());
     L.halo_bn = bn;
     return DC_OK;
@@ -1278,7 +1284,7 @@ int dc_pack_weights_bf16(dc_cache* c, int layer)
     const dc_layer_desc dg = group_view(L.d);                     // the layer itself when it is not grouped
     if (halo_ok(dg, h)) {
         // [cout][taps][cin / groups]: channel blocks never straddle a group (BN divides cout / groups)
-        const size_t n = (size_t)L.d.cout * L.d.kh * L.d.kw * h.kchunks * 64;
+        const size_t n = (size_t)dg.cout * n_groups(L.d) * L.d.kh * L.d.kw * h.kchunks * 64;
         DC_CUDA(cudaMalloc(&L.weight_halo, n * 2));
         c->bytes += n * 2;
         bool changed;
@@ -1298,7 +1304,7 @@ int dc_pack_weights_bf16(dc_cache* c, int layer)
         DC_CUDA(cudaGetLastError());
         return DC_OK;
     }
-    if (make_plan(L.d, p) || !smallc_ok(L.d)) return DC_OK;
+    if (make_plan(dg, p) || !smallc_ok(L.d)) return DC_OK;
     const int taps = L.d.kh * L.d.kw, kblocks = (taps + 1) / 2 * 2;
     const size_t wbytes = (size_t)kblocks * L.d.cout * 16, pbytes = (size_t)c->S * L.in_h * L.in_w * 16;
     DC_CUDA(cudaMalloc(&L.weight_packed, wbytes));
@@ -1638,6 +1644,7 @@ static bool cluster_fits(const dc_cache* c, const dc_layer_rt& L, const dc_layer
 // 0.3 % longer than the fastest one of each layer.
 static int cluster_rule(const dc_cache* c, const dc_layer_rt& L, const dc_layer_desc& d)
 {
+    if (L.d.cout % 32 != 0) return 0;                             // its finish knows whole blocks alone
     const int steps = d.kh * d.kw * ((d.cin + 63) / 64);
     const struct { int cs, steps; } take[3] = {{8, 48}, {4, 16}, {2, 26}};
     for (const auto& t : take)
@@ -1751,7 +1758,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     if (c->cfg.dtype != DC_BF16 || !encode_fn() || getenv("DC_NO_TENSOR_CORES")) return DC_OK;
     const bool grouped = n_groups(L.d) > 1;
     if (grouped && !dc_conv_bf16_supported(c, layer)) return DC_OK;
-    const dc_layer_desc de = grouped ? group_view(L.d) : (pad16_ok(L.d) ? padded16(L.d) : L.d);
+    const dc_layer_desc de = !grouped && pad16_ok(L.d) ? padded16(L.d) : group_view(L.d);
     const bool generic = make_plan(de, p);
     if (!generic && (grouped || !smallc_ok(L.d))) return DC_OK;
     if (getenv("DC_CONV_NO_TUNE")) return DC_OK;
@@ -1786,7 +1793,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
         if (ms < best) { best = ms; best_mt = L.tc_mt; best_bn = L.tc_bn; best_ctas = L.tc_ctas; best_flat = L.flat; best_ew = L.tc_ew; best_cs = L.tc_cs; }
     };
     // clusters of CTAs sum in parts, so their size follows from the layer's sizes; the other kernels are then not timed
-    const bool may_cluster = generic && !(de.cin < 16) && L.d.cin == de.cin * n_groups(L.d);
+    const bool may_cluster = generic && !(de.cin < 16) && L.d.cout % 32 == 0 && L.d.cin == de.cin * n_groups(L.d);
     const int cs = may_cluster && (only == 0 || only == 10) ? cluster_rule(c, L, de) : 0;
     // one CTA per SM with four or eight epilogue warps, or two CTAs per SM with four each
     for (int shape = 0; shape < 3 && cs == 0; ++shape) {
@@ -1808,7 +1815,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
                 L.tc_mt = mt; L.tc_bn = bn;
                 trial("tap-by-tap kernel");
                 // flat tiles where the 16 x 8 blocks leave a good part of their pixels outside the map
-                if (L.tiles_flat * 20 <= L.tiles_x * L.tiles_y * c->S * 19 || only >= 8) {
+                if (L.d.cout % 32 == 0 && (L.tiles_flat * 20 <= L.tiles_x * L.tiles_y * c->S * 19 || only >= 8)) {
                     L.flat = 1;
                     trial("tap-by-tap kernel, flat tiles");
                     L.flat = 0;

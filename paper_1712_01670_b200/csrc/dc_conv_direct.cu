@@ -122,6 +122,13 @@ int dc_conv_bf16_supported(const dc_cache* c, int layer);
 int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                         const int32_t* tile_count, const uint32_t* masks, int max_tiles);
 
+// Layers that the tensor cores take with their output channels filled up to blocks of 32 still take a caller's maps at any element: on
+// the CUDA cores, where such a map begins off a 16-byte boundary.
+bool dc_conv_any_element(const dc_cache* c, int layer, const void* in, const void* out)
+{
+    return c->L[layer].d.cout % 32 != 0 && ((uintptr_t)in % 16 != 0 || (uintptr_t)out % 16 != 0);
+}
+
 // in == nullptr: the layer's operand copy (L.in_s2d or L.in_padded) has been filled already
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                    const int32_t* tile_count, const uint32_t* masks, int max_tiles)
@@ -135,7 +142,7 @@ int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int3
         }
         in = L.in_s2d;
     }
-    if (c->cfg.dtype == DC_BF16 && dc_conv_bf16_supported(c, layer))
+    if (c->cfg.dtype == DC_BF16 && dc_conv_bf16_supported(c, layer) && !dc_conv_any_element(c, layer, in, out))
         return dc_launch_conv_bf16(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
     if (dc_dense_ok(L)) return dc_launch_dense(c, layer, in, out, masks);
     // (an output map that it could not store vectors to takes the kernel below)
@@ -183,7 +190,7 @@ int dc_pack_weights(dc_cache* c, int layer, const float* w_dev, const float* b_d
             if (rc != DC_OK) return rc;
         }
         const int rc = dc_pack_weights_bf16(c, layer);
-        if (rc != DC_OK || dc_conv_bf16_supported(c, layer)) return rc;
+        if (rc != DC_OK || (dc_conv_bf16_supported(c, layer) && L.d.cout % 32 == 0)) return rc;
     }
     const int rc = dc_pack_weights_f32(c, layer);
     return rc != DC_OK || L.weight_f32 ? rc : dc_pack_weights_simt(c, layer);

@@ -843,6 +843,41 @@ def test_conv_on_clusters(hi, wi, cin, cout, k, st, p, S, monkeypatch):
     _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, 10)
 
 
+@pytest.mark.parametrize("scheme", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("hi,wi,cin,cout,k,st,p,S", [
+    (33, 18, 32, 16, 3, 1, 1, 3),        # half of the only block
+    (16, 9, 64, 40, 5, 1, 2, 2),         # one 16-byte piece of the second
+    (20, 24, 48, 120, 3, 1, 1, 1),       # blocks of 128, the last 8 channels absent
+    (30, 33, 16, 24, 3, 2, 1, 2),        # strided: tap by tap alone
+])
+def test_conv_channels_filled_up_to_blocks(scheme, hi, wi, cin, cout, k, st, p, S, monkeypatch):
+    """Output channels that are no multiple of 32 on the tensor-core kernels."""
+    monkeypatch.setenv("DC_CONV_SCHEME", str(scheme))
+    if st == 1 or scheme <= 2:
+        _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, scheme)
+
+
+@pytest.mark.parametrize("st", [1, 2])
+def test_conv_channels_filled_up_take_maps_at_any_element(st):
+    nb = nets.NetBuilder(21, 18)
+    nb.conv(nb.conv(-1, 32, 1, 1, 0), 24, 3, st, 1, 1)
+    ws, bs = nets.random_weights(nb.layers, 5)
+    dc = DeepCache(18, 21, nb.layers, ws, bs, n_streams=2, block=16, search_range=4, dtype=B.DC_BF16, max_regions=4)
+    try:
+        assert B.dc_cache_layer_conv_scheme(dc.handle, 1) > 0
+        x = torch.from_numpy(rng(3).normal(size=(2, 21, 18, 32)).astype(np.float32)).to(dc.tdtype).cuda()
+        want = dc.conv_partial(1, x)
+        off = lambda t: torch.zeros(t.numel() + 8, dtype=dc.tdtype, device="cuda")[1:1 + t.numel()].view(t.shape)
+        xs = off(x)
+        xs.copy_(x)
+        for i, o in ((xs, torch.zeros_like(want)), (x, off(want)), (xs, off(want))):
+            B.dc_conv_partial(dc.handle, 1, i, None, None, None, o)
+            U.assert_map_close(o, want.float().cpu().numpy().astype(np.float64), True, "unaligned")
+        assert dc.status() == B.DC_OK
+    finally:
+        dc.close()
+
+
 @pytest.mark.parametrize("scheme", [8, 9])
 @pytest.mark.parametrize("hi,wi,cin,cout,k,st,p,S", [
     (7, 7, 128, 256, 3, 1, 1, 5),        # 7 pieces per stream: every tile holds pieces of two or three streams
