@@ -238,12 +238,12 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
             if (c->L[i].s2d_s) in = c->L[i].in_s2d;               // the kernels being timed read the block map
             DC_TRY(dc_conv_bf16_autotune(c, i, in));
         }
-    // element-wise adds whose later operand is a convolution on the cluster kernel are done by that kernel
+    // element-wise adds whose later operand is a convolution that takes them along are done by its kernel
     for (int j = 0; j < n && c->executable && cfg.dtype == DC_BF16; ++j) {
         const dc_layer_desc& d = c->L[j].d;
         if (d.kind != DC_ADD || d.in0 < 0 || d.in1 < 0 || d.in0 == d.in1) continue;
         dc_layer_rt& P = c->L[d.in0 > d.in1 ? d.in0 : d.in1];
-        if (P.d.kind == DC_CONV && P.tc_cs > 0 && P.fuse_add < 0) P.fuse_add = j;
+        if (P.d.kind == DC_CONV && P.fuse_add < 0 && dc_conv_takes_add(c, d.in0 > d.in1 ? d.in0 : d.in1)) P.fuse_add = j;
     }
     // who reads the frame as a map, and who reads the resized frame
     c->fused_input = need_input_map; c->resize_feeds = -1;

@@ -220,6 +220,7 @@ int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, co
                             const void* prev_out, void* out, int32_t* count, int32_t* px, unsigned long long* running);
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                    const int32_t* tile_count, const uint32_t* masks, int max_tiles);
+bool dc_conv_takes_add(const dc_cache* c, int layer);
 bool dc_conv_any_element(const dc_cache* c, int layer, const void* in, const void* out);
 // stride-1 layers and single output pixels on CUDA cores (dc_conv_simt.cu)
 bool dc_dense_ok(const dc_layer_rt& L);

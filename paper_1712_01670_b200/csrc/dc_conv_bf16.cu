@@ -52,6 +52,8 @@ struct TcArgs {
     int epi_warps = 4;            // epilogue warps of the CTA: 4 (192 threads) or 8 (320 threads)
     int early = 0;                // tile list, count and bitmaps are older than the kernel before this one (dc_lists_settled): read before the wait for it
     int slab_order = 0;           // tap-by-tap kernel: the steps in the column-slab kernels' order (see StepOrder)
+    // element-wise add of a later layer done here (k_conv_tc<1, true>): add_out = (this layer's output) + add_in (+ ReLU)
+    const __nv_bfloat16* add_in = nullptr; __nv_bfloat16* add_out = nullptr; int add_relu = 0;
     int bias_smem = 0;            // > 0: that many bias values (the launch's NB * BN, from channel block nb_off on) are staged in shared memory behind the control block
 };
 
@@ -152,6 +154,9 @@ __device__ __forceinline__ void stage_bias(const TcArgs& a, SmemCtl* ctl, int ep
 // holds tiles_per_group tiles and this CTA's first one is number tile_sub in it (a pair: 2 and its rank, with a.MT = 1).
 // remote_empty: 0, or the shared::cluster address of the pair leader's tmem_empty[0], on which this CTA's epilogue
 // threads arrive instead of on their own.
+// ADD: the launch visits every tile, and the add that follows is done in the same pass: reused pixels are read back from the output map, where
+// the reuse copy has put them; a step's other operands travel while its accumulator is waited for.
+template <bool ADD>
 __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uint32_t tmem_base, int n_items, int n_tiles, int warp, int lane,
                                               int first_item, int item_stride, int tiles_per_group, int tile_sub, uint32_t remote_empty,
                                               int epi_warps = 4)
@@ -185,16 +190,19 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
         const int tile_c0 = tile_n0, tile_c1 = tile_n1;
         const uint32_t mask_c0 = mask_n0, mask_c1 = mask_n1;
         fetch(item + item_stride);
-        ok = mbar_wait(&ctl->tmem_full[acc], acc_ph, ctl, a.status);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc_fence_after();
+        auto wait_full = [&]() -> bool {
+            ok = mbar_wait(&ctl->tmem_full[acc], acc_ph, ctl, a.status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) tc_fence_after();
+            return ok;
+        };
+        if (!ADD && !wait_full()) break;
         const float* bias = a.bias + (nb + a.nb_off) * a.BN;
         for (int j = 0; j < a.MT; ++j) {
             const int tile = j == 0 ? tile_c0 : tile_c1;
             if (tile < 0) break;
             const bool reused = ((j == 0 ? mask_c0 : mask_c1) >> mbit) & 1u;
-            bool active;
+            bool active, in_map;
             // write-back addressing, once per tile: piece k of this lane is the 16-byte part (lane & 3) of the pixel in
             // tile row q * 4 + k, column lane >> 2 (the warp's 32 pixels are 4 tile rows of 8)
             const size_t row_stride = (size_t)a.Wo * a.Co;
@@ -203,7 +211,8 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
             if (a.flat) {
                 const int gps = a.Ho * a.gpr;
                 const int g = tile * DC_TILE_H + prow, s = g / gps, loc = g - s * gps, y = loc / a.gpr, gx = loc - y * a.gpr;
-                active = g < a.n_groups_all && gx * DC_TILE_W + pcol < a.Wo && !reused;
+                in_map = g < a.n_groups_all && gx * DC_TILE_W + pcol < a.Wo;
+                active = in_map && !reused;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int gk = tile * DC_TILE_H + q * 4 + k, sk = gk / gps, lk = gk - sk * gps, yk = lk / a.gpr, xk = lk - yk * a.gpr;
@@ -212,7 +221,8 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
             } else {
                 const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
                 const int oy = ty * DC_TILE_H + prow, ox = tx * DC_TILE_W + pcol;
-                active = oy < a.Ho && ox < a.Wo && !reused;
+                in_map = oy < a.Ho && ox < a.Wo;
+                active = in_map && !reused;
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     wb_off[k] = ((size_t)s * a.Ho + ty * DC_TILE_H + q * 4 + k) * row_stride + (size_t)(tx * DC_TILE_W + (lane >> 2)) * a.Co + ch_off;
@@ -222,9 +232,22 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
             // directly would make every warp store touch 32 different lines 16 bytes at a time (half-written
             // sectors); instead the warp stages its 32 x 64 bytes in shared memory and writes them back with
             // 4 lanes per pixel, so each pixel's 64 bytes leave as two whole sectors.
-            const unsigned act_mask = __ballot_sync(0xffffffffu, active);
+            const unsigned act_mask = __ballot_sync(0xffffffffu, active), map_mask = ADD ? __ballot_sync(0xffffffffu, in_map) : 0u;
+            uint4 other[4], old[4];                              // ADD: the step's other operands, and its reused pixels
+            auto fetch_add = [&](int c) {
+                if constexpr (ADD) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const unsigned bit = c < c_end ? 1u << ((lane >> 2) + 8 * k) : 0u;
+                        if (map_mask & bit) other[k] = *(const uint4*)(a.add_in + wb_off[k] + c * 32);
+                        if (map_mask & ~act_mask & bit) old[k] = *(const uint4*)(a.out + wb_off[k] + c * 32);
+                    }
+                }
+            };
             const uint32_t stg = smem_u32(ctl->stage[warp - 2]);
             const uint32_t rd = stg + (lane >> 2) * 80 + (lane & 3) * 16, mine = stg + lane * 80;
+            fetch_add(c_begin);
+            if (ADD && !wait_full()) return;
             for (int c = c_begin; c < c_end; ++c) {
                 uint32_t r[32];
                 tmem_ld32(taddr + c * 32, r);
@@ -262,9 +285,19 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
                 const unsigned store = (int)ch_off + c * 32 < a.Co ? act_mask : 0u;     // (a last block that is filled up)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    if ((store >> ((lane >> 2) + 8 * k)) & 1u)
-                        *(uint4*)(a.out + wb_off[k] + c * 32) = lds128(rd + k * (8 * 80));
+                    const unsigned bit = 1u << ((lane >> 2) + 8 * k);
+                    if constexpr (!ADD) {
+                        if (store & bit) *(uint4*)(a.out + wb_off[k] + c * 32) = lds128(rd + k * (8 * 80));
+                    } else if (map_mask & bit) {
+                        uint4 o = old[k];
+                        if (store & bit) {
+                            o = lds128(rd + k * (8 * 80));
+                            *(uint4*)(a.out + wb_off[k] + c * 32) = o;
+                        }
+                        *(uint4*)(a.add_out + wb_off[k] + c * 32) = add_bf16x8(o, other[k], a.add_relu);
+                    }
                 }
+                fetch_add(c + 1);
                 __syncwarp();
             }
         }
@@ -275,7 +308,7 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
     }
 }
 
-template <int MT>
+template <int MT, bool ADD>
 __global__ void __launch_bounds__(kThreadsWide, 1)
 k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const TcArgs a)
 {
@@ -464,7 +497,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         __syncwarp();
     } else {
         // ---------------- epilogue ----------------
-        epilogue_loop(a, ctl, tmem_base, n_items, n_tiles, warp, lane, blockIdx.x, gridDim.x, a.MT, 0, 0u, a.epi_warps);
+        epilogue_loop<ADD>(a, ctl, tmem_base, n_items, n_tiles, warp, lane, blockIdx.x, gridDim.x, a.MT, 0, 0u, a.epi_warps);
     }
     tc_fence_before();
     __syncthreads();
@@ -589,7 +622,7 @@ k_conv_tc_smallc(const __grid_constant__ CUtensorMap tmA, const TcSmallArgs sa)
         }
         __syncwarp();
     } else {
-        epilogue_loop(a, ctl, tmem_base, n_items, n_items, warp, lane, blockIdx.x, gridDim.x, 1, 0, 0u, a.epi_warps);
+        epilogue_loop<false>(a, ctl, tmem_base, n_items, n_items, warp, lane, blockIdx.x, gridDim.x, 1, 0, 0u, a.epi_warps);
     }
     tc_fence_before();
     __syncthreads();
@@ -800,7 +833,7 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
         }
         __syncwarp();
     } else {
-        epilogue_loop(a, ctl, tmem_base, n_items, n_tiles, warp, lane, blockIdx.x, gridDim.x, a.MT, 0, 0u, a.epi_warps);
+        epilogue_loop<false>(a, ctl, tmem_base, n_items, n_tiles, warp, lane, blockIdx.x, gridDim.x, a.MT, 0, 0u, a.epi_warps);
     }
     tc_fence_before();
     __syncthreads();
@@ -973,7 +1006,7 @@ k_conv_tc_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     } else {
         // ---------------- epilogue: this CTA's tile; the accumulator is handed back on the leader's barrier ----------------
         const uint32_t remote_empty = map_to_cta(&ctl->tmem_empty[0], 0);
-        epilogue_loop(a, ctl, tmem_base, n_items, n_tiles, warp, lane, pair, n_pairs, 2, (int)rank, remote_empty);
+        epilogue_loop<false>(a, ctl, tmem_base, n_items, n_tiles, warp, lane, pair, n_pairs, 2, (int)rank, remote_empty);
     }
     tc_fence_before();
     __syncthreads();
@@ -1730,21 +1763,39 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     a.epi_warps = epi_warps_for(ctas);
     a.bias_smem = t_bias_bytes ? d.cout : 0;
     a.slab_order = L.weight_halo != nullptr;
+    a.add_in = (const __nv_bfloat16*)c->add_in; a.add_out = (__nv_bfloat16*)c->add_out; a.add_relu = c->add_relu;
     a.early = dc_lists_settled(c);
     set_wait_limit(c, a);
     static dc_once_per_device attr_set;
     if (attr_set.first(c->device)) {
-        DC_CUDA(cudaFuncSetAttribute(k_conv_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        DC_CUDA(cudaFuncSetAttribute(k_conv_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        DC_CUDA(cudaFuncSetAttribute(k_conv_tc<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        DC_CUDA(cudaFuncSetAttribute(k_conv_tc<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        DC_CUDA(cudaFuncSetAttribute(k_conv_tc<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     }
     long long items = (long long)(((max_tiles < 1 ? 1 : max_tiles) + p.MT - 1) / p.MT) * p.NB;
     int grid = items > c->num_sms * ctas ? c->num_sms * ctas : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
-    if (p.MT == 2) DC_CUDA(dc_launch_pdl(k_conv_tc<2>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
-    else DC_CUDA(dc_launch_pdl(k_conv_tc<1>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
+    if (a.add_out && p.MT != 1) return DC_ERR_CONFIG;
+    if (a.add_out) DC_CUDA(dc_launch_pdl(k_conv_tc<1, true>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
+    else if (p.MT == 2) DC_CUDA(dc_launch_pdl(k_conv_tc<2, false>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
+    else DC_CUDA(dc_launch_pdl(k_conv_tc<1, false>, dim3((unsigned)(grid)), threads_for(a.epi_warps), p.smem, c->stream, tmA, tmB, a));
     c->launches += 1;
     DC_CUDA(cudaGetLastError());
     return DC_OK;
+}
+
+// Does the layer's kernel take the add that follows it along?  On clusters always; tap by tap with one tile per item where every tile of
+// the layer has an SM: there a launch is a chain of latencies and the add one more of them (ResNet-50, one stream: 365 -> 346 us a frame).  With more
+// tiles than that the add as a kernel of its own, which reads half of its operand from L2, is the faster one.
+bool dc_conv_takes_add(const dc_cache* c, int layer)
+{
+    const dc_layer_rt& L = c->L[layer];
+    if (L.tc_cs > 0) return true;
+    TcPlan p;
+    if (c->cfg.dtype != DC_BF16 || !dc_conv_bf16_supported(c, layer) || n_groups(L.d) > 1 || L.s2d_s || L.d.cin < 16 || L.d.cout % 32 != 0 || L.tc_mt != 1) return false;
+    const int ctas = L.tc_ctas == 2 ? 2 : 1;
+    t_ring_kb = 200; t_epi_warps = L.tc_ew == 8 ? 8 : 4; t_bias_bytes = bias_bytes_for(L.d);
+    return make_plan(L.d, p, 1, L.tc_bn, ctas) && (long long)dc_layer_tiles(c, L) * p.NB <= c->num_sms;
 }
 
 // Picks, per convolution layer, the operand scheme and the work-item shape (tiles per item x channels per block)

@@ -962,6 +962,25 @@ def test_residual_add_in_the_cluster_kernel(S, monkeypatch):
     U.run_stream_parity(w, S, [0, 1, 2, 3, 4])
 
 
+@pytest.mark.parametrize("scheme,S", [(1, 1), (1, 9), (8, 4)])
+def test_residual_add_in_the_tap_by_tap_kernel(scheme, S, monkeypatch):
+    """The same with few tiles tap by tap: whole tiles and flat ones, the add with and without ReLU, after a projection too; as many
+    streams as leave every tile an SM (9: 72 or 144 items) take the add along, twice as many do not."""
+    monkeypatch.setenv("DC_CONV_SCHEME", str(scheme))
+    b = nets.NetBuilder(45, 53)
+    x = b.conv(-1, 64, 3, 2, 1)
+    for relu, proj in ((1, False), (0, True), (1, False)):
+        y = b.conv(b.conv(x, 32, 1, 1, 0), 64, 1, 1, 0, 0)
+        x = b.add(y, b.conv(x, 64, 1, 1, 0, 0) if proj else x, relu)
+    w = configs.small_cnn_stream()
+    w.layers, w.dtype, w.width, w.height, w.expire_n = b.layers, configs.DTYPE_BF16, 53, 45, 3
+    inner = w.make_streams
+    w.make_streams = lambda s, f, first=0: _cropped(inner(s, f), 45, 53)
+    U.run_stream_parity(w, S, [0, 1, 2, 3])
+    if S == 9:
+        U.run_stream_parity(w, S + 10, [0, 1])
+
+
 def test_first_frame_of_a_cache_reads_the_weights_of_its_choice():
     """The tuner packs weights for the widths it tries; the first frame, launched at once, must find the final packing: the
     same maps as the same frame given to the warm cache."""
