@@ -894,6 +894,19 @@ def test_conv_flat_tiles_across_rows_and_streams(scheme, hi, wi, cin, cout, k, s
     _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, scheme)
 
 
+@pytest.mark.parametrize("scheme", [8, 9])
+@pytest.mark.parametrize("hi,wi,cin,cout,st,S", [
+    (7, 7, 128, 96, 1, 5),               # rows of one group, the last tile not full
+    (14, 13, 64, 128, 1, 3),             # two groups, the second cut
+    (28, 56, 32, 64, 2, 2),              # every other row and column of the stack, four groups
+    (9, 120, 16, 32, 1, 2),              # a row is a tile
+])
+def test_conv_flat_tiles_as_whole_rows(scheme, hi, wi, cin, cout, st, S, monkeypatch):
+    """1 x 1 layers whose flat tiles are whole rows of the stacked streams."""
+    monkeypatch.setenv("DC_CONV_SCHEME", str(scheme))
+    _one_layer_full_and_partial(hi, wi, cin, cout, 1, st, 0, S, scheme)
+
+
 @pytest.mark.parametrize("hi,wi,cin,cout,k,S,groups", [
     (28, 28, 128, 256, 3, 2, 1),         # two chunks of 64 channels, CTA pairs too
     (13, 13, 96, 64, 5, 3, 1),           # 32-channel steps, a half-empty last chunk
