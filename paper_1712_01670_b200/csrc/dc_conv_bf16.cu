@@ -39,7 +39,8 @@ struct TcArgs {
     const int32_t* tile_list; const int32_t* tile_count; const uint32_t* masks;
     int Ho, Wo, Co, Ci, kh, kw, sh, sw, ph, pw, relu, tiles_x, tiles_y;
     int BN, NB, BK, kchunks, stages, a_bytes, b_bytes;
-    int nb_off;                   // grouped convolution: first channel block of the group this launch computes
+    int nb_off;                   // grouped convolution on clusters: first channel block of the group this launch computes
+    int nb_group, c_group;        // grouped convolution: channel blocks and input channels of a group (see group_view); ungrouped: all of them
     int MT, nbuf;                 // tiles per work item (1 or 2, sharing one B tile); TMEM accumulator sets (2, or 1 when MT * BN = 512)
     uint32_t idesc, sbo, layout_type;
     uint32_t tmem_cols;           // TMEM columns this CTA allocates: a power of two >= nbuf * MT * BN (256 at most when two CTAs share an SM)
@@ -379,7 +380,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             peek(blockIdx.x);
             bool entered = !a.early;
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int row0 = (item % a.NB + a.nb_off) * a.BN, tile = next;
+                const int row0 = (item % a.NB + a.nb_off) * a.BN, tile = next, c_off = item % a.NB / a.nb_group * a.c_group;
                 peek(item + gridDim.x);
                 int fs = 0, fx = 0, fy = 0; bool fon = false;
                 if (j < MT) {
@@ -407,7 +408,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                             tma_load_2d(r.data + b_at, &tmB, w, row0, full0 + r.off);
                         }
                         __syncwarp();                                   // the slot is free and its byte count announced: every lane brings its own group
-                        if (fon) tma_load_4d(r.data + lane * piece, &tmA, c, fx + kx, fy + ky, fs, full0 + r.off);
+                        if (fon) tma_load_4d(r.data + lane * piece, &tmA, c + c_off, fx + kx, fy + ky, fs, full0 + r.off);
                     }
                     r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
                     return true;
@@ -429,7 +430,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 enter();
             }
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int row0 = (item % a.NB + a.nb_off) * a.BN;
+                const int row0 = (item % a.NB + a.nb_off) * a.BN, c_off = item % a.NB / a.nb_group * a.c_group;
                 int sN[MT], xb[MT], yb[MT];
 #pragma unroll
                 for (int j = 0; j < MT; ++j) {
@@ -450,7 +451,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                         }
 #pragma unroll
                         for (int j = 0; j < MT; ++j)
-                            tma_load_4d(r.data + j * a.a_bytes, &tmA, c, xb[j] + kx, yb[j] + ky, sN[j], full0 + r.off);
+                            tma_load_4d(r.data + j * a.a_bytes, &tmA, c + c_off, xb[j] + kx, yb[j] + ky, sN[j], full0 + r.off);
                     }
                     r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
                     return true;
@@ -729,7 +730,7 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                 enter();
             }
             for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int nb = item % a.NB;
+                const int nb = item % a.NB, c_off = nb / a.nb_group * a.c_group;
                 int sN[MT], xb[MT], yb[MT];
 #pragma unroll
                 for (int j = 0; j < MT; ++j) {
@@ -748,13 +749,13 @@ k_conv_tc_halo(const __grid_constant__ CUtensorMap tmA, const TcHaloArgs ha)
                                 mbar_expect_tx(a_full0 + ra.off, (uint32_t)(MT * ha.patch_bytes));
 #pragma unroll
                                 for (int j = 0; j < MT; ++j)
-                                    tma_load_4d(ra.data + j * ha.patch_bytes, &tmA, cc * 64, xb[j] + kx, yb[j], sN[j], a_full0 + ra.off);
+                                    tma_load_4d(ra.data + j * ha.patch_bytes, &tmA, c_off + cc * 64, xb[j] + kx, yb[j], sN[j], a_full0 + ra.off);
                             } else {
                                 mbar_expect_tx(a_full0 + ra.off, (uint32_t)(MT * 8 * ha.PW * ha.PH * 16));
 #pragma unroll
                                 for (int j = 0; j < MT; ++j)
                                     for (int g = 0; g < 8; ++g)
-                                        tma_load_4d(ra.data + j * ha.patch_bytes + g * ha.plane_bytes, &tmA, cc * 64 + g * 8, xb[j], yb[j], sN[j], a_full0 + ra.off);
+                                        tma_load_4d(ra.data + j * ha.patch_bytes + g * ha.plane_bytes, &tmA, c_off + cc * 64 + g * 8, xb[j], yb[j], sN[j], a_full0 + ra.off);
                             }
                         }
                         ra.next(a0, (uint32_t)ha.a_stages, (uint32_t)a_slot);
@@ -1170,10 +1171,11 @@ static void set_wait_limit(dc_cache* c, TcArgs& a)
 }
 
 // A grouped convolution (AlexNet's layers 2, 4, 5) is `groups` independent convolutions, each from its own slice of
-// the input channels to its own slice of the output channels.  One launch per group: the input tensor map starts at
-// the group's first channel and spans the group's channels only (pixels keep the full layer's pitch), the weights
-// [cout][kh][kw][cin / groups] need no slicing, and the kernel adds the group's first channel block (nb_off) to the
-// channel blocks it reads weights for and writes.  This is the layer as one group sees it.
+// the input channels to its own slice of the output channels.  One launch does them all: a block of output channels belongs to one
+// group, and the producer takes its pixels from that group's first channel on (c_group).  The weights [cout][kh][kw][cin / groups] need
+// no slicing.  A chunk that reaches beyond the group's last channel brings the next group's, which no MMA reads (whole steps of
+// 16 channels).  AlexNet grouped, 96 streams: with a launch per group, each with a last round of its own, 363 us a pass, 342 so.  On clusters, for few
+// tiles, a launch per group (nb_off).  This is the layer as one group sees it.
 static int n_groups(const dc_layer_desc& d) { return d.groups > 1 ? d.groups : 1; }
 // Output channels come in blocks of 32.  An ungrouped layer whose channels do not is seen with them filled up (weight rows beyond the last
 // are zeros, by the loads or by k_pack_halo; the epilogue stores what exists): 32 -> 16 channels at 64 x 80, 16 streams, 27 us on
@@ -1183,6 +1185,14 @@ static dc_layer_desc group_view(const dc_layer_desc& d)
     dc_layer_desc g = d;
     g.cin = d.cin / n_groups(d); g.cout = d.cout / n_groups(d); g.groups = 1;
     if (n_groups(d) == 1 && d.cout % 32 != 0 && d.cout % 8 == 0 && d.cout <= 4096 && d.out_h * d.out_w > 1) g.cout = dc_div_up(d.cout, 32) * 32;
+    return g;
+}
+
+// The output channels of a launch: all groups'.
+static dc_layer_desc all_groups(const dc_layer_desc& d)
+{
+    dc_layer_desc g = group_view(d);
+    g.cout *= n_groups(d);
     return g;
 }
 
@@ -1414,7 +1424,7 @@ static int launch_smallc(dc_cache* c, int layer, const void* in, void* out, cons
     return DC_OK;
 }
 
-static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const void* in, void* out, const int32_t* tile_list,
+static int launch_halo(dc_cache* c, int layer, int mt, bool slab, const void* in, void* out, const int32_t* tile_list,
                        const int32_t* tile_count, const uint32_t* masks, int max_tiles)
 {
     dc_layer_rt& L = c->L[layer];
@@ -1426,11 +1436,11 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     bool repacked;
     const int prc = pack_halo(c, L, h.BN, &repacked);
     if (prc != DC_OK) return prc;
-    in = (const uint8_t*)in + (size_t)grp * d.cin * 2;            // the group's first input channel
+    const int G = n_groups(L.d);
     bool hit;
     CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, slab ? 5 : 3, 0, &hit);
     if (!hit) {
-        cuuint64_t dims[4] = {(cuuint64_t)d.cin, (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
+        cuuint64_t dims[4] = {(cuuint64_t)cin_all, (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
         const InPitch ip = in_pitch(L, cin_all);
         cuuint64_t strides[3] = {ip.px * 2, ip.row * 2, (cuuint64_t)L.in_h * ip.row * 2};
         cuuint32_t box[4] = {8, (cuuint32_t)h.PW, (cuuint32_t)h.PH, 1};
@@ -1449,7 +1459,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     a.bias = L.bias; a.out = (__nv_bfloat16*)out; a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;
     a.Ho = d.out_h; a.Wo = d.out_w; a.Co = cout_all; a.Ci = d.cin; a.kh = d.kh; a.kw = d.kw; a.sh = 1; a.sw = 1;
     a.ph = d.ph; a.pw = d.pw; a.relu = d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
-    a.BN = h.BN; a.NB = h.NB; a.nb_off = grp * h.NB; a.BK = 64; a.kchunks = h.kchunks; a.MT = mt; a.nbuf = mt * h.BN * 2 <= 512 ? 2 : 1;
+    a.BN = h.BN; a.NB = h.NB * G; a.nb_off = 0; a.nb_group = h.NB; a.c_group = d.cin; a.BK = 64; a.kchunks = h.kchunks; a.MT = mt; a.nbuf = mt * h.BN * 2 <= 512 ? 2 : 1;
     a.a_bytes = 0; a.b_bytes = h.b_bytes; a.sbo = 128; a.layout_type = 0;
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(h.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.status = c->status;
@@ -1471,7 +1481,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
     a.stages = st > kMaxStages ? kMaxStages : st;
     if (a.stages < 2) return DC_ERR_CONFIG;
     a.epi_warps = epi_warps_for(ctas);
-    a.bias_smem = t_bias_bytes ? d.cout : 0;
+    a.bias_smem = t_bias_bytes ? d.cout * G : 0;
     const size_t smem = (size_t)a_total + (size_t)a.stages * h.b_bytes + ctl_bytes(a.epi_warps) + t_bias_bytes + 1280;
     if (smem > 227 * 1024) return DC_ERR_CONFIG;
     static dc_once_per_device attr_set;
@@ -1481,7 +1491,7 @@ static int launch_halo(dc_cache* c, int layer, int grp, int mt, bool slab, const
         DC_CUDA(cudaFuncSetAttribute(k_conv_tc_halo<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         DC_CUDA(cudaFuncSetAttribute(k_conv_tc_halo<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     }
-    long long items = (long long)(((max_tiles < 1 ? 1 : max_tiles) + mt - 1) / mt) * h.NB;
+    long long items = (long long)(((max_tiles < 1 ? 1 : max_tiles) + mt - 1) / mt) * a.NB;
     int grid = items > c->num_sms * ctas ? c->num_sms * ctas : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
     if (slab) {
@@ -1596,11 +1606,11 @@ int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const
 {
     const int G = n_groups(c->L[layer].d);
     t_ring_kb = c->overlap_mode ? 182 : 200;
-    t_bias_bytes = bias_bytes_for(group_view(c->L[layer].d));
+    t_bias_bytes = bias_bytes_for(all_groups(c->L[layer].d));
     // eight epilogue warps take the registers that the block search of the next frame needs to stay resident beside
     // this kernel: while that overlap is in use the CTA keeps to four
     t_epi_warps = c->L[layer].tc_ew == 8 && !c->overlap_mode ? 8 : 4;
-    for (int grp = 0; grp < G; ++grp) {                           // a grouped layer: one launch per group
+    for (int grp = 0; grp < (c->L[layer].tc_cs > 0 ? G : 1); ++grp) {        // clusters: one launch per group
         int rc = launch_group(c, layer, grp, in, out, tile_list, tile_count, masks, max_tiles);
         if (rc == DC_ERR_CONFIG && t_ring_kb != 200) {            // the layer's tuned shape needs the full rings: it gets them
             t_ring_kb = 200;
@@ -1629,10 +1639,10 @@ static int generic_maps(dc_cache* c, dc_layer_rt& L, const dc_layer_desc& d, con
     if (!enc) return DC_ERR_CUDA;
     bool hit_a, hit_b;
     const int rows = flat_rows_of(L, d);
-    CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, rows ? 9 : L.flat ? 8 : 1, 0, &hit_a);
+    CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, L.tc_cs > 0 ? 10 : rows ? 9 : L.flat ? 8 : 1, 0, &hit_a);
     CUtensorMap* tmBp = tm_find(&L.tm_b, 1, nullptr, weights, 1, p.BN, &hit_b);
     if (!hit_a) {   // input map [S][Hi][Wi][Ci] bf16; box = BK channels x 16 columns x 8 rows x 1 stream
-        cuuint64_t dims[4] = {(cuuint64_t)d.cin, (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
+        cuuint64_t dims[4] = {(cuuint64_t)(L.tc_cs > 0 ? d.cin : cin_all), (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
         const InPitch ip = in_pitch(L, cin_all);
         cuuint64_t strides[3] = {ip.px * 2, ip.row * 2, (cuuint64_t)L.in_h * ip.row * 2};
         // a strided convolution reads every sw-th column / sh-th row: the box spans TW * sw x TH * sh input
@@ -1735,8 +1745,8 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     if (L.tc_cs > 0) return launch_cluster(c, layer, grp, in, out, tile_list, tile_count, masks, max_tiles);
     if (L.flat && L.tc_mt > 2) return DC_ERR_CONFIG;              // flat tiles exist in the tap-by-tap kernel only
     if (L.tc_mt == 7) return launch_pair(c, layer, in, out, tile_list, tile_count, masks, max_tiles);
-    if (L.tc_mt >= 5) return launch_halo(c, layer, grp, L.tc_mt - 4, true, in, out, tile_list, tile_count, masks, max_tiles);
-    if (L.tc_mt >= 3) return launch_halo(c, layer, grp, L.tc_mt - 2, false, in, out, tile_list, tile_count, masks, max_tiles);
+    if (L.tc_mt >= 5) return launch_halo(c, layer, L.tc_mt - 4, true, in, out, tile_list, tile_count, masks, max_tiles);
+    if (L.tc_mt >= 3) return launch_halo(c, layer, L.tc_mt - 2, false, in, out, tile_list, tile_count, masks, max_tiles);
     const bool grouped = n_groups(L.d) > 1;
     const bool pad16 = !grouped && pad16_ok(L.d) && L.weight_packed && L.in_padded;
     const dc_layer_desc d = pad16 ? padded16(L.d) : group_view(L.d);
@@ -1750,7 +1760,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
         c->launches += 1;
         in = L.in_padded;
     }
-    in = (const uint8_t*)in + (size_t)grp * d.cin * 2;            // the group's first input channel (grp = 0 when ungrouped)
+    const int G = n_groups(L.d);
     TcPlan p;
     int ctas = L.tc_ctas == 2 ? 2 : 1;
     if (ctas == 2 && !make_plan(d, p, L.tc_mt, L.tc_bn, 2)) ctas = 1;
@@ -1767,7 +1777,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     a.bias = L.bias; a.out = (__nv_bfloat16*)out; a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks;
     a.Ho = d.out_h; a.Wo = d.out_w; a.Co = cout_all; a.Ci = d.cin; a.kh = d.kh; a.kw = d.kw; a.sh = d.sh; a.sw = d.sw;
     a.ph = d.ph; a.pw = d.pw; a.relu = d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
-    a.BN = p.BN; a.NB = p.NB; a.nb_off = grp * p.NB; a.BK = p.BK; a.kchunks = d.cin / p.BK; a.stages = p.stages; a.MT = p.MT; a.nbuf = p.nbuf;
+    a.BN = p.BN; a.NB = p.NB * G; a.nb_off = 0; a.nb_group = p.NB; a.c_group = d.cin; a.BK = p.BK; a.kchunks = d.cin / p.BK; a.stages = p.stages; a.MT = p.MT; a.nbuf = p.nbuf;
     a.a_bytes = p.a_bytes; a.b_bytes = p.b_bytes; a.sbo = p.sbo; a.layout_type = p.layout_type;
     a.tmem_cols = tmem_cols_for(p.nbuf, p.MT, p.BN);
     // instruction descriptor: D = f32, A = B = bf16, both K-major, N = BN, M = 128
@@ -1775,7 +1785,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     a.status = c->status;
     a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr; a.flat_rows = flat_rows_of(L, d);
     a.epi_warps = epi_warps_for(ctas);
-    a.bias_smem = t_bias_bytes ? d.cout : 0;
+    a.bias_smem = t_bias_bytes ? d.cout * G : 0;
     a.slab_order = L.weight_halo != nullptr;
     a.add_in = (const __nv_bfloat16*)c->add_in; a.add_out = (__nv_bfloat16*)c->add_out; a.add_relu = c->add_relu;
     a.early = dc_lists_settled(c);
@@ -1786,7 +1796,7 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
         DC_CUDA(cudaFuncSetAttribute(k_conv_tc<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         DC_CUDA(cudaFuncSetAttribute(k_conv_tc<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     }
-    long long items = (long long)(((max_tiles < 1 ? 1 : max_tiles) + p.MT - 1) / p.MT) * p.NB;
+    long long items = (long long)(((max_tiles < 1 ? 1 : max_tiles) + p.MT - 1) / p.MT) * a.NB;
     int grid = items > c->num_sms * ctas ? c->num_sms * ctas : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
     if (a.add_out && p.MT != 1) return DC_ERR_CONFIG;
@@ -1865,7 +1875,7 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
         const int ctas = shape == 2 ? 2 : 1;
         L.tc_ctas = ctas; L.tc_ew = shape == 1 ? 8 : 4;
         t_epi_warps = L.tc_ew;                                        // make_plan below sizes the rings for it
-        t_bias_bytes = bias_bytes_for(de);
+        t_bias_bytes = bias_bytes_for(!grouped && pad16_ok(L.d) ? de : all_groups(L.d));
         if (!generic) {                                               // few input channels: one kernel shape, 1 or 2 CTAs per SM
             if (ctas == 2 && tmem_cols_for(2, 1, L.d.cout) > 256) continue;
             trial("few-channel kernel");
