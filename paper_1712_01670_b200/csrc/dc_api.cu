@@ -513,9 +513,11 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
         if (same) { DC_TRY(dc_launch_classify_all(c, cur)); classified = true; }
     }
     c->list_mark = refresh ? -1 : classified ? c->launches : DC_LISTS_FRESH;      // a full frame's lists are constant
+    bool copied = false;                                             // the last layer has filled the caller's buffer itself
     for (int i = 0; i < n; ++i) {
         dc_layer_rt& L = c->L[i];
         const void* in = layer_input(c, L.d.in0);
+        void* also = i == n - 1 && out_map_dev && dc_writes_twice(c, i, out_map_dev) ? out_map_dev : nullptr;
         switch (L.d.kind) {
         case DC_CONV: {
             const int tiles = dc_layer_tiles(c, L);
@@ -539,13 +541,13 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             break;
         }
         case DC_MAXPOOL: {
-            if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_maxpool(c, i, in, L.map[0], nullptr)); break; }
+            if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_maxpool(c, i, in, L.map[0], nullptr, also)); copied = also != nullptr; break; }
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
             if (!refresh) {           // Section 5's three steps on a pooling layer: copy, mark, compute the rest
                 if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
-                DC_TRY(dc_launch_maxpool(c, i, in, out, L.masks));
+                DC_TRY(dc_launch_maxpool(c, i, in, out, L.masks, nullptr));
             } else {
-                DC_TRY(dc_launch_maxpool(c, i, in, out, nullptr));
+                DC_TRY(dc_launch_maxpool(c, i, in, out, nullptr, nullptr));
             }
             L.cur ^= 1;
             break;
@@ -553,7 +555,8 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
         case DC_ADD: {
             const int later = L.d.in0 > L.d.in1 ? L.d.in0 : L.d.in1;
             if (later >= 0 && c->L[later].fuse_add == i) break;       // done by that convolution
-            DC_TRY(dc_launch_add(c, i, in, layer_input(c, L.d.in1)));
+            DC_TRY(dc_launch_add(c, i, in, layer_input(c, L.d.in1), also));
+            copied = also != nullptr;
             break;
         }
         case DC_RELU: DC_TRY(dc_launch_relu(c, i, in)); break;
@@ -583,7 +586,7 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
     c->frame_idx += 1;
     if (refresh) c->frames_full += 1; else c->frames_cached += 1;
     c->last_refreshed = refresh;
-    if (out_map_dev)
+    if (out_map_dev && !copied)
         DC_TRY(dc_launch_copy_map(c, layer_input(c, n - 1), out_map_dev, c->L[n - 1].map_bytes));
     if (stats) return fill_stats(c, refresh, stats);
     return DC_OK;

@@ -239,10 +239,11 @@ bool dc_conv_takes_frame(const dc_cache* c, int layer);      // the layer's oper
 int dc_launch_frame_operand(dc_cache* c, int layer, const uint8_t* frame, size_t pitch);
 int dc_launch_copy_map(dc_cache* c, const void* src, void* dst, size_t bytes);
 int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch);   // frame: 16-byte aligned rows
-int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
+bool dc_writes_twice(const dc_cache* c, int layer, const void* dst);                // also (pooling, add): a second copy of the map, or NULL
+int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks, void* also);
 int dc_launch_lrn(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
 int dc_launch_concat(dc_cache* c, int layer, const void* a, int ca, const void* b, int cb);
-int dc_launch_add(dc_cache* c, int layer, const void* a, const void* b);
+int dc_launch_add(dc_cache* c, int layer, const void* a, const void* b, void* also);
 int dc_launch_relu(dc_cache* c, int layer, const void* a);
 int dc_pack_weights(dc_cache* c, int layer, const float* w_dev, const float* b_dev);
 // true for layers that keep their last output as cached values: convolutions, and max pooling / LRN when cfg.cache_pool

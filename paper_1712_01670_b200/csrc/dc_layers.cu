@@ -185,10 +185,11 @@ template <> struct Vec16<__nv_bfloat16> {
 };
 
 // masks (optional): the layer's per-tile reuse bitmaps; a pixel whose bit is set was filled from the cache.
+// also: the caller's copy of the network's last map, or NULL (here and in the kernels below).
 // K x K windows with K known: the loads of an output vector are independent and travel together (a tap
 // outside the map is moved to the nearest row and column inside, whose tap is in the window too: the maximum is the same).  K = 0: any window, tap after tap.
 template <typename T, int K>
-__global__ void __launch_bounds__(256) k_maxpool_vec(const uint4* in, int Hi, int Wi, unsigned cv, dc_layer_desc L, unsigned total, uint4* out, const uint32_t* masks,
+__global__ void __launch_bounds__(256) k_maxpool_vec(const uint4* in, int Hi, int Wi, unsigned cv, dc_layer_desc L, unsigned total, uint4* out, uint4* also, const uint32_t* masks,
                                                      int tiles_x, int tiles_y)
 {
     dc_pdl_wait();
@@ -232,13 +233,14 @@ __global__ void __launch_bounds__(256) k_maxpool_vec(const uint4* in, int Hi, in
             }
         }
         out[i] = m;
+        if (also) also[i] = m;
     }
 }
 
 // 2 x 2 windows at stride 2 without padding (every window inside the map), no reuse bitmap: the four 16-byte
 // loads of an output vector are independent and issued together; 32-bit index arithmetic.
 template <typename T>
-__global__ void k_maxpool2x2_vec(const uint4* in, int Hi, int Wi, int cv, int out_h, int out_w, unsigned total, uint4* out)
+__global__ void k_maxpool2x2_vec(const uint4* in, int Hi, int Wi, int cv, int out_h, int out_w, unsigned total, uint4* out, uint4* also)
 {
     dc_pdl_wait();
     dc_pdl_release();
@@ -247,7 +249,9 @@ __global__ void k_maxpool2x2_vec(const uint4* in, int Hi, int Wi, int cv, int ou
         const uint4* p = in + (((size_t)s * Hi + 2 * oy) * Wi + 2 * ox) * cv + c;
         const size_t row = (size_t)Wi * cv;
         const uint4 v00 = dc_ld(p), v01 = dc_ld(p + cv), v10 = dc_ld(p + row), v11 = dc_ld(p + row + cv);
-        out[i] = Vec16<T>::vmax(Vec16<T>::vmax(v00, v01), Vec16<T>::vmax(v10, v11));
+        const uint4 m = Vec16<T>::vmax(Vec16<T>::vmax(v00, v01), Vec16<T>::vmax(v10, v11));
+        out[i] = m;
+        if (also) also[i] = m;
     }
 }
 
@@ -328,14 +332,16 @@ template <> struct VecOps<__nv_bfloat16> {
 // after it starts on what this kernel wrote last.  Its operands are not read again in this frame (streaming loads), so
 // they do not push those lines out.  ResNet-50 trunk, 128 streams: 3230 -> 3130 us for the whole pass.
 template <typename T>
-__global__ void k_add_vec(const uint4* a, const uint4* b, size_t nvec, int relu, uint4* out)
+__global__ void k_add_vec(const uint4* a, const uint4* b, size_t nvec, int relu, uint4* out, uint4* also)
 {
     dc_pdl_wait();
     dc_pdl_release();
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
         const size_t k = nvec - 1 - i;
         const uint4 va = __ldcs(a + k), vb = b ? __ldcs(b + k) : make_uint4(0, 0, 0, 0);
-        out[k] = VecOps<T>::add(va, vb, relu);
+        const uint4 v = VecOps<T>::add(va, vb, relu);
+        out[k] = v;
+        if (also) also[k] = v;
     }
 }
 
@@ -591,7 +597,7 @@ int dc_launch_resize(dc_cache* c, int layer, const uint8_t* frame, size_t pitch)
     return DC_OK;
 }
 
-int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks)
+int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks, void* also)
 {
     dc_layer_rt& L = c->L[layer];
     const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
@@ -602,15 +608,15 @@ int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const u
     for (size_t s0 = 0; per > 0; s0 += per) {
         const size_t nv = ((size_t)c->S - s0 < per ? (size_t)c->S - s0 : per) * out1;
         const uint4* from = (const uint4*)in + s0 * in1;
-        uint4* to = (uint4*)out + s0 * out1;
+        uint4 *to = (uint4*)out + s0 * out1, *to2 = also ? (uint4*)also + s0 * out1 : nullptr;
         const uint32_t* bits = masks ? masks + s0 * L.tiles_x * L.tiles_y * 4 : nullptr;
         const dim3 grid((unsigned)grid_for(c, nv, 256));
         if (!masks && L.d.kh == 2 && L.d.kw == 2 && L.d.sh == 2 && L.d.sw == 2 && L.d.ph == 0 && L.d.pw == 0 && 2 * L.d.out_h <= L.in_h && 2 * L.d.out_w <= L.in_w) {
             DISPATCH(c,
-                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<float>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, to)),
-                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<__nv_bfloat16>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, to)));
+                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<float>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, to, to2)),
+                DC_CUDA(dc_launch_pdl(k_maxpool2x2_vec<__nv_bfloat16>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, cv, L.d.out_h, L.d.out_w, (unsigned)nv, to, to2)));
         } else {
-#define DC_POOL(T, K) DC_CUDA(dc_launch_pdl(k_maxpool_vec<T, K>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, (unsigned)cv, L.d, (unsigned)nv, to, bits, L.tiles_x, L.tiles_y))
+#define DC_POOL(T, K) DC_CUDA(dc_launch_pdl(k_maxpool_vec<T, K>, grid, 256, 0, c->stream, from, L.in_h, L.in_w, (unsigned)cv, L.d, (unsigned)nv, to, to2, bits, L.tiles_x, L.tiles_y))
             if (L.d.kh == 3 && L.d.kw == 3) DISPATCH(c, DC_POOL(float, 3), DC_POOL(__nv_bfloat16, 3));
             else if (L.d.kh == 2 && L.d.kw == 2) DISPATCH(c, DC_POOL(float, 2), DC_POOL(__nv_bfloat16, 2));
             else DISPATCH(c, DC_POOL(float, 0), DC_POOL(__nv_bfloat16, 0));
@@ -628,7 +634,7 @@ int dc_launch_maxpool(dc_cache* c, int layer, const void* in, void* out, const u
     return DC_OK;
 }
 
-int dc_launch_add(dc_cache* c, int layer, const void* a, const void* b)
+int dc_launch_add(dc_cache* c, int layer, const void* a, const void* b, void* also)
 {
     dc_layer_rt& L = c->L[layer];
     const size_t n = (size_t)c->S * L.d.out_h * L.d.out_w * L.d.cout;
@@ -638,8 +644,8 @@ int dc_launch_add(dc_cache* c, int layer, const void* a, const void* b)
         const size_t nv = n * c->elt / 16;
         const dim3 grid((unsigned)grid_for(c, nv, 256));
         DISPATCH(c,
-            DC_CUDA(dc_launch_pdl(k_add_vec<float>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0])),
-            DC_CUDA(dc_launch_pdl(k_add_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0])));
+            DC_CUDA(dc_launch_pdl(k_add_vec<float>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0], (uint4*)also)),
+            DC_CUDA(dc_launch_pdl(k_add_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)b, nv, L.d.relu, (uint4*)L.map[0], (uint4*)also)));
     } else {
         const dim3 grid((unsigned)grid_for(c, n, 256));
         DISPATCH(c,
@@ -659,8 +665,8 @@ int dc_launch_relu(dc_cache* c, int layer, const void* a)
         const size_t nv = n * c->elt / 16;
         const dim3 grid((unsigned)grid_for(c, nv, 256));
         DISPATCH(c,
-            DC_CUDA(dc_launch_pdl(k_add_vec<float>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)nullptr, nv, 1, (uint4*)L.map[0])),
-            DC_CUDA(dc_launch_pdl(k_add_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)nullptr, nv, 1, (uint4*)L.map[0])));
+            DC_CUDA(dc_launch_pdl(k_add_vec<float>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)nullptr, nv, 1, (uint4*)L.map[0], (uint4*)nullptr)),
+            DC_CUDA(dc_launch_pdl(k_add_vec<__nv_bfloat16>, grid, 256, 0, c->stream, (const uint4*)a, (const uint4*)nullptr, nv, 1, (uint4*)L.map[0], (uint4*)nullptr)));
     } else {
         const dim3 grid((unsigned)grid_for(c, n, 256));
         DISPATCH(c,
@@ -723,6 +729,15 @@ int dc_launch_concat(dc_cache* c, int layer, const void* a, int ca, const void* 
         DC_CUDA(dc_launch_pdl(k_concat<float>, grid, 256, 0, c->stream, (const float*)a, ca, (const float*)b, cb, pixels, (float*)L.map[0])),
         DC_CUDA(dc_launch_pdl(k_concat<__nv_bfloat16>, grid, 256, 0, c->stream, (const __nv_bfloat16*)a, ca, (const __nv_bfloat16*)b, cb, pixels, (__nv_bfloat16*)L.map[0])));
     return DC_OK;
+}
+
+// May the layer's own kernel write its map a second time, into a caller's buffer?  (Whole maps of 16-byte vectors.)
+bool dc_writes_twice(const dc_cache* c, int layer, const void* dst)
+{
+    const dc_layer_desc& d = c->L[layer].d;
+    if ((uintptr_t)dst % 16 != 0) return false;
+    if (d.kind == DC_MAXPOOL) return !dc_layer_cached(c, layer) && (d.cout * c->elt) % 16 == 0 && units_per_piece(c, (size_t)d.out_h * d.out_w * (d.cout * c->elt / 16)) > 0;
+    return d.kind == DC_ADD && c->L[layer].map_bytes % 16 == 0;
 }
 
 // A map into a caller's buffer: by a kernel where both are 16-byte aligned, so that it joins the chain of kernels before it

@@ -11,7 +11,7 @@
 //   k_search_tss16  Step 2 for 16-pixel blocks with three step search: the same lane layout, one window that
 //              covers the whole reach of the search.
 //   k_verify   Steps 3-4: rounds the mean vector M, scores every block at M (reusing the Step 2
-//              score when the block's own best vector is M); k_verify16_prep / k_verify16_list for 16-pixel blocks.
+//              score when the block's own best vector is M); k_verify16_prep / k_verify16_list, or k_verify16_few, for 16-pixel blocks.
 //   k_merge    Step 5: maximal horizontal runs per block row, merged vertically when the
 //              spans are identical, emitted in (y, x) order by a CTA-wide ordered compaction.
 #include "dc_common.cuh"
@@ -1081,6 +1081,62 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
 // or the range for it, or its own best vector is M, so that Step 2 already holds the score (Section 4's second
 // acceleration, exact in that case) -- and lists the others.  k_verify16_list scores the listed blocks, one
 // half-warp per block and one lane per block row, so that no warp idles on blocks that were settled.
+struct Step4 { int Mx, My, K; bool settled; int ok; };
+// The global motion of stream s, and block b (number gi in all) where no pixels are needed to settle it.
+__device__ __forceinline__ Step4 settle16(const MatchArgs& a, unsigned gi, int s, int b, bool in_grid)
+{
+    const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * 16, y0 = by * 16, bw = min(16, a.W - x0), bh = min(16, a.H - y0);
+    const int4 sums = __ldcg((const int4*)a.acc + s);                            // Step 3: sum dx, sum dy, K (one 16-byte load)
+    Step4 r = {0, 0, sums.z, false, 0};
+    if (r.K > 0) { r.Mx = round_mean(sums.x, r.K); r.My = round_mean(sums.y, r.K); }
+    const bool cand_ok = in_grid && r.K > 0 && abs(r.Mx) <= a.R && abs(r.My) <= a.R && x0 + r.Mx >= 0 && y0 + r.My >= 0 &&
+                         x0 + r.Mx + bw <= a.W && y0 + r.My + bh <= a.H;
+    bool known = false; uint32_t v = 0;
+    if (cand_ok) {
+        const uint32_t own = ((const uint32_t*)a.mv)[gi];                         // (dx, dy) as one word
+        v = a.sse[gi];
+        known = (int16_t)(own & 0xffffu) == r.Mx && (int16_t)(own >> 16) == r.My && v != 0xffffffffu;
+    }
+    r.settled = in_grid && (!cand_ok || known);
+    r.ok = known && v <= a.limit[limit_index(a, bw, bh)];
+    return r;
+}
+// Lane r of 16: the SSE of row r of block b displaced by (Mx, My).
+__device__ __forceinline__ uint32_t score16(const MatchArgs& a, int s, int b, int Mx, int My, int r, bool on)
+{
+    const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * 16, y0 = by * 16, bw = min(16, a.W - x0), bh = min(16, a.H - y0);
+    if (!on || r >= bh) return 0;
+    RowCtx<1> rc;
+    rc.load_block(a.cur + (size_t)s * a.cur_stream + (size_t)y0 * a.cur_pitch + (size_t)x0 * 3, a.cur_pitch, r, 16, bw, bh);
+    // the 48 bytes of the displaced row lie in four aligned 16-byte chunks (rows of the frame copy are padded):
+    // four wide loads instead of thirteen narrow ones, then a word offset that is the same for a whole stream
+    const uint8_t* p = a.prev + (size_t)s * a.prev_stream + (size_t)(y0 + My + r) * a.prev_pitch + (size_t)(x0 + Mx) * 3;
+    const uint4* p16 = (const uint4*)((uintptr_t)p & ~(uintptr_t)15);
+    const uint4 c0 = dc_ld(p16), c1 = dc_ld(p16 + 1), c2 = dc_ld(p16 + 2), c3 = dc_ld(p16 + 3);
+    const uint32_t ww[16] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w, c2.x, c2.y, c2.z, c2.w, c3.x, c3.y, c3.z, c3.w};
+    const uint32_t boff = (uint32_t)(uintptr_t)p & 15u, sh = (boff & 3u) * 8u;
+    uint32_t w[13];
+    switch (boff >> 2) {
+    case 0:
+#pragma unroll
+        for (int j = 0; j < 13; ++j) w[j] = ww[j];
+        break;
+    case 1:
+#pragma unroll
+        for (int j = 0; j < 13; ++j) w[j] = ww[j + 1];
+        break;
+    case 2:
+#pragma unroll
+        for (int j = 0; j < 13; ++j) w[j] = ww[j + 2];
+        break;
+    default:
+#pragma unroll
+        for (int j = 0; j < 13; ++j) w[j] = ww[j + 3];
+        break;
+    }
+    return rc.sse_words(0, w, sh);
+}
+
 __global__ void __launch_bounds__(256) k_verify16_prep(MatchArgs a, uint32_t* list, int32_t* list_count)
 {
     dc_pdl_wait();
@@ -1090,30 +1146,15 @@ __global__ void __launch_bounds__(256) k_verify16_prep(MatchArgs a, uint32_t* li
     const unsigned gi = blockIdx.x * 256u + threadIdx.x;                          // S * Gx * Gy < 2^31
     const bool in_grid = gi < (unsigned)(per * a.S);
     const int s = in_grid ? (int)(gi / (unsigned)per) : a.S - 1, b = in_grid ? (int)(gi - (unsigned)s * per) : 0;
-    const int by = b / a.Gx, bx = b - by * a.Gx;
-    const int x0 = bx * 16, y0 = by * 16, bw = min(16, a.W - x0), bh = min(16, a.H - y0);
-    const int4 sums = __ldcg((const int4*)a.acc + s);                            // Step 3: sum dx, sum dy, K (one 16-byte load)
-    const int K = sums.z;
-    int Mx = 0, My = 0;
-    if (K > 0) { Mx = round_mean(sums.x, K); My = round_mean(sums.y, K); }
-    const bool cand_ok = in_grid && K > 0 && abs(Mx) <= a.R && abs(My) <= a.R && x0 + Mx >= 0 && y0 + My >= 0 &&
-                         x0 + Mx + bw <= a.W && y0 + My + bh <= a.H;
-    bool known = false; uint32_t v = 0;
-    if (cand_ok) {
-        const uint32_t own = ((const uint32_t*)a.mv)[gi];                         // (dx, dy) as one word
-        v = a.sse[gi];
-        known = (int16_t)(own & 0xffffu) == Mx && (int16_t)(own >> 16) == My && v != 0xffffffffu;
-    }
-    const bool settled = in_grid && (!cand_ok || known);
-    const int ok = known && v <= a.limit[limit_index(a, bw, bh)];
-    if (settled) a.matched[gi] = (uint8_t)ok;
-    if (in_grid && b == 0) { a.gmv[3 * s] = Mx; a.gmv[3 * s + 1] = My; a.gmv[3 * s + 2] = K; }
+    const Step4 r = settle16(a, gi, s, b, in_grid);
+    if (r.settled) a.matched[gi] = (uint8_t)r.ok;
+    if (in_grid && b == 0) { a.gmv[3 * s] = r.Mx; a.gmv[3 * s + 1] = r.My; a.gmv[3 * s + 2] = r.K; }
     // matched count: one atomic per warp and stream
     const unsigned same = __match_any_sync(0xffffffffu, s);
-    const unsigned oks = __ballot_sync(0xffffffffu, ok);
+    const unsigned oks = __ballot_sync(0xffffffffu, r.ok);
     if (lane == __ffs(same) - 1 && (oks & same)) atomicAdd(&a.acc[4 * s + 3], __popc(oks & same));
     // the blocks whose pixels must be read
-    const bool todo = in_grid && !settled;
+    const bool todo = in_grid && !r.settled;
     const unsigned tm = __ballot_sync(0xffffffffu, todo);
     if (tm) {
         int base = 0;
@@ -1135,48 +1176,36 @@ __global__ void __launch_bounds__(256) k_verify16_list(MatchArgs a, const uint32
         const bool on = i < n;
         const unsigned gi = on ? list[i] : 0u;
         const int s = (int)(gi / (unsigned)per), b = (int)(gi - (unsigned)s * per);
-        const int by = b / a.Gx, bx = b - by * a.Gx;
-        const int x0 = bx * 16, y0 = by * 16, bw = min(16, a.W - x0), bh = min(16, a.H - y0);
-        const int Mx = a.gmv[3 * s], My = a.gmv[3 * s + 1];
-        uint32_t acc = 0;
-        if (on && r < bh) {
-            RowCtx<1> rc;
-            rc.load_block(a.cur + (size_t)s * a.cur_stream + (size_t)y0 * a.cur_pitch + (size_t)x0 * 3, a.cur_pitch, r, 16, bw, bh);
-            // the 48 bytes of the displaced row lie in four aligned 16-byte chunks (rows of the frame copy are padded):
-            // four wide loads instead of thirteen narrow ones, then a word offset that is the same for a whole stream
-            const uint8_t* p = a.prev + (size_t)s * a.prev_stream + (size_t)(y0 + My + r) * a.prev_pitch + (size_t)(x0 + Mx) * 3;
-            const uint4* p16 = (const uint4*)((uintptr_t)p & ~(uintptr_t)15);
-            const uint4 c0 = dc_ld(p16), c1 = dc_ld(p16 + 1), c2 = dc_ld(p16 + 2), c3 = dc_ld(p16 + 3);
-            const uint32_t ww[16] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w, c2.x, c2.y, c2.z, c2.w, c3.x, c3.y, c3.z, c3.w};
-            const uint32_t boff = (uint32_t)(uintptr_t)p & 15u, sh = (boff & 3u) * 8u;
-            uint32_t w[13];
-            switch (boff >> 2) {
-            case 0:
-#pragma unroll
-                for (int j = 0; j < 13; ++j) w[j] = ww[j];
-                break;
-            case 1:
-#pragma unroll
-                for (int j = 0; j < 13; ++j) w[j] = ww[j + 1];
-                break;
-            case 2:
-#pragma unroll
-                for (int j = 0; j < 13; ++j) w[j] = ww[j + 2];
-                break;
-            default:
-#pragma unroll
-                for (int j = 0; j < 13; ++j) w[j] = ww[j + 3];
-                break;
-            }
-            acc = rc.sse_words(0, w, sh);
-        }
-        const uint32_t sse = __reduce_add_sync(half ? 0xffff0000u : 0x0000ffffu, acc);
+        const uint32_t sse = __reduce_add_sync(half ? 0xffff0000u : 0x0000ffffu, score16(a, s, b, a.gmv[3 * s], a.gmv[3 * s + 1], r, on));
         if (r == 0 && on) {
-            const int ok = sse <= a.limit[limit_index(a, bw, bh)];
+            const int by = b / a.Gx, bx = b - by * a.Gx;
+            const int ok = sse <= a.limit[limit_index(a, min(16, a.W - bx * 16), min(16, a.H - by * 16))];
             a.matched[gi] = (uint8_t)ok;
             if (ok) atomicAdd(&a.acc[4 * s + 3], 1);
         }
     }
+}
+
+// Both in one launch, a half-warp per block from the start, where the blocks are few and a launch counts.  With more blocks than the SMs
+// hold such warps the list deals the work out better (a whole pass in us, one launch and two: 8 full-HD streams, 65 280 blocks, 345
+// and 315; 32 of them 1891 and 1818; 720p, 6 streams, 21 600 blocks, 436 and 418).
+__global__ void __launch_bounds__(256) k_verify16_few(MatchArgs a)
+{
+    dc_pdl_wait();
+    dc_pdl_release();
+    const int lane = threadIdx.x & 31, r = lane & 15, half = lane >> 4, per = a.Gx * a.Gy;
+    const unsigned gi = (blockIdx.x * 8u + (threadIdx.x >> 5)) * 2u + half;
+    const bool in_grid = gi < (unsigned)(per * a.S);
+    const int s = in_grid ? (int)(gi / (unsigned)per) : a.S - 1, b = in_grid ? (int)(gi - (unsigned)s * per) : 0;
+    const Step4 v = settle16(a, gi, s, b, in_grid);
+    const bool todo = in_grid && !v.settled;
+    const uint32_t sse = __reduce_add_sync(half ? 0xffff0000u : 0x0000ffffu, score16(a, s, b, v.Mx, v.My, r, todo));
+    if (r != 0 || !in_grid) return;
+    if (b == 0) { a.gmv[3 * s] = v.Mx; a.gmv[3 * s + 1] = v.My; a.gmv[3 * s + 2] = v.K; }
+    const int by = b / a.Gx, bx = b - by * a.Gx;
+    const int ok = todo ? sse <= a.limit[limit_index(a, min(16, a.W - bx * 16), min(16, a.H - by * 16))] : v.ok;
+    a.matched[gi] = (uint8_t)ok;
+    if (ok) atomicAdd(&a.acc[4 * s + 3], 1);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1459,11 +1488,16 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
         DC_CUDA(dc_launch_pdl(k_accept_own, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a));
     } else if (a.B == 16) {
         dc_prof_scope ps(c, DC_ST_VERIFY);
-        int32_t* todo_count = long_count + 2;                       // zeroed with the Step 3 sums; the walk list is free again
-        DC_CUDA(dc_launch_pdl(k_verify16_prep, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a, (uint32_t*)c->long_list, todo_count));
-        DC_CUDA(dc_launch_pdl(k_verify16_list, dim3((unsigned)min(c->num_sms * 8, dc_div_up(a.S * a.Gx * a.Gy, 16))), 256, 0, c->stream, a,
-                              (const uint32_t*)c->long_list, (const int32_t*)todo_count));
-        c->launches += 1;
+        const int blocks = a.S * a.Gx * a.Gy;
+        if (blocks <= c->num_sms * 64) {
+            DC_CUDA(dc_launch_pdl(k_verify16_few, dim3((unsigned)dc_div_up(blocks, 16)), 256, 0, c->stream, a));
+        } else {
+            int32_t* todo_count = long_count + 2;                       // zeroed with the Step 3 sums; the walk list is free again
+            DC_CUDA(dc_launch_pdl(k_verify16_prep, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a, (uint32_t*)c->long_list, todo_count));
+            DC_CUDA(dc_launch_pdl(k_verify16_list, dim3((unsigned)min(c->num_sms * 8, dc_div_up(a.S * a.Gx * a.Gy, 16))), 256, 0, c->stream, a,
+                                  (const uint32_t*)c->long_list, (const int32_t*)todo_count));
+            c->launches += 1;
+        }
     } else {
         launch_verify_by_block(c, a);
     }

@@ -30,8 +30,14 @@ __device__ __forceinline__ void erode_axis(int x, int w, int k, int s, int p, in
 // Area resize n_in -> n_out: output o averages [floor(o n_in / n_out), ceil((o + 1) n_in / n_out) - 1].
 __device__ __forceinline__ void resize_axis(int x, int w, int n_in, int n_out, int& xo, int& wo)
 {
-    int first = (int)(((long long)x * n_out + n_in - 1) / n_in);
-    int last = (int)(((long long)(x + w) * n_out) / n_in) - 1;
+    int first, last;
+    if (n_in <= 32768 && n_out <= 32768 && (unsigned)x <= 32768u && (unsigned)w <= 32768u) {      // the products fit 32 bits
+        first = (int)(((unsigned)x * (unsigned)n_out + (unsigned)n_in - 1u) / (unsigned)n_in);
+        last = (int)((unsigned)(x + w) * (unsigned)n_out / (unsigned)n_in) - 1;
+    } else {
+        first = (int)(((long long)x * n_out + n_in - 1) / n_in);
+        last = (int)(((long long)(x + w) * n_out) / n_in) - 1;
+    }
     xo = first; wo = last - first + 1;
 }
 
@@ -39,9 +45,29 @@ __device__ __forceinline__ dc_region empty_region() { dc_region e = {0, 0, 0, 0,
 
 // A layer as propagation sees it.  from0 / from1: where the input's rectangle is: kFrame, kPrevious (the layer before, still in
 // registers), kTable (the table in global memory), or one of the kSlots places of the thread in shared memory; keep: the
-// place that this layer's own rectangle takes, or -1.
+// place that this layer's own rectangle takes, or -1.  drop: places whose rectangles no later layer needs (bit mask); closed: no later
+// layer reads the frame's rectangle or the table.
+// window: the rule is that of a sliding window whose strides are powers of two (convolutions, pooling; LRN is one at stride 1, ReLU one of
+// a single pixel): on either axis first = (x + c1) >> sh, last = (x + w + c2) >> sh.
 constexpr int kSlots = 6, kFrame = -1, kPrevious = -2, kTable = -3;
-struct PropLayer { int kind, kh, kw, sh, sw, ph, pw, in_h, in_w, out_h, out_w, in0, in1, from0, from1, keep; };
+struct __align__(16) PropLayer {
+    int window, c1x, c2x, shx, c1y, c2y, shy, from0;
+    int from1, two, in0, in1, keep, drop, closed, kind;
+    int kh, kw, sh, sw, ph, pw, in_h, in_w, out_h, out_w, pad0, pad1;
+};
+
+__device__ __forceinline__ dc_region apply_window(const PropLayer& L, dc_region a)
+{
+    const int dx = (a.x + L.c1x) >> L.shx, dw = ((a.x + a.w + L.c2x) >> L.shx) - dx + 1;
+    const int dy = (a.y + L.c1y) >> L.shy, dh = ((a.y + a.h + L.c2y) >> L.shy) - dy + 1;
+    // the cached side on its own; smaller size wins
+    const int qx = (a.sx + L.c1x) >> L.shx, qw = ((a.sx + a.w + L.c2x) >> L.shx) - qx + 1;
+    const int qy = (a.sy + L.c1y) >> L.shy, qh = ((a.sy + a.h + L.c2y) >> L.shy) - qy + 1;
+    const int w = min(dw, qw), h = min(dh, qh);
+    if (a.w <= 0 || a.h <= 0 || w <= 0 || h <= 0) return empty_region();
+    dc_region o = {dx, dy, w, h, qx, qy};
+    return o;
+}
 
 __device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
 {
@@ -62,12 +88,6 @@ __device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
         dc_region o = {dx, dy, w, h, qx, qy};
         return o;
     }
-    case DC_LRN: {
-        int r = L.ph;
-        if (a.w - 2 * r <= 0 || a.h - 2 * r <= 0) return empty_region();
-        dc_region o = {a.x + r, a.y + r, a.w - 2 * r, a.h - 2 * r, a.sx + r, a.sy + r};
-        return o;
-    }
     case DC_ADD: case DC_CONCAT: {
         // the overlapped region; both inputs must agree on the displacement
         if (b.w <= 0 || b.h <= 0) return empty_region();
@@ -85,13 +105,23 @@ __device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
     }
 }
 
-// One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a later layer than the next one needs (residual
-// branches) wait in shared memory, and so does the layer table: the walk is a chain of a few dozen arithmetic steps per
-// layer (through a table in global memory it was a chain of memory round trips: 48 us for the 71 layers of ResNet-50).
-// alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most
-// of a frame's erode within a few layers, and the reuse step tests every tile against all it is given.
-// out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): rectangles still
-// alive per layer and stream; with it the counters of the reuse step are zeroed.
+// The tables are 8-byte aligned: three stores, not six.
+__device__ __forceinline__ void store_region(dc_region* t, const dc_region& o)
+{
+    uint2* p = (uint2*)t;
+    p[0] = make_uint2(o.x, o.y); p[1] = make_uint2(o.w, o.h); p[2] = make_uint2(o.sx, o.sy);
+}
+
+// One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a later layer than
+// the next one needs (residual branches) wait in shared memory, and so does the layer table: the walk is a chain of a few dozen
+// arithmetic steps per layer (through a table in global memory it was a chain of memory round trips: 48 us for the 71 layers of
+// ResNet-50; with an atomic per rectangle and layer, waited for on the way, 27, 24 so; VGG, 8 full-HD frames, 12.5 and 7.7).  A warp whose rectangles have all vanished,
+// those kept for later layers too, writes the zeros of the layers that are left without walking them.
+// alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most of a
+// frame's erode within a few layers, and the reuse step tests every tile against all it is given.  A warp asks for its places in a
+// layer's list with one atomic and fills them while the next layer is worked out.
+// out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): the lists are wanted, and the
+// counters of the reuse step are zeroed.
 __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions,
                                                    const dc_region* in, const int32_t* n_in, dc_region* table, dc_region* live, int32_t* alive, int32_t* reuse_px,
                                                    int32_t* dirty_count, dc_region* out, int out_begin, int32_t* n_out)
@@ -99,8 +129,8 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
     __shared__ PropLayer sl[DC_MAX_LAYERS];
     extern __shared__ int32_t keep[];                      // [places in use][6][threads]
     __shared__ int32_t count[DC_MAX_LAYERS];
-    const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-    for (int i = tid; i < layer_end * (int)(sizeof(PropLayer) / 4); i += nt) ((int*)sl)[i] = __ldg((const int*)layers + i);
+    const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    for (int i = tid; i < layer_end * (int)(sizeof(PropLayer) / 16); i += nt) ((int4*)sl)[i] = __ldg((const int4*)layers + i);
     if (tid < DC_MAX_LAYERS) count[tid] = 0;
     dc_pdl_wait();
     dc_pdl_release();
@@ -109,9 +139,10 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
     const int n = min(n_in[s], max_regions);              // a caller's count beyond the table is cut, never written
     // a caller's list has zeros behind its rectangles
     const int rows = out ? max_regions : n;
-    for (int i = blockIdx.y * nt + tid; i < rows; i += gridDim.y * nt) {
+    for (int first = blockIdx.y * nt; first < rows; first += gridDim.y * nt) {
+        const int i = first + tid;
         const size_t slot = (size_t)s * max_regions + i;
-        const bool on = i < n;
+        const bool on = i < n, there = i < rows;
         const dc_region r0 = on ? in[slot] : empty_region();
         dc_region prev = r0;
         auto fetch = [&](int from, int layer) -> dc_region {
@@ -122,19 +153,44 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
             dc_region r = {k[0], k[nt], k[2 * nt], k[3 * nt], k[4 * nt], k[5 * nt]};
             return r;
         };
-        for (int l = 0; l < layer_end; ++l) {
+        uint32_t kept = 0;                                             // places that hold a living rectangle of this thread
+        unsigned noted = 0;                                            // the warp's living rectangles of the layer before (prev), and their
+        int place = 0;                                                 // first place in that layer's list (lane 0)
+        auto list_prev = [&](int layer) {
+            const int at = __shfl_sync(0xffffffffu, place, 0) + __popc(noted & ((1u << lane) - 1u));
+            if ((noted >> lane) & 1u) store_region(live + layer * layer_stride + (size_t)s * max_regions + at, prev);
+        };
+        int l = 0;
+        for (bool dead = i - lane >= rows; l < layer_end && !dead; ++l) {
             const PropLayer& L = sl[l];
             const dc_region a = fetch(L.from0, L.in0);
-            const dc_region b = L.kind == DC_ADD || L.kind == DC_CONCAT ? fetch(L.from1, L.in1) : a;
-            const dc_region o = apply_layer(L, a, b);
+            dc_region o;
+            if (L.window) o = apply_window(L, a);
+            else o = apply_layer(L, a, L.two ? fetch(L.from1, L.in1) : a);
+            kept &= ~(uint32_t)L.drop;
             if (L.keep >= 0) {
                 int32_t* k = keep + L.keep * 6 * nt + tid;
                 k[0] = o.x; k[nt] = o.y; k[2 * nt] = o.w; k[3 * nt] = o.h; k[4 * nt] = o.sx; k[5 * nt] = o.sy;
+                kept = o.w > 0 ? kept | (1u << L.keep) : kept & ~(1u << L.keep);
             }
-            table[l * layer_stride + slot] = o;
-            if (out && l >= out_begin) out[(l - out_begin) * layer_stride + slot] = o;
-            if (o.w > 0 && alive) live[l * layer_stride + (size_t)s * max_regions + atomicAdd(&count[l], 1)] = o;
+            if (there) {
+                store_region(table + l * layer_stride + slot, o);
+                if (out && l >= out_begin) out[(l - out_begin) * layer_stride + slot] = o;
+            }
+            if (noted) list_prev(l - 1);
+            const unsigned living = __ballot_sync(0xffffffffu, o.w > 0);
+            noted = alive ? living : 0u;
+            if (noted && lane == 0) place = atomicAdd(&count[l], __popc(noted));
+            dead = !living && L.closed && !__any_sync(0xffffffffu, kept != 0);
             prev = o;
+        }
+        if (noted) list_prev(l - 1);
+        // the zeros: a warp's rectangles are one run of memory
+        const int run = 3 * min(32, rows - (i - lane));
+        for (; l < layer_end; ++l) {
+            uint2* t = (uint2*)(table + l * layer_stride + slot - lane);
+            for (int k = lane; k < run; k += 32) t[k] = make_uint2(0, 0);
+            if (out && l >= out_begin && there) out[(l - out_begin) * layer_stride + slot] = empty_region();
         }
     }
     if (n_out && blockIdx.y == 0) for (int l = out_begin + tid; l < layer_end; l += nt) n_out[(l - out_begin) * S + s] = n_in[s];
@@ -599,10 +655,30 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
     for (int l = 0; l < n; ++l) {
         const dc_layer_desc& d = layers[l];
         const int ih = d.in0 < 0 ? c->cfg.height : layers[d.in0].out_h, iw = d.in0 < 0 ? c->cfg.width : layers[d.in0].out_w;
-        t[l] = {d.kind, d.kh, d.kw, d.sh, d.sw, d.ph, d.pw, ih, iw, d.out_h, d.out_w, d.in0, d.in1, from(l, d.in0), from(l, d.in1), -1};
-        for (int k = 0; k < kSlots; ++k) if (owner[k] >= 0 && last_use[owner[k]] <= l) owner[k] = -1;
+        PropLayer& e = t[l];
+        e = PropLayer();
+        e.kind = d.kind; e.kh = d.kh; e.kw = d.kw; e.sh = d.sh; e.sw = d.sw; e.ph = d.ph; e.pw = d.pw;
+        e.in_h = ih; e.in_w = iw; e.out_h = d.out_h; e.out_w = d.out_w; e.in0 = d.in0; e.in1 = d.in1;
+        e.from0 = from(l, d.in0); e.from1 = from(l, d.in1); e.keep = -1;
+        e.two = d.kind == DC_ADD || d.kind == DC_CONCAT;
+        auto window = [&](int kh, int kw, int sh, int sw, int ph, int pw) {
+            if ((sh & (sh - 1)) != 0 || (sw & (sw - 1)) != 0) return;
+            e.window = 1;
+            e.c1x = pw + sw - 1; e.c2x = pw - kw; e.c1y = ph + sh - 1; e.c2y = ph - kh;
+            while ((1 << e.shx) < sw) ++e.shx;
+            while ((1 << e.shy) < sh) ++e.shy;
+        };
+        if (d.kind == DC_CONV || d.kind == DC_MAXPOOL) window(d.kh, d.kw, d.sh, d.sw, d.ph, d.pw);
+        else if (d.kind == DC_LRN) window(2 * d.ph + 1, 2 * d.ph + 1, 1, 1, d.ph, d.ph);
+        else if (d.kind == DC_RELU) window(1, 1, 1, 1, 0, 0);
+        for (int k = 0; k < kSlots; ++k) if (owner[k] >= 0 && last_use[owner[k]] <= l) { owner[k] = -1; t[l].drop |= 1 << k; }
         if (last_use[l] > l)
             for (int k = 0; k < kSlots; ++k) if (owner[k] < 0) { owner[k] = l; t[l].keep = k; if (k >= c->prop_slots) c->prop_slots = k + 1; break; }
+    }
+    for (int l = n - 1, open = 0; l >= 0; --l) {
+        t[l].closed = !open;
+        auto outside = [](int from) { return from == kFrame || from == kTable; };
+        open = open || outside(t[l].from0) || (t[l].two && outside(t[l].from1));
     }
     if (cudaMalloc(&c->prop_table, sizeof(PropLayer) * n) != cudaSuccess) { cudaGetLastError(); return DC_ERR_ALLOC; }
     c->bytes += sizeof(PropLayer) * n;
