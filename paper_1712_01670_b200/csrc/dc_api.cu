@@ -204,7 +204,9 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
             L.tiles_x = dc_div_up(L.d.out_w, DC_TILE_W);
             L.tiles_y = dc_div_up(L.d.out_h, DC_TILE_H);
             L.gpr = dc_div_up(L.d.out_w, DC_TILE_W);
-            L.tiles_flat = (int)(((size_t)S * L.d.out_h * L.gpr + DC_TILE_H - 1) / DC_TILE_H);
+            const int image = L.d.out_h * L.gpr, images = image <= DC_TILE_H ? DC_TILE_H / image : 0;
+            L.gpt = L.d.kind == DC_CONV && L.d.kh * L.d.kw > 1 && images > 1 && S > 1 ? images * image : DC_TILE_H;
+            L.tiles_flat = (int)(((size_t)S * image + L.gpt - 1) / L.gpt);
             size_t tiles = (size_t)L.tiles_x * L.tiles_y * S;             // never fewer than the flat tiles
             if (tiles > max_tiles) max_tiles = tiles;
             all_count[i] = (int32_t)tiles; all_count[n + i] = L.tiles_flat;

@@ -43,7 +43,8 @@ struct dc_layer_rt {
     // whatever the map's height, and across streams; only a row's last group can hold fewer than 8 pixels.
     int flat;                       // 1: this layer's tile list, bitmaps and convolution use flat tiles
     int gpr;                        // groups per image row = ceil(out_w / 8)
-    int tiles_flat;                 // ceil(S * out_h * gpr / 16)
+    int gpt;                        // groups per flat tile: 16, or those of as many whole images as fit (small maps under kernels of more than one tap)
+    int tiles_flat;                 // ceil(S * out_h * gpr / gpt)
     void* map[2];                   // conv: current / cached output (ping-pong); others: map[0]
     int cur;                        // conv: which of map[] holds the newest output
     size_t map_bytes;               // bytes of one map, all streams

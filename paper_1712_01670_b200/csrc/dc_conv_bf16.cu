@@ -49,8 +49,8 @@ struct TcArgs {
     int skip_loads;               // failure-detection tests: the producer issues no copy, so the other roles' waits run out
     // flat tiles (tap-by-tap kernel only): row i of tile t is group t * 16 + i, a group being 8 output pixels of one
     // image row, numbered (stream * Ho + y) * gpr + column group; n_groups_all = S * Ho * gpr.  0: 16 x 8 blocks.
-    int flat = 0, gpr = 0, n_groups_all = 0;
-    int flat_rows = 0;            // > 0: a flat tile is that many whole rows of the stacked streams (flat_rows_of)
+    int flat = 0, gpr = 0, gpt = DC_TILE_H, n_groups_all = 0;         // gpt: groups per tile (dc_layer_rt)
+    int flat_rows = 0, flat_images = 0;   // > 0: a flat tile is that many whole rows of the stacked streams, whole images (flat_box)
     int epi_warps = 4;            // epilogue warps of the CTA: 4 (192 threads) or 8 (320 threads)
     int early = 0;                // tile list, count and bitmaps are older than the kernel before this one (dc_lists_settled): read before the wait for it
     int slab_order = 0;           // tap-by-tap kernel: the steps in the column-slab kernels' order (see StepOrder)
@@ -212,12 +212,12 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
             size_t wb_off[4];                                   // element offset of piece k's pixel
             if (a.flat) {
                 const int gps = a.Ho * a.gpr;
-                const int g = tile * DC_TILE_H + prow, s = g / gps, loc = g - s * gps, y = loc / a.gpr, gx = loc - y * a.gpr;
-                in_map = g < a.n_groups_all && gx * DC_TILE_W + pcol < a.Wo;
+                const int g = tile * a.gpt + prow, s = g / gps, loc = g - s * gps, y = loc / a.gpr, gx = loc - y * a.gpr;
+                in_map = prow < a.gpt && g < a.n_groups_all && gx * DC_TILE_W + pcol < a.Wo;
                 active = in_map && !reused;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const int gk = tile * DC_TILE_H + q * 4 + k, sk = gk / gps, lk = gk - sk * gps, yk = lk / a.gpr, xk = lk - yk * a.gpr;
+                    const int gk = tile * a.gpt + q * 4 + k, sk = gk / gps, lk = gk - sk * gps, yk = lk / a.gpr, xk = lk - yk * a.gpr;
                     wb_off[k] = (((size_t)sk * a.Ho + yk) * a.Wo + xk * DC_TILE_W + (lane >> 2)) * a.Co + ch_off;
                 }
             } else {
@@ -369,7 +369,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             });
             return n;
         };
-        if (a.flat && !a.flat_rows) {
+        if (a.flat && !a.flat_rows && !a.flat_images) {
             // flat tiles: lane l fetches group (l & 15) of tile (l >> 4), one box of 8 pixels per tap and chunk
             const int j = lane >> 4;
             int next = 0;                                       // this lane's tile of the item to come
@@ -384,8 +384,8 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                 peek(item + gridDim.x);
                 int fs = 0, fx = 0, fy = 0; bool fon = false;
                 if (j < MT) {
-                    const int gps = a.Ho * a.gpr, g = tile * DC_TILE_H + (lane & 15);
-                    fon = g < a.n_groups_all;                   // the last tile may have fewer groups: their rows stay as they are (never stored)
+                    const int gps = a.Ho * a.gpr, g = tile * a.gpt + (lane & 15);
+                    fon = (lane & 15) < a.gpt && g < a.n_groups_all;                   // the last tile may have fewer groups: their rows stay as they are (never stored)
                     fs = g / gps;
                     const int loc = g - fs * gps, y = loc / a.gpr;
                     fx = (loc - y * a.gpr) * DC_TILE_W * a.sw - a.pw; fy = y * a.sh - a.ph;
@@ -424,7 +424,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     if (item < n_items) next[j] = __ldcg(a.tile_list + (first + j < n_tiles ? first + j : first));
             };
             peek(blockIdx.x);
-            const uint32_t tx = b_at + (uint32_t)a.b_bytes;
+            const uint32_t tx = (uint32_t)(MT * a.a_bytes / DC_TILE_H * a.gpt + a.b_bytes);
             if (a.early) {
                 if ((int)blockIdx.x < n_items) ahead = weights_ahead(tx, ((int)blockIdx.x % a.NB + a.nb_off) * a.BN);
                 enter();
@@ -438,6 +438,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx_ = t - ty * a.tiles_x;
                     sN[j] = s; xb[j] = tx_ * DC_TILE_W * a.sw - a.pw; yb[j] = ty * DC_TILE_H * a.sh - a.ph;
                     if (a.flat_rows) { sN[j] = xb[j] = 0; yb[j] = tile * a.flat_rows * a.sh; }
+                    if (a.flat_images) { sN[j] = tile * a.flat_images; xb[j] = -a.pw; yb[j] = -a.ph; }
                 }
                 peek(item + gridDim.x);
                 order.walk([&](int c, int kx, int ky, int w) {
@@ -1621,14 +1622,21 @@ int dc_launch_conv_bf16(dc_cache* c, int layer, const void* in, void* out, const
     return DC_OK;
 }
 
-// Flat tiles of a 1 x 1 layer whose rows are 1, 2, 4, 8 or 16 groups: the streams' rows lie one under another, so a tile is 16, 8, 4, 2 or 1 whole
-// rows of that stack and comes as one box (columns beyond the row's end are zeros) where it took 16 boxes, one per group.  Returns the
-// rows, 0: not such a layer.  512 -> 2048 at 7 x 7, 128 streams: 28 -> 20 us (128 tiles, 56 flat ones), 2048 -> 512 25 -> 16.
-static int flat_rows_of(const dc_layer_rt& L, const dc_layer_desc& d)
+// Flat tiles that come as one box, where they took 16, one per group.
+// rows: a 1 x 1 layer whose rows are 1, 2, 4, 8 or 16 groups.  The streams' rows lie one under another, so a tile is 16, 8, 4, 2 or 1 whole
+// rows of that stack (columns beyond the row's end are zeros).  images: a small map under a larger kernel.  A tile is as many whole
+// images as fit (gpt groups); the box displaced by a tap is cut at every image's edges.
+// 128 streams, 7 x 7: 512 -> 2048 28 -> 20 us, 2048 -> 512 25 -> 16, 3 x 3 512 -> 512 50 -> 28 (128 tiles, then 56 and 64).
+struct FlatBox { int rows, images; };
+static FlatBox flat_box(const dc_layer_rt& L, const dc_layer_desc& d)
 {
-    if (!L.flat || L.s2d_s || d.kh != 1 || d.kw != 1 || d.ph != 0 || d.pw != 0 || L.in_h != d.out_h * d.sh || DC_TILE_H % L.gpr != 0) return 0;
+    FlatBox f = {0, 0};
+    if (!L.flat || L.s2d_s || DC_TILE_W * L.gpr * d.sw > 256) return f;          // TMA box limit
     const int rows = DC_TILE_H / L.gpr;
-    return DC_TILE_W * L.gpr * d.sw <= 256 && rows * d.sh <= 256 ? rows : 0;          // TMA box limit
+    if (d.kh == 1 && d.kw == 1) {
+        if (d.ph == 0 && d.pw == 0 && L.in_h == d.out_h * d.sh && DC_TILE_H % L.gpr == 0 && rows * d.sh <= 256) f.rows = rows;
+    } else if (L.gpt % (d.out_h * L.gpr) == 0 && d.out_h * d.sh <= 256) f.images = L.gpt / (d.out_h * L.gpr);
+    return f;
 }
 
 // Tensor maps of the tap-by-tap kernels: the input (16 x 8 windows, or single row pieces for flat tiles) and the weights.
@@ -1638,8 +1646,8 @@ static int generic_maps(dc_cache* c, dc_layer_rt& L, const dc_layer_desc& d, con
     EncodeTiledFn enc = encode_fn();
     if (!enc) return DC_ERR_CUDA;
     bool hit_a, hit_b;
-    const int rows = flat_rows_of(L, d);
-    CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, L.tc_cs > 0 ? 10 : rows ? 9 : L.flat ? 8 : 1, 0, &hit_a);
+    const FlatBox fb = flat_box(L, d);
+    CUtensorMap* tmAp = tm_find(L.tm_a, 4, &L.tm_next, in, L.tc_cs > 0 ? 10 : fb.rows || fb.images ? 9 : L.flat ? 8 : 1, 0, &hit_a);
     CUtensorMap* tmBp = tm_find(&L.tm_b, 1, nullptr, weights, 1, p.BN, &hit_b);
     if (!hit_a) {   // input map [S][Hi][Wi][Ci] bf16; box = BK channels x 16 columns x 8 rows x 1 stream
         cuuint64_t dims[4] = {(cuuint64_t)(L.tc_cs > 0 ? d.cin : cin_all), (cuuint64_t)L.in_w, (cuuint64_t)L.in_h, (cuuint64_t)c->S};
@@ -1650,7 +1658,9 @@ static int generic_maps(dc_cache* c, dc_layer_rt& L, const dc_layer_desc& d, con
         // (flat tiles: one image row of 8 pixels per box)
         cuuint32_t box[4] = {(cuuint32_t)p.BK, (cuuint32_t)(DC_TILE_W * d.sw), (cuuint32_t)(L.flat ? 1 : DC_TILE_H * d.sh), 1};
         cuuint32_t estr[4] = {1, (cuuint32_t)d.sw, (cuuint32_t)(L.flat ? 1 : d.sh), 1};
-        if (rows) { dims[2] *= (cuuint64_t)c->S; dims[3] = 1; box[1] *= (cuuint32_t)L.gpr; box[2] = (cuuint32_t)(rows * d.sh); estr[2] = (cuuint32_t)d.sh; }
+        if (fb.rows) { dims[2] *= (cuuint64_t)c->S; dims[3] = 1; }
+        if (fb.images) box[3] = (cuuint32_t)fb.images;
+        if (fb.rows || fb.images) { box[1] *= (cuuint32_t)L.gpr; box[2] = (cuuint32_t)((fb.rows ? fb.rows : d.out_h) * d.sh); estr[2] = (cuuint32_t)d.sh; }
         if (enc(tmAp, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(in), dims, strides, box, estr,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, p.swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) { tm_drop(L.tm_a, 4, tmAp); tm_drop(&L.tm_b, 1, tmBp); return DC_ERR_CUDA; }
@@ -1783,7 +1793,8 @@ static int launch_group(dc_cache* c, int layer, int grp, const void* in, void* o
     // instruction descriptor: D = f32, A = B = bf16, both K-major, N = BN, M = 128
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     a.status = c->status;
-    a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr; a.flat_rows = flat_rows_of(L, d);
+    a.flat = L.flat; a.gpr = L.gpr; a.n_groups_all = c->S * d.out_h * L.gpr; a.gpt = L.flat ? L.gpt : DC_TILE_H;
+    a.flat_rows = flat_box(L, d).rows; a.flat_images = flat_box(L, d).images;
     a.epi_warps = epi_warps_for(ctas);
     a.bias_smem = t_bias_bytes ? d.cout * G : 0;
     a.slab_order = L.weight_halo != nullptr;

@@ -271,7 +271,7 @@ struct ClassifyArgs {
     const uint8_t* prev; uint8_t* out;           // maps as bytes
     int Ho, Wo, px_bytes;                        // px_bytes = cout * element size (multiple of 16)
     int tiles_x, tiles_y, S;
-    int gpr, n_tiles;                            // gpr > 0: flat tiles of 16 groups of 8 pixels, gpr groups per image row; n_tiles: tiles in all
+    int gpr, gpt, n_tiles;                       // gpr > 0: flat tiles of gpt (up to 16) groups of 8 pixels, gpr groups per image row; n_tiles: tiles in all
     uint32_t* masks; int32_t* dirty_list; int32_t* dirty_count; int32_t* reuse_px;
     const int32_t* alive;                        // per stream: rectangles alive at this layer, or NULL (unknown)
     unsigned long long* reused_total;
@@ -396,18 +396,18 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
 }
 
 
-// The same for a layer with flat tiles: row i of the tile's bitmap is group tile * 16 + i, a group being 8 pixels of
+// The same for a layer with flat tiles: row i of the tile's bitmap is group tile * gpt + i, a group being 8 pixels of
 // one image row, numbered (stream * Ho + y) * gpr + column group.  A tile may hold groups of several streams (small
 // maps); each stream's rectangles are tested against that stream's groups only.
 __device__ __forceinline__ void classify_tile_flat(const ClassifyArgs& a, const int tile, const int part, const int lane, CopyLane& cl)
 {
     const int gps = a.Ho * a.gpr;                                  // groups per stream
-    const int G0 = tile * DC_TILE_H, G1 = min(G0 + DC_TILE_H, a.S * gps);
+    const int G0 = tile * a.gpt, G1 = min(G0 + a.gpt, a.S * gps);
     uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0;
     int in_tile;
     {   // pixels of the tile that exist: a row's last group may be cut by the map's width
         const int g = G0 + lane, loc = g % gps, gx = loc % a.gpr;
-        in_tile = __reduce_add_sync(0xffffffffu, (lane < DC_TILE_H && g < G1) ? min(DC_TILE_W, a.Wo - gx * DC_TILE_W) : 0);
+        in_tile = __reduce_add_sync(0xffffffffu, g < G1 ? min(DC_TILE_W, a.Wo - gx * DC_TILE_W) : 0);
     }
     const int segs_max = (DC_TILE_W * a.px_bytes + kSeg - 1) / kSeg;   // segments of a whole group's pixels
     for (int s = G0 / gps; s * gps < G1; ++s) {
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy(ClassifyArgs 
 // Warps are numbered through all layers' tiles; first_warp is the running sum.
 struct ClassifyLayer {
     const dc_region* regions; uint8_t* map[2];
-    int Ho, Wo, px_bytes, tiles_x, tiles_y, first_warp, gpr, parts;
+    int Ho, Wo, px_bytes, tiles_x, tiles_y, first_warp, gpr, gpt, parts;
     uint32_t* masks; int32_t* dirty_list; int32_t* dirty_count; int32_t* reuse_px;
     const int32_t* alive; unsigned long long* reused_total; int32_t* status;
 };
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
     a.regions = L.regions; a.n_regions = L.alive; a.max_regions = max_regions;     // the rectangles left at this layer
     a.prev = L.map[cur]; a.out = L.map[cur ^ 1];
     a.Ho = L.Ho; a.Wo = L.Wo; a.px_bytes = L.px_bytes; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y; a.S = S;
-    a.gpr = L.gpr; a.n_tiles = 0;
+    a.gpr = L.gpr; a.gpt = L.gpt; a.n_tiles = 0;
     a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = L.dirty_count; a.reuse_px = L.reuse_px;
     a.alive = L.alive; a.reused_total = L.reused_total; a.status = L.status;
     a.parts = L.parts; a.running = nullptr;
@@ -595,7 +595,7 @@ int dc_build_classify_table(dc_cache* c)
         e.map[0] = (uint8_t*)L.map[0]; e.map[1] = (uint8_t*)L.map[1];
         e.Ho = L.d.out_h; e.Wo = L.d.out_w; e.px_bytes = L.d.cout * c->elt;
         e.tiles_x = L.tiles_x; e.tiles_y = L.tiles_y; e.first_warp = warps;
-        e.gpr = L.flat ? L.gpr : 0;
+        e.gpr = L.flat ? L.gpr : 0; e.gpt = L.gpt;
         e.masks = L.masks; e.dirty_list = L.dirty_list; e.dirty_count = c->dirty_count + i;
         e.reuse_px = c->reuse_px + (size_t)i * c->S; e.alive = c->alive + (size_t)i * c->S;
         e.reused_total = c->reused_total + i;
@@ -714,7 +714,7 @@ int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, co
     a.prev = (const uint8_t*)prev_out; a.out = (uint8_t*)out;
     a.Ho = L.d.out_h; a.Wo = L.d.out_w; a.px_bytes = L.d.cout * c->elt;
     a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y; a.S = c->S;
-    a.gpr = L.flat ? L.gpr : 0; a.n_tiles = dc_layer_tiles(c, L);
+    a.gpr = L.flat ? L.gpr : 0; a.gpt = L.gpt; a.n_tiles = dc_layer_tiles(c, L);
     a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = count;
     a.reuse_px = px;
     a.running = running; a.parts = copy_parts(c, dc_layer_tiles(c, L), a.px_bytes);

@@ -907,6 +907,21 @@ def test_conv_flat_tiles_as_whole_rows(scheme, hi, wi, cin, cout, st, S, monkeyp
     _one_layer_full_and_partial(hi, wi, cin, cout, 1, st, 0, S, scheme)
 
 
+@pytest.mark.parametrize("scheme", [8, 9])
+@pytest.mark.parametrize("hi,wi,cin,cout,k,st,p,S", [
+    (7, 7, 64, 128, 3, 1, 1, 5),         # two images a tile, 14 of 16 groups, the last tile half full
+    (4, 6, 32, 64, 3, 1, 1, 9),          # four images
+    (3, 13, 64, 32, 5, 1, 2, 5),         # rows of two groups, two images
+    (14, 14, 128, 64, 3, 2, 1, 4),       # strided
+    (16, 8, 64, 64, 3, 1, 1, 2),         # an image is a tile: groups one by one
+    (1, 5, 16, 32, 2, 1, 1, 7),          # a last row that reads padding alone
+])
+def test_conv_flat_tiles_as_whole_images(scheme, hi, wi, cin, cout, k, st, p, S, monkeypatch):
+    """Small maps under kernels of more than one tap: flat tiles of whole images."""
+    monkeypatch.setenv("DC_CONV_SCHEME", str(scheme))
+    _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, scheme)
+
+
 @pytest.mark.parametrize("hi,wi,cin,cout,k,S,groups", [
     (28, 28, 128, 256, 3, 2, 1),         # two chunks of 64 channels, CTA pairs too
     (13, 13, 96, 64, 5, 3, 1),           # 32-channel steps, a half-empty last chunk
