@@ -25,7 +25,8 @@
 //
 // Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf).  A tile that holds one is marked by the warps
 // that split it and its pixels are computed once more with FMAs from the float weights; weights like that keep the layer
-// on the CUDA cores.
+// on the CUDA cores.  The same is done for a pixel with a sum that is not finite: where operands that do split add up to more than a
+// float holds, the three accumulators can become infinities of either sign, and their sum NaN.
 #include "dc_common.cuh"
 #include "dc_tcgen05.cuh"
 
@@ -286,12 +287,16 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
             const int nb = item % a.NB, grp = nb / a.nb_g, c0 = (nb - grp * a.nb_g) * BN + half * CH, n = min(CH, a.Cog - c0);
             float* const tile_out = a.out + (((size_t)s * a.Ho + ty * DC_TILE_H) * a.Wo + tx * DC_TILE_W) * a.Co + grp * a.Cog + c0;
             const float* bias = a.bias + grp * a.Cog + c0;
-            if (ctl->odd[seq % kTileFlags] == seq + 1) {
-                // a value of the patch does not split: this pixel once more, by FMAs
+            float beyond = 0.f;                                            // NaN if a sum is not finite
+#pragma unroll
+            for (int j = 0; j < CH; ++j) beyond = fmaf(sum[j], 0.f, beyond);
+            const bool redo = active && (beyond != beyond || ctl->odd[seq % kTileFlags] == seq + 1);
+            if (redo) {
+                // a value of the patch does not split, or a sum of this pixel overflowed: the pixel once more, by FMAs
                 float* o = tile_out + ((size_t)row * a.Wo + col) * a.Co;
                 const float* w = a.w + (size_t)(grp * a.Cog + c0) * KW * KW * a.Cig;
 #pragma unroll 1
-                for (int j = 0; j < (active ? n : 0); ++j) {
+                for (int j = 0; j < n; ++j) {
                     float v = 0.f;
 #pragma unroll 1
                     for (int t = 0; t < KW * KW; ++t) {
@@ -305,11 +310,10 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
                     v += __ldg(bias + j);
                     o[j] = a.relu ? fmaxf(v, 0.f) : v;
                 }
-                continue;
             }
             // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
             // warp touched 32 lines, and the stores took as long as the MMAs)
-            const uint32_t todo = __ballot_sync(0xffffffffu, active);
+            const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
             const int part = lane % (STAGE_CH / 4);
 #pragma unroll
             for (int c = 0; c < CH; c += STAGE_CH) {

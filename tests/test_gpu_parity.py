@@ -1488,6 +1488,42 @@ def test_conv_fp32_on_tensor_cores_with_values_that_do_not_split():
         dc.close()
 
 
+@pytest.mark.parametrize("relu", [0, 1])
+@pytest.mark.parametrize("cin,cout,k,H,W,S,groups", [(32, 64, 3, 48, 40, 1, 1), (64, 32, 1, 33, 21, 2, 1), (40, 72, 5, 30, 22, 2, 2), (64, 64, 3, 113, 113, 4, 1)])
+def test_conv_fp32_sums_beyond_the_largest_float(cin, cout, k, H, W, S, groups, relu, monkeypatch):
+    """Finite operands whose sums leave the float range: infinities as from a chain of FMAs, never NaN, and +infinity after ReLU.  All the
+    products of a channel have one sign, so that the order of the sum does not matter; most pixels stay far below."""
+    g = rng(cin + cout + k)
+    nb = nets.NetBuilder(H, W)
+    nb.conv(nb.conv(-1, cin, 1, 1, 0), cout, k, 1, k // 2, relu, groups=groups)
+    wts = np.abs(g.normal(0, 0.1, size=(cout, k, k, cin // groups))).astype(np.float32) + np.float32(0.1)
+    wts[1::2] *= -1
+    wts[:8] = np.ldexp(wts[:8], 70)
+    bias = g.normal(0, 0.1, size=cout).astype(np.float32)
+    x = g.uniform(0.5, 1.0, size=(S, H, W, cin)).astype(np.float32)
+    x[:, 5:9, 3:7] = np.ldexp(x[:, 5:9, 3:7], 60)                   # sums of 2^130 and more
+    x[:, 20:24, 14:17] = np.ldexp(x[:, 20:24, 14:17], 70)           # 2^140
+    x[:, 20:22, 2:4] = np.ldexp(x[:, 20:22, 2:4], 40)               # 2^110: large and finite
+    x = torch.from_numpy(x).cuda()
+    out = []
+    for cores in (False, True):
+        if cores:
+            monkeypatch.setenv("DC_NO_TENSOR_CORES", "1")
+        dc = DeepCache(W, H, nb.layers, [np.zeros((cin, 1, 1, 3), np.float32), wts], [np.zeros(cin, np.float32), bias], n_streams=S, block=16,
+                       search_range=4, dtype=B.DC_FP32, max_regions=4)
+        out.append(dc.conv_partial(1, x))
+        if not cores:                                               # reuse leaves the other pixels' bits as they are
+            regs, n = torch.zeros((S, 4, 6), dtype=torch.int32, device="cuda"), torch.ones(S, dtype=torch.int32, device="cuda")
+            regs[:, 0] = torch.tensor([2, 4, 6, 2, 2, 4], dtype=torch.int32)
+            assert torch.equal(dc.conv_partial(1, x, out[0], regs, n), out[0])
+        dc.close()
+    got, want = out
+    over = torch.isinf(want)
+    assert over.sum() >= S * 20 * 4 and not torch.isnan(want).any()
+    assert torch.equal(torch.isinf(got), over) and torch.equal(got[over], want[over])
+    assert torch.allclose(got[~over], want[~over], rtol=1e-5, atol=1e-4)        # sums of one sign: both within (terms) 2^-24 of the exact one
+
+
 def test_conv_fp32_weights_that_do_not_split(monkeypatch):
     g = rng(78)
     nb = nets.NetBuilder(24, 40)
