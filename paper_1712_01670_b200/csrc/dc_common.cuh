@@ -61,7 +61,7 @@ struct dc_layer_rt {
     void* weight_halo;              // conv, bf16: weights packed for the patch-reuse and column-slab kernels
     int halo_bn;                    // channels per block that packing is grouped by
     float* weight_simt;             // conv on the register-blocked CUDA-core kernel: its packed weights (dc_conv_simt.cu)
-    void* weight_f32;               // conv, fp32, on the tensor cores: weights split into bf16 pieces (dc_conv_f32.cu)
+    void* weight_f32;               // conv, fp32, on the tensor cores: weights split into bf16 pieces, and as floats behind them (dc_conv_f32.cu)
     void* in_padded;                // conv, bf16, cin <= 8: input with channels padded to 8
     void* in_s2d;                   // conv, bf16, strided over few channels: the space-to-depth copy of the input the rewritten layer reads (dc_conv_s2d.cu)
     int s2d_ws, s2d_cs;             // ... columns of the block map and channels of its pixels

@@ -26,7 +26,8 @@
 // Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf).  A tile that holds one is marked by the warps
 // that split it and its pixels are computed once more with FMAs from the float weights; weights like that keep the layer
 // on the CUDA cores.  The same is done for a pixel with a sum that is not finite: where operands that do split add up to more than a
-// float holds, the three accumulators can become infinities of either sign, and their sum NaN.
+// float holds, the three accumulators can become infinities of either sign, and their sum NaN.  With all pixels computed so, 64 -> 64 channels,
+// 3 x 3 at 113 x 113, 4 streams, takes 394 us (43 on the tensor cores, 118 on k_conv_simt; a channel after the other from global memory 12 ms).
 #include "dc_common.cuh"
 #include "dc_tcgen05.cuh"
 
@@ -40,7 +41,8 @@ constexpr int kTileFlags = 8;                     // more than the items between
 constexpr unsigned long long kWaitLimitF = 2000000000ull;
 
 struct F32Args {
-    const float* in; const float* w; const uint8_t* wp; const float* bias; float* out;   // wp: [groups * nb_g][chunks][taps][4][3 BN][8] bf16
+    const float* in; const uint8_t* wp; const float* w; const float* bias; float* out;   // wp: [groups * nb_g][chunks][taps][4][3 BN][8] bf16
+                                                  // w: [groups][taps][Cig filled up to 16s][nb_g * BN] float, for pixels computed by FMAs
     const int32_t* tile_list; const int32_t* tile_count; const uint32_t* masks;
     int Hi, Wi, Ci, Ho, Wo, Co, p, relu, tiles_x, tiles_y;
     int Cig, Cog, nb_g, NB, chunks, ks_last;      // channels per group; blocks per group and in all; patches; steps of 16 channels in the last
@@ -291,29 +293,67 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
 #pragma unroll
             for (int j = 0; j < CH; ++j) beyond = fmaf(sum[j], 0.f, beyond);
             const bool redo = active && (beyond != beyond || ctl->odd[seq % kTileFlags] == seq + 1);
-            if (redo) {
-                // a value of the patch does not split, or a sum of this pixel overflowed: the pixel once more, by FMAs
-                float* o = tile_out + ((size_t)row * a.Wo + col) * a.Co;
-                const float* w = a.w + (size_t)(grp * a.Cog + c0) * KW * KW * a.Cig;
-#pragma unroll 1
-                for (int j = 0; j < n; ++j) {
-                    float v = 0.f;
+            if (__any_sync(0xffffffffu, redo)) {
+                // A value of the patch does not split, or a sum overflowed: such pixels once more, by FMAs.  The warp brings the weights of 16
+                // channels to shared memory while the ones before are in use; 16 channels of a tap are a sum of their own, which keeps the error
+                // below that of one chain.
+                const int cog = a.nb_g * BN, cig = (a.Cig + 15) & ~15;
+#pragma unroll
+                for (int h = 0; h < CH; h += 16) {
+                    const float* k = a.w + ((size_t)grp * KW * KW * cig + lane / 4) * cog + c0 + h + lane % 4 * 4;
+                    float4 w0 = __ldg((const float4*)k), w1 = __ldg((const float4*)(k + 8 * (size_t)cog));
+                    if (redo) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[h + j] = 0.f;
+                    }
 #pragma unroll 1
                     for (int t = 0; t < KW * KW; ++t) {
                         const int iy = y - a.p + t / KW, ix = x - a.p + t % KW;
-                        if (iy < 0 || iy >= a.Hi || ix < 0 || ix >= a.Wi) continue;
+                        const bool inside = redo && iy >= 0 && iy < a.Hi && ix >= 0 && ix < a.Wi;
                         const float* p = a.in + (((size_t)s * a.Hi + iy) * a.Wi + ix) * a.Ci + grp * a.Cig;
-                        const float* k = w + ((size_t)j * KW * KW + t) * a.Cig;
 #pragma unroll 1
-                        for (int c = 0; c < a.Cig; ++c) v = fmaf(dc_ld(p + c), __ldg(k + c), v);
+                        for (int c = 0; c < cig; c += 16) {
+                            float e[16], part[16];
+#pragma unroll
+                            for (int i = 0; i < 16; i += 4) {
+                                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                                if (inside && c + i < a.Cig) {
+                                    if (a.vec) v = dc_ld((const float4*)(p + c + i));
+                                    else {
+                                        v.x = dc_ld(p + c + i);
+                                        if (c + i + 1 < a.Cig) v.y = dc_ld(p + c + i + 1);
+                                        if (c + i + 2 < a.Cig) v.z = dc_ld(p + c + i + 2);
+                                        if (c + i + 3 < a.Cig) v.w = dc_ld(p + c + i + 3);
+                                    }
+                                }
+                                e[i] = v.x; e[i + 1] = v.y; e[i + 2] = v.z; e[i + 3] = v.w;
+                            }
+                            __syncwarp();
+                            sts128(stage + lane * 16, __float_as_uint(w0.x), __float_as_uint(w0.y), __float_as_uint(w0.z), __float_as_uint(w0.w));
+                            sts128(stage + 512 + lane * 16, __float_as_uint(w1.x), __float_as_uint(w1.y), __float_as_uint(w1.z), __float_as_uint(w1.w));
+                            __syncwarp();
+                            if (t + 1 < KW * KW || c + 16 < cig) { k += 16 * (size_t)cog; w0 = __ldg((const float4*)k); w1 = __ldg((const float4*)(k + 8 * (size_t)cog)); }
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) part[j] = 0.f;
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+#pragma unroll
+                                for (int j = 0; j < 16; j += 4) {
+                                    const uint4 w = lds128(stage + i * 64 + j * 4);
+                                    part[j] = fmaf(e[i], __uint_as_float(w.x), part[j]); part[j + 1] = fmaf(e[i], __uint_as_float(w.y), part[j + 1]);
+                                    part[j + 2] = fmaf(e[i], __uint_as_float(w.z), part[j + 2]); part[j + 3] = fmaf(e[i], __uint_as_float(w.w), part[j + 3]);
+                                }
+                            if (redo) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) sum[h + j] += part[j];
+                            }
+                        }
                     }
-                    v += __ldg(bias + j);
-                    o[j] = a.relu ? fmaxf(v, 0.f) : v;
                 }
             }
             // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
             // warp touched 32 lines, and the stores took as long as the MMAs)
-            const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
+            const uint32_t todo = __ballot_sync(0xffffffffu, active);
             const int part = lane % (STAGE_CH / 4);
 #pragma unroll
             for (int c = 0; c < CH; c += STAGE_CH) {
@@ -450,6 +490,19 @@ __global__ void k_pack_f32(const float* w, int taps, int Cig, int Cog, int nb_g,
     }
 }
 
+// The same weights as floats, [cout][taps][Cig] -> [groups][taps][Cig filled up to 16s][nb_g * BN] with zeros beyond the last channels.
+__global__ void k_pack_f32_fma(const float* w, int taps, int Cig, int Cog, int cig, int cog, size_t total, float* out)
+{
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        size_t r = i;
+        const int n = (int)(r % cog); r /= cog;
+        const int c = (int)(r % cig); r /= cig;
+        const int t = (int)(r % taps);
+        const size_t grp = r / taps;
+        out[i] = n < Cog && c < Cig ? w[((grp * Cog + n) * taps + t) * Cig + c] : 0.f;
+    }
+}
+
 // An MMA takes some 40 clocks for its pixels whatever its width: a step of 16 channels measured 240 clocks for 32 output channels and 310 for
 // 64.  Wide blocks, then, unless they leave SMs without an item: whichever takes fewer clocks with every tile dirty.
 int f32_bn(const dc_cache* c, const dc_layer_rt& L)
@@ -470,10 +523,13 @@ static bool f32_ok(const dc_cache* c, const dc_layer_desc& d)
            (d.kw == 1 || d.kw == 3 || d.kw == 5) && d.cin / G >= 16 && d.cout / G >= 32 && (d.cout / G) % 4 == 0;
 }
 
-static size_t f32_weight_bytes(const dc_cache* c, const dc_layer_rt& L)
+// Bytes of the pieces, and of the float weights that lie behind them (dc_layer_rt::weight_f32).
+struct F32Bytes { size_t pieces, floats; };
+static F32Bytes f32_weight_bytes(const dc_cache* c, const dc_layer_rt& L)
 {
-    const int G = L.d.groups > 1 ? L.d.groups : 1, BN = f32_bn(c, L);
-    return (size_t)G * dc_div_up(L.d.cout / G, BN) * dc_div_up(L.d.cin / G, kChF) * L.d.kh * L.d.kw * 4 * 3 * BN * 16;
+    const int G = L.d.groups > 1 ? L.d.groups : 1, BN = f32_bn(c, L), cig = L.d.cin / G;
+    const size_t rows = (size_t)G * dc_div_up(L.d.cout / G, BN) * BN * L.d.kh * L.d.kw;
+    return {rows * dc_div_up(cig, kChF) * kChF * 3 * 2, rows * ((cig + 15) & ~15) * sizeof(float)};
 }
 
 int dc_pack_weights_f32(dc_cache* c, int layer)
@@ -482,11 +538,14 @@ int dc_pack_weights_f32(dc_cache* c, int layer)
     if (!f32_ok(c, L.d) || dc_dense_ok(L) || getenv("DC_NO_TENSOR_CORES")) return DC_OK;
     const int G = L.d.groups > 1 ? L.d.groups : 1, cig = L.d.cin / G, cog = L.d.cout / G, taps = L.d.kh * L.d.kw;
     const int BN = f32_bn(c, L), nb_g = dc_div_up(cog, BN), chunks = dc_div_up(cig, kChF);
-    const size_t bytes = f32_weight_bytes(c, L);
-    DC_CUDA(cudaMalloc(&L.weight_f32, bytes));
-    c->bytes += bytes;
-    int grid = (int)((bytes / 6 + 255) / 256); if (grid > c->num_sms * 8) grid = c->num_sms * 8;
-    k_pack_f32<<<grid, 256, 0, c->stream>>>((const float*)L.weight, taps, cig, cog, nb_g, G * nb_g, chunks, BN, (__nv_bfloat16*)L.weight_f32, c->reuse_px + layer);
+    const F32Bytes bytes = f32_weight_bytes(c, L);
+    DC_CUDA(cudaMalloc(&L.weight_f32, bytes.pieces + bytes.floats));
+    c->bytes += bytes.pieces + bytes.floats;
+    auto grid = [&](size_t n) { const size_t g = (n + 255) / 256, most = (size_t)c->num_sms * 8; return (int)(g < most ? g : most); };
+    k_pack_f32<<<grid(bytes.pieces / 6), 256, 0, c->stream>>>((const float*)L.weight, taps, cig, cog, nb_g, G * nb_g, chunks, BN, (__nv_bfloat16*)L.weight_f32, c->reuse_px + layer);
+    DC_CUDA(cudaGetLastError());
+    k_pack_f32_fma<<<grid(bytes.floats / 4), 256, 0, c->stream>>>((const float*)L.weight, taps, cig, cog, (cig + 15) & ~15, nb_g * BN, bytes.floats / 4,
+                                                                 (float*)((uint8_t*)L.weight_f32 + bytes.pieces));
     DC_CUDA(cudaGetLastError());
     return DC_OK;
 }
@@ -506,7 +565,8 @@ int dc_settle_weights_f32(dc_cache* c)
         if (!L.weight_f32 || !odd[i]) continue;
         cudaFree(L.weight_f32);
         L.weight_f32 = nullptr;
-        c->bytes -= f32_weight_bytes(c, L);
+        const F32Bytes bytes = f32_weight_bytes(c, L);
+        c->bytes -= bytes.pieces + bytes.floats;
         const int rc = dc_pack_weights_simt(c, i);
         if (rc != DC_OK) return rc;
     }
@@ -533,7 +593,7 @@ int dc_launch_conv_f32(dc_cache* c, int layer, const void* in, void* out, const 
     dc_layer_rt& L = c->L[layer];
     const int G = L.d.groups > 1 ? L.d.groups : 1, BN = f32_bn(c, L);
     F32Args a;
-    a.in = (const float*)in; a.w = (const float*)L.weight; a.wp = (const uint8_t*)L.weight_f32; a.bias = L.bias; a.out = (float*)out;
+    a.in = (const float*)in; a.wp = (const uint8_t*)L.weight_f32; a.w = (const float*)(a.wp + f32_weight_bytes(c, L).pieces); a.bias = L.bias; a.out = (float*)out;
     a.tile_list = tile_list; a.tile_count = tile_count; a.masks = masks; a.early = dc_lists_settled(c);
     a.Hi = L.in_h; a.Wi = L.in_w; a.Ci = L.d.cin; a.Ho = L.d.out_h; a.Wo = L.d.out_w; a.Co = L.d.cout;
     a.p = L.d.ph; a.relu = L.d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;

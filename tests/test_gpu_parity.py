@@ -1524,6 +1524,52 @@ def test_conv_fp32_sums_beyond_the_largest_float(cin, cout, k, H, W, S, groups, 
     assert torch.allclose(got[~over], want[~over], rtol=1e-5, atol=1e-4)        # sums of one sign: both within (terms) 2^-24 of the exact one
 
 
+@pytest.mark.parametrize("cin,cout,k,H,W,S,groups", [(64, 64, 3, 113, 113, 4, 1), (32, 32, 3, 60, 50, 2, 1), (40, 72, 5, 30, 22, 2, 2), (71, 36, 1, 40, 33, 3, 1), (19, 40, 3, 19, 25, 2, 1)])
+def test_conv_fp32_every_tile_computed_by_fmas(cin, cout, k, H, W, S, groups, monkeypatch):
+    """An infinity in every tile: the pixels that do not see it are no further from 64-bit sums than the CUDA-core kernel's, and a pass
+    takes a small multiple of that kernel's time (1.4 to 3.4 measured; the bound leaves room for a busy host)."""
+    g = rng(cin * 3 + cout + k)
+    nb = nets.NetBuilder(H, W)
+    x0 = nb.conv(-1, cin - 3 if cin % 4 else cin, 1, 1, 0)
+    if nb.shape(x0)[2] < cin:
+        x0 = nb.concat(x0, -1)
+    nb.conv(x0, cout, k, 1, k // 2, 0, groups=groups)
+    li = len(nb.layers) - 1
+    wts = g.normal(0, np.sqrt(2.0 / (k * k * cin / groups)), size=(cout, k, k, cin // groups)).astype(np.float32)
+    bias = g.normal(0, 0.1, size=cout).astype(np.float32)
+    ws = [np.zeros((l["cout"], 1, 1, 3), np.float32) if l["kind"] == 0 else None for l in nb.layers[:-1]] + [wts]
+    bs = [np.zeros(l["cout"], np.float32) if l["kind"] == 0 else None for l in nb.layers[:-1]] + [bias]
+    x = torch.from_numpy(g.normal(size=(S, H, W, cin)).astype(np.float32)).cuda()
+    want = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), torch.from_numpy(wts).cuda().double().permute(0, 3, 1, 2),
+                                      torch.from_numpy(bias).cuda().double(), padding=k // 2, groups=groups).permute(0, 2, 3, 1)
+    seen = torch.zeros((S, H, W), dtype=torch.bool, device="cuda")
+    for y in range(0, H, 16):
+        for xx in range(0, W, 8):
+            x[:, y, xx, ::cin // groups] = float("inf")             # in every group's first channel
+            seen[:, max(0, y - k // 2):y + k // 2 + 1, max(0, xx - k // 2):xx + k // 2 + 1] = True
+    clear = ~seen
+    err, us = [], []
+    for cores in (False, True):
+        if cores:
+            monkeypatch.setenv("DC_NO_TENSOR_CORES", "1")
+        dc = DeepCache(W, H, nb.layers, ws, bs, n_streams=S, block=16, search_range=4, dtype=B.DC_FP32, max_regions=4)
+        out = dc.conv_partial(li, x)
+        assert not torch.isfinite(out[seen]).any() and torch.isfinite(out[clear]).all()
+        err.append(float((out.double() - want)[clear].norm() / want[clear].norm()))
+        best = 1e9
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            B.dc_conv_partial(dc.handle, li, x, None, None, None, out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3)
+        us.append(best)
+        dc.close()
+    assert err[0] <= 1.1 * err[1]                                   # (two roundings of the same data: 1.1 for their chance)
+    assert us[0] <= 5 * us[1] + 50
+
+
 def test_conv_fp32_weights_that_do_not_split(monkeypatch):
     g = rng(78)
     nb = nets.NetBuilder(24, 40)
