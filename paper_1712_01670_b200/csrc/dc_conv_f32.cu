@@ -1,7 +1,7 @@
 // Partial convolution of float32 maps on the 5th-generation tensor cores, without giving up float32 accuracy.
 //
-// A float has 24 significant bits, a bf16 eight: every operand is the exact sum of three bf16 pieces, x = x0 + x1 + x2 (each the
-// nearest bf16 of what is left).  The product of two operands is then six tensor-core products of pieces,
+// A float has 24 significant bits, a bf16 eight: an operand of 2^-110 or more is the exact sum of three bf16 pieces, x = x0 + x1 + x2
+// (each the nearest bf16 of what is left).  The product of two operands is then six tensor-core products of pieces,
 //     x0 w0  +  (x0 w1 + x1 w0)  +  (x0 w2 + x1 w1 + x2 w0),
 // whose remainder (x1 w2 and smaller) is below 2^-26 of the product.  Products of bf16 are exact in fp32; what rounds is the sum,
 // and there the tensor core is kept on a short leash: it adds up one kernel row of 32 channels (terms of each of the three sizes in
@@ -23,7 +23,8 @@
 // Measured, 24 streams, all tiles, us (CUDA cores, here): 32 -> 32 at 227 x 227 451, 203; 32 -> 64 at 113 x 113 246, 80; 64 -> 64 461, 134;
 // 64 -> 128 at 56 x 56 213, 71.  One stream: 29.4, 14.6; 19.8, 8.9; 32.5, 13.1; 17.3, 11.0.
 //
-// Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf).  A tile that holds one is marked by the warps
+// Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf), nor do most floats below 2^-110, whose last bits lie under the
+// smallest bf16 of 2^-133: whatever leaves a remainder behind its third piece.  A tile that holds one is marked by the warps
 // that split it and its pixels are computed once more with FMAs from the float weights; weights like that keep the layer
 // on the CUDA cores.  The same is done for a pixel with a sum that is not finite: where operands that do split add up to more than a
 // float holds, the three accumulators can become infinities of either sign, and their sum NaN.  With all pixels computed so, 64 -> 64 channels,
@@ -92,15 +93,16 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// Two floats into three pairs of pieces; `odd` becomes NaN if one of them does not split.
-__device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2, float& odd)
+// Two floats into three pairs of pieces; one of the low 16 bits of `odd` is set if one of them does not split: what is left for the third
+// piece is no bf16 itself, or NaN (whose bits are all ones).
+__device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2, uint32_t& odd)
 {
     p0 = bf16_pair(a, b);
     a -= __uint_as_float(p0 << 16); b -= __uint_as_float(p0 & 0xffff0000u);
     p1 = bf16_pair(a, b);
     a -= __uint_as_float(p1 << 16); b -= __uint_as_float(p1 & 0xffff0000u);
     p2 = bf16_pair(a, b);
-    odd = fmaf(a, 0.f, odd); odd = fmaf(b, 0.f, odd);
+    odd |= __float_as_uint(a) | __float_as_uint(b);
 }
 
 template <int BN, int KW>
@@ -425,7 +427,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
         auto split = [&](const float4 (&v)[UNITS][2], Patch b) -> bool {
             const int c_end = 16 * k_steps(b.cc);                          // channels of this patch that the MMAs read
             if (!f_wait_warp(a_empty0 + 8u * slot, phase ^ 1u, lane, ctl, a.status)) return false;
-            float odd = 0.f;
+            uint32_t odd = 0;
 #pragma unroll
             for (int i = 0; i < UNITS; ++i) {
                 if (so[i] < 0 || cg[i] >= c_end) continue;
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
                 sts128(at + PIECE, p1[0], p1[1], p1[2], p1[3]);
                 sts128(at + 2 * PIECE, p2[0], p2[1], p2[2], p2[3]);
             }
-            if (odd != odd) ctl->odd[b.seq % kTileFlags] = b.seq + 1;
+            if (odd & 0xffffu) ctl->odd[b.seq % kTileFlags] = b.seq + 1;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&ctl->a_full[slot]);
@@ -486,7 +488,7 @@ __global__ void k_pack_f32(const float* w, int taps, int Cig, int Cog, int nb_g,
             o[(size_t)p * BN * 8] = b;
             v -= __bfloat162float(b);
         }
-        if (!(v - v == 0.f)) *odd = 1;
+        if (v != 0.f) *odd = 1;                                           // (NaN too)
     }
 }
 

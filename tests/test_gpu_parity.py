@@ -1547,8 +1547,8 @@ def test_conv_fp32_every_tile_computed_by_fmas(cin, cout, k, H, W, S, groups, mo
         for xx in range(0, W, 8):
             x[:, y, xx, ::cin // groups] = float("inf")             # in every group's first channel
             seen[:, max(0, y - k // 2):y + k // 2 + 1, max(0, xx - k // 2):xx + k // 2 + 1] = True
-    clear = ~seen
-    err, us = [], []
+    clear, plain = ~seen, torch.where(torch.isinf(x), 1.0, x)
+    err, us, us_plain = [], [], []
     for cores in (False, True):
         if cores:
             monkeypatch.setenv("DC_NO_TENSOR_CORES", "1")
@@ -1556,18 +1556,43 @@ def test_conv_fp32_every_tile_computed_by_fmas(cin, cout, k, H, W, S, groups, mo
         out = dc.conv_partial(li, x)
         assert not torch.isfinite(out[seen]).any() and torch.isfinite(out[clear]).all()
         err.append(float((out.double() - want)[clear].norm() / want[clear].norm()))
-        best = 1e9
-        for _ in range(5):
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            B.dc_conv_partial(dc.handle, li, x, None, None, None, out)
-            b.record()
-            torch.cuda.synchronize()
-            best = min(best, a.elapsed_time(b) * 1e3)
-        us.append(best)
+        for inp, times in ((x, us), (plain, us_plain)):
+            best = 1e9
+            for _ in range(5):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                B.dc_conv_partial(dc.handle, li, inp, None, None, None, out)
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b) * 1e3)
+            times.append(best)
         dc.close()
     assert err[0] <= 1.1 * err[1]                                   # (two roundings of the same data: 1.1 for their chance)
     assert us[0] <= 5 * us[1] + 50
+    assert S * H * W < 40000 or us_plain[0] < us_plain[1]           # without such values no tile goes there: 43 and 118 us
+
+
+@pytest.mark.parametrize("e,f", [(-100, 60), (-108, 60), (-112, 60), (-118, 100), (-122, 100), (-126, 100), (-140, 120), (60, -105), (100, -112), (100, -118), (110, -126)])
+def test_conv_fp32_operands_too_small_to_split(e, f, monkeypatch):
+    """Inputs of 2^e and weights of 2^f: the third bf16 piece of a float below 2^-110 is cut, or all of them.  Against 64-bit sums and the
+    CUDA-core kernel: the error in the 2-norm is no larger than the latter's (0.6 to 0.7 of it)."""
+    g = rng(79)
+    nb = nets.NetBuilder(48, 40)
+    nb.conv(nb.conv(-1, 32, 1, 1, 0), 64, 3, 1, 1, 0)
+    wts = np.ldexp(g.normal(size=(64, 3, 3, 32)).astype(np.float32), f)
+    x = np.zeros((1, 48, 40, 32), np.float32)
+    x[:, :30] = np.ldexp(g.normal(size=(1, 30, 40, 32)).astype(np.float32), e)      # (zeros split)
+    x = torch.from_numpy(x).cuda()
+    want = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), torch.from_numpy(wts).cuda().double().permute(0, 3, 1, 2), padding=1).permute(0, 2, 3, 1)
+    err = []
+    for cores in (False, True):
+        if cores:
+            monkeypatch.setenv("DC_NO_TENSOR_CORES", "1")
+        dc = DeepCache(40, 48, nb.layers, [np.zeros((32, 1, 1, 3), np.float32), wts], [np.zeros(32, np.float32), np.zeros(64, np.float32)],
+                       n_streams=1, block=16, search_range=4, dtype=B.DC_FP32, max_regions=4)
+        err.append(float((dc.conv_partial(1, x).double() - want).norm() / want.norm()))
+        dc.close()
+    assert err[0] <= 1.1 * err[1] and err[1] < 3e-7
 
 
 def test_conv_fp32_weights_that_do_not_split(monkeypatch):
