@@ -228,6 +228,7 @@ bool dc_dense_ok(const dc_layer_rt& L);
 int dc_launch_conv_simt(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,
                         const int32_t* tile_count, const uint32_t* masks, int max_tiles);
 bool dc_conv_simt_stores(const dc_cache* c, const void* out);   // out lies where dc_launch_conv_simt can store
+void dc_simt_order(const dc_cache* c, const dc_layer_rt& L, int* ci, int* ks);   // the order of its sums: every ks-th run of ci channels in a chain of its own
 int dc_launch_dense(dc_cache* c, int layer, const void* in, void* out, const uint32_t* masks);
 int dc_pack_weights_simt(dc_cache* c, int layer);
 // float32 stride-1 layers on the tensor cores (dc_conv_f32.cu)

@@ -28,7 +28,7 @@
 // that split it and its pixels are computed once more with FMAs from the float weights; weights like that keep the layer
 // on the CUDA cores.  The same is done for a pixel with a sum that is not finite: where operands that do split add up to more than a
 // float holds, the three accumulators can become infinities of either sign, and their sum NaN.  With all pixels computed so, 64 -> 64 channels,
-// 3 x 3 at 113 x 113, 4 streams, takes 394 us (43 on the tensor cores, 118 on k_conv_simt; a channel after the other from global memory 12 ms).
+// 3 x 3 at 113 x 113, 4 streams, takes 405 us (43 on the tensor cores, 118 on k_conv_simt; a channel after the other from global memory 12 ms).
 #include "dc_common.cuh"
 #include "dc_tcgen05.cuh"
 
@@ -43,10 +43,11 @@ constexpr unsigned long long kWaitLimitF = 2000000000ull;
 
 struct F32Args {
     const float* in; const uint8_t* wp; const float* w; const float* bias; float* out;   // wp: [groups * nb_g][chunks][taps][4][3 BN][8] bf16
-                                                  // w: [groups][taps][Cig filled up to 16s][nb_g * BN] float, for pixels computed by FMAs
+                                                  // w: [groups][Cig filled up to 16s][taps][nb_g * BN] float, for pixels computed by FMAs
     const int32_t* tile_list; const int32_t* tile_count; const uint32_t* masks;
     int Hi, Wi, Ci, Ho, Wo, Co, p, relu, tiles_x, tiles_y;
     int Cig, Cog, nb_g, NB, chunks, ks_last;      // channels per group; blocks per group and in all; patches; steps of 16 channels in the last
+    int fma_ci, fma_ks;                           // sums by FMAs: every fma_ks-th run of fma_ci channels in a chain of its own (dc_simt_order)
     int stages;
     int vec;                                      // four input channels are one aligned load
     int early;
@@ -55,8 +56,15 @@ struct F32Args {
     int skip_loads;
 };
 
-// Channels of the output's staging (32 pixels for each warp): a warp's half, or as many as fit.
+// Channels of the output's staging (32 pixels for each warp): a warp's half, or as many as fit.  Its bytes for a warp: at least what
+// fma_pixels keeps there, some channels of the window that 4 x 8 pixels see and their weights for 16 channels of the output.
 __host__ __device__ constexpr int f32_stage_ch(int BN, int KW) { return BN == 32 ? 16 : KW == 5 ? 8 : 32; }
+__host__ __device__ constexpr int f32_window_ch(int KW) { return KW == 5 ? 1 : 8; }
+__host__ __device__ constexpr int f32_stage_bytes(int BN, int KW)
+{
+    const int out = 32 * (f32_stage_ch(BN, KW) + 4) * 4, fma = (KW == 1 ? f32_window_ch(KW) : KW * KW) * 64 + f32_window_ch(KW) * (DC_TILE_W + KW - 1) * (4 + KW - 1) * 4;
+    return out > fma ? out : fma;
+}
 
 struct __align__(16) CtlF {
     unsigned long long full[kStagesF], empty[kStagesF], a_full[2], a_empty[2], t_full[2], t_empty[2];
@@ -87,6 +95,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r)
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void sts32(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+__device__ __forceinline__ float lds32(uint32_t addr)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
 {
     uint32_t r;
@@ -103,6 +118,97 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t&
     a -= __uint_as_float(p1 << 16); b -= __uint_as_float(p1 & 0xffff0000u);
     p2 = bf16_pair(a, b);
     odd |= __float_as_uint(a) | __float_as_uint(b);
+}
+
+// A warp's 4 x 8 pixels, from row y0, column x0 of stream s on, whose `redo` is set, channels c0 ... of group grp, by FMAs: a value of the patch
+// does not split, or a sum overflowed.  In the order of k_conv_simt's sums, so that the bits are that kernel's, also where the order decides
+// between infinity and NaN.  XC channels of the window that the pixels see and the weights of STEP channels lie in shared memory (`stage`, the warp's
+// own); the weights travel while the ones before are in use.
+template <int BN, int KW>
+__device__ __forceinline__ void fma_pixels(const F32Args& a, uint32_t stage, int s, int y0, int x0, int grp, int c0, bool redo)
+{
+    constexpr int TAPS = KW * KW, WX = DC_TILE_W + KW - 1, WIN = WX * (4 + KW - 1), XC = f32_window_ch(KW), STEP = KW == 1 ? XC : 1;
+    constexpr int ROWS = STEP * TAPS, QUADS = ROWS * 4, WQ = (QUADS + 31) / 32, XQ = XC < 4 ? 1 : XC / 4;
+    const int lane = threadIdx.x & 31, cog = a.nb_g * BN, cig = (a.Cig + 15) & ~15, ci = a.fma_ci, n_ks = a.fma_ks;
+    const float* const in = a.in + (size_t)s * a.Hi * a.Wi * a.Ci + grp * a.Cig;
+    const uint32_t window = stage + ROWS * 64, mine = window + (lane / DC_TILE_W * WX + lane % DC_TILE_W) * 4;
+    auto fill = [&](int c) {                                               // channels c ... of the window, [channel][pixel]
+#pragma unroll 1
+        for (int u = lane; u < WIN * XQ; u += 32) {
+            const int px = u / XQ, i = u % XQ * 4, wy = px / WX, y = y0 - a.p + wy, x = x0 - a.p + px - wy * WX;
+            const int left = (unsigned)y < (unsigned)a.Hi && (unsigned)x < (unsigned)a.Wi ? a.Cig - c - i : 0;
+            const float* p = in + ((size_t)y * a.Wi + x) * a.Ci + c + i;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (XC >= 4 && a.vec) { if (left > 0) v = dc_ld((const float4*)p); }
+            else {
+                if (left > 0) v.x = dc_ld(p);
+                if (XC > 1 && left > 1) v.y = dc_ld(p + 1);
+                if (XC > 2 && left > 2) v.z = dc_ld(p + 2);
+                if (XC > 3 && left > 3) v.w = dc_ld(p + 3);
+            }
+            const uint32_t at = window + (i * WIN + px) * 4;
+            sts32(at, v.x);
+            if constexpr (XC > 1) { sts32(at + WIN * 4, v.y); sts32(at + 2 * WIN * 4, v.z); sts32(at + 3 * WIN * 4, v.w); }
+        }
+    };
+#pragma unroll 1
+    for (int c_out = c0; c_out < min(c0 + BN / 2, a.Cog); c_out += 16) {
+        const float* const k0 = a.w + ((size_t)grp * TAPS * cig + lane / 4) * cog + c_out + lane % 4 * 4;
+        float sum[16];
+#pragma unroll 1
+        for (int ks = 0; ks < n_ks; ++ks) {
+            float part[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) part[j] = 0.f;
+            float4 wn[WQ];
+            auto weights = [&](int c) {
+#pragma unroll
+                for (int q = 0; q < WQ; ++q)
+                    if (lane + 32 * q < QUADS) wn[q] = __ldg((const float4*)(k0 + ((size_t)c * TAPS + 8 * q) * cog));
+            };
+            int c = ks * ci;
+            if (c < a.Cig) weights(c);
+#pragma unroll 1
+            while (c < a.Cig) {
+                __syncwarp();
+                fill(c);
+#pragma unroll 1
+                for (int i = 0; i < XC; i += STEP) {
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < WQ; ++q)
+                        if (lane + 32 * q < QUADS)
+                            sts128(stage + (lane + 32 * q) * 16, __float_as_uint(wn[q].x), __float_as_uint(wn[q].y), __float_as_uint(wn[q].z), __float_as_uint(wn[q].w));
+                    __syncwarp();
+                    c += STEP;
+                    if (c % ci == 0) c += (n_ks - 1) * ci;                 // the chain's next run of channels
+                    if (c < cig) weights(c);
+#pragma unroll
+                    for (int r = 0; r < ROWS; ++r) {
+                        const float v = lds32(mine + ((i + r / TAPS) * WIN + r % TAPS / KW * WX + r % TAPS % KW) * 4);
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4) {
+                            const uint4 w = lds128(stage + r * 64 + j * 4);
+                            part[j] = fmaf(v, __uint_as_float(w.x), part[j]); part[j + 1] = fmaf(v, __uint_as_float(w.y), part[j + 1]);
+                            part[j + 2] = fmaf(v, __uint_as_float(w.z), part[j + 2]); part[j + 3] = fmaf(v, __uint_as_float(w.w), part[j + 3]);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[j] = ks == 0 ? part[j] : sum[j] + part[j];
+        }
+        float* o = a.out + (((size_t)s * a.Ho + y0 + lane / DC_TILE_W) * a.Wo + x0 + lane % DC_TILE_W) * a.Co + grp * a.Cog + c_out;
+        const float* bias = a.bias + grp * a.Cog + c_out;
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+            if (!redo || c_out + j >= a.Cog) continue;                     // channels come in fours
+            float4 v = make_float4(sum[j] + __ldg(bias + j), sum[j + 1] + __ldg(bias + j + 1), sum[j + 2] + __ldg(bias + j + 2), sum[j + 3] + __ldg(bias + j + 3));
+            if (a.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+            *(float4*)(o + j) = v;
+        }
+    }
+    __syncwarp();
 }
 
 template <int BN, int KW>
@@ -249,7 +355,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
         auto tile_of = [&](int item) { return item < n_items ? __ldcg(a.tile_list + item / a.NB) : 0; };
         int next = tile_of(blockIdx.x);
         if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
-        const uint32_t stage = smem_u32(ctl + 1) + (warp - 2) * 32 * STAGE_PITCH;
+        const uint32_t stage = smem_u32(ctl + 1) + (warp - 2) * f32_stage_bytes(BN, KW);
         uint32_t set = 0, set_ph = 0;
         int seq = 0;
         for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++seq) {
@@ -295,67 +401,9 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
 #pragma unroll
             for (int j = 0; j < CH; ++j) beyond = fmaf(sum[j], 0.f, beyond);
             const bool redo = active && (beyond != beyond || ctl->odd[seq % kTileFlags] == seq + 1);
-            if (__any_sync(0xffffffffu, redo)) {
-                // A value of the patch does not split, or a sum overflowed: such pixels once more, by FMAs.  The warp brings the weights of 16
-                // channels to shared memory while the ones before are in use; 16 channels of a tap are a sum of their own, which keeps the error
-                // below that of one chain.
-                const int cog = a.nb_g * BN, cig = (a.Cig + 15) & ~15;
-#pragma unroll
-                for (int h = 0; h < CH; h += 16) {
-                    const float* k = a.w + ((size_t)grp * KW * KW * cig + lane / 4) * cog + c0 + h + lane % 4 * 4;
-                    float4 w0 = __ldg((const float4*)k), w1 = __ldg((const float4*)(k + 8 * (size_t)cog));
-                    if (redo) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) sum[h + j] = 0.f;
-                    }
-#pragma unroll 1
-                    for (int t = 0; t < KW * KW; ++t) {
-                        const int iy = y - a.p + t / KW, ix = x - a.p + t % KW;
-                        const bool inside = redo && iy >= 0 && iy < a.Hi && ix >= 0 && ix < a.Wi;
-                        const float* p = a.in + (((size_t)s * a.Hi + iy) * a.Wi + ix) * a.Ci + grp * a.Cig;
-#pragma unroll 1
-                        for (int c = 0; c < cig; c += 16) {
-                            float e[16], part[16];
-#pragma unroll
-                            for (int i = 0; i < 16; i += 4) {
-                                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                                if (inside && c + i < a.Cig) {
-                                    if (a.vec) v = dc_ld((const float4*)(p + c + i));
-                                    else {
-                                        v.x = dc_ld(p + c + i);
-                                        if (c + i + 1 < a.Cig) v.y = dc_ld(p + c + i + 1);
-                                        if (c + i + 2 < a.Cig) v.z = dc_ld(p + c + i + 2);
-                                        if (c + i + 3 < a.Cig) v.w = dc_ld(p + c + i + 3);
-                                    }
-                                }
-                                e[i] = v.x; e[i + 1] = v.y; e[i + 2] = v.z; e[i + 3] = v.w;
-                            }
-                            __syncwarp();
-                            sts128(stage + lane * 16, __float_as_uint(w0.x), __float_as_uint(w0.y), __float_as_uint(w0.z), __float_as_uint(w0.w));
-                            sts128(stage + 512 + lane * 16, __float_as_uint(w1.x), __float_as_uint(w1.y), __float_as_uint(w1.z), __float_as_uint(w1.w));
-                            __syncwarp();
-                            if (t + 1 < KW * KW || c + 16 < cig) { k += 16 * (size_t)cog; w0 = __ldg((const float4*)k); w1 = __ldg((const float4*)(k + 8 * (size_t)cog)); }
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) part[j] = 0.f;
-#pragma unroll
-                            for (int i = 0; i < 16; ++i)
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4) {
-                                    const uint4 w = lds128(stage + i * 64 + j * 4);
-                                    part[j] = fmaf(e[i], __uint_as_float(w.x), part[j]); part[j + 1] = fmaf(e[i], __uint_as_float(w.y), part[j + 1]);
-                                    part[j + 2] = fmaf(e[i], __uint_as_float(w.z), part[j + 2]); part[j + 3] = fmaf(e[i], __uint_as_float(w.w), part[j + 3]);
-                                }
-                            if (redo) {
-#pragma unroll
-                                for (int j = 0; j < 16; ++j) sum[h + j] += part[j];
-                            }
-                        }
-                    }
-                }
-            }
             // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
             // warp touched 32 lines, and the stores took as long as the MMAs)
-            const uint32_t todo = __ballot_sync(0xffffffffu, active);
+            const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
             const int part = lane % (STAGE_CH / 4);
 #pragma unroll
             for (int c = 0; c < CH; c += STAGE_CH) {
@@ -376,6 +424,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
                     if ((todo >> p) & 1u) *(float4*)(tile_out + ((size_t)(q * 4 + p / 8) * a.Wo + p % 8) * a.Co + c + 4 * part) = v;
                 }
             }
+            if (__any_sync(0xffffffffu, redo)) fma_pixels<BN, KW>(a, stage, s, ty * DC_TILE_H + q * 4, tx * DC_TILE_W, grp, c0, redo);     // (the sums are done with: no registers to save)
         }
     } else {
         // ---------------- input patches, split into pieces ----------------
@@ -492,15 +541,15 @@ __global__ void k_pack_f32(const float* w, int taps, int Cig, int Cog, int nb_g,
     }
 }
 
-// The same weights as floats, [cout][taps][Cig] -> [groups][taps][Cig filled up to 16s][nb_g * BN] with zeros beyond the last channels.
+// The same weights as floats, [cout][taps][Cig] -> [groups][Cig filled up to 16s][taps][nb_g * BN] with zeros beyond the last channels.
 __global__ void k_pack_f32_fma(const float* w, int taps, int Cig, int Cog, int cig, int cog, size_t total, float* out)
 {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         size_t r = i;
         const int n = (int)(r % cog); r /= cog;
-        const int c = (int)(r % cig); r /= cig;
-        const int t = (int)(r % taps);
-        const size_t grp = r / taps;
+        const int t = (int)(r % taps); r /= taps;
+        const int c = (int)(r % cig);
+        const size_t grp = r / cig;
         out[i] = n < Cog && c < Cig ? w[((grp * Cog + n) * taps + t) * Cig + c] : 0.f;
     }
 }
@@ -578,7 +627,7 @@ int dc_settle_weights_f32(dc_cache* c)
 template <int BN, int KW>
 static int launch_f32(dc_cache* c, F32Args& a, int grid)
 {
-    constexpr int a_total = 2 * 3 * 4 * 16 * (DC_TILE_W + KW - 1) * (DC_TILE_H + KW - 1), stage = KW * 4 * 3 * BN * 16, staging = kSumWarps * 32 * (f32_stage_ch(BN, KW) + 4) * 4;
+    constexpr int a_total = 2 * 3 * 4 * 16 * (DC_TILE_W + KW - 1) * (DC_TILE_H + KW - 1), stage = KW * 4 * 3 * BN * 16, staging = kSumWarps * f32_stage_bytes(BN, KW);
     constexpr int room = (226 * 1024 - (int)sizeof(CtlF) - staging - a_total) / stage;
     static_assert(room >= 2, "two kernel rows of weights fit");
     a.stages = room > kStagesF ? kStagesF : room;
@@ -601,6 +650,7 @@ int dc_launch_conv_f32(dc_cache* c, int layer, const void* in, void* out, const 
     a.p = L.d.ph; a.relu = L.d.relu; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y;
     a.Cig = L.d.cin / G; a.Cog = L.d.cout / G; a.nb_g = dc_div_up(a.Cog, BN); a.NB = G * a.nb_g; a.chunks = dc_div_up(a.Cig, kChF);
     a.ks_last = (a.Cig - (a.chunks - 1) * kChF + 15) / 16;
+    dc_simt_order(c, L, &a.fma_ci, &a.fma_ks);
     a.vec = a.Ci % 4 == 0 && a.Cig % 4 == 0 && (uintptr_t)in % 16 == 0;
     a.status = c->status; a.wait_ns = kWaitLimitF; a.skip_loads = 0;
     if (c->debug_stall_ms > 0) { a.wait_ns = (unsigned long long)c->debug_stall_ms * 1000000ull; a.skip_loads = 1; c->debug_stall_ms = 0; }

@@ -366,6 +366,12 @@ static SimtShape simt_shape(const dc_cache* c, const dc_layer_rt& L)
     return s;
 }
 
+void dc_simt_order(const dc_cache* c, const dc_layer_rt& L, int* ci, int* ks)
+{
+    const SimtShape s = simt_shape(c, L);
+    *ci = s.CI; *ks = s.KS;
+}
+
 template <typename T, int KW, int CI, int BN, int TC, int KS>
 static int launch_simt(dc_cache* c, const SimtArgs& a, int max_tiles)
 {
