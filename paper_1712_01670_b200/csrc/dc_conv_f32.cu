@@ -23,12 +23,14 @@
 // Measured, 24 streams, all tiles, us (CUDA cores, here): 32 -> 32 at 227 x 227 451, 203; 32 -> 64 at 113 x 113 246, 80; 64 -> 64 461, 134;
 // 64 -> 128 at 56 x 56 213, 71.  One stream: 29.4, 14.6; 19.8, 8.9; 32.5, 13.1; 17.3, 11.0.
 //
-// Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf), nor do most floats below 2^-110, whose last bits lie under the
-// smallest bf16 of 2^-133: whatever leaves a remainder behind its third piece.  A tile that holds one is marked by the warps
-// that split it and its pixels are computed once more with FMAs from the float weights; weights like that keep the layer
-// on the CUDA cores.  The same is done for a pixel with a sum that is not finite: where operands that do split add up to more than a
-// float holds, the three accumulators can become infinities of either sign, and their sum NaN.  With all pixels computed so, 64 -> 64 channels,
-// 3 x 3 at 113 x 113, 4 streams, takes 405 us (43 on the tensor cores, 118 on k_conv_simt; a channel after the other from global memory 12 ms).
+// Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf), nor do most floats below 2^-110, whose last bits lie
+// under the smallest bf16 of 2^-133: whatever leaves a remainder behind its third piece.  The warps that split a tile mark it if it
+// holds one, and its pixels are computed by FMAs (fma_pixels); weights like that keep the layer on the CUDA cores.
+// FMAs compute two kinds of pixels more.  A sum that is not finite: where operands that do split add up to more than a float holds, the
+// accumulators of the three sizes can become infinities of either sign, and their sum NaN.  A sum below 2^-100 other than zero: its
+// small terms lie where floats have fewer bits, and the tensor core cuts there more often than FMAs round (twice the error at 2^-132).
+// With every pixel computed so, 64 -> 64 channels, 3 x 3 at 113 x 113, 4 streams, takes 405 us (43 on the tensor cores, 118 on
+// k_conv_simt; a channel after the other from global memory took 12 ms).
 #include "dc_common.cuh"
 #include "dc_tcgen05.cuh"
 
@@ -39,6 +41,7 @@ constexpr int kStagesF = 8;                       // weight stages at most
 constexpr int kChF = 32;                          // input channels per patch
 constexpr int kRowsPerDrain1 = 3;                 // 1 x 1 kernels: patches between two drains (6 steps of 16 channels, as a row of a 3 x 3 kernel)
 constexpr int kTileFlags = 8;                     // more than the items between the splitting warps and the epilogue (at most 5)
+constexpr float kSmallSum = 0x1p-100f;            // below it the tensor core's cuts at 2^-149 may count for more than an FMA's roundings
 constexpr unsigned long long kWaitLimitF = 2000000000ull;
 
 struct F32Args {
@@ -102,6 +105,18 @@ __device__ __forceinline__ float lds32(uint32_t addr)
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
     return v;
 }
+__device__ __forceinline__ float max3_abs(float a, float b, float c)       // of the magnitudes; NaN if one of them is
+{
+    float r;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float min3_abs(float a, float b, float c)       // of the magnitudes that are not NaN
+{
+    float r;
+    asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
 {
     uint32_t r;
@@ -123,9 +138,10 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& p0, uint32_t&
 // A warp's 4 x 8 pixels, from row y0, column x0 of stream s on, whose `redo` is set, channels c0 ... of group grp, by FMAs: a value of the patch
 // does not split, or a sum overflowed.  In the order of k_conv_simt's sums, so that the bits are that kernel's, also where the order decides
 // between infinity and NaN.  XC channels of the window that the pixels see and the weights of STEP channels lie in shared memory (`stage`, the warp's
-// own); the weights travel while the ones before are in use.
+// own); the weights travel while the ones before are in use.  A call, and behind the stores, where the sums are no longer needed: inlined, or with
+// the sums to keep, its registers cost the ordinary tiles 2 to 20 % (small CNN, 24 streams: 710 us a pass so, 732 inlined, 705 without it).
 template <int BN, int KW>
-__device__ __forceinline__ void fma_pixels(const F32Args& a, uint32_t stage, int s, int y0, int x0, int grp, int c0, bool redo)
+__device__ __noinline__ void fma_pixels(const F32Args& a, uint32_t stage, int s, int y0, int x0, int grp, int c0, bool redo)
 {
     constexpr int TAPS = KW * KW, WX = DC_TILE_W + KW - 1, WIN = WX * (4 + KW - 1), XC = f32_window_ch(KW), STEP = KW == 1 ? XC : 1;
     constexpr int ROWS = STEP * TAPS, QUADS = ROWS * 4, WQ = (QUADS + 31) / 32, XQ = XC < 4 ? 1 : XC / 4;
@@ -212,7 +228,7 @@ __device__ __forceinline__ void fma_pixels(const F32Args& a, uint32_t stage, int
 }
 
 template <int BN, int KW>
-__global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
+__global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant__ F32Args a)
 {
     constexpr int PW = DC_TILE_W + KW - 1, PX = PW * (DC_TILE_H + KW - 1), PLANE = PX * 16, PIECE = 4 * PLANE, A_SLOT = 3 * PIECE;
     constexpr int TAP = 4 * 3 * BN * 16, B_STAGE = KW * TAP;              // weights of a tap, of a kernel row
@@ -397,10 +413,15 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
             const int nb = item % a.NB, grp = nb / a.nb_g, c0 = (nb - grp * a.nb_g) * BN + half * CH, n = min(CH, a.Cog - c0);
             float* const tile_out = a.out + (((size_t)s * a.Ho + ty * DC_TILE_H) * a.Wo + tx * DC_TILE_W) * a.Co + grp * a.Cog + c0;
             const float* bias = a.bias + grp * a.Cog + c0;
-            float beyond = 0.f;                                            // NaN if a sum is not finite
+            float most = 0.f, least = INFINITY;                            // magnitudes; NaN counts among the largest
 #pragma unroll
-            for (int j = 0; j < CH; ++j) beyond = fmaf(sum[j], 0.f, beyond);
-            const bool redo = active && (beyond != beyond || ctl->odd[seq % kTileFlags] == seq + 1);
+            for (int j = 0; j < CH; j += 2) { most = max3_abs(most, sum[j], sum[j + 1]); least = min3_abs(least, sum[j], sum[j + 1]); }
+            bool small = false;
+            if (least < kSmallSum) {
+#pragma unroll
+                for (int j = 0; j < CH; ++j) small = small || (fabsf(sum[j]) < kSmallSum && sum[j] != 0.f);
+            }
+            const bool redo = active && (!(most < INFINITY) || small || ctl->odd[seq % kTileFlags] == seq + 1);
             // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
             // warp touched 32 lines, and the stores took as long as the MMAs)
             const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
@@ -424,7 +445,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const F32Args a)
                     if ((todo >> p) & 1u) *(float4*)(tile_out + ((size_t)(q * 4 + p / 8) * a.Wo + p % 8) * a.Co + c + 4 * part) = v;
                 }
             }
-            if (__any_sync(0xffffffffu, redo)) fma_pixels<BN, KW>(a, stage, s, ty * DC_TILE_H + q * 4, tx * DC_TILE_W, grp, c0, redo);     // (the sums are done with: no registers to save)
+            if (__any_sync(0xffffffffu, redo)) fma_pixels<BN, KW>(a, stage, s, ty * DC_TILE_H + q * 4, tx * DC_TILE_W, grp, c0, redo);
         }
     } else {
         // ---------------- input patches, split into pieces ----------------

@@ -1621,6 +1621,29 @@ def test_conv_fp32_operands_too_small_to_split(e, f, monkeypatch):
     assert err[0] <= 1.1 * err[1] and err[1] < 3e-7
 
 
+@pytest.mark.parametrize("e,f", [(-55, -55), (-60, -60), (-63, -63), (-66, -66), (-70, -70), (-73, -70), (-20, -100)])
+def test_conv_fp32_products_where_floats_have_fewer_bits(e, f, monkeypatch):
+    """Inputs of 2^e and weights of 2^f that split, but whose small products or sums lie under the smallest normal float: no further from 64-bit
+    sums than the CUDA-core kernel."""
+    g = rng(79)
+    nb = nets.NetBuilder(48, 40)
+    nb.conv(nb.conv(-1, 32, 1, 1, 0), 64, 3, 1, 1, 0)
+    wts = np.ldexp(g.normal(size=(64, 3, 3, 32)).astype(np.float32), f)
+    x = np.zeros((1, 48, 40, 32), np.float32)
+    x[:, :30] = np.ldexp(g.normal(size=(1, 30, 40, 32)).astype(np.float32), e)      # (zeros split)
+    x = torch.from_numpy(x).cuda()
+    want = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), torch.from_numpy(wts).cuda().double().permute(0, 3, 1, 2), padding=1).permute(0, 2, 3, 1)
+    err = []
+    for cores in (False, True):
+        if cores:
+            monkeypatch.setenv("DC_NO_TENSOR_CORES", "1")
+        dc = DeepCache(40, 48, nb.layers, [np.zeros((32, 1, 1, 3), np.float32), wts], [np.zeros(32, np.float32), np.zeros(64, np.float32)],
+                       n_streams=1, block=16, search_range=4, dtype=B.DC_FP32, max_regions=4)
+        err.append(float((dc.conv_partial(1, x).double() - want).norm() / want.norm()))
+        dc.close()
+    assert err[0] <= err[1]
+
+
 def test_conv_fp32_weights_that_do_not_split(monkeypatch):
     g = rng(78)
     nb = nets.NetBuilder(24, 40)
