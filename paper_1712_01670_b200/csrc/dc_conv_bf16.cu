@@ -1180,7 +1180,8 @@ static void set_wait_limit(dc_cache* c, TcArgs& a)
 static int n_groups(const dc_layer_desc& d) { return d.groups > 1 ? d.groups : 1; }
 // Output channels come in blocks of 32.  An ungrouped layer whose channels do not is seen with them filled up (weight rows beyond the last
 // are zeros, by the loads or by k_pack_halo; the epilogue stores what exists): 32 -> 16 channels at 64 x 80, 16 streams, 27 us on
-// the CUDA cores, 7 here.  Single output pixels stay with k_dense, and with more than 4096 channels the bias is not staged.
+// the CUDA cores, 7 here; the error against 64-bit sums is the same, 1.6485e-3, nearly all of it the rounding to bf16.  Single
+// output pixels stay with k_dense, and with more than 4096 channels the bias is not staged.
 static dc_layer_desc group_view(const dc_layer_desc& d)
 {
     dc_layer_desc g = d;

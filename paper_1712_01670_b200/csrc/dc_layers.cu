@@ -378,10 +378,12 @@ __global__ void k_lrn(const T* in, int H, int W, int C, int S, int r, float alph
     }
 }
 
-// The same for 16-byte vectors of channels, R known.  A thread takes Y rows of one column, so that the squares of a row are summed along x
-// once for all the outputs above and below it, and beta = 3/4 (the default) takes two reciprocal square roots (inverse_3_4).
-// What bounds it: instructions (some 200 per vector of eight channels) and the loads behind them.  16 streams, 32 channels at 128 x 160, R = 1: 43 us (a thread per output, two correctly
-// rounded square roots and a division), 24 now; 64 channels at 32 x 40, R = 2, Y = 1: 14, 10.
+// The same for 16-byte vectors of channels, R known.  A thread takes Y rows of one column, so that the squares of a row are
+// summed along x once for all the outputs above and below it, and beta = 3/4 (the default) takes two reciprocal square
+// roots (inverse_3_4).  What bounds it: instructions (some 200 per vector of eight channels) and the loads behind them.
+// us with a thread per output, two rounded square roots and a division, and so (16 streams):
+//   32 channels at 128 x 160, R = 1           43, 24
+//   64 channels at 32 x 40, R = 2 (Y = 1)     14, 10
 template <typename T> struct Unpack;
 template <> struct Unpack<float> {
     static __device__ __forceinline__ void get(uint4 v, float* f) { f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w); }
@@ -403,8 +405,8 @@ template <> struct Unpack<__nv_bfloat16> {
     }
 };
 
-// d^(-3/4): d^(-1/2) and then (d^(1/2))^(-1/2), each with one Newton step (relative error below 2^-23 together, as the two rounded square
-// roots and the division that they replace).
+// d^(-3/4): d^(-1/2) and then (d^(1/2))^(-1/2), each with one Newton step (relative error up to 1.5 * 2^-23 together; up to
+// 1.9 with the two rounded square roots and the division that they replace).
 __device__ __forceinline__ float rsqrt_step(float d)
 {
     const float y = rsqrtf(d), e = fmaf(-d * y, y, 1.f);

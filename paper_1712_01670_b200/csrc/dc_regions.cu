@@ -112,11 +112,12 @@ __device__ __forceinline__ void store_region(dc_region* t, const dc_region& o)
     p[0] = make_uint2(o.x, o.y); p[1] = make_uint2(o.w, o.h); p[2] = make_uint2(o.sx, o.sy);
 }
 
-// One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a later layer than
-// the next one needs (residual branches) wait in shared memory, and so does the layer table: the walk is a chain of a few dozen
-// arithmetic steps per layer (through a table in global memory it was a chain of memory round trips: 48 us for the 71 layers of
-// ResNet-50; with an atomic per rectangle and layer, waited for on the way, 27, 24 so; VGG, 8 full-HD frames, 12.5 and 7.7).  A warp whose rectangles have all vanished,
-// those kept for later layers too, writes the zeros of the layers that are left without walking them.
+// One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a
+// later layer than the next one needs (residual branches) wait in shared memory, and so does the layer table: the walk is
+// a chain of a few dozen arithmetic steps per layer.  A warp whose rectangles have all vanished, those kept for later layers
+// too, writes the zeros of the layers that are left without walking them.
+// us for ResNet-50's 71 layers: table in global memory 48, an atomic per rectangle and layer 27, so 24; VGG, 8 full-HD
+// frames: 12.5 with the atomics, 7.7 so.
 // alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most of a
 // frame's erode within a few layers, and the reuse step tests every tile against all it is given.  A warp asks for its places in a
 // layer's list with one atomic and fills them while the next layer is worked out.
