@@ -126,7 +126,6 @@ struct dc_cache {
     int32_t* n_regions;             // [S]
     dc_region* table;               // [n_layers][S][max_regions]
     dc_region* live;                // [n_layers][S][max_regions] per layer the rectangles that have not eroded away, closed up
-    int prop_slots;                 // rectangles a thread of region propagation keeps for later layers
     void* prop_table;               // [n_layers] the layer table as region propagation reads it (dc_regions.cu)
     int32_t* dirty_count;           // [n_layers]
     int32_t* partial;               // dc_conv_partial: a running 64-bit counter (zero between launches), dirty tiles, [S] reused pixels (not read)

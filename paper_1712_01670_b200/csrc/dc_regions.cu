@@ -1,8 +1,8 @@
 // Region propagation (Section 5, Table 2) and the reuse step of the cache-aware convolution
 // (Section 5, "Reuse": copy cached regions, build the bitmap, list what is left to compute).
 //
-//   k_propagate      one thread per (stream, rectangle slot) walks the layer table in order and
-//                    writes the rectangle's image after every layer; a vanished rectangle is all zeros.
+//   k_propagate      four lanes per (stream, rectangle slot) walk the layer table in order and
+//                    leave the rectangle's image after every layer; a vanished rectangle is all zeros.
 //   k_classify_copy  one warp per 16x8 output tile: lanes test the stream's rectangles against
 //                    the tile, OR their coverage into a 128-bit bitmap, the warp copies each
 //                    covered row span from the cached map with bulk copies (global -> shared ->
@@ -43,155 +43,155 @@ __device__ __forceinline__ void resize_axis(int x, int w, int n_in, int n_out, i
 
 __device__ __forceinline__ dc_region empty_region() { dc_region e = {0, 0, 0, 0, 0, 0}; return e; }
 
-// A layer as propagation sees it.  from0 / from1: where the input's rectangle is: kFrame, kPrevious (the layer before, still in
-// registers), kTable (the table in global memory), or one of the kSlots places of the thread in shared memory; keep: the
-// place that this layer's own rectangle takes, or -1.  drop: places whose rectangles no later layer needs (bit mask); closed: no later
-// layer reads the frame's rectangle or the table.
-// window: the rule is that of a sliding window whose strides are powers of two (convolutions, pooling; LRN is one at stride 1, ReLU one of
-// a single pixel): on either axis first = (x + c1) >> sh, last = (x + w + c2) >> sh.
-constexpr int kSlots = 6, kFrame = -1, kPrevious = -2, kTable = -3;
-struct __align__(16) PropLayer {
-    int window, c1x, c2x, shx, c1y, c2y, shy, from0;
-    int from1, two, in0, in1, keep, drop, closed, kind;
-    int kh, kw, sh, sw, ph, pw, in_h, in_w, out_h, out_w, pad0, pad1;
-};
+// A layer as propagation sees it, the fields of the horizontal axis and of the vertical one side by side.
+// axis[]: {c1, c2, sh, simple}.  The rule of a sliding window whose strides are powers of two (convolutions, pooling; LRN is one at stride 1,
+// ReLU one of a single pixel) is, on either axis, first = (x + c1) >> sh, last = (x + w + c2) >> sh.  simple: such a window on the layer
+// before.
+// links: {in0, in1, kind, until}; kind: kWindow or the layer's; until: the last layer that reads this one's rectangle, kept (later than the
+// next one), and at least the last layer that reads the frame's.
+// rule[]: for the rules that are no such window: {kernel, stride, padding, -}, resize {input, output, -, -}.
+constexpr int kWindow = -1;
+constexpr int kLanes = 4;                                  // lanes per rectangle
+constexpr size_t kWalkBytes = 160 * 1024;                  // shared memory for the rectangles of a batch at all layers
+struct __align__(16) PropLayer { int4 axis[2], links, rule[2]; };
 
-__device__ __forceinline__ dc_region apply_window(const PropLayer& L, dc_region a)
+// A lane's share of a rectangle: where it starts and how long it is on one axis, in the frame (lanes 0: x, 1: y of the four) or in the
+// cached map (2: x, 3: y).  The two shares of an axis have the same length.  A vanished rectangle is all zeros.
+struct Span { int at, len; };
+
+__device__ __forceinline__ Span window_rule(int4 ax, Span a)
 {
-    const int dx = (a.x + L.c1x) >> L.shx, dw = ((a.x + a.w + L.c2x) >> L.shx) - dx + 1;
-    const int dy = (a.y + L.c1y) >> L.shy, dh = ((a.y + a.h + L.c2y) >> L.shy) - dy + 1;
-    // the cached side on its own; smaller size wins
-    const int qx = (a.sx + L.c1x) >> L.shx, qw = ((a.sx + a.w + L.c2x) >> L.shx) - qx + 1;
-    const int qy = (a.sy + L.c1y) >> L.shy, qh = ((a.sy + a.h + L.c2y) >> L.shy) - qy + 1;
-    const int w = min(dw, qw), h = min(dh, qh);
-    if (a.w <= 0 || a.h <= 0 || w <= 0 || h <= 0) return empty_region();
-    dc_region o = {dx, dy, w, h, qx, qy};
+    Span o;
+    o.at = (a.at + ax.x) >> ax.z;
+    o.len = ((a.at + a.len + ax.y) >> ax.z) - o.at + 1;
+    return o;
+}
+// The same for every other layer, the same one in all lanes of the warp.
+__device__ Span general_rule(const PropLayer& L, int lane, Span a, Span b)
+{
+    const unsigned all = 0xffffffffu;
+    const int4 z = L.rule[lane & 1];
+    Span o = {0, 0};
+    switch (L.links.z) {
+    case kWindow: o = window_rule(L.axis[lane & 1], a); break;
+    case DC_CONV: case DC_MAXPOOL: erode_axis(a.at, a.len, z.x, z.y, z.z, o.at, o.len); break;
+    case DC_RESIZE_AREA: resize_axis(a.at, a.len, z.x, z.y, o.at, o.len); break;
+    case DC_ADD: case DC_CONCAT: {
+        // the overlapped region; both inputs must agree on the displacement, on both axes
+        const int da = __shfl_xor_sync(all, a.at, 2) - a.at, db = __shfl_xor_sync(all, b.at, 2) - b.at;
+        const unsigned same = __ballot_sync(all, da == db) >> (lane & ~3);
+        o.at = max(a.at, b.at);
+        o.len = (same & 3u) == 3u && b.len > 0 ? min(a.at + a.len, b.at + b.len) - o.at : 0;
+        break;
+    }
+    case DC_FC: break;
+    default: o = a;
+    }
     return o;
 }
 
-__device__ dc_region apply_layer(const PropLayer& L, dc_region a, dc_region b)
-{
-    if (a.w <= 0 || a.h <= 0) return empty_region();
-    switch (L.kind) {
-    case DC_CONV: case DC_MAXPOOL: case DC_RESIZE_AREA: {
-        // D_t on the current rectangle and, independently, on the cached one; smaller size wins
-        int dx, dw, dy, dh, qx, qw, qy, qh;
-        if (L.kind == DC_RESIZE_AREA) {
-            resize_axis(a.x, a.w, L.in_w, L.out_w, dx, dw);  resize_axis(a.y, a.h, L.in_h, L.out_h, dy, dh);
-            resize_axis(a.sx, a.w, L.in_w, L.out_w, qx, qw); resize_axis(a.sy, a.h, L.in_h, L.out_h, qy, qh);
-        } else {
-            erode_axis(a.x, a.w, L.kw, L.sw, L.pw, dx, dw);  erode_axis(a.y, a.h, L.kh, L.sh, L.ph, dy, dh);
-            erode_axis(a.sx, a.w, L.kw, L.sw, L.pw, qx, qw); erode_axis(a.sy, a.h, L.kh, L.sh, L.ph, qy, qh);
-        }
-        int w = min(dw, qw), h = min(dh, qh);
-        if (w <= 0 || h <= 0) return empty_region();
-        dc_region o = {dx, dy, w, h, qx, qy};
-        return o;
-    }
-    case DC_ADD: case DC_CONCAT: {
-        // the overlapped region; both inputs must agree on the displacement
-        if (b.w <= 0 || b.h <= 0) return empty_region();
-        if (a.sx - a.x != b.sx - b.x || a.sy - a.y != b.sy - b.y) return empty_region();
-        int x0 = max(a.x, b.x), y0 = max(a.y, b.y);
-        int x1 = min(a.x + a.w, b.x + b.w), y1 = min(a.y + a.h, b.y + b.h);
-        if (x1 <= x0 || y1 <= y0) return empty_region();
-        dc_region o = {x0, y0, x1 - x0, y1 - y0, x0 + (a.sx - a.x), y0 + (a.sy - a.y)};
-        return o;
-    }
-    case DC_FC:
-        return empty_region();
-    default:
-        return a;
-    }
-}
-
-// The tables are 8-byte aligned: three stores, not six.
-__device__ __forceinline__ void store_region(dc_region* t, const dc_region& o)
-{
-    uint2* p = (uint2*)t;
-    p[0] = make_uint2(o.x, o.y); p[1] = make_uint2(o.w, o.h); p[2] = make_uint2(o.sx, o.sy);
-}
-
-// One CTA per stream (more for a caller's lists, which count nothing), a thread one rectangle at a time.  Rectangles that a
-// later layer than the next one needs (residual branches) wait in shared memory, and so does the layer table: the walk is
-// a chain of a few dozen arithmetic steps per layer.  A warp whose rectangles have all vanished, those kept for later layers
-// too, writes the zeros of the layers that are left without walking them.
-// us for ResNet-50's 71 layers: table in global memory 48, an atomic per rectangle and layer 27, so 24; VGG, 8 full-HD
-// frames: 12.5 with the atomics, 7.7 so.
+// One CTA per stream (more for a caller's lists, which count nothing), batches of as many rectangles as have room in shared memory at all
+// layers.  First the walk, four lanes per rectangle: the two axes of the rectangle and of its cached image, which only meet where their
+// lengths are compared.  It leaves its rectangles in shared memory and does nothing else, because what bounds it is the chain of a lane's
+// instructions from layer to layer.  A warp whose rectangles have all vanished, those that later layers read too, stops.  Then all warps,
+// a layer at a time each, write the table and the lists.
+// us for ResNet-50's 71 layers, one stream: a thread per rectangle that also wrote the table and asked for its places in the lists layer
+// by layer 26, so 11.
 // alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most of a
-// frame's erode within a few layers, and the reuse step tests every tile against all it is given.  A warp asks for its places in a
-// layer's list with one atomic and fills them while the next layer is worked out.
+// frame's erode within a few layers, and the reuse step tests every tile against all it is given.
 // out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): the lists are wanted, and the
 // counters of the reuse step are zeroed.
-__global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions,
+// walkers: threads that walk (a multiple of 32); dynamic shared memory: 8 * layer_end * walkers bytes.
+__global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions, int walkers,
                                                    const dc_region* in, const int32_t* n_in, dc_region* table, dc_region* live, int32_t* alive, int32_t* reuse_px,
                                                    int32_t* dirty_count, dc_region* out, int out_begin, int32_t* n_out)
 {
     __shared__ PropLayer sl[DC_MAX_LAYERS];
-    extern __shared__ int32_t keep[];                      // [places in use][6][threads]
-    __shared__ int32_t count[DC_MAX_LAYERS];
-    const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+    __shared__ int32_t count[DC_MAX_LAYERS], end_of[32];   // end_of: per walking warp, the layer at which it stopped
+    extern __shared__ __align__(16) int32_t at_all[];      // [layer_end][walkers], then the lengths likewise
+    const unsigned all = 0xffffffffu;
+    const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, per_batch = walkers / kLanes;
+    int32_t* const len_all = at_all + layer_end * walkers;
     for (int i = tid; i < layer_end * (int)(sizeof(PropLayer) / 16); i += nt) ((int4*)sl)[i] = __ldg((const int4*)layers + i);
     if (tid < DC_MAX_LAYERS) count[tid] = 0;
     dc_pdl_wait();
     dc_pdl_release();
-    __syncthreads();
-    const size_t layer_stride = (size_t)S * max_regions;
     const int n = min(n_in[s], max_regions);              // a caller's count beyond the table is cut, never written
     // a caller's list has zeros behind its rectangles
     const int rows = out ? max_regions : n;
-    for (int first = blockIdx.y * nt; first < rows; first += gridDim.y * nt) {
-        const int i = first + tid;
-        const size_t slot = (size_t)s * max_regions + i;
-        const bool on = i < n, there = i < rows;
-        const dc_region r0 = on ? in[slot] : empty_region();
-        dc_region prev = r0;
-        auto fetch = [&](int from, int layer) -> dc_region {
-            if (from == kFrame) return r0;
-            if (from == kPrevious) return prev;
-            if (from == kTable) return on ? table[layer * layer_stride + slot] : empty_region();
-            const int32_t* k = keep + from * 6 * nt + tid;
-            dc_region r = {k[0], k[nt], k[2 * nt], k[3 * nt], k[4 * nt], k[5 * nt]};
-            return r;
-        };
-        uint32_t kept = 0;                                             // places that hold a living rectangle of this thread
-        unsigned noted = 0;                                            // the warp's living rectangles of the layer before (prev), and their
-        int place = 0;                                                 // first place in that layer's list (lane 0)
-        auto list_prev = [&](int layer) {
-            const int at = __shfl_sync(0xffffffffu, place, 0) + __popc(noted & ((1u << lane) - 1u));
-            if ((noted >> lane) & 1u) store_region(live + layer * layer_stride + (size_t)s * max_regions + at, prev);
-        };
-        int l = 0;
-        for (bool dead = i - lane >= rows; l < layer_end && !dead; ++l) {
-            const PropLayer& L = sl[l];
-            const dc_region a = fetch(L.from0, L.in0);
-            dc_region o;
-            if (L.window) o = apply_window(L, a);
-            else o = apply_layer(L, a, L.two ? fetch(L.from1, L.in1) : a);
-            kept &= ~(uint32_t)L.drop;
-            if (L.keep >= 0) {
-                int32_t* k = keep + L.keep * 6 * nt + tid;
-                k[0] = o.x; k[nt] = o.y; k[2 * nt] = o.w; k[3 * nt] = o.h; k[4 * nt] = o.sx; k[5 * nt] = o.sy;
-                kept = o.w > 0 ? kept | (1u << L.keep) : kept & ~(1u << L.keep);
-            }
-            if (there) {
-                store_region(table + l * layer_stride + slot, o);
-                if (out && l >= out_begin) out[(l - out_begin) * layer_stride + slot] = o;
-            }
-            if (noted) list_prev(l - 1);
-            const unsigned living = __ballot_sync(0xffffffffu, o.w > 0);
-            noted = alive ? living : 0u;
-            if (noted && lane == 0) place = atomicAdd(&count[l], __popc(noted));
-            dead = !living && L.closed && !__any_sync(0xffffffffu, kept != 0);
-            prev = o;
+    const size_t layer_stride = (size_t)S * max_regions;
+    for (int first = blockIdx.y * per_batch; first < rows; first += gridDim.y * per_batch) {
+        const int i = first + tid / kLanes;
+        Span r0 = {0, 0};
+        if (tid < walkers && i < n) {
+            const int32_t* r = (const int32_t*)(in + (size_t)s * max_regions + i);
+            r0.at = r[lane & 2 ? 4 + (lane & 1) : lane & 1]; r0.len = r[2 + (lane & 1)];
         }
-        if (noted) list_prev(l - 1);
-        // the zeros: a warp's rectangles are one run of memory
-        const int run = 3 * min(32, rows - (i - lane));
-        for (; l < layer_end; ++l) {
-            uint2* t = (uint2*)(table + l * layer_stride + slot - lane);
-            for (int k = lane; k < run; k += 32) t[k] = make_uint2(0, 0);
-            if (out && l >= out_begin && there) out[(l - out_begin) * layer_stride + slot] = empty_region();
+        __syncthreads();                                   // the layer table; the batch before has been written
+        if (tid < walkers) {
+            const int group = lane & ~3, axis = lane & 1;
+            int l = 0, until = sl[0].links.w;
+            int32_t* at = at_all + tid; int32_t* len = len_all + tid;
+            Span a = r0;
+            unsigned living = __ballot_sync(all, a.len > 0);
+            int4 ax = sl[0].axis[axis];
+            // no later layer reads what is left, or nothing is left at all
+            for (; l < layer_end && (living != 0 || l <= until); ++l, at += walkers, len += walkers) {
+                const int4 ax1 = ax;
+                const int until1 = sl[l].links.w;
+                ax = sl[min(l + 1, layer_end - 1)].axis[axis];
+                Span o;
+                if (ax1.w) o = window_rule(ax1, a);
+                else {
+                    const PropLayer& L = sl[l];
+                    auto fetch = [&](int from) -> Span {
+                        if (from == l - 1 && l > 0) return a;
+                        if (from < 0) return r0;
+                        return Span{at_all[from * walkers + tid], len_all[from * walkers + tid]};
+                    };
+                    const Span b = L.links.z == DC_ADD || L.links.z == DC_CONCAT ? fetch(L.links.y) : Span{0, 0};
+                    a = fetch(L.links.x);
+                    o = general_rule(L, lane, a, b);
+                }
+                // the cached side on its own; smaller size wins; nothing is left unless something is on both axes
+                o.len = min(o.len, __shfl_xor_sync(all, o.len, 2));
+                const unsigned some = __ballot_sync(all, o.len > 0 && a.len > 0);
+                living = some & (some >> 1) & 0x11111111u;
+                const bool on = (living >> group) & 1u;
+                a.at = on ? o.at : 0; a.len = on ? o.len : 0;
+                *at = a.at; *len = a.len;
+                if (living) until = max(until, until1);
+            }
+            if (lane == 0) end_of[warp] = l;
+        }
+        __syncthreads();
+        // a layer per warp, a rectangle per lane
+        const int here = min(per_batch, rows - first);
+        for (int l = warp; l < layer_end; l += nt >> 5) {
+            int listed = count[l];
+            const size_t row = l * layer_stride + (size_t)s * max_regions;
+            for (int k0 = 0; k0 < here; k0 += 32) {
+                const int k = k0 + lane;
+                int2 at = {0, 0}, len = {0, 0}, src = {0, 0};
+                if (k < here && l < end_of[k >> 3]) {
+                    const int32_t* p = at_all + l * walkers + k * kLanes;
+                    at = *(const int2*)p; src = *(const int2*)(p + 2);
+                    len = *(const int2*)(len_all + l * walkers + k * kLanes);
+                }
+                if (k < here) {
+                    int2* t = (int2*)(table + row + first + k);      // the tables are 8-byte aligned
+                    t[0] = at; t[1] = len; t[2] = src;
+                    if (out && l >= out_begin) out[row - out_begin * layer_stride + first + k] = dc_region{at.x, at.y, len.x, len.y, src.x, src.y};
+                }
+                if (!alive) continue;
+                const unsigned m = __ballot_sync(all, len.x > 0);
+                if (len.x > 0) {
+                    int2* t = (int2*)(live + row + listed + __popc(m & ((1u << lane) - 1u)));
+                    t[0] = at; t[1] = len; t[2] = src;
+                }
+                listed += __popc(m);
+            }
+            if (lane == 0) count[l] = listed;
         }
     }
     if (n_out && blockIdx.y == 0) for (int l = out_begin + tid; l < layer_end; l += nt) n_out[(l - out_begin) * S + s] = n_in[s];
@@ -638,48 +638,35 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
 {
     const int n = c->n_layers;
     PropLayer t[DC_MAX_LAYERS];
-    int last_use[DC_MAX_LAYERS];                           // last layer that needs l's rectangle other than as "the layer before"
+    int last_use[DC_MAX_LAYERS], frame_use = -1;           // last layer that reads l's rectangle other than as "the layer before", or the frame's
     for (int l = 0; l < n; ++l) last_use[l] = -1;
     for (int l = 0; l < n; ++l) {
         const dc_layer_desc& d = layers[l];
+        const bool two = d.kind == DC_ADD || d.kind == DC_CONCAT;
+        if (d.in0 < 0 || (two && d.in1 < 0)) frame_use = l;
         if (d.in0 >= 0 && d.in0 != l - 1) last_use[d.in0] = l;
-        if ((d.kind == DC_ADD || d.kind == DC_CONCAT) && d.in1 >= 0 && d.in1 != l - 1) last_use[d.in1] = l;
+        if (two && d.in1 >= 0 && d.in1 != l - 1) last_use[d.in1] = l;
     }
-    int owner[kSlots];
-    for (int k = 0; k < kSlots; ++k) owner[k] = -1;
-    auto from = [&](int l, int in) {
-        if (in < 0) return kFrame;
-        if (in == l - 1) return kPrevious;
-        for (int k = 0; k < kSlots; ++k) if (owner[k] == in) return k;
-        return kTable;
-    };
     for (int l = 0; l < n; ++l) {
         const dc_layer_desc& d = layers[l];
         const int ih = d.in0 < 0 ? c->cfg.height : layers[d.in0].out_h, iw = d.in0 < 0 ? c->cfg.width : layers[d.in0].out_w;
         PropLayer& e = t[l];
         e = PropLayer();
-        e.kind = d.kind; e.kh = d.kh; e.kw = d.kw; e.sh = d.sh; e.sw = d.sw; e.ph = d.ph; e.pw = d.pw;
-        e.in_h = ih; e.in_w = iw; e.out_h = d.out_h; e.out_w = d.out_w; e.in0 = d.in0; e.in1 = d.in1;
-        e.from0 = from(l, d.in0); e.from1 = from(l, d.in1); e.keep = -1;
-        e.two = d.kind == DC_ADD || d.kind == DC_CONCAT;
+        e.links = make_int4(d.in0 < 0 ? -1 : d.in0, d.in1 < 0 ? -1 : d.in1, d.kind, last_use[l] > frame_use ? last_use[l] : frame_use);
+        e.rule[0] = d.kind == DC_RESIZE_AREA ? make_int4(iw, d.out_w, 0, 0) : make_int4(d.kw, d.sw, d.pw, 0);
+        e.rule[1] = d.kind == DC_RESIZE_AREA ? make_int4(ih, d.out_h, 0, 0) : make_int4(d.kh, d.sh, d.ph, 0);
         auto window = [&](int kh, int kw, int sh, int sw, int ph, int pw) {
             if ((sh & (sh - 1)) != 0 || (sw & (sw - 1)) != 0) return;
-            e.window = 1;
-            e.c1x = pw + sw - 1; e.c2x = pw - kw; e.c1y = ph + sh - 1; e.c2y = ph - kh;
-            while ((1 << e.shx) < sw) ++e.shx;
-            while ((1 << e.shy) < sh) ++e.shy;
+            const int simple = l == 0 || d.in0 == l - 1;       // layer 0 reads the frame, which is what the walk starts from
+            e.links.z = kWindow;
+            e.axis[0] = make_int4(pw + sw - 1, pw - kw, 0, simple);
+            e.axis[1] = make_int4(ph + sh - 1, ph - kh, 0, simple);
+            while ((1 << e.axis[0].z) < sw) ++e.axis[0].z;
+            while ((1 << e.axis[1].z) < sh) ++e.axis[1].z;
         };
         if (d.kind == DC_CONV || d.kind == DC_MAXPOOL) window(d.kh, d.kw, d.sh, d.sw, d.ph, d.pw);
         else if (d.kind == DC_LRN) window(2 * d.ph + 1, 2 * d.ph + 1, 1, 1, d.ph, d.ph);
         else if (d.kind == DC_RELU) window(1, 1, 1, 1, 0, 0);
-        for (int k = 0; k < kSlots; ++k) if (owner[k] >= 0 && last_use[owner[k]] <= l) { owner[k] = -1; t[l].drop |= 1 << k; }
-        if (last_use[l] > l)
-            for (int k = 0; k < kSlots; ++k) if (owner[k] < 0) { owner[k] = l; t[l].keep = k; if (k >= c->prop_slots) c->prop_slots = k + 1; break; }
-    }
-    for (int l = n - 1, open = 0; l >= 0; --l) {
-        t[l].closed = !open;
-        auto outside = [](int from) { return from == kFrame || from == kTable; };
-        open = open || outside(t[l].from0) || (t[l].two && outside(t[l].from1));
     }
     if (cudaMalloc(&c->prop_table, sizeof(PropLayer) * n) != cudaSuccess) { cudaGetLastError(); return DC_ERR_ALLOC; }
     c->bytes += sizeof(PropLayer) * n;
@@ -692,13 +679,15 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
 int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out)
 {
     dc_prof_scope ps(c, DC_ST_PROPAGATE);
-    // a thread per rectangle where the frame can have many
-    const int threads = c->max_regions > 512 ? 1024 : 256;
-    const size_t smem = (size_t)c->prop_slots * 6 * threads * sizeof(int32_t);
+    // as many walkers as the rectangles need and shared memory has room for, and at least eight warps for the writing
+    const int room = (int)(kWalkBytes / (8 * (size_t)layer_end)) / 32 * 32, most = room > 1024 ? 1024 : room;
+    const int walkers = c->max_regions >= most / kLanes ? most : dc_div_up(c->max_regions * kLanes, 32) * 32;
+    const int threads = walkers < 256 ? 256 : walkers;
+    const size_t smem = 8 * (size_t)layer_end * walkers;
     static dc_once_per_device attr_set;
-    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_propagate, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlots * 6 * 1024 * (int)sizeof(int32_t)));
-    const dim3 grid((unsigned)c->S, for_frame ? 1u : (unsigned)dc_div_up(c->max_regions, threads));
-    DC_CUDA(dc_launch_pdl(k_propagate, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, in, n_in,
+    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_propagate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+    const dim3 grid((unsigned)c->S, for_frame ? 1u : (unsigned)dc_div_up(c->max_regions, walkers / kLanes));
+    DC_CUDA(dc_launch_pdl(k_propagate, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, walkers, in, n_in,
                           c->table, c->live, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
     c->launches += 1;
     return DC_OK;

@@ -531,6 +531,36 @@ def test_propagate_strides_that_are_no_power_of_two():
     check_propagation(b.layers, 140, 120, 3)
 
 
+def test_propagate_more_rectangles_than_a_batch_holds():
+    """A frame's rectangles in several batches (a deep network leaves room for few of them at once): table, lists and counts of every layer."""
+    b = nets.NetBuilder(128, 128)
+    x = b.conv(-1, 16, 3, 1, 1)
+    for _ in range(59):
+        x = b.conv(x, 16, 1, 1, 0)
+    ws, bs = nets.random_weights(b.layers, 2)
+    dc = DeepCache(128, 128, b.layers, ws, bs, n_streams=2, block=4, search_range=0, dtype=B.DC_BF16)
+    try:
+        f0 = rng(5).integers(0, 256, (2, 128, 128, 3), dtype=np.uint8)
+        f1 = f0.copy()
+        for s in range(2):
+            for y in range(32):
+                for bx in range((y + s) % 3, 32, 3):
+                    f1[s, 4 * y:4 * y + 4, 4 * bx:4 * bx + 4] ^= 0x80
+        dc.infer_frame(f0)
+        _, stats = dc.infer_frame(f1, want_stats=True)
+        regs0, n = dc.layer_regions(-1)
+        for s in range(2):
+            count = int(n[s])
+            assert count > 300
+            want = orc.propagate(b.layers, (128, 128), U.regions_np(regs0[s, :count]))
+            for li in range(len(b.layers)):
+                regs, _ = dc.layer_regions(li)
+                U.assert_regions_equal(U.regions_np(regs[s, :count]), want[li], f"layer {li} stream {s}")
+                assert abs(stats[s].reuse_ratio[li] - float((want[li]["w"] * want[li]["h"]).sum()) / 128 ** 2) < 1e-6
+    finally:
+        dc.close()
+
+
 # ------------------------------------------------------------------ dc_conv_partial
 @pytest.mark.parametrize("dtype", [B.DC_FP32, B.DC_BF16])
 @pytest.mark.parametrize("hi,wi,cin,cout,k,s,p,relu", [
