@@ -486,18 +486,6 @@ __host__ __device__ constexpr int point_y(int i)
     constexpr int t[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1};
     return t[i];
 }
-// The points for look-ups with a run-time index (the same in all lanes of a warp: one constant-cache access).
-__constant__ int c_point_x[13] = {0, -1, 1, -2, 2, -1, 1, 0, 0, 0, -1, 1, 0};
-__constant__ int c_point_y[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1};
-// Per point and window pitch: byte offset of the point's candidate from the centre's, << 16, | the low 16 bits of the
-// point's tie-key offset (py << 8) + px taken modulo 2^16.
-__host__ __device__ constexpr int point_word(int i, int pitch)
-{
-    return (int)(((unsigned)((point_y(i) * pitch + point_x(i)) * 4) << 16) | ((unsigned)(point_y(i) * 256 + point_x(i)) & 0xffffu));
-}
-#define DC_POINT_ROW(p) {point_word(0, p), point_word(1, p), point_word(2, p), point_word(3, p), point_word(4, p), point_word(5, p), \
-                         point_word(6, p), point_word(7, p), point_word(8, p), point_word(9, p), point_word(10, p), point_word(11, p), point_word(12, p)}
-
 // displacements that keep the block inside the previous frame and the search range
 struct WalkBounds { int dx_lo, dx_hi, dy_lo, dy_hi; };
 
@@ -505,19 +493,6 @@ __device__ __forceinline__ WalkBounds walk_bounds(const MatchArgs& a, int x0, in
 {
     WalkBounds b = {max(-a.R, -x0), min(a.R, a.W - bw - x0), max(-a.R, -y0), min(a.R, a.H - bh - y0)};
     return b;
-}
-// which of the 13 points around (cx, cy) are valid candidates
-__device__ __forceinline__ uint32_t valid_points(int cx, int cy, const WalkBounds& b)
-{
-    if (cx - 2 >= b.dx_lo && cx + 2 <= b.dx_hi && cy - 2 >= b.dy_lo && cy + 2 <= b.dy_hi) return 0x1fffu;
-    // near the frame's edge or the range limit (rare): a real loop, so that it is not merged into the path above
-    uint32_t m = 0;
-#pragma unroll 1
-    for (int i = 0; i < 13; ++i) {
-        const int dx = cx + c_point_x[i], dy = cy + c_point_y[i];
-        if (dx >= b.dx_lo && dx <= b.dx_hi && dy >= b.dy_lo && dy <= b.dy_hi) m |= 1u << i;
-    }
-    return m;
 }
 __device__ __forceinline__ uint32_t tie_key(int dx, int dy)
 {
@@ -571,41 +546,82 @@ __device__ __forceinline__ uint32_t lds_at(uint32_t p)
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(p), "n"(OFF) : "memory");
     return v;
 }
-// The candidate's offset from p is known at compile time: the eight loads need no address arithmetic.
-template <int OFF>
-__device__ __forceinline__ uint32_t score_at_fixed(uint32_t p, const uint32_t (&cw)[8], bool row_on)
-{
-    const uint32_t w0 = lds_at<OFF>(p), w1 = lds_at<OFF + 8>(p), w2 = lds_at<OFF + 16>(p), w3 = lds_at<OFF + 24>(p);
-    const uint32_t w4 = lds_at<OFF + 32>(p), w5 = lds_at<OFF + 40>(p), w6 = lds_at<OFF + 48>(p), w7 = lds_at<OFF + 56>(p);
-    uint32_t a0 = 0, a1 = 0, d;
-    d = __vabsdiffu4(cw[0], w0); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[1], w1); a1 = __dp4a(d, d, a1);
-    d = __vabsdiffu4(cw[2], w2); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[3], w3); a1 = __dp4a(d, d, a1);
-    d = __vabsdiffu4(cw[4], w4); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[5], w5); a1 = __dp4a(d, d, a1);
-    d = __vabsdiffu4(cw[6], w6); a0 = __dp4a(d, d, a0);
-    d = __vabsdiffu4(cw[7], w7); a1 = __dp4a(d, d, a1);
-    const uint32_t mine = row_on ? a0 + a1 : 0u;
-    uint32_t sum;
-    asm volatile("redux.sync.add.u32 %0, %1, 0xffffffff;" : "=r"(sum) : "r"(mine));
-    return sum;
-}
-
-// Scores the points of the compile-time set MASK around the centre whose candidate starts at pc: straight-line code,
-// every load at a fixed offset.  Tracks the smallest SSE (ms), the point that gave it (mi) and whether two of
-// the scores that mattered were equal (tie): the caller settles the rare ties with the exact order.
-template <uint32_t MASK, int PITCH, int I = 0>
-__device__ __forceinline__ void score_fixed_set(uint32_t pc, const uint32_t (&cw)[8], bool row_on, uint32_t& ms, int& mi, bool& tie)
-{
-    if constexpr (I < 13) {
-        if constexpr (((MASK >> I) & 1u) != 0) {
-            const uint32_t s = score_at_fixed<(point_y(I) * PITCH + point_x(I)) * 4>(pc, cw, row_on);
-            tie |= s == ms;                                   // selects, no branches: the code stays straight
-            mi = s < ms ? I : mi;
-            ms = min(ms, s);
+// Candidates of one window row, at compile-time displacements LO + 2 m for the set bits m of DXS: they are shifted by whole words against
+// one another, so a word is loaded once for all of them.  p: the address of displacement 0 in that row; n_px: how many of the lane's pixels
+// lie inside the frame.  sum(m, value) takes the scores.
+__host__ __device__ constexpr int high_bit(unsigned long long m) { int n = -1; for (; m; m >>= 1) ++n; return n; }
+__host__ __device__ constexpr int bits_of(unsigned long long m) { int n = 0; for (; m; m &= m - 1) ++n; return n; }
+template <int LO, unsigned long long DXS>
+struct RowWords {
+    static constexpr int N = 8 + high_bit(DXS);
+    uint32_t w[N];
+    template <int K = 0>
+    __device__ __forceinline__ void load(uint32_t p)
+    {
+        if constexpr (K < N) {
+            if constexpr (((DXS << 7) >> K & 0xffull) != 0) w[K] = lds_at<(LO + 2 * K) * 4>(p);         // some m with 0 <= K - m < 8
+            load<K + 1>(p);
         }
-        score_fixed_set<MASK, PITCH, I + 1>(pc, cw, row_on, ms, mi, tie);
+    }
+    template <bool CLIP, typename Sum>
+    __device__ __forceinline__ void score(const uint32_t (&cw)[8], bool row_on, int n_px, const Sum& sum) const
+    {
+        constexpr int C = bits_of(DXS);
+        uint32_t acc[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[c] = 0;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            int c = 0;
+#pragma unroll
+            for (int m = 0; m <= high_bit(DXS); ++m)
+                if (DXS >> m & 1) {
+                    if (k - m >= 0 && k - m < 8) {
+                        const uint32_t d = !CLIP || k - m < n_px ? __vabsdiffu4(cw[(k - m) & 7], w[k]) : 0u;
+                        acc[c] = __dp4a(d, d, acc[c]);
+                    }
+                    ++c;
+                }
+        }
+        int c = 0;
+#pragma unroll
+        for (int m = 0; m <= high_bit(DXS); ++m)
+            if (DXS >> m & 1) { sum(m, __reduce_add_sync(0xffffffffu, row_on ? acc[c] : 0u)); ++c; }
+    }
+};
+
+// The points of the compile-time set MASK around the centre whose candidate starts at pc, row by row: straight-line code, every load at a
+// fixed offset.  Lane i keeps the score of point i.  AHEAD: the words of all rows are on their way before the first is used.
+__host__ __device__ constexpr int point_at(uint32_t mask, int x, int y)
+{
+    for (int i = 0; i < 13; ++i) if ((mask >> i & 1) && point_x(i) == x && point_y(i) == y) return i;
+    return -1;
+}
+__host__ __device__ constexpr int row_lo(uint32_t mask, int y)                     // smallest x of the row's points, 3: none
+{
+    for (int x = -2; x <= 2; ++x) if (point_at(mask, x, y) >= 0) return x;
+    return 3;
+}
+__host__ __device__ constexpr unsigned long long row_dxs(uint32_t mask, int y)
+{
+    unsigned long long b = 0;
+    for (int m = 0; row_lo(mask, y) + 2 * m <= 2; ++m) if (point_at(mask, row_lo(mask, y) + 2 * m, y) >= 0) b |= 1ull << m;
+    return b;
+}
+template <uint32_t MASK, int PITCH, bool AHEAD, int Y = -2>
+__device__ __forceinline__ void score_set(uint32_t pc, const uint32_t (&cw)[8], bool row_on, int lane, uint32_t& mine)
+{
+    if constexpr (Y <= 2) {
+        if constexpr (row_lo(MASK, Y) <= 2) {
+            constexpr int LO = row_lo(MASK, Y);
+            RowWords<LO + Y * PITCH, row_dxs(MASK, Y)> row;
+            row.load(pc);
+            if constexpr (AHEAD) score_set<MASK, PITCH, AHEAD, Y + 1>(pc, cw, row_on, lane, mine);
+            row.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == point_at(MASK, LO + 2 * m, Y) ? v : mine; });
+            if constexpr (!AHEAD) score_set<MASK, PITCH, AHEAD, Y + 1>(pc, cw, row_on, lane, mine);
+        } else {
+            score_set<MASK, PITCH, AHEAD, Y + 1>(pc, cw, row_on, lane, mine);
+        }
     }
 }
 
@@ -614,119 +630,134 @@ __device__ __forceinline__ void score_fixed_set(uint32_t pc, const uint32_t (&cw
 // A round scores one of ten point sets around the current centre: kind 0-7, the points of the large diamond that are
 // new after the move along diamond point `kind` (the others lost to the new centre already and cannot win); kind 8,
 // the first round (centre and all eight points); kind 9, the small diamond.  Outside the first round the centre is
-// the best point so far and bs its SSE.  When all 13 points around the centre are valid candidates the round runs
-// as straight-line code for its set and decides by SSE alone: a point that beats the centre becomes the next centre
-// and names the next round's kind.  Should two SSEs that matter be equal, or the frame edge or the range limit cut
-// the set, the round is (re)done point by point under the full order (SSE, |dx| + |dy|, dy, dx): same result.
+// the best point so far and bs its SSE.  Every point around the centre is staged, so the round runs as straight-line code for
+// its set whatever the frame's edge and the range allow; lane i then drops point i where it is no valid candidate, and the smallest score
+// wins, or the smallest (|dx| + |dy|, dy, dx) among equal ones.  (With a separate path for cut sets and ties, point by point, the walks
+// at the edges set the time of a small frame.)
 constexpr int KIND_FIRST = 8, KIND_SMALL = 9;
+__host__ __device__ constexpr uint32_t kind_mask(int kind)
+{
+    constexpr uint32_t t[10] = {31u, 11u, 21u, 171u, 213u, 168u, 208u, 248u, 0x1ffu, 0x1e00u};
+    return t[kind];
+}
 __constant__ uint32_t c_kind_mask[10] = {31u, 11u, 21u, 171u, 213u, 168u, 208u, 248u, 0x1ffu, 0x1e00u};
-// diamond point of a move (mx, my), indexed by ((my + 2) * 5 + (mx + 2)) >> 1
-__constant__ int c_kind_of_move[13] = {0, 0, 0, 1, 2, 3, 0, 4, 5, 6, 0, 7, 0};
+
+// Displacements in a walk are pairs of 16-bit numbers in one register, dy + kBias above dx + kBias: both axes are compared at once, and
+// a lane's registers are what bounds the warps per SM.
+constexpr int kBias = 128;
+__host__ __device__ constexpr int pair(int dx, int dy) { return dy * 65536 + dx; }                 // a difference of displacements
+__host__ __device__ constexpr int disp(int dx, int dy) { return pair(dx + kBias, dy + kBias); }
+__device__ __forceinline__ int disp_x(int d) { return (d & 0xffff) - kBias; }
+__device__ __forceinline__ int disp_y(int d) { return (d >> 16) - kBias; }
+struct Within { int lo, hi; };                                                                     // a range of displacements
+__device__ __forceinline__ bool within(int d, Within r) { return (int)__vminu2(__vmaxu2((unsigned)d, (unsigned)r.lo), (unsigned)r.hi) == d; }
+
+__device__ __forceinline__ Within walk_range(const WalkBounds& b) { return Within{disp(b.dx_lo, b.dy_lo), disp(b.dx_hi, b.dy_hi)}; }
 
 struct WalkW {
-    int cx, cy, kind;           // centre, and how it was reached
+    int at, kind;               // centre, and how it was reached
     uint32_t bs;                // SSE of the best point so far (the centre, after the first round)
-    int nx, ny; uint32_t ns;    // on return 2: the centre the walk has chosen and not yet moved to, and its SSE
+    int next, nk; uint32_t ns;  // on return 2: the centre the walk has chosen and not yet moved to, the kind of that move, and its SSE
 };
 
-// Three points of such a round at a time, their loads in flight together; n_px: how many of the lane's eight pixels lie
-// inside the frame (fewer than eight for the last block column of a width that is not a multiple of 16).
-struct Edge3 { uint32_t s[3]; };
-__device__ __forceinline__ Edge3 score3(const uint32_t (&p)[3], const uint32_t (&cw)[8], bool row_on, int n_px)
+// Blocks that the frame's right edge cuts: the points of a set three at a time; n_px: how many of the lane's eight pixels lie inside.
+template <int PITCH>
+__device__ __forceinline__ void score_clipped(uint32_t set, uint32_t pc, uint32_t off, const uint32_t (&cw)[8], bool row_on, int n_px, int lane, uint32_t& mine)
 {
-    uint32_t acc[3] = {0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
+#pragma unroll 1
+    while (set) {                                                 // the same in all lanes
+        uint32_t p[3], acc[3] = {0, 0, 0}; int at[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            uint32_t w;
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(p[k] + 8u * j) : "memory");
-            const uint32_t d = j < n_px ? __vabsdiffu4(cw[j], w) : 0u;
-            acc[k] = __dp4a(d, d, acc[k]);
+            at[k] = set ? __ffs(set) - 1 : -1;                    // none left: the centre once more, kept by no lane
+            p[k] = pc + __shfl_sync(0xffffffffu, off, set ? at[k] : 8);
+            set &= set - 1;
         }
-    Edge3 r;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) r.s[k] = __reduce_add_sync(0xffffffffu, row_on ? acc[k] : 0u);
-    return r;
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const uint32_t w = lds_at<0>(p[k] + 8u * j), d = j < n_px ? __vabsdiffu4(cw[j], w) : 0u;
+                acc[k] = __dp4a(d, d, acc[k]);
+            }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t sum = __reduce_add_sync(0xffffffffu, row_on ? acc[k] : 0u);
+            mine = lane == at[k] ? sum : mine;
+        }
+    }
+}
+
+// This lane's point (lanes 0 to 12), from the centre.
+__device__ __forceinline__ int lane_point(int lane)
+{
+    // x + 2 and y + 2 of the points, three bits each
+    constexpr auto pack = [](bool y) { unsigned long long v = 0; for (int i = 0; i < 13; ++i) v |= (unsigned long long)((y ? point_y(i) : point_x(i)) + 2) << (3 * i); return v; };
+    constexpr unsigned long long X = pack(false), Y = pack(true);
+    const int i = lane < 13 ? lane : 8;
+    return pair((int)(X >> (3 * i) & 7) - 2, (int)(Y >> (3 * i) & 7) - 2);
+}
+// Shared-memory bytes from a candidate to the one displaced by a pair.
+template <int PITCH>
+__device__ __forceinline__ uint32_t bytes_of(int p)
+{
+    const int y = (p + 0x8000) >> 16;
+    return (uint32_t)(4 * p + y * (4 * PITCH - 4 * 65536));
 }
 
 //   lane_base  shared-memory address of this lane's first word of the candidate at displacement (0, 0);
 //              (dx, dy) is at lane_base + (dy * PITCH + dx) * 4
-//   reach(x, y)  true when every point around centre (x, y) is staged
-// Returns 1 when the walk has finished (result: w.cx, w.cy, w.bs), 2 when the next centre is out of reach.
-template <int PITCH, typename Reach>
+//   valid  displacements that keep the block inside the previous frame and the search range
+//   reach  centres around which every point is staged
+//   AHEAD  the loads of a whole round travel together
+// Returns 1 when the walk has finished (result: w.at, w.bs), 2 when the next centre is out of reach.
+template <int PITCH, bool AHEAD>
 __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base, const uint32_t (&cw)[8], bool row_on, int n_px, bool clipped,
-                                         const WalkBounds& wb, WalkW& w, const Reach& reach)
+                                         Within valid, WalkW& w, Within reach)
 {
-    static __constant__ int c_points[13] = DC_POINT_ROW(PITCH);
-    const int max_moves = (2 * a.R + 1) * (2 * a.R + 1);          // every move strictly lowers the key: never reached
-    // all 13 points valid  <=>  cx in [dx_lo + 2, dx_hi - 2] and cy likewise: one unsigned compare per axis
-    const int ix_lo = wb.dx_lo + 2, iy_lo = wb.dy_lo + 2;
-    const unsigned ix_span = (unsigned)max(wb.dx_hi - 2 - ix_lo, -1), iy_span = (unsigned)max(wb.dy_hi - 2 - iy_lo, -1);
-    const bool roomy = !clipped && wb.dx_hi - 2 >= ix_lo && wb.dy_hi - 2 >= iy_lo;
-    uint32_t pc = lane_base + (uint32_t)((w.cy * PITCH + w.cx) * 4);
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, point = lane_point(lane);
+    uint32_t pc = lane_base + bytes_of<PITCH>(w.at - disp(0, 0));
 #pragma unroll 1
-    for (int move = 0;; ++move) {
-        const bool interior = roomy && (unsigned)(w.cx - ix_lo) <= ix_span && (unsigned)(w.cy - iy_lo) <= iy_span;
-        uint32_t ms = 0xffffffffu; int mi = 8; bool tie = !interior;
-        if (interior) {
+    for (int moves_left = (2 * a.R + 1) * (2 * a.R + 1);; --moves_left) {      // every move strictly lowers the key: never used up
+        uint32_t mine = 0xffffffffu;
+        if (!clipped) {
             switch (w.kind) {
-            case 0: score_fixed_set<31u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 1: score_fixed_set<11u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 2: score_fixed_set<21u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 3: score_fixed_set<171u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 4: score_fixed_set<213u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 5: score_fixed_set<168u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 6: score_fixed_set<208u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case 7: score_fixed_set<248u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            case KIND_FIRST: score_fixed_set<0x1ffu, PITCH>(pc, cw, row_on, ms, mi, tie); break;
-            default: score_fixed_set<0x1e00u, PITCH>(pc, cw, row_on, ms, mi, tie); break;
+            case 0: score_set<kind_mask(0), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 1: score_set<kind_mask(1), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 2: score_set<kind_mask(2), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 3: score_set<kind_mask(3), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 4: score_set<kind_mask(4), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 5: score_set<kind_mask(5), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 6: score_set<kind_mask(6), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case 7: score_set<kind_mask(7), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            case KIND_FIRST: score_set<kind_mask(KIND_FIRST), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
+            default: score_set<kind_mask(KIND_SMALL), PITCH, AHEAD>(pc, cw, row_on, lane, mine); break;
             }
-            tie |= ms == w.bs;
-        }
-        int nx = w.cx, ny = w.cy;                                 // the best point after this round
-        uint32_t ns = w.bs;
-        if (!tie) {
-            if (ms < w.bs) { ns = ms; nx = w.cx + c_point_x[mi]; ny = w.cy + c_point_y[mi]; }
         } else {
-            // the exact order
-            uint32_t m = c_kind_mask[w.kind] & valid_points(w.cx, w.cy, wb);
-            uint32_t bt = w.kind == KIND_FIRST ? 0xffffffffu : tie_key(w.cx, w.cy);
-            const uint32_t kc = ((uint32_t)(w.cy + 128) << 8) | (uint32_t)(w.cx + 128);  // low half of the centre's tie key
-#pragma unroll 1
-            while (m) {                                           // three candidates per turn; m is the same in all lanes
-                int pw[3]; uint32_t p[3]; bool on[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    on[k] = m != 0;
-                    pw[k] = on[k] ? c_points[__ffs(m) - 1] : 0;   // none left: the centre once more, ignored
-                    p[k] = pc + (uint32_t)(pw[k] >> 16);
-                    m &= m - 1;
-                }
-                const Edge3 e = score3(p, cw, row_on, n_px);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const uint32_t s = e.s[k];
-                    if (!on[k] || s > ns) continue;
-                    const uint32_t lo = (kc + (uint32_t)pw[k]) & 0xffffu;            // ((dy + 128) << 8) | (dx + 128)
-                    const int dx = (int)(lo & 0xff) - 128, dy = (int)(lo >> 8) - 128;
-                    const uint32_t kt = ((uint32_t)(abs(dx) + abs(dy)) << 16) | lo;
-                    if (s < ns || kt < bt) { ns = s; bt = kt; nx = dx; ny = dy; }
-                }
-            }
+            score_clipped<PITCH>(c_kind_mask[w.kind], pc, bytes_of<PITCH>(point), cw, row_on, n_px, lane, mine);
         }
-        if (w.kind == KIND_SMALL) { w.cx = nx; w.cy = ny; w.bs = ns; return 1; }       // the small diamond's best is the result
-        if (nx == w.cx && ny == w.cy) { w.bs = ns; w.kind = KIND_SMALL; continue; }    // centre won: small diamond, then done
-        if (move >= max_moves) {                                  // a walk cut here is not valid: say so
-            if ((threadIdx.x & 31) == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
+        if (lane == 8 && w.kind != KIND_FIRST) mine = w.bs;       // the centre
+        const int d = w.at + point;
+        if (!within(d, valid)) mine = 0xffffffffu;
+        const uint32_t ns = __reduce_min_sync(all, mine);
+        unsigned best = __ballot_sync(all, mine == ns);
+        if (best & (best - 1)) {                                  // equal scores: the exact order among them
+            const uint32_t kt = tie_key(disp_x(d), disp_y(d)), kb = __reduce_min_sync(all, mine == ns ? kt : 0xffffffffu);
+            best = __ballot_sync(all, mine == ns && kt == kb);
+        }
+        const int g = __ffs(best) - 1;                            // the best point after this round
+        const int next = __shfl_sync(all, d, g);
+        if (w.kind == KIND_SMALL) { w.at = next; w.bs = ns; return 1; }                // the small diamond's best is the result
+        if (g == 8) { w.bs = ns; w.kind = KIND_SMALL; continue; }                      // centre won: small diamond, then done
+        if (moves_left <= 0) {                                    // a walk cut here is not valid: say so
+            if (lane == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
             w.bs = ns;
             return 1;
         }
-        if (!reach(nx, ny)) { w.nx = nx; w.ny = ny; w.ns = ns; return 2; }
-        const int mx = nx - w.cx, my = ny - w.cy;
-        w.kind = c_kind_of_move[((my + 2) * 5 + (mx + 2)) >> 1];
-        pc += (uint32_t)((my * PITCH + mx) * 4);
-        w.cx = nx; w.cy = ny; w.bs = ns;
+        if (!within(next, reach)) { w.next = next; w.nk = g; w.ns = ns; return 2; }
+        pc += bytes_of<PITCH>(next - w.at);
+        w.kind = g; w.at = next; w.bs = ns;
     }
 }
 // how many of a lane's pixels h, h + 2, ... of a block row of bw pixels exist
@@ -736,17 +767,19 @@ __device__ __forceinline__ int lane_pixel_count(int bw, int h) { return (bw - h 
 // and 12 pixels to its left and right (its left edge stays a multiple of 4 pixels, so that 4 pixels are 12 aligned
 // bytes of the packed frame).  A walk whose next centre is out of reach is handed to phase 2.  Launched without k-skip
 // only (every block is searched).
+// What bounds it: instruction issue (3.3 of 4 per clock and SM on 8 full-HD streams, 105 us; 126 while cut point sets and ties had a path
+// of their own), or, with few tiles, the longest walk: a round is a trip to shared memory and back.  Up to two tiles per SM the instance
+// with AHEAD runs, which has the loads of a whole round in flight (64 registers a thread): one stream of 227 x 227, 8.7 -> 5.5 us, with noise
+// in it and the walks of phase 2 28 -> 17.  (A whole pass, us, without and with it: VGG, two 640 x 360 streams 218 and 210; AlexNet, 18
+// streams, 142 and 140.)
 constexpr int W_VS = 2, W_WRY = 10, W_SIDE = 12;
 constexpr int W_COLS = 128 + 2 * W_SIDE;                    // staged pixels per window row
 constexpr int W_PITCH = 154;                                // words per window row
 constexpr int W_ROWS = 16 * W_VS + 2 * W_WRY;
 static_assert(W_PITCH % 4 == 2 && W_PITCH >= W_COLS && W_COLS % 4 == 0, "conflict-free pitch, whole groups of 4 pixels");
 
-struct TileReach {
-    __device__ __forceinline__ bool operator()(int cx, int cy) const { return abs(cx) + 2 <= W_SIDE && abs(cy) + 2 <= W_WRY; }
-};
-
-__global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, uint4* long_list, int32_t* long_count)
+template <bool AHEAD>
+__global__ void __launch_bounds__(W_VS * 8 * 32, AHEAD ? 2 : 3) k_search_dsw(MatchArgs a, uint4* long_list, int32_t* long_count)
 {
     dc_pdl_wait();
     dc_pdl_release();
@@ -756,7 +789,7 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
     __shared__ int32_t sums[3];
     const int strip = blockIdx.x, vg = blockIdx.y, s = blockIdx.z;        // grid: strips of 8 blocks x groups of W_VS block rows x streams
     const int xs = strip * 128, yb = vg * 16 * W_VS;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
     const int by = vg * W_VS + (warp >> 3), bx = strip * 8 + (warp & 7);
     const int x0 = bx * 16, y0 = by * 16;
     const bool searched = bx < a.Gx && by < a.Gy;
@@ -793,17 +826,19 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
         const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
         const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(win) +
                                    (uint32_t)((((warp >> 3) * 16 + r + W_WRY) * W_PITCH + (x0 - xs + W_SIDE) + h) * 4);
-        WalkW w = {0, 0, KIND_FIRST, 0xffffffffu, 0, 0, 0u};
-        const int st = warp_walk<W_PITCH>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, wb, w, TileReach());
+        WalkW w = {disp(0, 0), KIND_FIRST, 0xffffffffu, 0, 0, 0u};
+        const Within reach = {disp(2 - W_SIDE, 2 - W_WRY), disp(W_SIDE - 2, W_WRY - 2)};
+        const int st = warp_walk<W_PITCH, AHEAD>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, walk_range(wb), w, reach);
         if (lane == 0) {
             if (st == 1) {
-                a.mv[2 * g] = (int16_t)w.cx; a.mv[2 * g + 1] = (int16_t)w.cy; a.sse[g] = w.bs;
+                const int dx = disp_x(w.at), dy = disp_y(w.at);
+                a.mv[2 * g] = (int16_t)dx; a.mv[2 * g + 1] = (int16_t)dy; a.sse[g] = w.bs;
                 if (w.bs <= a.limit[limit_index(a, bw, bh)]) {        // PSNR > T: member of Step 3's set S
-                    atomicAdd(&sums[0], w.cx); atomicAdd(&sums[1], w.cy); atomicAdd(&sums[2], 1);
+                    atomicAdd(&sums[0], dx); atomicAdd(&sums[1], dy); atomicAdd(&sums[2], 1);
                 }
-            } else {                                                  // block, chosen next centre, its SSE, centre it was found from
+            } else {                                                  // block, chosen next centre, its SSE, the kind of that move
                 const int slot = atomicAdd(long_count, 1);
-                long_list[slot] = make_uint4((uint32_t)g, tie_key(w.nx, w.ny), w.ns, (uint32_t)(w.cx + 128) | ((uint32_t)(w.cy + 128) << 8));
+                long_list[slot] = make_uint4((uint32_t)g, (uint32_t)w.next, w.ns, (uint32_t)w.nk);
             }
         }
     }
@@ -820,12 +855,12 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, 3) k_search_dsw(MatchArgs a, ui
 // ---------------------------------------------------------------------------------------------
 // Layout of the diamond kernel: one word per pixel, lane 2 r + h scores every other pixel of block row r, no bank
 // conflicts.  The window reaches `side` pixels (2 S0 - 1, rounded up to four) to the left and right and wr = 2 S0 - 1
-// rows up and down, so every point of the search is staged.  A step scores its eight points in two batches of four,
-// 32 loads in flight each, and decides by SSE alone; when two of the scores that matter are equal the exact order
-// (SSE, |dx| + |dy|, dy, dx) picks from the same scores.
-// What bounds it: issue slots - 8 loads, 8 differences, 8 multiply-adds and a warp sum per point and block.  Measured
-// on 8 full-HD frames, range 16: 140 us with 4 lanes per block and byte-aligned rows (a bank conflict and a realignment
-// per word), 126 us so.
+// rows up and down, so every point of the search is staged.  A step scores its eight points row by row and decides by SSE alone; when
+// two of the scores that matter are equal the exact order (SSE, |dx| + |dy|, dy, dx) picks from the same scores.
+// What bounds it: issue slots - 8 differences, 8 multiply-adds and a warp sum per point and block, and the loads, which the points of a
+// row share where the step is 8 or less.  Measured on 8 full-HD frames, range 16: 140 us with 4 lanes per block and byte-aligned rows (a
+// bank conflict and a realignment per word), 126 with 8 loads per point and two CTAs per SM, 114 so.  AHEAD (up to a tile per SM): the
+// loads of a step travel together; two 640 x 360 streams 9.9 -> 5.8 us.
 constexpr int TSS_VS = 2;
 struct TssShape { int s0, wr, side, pitch; };
 static TssShape tss_shape(int R)
@@ -840,68 +875,93 @@ static TssShape tss_shape(int R)
 }
 static size_t tss_window_bytes(const TssShape& t) { return (size_t)(16 * TSS_VS + 2 * t.wr) * t.pitch * sizeof(uint32_t); }
 
-// SSE of N candidates over this lane's pixels, summed over the warp (n_px: the lane's pixels inside the frame)
-template <bool CLIP, int N>
-__device__ __forceinline__ void score_n(const uint32_t (&p)[N], const uint32_t (&cw)[8], bool row_on, int n_px, uint32_t* out)
+// The eight points of a step of compile-time length, row by row (the middle of the centre's row is the best point so far).
+template <int STEP, bool AHEAD, int Y = -1>
+__device__ __forceinline__ void tss_score(uint32_t pc, uint32_t row_bytes, const uint32_t (&cw)[8], bool row_on, int lane, uint32_t& mine)
 {
-    uint32_t w[N][8];
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        w[k][0] = lds_at<0>(p[k]); w[k][1] = lds_at<8>(p[k]); w[k][2] = lds_at<16>(p[k]); w[k][3] = lds_at<24>(p[k]);
-        w[k][4] = lds_at<32>(p[k]); w[k][5] = lds_at<40>(p[k]); w[k][6] = lds_at<48>(p[k]); w[k][7] = lds_at<56>(p[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-        uint32_t a0 = 0, a1 = 0;
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            uint32_t d = !CLIP || j < n_px ? __vabsdiffu4(cw[j], w[k][j]) : 0u; a0 = __dp4a(d, d, a0);
-            d = !CLIP || j + 1 < n_px ? __vabsdiffu4(cw[j + 1], w[k][j + 1]) : 0u; a1 = __dp4a(d, d, a1);
+    if constexpr (Y <= 1) {
+        const uint32_t p = pc + (uint32_t)Y * row_bytes;
+        constexpr int G = 3 * (Y + 1);
+        if constexpr (STEP == 1) {                                // an odd step: its sides are no whole words from its middle
+            RowWords<-1, 3ull> sides;
+            RowWords<0, 1ull> middle;
+            sides.load(p);
+            if constexpr (Y != 0) middle.load(p);
+            if constexpr (AHEAD) tss_score<STEP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, lane, mine);
+            sides.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == G + 2 * m ? v : mine; });
+            if constexpr (Y != 0) middle.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == G + 1 ? v : mine; });
+        } else {
+            constexpr unsigned long long DXS = 1ull | (Y != 0 ? 1ull << (STEP / 2) : 0ull) | 1ull << STEP;
+            RowWords<-STEP, DXS> row;
+            row.load(p);
+            if constexpr (AHEAD) tss_score<STEP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, lane, mine);
+            row.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == G + 2 * m / STEP ? v : mine; });
         }
-        out[k] = __reduce_add_sync(0xffffffffu, row_on ? a0 + a1 : 0u);
+        if constexpr (!AHEAD) tss_score<STEP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, lane, mine);
     }
 }
 
 // Lane g < 9 settles point g of the 3 x 3 grid (4: its centre, the best so far): its displacement, validity and tie key
 // are computed once per step and not point by point.
-template <bool CLIP>
+template <bool CLIP, bool AHEAD>
 __device__ __forceinline__ void tss_walk(uint32_t lane_base, int pitch, int s0, const uint32_t (&cw)[8], bool row_on, int n_px,
-                                         const WalkBounds& wb, int& cx, int& cy, uint32_t& bs)
+                                         Within valid, int& at, uint32_t& bs)
 {
-    const int lane = threadIdx.x & 31, gx = lane % 3 - 1, gy = lane / 3 - 1;
-    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4, centre = lane == 4;
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, point = pair(lane % 3 - 1, lane / 3 - 1);
     {   // the zero vector
-        const uint32_t p[1] = {lane_base};
-        score_n<CLIP, 1>(p, cw, row_on, n_px, &bs);
+        RowWords<0, 1ull> zero;
+        zero.load(lane_base);
+        zero.template score<CLIP>(cw, row_on, n_px, [&](int, uint32_t v) { bs = v; });
     }
-    cx = cy = 0;
+    at = disp(0, 0);
     uint32_t pc = lane_base;
 #pragma unroll 1
     for (int step = s0; step > 0; step >>= 1) {
-        const uint32_t ox = (uint32_t)step * 4u, oy = (uint32_t)(step * pitch) * 4u;
-        uint32_t sc[8];
-        const uint32_t up[4] = {pc - oy - ox, pc - oy, pc - oy + ox, pc - ox}, dn[4] = {pc + ox, pc + oy - ox, pc + oy, pc + oy + ox};
-        score_n<CLIP, 4>(up, cw, row_on, n_px, sc);
-        score_n<CLIP, 4>(dn, cw, row_on, n_px, sc + 4);
-        // sc[0..3]: points 0 to 3, sc[4..7]: points 5 to 8
-        const uint32_t q0 = b0 ? sc[1] : sc[0], q1 = b0 ? sc[3] : sc[2], q2 = b0 ? sc[4] : bs, q3 = b0 ? sc[6] : sc[5];
-        uint32_t mine = b2 ? (b1 ? q3 : q2) : (b1 ? q1 : q0);
-        if (lane == 8) mine = sc[7];
-        const int dx = cx + gx * step, dy = cy + gy * step;
-        if (lane > 8 || (!centre && (dx < wb.dx_lo || dx > wb.dx_hi || dy < wb.dy_lo || dy > wb.dy_hi))) mine = 0xffffffffu;
-        bs = __reduce_min_sync(0xffffffffu, mine);
-        unsigned best = __ballot_sync(0xffffffffu, mine == bs);
+        const uint32_t row_bytes = (uint32_t)(step * pitch) * 4u;
+        uint32_t mine = lane == 4 ? bs : 0xffffffffu;
+        if (!CLIP) {
+            switch (step) {
+            case 1: tss_score<1, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
+            case 2: tss_score<2, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
+            case 4: tss_score<4, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
+            case 8: tss_score<8, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
+            case 16: tss_score<16, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
+            default: tss_score<32, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
+            }
+        } else {
+            constexpr int BATCH = AHEAD ? 4 : 1;                  // blocks that the frame's right edge cuts
+#pragma unroll 1
+            for (int k0 = 0; k0 < 8; k0 += BATCH) {
+                RowWords<0, 1ull> one[BATCH];
+#pragma unroll
+                for (int k = 0; k < BATCH; ++k) {
+                    const int q = k0 + k + (k0 + k >= 4);
+                    one[k].load(pc + (uint32_t)(q / 3 - 1) * row_bytes + (uint32_t)((q % 3 - 1) * step * 4));
+                }
+#pragma unroll
+                for (int k = 0; k < BATCH; ++k) {
+                    const int q = k0 + k + (k0 + k >= 4);
+                    one[k].template score<true>(cw, row_on, n_px, [&](int, uint32_t v) { mine = lane == q ? v : mine; });
+                }
+            }
+        }
+        const int d = at + step * point;
+        if (!within(d, valid)) mine = 0xffffffffu;
+        bs = __reduce_min_sync(all, mine);
+        unsigned best = __ballot_sync(all, mine == bs);
         if (best & (best - 1)) {                                  // equal scores: the exact order among them
-            const uint32_t kt = tie_key(dx, dy), kb = __reduce_min_sync(0xffffffffu, mine == bs ? kt : 0xffffffffu);
-            best = __ballot_sync(0xffffffffu, mine == bs && kt == kb);
+            const uint32_t kt = tie_key(disp_x(d), disp_y(d)), kb = __reduce_min_sync(all, mine == bs ? kt : 0xffffffffu);
+            best = __ballot_sync(all, mine == bs && kt == kb);
         }
         const int g = __ffs(best) - 1, my = g / 3 - 1, mx = g - 3 * (my + 1) - 1;
-        cx += mx * step; cy += my * step;
+        at += step * pair(mx, my);
         pc += (uint32_t)((my * pitch + mx) * step * 4);
     }
 }
 
-__global__ void __launch_bounds__(TSS_VS * 8 * 32, 2) k_search_tss16(MatchArgs a, TssShape t)
+template <bool AHEAD>
+__global__ void __launch_bounds__(TSS_VS * 8 * 32, AHEAD ? 1 : 3) k_search_tss16(MatchArgs a, TssShape t)
 {
     dc_pdl_wait();
     dc_pdl_release();
@@ -910,7 +970,7 @@ __global__ void __launch_bounds__(TSS_VS * 8 * 32, 2) k_search_tss16(MatchArgs a
     constexpr int THREADS = TSS_VS * 8 * 32;
     const int strip = blockIdx.x, vg = blockIdx.y, s = blockIdx.z;
     const int xs = strip * 128, yb = vg * 16 * TSS_VS;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
     const int by = vg * TSS_VS + (warp >> 3), bx = strip * 8 + (warp & 7);
     const int x0 = bx * 16, y0 = by * 16;
     const bool searched = bx < a.Gx && by < a.Gy;
@@ -923,7 +983,7 @@ __global__ void __launch_bounds__(TSS_VS * 8 * 32, 2) k_search_tss16(MatchArgs a
     const uint8_t* prev = a.prev + (size_t)s * a.prev_stream;
     // groups of 4 pixels, five in flight per thread; a thread's next group is THREADS further: rows and columns by addition
     const int groups = (128 + 2 * t.side) / 4, rows = 16 * TSS_VS + 2 * t.wr, row_add = THREADS / groups, col_add = THREADS - row_add * groups;
-    constexpr int UNR = 5;
+    constexpr int UNR = AHEAD ? 5 : 3;
     for (int row = threadIdx.x / groups, gq = threadIdx.x - row * groups; row < rows;) {
         uint32_t pa[UNR], pb[UNR], pc[UNR];
         uint32_t* dst[UNR];
@@ -944,9 +1004,10 @@ __global__ void __launch_bounds__(TSS_VS * 8 * 32, 2) k_search_tss16(MatchArgs a
         const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
         const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(tss_win) +
                                    (uint32_t)((((warp >> 3) * 16 + r + t.wr) * t.pitch + (x0 - xs + t.side) + h) * 4);
-        int cx, cy; uint32_t bs;
-        if (bw == 16) tss_walk<false>(lane_base, t.pitch, t.s0, cw, row_on, 8, wb, cx, cy, bs);
-        else tss_walk<true>(lane_base, t.pitch, t.s0, cw, row_on, lane_pixel_count(bw, h), wb, cx, cy, bs);
+        int at; uint32_t bs;
+        if (bw == 16) tss_walk<false, AHEAD>(lane_base, t.pitch, t.s0, cw, row_on, 8, walk_range(wb), at, bs);
+        else tss_walk<true, AHEAD>(lane_base, t.pitch, t.s0, cw, row_on, lane_pixel_count(bw, h), walk_range(wb), at, bs);
+        const int cx = disp_x(at), cy = disp_y(at);
         if (lane == 0) {
             a.mv[2 * g] = (int16_t)cx; a.mv[2 * g + 1] = (int16_t)cy; a.sse[g] = bs;
             if (bs <= a.limit[limit_index(a, bw, bh)]) {          // PSNR > T: member of Step 3's set S
@@ -974,8 +1035,8 @@ __global__ void k_mark_unsearched(MatchArgs a)
 }
 
 // Phase 2: the walks that left their tile's window.  A warp takes walks off the list one after the other (atomic
-// cursor); the walk gets a private window of P_ROWS x P_COLS pixels around its centre, re-staged around the next
-// centre whenever that is out of reach.  A continued walk makes exactly the move it had chosen (new points only),
+// cursor); the walk gets a private window of P_ROWS x P_COLS pixels, re-staged whenever the next centre is out of reach, its middle two
+// moves ahead of the centre in the walk's direction.  A continued walk makes exactly the move it had chosen (new points only),
 // so the sequence of scored candidates is the uninterrupted walk's.
 // With k-skip (Section 4) the searched blocks lie k blocks apart and share no window: there is no phase 1 then,
 // and this kernel walks every searched block from its start (long_list == nullptr; item i is the
@@ -983,14 +1044,11 @@ __global__ void k_mark_unsearched(MatchArgs a)
 constexpr int P_WARPS = 8;
 constexpr int P_REACH = 8;                                  // staged pixels above and left of the block at the window's centre
 constexpr int P_ROWS = 16 + 2 * P_REACH, P_COLS = 36, P_PITCH = 38;
+// Four CTAs per SM: 8 full-HD streams 58 us, 74 with five, whose registers spill.
 static_assert(P_PITCH % 4 == 2 && P_PITCH >= P_COLS && P_COLS % 4 == 0 && P_COLS >= 16 + 2 * P_REACH + 3, "window of a walk");
 
-struct PrivateReach {
-    int wcx, wcy;
-    __device__ __forceinline__ bool operator()(int cx, int cy) const { return abs(cx - wcx) + 2 <= P_REACH && abs(cy - wcy) + 2 <= P_REACH; }
-};
-
-__global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a, const uint4* long_list, const int32_t* long_count, int32_t* cursor)
+template <bool AHEAD>
+__global__ void __launch_bounds__(P_WARPS * 32, AHEAD ? 2 : 4) k_search_dsw_long(MatchArgs a, const uint4* long_list, const int32_t* long_count, int32_t* cursor)
 {
     dc_pdl_wait();
     dc_pdl_release();
@@ -1009,16 +1067,15 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
         idx = __shfl_sync(0xffffffffu, idx, 0);
         if (idx >= n) break;
         size_t g;
-        WalkW w = {0, 0, KIND_FIRST, 0xffffffffu, 0, 0, 0u};
+        WalkW w = {disp(0, 0), KIND_FIRST, 0xffffffffu, 0, 0, 0u};
         if (direct) {
             const int ss = idx / (sgx * sgy), q = idx - ss * sgx * sgy, sby = q / sgx, sbx = q - sby * sgx;
             g = (size_t)ss * per + (size_t)(sby * a.skip_k) * a.Gx + sbx * a.skip_k;
         } else {
             const uint4 e = long_list[idx];
             g = e.x; w.bs = e.z;
-            const int ox = (int)(e.w & 0xff) - 128, oy = (int)((e.w >> 8) & 0xff) - 128;      // the centre the walk stopped at
-            w.cx = (int)(e.y & 0xff) - 128; w.cy = (int)((e.y >> 8) & 0xff) - 128;            // the move it had chosen: make it
-            w.kind = c_kind_of_move[((w.cy - oy + 2) * 5 + (w.cx - ox + 2)) >> 1];
+            w.at = (int)e.y;                                                                  // the move it had chosen: make it
+            w.kind = (int)e.w;
         }
         const int s = (int)(g / per), b = (int)(g - (size_t)s * per), by = b / a.Gx, bx = b - by * a.Gx;
         const int x0 = bx * 16, y0 = by * 16, bh = min(16, a.H - y0), bw = min(16, a.W - x0);
@@ -1026,12 +1083,14 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
         uint32_t cw[8];
         load_lane_pixels(a.cur + (size_t)s * a.cur_stream + (size_t)(row_on ? y0 + r : y0) * a.cur_pitch + (size_t)x0 * 3, h, row_on, cw);
         const uint8_t* prev = a.prev + (size_t)s * a.prev_stream;
-        const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
+        const Within valid = walk_range(walk_bounds(a, x0, y0, bw, bh));
 #pragma unroll 1
         for (int round = 0;; ++round) {
-            // the window around the centre that is scored next
-            const PrivateReach reach = {w.cx, w.cy};
-            const int wx0 = (x0 + w.cx - P_REACH) & ~3, wy0 = y0 + w.cy - P_REACH;
+            // the window for the centre that is scored next
+            constexpr int AROUND = P_REACH - 2;
+            const int centre = w.at + 2 * lane_point(w.kind);
+            const Within reach = {centre - pair(AROUND, AROUND), centre + pair(AROUND, AROUND)};
+            const int wx0 = (x0 + disp_x(centre) - P_REACH) & ~3, wy0 = y0 + disp_y(centre) - P_REACH;
             {   // a lane keeps its group of 4 pixels (one column position) and goes down the rows, 3 rows apart
                 constexpr int GROUPS = P_COLS / 4, RPP = 32 / GROUPS, PASSES = (P_ROWS + RPP - 1) / RPP, HALF = (PASSES + 1) / 2;
                 const int gq = lane % GROUPS, row0 = lane / GROUPS, px0 = wx0 + 4 * gq;
@@ -1061,18 +1120,18 @@ __global__ void __launch_bounds__(P_WARPS * 32, 5) k_search_dsw_long(MatchArgs a
             // this lane's first word at displacement (0, 0): frame row y0 + r, pixel x0 + h, relative to the window's
             // origin (it may lie outside the window; only displacements near the centre are ever addressed)
             const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)(((r + y0 - wy0) * P_PITCH + (x0 - wx0) + h) * 4);
-            const int st = warp_walk<P_PITCH>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, wb, w, reach);
+            const int st = warp_walk<P_PITCH, AHEAD>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, valid, w, reach);
             if (st == 1) break;
             if (round >= max_rounds) {                                   // never reached; a walk cut here is not valid
                 if (lane == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
                 break;
             }
             // make the chosen move; the next round scores its new points in a window around the new centre
-            w.kind = c_kind_of_move[((w.ny - w.cy + 2) * 5 + (w.nx - w.cx + 2)) >> 1];
-            w.cx = w.nx; w.cy = w.ny; w.bs = w.ns;
+            w.kind = w.nk;
+            w.at = w.next; w.bs = w.ns;
             __syncwarp();                                                // every lane has finished reading the old window
         }
-        if (lane == 0) publish_block(a, s, g, bw, bh, ((unsigned long long)w.bs << 32) | tie_key(w.cx, w.cy));
+        if (lane == 0) publish_block(a, s, g, bw, bh, ((unsigned long long)w.bs << 32) | tie_key(disp_x(w.at), disp_y(w.at)));
     }
 }
 
@@ -1442,26 +1501,32 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
     // Step 3 sums and, behind them, the counter of walks handed to the second search phase: zeroed by the frame copy
     int32_t* long_count = c->mv_acc + 4 * c->S;
     // walks that phase 2 may get: no more warps than blocks
-    const dim3 long_grid((unsigned)min(c->num_sms * 5, dc_div_up(a.S * a.Gx * a.Gy, P_WARPS)));
+    const dim3 long_grid((unsigned)min(c->num_sms * 4, dc_div_up(a.S * a.Gx * a.Gy, P_WARPS)));
     if (a.B == 16 && a.search == DC_SEARCH_DIAMOND) {
         {
             dc_prof_scope ps(c, DC_ST_SEARCH);
+            const bool few = (long long)((a.Gx + 7) / 8) * ((a.Gy + W_VS - 1) / W_VS) * a.S <= 2 * c->num_sms;
             if (a.skip_k <= 1) {
                 const dim3 tiles((a.Gx + 7) / 8, (a.Gy + W_VS - 1) / W_VS, a.S);
-                DC_CUDA(dc_launch_pdl(k_search_dsw, tiles, W_VS * 8 * 32, 0, c->stream, a, c->long_list, long_count));
-                DC_CUDA(dc_launch_pdl(k_search_dsw_long, long_grid, P_WARPS * 32, 0, c->stream, a, (const uint4*)c->long_list, (const int32_t*)long_count, long_count + 1));
+                DC_CUDA(dc_launch_pdl(few ? k_search_dsw<true> : k_search_dsw<false>, tiles, W_VS * 8 * 32, 0, c->stream, a, c->long_list, long_count));
+                DC_CUDA(dc_launch_pdl(few ? k_search_dsw_long<true> : k_search_dsw_long<false>, long_grid, P_WARPS * 32, 0, c->stream, a, (const uint4*)c->long_list, (const int32_t*)long_count, long_count + 1));
             } else {
                 DC_CUDA(dc_launch_pdl(k_mark_unsearched, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, 256)), 256, 0, c->stream, a));
-                DC_CUDA(dc_launch_pdl(k_search_dsw_long, long_grid, P_WARPS * 32, 0, c->stream, a, (const uint4*)nullptr, (const int32_t*)long_count, long_count + 1));
+                DC_CUDA(dc_launch_pdl(few ? k_search_dsw_long<true> : k_search_dsw_long<false>, long_grid, P_WARPS * 32, 0, c->stream, a, (const uint4*)nullptr, (const int32_t*)long_count, long_count + 1));
             }
             c->launches += 1;
         }
     } else if (a.B == 16 && a.search == DC_SEARCH_THREE_STEP && a.skip_k <= 1) {
         const TssShape t = tss_shape(a.R);
         static dc_once_per_device attr_set;
-        if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_search_tss16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tss_window_bytes(tss_shape(64))));
+        if (attr_set.first(c->device)) {
+            const int most = (int)tss_window_bytes(tss_shape(64));
+            DC_CUDA(cudaFuncSetAttribute(k_search_tss16<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+            DC_CUDA(cudaFuncSetAttribute(k_search_tss16<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        }
         dc_prof_scope ps(c, DC_ST_SEARCH);
-        DC_CUDA(dc_launch_pdl(k_search_tss16, dim3((unsigned)((a.Gx + 7) / 8), (unsigned)((a.Gy + TSS_VS - 1) / TSS_VS), (unsigned)a.S), TSS_VS * 8 * 32,
+        const dim3 tiles((unsigned)((a.Gx + 7) / 8), (unsigned)((a.Gy + TSS_VS - 1) / TSS_VS), (unsigned)a.S);
+        DC_CUDA(dc_launch_pdl((long long)tiles.x * tiles.y * tiles.z <= c->num_sms ? k_search_tss16<true> : k_search_tss16<false>, tiles, TSS_VS * 8 * 32,
                               tss_window_bytes(t), c->stream, a, t));
     } else if (a.B == 16 && a.search == DC_SEARCH_EXHAUSTIVE && a.R <= E_MAXR && a.W >= 16 && a.H >= 16) {
         const int chunks = (2 * a.R + 1 + E_DY - 1) / E_DY;

@@ -210,6 +210,33 @@ def test_match_three_step_16_windows(R, shape):
     check_pairs([(prev, far), (const, const), (smooth, np.roll(smooth, 2, axis=1)), (prev, smooth)], 16, R, B.DC_SEARCH_THREE_STEP)
 
 
+@pytest.mark.parametrize("search,R", [(B.DC_SEARCH_DIAMOND, 1), (B.DC_SEARCH_DIAMOND, 5), (B.DC_SEARCH_DIAMOND, 40), (B.DC_SEARCH_THREE_STEP, 3), (B.DC_SEARCH_THREE_STEP, 31)])
+def test_match_16_many_tiles(search, R):
+    """Enough tiles for the search's instance of many warps per SM, with what its rounds meet at the edges: strips and blocks cut on either
+    side, range limits next to the start, equal scores, walks that leave the staged window."""
+    g = rng(R)
+    H, W = 70, 147
+    x, y = np.meshgrid(np.arange(W), np.arange(H))
+    pairs = []
+    for i in range(60):
+        kind = i % 4
+        if kind == 0:                                              # smooth: long walks along a slope
+            base = np.stack([np.hypot(x - W * g.random(), y - H * g.random()) * g.uniform(0.5, 1.5) for _ in range(3)], -1)
+            prev = base.astype(np.int64).astype(np.uint8)
+            cur = np.roll(prev, (int(g.integers(-9, 10)), int(g.integers(-20, 21))), axis=(0, 1))
+        elif kind == 1:                                            # few levels: many equal scores
+            prev = (g.integers(0, 2, (H, W, 3)) * 90).astype(np.uint8)
+            cur = np.roll(prev, (1, -2), axis=(0, 1))
+        elif kind == 2:
+            prev = np.repeat(np.repeat(((x // 4) % 3 * 40).astype(np.uint8)[..., None], 3, 2), 1, 0)
+            cur = np.roll(prev, 2, axis=1)
+        else:
+            prev = g.integers(0, 256, (H, W, 3), dtype=np.uint8)
+            cur = np.roll(prev, (-2, 2), axis=(0, 1))
+        pairs.append((prev, cur))
+    check_pairs(pairs, 16, R, search)
+
+
 @pytest.mark.parametrize("h,w,k,st,p", [(33, 41, 3, 2, 1), (32, 32, 7, 2, 3), (47, 35, 5, 3, 2), (30, 31, 7, 3, 0), (39, 227, 11, 4, 0), (41, 43, 11, 4, 5)])
 def test_frame_into_block_map(h, w, k, st, p):
     """A frame goes straight into a strided first layer's block map: blocks of 2, 3 and 4, padding on every side, rows that
