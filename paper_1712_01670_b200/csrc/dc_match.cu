@@ -16,11 +16,10 @@
 //              spans are identical, emitted in (y, x) order by a CTA-wide ordered compaction.
 #include "dc_common.cuh"
 #include "dc_search_win.cuh"
+#include "dc_walk.cuh"
 
 namespace {
 
-constexpr int WARPS = 8;
-constexpr int MAX_ROW_WORDS = 24;       // block <= 32 px -> 96 bytes per row
 
 struct MatchArgs {
     const uint8_t* cur;  size_t cur_pitch;  size_t cur_stream;
@@ -36,91 +35,6 @@ __device__ __forceinline__ unsigned long long cand_key(uint32_t sse, int dx, int
     // lexicographic (SSE, |dx|+|dy|, dy, dx) packed into one integer
     return ((unsigned long long)sse << 32) | ((unsigned long long)(abs(dx) + abs(dy)) << 16) |
            ((unsigned long long)(dy + 128) << 8) | (unsigned long long)(dx + 128);
-}
-
-template <int ITERS>
-struct BlockCtx {
-    const uint32_t* cur_sm;     // this warp's copy of the current block, row stride MAX_ROW_WORDS
-    const uint8_t* prev;        // previous frame of this stream
-    size_t prev_pitch;
-    int W, H, R, x0, y0, bw, bh, lane;
-    int off[ITERS];             // per lane item: byte offset of (row, word) inside a candidate
-    int smi[ITERS];             // index into cur_sm, -1 = no item
-    uint32_t msk[ITERS];        // valid bytes of the word
-
-    __device__ __forceinline__ void setup()
-    {
-        const int row_bytes = bw * 3, wpr = (row_bytes + 3) >> 2, items = bh * wpr;
-#pragma unroll
-        for (int it = 0; it < ITERS; ++it) {
-            int item = it * 32 + lane;
-            if (item < items) {
-                int row = item / wpr, wi = item - row * wpr;
-                int nb = row_bytes - wi * 4;
-                off[it] = row * (int)prev_pitch + wi * 4;
-                smi[it] = row * MAX_ROW_WORDS + wi;
-                msk[it] = nb >= 4 ? 0xffffffffu : ((1u << (nb * 8)) - 1u);
-            } else { off[it] = 0; smi[it] = -1; msk[it] = 0; }
-        }
-    }
-    __device__ __forceinline__ bool valid(int dx, int dy) const
-    {
-        return abs(dx) <= R && abs(dy) <= R && x0 + dx >= 0 && y0 + dy >= 0 &&
-               x0 + dx + bw <= W && y0 + dy + bh <= H;
-    }
-    // SSE of the block against the previous frame displaced by (dx, dy); same value in all lanes
-    __device__ __forceinline__ uint32_t sse(int dx, int dy) const
-    {
-        const uint8_t* base = prev + (size_t)(y0 + dy) * prev_pitch + (size_t)(x0 + dx) * 3;
-        uint32_t acc = 0;
-#pragma unroll
-        for (int it = 0; it < ITERS; ++it) {
-            if (smi[it] >= 0) {
-                const uint8_t* p = base + off[it];
-                uintptr_t a = (uintptr_t)p;
-                const uint32_t* q = (const uint32_t*)(a & ~(uintptr_t)3);
-                uint32_t sh = ((uint32_t)a & 3u) * 8u;
-                uint32_t lo = dc_ld(q), hi = dc_ld(q + 1);
-                uint32_t pv = __funnelshift_r(lo, hi, sh) & msk[it];
-                uint32_t d = __vabsdiffu4(cur_sm[smi[it]], pv);
-                acc = __dp4a(d, d, acc);
-            }
-        }
-        return __reduce_add_sync(0xffffffffu, acc);
-    }
-};
-
-template <int ITERS>
-__device__ __forceinline__ bool load_block(const MatchArgs& a, uint32_t* sm, BlockCtx<ITERS>& c, int& s, int& b)
-{
-    int warp = blockIdx.x * WARPS + (threadIdx.x >> 5);
-    int per = a.Gx * a.Gy;
-    if (warp >= per * a.S) return false;
-    s = warp / per; b = warp - s * per;
-    int by = b / a.Gx, bx = b - by * a.Gx;
-    c.lane = threadIdx.x & 31;
-    c.x0 = bx * a.B; c.y0 = by * a.B;
-    c.bw = min(a.B, a.W - c.x0); c.bh = min(a.B, a.H - c.y0);
-    c.W = a.W; c.H = a.H; c.R = a.R;
-    c.prev = a.prev + (size_t)s * a.prev_stream; c.prev_pitch = a.prev_pitch;
-    c.cur_sm = sm;
-    c.setup();
-    // the current block: byte loads (the caller's frame has no alignment or padding promise)
-    const uint8_t* cur = a.cur + (size_t)s * a.cur_stream + (size_t)c.y0 * a.cur_pitch + (size_t)c.x0 * 3;
-    const int row_bytes = c.bw * 3;
-#pragma unroll
-    for (int it = 0; it < ITERS; ++it) {
-        if (c.smi[it] >= 0) {
-            int row = c.smi[it] / MAX_ROW_WORDS, wi = c.smi[it] - row * MAX_ROW_WORDS;
-            const uint8_t* p = cur + (size_t)row * a.cur_pitch + wi * 4;
-            uint32_t v = 0;
-            for (int k = 0; k < 4; ++k)
-                if (wi * 4 + k < row_bytes) v |= (uint32_t)dc_ld(p + k) << (8 * k);
-            sm[c.smi[it]] = v;
-        }
-    }
-    __syncwarp();
-    return true;
 }
 
 __device__ __forceinline__ int limit_index(const MatchArgs& a, int bw, int bh)
@@ -158,30 +72,98 @@ __global__ void k_accept_own(MatchArgs a)
     }
 }
 
-template <int ITERS>
-__global__ void __launch_bounds__(WARPS * 32) k_verify(MatchArgs a)
+struct Step4 { int Mx, My, K; bool settled; int ok; };
+// The global motion of stream s, and block b (number gi in all) where no pixels are needed to settle it.
+__device__ __forceinline__ Step4 settle(const MatchArgs& a, int B, unsigned gi, int s, int b, bool in_grid)
+{
+    const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * B, y0 = by * B, bw = min(B, a.W - x0), bh = min(B, a.H - y0);
+    const int4 sums = __ldcg((const int4*)a.acc + s);                            // Step 3: sum dx, sum dy, K (one 16-byte load)
+    Step4 r = {0, 0, sums.z, false, 0};
+    if (r.K > 0) { r.Mx = round_mean(sums.x, r.K); r.My = round_mean(sums.y, r.K); }
+    const bool cand_ok = in_grid && r.K > 0 && abs(r.Mx) <= a.R && abs(r.My) <= a.R && x0 + r.Mx >= 0 && y0 + r.My >= 0 &&
+                         x0 + r.Mx + bw <= a.W && y0 + r.My + bh <= a.H;
+    bool known = false; uint32_t v = 0;
+    if (cand_ok) {
+        const uint32_t own = ((const uint32_t*)a.mv)[gi];                         // (dx, dy) as one word
+        v = a.sse[gi];
+        known = (int16_t)(own & 0xffffu) == r.Mx && (int16_t)(own >> 16) == r.My && v != 0xffffffffu;
+    }
+    r.settled = in_grid && (!cand_ok || known);
+    r.ok = known && v <= a.limit[limit_index(a, bw, bh)];
+    return r;
+}
+// The SSE of row r of block b displaced by (Mx, My), for any block size: the aligned words that hold the row in the new frame, the previous
+// frame's bytes shifted to their places, five words in flight.
+__device__ __forceinline__ uint32_t row_sse(const MatchArgs& a, int s, int b, int Mx, int My, int r, bool on)
+{
+    const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * a.B, y0 = by * a.B, bw = min(a.B, a.W - x0), bh = min(a.B, a.H - y0);
+    if (!on || r >= bh) return 0;
+    const uint8_t* c = a.cur + (size_t)s * a.cur_stream + (size_t)(y0 + r) * a.cur_pitch + (size_t)x0 * 3;
+    const int skip = (int)((uintptr_t)c & 3u), words = (skip + bw * 3 + 3) >> 2, tail = skip + bw * 3 - 4 * (words - 1);   // 1 to 4 bytes of the last word
+    const uint8_t* p = a.prev + (size_t)s * a.prev_stream + (size_t)(y0 + My + r) * a.prev_pitch + (size_t)(x0 + Mx) * 3 - skip;
+    const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u;
+    const uint32_t* cq = (const uint32_t*)(c - skip);
+    const uint32_t* pq = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
+    uint32_t acc = 0, lo = (const uint8_t*)pq >= a.prev ? dc_ld(pq) : 0u;        // bytes before the row are masked; none lie before the buffer
+    for (int j0 = 0; j0 < words; j0 += 5) {
+        uint32_t cw[5], hi[5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j) { const bool in = j0 + j < words; cw[j] = in ? dc_ld(cq + j0 + j) : 0u; hi[j] = in ? dc_ld(pq + j0 + j + 1) : 0u; }
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            uint32_t m = j0 + j < words ? 0xffffffffu : 0u;
+            if (j0 + j == words - 1) m >>= 8 * (4 - tail);
+            if (j0 + j == 0) m &= 0xffffffffu << (8 * skip);
+            const uint32_t d = __vabsdiffu4(cw[j], __funnelshift_r(lo, hi[j], sh)) & m;
+            acc = __dp4a(d, d, acc);
+            lo = hi[j];
+        }
+    }
+    return acc;
+}
+
+// Steps 3-4 for any block size (16-pixel blocks have kernels of their own).  A warp takes `share` blocks: a lane settles one from its own
+// vector where that is M, or where M leaves the frame or the range, then LPB lanes, one per row, score each of the others.
+// What bounds it: the latency of a row's loads; so few blocks per warp, two where the frame has few.  720p, 4 streams, 10-pixel blocks:
+// 29 us with a warp per block that fetched every block byte by byte, 12.5 so.
+template <int LPB>
+__global__ void __launch_bounds__(256) k_verify(MatchArgs a, int share)
 {
     dc_pdl_wait();
     dc_pdl_release();
-    __shared__ uint32_t sm_all[WARPS][32 * MAX_ROW_WORDS];
-    BlockCtx<ITERS> c; int s, b;
-    if (!load_block<ITERS>(a, sm_all[threadIdx.x >> 5], c, s, b)) return;
-    int K = a.acc[4 * s + 2];
-    int Mx = 0, My = 0;
-    if (K > 0) { Mx = round_mean(a.acc[4 * s + 0], K); My = round_mean(a.acc[4 * s + 1], K); }
-    int ok = 0;
-    if (K > 0 && c.valid(Mx, My)) {
-        const size_t g = (size_t)s * a.Gx * a.Gy + b;
-        // Section 4's second acceleration: a score that Step 2 already computed for the pair (block, block + M)
-        // is taken over instead of being recomputed -- exact when the block's best vector is M itself
-        uint32_t v = (a.mv[2 * g] == Mx && a.mv[2 * g + 1] == My && a.sse[g] != 0xffffffffu) ? a.sse[g] : c.sse(Mx, My);
-        ok = v <= a.limit[limit_index(a, c.bw, c.bh)];
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31, r = lane % LPB, half = lane / LPB, per = a.Gx * a.Gy;
+    const unsigned gi = (blockIdx.x * 8u + (threadIdx.x >> 5)) * (unsigned)share + (unsigned)lane;
+    const bool in_grid = lane < share && gi < (unsigned)(per * a.S);
+    const int s = in_grid ? (int)(gi / (unsigned)per) : a.S - 1, b = in_grid ? (int)(gi - (unsigned)s * per) : 0;
+    const Step4 v = settle(a, a.B, gi, s, b, in_grid);
+    int ok = v.ok;
+    if (in_grid && b == 0) { a.gmv[3 * s] = v.Mx; a.gmv[3 * s + 1] = v.My; a.gmv[3 * s + 2] = v.K; }
+    unsigned todo = __ballot_sync(all, in_grid && !v.settled);
+    while (todo) {                                                               // the same in all lanes
+        int i = __ffs(todo) - 1; bool on = true;
+        todo &= todo - 1;
+        const int mine = i;
+        int second = -1;
+        if (LPB == 16) {
+            if (todo) { second = __ffs(todo) - 1; todo &= todo - 1; }
+            if (half) { on = second >= 0; i = on ? second : i; }
+        }
+        const int Mx = __shfl_sync(all, v.Mx, i), My = __shfl_sync(all, v.My, i), si = __shfl_sync(all, s, i), bi = __shfl_sync(all, b, i);
+        uint32_t sse = row_sse(a, si, bi, Mx, My, r, on);
+#pragma unroll
+        for (int o = LPB / 2; o > 0; o >>= 1) sse += __shfl_xor_sync(all, sse, o);
+        const uint32_t other = LPB == 16 ? __shfl_xor_sync(all, sse, 16) : 0u;   // every lane knows both halves' sums
+        const uint32_t first_sse = half ? other : sse, second_sse = half ? sse : other;
+        if (lane == mine || lane == second) {
+            const int by = b / a.Gx, bx = b - by * a.Gx;
+            ok = (lane == mine ? first_sse : second_sse) <= a.limit[limit_index(a, min(a.B, a.W - bx * a.B), min(a.B, a.H - by * a.B))];
+        }
     }
-    if (c.lane == 0) {
-        a.matched[(size_t)s * a.Gx * a.Gy + b] = (uint8_t)ok;
-        if (ok) atomicAdd(&a.acc[4 * s + 3], 1);
-        if (b == 0) { a.gmv[3 * s] = Mx; a.gmv[3 * s + 1] = My; a.gmv[3 * s + 2] = K; }
-    }
+    if (in_grid) a.matched[gi] = (uint8_t)ok;
+    // matched count: one atomic per warp and stream
+    const unsigned same = __match_any_sync(all, s), oks = __ballot_sync(all, in_grid && ok);
+    if (lane == __ffs(same) - 1 && (oks & same)) atomicAdd(&a.acc[4 * s + 3], __popc(oks & same));
 }
 
 // Step 5: maximal horizontal runs of matched blocks per block row; a run continues the rectangle above it only when the
@@ -474,18 +456,6 @@ __device__ __forceinline__ void publish_block(const MatchArgs& a, int s, size_t 
 // different banks for every displacement (bank = r p + h + const, and r p / 2 runs through all residues mod 16),
 // so shared memory is read without conflicts, and all lanes of a warp follow the same walk, so no lane waits for
 // another block.  The points of the two diamonds sit at compile-time offsets from the centre's address.
-//
-// Points: 0-7 the large diamond, 8 its centre, 9-12 the small diamond.
-__host__ __device__ constexpr int point_x(int i)
-{
-    constexpr int t[13] = {0, -1, 1, -2, 2, -1, 1, 0, 0, 0, -1, 1, 0};
-    return t[i];
-}
-__host__ __device__ constexpr int point_y(int i)
-{
-    constexpr int t[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1};
-    return t[i];
-}
 // displacements that keep the block inside the previous frame and the search range
 struct WalkBounds { int dx_lo, dx_hi, dy_lo, dy_hi; };
 
@@ -494,11 +464,6 @@ __device__ __forceinline__ WalkBounds walk_bounds(const MatchArgs& a, int x0, in
     WalkBounds b = {max(-a.R, -x0), min(a.R, a.W - bw - x0), max(-a.R, -y0), min(a.R, a.H - bh - y0)};
     return b;
 }
-__device__ __forceinline__ uint32_t tie_key(int dx, int dy)
-{
-    return ((uint32_t)(abs(dx) + abs(dy)) << 16) | ((uint32_t)(dy + 128) << 8) | (uint32_t)(dx + 128);
-}
-
 // The 8 pixels of row r (48 bytes at `row`, 16-byte aligned) that lane parity h scores, one word each.
 __device__ __forceinline__ void load_lane_pixels(const uint8_t* row, int h, bool on, uint32_t (&cw)[8])
 {
@@ -537,15 +502,6 @@ __device__ __forceinline__ void load_pixels4(const uint8_t* prev, size_t pitch, 
     }
 }
 
-// SSE of this lane's 8 pixels against the candidate whose first word for this lane is at shared-memory address p,
-// summed over the warp.  Explicit shared-space loads at fixed offsets from one address register.
-template <int OFF>
-__device__ __forceinline__ uint32_t lds_at(uint32_t p)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(p), "n"(OFF) : "memory");
-    return v;
-}
 // Candidates of one window row, at compile-time displacements LO + 2 m for the set bits m of DXS: they are shifted by whole words against
 // one another, so a word is loaded once for all of them.  p: the address of displacement 0 in that row; n_px: how many of the lane's pixels
 // lie inside the frame.  sum(m, value) takes the scores.
@@ -627,31 +583,10 @@ __device__ __forceinline__ void score_set(uint32_t pc, const uint32_t (&cw)[8], 
 
 // One block's walk, by one warp, for as long as it stays inside the staged window.
 //
-// A round scores one of ten point sets around the current centre: kind 0-7, the points of the large diamond that are
-// new after the move along diamond point `kind` (the others lost to the new centre already and cannot win); kind 8,
-// the first round (centre and all eight points); kind 9, the small diamond.  Outside the first round the centre is
-// the best point so far and bs its SSE.  Every point around the centre is staged, so the round runs as straight-line code for
-// its set whatever the frame's edge and the range allow; lane i then drops point i where it is no valid candidate, and the smallest score
-// wins, or the smallest (|dx| + |dy|, dy, dx) among equal ones.  (With a separate path for cut sets and ties, point by point, the walks
-// at the edges set the time of a small frame.)
-constexpr int KIND_FIRST = 8, KIND_SMALL = 9;
-__host__ __device__ constexpr uint32_t kind_mask(int kind)
-{
-    constexpr uint32_t t[10] = {31u, 11u, 21u, 171u, 213u, 168u, 208u, 248u, 0x1ffu, 0x1e00u};
-    return t[kind];
-}
-__constant__ uint32_t c_kind_mask[10] = {31u, 11u, 21u, 171u, 213u, 168u, 208u, 248u, 0x1ffu, 0x1e00u};
-
-// Displacements in a walk are pairs of 16-bit numbers in one register, dy + kBias above dx + kBias: both axes are compared at once, and
-// a lane's registers are what bounds the warps per SM.
-constexpr int kBias = 128;
-__host__ __device__ constexpr int pair(int dx, int dy) { return dy * 65536 + dx; }                 // a difference of displacements
-__host__ __device__ constexpr int disp(int dx, int dy) { return pair(dx + kBias, dy + kBias); }
-__device__ __forceinline__ int disp_x(int d) { return (d & 0xffff) - kBias; }
-__device__ __forceinline__ int disp_y(int d) { return (d >> 16) - kBias; }
-struct Within { int lo, hi; };                                                                     // a range of displacements
-__device__ __forceinline__ bool within(int d, Within r) { return (int)__vminu2(__vmaxu2((unsigned)d, (unsigned)r.lo), (unsigned)r.hi) == d; }
-
+// Outside the first round the centre is the best point so far and bs its SSE.  Every point around the centre is staged, so a round runs as
+// straight-line code for its set whatever the frame's edge and the range allow; lane i then drops point i where it is no valid candidate, and
+// the smallest score wins, or the smallest (|dx| + |dy|, dy, dx) among equal ones.  (With a path for cut sets and ties, point by point, the
+// walks at the edges set the time of a small frame.)
 __device__ __forceinline__ Within walk_range(const WalkBounds& b) { return Within{disp(b.dx_lo, b.dy_lo), disp(b.dx_hi, b.dy_hi)}; }
 
 struct WalkW {
@@ -688,15 +623,6 @@ __device__ __forceinline__ void score_clipped(uint32_t set, uint32_t pc, uint32_
     }
 }
 
-// This lane's point (lanes 0 to 12), from the centre.
-__device__ __forceinline__ int lane_point(int lane)
-{
-    // x + 2 and y + 2 of the points, three bits each
-    constexpr auto pack = [](bool y) { unsigned long long v = 0; for (int i = 0; i < 13; ++i) v |= (unsigned long long)((y ? point_y(i) : point_x(i)) + 2) << (3 * i); return v; };
-    constexpr unsigned long long X = pack(false), Y = pack(true);
-    const int i = lane < 13 ? lane : 8;
-    return pair((int)(X >> (3 * i) & 7) - 2, (int)(Y >> (3 * i) & 7) - 2);
-}
 // Shared-memory bytes from a candidate to the one displaced by a pair.
 template <int PITCH>
 __device__ __forceinline__ uint32_t bytes_of(int p)
@@ -740,13 +666,8 @@ __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base,
         if (lane == 8 && w.kind != KIND_FIRST) mine = w.bs;       // the centre
         const int d = w.at + point;
         if (!within(d, valid)) mine = 0xffffffffu;
-        const uint32_t ns = __reduce_min_sync(all, mine);
-        unsigned best = __ballot_sync(all, mine == ns);
-        if (best & (best - 1)) {                                  // equal scores: the exact order among them
-            const uint32_t kt = tie_key(disp_x(d), disp_y(d)), kb = __reduce_min_sync(all, mine == ns ? kt : 0xffffffffu);
-            best = __ballot_sync(all, mine == ns && kt == kb);
-        }
-        const int g = __ffs(best) - 1;                            // the best point after this round
+        uint32_t ns;
+        const int g = best_lane(mine, d, ns);                     // the best point after this round
         const int next = __shfl_sync(all, d, g);
         if (w.kind == KIND_SMALL) { w.at = next; w.bs = ns; return 1; }                // the small diamond's best is the result
         if (g == 8) { w.bs = ns; w.kind = KIND_SMALL; continue; }                      // centre won: small diamond, then done
@@ -948,13 +869,7 @@ __device__ __forceinline__ void tss_walk(uint32_t lane_base, int pitch, int s0, 
         }
         const int d = at + step * point;
         if (!within(d, valid)) mine = 0xffffffffu;
-        bs = __reduce_min_sync(all, mine);
-        unsigned best = __ballot_sync(all, mine == bs);
-        if (best & (best - 1)) {                                  // equal scores: the exact order among them
-            const uint32_t kt = tie_key(disp_x(d), disp_y(d)), kb = __reduce_min_sync(all, mine == bs ? kt : 0xffffffffu);
-            best = __ballot_sync(all, mine == bs && kt == kb);
-        }
-        const int g = __ffs(best) - 1, my = g / 3 - 1, mx = g - 3 * (my + 1) - 1;
+        const int g = best_lane(mine, d, bs), my = g / 3 - 1, mx = g - 3 * (my + 1) - 1;
         at += step * pair(mx, my);
         pc += (uint32_t)((my * pitch + mx) * step * 4);
     }
@@ -1140,26 +1055,7 @@ __global__ void __launch_bounds__(P_WARPS * 32, AHEAD ? 2 : 4) k_search_dsw_long
 // or the range for it, or its own best vector is M, so that Step 2 already holds the score (Section 4's second
 // acceleration, exact in that case) -- and lists the others.  k_verify16_list scores the listed blocks, one
 // half-warp per block and one lane per block row, so that no warp idles on blocks that were settled.
-struct Step4 { int Mx, My, K; bool settled; int ok; };
-// The global motion of stream s, and block b (number gi in all) where no pixels are needed to settle it.
-__device__ __forceinline__ Step4 settle16(const MatchArgs& a, unsigned gi, int s, int b, bool in_grid)
-{
-    const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * 16, y0 = by * 16, bw = min(16, a.W - x0), bh = min(16, a.H - y0);
-    const int4 sums = __ldcg((const int4*)a.acc + s);                            // Step 3: sum dx, sum dy, K (one 16-byte load)
-    Step4 r = {0, 0, sums.z, false, 0};
-    if (r.K > 0) { r.Mx = round_mean(sums.x, r.K); r.My = round_mean(sums.y, r.K); }
-    const bool cand_ok = in_grid && r.K > 0 && abs(r.Mx) <= a.R && abs(r.My) <= a.R && x0 + r.Mx >= 0 && y0 + r.My >= 0 &&
-                         x0 + r.Mx + bw <= a.W && y0 + r.My + bh <= a.H;
-    bool known = false; uint32_t v = 0;
-    if (cand_ok) {
-        const uint32_t own = ((const uint32_t*)a.mv)[gi];                         // (dx, dy) as one word
-        v = a.sse[gi];
-        known = (int16_t)(own & 0xffffu) == r.Mx && (int16_t)(own >> 16) == r.My && v != 0xffffffffu;
-    }
-    r.settled = in_grid && (!cand_ok || known);
-    r.ok = known && v <= a.limit[limit_index(a, bw, bh)];
-    return r;
-}
+
 // Lane r of 16: the SSE of row r of block b displaced by (Mx, My).
 __device__ __forceinline__ uint32_t score16(const MatchArgs& a, int s, int b, int Mx, int My, int r, bool on)
 {
@@ -1205,7 +1101,7 @@ __global__ void __launch_bounds__(256) k_verify16_prep(MatchArgs a, uint32_t* li
     const unsigned gi = blockIdx.x * 256u + threadIdx.x;                          // S * Gx * Gy < 2^31
     const bool in_grid = gi < (unsigned)(per * a.S);
     const int s = in_grid ? (int)(gi / (unsigned)per) : a.S - 1, b = in_grid ? (int)(gi - (unsigned)s * per) : 0;
-    const Step4 r = settle16(a, gi, s, b, in_grid);
+    const Step4 r = settle(a, 16, gi, s, b, in_grid);
     if (r.settled) a.matched[gi] = (uint8_t)r.ok;
     if (in_grid && b == 0) { a.gmv[3 * s] = r.Mx; a.gmv[3 * s + 1] = r.My; a.gmv[3 * s + 2] = r.K; }
     // matched count: one atomic per warp and stream
@@ -1256,7 +1152,7 @@ __global__ void __launch_bounds__(256) k_verify16_few(MatchArgs a)
     const unsigned gi = (blockIdx.x * 8u + (threadIdx.x >> 5)) * 2u + half;
     const bool in_grid = gi < (unsigned)(per * a.S);
     const int s = in_grid ? (int)(gi / (unsigned)per) : a.S - 1, b = in_grid ? (int)(gi - (unsigned)s * per) : 0;
-    const Step4 v = settle16(a, gi, s, b, in_grid);
+    const Step4 v = settle(a, 16, gi, s, b, in_grid);
     const bool todo = in_grid && !v.settled;
     const uint32_t sse = __reduce_add_sync(half ? 0xffff0000u : 0x0000ffffu, score16(a, s, b, v.Mx, v.My, r, todo));
     if (r != 0 || !in_grid) return;
@@ -1435,21 +1331,13 @@ __global__ void __launch_bounds__(256) k_copy_frame(const uint8_t* src, const ui
     }
 }
 
-template <int ITERS>
-void launch_verify(dc_cache* c, MatchArgs& a)
+void launch_verify(dc_cache* c, const MatchArgs& a)
 {
     dc_prof_scope ps(c, DC_ST_VERIFY);
-    dc_launch_pdl(k_verify<ITERS>, dim3((unsigned)dc_div_up(a.S * a.Gx * a.Gy, WARPS)), WARPS * 32, 0, c->stream, a);    // errors: cudaGetLastError below
-}
-
-void launch_verify_by_block(dc_cache* c, MatchArgs& a)
-{
-    int row_words = (a.B * 3 + 3) / 4, iters = dc_div_up(a.B * row_words, 32);
-    if (iters <= 2) launch_verify<2>(c, a);
-    else if (iters <= 3) launch_verify<3>(c, a);
-    else if (iters <= 6) launch_verify<6>(c, a);
-    else if (iters <= 12) launch_verify<12>(c, a);
-    else launch_verify<24>(c, a);
+    const int blocks = a.S * a.Gx * a.Gy, share = blocks <= c->num_sms * 64 ? 2 : 8;
+    const dim3 grid((unsigned)dc_div_up(blocks, 8 * share));
+    if (a.B <= 16) dc_launch_pdl(k_verify<16>, grid, 256, 0, c->stream, a, share);       // errors: cudaGetLastError below
+    else dc_launch_pdl(k_verify<32>, grid, 256, 0, c->stream, a, share);
 }
 
 // Step 2 over staged windows: every block, or (only_clipped, see dc_win_args) those that the 16-pixel kernels leave out
@@ -1564,7 +1452,7 @@ int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key
             c->launches += 1;
         }
     } else {
-        launch_verify_by_block(c, a);
+        launch_verify(c, a);
     }
     {
         dc_prof_scope ps(c, DC_ST_MERGE);

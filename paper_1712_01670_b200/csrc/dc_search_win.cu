@@ -14,10 +14,10 @@
 // Candidates are ordered by (SSE, |dx| + |dy|, dy, dx).  Integer arithmetic only.
 //
 // What bounds them: with few blocks the chain of rounds of one walk (a round is one trip to shared memory and back),
-// otherwise instruction issue.  The kernels before kept one warp per block too, but fetched every candidate from global
-// memory, two loads and a funnel shift per four bytes (byte by byte without a cache).
+// otherwise instruction issue.
 #include "dc_common.cuh"
 #include "dc_search_win.cuh"
+#include "dc_walk.cuh"
 
 namespace {
 
@@ -26,11 +26,6 @@ constexpr int kMaxWarps = 16;
 // Pixels around the tile that walks over a longer range stage at least.  A walk visits a few dozen candidates near its start;
 // staging 64 pixels on every side of a few small blocks cost more than all of them (see dc_launch_search_win).
 constexpr int kWalkReach = 32;
-
-__device__ __forceinline__ uint32_t tie_of(int dx, int dy)
-{
-    return ((uint32_t)(abs(dx) + abs(dy)) << 16) | ((uint32_t)(dy + 128) << 8) | (uint32_t)(dx + 128);
-}
 
 // Pixel at byte address p of a buffer [lo, hi): whole aligned words where they lie inside the buffer, bytes at its ends.
 __device__ __forceinline__ uint32_t load_pixel(const uint8_t* p, const uint8_t* lo, const uint8_t* hi)
@@ -49,9 +44,8 @@ struct Tile { int s, bx0, by0, nbx, nby; };       // stream, first block, blocks
 __device__ __forceinline__ Tile tile_of(const dc_win_args& a)
 {
     Tile t;
-    const int tx = blockIdx.x % a.tiles_x, u = blockIdx.x / a.tiles_x;
-    t.s = u / a.tiles_y;
-    t.bx0 = tx * a.TX; t.by0 = (u - t.s * a.tiles_y) * a.TY;
+    t.s = blockIdx.z;
+    t.bx0 = blockIdx.x * a.TX; t.by0 = blockIdx.y * a.TY;
     t.nbx = min(a.TX, a.Gx - t.bx0); t.nby = min(a.TY, a.Gy - t.by0);
     return t;
 }
@@ -71,37 +65,38 @@ __device__ __forceinline__ bool any_mine(const dc_win_args& a, const Tile& t)
     return a.only_clipped == 0 || right || bottom;
 }
 
-// The window, rows warp by warp, a lane four pixels: the 12 bytes come as four aligned words, whatever the row's
-// alignment.  Groups that cross the frame's left or right edge, and the few at the ends of the buffer, go pixel by pixel.
-// What lies outside the frame is never part of a valid candidate.
+// The window, rows warp by warp, a lane four pixels: the 12 bytes come as four aligned words, whatever the row's alignment, also where some of
+// them lie beside the frame (what does is never part of a valid candidate).  Only lanes whose words may leave the buffer, at its two
+// ends, go pixel by pixel.
 __device__ __forceinline__ void stage_window(const dc_win_args& a, const Tile& t, uint32_t* win)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    const int x0 = t.bx0 * a.B - a.Rw, y0 = t.by0 * a.B - a.Rw;
+    const int x0 = t.bx0 * a.B - a.Rw, y0 = t.by0 * a.B - a.Rw, margin = a.margin, cols = a.win_cols - margin;
     const uint8_t* prev = a.prev + (size_t)t.s * a.prev_stream;
-    const int y_lo = max(y0, 0), y_hi = min(y0 + a.win_rows, a.H) - 1;
-    const uint8_t* first = prev + (size_t)y_lo * a.prev_pitch + (size_t)max(x0, 0) * 3;
-    const uint8_t* last = prev + (size_t)y_hi * a.prev_pitch + (size_t)min(x0 + a.win_cols, a.W) * 3;
-    const bool words = (const uint8_t*)((uintptr_t)first & ~(uintptr_t)3) >= a.prev && last + 8 <= a.prev_end;
+    const int y_lo = max(y0 + margin, 0), y_hi = min(y0 + a.win_rows - margin, a.H) - 1;
     // a narrow window: several rows per warp
-    const int lpr = a.win_cols > 64 ? 32 : a.win_cols > 32 ? 16 : 8, rpw = 32 / lpr, l = lane % lpr;
-#pragma unroll 2
-    for (int y = y_lo + warp * rpw + lane / lpr; y <= y_hi; y += warps * rpw) {
-        const uint8_t* row = prev + (size_t)y * a.prev_pitch;
-        uint32_t* dst = win + (y - y0) * a.win_pitch;
-        for (int c = 4 * l; c < a.win_cols; c += 4 * lpr) {
-            const int x = x0 + c;
-            if (words && x >= 0 && x + 4 <= a.W) {
-                const uint8_t* p = row + (size_t)x * 3;
+    const int lpr = cols - margin > 64 ? 32 : cols - margin > 32 ? 16 : 8, rpw = 32 / lpr, l = lane & (lpr - 1);
+    const int first_row = y_lo + warp * rpw + lane / lpr, row_step = warps * rpw;
+    const uint32_t m = 0x00ffffffu;
+    for (int c = margin + 4 * l; c < cols; c += 4 * lpr) {             // once, but for windows wider than 128 pixels
+        const int x = x0 + c;
+        if (x + 4 <= 0 || x >= a.W) continue;
+        uint32_t* dst = win + (first_row - y0) * a.win_pitch + c;
+        const uint8_t* p = prev + (ptrdiff_t)first_row * (ptrdiff_t)a.prev_pitch + (ptrdiff_t)x * 3;
+        if (p - 3 >= a.prev && prev + (ptrdiff_t)y_hi * (ptrdiff_t)a.prev_pitch + (ptrdiff_t)x * 3 + 16 <= a.prev_end) {
+#pragma unroll 3
+            for (int y = first_row; y <= y_hi; y += row_step, p += row_step * a.prev_pitch, dst += row_step * a.win_pitch) {
                 const uint32_t* q = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
-                const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u, m = 0x00ffffffu;
-                const uint32_t w0 = dc_ld(q), w1 = dc_ld(q + 1), w2 = dc_ld(q + 2), w3 = sh ? dc_ld(q + 3) : 0u;
+                const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u;
+                const uint32_t w0 = dc_ld(q), w1 = dc_ld(q + 1), w2 = dc_ld(q + 2), w3 = dc_ld(q + 3);
                 const uint32_t b0 = __funnelshift_r(w0, w1, sh), b1 = __funnelshift_r(w1, w2, sh), b2 = __funnelshift_r(w2, w3, sh);
-                dst[c] = b0 & m; dst[c + 1] = __funnelshift_r(b0, b1, 24) & m; dst[c + 2] = __funnelshift_r(b1, b2, 16) & m; dst[c + 3] = b2 >> 8;
-            } else {
-                for (int k = 0; k < 4; ++k)
-                    if (x + k >= 0 && x + k < a.W) dst[c + k] = load_pixel(row + (size_t)(x + k) * 3, a.prev, a.prev_end);
+                dst[0] = b0 & m; dst[1] = __funnelshift_r(b0, b1, 24) & m; dst[2] = __funnelshift_r(b1, b2, 16) & m; dst[3] = b2 >> 8;
             }
+        } else {
+            for (int y = first_row; y <= y_hi; y += row_step, p += row_step * a.prev_pitch, dst += row_step * a.win_pitch)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (x + k >= 0 && x + k < a.W) dst[k] = load_pixel(p + 3 * k, a.prev, a.prev_end);
         }
     }
 }
@@ -135,52 +130,25 @@ __device__ __forceinline__ void flush_sums(const dc_win_args& a, const Tile& t, 
 }
 
 // ---- walks -----------------------------------------------------------------------------------------------------------
-// Points around a centre: 0-7 the large diamond, 8 the centre, 9-12 the small diamond.  A round of the diamond search
-// scores one of ten sets: after the move along point `kind` (0-7) the points of the large diamond that are new (the
-// others lost to the new centre already and cannot win), 8 the first round, 9 the small diamond.
-__host__ __device__ constexpr int pt_x(int i) { constexpr int t[13] = {0, -1, 1, -2, 2, -1, 1, 0, 0, 0, -1, 1, 0}; return t[i]; }
-__host__ __device__ constexpr int pt_y(int i) { constexpr int t[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1}; return t[i]; }
-__constant__ int c_pt_x[13] = {0, -1, 1, -2, 2, -1, 1, 0, 0, 0, -1, 1, 0};
-__constant__ int c_pt_y[13] = {-2, -1, -1, 0, 0, 1, 1, 2, 0, -1, 0, 0, 1};
-constexpr int KIND_FIRST = 8, KIND_SMALL = 9;
-__host__ __device__ constexpr uint32_t set_of(int kind)
-{
-    constexpr uint32_t t[10] = {31u, 11u, 21u, 171u, 213u, 168u, 208u, 248u, 0x1ffu, 0x1e00u};
-    return t[kind];
-}
-__constant__ uint32_t c_set[10] = {31u, 11u, 21u, 171u, 213u, 168u, 208u, 248u, 0x1ffu, 0x1e00u};
-// kind of a move (mx, my), indexed by ((my + 2) * 5 + (mx + 2)) >> 1
-__constant__ int c_kind[13] = {0, 0, 0, 1, 2, 3, 0, 4, 5, 6, 0, 7, 0};
-
-template <int OFF>
-__device__ __forceinline__ uint32_t lds_off(uint32_t p)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(p), "n"(OFF) : "memory");
-    return v;
-}
-
-// FAR: the window holds fewer than R pixels around the tile.
-template <int ITERS, bool FAR>
+// FAR: the window holds fewer than R pixels around the tile.  BT, PT: block edge and window pitch where they are known at compile time
+// (walk_pitch), else 0.
+template <int ITERS, bool FAR, int BT, int PT>
 struct Walk {
     uint32_t base;                  // shared-memory byte address of displacement (0, 0)
-    int pitch4;                     // window row in bytes
-    int dx_lo, dx_hi, dy_lo, dy_hi; // displacements that keep the block inside the frame and the range
+    int pitch4_;                    // window row in bytes
+    Within valid;                   // displacements that keep the block inside the frame and the range
     const dc_win_args* args;        // FAR: where candidates outside the window come from:
     const uint8_t* home;            // the block's position in the previous frame
     uint32_t cw[ITERS], off[ITERS]; // this lane's pixels and their byte offsets in the window
     uint32_t on;                    // which of them exist
     bool whole;                     // the block is not clipped: the first FULL exist in every lane
     static constexpr int FULL = ITERS <= 8 ? ITERS - 1 : ITERS / 2;
-    int bx, by; uint32_t bs;        // best point so far and its SSE
+    int at; uint32_t bs;            // best point so far and its SSE
 
-    __device__ __forceinline__ bool staged(int cx, int cy, int reach) const
+    __device__ __forceinline__ int pitch4() const { return PT ? PT * 4 : pitch4_; }
+    __device__ __forceinline__ bool staged(int dx, int dy, int reach) const
     {
-        return !FAR || (abs(cx) + reach <= kWalkReach && abs(cy) + reach <= kWalkReach);
-    }
-    __device__ __forceinline__ bool inside(int cx, int cy, int reach) const
-    {
-        return cx - reach >= dx_lo && cx + reach <= dx_hi && cy - reach >= dy_lo && cy + reach <= dy_hi && staged(cx, cy, reach);
+        return !FAR || (abs(dx) + reach <= kWalkReach && abs(dy) + reach <= kWalkReach);
     }
     // A candidate outside the window, from global memory: eight of the lane's pixels in flight.
     __device__ uint32_t far(int dx, int dy) const
@@ -226,41 +194,44 @@ struct Walk {
     __device__ __forceinline__ uint32_t score(int dx, int dy) const
     {
         if (FAR && !staged(dx, dy, 0)) return far(dx, dy);
-        const uint32_t p = base + (uint32_t)(dy * pitch4 + dx * 4);
+        const uint32_t p = base + (uint32_t)(dy * pitch4() + dx * 4);
         uint32_t acc = 0;
 #pragma unroll
         for (int i = 0; i < ITERS; ++i) {
-            const uint32_t d = ((on >> i) & 1u) ? __vabsdiffu4(cw[i], lds_off<0>(p + off[i])) : 0u;
+            const uint32_t d = ((on >> i) & 1u) ? __vabsdiffu4(cw[i], lds_at<0>(p + off[i])) : 0u;
             acc = __dp4a(d, d, acc);
         }
         return __reduce_add_sync(0xffffffffu, acc);
     }
-    // One point under the full order (SSE, |dx| + |dy|, dy, dx).
-    __device__ __forceinline__ void consider(int dx, int dy, uint32_t& ns, int& nx, int& ny) const
+    // The points of `set` one by one, for blocks that the frame's edge cuts and centres near the end of the window.  d: the lanes' points.
+    __device__ __forceinline__ void slow_set(unsigned set, int d, int lane, uint32_t& mine) const
     {
-        if (dx < dx_lo || dx > dx_hi || dy < dy_lo || dy > dy_hi) return;
-        const uint32_t s = score(dx, dy);
-        if (s < ns || (s == ns && tie_of(dx, dy) < tie_of(nx, ny))) { ns = s; nx = dx; ny = dy; }
+#pragma unroll 1
+        while (set) {
+            const int i = __ffs(set) - 1, p = __shfl_sync(0xffffffffu, d, i);
+            set &= set - 1;
+            const uint32_t s = score(disp_x(p), disp_y(p));
+            mine = lane == i ? s : mine;
+        }
     }
-    // The points of SET around (cx, cy), all valid, as straight-line code: smallest SSE and its point; tie: two scores
-    // that matter were equal, the round has to be redone under the full order.
+    // The points of SET around the centre at pc, all staged, as straight-line code; lane i keeps the score of point i.
     template <uint32_t SET>
-    __device__ __forceinline__ void fast_set(int cx, int cy, uint32_t& ms, int& mi, bool& tie) const
+    __device__ __forceinline__ void fast_set(uint32_t pc, int lane, uint32_t& mine) const
     {
-        const uint32_t pc = base + (uint32_t)(cy * pitch4 + cx * 4);
         uint32_t s[13];
 #pragma unroll
         for (int k = 0; k < 13; ++k) s[k] = 0;
 #pragma unroll
         for (int i = 0; i < ITERS; ++i) add_point<SET, 0>(i, pc + off[i], s);
-        pick<SET, 0>(s, ms, mi, tie);
+        keep<SET, 0>(s, lane, mine);
     }
     template <uint32_t SET, int I>
     __device__ __forceinline__ void add_point(int i, uint32_t p, uint32_t (&s)[13]) const
     {
         if constexpr (I < 13) {
             if constexpr (((SET >> I) & 1u) != 0) {
-                uint32_t d = __vabsdiffu4(cw[i], lds_off<pt_x(I) * 4>(p + (uint32_t)(pt_y(I) * pitch4)));
+                const uint32_t v = PT ? lds_at<(point_y(I) * PT + point_x(I)) * 4>(p) : lds_at<point_x(I) * 4>(p + (uint32_t)(point_y(I) * pitch4_));
+                uint32_t d = __vabsdiffu4(cw[i], v);
                 if (i >= FULL) d &= 0u - ((on >> i) & 1u);
                 s[I] = __dp4a(d, d, s[I]);
             }
@@ -268,77 +239,72 @@ struct Walk {
         }
     }
     template <uint32_t SET, int I>
-    __device__ __forceinline__ void pick(const uint32_t (&s)[13], uint32_t& ms, int& mi, bool& tie) const
+    __device__ __forceinline__ void keep(const uint32_t (&s)[13], int lane, uint32_t& mine) const
     {
         if constexpr (I < 13) {
             if constexpr (((SET >> I) & 1u) != 0) {
                 const uint32_t v = __reduce_add_sync(0xffffffffu, s[I]);
-                tie |= v == ms;
-                mi = v < ms ? I : mi;
-                ms = min(ms, v);
+                mine = lane == I ? v : mine;
             }
-            pick<SET, I + 1>(s, ms, mi, tie);
+            keep<SET, I + 1>(s, lane, mine);
         }
     }
-    // large diamond until its centre wins, then one small diamond
+    // large diamond until its centre wins, then one small diamond.  A point's score stands in its lane, which drops it where it is no valid
+    // candidate (a centre's points are staged, whatever the range); the best lane names the next centre.
     __device__ __forceinline__ void diamond(int R, int32_t* status)
     {
-        bx = by = 0; bs = 0xffffffffu;
+        const unsigned all = 0xffffffffu;
+        const int lane = threadIdx.x & 31, point = lane_point(lane);
+        at = disp(0, 0); bs = 0xffffffffu;
         int kind = KIND_FIRST;
-        const int max_moves = (2 * R + 1) * (2 * R + 1);              // every move strictly lowers the key: never reached
 #pragma unroll 1
-        for (int m = 0;; ++m) {
-            const int cx = bx, cy = by;
-            uint32_t ms = 0xffffffffu; int mi = 8; bool tie = true;
-            if (whole && inside(cx, cy, 2)) {
-                tie = false;
+        for (int moves_left = (2 * R + 1) * (2 * R + 1);; --moves_left) {     // every move strictly lowers the key: never used up
+            const int cx = disp_x(at), cy = disp_y(at), d = at + point;
+            const bool ok = lane < 13 && within(d, valid);
+            uint32_t mine = 0xffffffffu;
+            if (whole && staged(cx, cy, 2)) {
+                const uint32_t pc = base + (uint32_t)(cy * pitch4() + cx * 4);
                 switch (kind) {
-                case 0: fast_set<set_of(0)>(cx, cy, ms, mi, tie); break;
-                case 1: fast_set<set_of(1)>(cx, cy, ms, mi, tie); break;
-                case 2: fast_set<set_of(2)>(cx, cy, ms, mi, tie); break;
-                case 3: fast_set<set_of(3)>(cx, cy, ms, mi, tie); break;
-                case 4: fast_set<set_of(4)>(cx, cy, ms, mi, tie); break;
-                case 5: fast_set<set_of(5)>(cx, cy, ms, mi, tie); break;
-                case 6: fast_set<set_of(6)>(cx, cy, ms, mi, tie); break;
-                case 7: fast_set<set_of(7)>(cx, cy, ms, mi, tie); break;
-                case KIND_FIRST: fast_set<set_of(KIND_FIRST)>(cx, cy, ms, mi, tie); break;
-                default: fast_set<set_of(KIND_SMALL)>(cx, cy, ms, mi, tie); break;
+                case 0: fast_set<kind_mask(0)>(pc, lane, mine); break;
+                case 1: fast_set<kind_mask(1)>(pc, lane, mine); break;
+                case 2: fast_set<kind_mask(2)>(pc, lane, mine); break;
+                case 3: fast_set<kind_mask(3)>(pc, lane, mine); break;
+                case 4: fast_set<kind_mask(4)>(pc, lane, mine); break;
+                case 5: fast_set<kind_mask(5)>(pc, lane, mine); break;
+                case 6: fast_set<kind_mask(6)>(pc, lane, mine); break;
+                case 7: fast_set<kind_mask(7)>(pc, lane, mine); break;
+                case KIND_FIRST: fast_set<kind_mask(KIND_FIRST)>(pc, lane, mine); break;
+                default: fast_set<kind_mask(KIND_SMALL)>(pc, lane, mine); break;
                 }
-                tie |= ms == bs;
-            }
-            if (!tie) {
-                if (ms < bs) { bs = ms; bx = cx + c_pt_x[mi]; by = cy + c_pt_y[mi]; }
             } else {
-                uint32_t set = c_set[kind], ns = bs; int nx = cx, ny = cy;
-                if (kind == KIND_FIRST) { ns = score(0, 0); set &= ~0x100u; }     // the centre is the first candidate
-#pragma unroll 1
-                while (set) {
-                    const int i = __ffs(set) - 1;
-                    set &= set - 1;
-                    consider(cx + c_pt_x[i], cy + c_pt_y[i], ns, nx, ny);
-                }
-                bs = ns; bx = nx; by = ny;
+                slow_set(c_kind_mask[kind] & __ballot_sync(all, ok), d, lane, mine);
             }
+            if (lane == 8 && kind != KIND_FIRST) mine = bs;               // the centre
+            if (!ok) mine = 0xffffffffu;
+            const int g = best_lane(mine, d, bs);
+            at = __shfl_sync(all, d, g);
             if (kind == KIND_SMALL) return;
-            if (bx == cx && by == cy) { kind = KIND_SMALL; continue; }
-            if (m >= max_moves) { if ((threadIdx.x & 31) == 0 && status) atomicExch(status, (int)DC_ERR_TIMEOUT); return; }
-            kind = c_kind[((by - cy + 2) * 5 + (bx - cx + 2)) >> 1];
+            if (g == 8) { kind = KIND_SMALL; continue; }
+            if (moves_left <= 0) { if (lane == 0 && status) atomicExch(status, (int)DC_ERR_TIMEOUT); return; }
+            kind = g;
         }
     }
-    // nine-point passes with step S0, S0/2, ..., 1; S0 = largest power of two with 2 S0 - 1 <= R
+    // nine-point passes with step S0, S0/2, ..., 1; S0 = largest power of two with 2 S0 - 1 <= R.  Lane g < 9 holds point g of the grid
+    // (4: its centre, the best so far).
     __device__ __forceinline__ void three_step(int R)
     {
-        bx = by = 0; bs = score(0, 0);
+        const unsigned all = 0xffffffffu;
+        const int lane = threadIdx.x & 31, point = pair(lane % 3 - 1, lane / 3 - 1);
+        at = disp(0, 0); bs = score(0, 0);
         int step = R < 1 ? 0 : 1;
         while (step > 0 && 4 * step - 1 <= R) step *= 2;
 #pragma unroll 1
         for (; step >= 1; step >>= 1) {
-            const int cx = bx, cy = by;
-            bool tie = true;
-            uint32_t ms = 0xffffffffu; int mi = 4;
-            if (whole && inside(cx, cy, step)) {
-                tie = false;
-                const uint32_t pc = base + (uint32_t)(cy * pitch4 + cx * 4);
+            const int cx = disp_x(at), cy = disp_y(at), d = at + step * point;
+            const bool ok = lane < 9 && within(d, valid);
+            uint32_t mine = 0xffffffffu;
+            if (whole && staged(cx, cy, step)) {
+                const uint32_t pc = base + (uint32_t)(cy * pitch4() + cx * 4);
                 uint32_t s[9];
 #pragma unroll
                 for (int k = 0; k < 9; ++k) s[k] = 0;
@@ -347,71 +313,80 @@ struct Walk {
 #pragma unroll
                     for (int k = 0; k < 9; ++k)
                         if (k != 4) {
-                            uint32_t d = __vabsdiffu4(cw[i], lds_off<0>(pc + off[i] + (uint32_t)((k / 3 - 1) * step * pitch4 + (k % 3 - 1) * step * 4)));
-                            if (i >= FULL) d &= 0u - ((on >> i) & 1u);
-                            s[k] = __dp4a(d, d, s[k]);
+                            uint32_t e = __vabsdiffu4(cw[i], lds_at<0>(pc + off[i] + (uint32_t)((k / 3 - 1) * step * pitch4() + (k % 3 - 1) * step * 4)));
+                            if (i >= FULL) e &= 0u - ((on >> i) & 1u);
+                            s[k] = __dp4a(e, e, s[k]);
                         }
 #pragma unroll
                 for (int k = 0; k < 9; ++k)
-                    if (k != 4) {
-                        const uint32_t v = __reduce_add_sync(0xffffffffu, s[k]);
-                        tie |= v == ms;
-                        mi = v < ms ? k : mi;
-                        ms = min(ms, v);
-                    }
-                tie |= ms == bs;
-            }
-            if (!tie) {
-                if (ms < bs) { bs = ms; bx = cx + (mi % 3 - 1) * step; by = cy + (mi / 3 - 1) * step; }
+                    if (k != 4) { const uint32_t v = __reduce_add_sync(all, s[k]); mine = lane == k ? v : mine; }
             } else {
-                uint32_t ns = bs; int nx = cx, ny = cy;
-#pragma unroll 1
-                for (int k = 0; k < 9; ++k)
-                    if (k != 4) consider(cx + (k % 3 - 1) * step, cy + (k / 3 - 1) * step, ns, nx, ny);
-                bs = ns; bx = nx; by = ny;
+                slow_set(0x1efu & __ballot_sync(all, ok), d, lane, mine);
             }
+            if (lane == 4) mine = bs;
+            if (!ok) mine = 0xffffffffu;
+            const int g = best_lane(mine, d, bs);
+            at = __shfl_sync(all, d, g);
         }
     }
 };
 
-// three CTAs per SM where the lane's pixels leave the registers for it (10-pixel blocks, 720p, 4 streams: 78 us, 90 with
-// two; 16-pixel blocks with three: twice as slow)
-template <int ITERS, bool FAR>
-__global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 && !FAR ? 3 : ITERS <= 8 ? 2 : 1) k_win_walk(const __grid_constant__ dc_win_args a)
+// Window pitch of the instances that know their block edge: room for eight blocks and a range of 16 around them, congruent to B modulo 32.
+__host__ __device__ constexpr int walk_pitch(int B) { return 8 * B + 36 + ((B - (8 * B + 36)) % 32 + 32) % 32; }
+
+// Three CTAs per SM where the lane's pixels leave the registers for it (10-pixel blocks, 720p, 4 streams: 78 us, 90 with two; 16-pixel blocks
+// with three: twice as slow).  AHEAD: two, with 64 registers a thread for the loads of a round; up to two tiles per SM it is the faster one
+// (16 streams of 160 x 128, 10 pixels: 16.3 and 10.8 us).
+// What it spends its instructions on (720p, 4 streams, 10 pixels, 1430 per block before): the candidates a third, so addresses known at compile
+// time, window rows by addition and whole blocks without a test per pixel: 80 us with run-time addresses and a path of their own for cut
+// rounds, 65 without these two, 57 so.
+template <int ITERS, bool FAR, int BT, bool AHEAD>
+__global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 && !FAR && !AHEAD ? 3 : ITERS <= 8 ? 2 : 1) k_win_walk(const __grid_constant__ dc_win_args a)
 {
     extern __shared__ __align__(16) uint32_t win[];
     __shared__ int32_t sums[4];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int PT = BT ? walk_pitch(BT) : 0;
+    const int B = BT ? BT : a.B;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     dc_pdl_wait();
     dc_pdl_release();
     const Tile t = tile_of(a);
     if (!any_mine(a, t)) return;
-    const int ly = warp / a.TX, lx = warp - ly * a.TX, bx = t.bx0 + lx, by = t.by0 + ly;
+    const int ly = warp * a.inv_TX >> 16, lx = warp - ly * a.TX, bx = t.bx0 + lx, by = t.by0 + ly;
     const bool block = ly < a.TY && lx < t.nbx && ly < t.nby && mine(a, bx, by), walk = block && searched(a, bx, by);
-    Walk<ITERS, FAR> w;
-    const int x0 = bx * a.B, y0 = by * a.B, bw = min(a.B, a.W - x0), bh = min(a.B, a.H - y0);
+    Walk<ITERS, FAR, BT, PT> w;
+    const int x0 = bx * B, y0 = by * B, bw = min(B, a.W - x0), bh = min(B, a.H - y0);
     w.on = 0;
+    w.whole = walk && bw == B && bh == B;
+    const uint8_t* home = a.cur + (size_t)t.s * a.cur_stream + (size_t)y0 * a.cur_pitch + (size_t)x0 * 3;
+    // two aligned words around any pixel of the block lie inside the buffer (the same in all lanes)
+    const bool words = home - 3 >= a.cur && home + (size_t)(B - 1) * a.cur_pitch + (size_t)B * 3 + 8 <= a.cur_end;
 #pragma unroll
     for (int i = 0; i < ITERS; ++i) {                                 // issued first: in flight while the window is staged
-        const int p = i * 32 + lane, r = p / a.B, c = p - r * a.B;
+        const int p = i * 32 + lane, r = p / B, c = p - r * B;
+        const bool exists = p < B * B;
+        w.off[i] = exists ? (uint32_t)(r * (PT ? PT : a.win_pitch) + c) * 4u : 0u;     // a lane without a last pixel reads the block's first one, masked
         w.cw[i] = 0;
-        w.off[i] = p < a.B * a.B ? (uint32_t)(r * a.win_pitch + c) * 4u : 0u;   // a lane without a last pixel reads the block's first one, masked
-        if (walk && r < bh && c < bw) {
+        if (w.whole && words) {
+            const uint8_t* q = home + (exists ? (size_t)r * a.cur_pitch + c * 3 : 0);
+            const uint32_t* v = (const uint32_t*)((uintptr_t)q & ~(uintptr_t)3);
+            w.cw[i] = __funnelshift_r(dc_ld(v), dc_ld(v + 1), ((uint32_t)(uintptr_t)q & 3u) * 8u) & 0x00ffffffu;
+            if (exists) w.on |= 1u << i;
+        } else if (walk && r < bh && c < bw) {
             w.on |= 1u << i;
-            w.cw[i] = load_pixel(a.cur + (size_t)t.s * a.cur_stream + (size_t)(y0 + r) * a.cur_pitch + (size_t)(x0 + c) * 3, a.cur, a.cur_end);
+            w.cw[i] = load_pixel(home + (size_t)r * a.cur_pitch + c * 3, a.cur, a.cur_end);
         }
     }
     if (threadIdx.x < 4) sums[threadIdx.x] = 0;
     stage_window(a, t, win);
     __syncthreads();
     if (walk) {
-        w.base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)((ly * a.B + a.Rw) * a.win_pitch + lx * a.B + a.Rw) * 4u;
+        w.base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)((ly * B + a.Rw) * (PT ? PT : a.win_pitch) + lx * B + a.Rw) * 4u;
         if (FAR) { w.args = &a; w.home = a.prev + (size_t)t.s * a.prev_stream + (size_t)y0 * a.prev_pitch + (size_t)x0 * 3; }
-        w.pitch4 = a.win_pitch * 4;
-        w.dx_lo = max(-a.R, -x0); w.dx_hi = min(a.R, a.W - bw - x0); w.dy_lo = max(-a.R, -y0); w.dy_hi = min(a.R, a.H - bh - y0);
-        w.whole = bw == a.B && bh == a.B;
+        w.pitch4_ = a.win_pitch * 4;
+        w.valid = Within{disp(max(-a.R, -x0), max(-a.R, -y0)), disp(min(a.R, a.W - bw - x0), min(a.R, a.H - bh - y0))};
         if (a.search == DC_SEARCH_THREE_STEP) w.three_step(a.R); else w.diamond(a.R, a.status);
-        if (lane == 0) publish(a, t, bx, by, w.bx, w.by, w.bs, sums);
+        if (lane == 0) publish(a, t, bx, by, disp_x(w.at), disp_y(w.at), w.bs, sums);
     } else if (block && lane == 0) {
         mark_skipped(a, t, bx, by);
     }
@@ -494,7 +469,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32) k_win_all(const dc_win_args a)
         for (int d = 0; d < E_ROWS; ++d) {
             const int dy = dy0 + d;
             if (x_ok && dy <= a.R && y0 + dy >= 0 && y0 + dy + bh <= a.H) {
-                const unsigned long long v = ((unsigned long long)acc[d] << 32) | tie_of(dx, dy);
+                const unsigned long long v = ((unsigned long long)acc[d] << 32) | tie_key(dx, dy);
                 key = v < key ? v : key;
             }
         }
@@ -521,7 +496,7 @@ template <typename K>
 int launch(K kernel, const dc_win_args& a, int threads, size_t smem, int device, dc_once_per_device& attr_set, cudaStream_t stream)
 {
     if (attr_set.first(device)) DC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
-    DC_CUDA(dc_launch_pdl(kernel, dim3((unsigned)(a.tiles_x * a.tiles_y * a.S)), threads, smem, stream, a));
+    DC_CUDA(dc_launch_pdl(kernel, dim3((unsigned)a.tiles_x, (unsigned)a.tiles_y, (unsigned)a.S), threads, smem, stream, a));
     return DC_OK;
 }
 
@@ -531,19 +506,22 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
 {
     const bool all = a.search == DC_SEARCH_EXHAUSTIVE;
     size_t smem = 0;
+    bool known = false;                                               // block edge and pitch fit an instance that knows them
     auto shape = [&](int TX, int TY) {
-        a.TX = TX; a.TY = TY;
+        a.TX = TX; a.TY = TY; a.inv_TX = (65536 + TX - 1) / TX;
         a.tiles_x = dc_div_up(a.Gx, TX); a.tiles_y = dc_div_up(a.Gy, TY);
-        a.win_cols = (TX * a.B + 2 * a.Rw + 3) & ~3;                  // staged in groups of four
+        a.win_cols = ((TX * a.B + 2 * (a.Rw - a.margin) + 3) & ~3) + 2 * a.margin;   // staged in groups of four
         a.win_rows = TY * a.B + 2 * a.Rw + (all ? E_ROWS - 1 : 0);    // rows only touched by displacements beyond R (scored, never compared)
         a.win_pitch = a.win_cols + ((a.B - a.win_cols) % 32 + 32) % 32;   // = B modulo 32
+        known = !all && a.margin && a.B <= 16 && a.win_cols <= walk_pitch(a.B);
+        if (known) a.win_pitch = walk_pitch(a.B);
         smem = (size_t)a.win_rows * a.win_pitch * 4 + (all ? (size_t)TX * TY * a.B * a.B * 4 : 0);
     };
     // Wide tiles stage fewer window pixels per block; they shrink while the window is too large for three CTAs per SM, and
     // while the frames have fewer tiles than the machine has SMs (down to two blocks, one for the exhaustive search).
     int TX = 0, TY = 0;
-    auto fit = [&](int Rw) {                                          // returns the window pixels staged per block
-        a.Rw = Rw;
+    auto fit = [&](int Rw, int margin) {                              // returns the window pixels staged per block
+        a.Rw = Rw + margin; a.margin = margin;
         TX = a.Gx < 8 ? a.Gx : 8; TY = TX < 4 ? 4 : 2;
         if (TY > a.Gy) TY = a.Gy;
         shape(TX, TY);
@@ -557,17 +535,28 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     // Walks over a long range: a window of kWalkReach where that stages less than a fifth per block.  (Match calls with the whole
     // window and with the capped one, range 64, diamond: 1080p, 16 streams, 8-pixel blocks, 13 times the pixels: 13456 and 1610 us;
     // 20 pixels, 6.6 times: 4145 and 2184; 227 x 227, 24 pixels, 2.7 times: 72 and 125.  Range 40, 1.4 to 1.8 times: 513 and 571.)
-    const int whole = fit(a.R);
+    // The points around a centre at the end of the range lie up to two pixels beyond it: room for them, not staged.
+    const int beyond = a.search == DC_SEARCH_DIAMOND ? 2 : 0, whole = fit(a.R, beyond);
     bool far = !all && a.R > kWalkReach;
-    if (far && whole <= 5 * fit(kWalkReach)) { far = false; fit(a.R); }
+    if (far && whole <= 5 * fit(kWalkReach, 0)) { far = false; fit(a.R, beyond); }
     // exhaustive: as many warps as there are groups of 32 items, up to 16
     const int n_d = 2 * a.R + 1, groups = (n_d * dc_div_up(n_d, E_ROWS) + 31) / 32;
     int warps = TX * TY < 8 ? 8 : TX * TY;                            // walks: a warp per block; spare ones help to stage the window
     if (all) { const long long units = (long long)TX * TY * groups; warps = units < 4 ? 4 : units > kMaxWarps ? kMaxWarps : (int)units; }
     if (all) { static dc_once_per_device set; return launch(k_win_all, a, warps * 32, smem, device, set, stream); }
-    // one instance per number of pixels a lane owns, up to 16-pixel blocks
-#define DC_WALK_(n, f) { static dc_once_per_device set; return launch(k_win_walk<n, f>, a, warps * 32, smem, device, set, stream); }
-#define DC_WALK(n) { if (far) DC_WALK_(n, true) DC_WALK_(n, false) }
+    // one instance per block edge up to 16, for ranges whose window fits its pitch (three step search: addresses with run-time steps gain
+    // nothing from it), and one per number of pixels a lane owns
+#define DC_WALK_(n, f, b, ah) { static dc_once_per_device set; return launch(k_win_walk<n, f, b, ah>, a, warps * 32, smem, device, set, stream); }
+    const bool few = (long long)a.tiles_x * a.tiles_y * a.S <= 2 * num_sms;
+    if (known) switch (a.B) {
+#define DC_WALK(b) case b: if (few) DC_WALK_((b * b + 31) / 32, false, b, true) DC_WALK_((b * b + 31) / 32, false, b, false)
+        DC_WALK(4) DC_WALK(5) DC_WALK(6) DC_WALK(7) DC_WALK(8) DC_WALK(9) DC_WALK(10) DC_WALK(11)
+#undef DC_WALK
+#define DC_WALK(b) case b: DC_WALK_((b * b + 31) / 32, false, b, false)
+        DC_WALK(12) DC_WALK(13) DC_WALK(14) DC_WALK(15) DC_WALK(16)
+#undef DC_WALK
+    }
+#define DC_WALK(n) { if (far) DC_WALK_(n, true, 0, false) DC_WALK_(n, false, 0, false) }
     switch (dc_div_up(a.B * a.B, 32)) {
     case 1: DC_WALK(1)
     case 2: DC_WALK(2)

@@ -12,8 +12,8 @@ struct dc_win_args {
     int16_t* mv; uint32_t* sse; int32_t* acc;   // acc: [S][4], zeroed: sums of Step 3
     int32_t* status;                     // device status word, or NULL
     // set by dc_launch_search_win
-    int Rw;                              // pixels around the tile that the window holds: R, or kWalkReach for walks
-    int TX, TY, tiles_x, tiles_y, win_rows, win_cols, win_pitch;
+    int Rw, margin;                      // pixels around the tile that the window has room for, and how many of them are not staged
+    int TX, TY, inv_TX, tiles_x, tiles_y, win_rows, win_cols, win_pitch;   // n / TX = n * inv_TX >> 16 for n < 32
 };
 
 // Enqueues the search; fails only with DC_ERR_CUDA.

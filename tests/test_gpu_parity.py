@@ -210,10 +210,13 @@ def test_match_three_step_16_windows(R, shape):
     check_pairs([(prev, far), (const, const), (smooth, np.roll(smooth, 2, axis=1)), (prev, smooth)], 16, R, B.DC_SEARCH_THREE_STEP)
 
 
-@pytest.mark.parametrize("search,R", [(B.DC_SEARCH_DIAMOND, 1), (B.DC_SEARCH_DIAMOND, 5), (B.DC_SEARCH_DIAMOND, 40), (B.DC_SEARCH_THREE_STEP, 3), (B.DC_SEARCH_THREE_STEP, 31)])
-def test_match_16_many_tiles(search, R):
-    """Enough tiles for the search's instance of many warps per SM, with what its rounds meet at the edges: strips and blocks cut on either
-    side, range limits next to the start, equal scores, walks that leave the staged window."""
+@pytest.mark.parametrize("search,R,block", [(B.DC_SEARCH_DIAMOND, 1, 16), (B.DC_SEARCH_DIAMOND, 5, 16), (B.DC_SEARCH_DIAMOND, 40, 16),
+                                            (B.DC_SEARCH_THREE_STEP, 3, 16), (B.DC_SEARCH_THREE_STEP, 31, 16), (B.DC_SEARCH_DIAMOND, 1, 10),
+                                            (B.DC_SEARCH_DIAMOND, 12, 10), (B.DC_SEARCH_DIAMOND, 18, 4), (B.DC_SEARCH_DIAMOND, 30, 10),
+                                            (B.DC_SEARCH_DIAMOND, 16, 11), (B.DC_SEARCH_DIAMOND, 7, 13), (B.DC_SEARCH_THREE_STEP, 9, 10)])
+def test_match_many_tiles(search, R, block):
+    """Enough tiles for the searches' instances of many warps per SM, with what their rounds meet at the edges: strips and blocks cut on
+    either side, range limits next to the start, equal scores, walks that leave the staged window, ranges beyond a fixed pitch."""
     g = rng(R)
     H, W = 70, 147
     x, y = np.meshgrid(np.arange(W), np.arange(H))
@@ -234,7 +237,7 @@ def test_match_16_many_tiles(search, R):
             prev = g.integers(0, 256, (H, W, 3), dtype=np.uint8)
             cur = np.roll(prev, (-2, 2), axis=(0, 1))
         pairs.append((prev, cur))
-    check_pairs(pairs, 16, R, search)
+    check_pairs(pairs, block, R, search)
 
 
 @pytest.mark.parametrize("h,w,k,st,p", [(33, 41, 3, 2, 1), (32, 32, 7, 2, 3), (47, 35, 5, 3, 2), (30, 31, 7, 3, 0), (39, 227, 11, 4, 0), (41, 43, 11, 4, 5)])
