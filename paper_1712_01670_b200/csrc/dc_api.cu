@@ -428,13 +428,14 @@ int dc_match_blocks(dc_cache* c, const uint8_t* frame_dev, size_t pitch, int16_t
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
     if (!c->key_valid) return DC_ERR_STATE;
     DC_TRY(cancel_lookahead(c));
-    uint8_t* scratch = c->key[(c->key_cur + 1) % 3];                             // scratch copy; the cache key stays
-    DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, scratch, c->mv_acc));
+    const bool in_place = dc_match_in_place(c, frame_dev, pitch);
+    uint8_t* scratch = in_place ? nullptr : c->key[(c->key_cur + 1) % 3];        // scratch copy; the cache key stays
+    if (!in_place) DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, scratch, c->mv_acc));
     // the kernels write the caller's arrays themselves; vectors are read back as 32-bit words, so an oddly aligned array of
     // vectors is filled by a copy instead
     const bool direct_mv = block_mv_dev && (uintptr_t)block_mv_dev % 4 == 0;
     const dc_match_out out = {direct_mv ? block_mv_dev : nullptr, block_sse_dev, matched_dev, global_mv_dev, regions_dev, n_regions_dev};
-    DC_TRY(dc_launch_match(c, scratch, c->key[c->key_cur], &out));
+    DC_TRY(dc_launch_match(c, scratch, c->key[c->key_cur], &out, in_place ? frame_dev : nullptr, pitch));
     if (block_mv_dev && !direct_mv)
         DC_CUDA(cudaMemcpyAsync(block_mv_dev, c->blk_mv, (size_t)c->S * c->Gx * c->Gy * 2 * sizeof(int16_t), cudaMemcpyDeviceToDevice, c->stream));
     return mark_key(c);                                             // the scratch copy has been read
@@ -489,18 +490,21 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
     // (see ring_budget())
     c->overlap_mode = looked_ahead && matcher_is_large(c);
     g_dc_pdl = !c->overlap_mode;
+    const uint8_t* in_place = nullptr;                               // the frame, if the search reads it there and copies it as it goes
     if (looked_ahead) {
         // dc_lookahead_frame already copied this frame in and (unless it is a full frame) matched it
         DC_CUDA(cudaStreamWaitEvent(c->stream, c->ev_match, 0));
         c->la_frame = nullptr;
     } else {
         DC_TRY(cancel_lookahead(c));
-        DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, frame_copy, c->mv_acc));
+        if (!refresh && dc_match_in_place(c, frame_dev, pitch)) in_place = frame_dev;
+        else DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, frame_copy, c->mv_acc));
     }
-    DC_TRY(mark_key(c));
+    if (!in_place) DC_TRY(mark_key(c));
     if (!refresh) {
         if (looked_ahead && c->la_matched) dc_use_match_set(c, c->mset_cur ^ 1);              // results are waiting there
-        else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur], nullptr));
+        else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur], nullptr, in_place, pitch));
+        if (in_place) DC_TRY(mark_key(c));                                                    // the search has made the copy
         DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n, true, nullptr, 0, nullptr));
     }
     if (c->input_map && !c->fused_input) DC_TRY(dc_launch_input_map(c, frame_copy, c->key_pitch));
@@ -631,10 +635,11 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     c->stream = c->la_stream;                                       // the launchers enqueue on c->stream
     uint8_t* next_copy = c->key[(c->key_cur + 1) % 3];
     g_dc_pdl = !matcher_is_large(c);                                // as in the inference it runs beside
+    // a copy first, also where the search could read the frame: what it moves travels beside the convolutions, the search takes issue slots
     int rc = dc_launch_copy_frame(c, frame_dev, pitch, next_copy, c->mset[main_set ^ 1].mv_acc);
     if (rc == DC_OK && !next_is_full) {
         dc_use_match_set(c, main_set ^ 1);
-        rc = dc_launch_match(c, next_copy, c->key[c->key_cur], nullptr);
+        rc = dc_launch_match(c, next_copy, c->key[c->key_cur], nullptr, nullptr, 0);
         dc_use_match_set(c, main_set);
     }
     c->stream = main_stream;
@@ -689,6 +694,7 @@ int dc_infer_frame_host(dc_cache* c, const uint8_t* frame_host, size_t pitch, vo
         for (int k = 0; k < 2; ++k) if (!c->prefetched[k]) { slot = k; break; }
         if (slot < 0) {                                           // both buffers hold prefetches of other frames: drop one
             DC_CUDA(cudaStreamSynchronize(c->copy_stream));
+            DC_TRY(cancel_lookahead(c));                          // it may be matching that frame where it lies
             slot = 0;
         }
         DC_CUDA(cudaMemcpyAsync(c->staging[slot], frame_host, bytes, cudaMemcpyHostToDevice, c->stream));

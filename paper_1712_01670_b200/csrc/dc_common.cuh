@@ -212,7 +212,10 @@ static inline cudaError_t dc_launch_pdl(void (*kernel)(KArgs...), dim3 grid, int
 int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst, int32_t* zero);
 // arrays of a caller of dc_match_blocks that the kernels write themselves (NULL: not wanted)
 struct dc_match_out { int16_t* mv; uint32_t* sse; uint8_t* matched; int32_t* gmv; dc_region* regions; int32_t* n_regions; };
-int dc_launch_match(dc_cache* c, const uint8_t* cur_key, const uint8_t* prev_key, const dc_match_out* out);   // both frames in key-frame layout
+// cur_key, prev_key: frames in key-frame layout.  frame (or NULL): the new frame where the caller has it, if dc_match_in_place says so; the
+// search then reads it there, and cur_key (or NULL) becomes its copy as the search goes.
+int dc_launch_match(dc_cache* c, uint8_t* cur_key, const uint8_t* prev_key, const dc_match_out* out, const uint8_t* frame, size_t pitch);
+bool dc_match_in_place(const dc_cache* c, const uint8_t* frame, size_t pitch);
 void dc_use_match_set(dc_cache* c, int k);
 int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers);
 int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out);

@@ -1424,6 +1424,55 @@ def test_lookahead_gives_identical_results():
         dc.close()
 
 
+@pytest.mark.parametrize("search,R", [(B.DC_SEARCH_DIAMOND, 12), (B.DC_SEARCH_THREE_STEP, 9)])
+@pytest.mark.parametrize("W,H,S", [(64, 48, 2), (144, 70, 3), (64, 37, 160)])
+def test_frames_matched_where_they_lie(search, R, W, H, S):
+    """Frames of whole aligned blocks are read by the search where the caller has them, others through a copy: the same frames at any pitch and
+    start give the same matches, outputs and keys, frame by frame, announced or not, also from a buffer that is filled anew behind a call."""
+    g = rng(W + R)
+    coarse = torch.from_numpy(g.integers(0, 256, (S, 3, H // 8 + 6, W // 8 + 6)).astype(np.float32))
+    base = torch.nn.functional.interpolate(coarse, scale_factor=8, mode="bilinear").permute(0, 2, 3, 1).numpy().astype(np.uint8)
+    frames = np.stack([base[:, 3 * t:3 * t + H, 20 - 2 * t:20 - 2 * t + W] for t in range(5)])
+    frames[3, :, :17, :20] ^= 0x55
+    nb = nets.NetBuilder(H, W)
+    nb.conv(nb.conv(-1, 16, 3, 1, 1), 16, 3, 1, 1)
+    ws, bs = nets.random_weights(nb.layers, 5)
+    records = []
+    for pitch, start, ahead in ((W * 3, 0, False), (W * 3, 0, True), (W * 3 + 48, 16, False), (W * 3 + 7, 0, False), (W * 3, 5, True), (W * 3 + 16, 8, False)):
+        dc = DeepCache(W, H, nb.layers, ws, bs, n_streams=S, block=16, search_range=R, search=search, dtype=B.DC_FP32, expire_n=4)
+        bufs = [torch.zeros(start + S * H * pitch, dtype=torch.uint8, device="cuda") for _ in range(2)]
+
+        def put(t):
+            v = bufs[t % 2][start:].view(S, H, pitch)[:, :, :W * 3]
+            v.copy_(torch.from_numpy(np.ascontiguousarray(frames[t])).cuda().reshape(S, H, W * 3))
+            return bufs[t % 2][start:]
+
+        rec, f = [], put(0)
+        for t in range(5):
+            out = torch.empty(dc.out_shape(-1), device="cuda")
+            B.dc_infer_frame(dc.handle, f, pitch, out)
+            if t + 1 < 5:
+                f = put(t + 1)                                    # behind the call, on the same stream
+                if ahead:
+                    B.dc_lookahead_frame(dc.handle, f, pitch)
+                elif t == 1:
+                    mv = torch.zeros((S, dc.Gy, dc.Gx, 2), dtype=torch.int16, device="cuda")
+                    matched = torch.zeros((S, dc.Gy, dc.Gx), dtype=torch.uint8, device="cuda")
+                    B.dc_match_blocks(dc.handle, f, pitch, mv, None, matched, None, None, None)
+                    rec_match = (mv, matched)
+            rec.append((out, dc.layer_regions(-1)[1]))
+        assert dc.status() == B.DC_OK
+        records.append((rec, None if ahead else rec_match))
+        torch.cuda.synchronize()
+        dc.close()
+    assert records[0][1][1].any()
+    for rec, match in records[1:]:
+        for (o0, n0), (o1, n1) in zip(records[0][0], rec):
+            assert torch.equal(o0, o1) and torch.equal(n0, n1)
+        if match is not None:
+            assert all(torch.equal(x, y) for x, y in zip(records[0][1], match))
+
+
 def test_lookahead_waits_for_the_calls_between():
     """dc_lookahead_frame right behind dc_match_blocks (whose frame lies where the announced one goes) and behind
     dc_cache_set_key (which changes the key that it is matched against)."""
