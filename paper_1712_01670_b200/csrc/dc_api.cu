@@ -26,6 +26,7 @@ void dc_use_match_set(dc_cache* c, int k)
     c->mset_cur = k;
     c->blk_mv = m.blk_mv; c->blk_sse = m.blk_sse; c->matched = m.matched; c->run_end = m.run_end; c->mv_acc = m.mv_acc;
     c->long_list = m.long_list; c->gmv = m.gmv; c->regions0 = m.regions0; c->n_regions = m.n_regions;
+    c->table = m.table; c->live = m.live; c->dirty_count = m.dirty_count; c->reuse_px = m.reuse_px; c->alive = m.alive; c->classify_table = m.classify_table;
 }
 
 bool dc_layer_cached(const dc_cache* c, int layer)
@@ -47,6 +48,31 @@ int dev_alloc(dc_cache* c, T** p, size_t count)
     return DC_OK;
 }
 #define DC_TRY(expr) do { int rc__ = (expr); if (rc__ != DC_OK) return rc__; } while (0)
+
+// What region propagation writes, and the table that the reuse step reads it by (dc_build_classify_table).
+int alloc_tables(dc_cache* c, dc_match_set& m)
+{
+    const size_t n = (size_t)c->n_layers, per_layer = (size_t)c->S * c->max_regions;
+    DC_TRY(dev_alloc(c, &m.table, n * per_layer));
+    DC_TRY(dev_alloc(c, &m.live, n * per_layer));
+    DC_TRY(dev_alloc(c, &m.dirty_count, n));
+    DC_TRY(dev_alloc(c, &m.reuse_px, n * c->S * 2));
+    m.alive = m.reuse_px + n * c->S;
+    DC_CUDA(cudaMemsetAsync(m.table, 0, sizeof(dc_region) * n * per_layer, c->stream));
+    DC_CUDA(cudaMemsetAsync(m.reuse_px, 0, sizeof(int32_t) * n * c->S * 2, c->stream));
+    return DC_OK;
+}
+void free_tables(dc_match_set& m)
+{
+    cudaFree(m.table); cudaFree(m.live); cudaFree(m.dirty_count); cudaFree(m.reuse_px); cudaFree(m.classify_table);
+    m.table = m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = nullptr; m.classify_table = nullptr;
+}
+void share_tables(dc_cache* c)
+{
+    dc_match_set& m = c->mset[1]; const dc_match_set& o = c->mset[0];
+    m.table = o.table; m.live = o.live; m.dirty_count = o.dirty_count; m.reuse_px = o.reuse_px; m.alive = o.alive; m.classify_table = o.classify_table;
+}
+bool own_tables(const dc_cache* c) { return c->mset[1].table != c->mset[0].table; }
 
 // Can dc_infer_frame run this layer?  LRN needs its window stated consistently, a fully-connected layer must cover
 // its whole input map (it then runs as that convolution).
@@ -152,22 +178,17 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
         DC_TRY(dev_alloc(c, &m.n_regions, (size_t)S));
         DC_CUDA(cudaMemsetAsync(m.n_regions, 0, sizeof(int32_t) * S, c->stream));
     }
+    DC_TRY(alloc_tables(c, c->mset[0]));
+    share_tables(c);
     dc_use_match_set(c, 0);
-    DC_TRY(dev_alloc(c, &c->table, (size_t)n * S * c->max_regions));
-    DC_TRY(dev_alloc(c, &c->live, (size_t)n * S * c->max_regions));
     DC_TRY(dc_build_propagate_table(c, layers));
-    DC_TRY(dev_alloc(c, &c->dirty_count, (size_t)n));
     DC_TRY(dev_alloc(c, &c->all_count, (size_t)n * 2));
     DC_TRY(dev_alloc(c, &c->partial, (size_t)S + 3));
     DC_CUDA(cudaMemsetAsync(c->partial, 0, sizeof(int32_t) * (S + 3), c->stream));
-    DC_TRY(dev_alloc(c, &c->reuse_px, (size_t)n * S * 2));
-    c->alive = c->reuse_px + (size_t)n * S;
-    DC_CUDA(cudaMemsetAsync(c->reuse_px, 0, sizeof(int32_t) * n * S * 2, c->stream));
     DC_TRY(dev_alloc(c, &c->status, (size_t)1));
     DC_TRY(dev_alloc(c, &c->reused_total, (size_t)n));
     DC_CUDA(cudaMemsetAsync(c->reused_total, 0, sizeof(unsigned long long) * n, c->stream));
     DC_CUDA(cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream));
-    DC_CUDA(cudaMemsetAsync(c->table, 0, sizeof(dc_region) * n * S * c->max_regions, c->stream));
 
     // PSNR > T as an integer bound on the SSE, for the four block shapes of a clipped grid
     for (int i = 0; i < 4; ++i) {
@@ -261,7 +282,9 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
         if (d.kind == DC_CONV && d.in0 == resize && dc_conv_takes_frame(c, i) && !c->L[i].s2d_s) { c->resize_feeds = i; ++readers; }
     }
     if (readers != 1) c->resize_feeds = -1;
-    if (c->executable) DC_TRY(dc_build_classify_table(c));       // after the tuner: it decides each layer's tile geometry
+    if (c->executable) DC_TRY(dc_build_classify_table(c, c->mset[0]));       // after the tuner: it decides each layer's tile geometry
+    share_tables(c);
+    dc_use_match_set(c, 0);
     DC_CUDA(cudaStreamSynchronize(c->stream));
     return DC_OK;
 }
@@ -279,9 +302,10 @@ void release(dc_cache* c)
         cudaFree(m.blk_mv); cudaFree(m.blk_sse); cudaFree(m.matched); cudaFree(m.run_end); cudaFree(m.mv_acc);
         cudaFree(m.long_list); cudaFree(m.gmv); cudaFree(m.regions0); cudaFree(m.n_regions);
     }
-    cudaFree(c->table); cudaFree(c->live); cudaFree(c->classify_table);
-    cudaFree(c->prop_table); cudaFree(c->dirty_count); cudaFree(c->partial); cudaFree(c->all_count);
-    cudaFree(c->reuse_px); cudaFree(c->zero_masks); cudaFree(c->status); cudaFree(c->input_map);
+    if (own_tables(c)) free_tables(c->mset[1]);
+    free_tables(c->mset[0]);
+    cudaFree(c->prop_table); cudaFree(c->partial); cudaFree(c->all_count);
+    cudaFree(c->zero_masks); cudaFree(c->status); cudaFree(c->input_map);
     if (c->stats_pinned) cudaFreeHost(c->stats_pinned);
     for (int i = 0; i < c->n_layers; ++i) {
         dc_layer_rt& L = c->L[i];
@@ -505,7 +529,8 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
         if (looked_ahead && c->la_matched) dc_use_match_set(c, c->mset_cur ^ 1);              // results are waiting there
         else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur], nullptr, in_place, pitch));
         if (in_place) DC_TRY(mark_key(c));                                                    // the search has made the copy
-        DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n, true, nullptr, 0, nullptr));
+        if (!looked_ahead || !c->la_propagated)
+            DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n, true, nullptr, 0, nullptr));
     }
     if (c->input_map && !c->fused_input) DC_TRY(dc_launch_input_map(c, frame_copy, c->key_pitch));
     const size_t per_layer = (size_t)S * c->max_regions;
@@ -615,6 +640,21 @@ static int ensure_lookahead_stream(dc_cache* c)
     DC_CUDA(cudaEventCreateWithFlags(&c->ev_key, cudaEventDisableTiming));
     DC_CUDA(cudaEventCreateWithFlags(&c->ev_match, cudaEventDisableTiming));
     DC_CUDA(cudaEventRecord(c->ev_key, c->stream));     // first use: everything enqueued so far
+    // tables of their own for the announced frame's rectangles; without the memory for them propagation stays with the inference
+    const size_t before = c->bytes;
+    dc_match_set m = c->mset[1];
+    m.table = m.live = nullptr; m.dirty_count = m.reuse_px = nullptr; m.classify_table = nullptr;
+    cudaStream_t main_stream = c->stream;
+    c->stream = c->la_stream;                           // zeroed there, where they are written first
+    const bool ok = alloc_tables(c, m) == DC_OK && dc_build_classify_table(c, m) == DC_OK;
+    c->stream = main_stream;
+    if (ok) {
+        c->mset[1] = m;
+    } else {
+        cudaGetLastError();
+        free_tables(m);
+        c->bytes = before;
+    }
     return DC_OK;
 }
 
@@ -640,7 +680,14 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     if (rc == DC_OK && !next_is_full) {
         dc_use_match_set(c, main_set ^ 1);
         rc = dc_launch_match(c, next_copy, c->key[c->key_cur], nullptr, nullptr, 0);
+        // The rectangles through the layers too, unless the matcher is large: the walk wants much of an SM's shared memory and would wait
+        // between the convolutions for it.  A pass in us, propagated by the inference and so: ResNet-50, one stream, 336 and 326; VGG, 6 streams of
+        // 720p from host memory, 417 and 410; small CNN, 4 streams, 174 and 171; 24 streams of ResNet-50 and more the same.
+        c->la_propagated = rc == DC_OK && own_tables(c) && !matcher_is_large(c);
+        if (c->la_propagated) rc = dc_launch_propagate(c, c->regions0, c->n_regions, c->n_layers, true, nullptr, 0, nullptr);
         dc_use_match_set(c, main_set);
+    } else {
+        c->la_propagated = false;
     }
     c->stream = main_stream;
     g_dc_pdl = true;

@@ -73,11 +73,13 @@ struct dc_layer_rt {
     int tm_next;                    // which of tm_a[] a new input base replaces
 };
 
-// Everything one run of the matcher writes.  Two sets exist so that the matcher may already work on the
-// next frame (dc_lookahead_frame) while inference of the current frame still reads its own set.
+// Everything one run of the matcher and of region propagation writes.  Two sets exist so that both may already work on the
+// next frame (dc_lookahead_frame) while inference of the current frame still reads its own set.  What propagation writes is there
+// once, in both sets, until a frame has been announced.
 struct dc_match_set {
     int16_t* blk_mv; uint32_t* blk_sse; uint8_t* matched; uint16_t* run_end; int32_t* mv_acc; uint4* long_list;
     int32_t* gmv; dc_region* regions0; int32_t* n_regions;
+    dc_region* table; dc_region* live; int32_t* dirty_count; int32_t* reuse_px; int32_t* alive; void* classify_table;
 };
 
 struct dc_cache {
@@ -96,11 +98,11 @@ struct dc_cache {
 
     uint8_t* key[3];                // key frames [S][H][key_pitch]: key[key_cur] is the cached previous frame,
     int key_cur;                    // key[(key_cur + 1) % 3] receives the frame being processed or looked ahead
-    dc_match_set mset[2];           // the members blk_mv ... n_regions below alias mset[mset_cur]
+    dc_match_set mset[2];           // the members blk_mv ... alive below, and classify_table, alias mset[mset_cur]
     int mset_cur;
     cudaStream_t la_stream;         // dc_lookahead_frame: matcher of the next frame beside the current inference
     cudaEvent_t ev_key, ev_match;   // main stream: frame copied in; side stream: lookahead finished
-    const uint8_t* la_frame; size_t la_pitch; bool la_matched;
+    const uint8_t* la_frame; size_t la_pitch; bool la_matched, la_propagated;
     bool last_refreshed;
     bool overlap_mode;              // the last frame was looked ahead: the next one's matching will run beside this inference
     void* classify_table; int n_cached, classify_warps;   // all cached layers' classification in one launch (dc_regions.cu)
@@ -252,7 +254,7 @@ int dc_launch_relu(dc_cache* c, int layer, const void* a);
 int dc_pack_weights(dc_cache* c, int layer, const float* w_dev, const float* b_dev);
 // true for layers that keep their last output as cached values: convolutions, and max pooling / LRN when cfg.cache_pool
 bool dc_layer_cached(const dc_cache* c, int layer);
-int dc_build_classify_table(dc_cache* c);
+int dc_build_classify_table(dc_cache* c, dc_match_set& m);
 int dc_launch_classify_all(dc_cache* c, int cur);
 int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in);
 bool dc_s2d_eligible(const dc_cache* c, const dc_layer_desc& d);

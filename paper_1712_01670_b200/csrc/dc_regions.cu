@@ -579,8 +579,8 @@ static int copy_parts(const dc_cache* c, long long tiles_in_launch, int px_bytes
     return room < 1 ? 1 : room > 8 ? 8 : (int)room;
 }
 
-// Builds the device table for k_classify_copy_all (once, after every map is allocated).
-int dc_build_classify_table(dc_cache* c)
+// Builds the device table for k_classify_copy_all over the rectangles and counters of a match set (once, after every map is allocated).
+int dc_build_classify_table(dc_cache* c, dc_match_set& m)
 {
     const int n = c->n_layers;
     ClassifyLayer* h = (ClassifyLayer*)malloc(sizeof(ClassifyLayer) * (n > 0 ? n : 1));
@@ -592,13 +592,13 @@ int dc_build_classify_table(dc_cache* c)
         if (!dc_layer_cached(c, i)) continue;
         dc_layer_rt& L = c->L[i];
         ClassifyLayer& e = h[k++];
-        e.regions = c->live + (size_t)i * c->S * c->max_regions;
+        e.regions = m.live + (size_t)i * c->S * c->max_regions;
         e.map[0] = (uint8_t*)L.map[0]; e.map[1] = (uint8_t*)L.map[1];
         e.Ho = L.d.out_h; e.Wo = L.d.out_w; e.px_bytes = L.d.cout * c->elt;
         e.tiles_x = L.tiles_x; e.tiles_y = L.tiles_y; e.first_warp = warps;
         e.gpr = L.flat ? L.gpr : 0; e.gpt = L.gpt;
-        e.masks = L.masks; e.dirty_list = L.dirty_list; e.dirty_count = c->dirty_count + i;
-        e.reuse_px = c->reuse_px + (size_t)i * c->S; e.alive = c->alive + (size_t)i * c->S;
+        e.masks = L.masks; e.dirty_list = L.dirty_list; e.dirty_count = m.dirty_count + i;
+        e.reuse_px = m.reuse_px + (size_t)i * c->S; e.alive = m.alive + (size_t)i * c->S;
         e.reused_total = c->reused_total + i;
         e.status = c->status;
         e.parts = copy_parts(c, tiles, e.px_bytes);
@@ -607,8 +607,8 @@ int dc_build_classify_table(dc_cache* c)
     c->n_cached = k; c->classify_warps = warps;
     int rc = DC_OK;
     if (k > 0) {
-        if (cudaMalloc(&c->classify_table, sizeof(ClassifyLayer) * k) != cudaSuccess) { cudaGetLastError(); rc = DC_ERR_ALLOC; }
-        else if (cudaMemcpy(c->classify_table, h, sizeof(ClassifyLayer) * k, cudaMemcpyHostToDevice) != cudaSuccess) rc = DC_ERR_CUDA;
+        if (cudaMalloc(&m.classify_table, sizeof(ClassifyLayer) * k) != cudaSuccess) { cudaGetLastError(); rc = DC_ERR_ALLOC; }
+        else if (cudaMemcpy(m.classify_table, h, sizeof(ClassifyLayer) * k, cudaMemcpyHostToDevice) != cudaSuccess) rc = DC_ERR_CUDA;
         else c->bytes += sizeof(ClassifyLayer) * k;
     }
     free(h);
