@@ -1909,6 +1909,14 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
                 }
             }
         }
+        // few tiles: narrow blocks, while every item has an SM, spread the epilogue (a launch is then a chain of latencies, and of its 5 us
+        // 2.7 were four steps of 32 channels with the add that follows: ResNet-50, one stream, 325 us a frame, 300 so)
+        for (int bn = 64; bn >= 32 && shape == 0; bn -= 32) {
+            TcPlan q;
+            if (2 * bn >= default_bn || de.cout % bn != 0 || (long long)dc_layer_tiles(c, L) * (L.d.cout / bn) > c->num_sms || !make_plan(de, q, 1, bn, ctas)) continue;
+            L.tc_mt = 1; L.tc_bn = bn;
+            trial("tap-by-tap kernel, narrow blocks");
+        }
         HaloPlan h0;
         if (L.weight_halo && halo_ok(de, h0)) {
             for (int bn = h0.BN; (bn >= 64 || bn == h0.BN) && bn >= h0.BN / 2; bn -= 32) {
