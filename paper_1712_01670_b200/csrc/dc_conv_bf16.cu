@@ -198,11 +198,10 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
             if (ok) tc_fence_after();
             return ok;
         };
-        if (!ADD && !wait_full()) break;
         const float* bias = a.bias + (nb + a.nb_off) * a.BN;
         for (int j = 0; j < a.MT; ++j) {
             const int tile = j == 0 ? tile_c0 : tile_c1;
-            if (tile < 0) break;
+            if (tile < 0) { if (j == 0 && !wait_full()) return; break; }        // a pair's second CTA without a tile: its turn all the same
             const bool reused = ((j == 0 ? mask_c0 : mask_c1) >> mbit) & 1u;
             bool active, in_map;
             // write-back addressing, once per tile: piece k of this lane is the 16-byte part (lane & 3) of the pixel in
@@ -249,7 +248,7 @@ __device__ __forceinline__ void epilogue_loop(const TcArgs& a, SmemCtl* ctl, uin
             const uint32_t stg = smem_u32(ctl->stage[warp - 2]);
             const uint32_t rd = stg + (lane >> 2) * 80 + (lane & 3) * 16, mine = stg + lane * 80;
             fetch_add(c_begin);
-            if (ADD && !wait_full()) return;
+            if (j == 0 && !wait_full()) return;                  // the addresses are worked out while the accumulator is
             for (int c = c_begin; c < c_end; ++c) {
                 uint32_t r[32];
                 tmem_ld32(taddr + c * 32, r);
@@ -425,13 +424,11 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             };
             peek(blockIdx.x);
             const uint32_t tx = (uint32_t)(MT * a.a_bytes / DC_TILE_H * a.gpt + a.b_bytes);
-            if (a.early) {
-                if ((int)blockIdx.x < n_items) ahead = weights_ahead(tx, ((int)blockIdx.x % a.NB + a.nb_off) * a.BN);
-                enter();
-            }
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-                const int row0 = (item % a.NB + a.nb_off) * a.BN, c_off = item % a.NB / a.nb_group * a.c_group;
-                int sN[MT], xb[MT], yb[MT];
+            int row0 = 0, c_off = 0, sN[MT], xb[MT], yb[MT];
+            auto place = [&](int item) {                            // where the item's boxes lie
+                if (item >= n_items) return;
+                const int nb = item % a.NB;
+                row0 = (nb + a.nb_off) * a.BN; c_off = nb / a.nb_group * a.c_group;
 #pragma unroll
                 for (int j = 0; j < MT; ++j) {
                     const int tile = next[j];
@@ -440,6 +437,13 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     if (a.flat_rows) { sN[j] = xb[j] = 0; yb[j] = tile * a.flat_rows * a.sh; }
                     if (a.flat_images) { sN[j] = tile * a.flat_images; xb[j] = -a.pw; yb[j] = -a.ph; }
                 }
+            };
+            place(blockIdx.x);
+            if (a.early) {
+                if ((int)blockIdx.x < n_items) ahead = weights_ahead(tx, row0);
+                enter();
+            }
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
                 peek(item + gridDim.x);
                 order.walk([&](int c, int kx, int ky, int w) {
                     ok = mbar_wait_a(empty0 + r.off, r.phase ^ 1u, ctl, a.status);
@@ -457,6 +461,7 @@ k_conv_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                     r.next(r0, (uint32_t)a.stages, (uint32_t)stage_bytes);
                     return true;
                 });
+                place(item + gridDim.x);
             }
         }
         __syncwarp();
