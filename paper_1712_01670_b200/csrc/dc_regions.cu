@@ -304,6 +304,9 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
     const int X0 = tx * DC_TILE_W, Y0 = ty * DC_TILE_H;
     const int X1 = min(X0 + DC_TILE_W, a.Wo), Y1 = min(Y0 + DC_TILE_H, a.Ho);
     const dc_region* regs = a.regions + (size_t)s * a.max_regions;
+    // the first rectangles travel with their number (the list has room for max_regions)
+    dc_region first = empty_region();
+    if (lane < a.max_regions) first = regs[lane];
     // every rectangle of this stream has eroded away before this layer: nothing to test or copy
     const int n = (a.alive && a.alive[s] == 0) ? 0 : min(a.n_regions[s], a.max_regions);
     const size_t map_base = (size_t)s * a.Ho * a.Wo * a.px_bytes;
@@ -313,7 +316,7 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
         dc_region r = empty_region();
         int ix0 = 0, ix1 = 0, iy0 = 0, iy1 = 0;
         if (i < n) {
-            r = regs[i];
+            r = base == 0 ? first : regs[i];
             // Rectangles made by Step 5 and Table 2 lie inside the map on both sides.  One that does not (a caller's
             // own list) is not reused: neither side is ever addressed outside its map; the status word records it.
             const bool inside = r.x >= 0 && r.y >= 0 && r.sx >= 0 && r.sy >= 0 && r.w <= a.Wo && r.h <= a.Ho &&
@@ -344,11 +347,11 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
         if (hits == 0) continue;
         const int span_bytes = hit ? (ix1 - ix0) * a.px_bytes : 0;
         const int segs = (span_bytes + kSeg - 1) / kSeg, mine = hit ? (iy1 - iy0) * segs : 0;
-        int first = mine;                                               // inclusive sum over the lanes, then this lane's start
+        int begin = mine;                                               // inclusive sum over the lanes, then this lane's start
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, first, o); if (lane >= o) first += v; }
-        const int items = __shfl_sync(0xffffffffu, first, 31);
-        first -= mine;
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, begin, o); if (lane >= o) begin += v; }
+        const int items = __shfl_sync(0xffffffffu, begin, 31);
+        begin -= mine;
         const int src_y = iy0 - r.y + r.sy, src_x = ix0 - r.x + r.sx;   // cached position of (ix0, iy0)
         for (int i0 = part * 32; i0 < items && !cl.dead; i0 += 32 * a.parts) {
             const int it = i0 + lane;
@@ -356,9 +359,9 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
             int owner = 0;                                              // the lane whose rectangle segment `it` belongs to
             for (unsigned h = hits; h; h &= h - 1) {
                 const int k = __ffs(h) - 1;
-                if (it >= __shfl_sync(0xffffffffu, first, k)) owner = k;
+                if (it >= __shfl_sync(0xffffffffu, begin, k)) owner = k;
             }
-            const int o_first = __shfl_sync(0xffffffffu, first, owner), o_segs = max(1, __shfl_sync(0xffffffffu, segs, owner));
+            const int o_first = __shfl_sync(0xffffffffu, begin, owner), o_segs = max(1, __shfl_sync(0xffffffffu, segs, owner));
             const int o_span = __shfl_sync(0xffffffffu, span_bytes, owner);
             const int o_x = __shfl_sync(0xffffffffu, ix0, owner), o_y = __shfl_sync(0xffffffffu, iy0, owner);
             const int o_sx = __shfl_sync(0xffffffffu, src_x, owner), o_sy = __shfl_sync(0xffffffffu, src_y, owner);
@@ -543,25 +546,29 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
 {
     extern __shared__ uint8_t copy_smem[];
     CopyLane cl = copy_lane_setup(copy_smem);
-    dc_pdl_wait();
-    dc_pdl_release();
+    // The table was complete when the cache was created: a warp finds its layer and tile while the kernel before still runs (half a dozen
+    // loads one behind another; a pass in us before and so: small CNN, one
+    // stream, 86.4 and 85.8; every layer kind, 16 streams, 162.2 and 160.6).
     const int w = blockIdx.x * kCopyWarps + (threadIdx.x >> 5);
-    if (w >= total_warps) return;                       // no copy was issued by this warp
     int lo = 0, hi = n_cached - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (layers[mid].first_warp <= w) lo = mid; else hi = mid - 1;
+        if (__ldg(&layers[mid].first_warp) <= w) lo = mid; else hi = mid - 1;
     }
     const ClassifyLayer& L = layers[lo];
     ClassifyArgs a;
     a.regions = L.regions; a.n_regions = L.alive; a.max_regions = max_regions;     // the rectangles left at this layer
-    a.prev = L.map[cur]; a.out = L.map[cur ^ 1];
+    const uint8_t* const m0 = L.map[0]; const uint8_t* const m1 = L.map[1];
+    a.prev = cur ? m1 : m0; a.out = (uint8_t*)(cur ? m0 : m1);
     a.Ho = L.Ho; a.Wo = L.Wo; a.px_bytes = L.px_bytes; a.tiles_x = L.tiles_x; a.tiles_y = L.tiles_y; a.S = S;
     a.gpr = L.gpr; a.gpt = L.gpt; a.n_tiles = 0;
     a.masks = L.masks; a.dirty_list = L.dirty_list; a.dirty_count = L.dirty_count; a.reuse_px = L.reuse_px;
     a.alive = L.alive; a.reused_total = L.reused_total; a.status = L.status;
     a.parts = L.parts; a.running = nullptr;
     const int u = w - L.first_warp, tile = u / a.parts, part = u - tile * a.parts;
+    dc_pdl_wait();
+    dc_pdl_release();
+    if (w >= total_warps) return;                       // no copy was issued by this warp
     if (a.gpr > 0) classify_tile_flat(a, tile, part, threadIdx.x & 31, cl);
     else classify_tile(a, tile, part, threadIdx.x & 31, cl);
     rs_wait_all();
