@@ -15,8 +15,9 @@
 // Work item: one dirty 16 x 8 tile (128 pixels = M) times BN channels; persistent CTAs, one per SM.  16 warps:
 //   0      weights: one bulk copy per (32 channels, kernel row), packed as the MMA reads them
 //   1      MMA issue
-//   2-9    the sums: tensor memory -> registers after every kernel row; bias, ReLU, store of the pixels not reused (a warp: 32 pixels,
-//          half of the channels)
+//   2-9    the sums: tensor memory -> registers after every kernel row; bias, ReLU, store of the pixels not reused.  A warp has 32 pixels and
+//          half of the channels, or (TURNS: more items than SMs) all of them of every other item: four warps empty the accumulators of one
+//          item while the other four finish the one before.
 //   10-15  input: the (16 + kh - 1) x (8 + kw - 1) patch of 32 channels, split into pieces on its way to shared memory (planes of
 //          8 channels, 16 bytes a pixel: every tap is a shifted view of it, as in the patch scheme of the bf16 kernels)
 // What bounds it: the tensor pipe (see f32_bn), and beside it the sums' way out: without MMAs 0.8 of the time, without the stores 0.9.
@@ -40,7 +41,7 @@ constexpr int kSumWarps = 8, kSplitWarps = 6, kThreadsF = 32 * (2 + kSumWarps + 
 constexpr int kStagesF = 8;                       // weight stages at most
 constexpr int kChF = 32;                          // input channels per patch
 constexpr int kRowsPerDrain1 = 3;                 // 1 x 1 kernels: patches between two drains (6 steps of 16 channels, as a row of a 3 x 3 kernel)
-constexpr int kTileFlags = 8;                     // more than the items between the splitting warps and the epilogue (at most 5)
+constexpr int kTileFlags = 8;                     // more than the items between the splitting warps and the epilogue (at most 6)
 constexpr float kSmallSum = 0x1p-100f;            // below it the tensor core's cuts at 2^-149 may count for more than an FMA's roundings
 constexpr unsigned long long kWaitLimitF = 2000000000ull;
 
@@ -70,7 +71,7 @@ __host__ __device__ constexpr int f32_stage_bytes(int BN, int KW)
 }
 
 struct __align__(16) CtlF {
-    unsigned long long full[kStagesF], empty[kStagesF], a_full[2], a_empty[2], t_full[2], t_empty[2];
+    unsigned long long full[kStagesF], empty[kStagesF], a_full[2], a_empty[2], t_full[4], t_empty[2];     // t_full: [2 groups of sum warps][2 sets]
     uint32_t tmem_base;
     volatile int abort_flag;
     unsigned long long wait_ns;
@@ -227,7 +228,7 @@ __device__ __noinline__ void fma_pixels(const F32Args& a, uint32_t stage, int s,
     __syncwarp();
 }
 
-template <int BN, int KW>
+template <int BN, int KW, bool TURNS>
 __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant__ F32Args a)
 {
     constexpr int PW = DC_TILE_W + KW - 1, PX = PW * (DC_TILE_H + KW - 1), PLANE = PX * 16, PIECE = 4 * PLANE, A_SLOT = 3 * PIECE;
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
         for (int i = 0; i < a.stages; ++i) { mbar_init(&ctl->full[i], 1); mbar_init(&ctl->empty[i], 1); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&ctl->a_full[i], kSplitWarps); mbar_init(&ctl->a_empty[i], 1);
-            mbar_init(&ctl->t_full[i], 1); mbar_init(&ctl->t_empty[i], kSumWarps);
+            mbar_init(&ctl->t_full[i], 1); mbar_init(&ctl->t_full[2 + i], 1); mbar_init(&ctl->t_empty[i], TURNS ? kSumWarps / 2 : kSumWarps);
         }
         for (int i = 0; i < kTileFlags; ++i) ctl->odd[i] = 0;
         ctl->abort_flag = 0;
@@ -267,6 +268,9 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
     const uint32_t t_full0 = smem_u32(&ctl->t_full[0]), t_empty0 = smem_u32(&ctl->t_empty[0]);
     auto k_steps = [&](int cc) { return cc + 1 < a.chunks ? kChF / 16 : a.ks_last; };
+    // All of a layer's weights in the ring: they stay there, sent once.  Shared memory's bandwidth is what bounds a kernel row, and a fifth of
+    // that went into weights that were there before (32 -> 32 at 227 x 227, 24 streams: 133 us so, 129 resident).
+    const bool resident = a.NB == 1 && a.chunks * KW <= a.stages;
 
     if (warp == 0) {
         // ---------------- weights ----------------
@@ -308,6 +312,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
                         }
                         r.next(r0, (uint32_t)a.stages, (uint32_t)B_STAGE);
                     }
+                if (resident) break;
             }
             // on an abort: give the copies already issued a bounded chance to land before the CTA exits
             if (!ok) { const unsigned long long t0 = now_ns(); while (now_ns() - t0 < 2000000ull) { } }
@@ -323,16 +328,18 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
             const uint32_t i3 = f_idesc(3 * BN), i2 = f_idesc(2 * BN), i1 = f_idesc(BN);
             RingPos rb, ra;
             rb.start(b0, (uint32_t)a.stages); ra.start(a0, 2);
-            uint32_t set = 0, set_ph = 0;
+            uint32_t set = 0, set_ph = 0, group = 0;                           // group: of sum warps, whose turn the item is
             bool ok = true;
-            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+            for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, group ^= TURNS ? 2u : 0u) {
                 int rows = 0;                                              // kernel rows in the accumulator set
+                const bool fresh = !resident || item == (int)blockIdx.x;   // weights to wait for
+                if (resident) rb.start(b0, (uint32_t)a.stages);
                 for (int cc = 0; cc < a.chunks && ok; ++cc) {
                     ok = f_wait(a_full0 + ra.off, ra.phase, ctl, a.status);
                     const bool two = k_steps(cc) == 2;
                     for (int ky = 0; ky < KW && ok; ++ky) {
                         if (rows == 0) ok = f_wait(t_empty0 + 8u * set, set_ph ^ 1u, ctl, a.status);
-                        ok = ok && f_wait(full0 + rb.off, rb.phase, ctl, a.status);
+                        if (fresh) ok = ok && f_wait(full0 + rb.off, rb.phase, ctl, a.status);
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t d = tmem_base + set * kSet, at = ra.data + (uint32_t)(ky * PW);
@@ -347,10 +354,10 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
                                     umma_chunk(d + BN, al + (PIECE >> 4), a_hi, 0, bl, b_hi, 0, i2, 1u, 1);
                                     umma_chunk(d + 2 * BN, al + 2 * (PIECE >> 4), a_hi, 0, bl, b_hi, 0, i1, 1u, 1);
                                 }
-                        umma_commit_at(empty0 + rb.off);
+                        if (!resident) umma_commit_at(empty0 + rb.off);
                         rb.next(b0, (uint32_t)a.stages, (uint32_t)B_STAGE >> 4);
                         if (++rows == kRows || (cc + 1 == a.chunks && ky + 1 == KW)) {
-                            umma_commit_at(t_full0 + 8u * set);
+                            umma_commit_at(t_full0 + 8u * (group + set));
                             rows = 0;
                             set ^= 1u;
                             if (set == 0) set_ph ^= 1u;
@@ -364,27 +371,31 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
         __syncwarp();
     } else if (warp < 2 + kSumWarps) {
         // ---------------- sums, bias, ReLU, store ----------------
-        constexpr int CH = BN / 2;                                        // channels of this thread's pixel
-        const int q = warp & 3, half = (warp - 2) >> 2, m = q * 32 + lane, row = m / DC_TILE_W, col = m % DC_TILE_W;
+        constexpr int HALF = BN / 2, CH = TURNS ? BN : HALF;              // channels of this thread's pixel; those whose outcome is decided together
+        const int q = warp & 3, group = (warp - 2) >> 2, half = TURNS ? 0 : group, m = q * 32 + lane, row = m / DC_TILE_W, col = m % DC_TILE_W;
         const uint32_t lanes = (uint32_t)(q * 32) << 16;
         const int drains = (a.chunks * KW + kRows - 1) / kRows;
         auto tile_of = [&](int item) { return item < n_items ? __ldcg(a.tile_list + item / a.NB) : 0; };
-        int next = tile_of(blockIdx.x);
+        const int first = TURNS ? group : 0, every = TURNS ? 2 : 1;       // of the CTA's items, this warp's
+        int next = tile_of(blockIdx.x + first * gridDim.x);
         if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
         const uint32_t stage = smem_u32(ctl + 1) + (warp - 2) * f32_stage_bytes(BN, KW);
-        uint32_t set = 0, set_ph = 0;
-        int seq = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++seq) {
+        const uint32_t t_full = t_full0 + (TURNS ? 16u * group : 0u);
+        uint32_t phases = 0;                                               // bit s: of set s, for this group
+        int seq = first;
+        for (int item = blockIdx.x + first * gridDim.x; item < n_items; item += every * gridDim.x, seq += every) {
             const int tile = next;
-            next = tile_of(item + gridDim.x);
+            next = tile_of(item + every * gridDim.x);
             const uint32_t word = __ldcg(a.masks + (size_t)tile * 4 + (row >> 2));
             float sum[CH];
 #pragma unroll
             for (int j = 0; j < CH; ++j) sum[j] = 0.f;
             bool ok = true;
-            for (int u = 0; u < drains; ++u) {
-                ok = f_wait_warp(t_full0 + 8u * set, set_ph, lane, ctl, a.status);
+            uint32_t set = (uint32_t)(seq * drains) & 1u;
+            for (int u = 0; u < drains; ++u, set ^= 1u) {
+                ok = f_wait_warp(t_full + 8u * set, (phases >> set) & 1u, lane, ctl, a.status);
                 if (!ok) break;
+                phases ^= 1u << set;
                 tc_fence_after();
                 const uint32_t d = tmem_base + lanes + set * kSet + half * CH;
 #pragma unroll
@@ -403,49 +414,52 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl->t_empty[set]);
-                set ^= 1u;
-                if (set == 0) set_ph ^= 1u;
             }
             if (!ok) break;
             const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
             const int y = ty * DC_TILE_H + row, x = tx * DC_TILE_W + col;
-            const bool active = y < a.Ho && x < a.Wo && !((word >> (8 * (row & 3) + col)) & 1u);
-            const int nb = item % a.NB, grp = nb / a.nb_g, c0 = (nb - grp * a.nb_g) * BN + half * CH, n = min(CH, a.Cog - c0);
-            float* const tile_out = a.out + (((size_t)s * a.Ho + ty * DC_TILE_H) * a.Wo + tx * DC_TILE_W) * a.Co + grp * a.Cog + c0;
-            const float* bias = a.bias + grp * a.Cog + c0;
-            float most = 0.f, least = INFINITY;                            // magnitudes; NaN counts among the largest
+            const bool active = y < a.Ho && x < a.Wo && !((word >> (8 * (row & 3) + col)) & 1u), odd = ctl->odd[seq % kTileFlags] == seq + 1;
+            const int nb = item % a.NB, grp = nb / a.nb_g;
 #pragma unroll
-            for (int j = 0; j < CH; j += 2) { most = max3_abs(most, sum[j], sum[j + 1]); least = min3_abs(least, sum[j], sum[j + 1]); }
-            bool small = false;
-            if (least < kSmallSum) {
+            for (int h = 0; h < CH; h += HALF) {
+                const int c0 = (nb - grp * a.nb_g) * BN + half * HALF + h, n = min(HALF, a.Cog - c0);
+                float* const tile_out = a.out + (((size_t)s * a.Ho + ty * DC_TILE_H) * a.Wo + tx * DC_TILE_W) * a.Co + grp * a.Cog + c0;
+                const float* bias = a.bias + grp * a.Cog + c0;
+                float most = 0.f, least = INFINITY;                        // magnitudes; NaN counts among the largest
 #pragma unroll
-                for (int j = 0; j < CH; ++j) small = small || (fabsf(sum[j]) < kSmallSum && sum[j] != 0.f);
-            }
-            const bool redo = active && (!(most < INFINITY) || small || ctl->odd[seq % kTileFlags] == seq + 1);
-            // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
-            // warp touched 32 lines, and the stores took as long as the MMAs)
-            const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
-            const int part = lane % (STAGE_CH / 4);
+                for (int j = 0; j < HALF; j += 2) { most = max3_abs(most, sum[h + j], sum[h + j + 1]); least = min3_abs(least, sum[h + j], sum[h + j + 1]); }
+                bool small = false;
+                if (least < kSmallSum) {
 #pragma unroll
-            for (int c = 0; c < CH; c += STAGE_CH) {
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < STAGE_CH; j += 4)
-                    sts128(stage + lane * STAGE_PITCH + j * 4, __float_as_uint(sum[c + j]), __float_as_uint(sum[c + j + 1]), __float_as_uint(sum[c + j + 2]), __float_as_uint(sum[c + j + 3]));
-                __syncwarp();
-                if (c + 4 * part >= n) continue;                           // channels come in fours
-                const float* pb = bias + c + 4 * part;
-                const float b0 = __ldg(pb), b1 = __ldg(pb + 1), b2 = __ldg(pb + 2), b3 = __ldg(pb + 3);
-#pragma unroll
-                for (int i = 0; i < STAGE_CH / 4; ++i) {
-                    const int p = i * (128 / STAGE_CH) + lane / (STAGE_CH / 4);
-                    const uint4 w = lds128(stage + p * STAGE_PITCH + part * 16);
-                    float4 v = make_float4(__uint_as_float(w.x) + b0, __uint_as_float(w.y) + b1, __uint_as_float(w.z) + b2, __uint_as_float(w.w) + b3);
-                    if (a.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
-                    if ((todo >> p) & 1u) *(float4*)(tile_out + ((size_t)(q * 4 + p / 8) * a.Wo + p % 8) * a.Co + c + 4 * part) = v;
+                    for (int j = 0; j < HALF; ++j) small = small || (fabsf(sum[h + j]) < kSmallSum && sum[h + j] != 0.f);
                 }
+                const bool redo = active && (!(most < INFINITY) || small || odd);
+                // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
+                // warp touched 32 lines, and the stores took as long as the MMAs)
+                const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
+                const int part = lane % (STAGE_CH / 4);
+#pragma unroll
+                for (int c = 0; c < HALF; c += STAGE_CH) {
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < STAGE_CH; j += 4)
+                        sts128(stage + lane * STAGE_PITCH + j * 4, __float_as_uint(sum[h + c + j]), __float_as_uint(sum[h + c + j + 1]),
+                               __float_as_uint(sum[h + c + j + 2]), __float_as_uint(sum[h + c + j + 3]));
+                    __syncwarp();
+                    if (c + 4 * part >= n) continue;                       // channels come in fours
+                    const float* pb = bias + c + 4 * part;
+                    const float b0 = __ldg(pb), b1 = __ldg(pb + 1), b2 = __ldg(pb + 2), b3 = __ldg(pb + 3);
+#pragma unroll
+                    for (int i = 0; i < STAGE_CH / 4; ++i) {
+                        const int p = i * (128 / STAGE_CH) + lane / (STAGE_CH / 4);
+                        const uint4 w = lds128(stage + p * STAGE_PITCH + part * 16);
+                        float4 v = make_float4(__uint_as_float(w.x) + b0, __uint_as_float(w.y) + b1, __uint_as_float(w.z) + b2, __uint_as_float(w.w) + b3);
+                        if (a.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+                        if ((todo >> p) & 1u) *(float4*)(tile_out + ((size_t)(q * 4 + p / 8) * a.Wo + p % 8) * a.Co + c + 4 * part) = v;
+                    }
+                }
+                if (__any_sync(0xffffffffu, redo)) fma_pixels<BN, KW>(a, stage, s, ty * DC_TILE_H + q * 4, tx * DC_TILE_W, grp, c0, redo);
             }
-            if (__any_sync(0xffffffffu, redo)) fma_pixels<BN, KW>(a, stage, s, ty * DC_TILE_H + q * 4, tx * DC_TILE_W, grp, c0, redo);
         }
     } else {
         // ---------------- input patches, split into pieces ----------------
@@ -648,7 +662,7 @@ int dc_settle_weights_f32(dc_cache* c)
 // A CTA takes its SM whole (512 threads of 128 registers), also where the next frame is matched beside it: a VGG-16 trunk in float32 on full-HD
 // frames with the next one announced takes 1.07, 3.2 and 6.7 ms a pass for 4, 16 and 32 streams so, and took 3.1, 10.1 and 19.5 on
 // k_conv_simt, whose CTAs leave the search room.
-template <int BN, int KW>
+template <int BN, int KW, bool TURNS>
 static int launch_f32(dc_cache* c, F32Args& a, int grid)
 {
     constexpr int a_total = 2 * 3 * 4 * 16 * (DC_TILE_W + KW - 1) * (DC_TILE_H + KW - 1), stage = KW * 4 * 3 * BN * 16, staging = kSumWarps * f32_stage_bytes(BN, KW);
@@ -657,8 +671,8 @@ static int launch_f32(dc_cache* c, F32Args& a, int grid)
     a.stages = room > kStagesF ? kStagesF : room;
     const size_t smem = (size_t)a_total + (size_t)a.stages * stage + sizeof(CtlF) + staging + 128;
     static dc_once_per_device attr_set;
-    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_conv_f32<BN, KW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    DC_CUDA(dc_launch_pdl(k_conv_f32<BN, KW>, dim3((unsigned)grid), kThreadsF, smem, c->stream, a));
+    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_conv_f32<BN, KW, TURNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    DC_CUDA(dc_launch_pdl(k_conv_f32<BN, KW, TURNS>, dim3((unsigned)grid), kThreadsF, smem, c->stream, a));
     return DC_OK;
 }
 
@@ -682,7 +696,12 @@ int dc_launch_conv_f32(dc_cache* c, int layer, const void* in, void* out, const 
     const int grid = items > c->num_sms ? c->num_sms : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
     c->launches += 1;
-    if (L.d.kw == 1) return BN == 64 ? launch_f32<64, 1>(c, a, grid) : launch_f32<32, 1>(c, a, grid);
-    if (L.d.kw == 3) return BN == 64 ? launch_f32<64, 3>(c, a, grid) : launch_f32<32, 3>(c, a, grid);
-    return BN == 64 ? launch_f32<64, 5>(c, a, grid) : launch_f32<32, 5>(c, a, grid);
+    // Several items of 32 channels per CTA: TURNS.  With one each its eight warps finish it sooner together; sums of 64 channels are more than a
+    // thread's registers hold beside the rest (32 -> 32 at 227 x 227, 24 streams, 129 us without and 121 with it; 64-channel blocks 85.6 and 88).
+    const bool turns = BN == 32 && items > c->num_sms;
+#define DC_F32(kw) return turns ? launch_f32<32, kw, true>(c, a, grid) : BN == 64 ? launch_f32<64, kw, false>(c, a, grid) : launch_f32<32, kw, false>(c, a, grid)
+    if (L.d.kw == 1) DC_F32(1);
+    if (L.d.kw == 3) DC_F32(3);
+    DC_F32(5);
+#undef DC_F32
 }
