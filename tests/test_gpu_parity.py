@@ -1701,6 +1701,40 @@ def test_conv_fp32_on_tensor_cores_with_values_that_do_not_split():
         dc.close()
 
 
+@pytest.mark.parametrize("cin,k,S", [(32, 3, 24), (32, 3, 10), (96, 3, 24), (16, 5, 24), (32, 1, 24), (200, 1, 11)])
+def test_conv_fp32_items_in_turns(cin, k, S):
+    """Layers with several items per CTA, finished by two groups of warps in turn, with weights that stay in shared memory (one patch of channels)
+    and that do not: stream by stream the bits of one stream alone, where every item has an SM, also where pixels are left to FMAs or reused."""
+    g = rng(cin + k)
+    H, W = 48, 39
+    nb = nets.NetBuilder(H, W)
+    nb.conv(nb.conv(-1, cin, 1, 1, 0), 32, k, 1, k // 2, 0)
+    wts = g.normal(0, np.sqrt(2.0 / (k * k * cin)), size=(32, k, k, cin)).astype(np.float32)
+    bias = g.normal(0, 0.1, size=32).astype(np.float32)
+    x = g.normal(size=(S, H, W, cin)).astype(np.float32)
+    x[::3, 5, 7, 1], x[1::4, 33, 20, 0] = np.inf, np.float32(2.0 ** -120 * 1.2345678)
+    x[::2, 16:32, 8:16] = 0.0
+    x, prev = torch.from_numpy(x).cuda(), torch.from_numpy(g.normal(size=(S, H, W, 32)).astype(np.float32)).cuda()
+    regs, n = torch.zeros((S, 4, 6), dtype=torch.int32, device="cuda"), torch.ones(S, dtype=torch.int32, device="cuda")
+    regs[:, 0] = torch.tensor([3, 2, 30, 21, 1, 4], dtype=torch.int32)
+
+    def run(lo, hi):
+        dc = DeepCache(W, H, nb.layers, [np.zeros((cin, 1, 1, 3), np.float32), wts], [np.zeros(cin, np.float32), bias], n_streams=hi - lo, block=16,
+                       search_range=4, dtype=B.DC_FP32, max_regions=4)
+        try:
+            outs = [dc.conv_partial(1, x[lo:hi]), dc.conv_partial(1, x[lo:hi], prev[lo:hi], regs[lo:hi], n[lo:hi])]
+            assert dc.status() == B.DC_OK
+            return outs
+        finally:
+            dc.close()
+
+    full, part = run(0, S)
+    assert (~torch.isfinite(full)).any()
+    for s in range(S):
+        one_full, one_part = run(s, s + 1)
+        assert torch.allclose(full[s], one_full[0], rtol=0, atol=0, equal_nan=True) and torch.allclose(part[s], one_part[0], rtol=0, atol=0, equal_nan=True)
+
+
 @pytest.mark.parametrize("relu", [0, 1])
 @pytest.mark.parametrize("cin,cout,k,H,W,S,groups", [(32, 64, 3, 48, 40, 1, 1), (64, 32, 1, 33, 21, 2, 1), (40, 72, 5, 30, 22, 2, 2), (64, 64, 3, 113, 113, 4, 1)])
 def test_conv_fp32_sums_beyond_the_largest_float(cin, cout, k, H, W, S, groups, relu, monkeypatch):
