@@ -380,10 +380,11 @@ __global__ void k_lrn(const T* in, int H, int W, int C, int S, int r, float alph
 
 // The same for 16-byte vectors of channels, R known.  A thread takes Y rows of one column, so that the squares of a row are
 // summed along x once for all the outputs above and below it, and beta = 3/4 (the default) takes two reciprocal square
-// roots (inverse_3_4).  What bounds it: instructions (some 200 per vector of eight channels) and the loads behind them.
-// us with a thread per output, two rounded square roots and a division, and so (16 streams):
-//   32 channels at 128 x 160, R = 1           43, 24
-//   64 channels at 32 x 40, R = 2 (Y = 1)     14, 10
+// roots (inverse_3_4); sums and Newton steps two floats to an instruction.  What bounds it: the loads of a strip, all in flight at once, then
+// some 150 instructions per vector; four CTAs per SM hide the one behind the other (R = 2: two, whose registers hold its loads).
+// us with a thread per output, two rounded square roots and a division; one float to an instruction; and so (16 streams):
+//   32 channels at 128 x 160, R = 1           43, 23, 20.6
+//   64 channels at 32 x 40, R = 2 (Y = 1)     14, 9.5, 8.6
 template <typename T> struct Unpack;
 template <> struct Unpack<float> {
     static __device__ __forceinline__ void get(uint4 v, float* f) { f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y); f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w); }
@@ -405,21 +406,44 @@ template <> struct Unpack<__nv_bfloat16> {
     }
 };
 
+// Two floats at a time (one instruction, each rounded as on its own).
+#define DC_PAIR_OP(name, op)                                                                                                              \
+    __device__ __forceinline__ float2 name(float2 a, float2 b)                                                                            \
+    {                                                                                                                                     \
+        float2 r;                                                                                                                         \
+        asm("{\n\t.reg .b64 x, y, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t" op ".rn.f32x2 w, x, y;\n\tmov.b64 {%0, %1}, w;\n\t}" \
+            : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                                              \
+        return r;                                                                                                                         \
+    }
+DC_PAIR_OP(add2, "add")
+DC_PAIR_OP(mul2, "mul")
+#undef DC_PAIR_OP
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 r;
+    asm("{\n\t.reg .b64 x, y, z, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\tfma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+__device__ __forceinline__ float2 pair_of(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float min3_nan(float a, float b, float c) { float r; asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
+__device__ __forceinline__ float max3_nan(float a, float b, float c) { float r; asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
+
 // d^(-3/4): d^(-1/2) and then (d^(1/2))^(-1/2), each with one Newton step (relative error up to 1.5 * 2^-23 together; up to
 // 1.9 with the two rounded square roots and the division that they replace).
-__device__ __forceinline__ float rsqrt_step(float d)
+__device__ __forceinline__ float2 rsqrt_step(float2 d)
 {
-    const float y = rsqrtf(d), e = fmaf(-d * y, y, 1.f);
-    return fmaf(0.5f * y, e, y);
+    const float2 y = make_float2(rsqrtf(d.x), rsqrtf(d.y)), e = fma2(mul2(make_float2(-d.x, -d.y), y), y, pair_of(1.f));
+    return fma2(mul2(pair_of(0.5f), y), e, y);
 }
-__device__ __forceinline__ float inverse_3_4(float d)
+__device__ __forceinline__ float2 inverse_3_4(float2 d)
 {
-    const float y = rsqrt_step(d);
-    return y * rsqrt_step(d * y);
+    const float2 y = rsqrt_step(d);
+    return mul2(y, rsqrt_step(mul2(d, y)));
 }
 
 template <typename T, int R, int Y>
-__global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, unsigned cv, float alpha_n2, float beta, float kappa, unsigned strips, unsigned total, uint4* out,
+__global__ void __launch_bounds__(256, R == 1 ? 4 : 2) k_lrn_vec(const uint4* in, int H, int W, unsigned cv, float alpha_n2, float beta, float kappa, unsigned strips, unsigned total, uint4* out,
                                                  const uint32_t* masks, int tiles_x, int tiles_y)
 {
     constexpr int N = Vec16<T>::N;
@@ -443,11 +467,11 @@ __global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, 
         if (todo == 0) continue;
         const size_t at = ((size_t)s * H + y0) * W + x;
         const uint4* base = in + at * cv + c;
-        float sum[Y][N];
+        float2 sum[Y][N / 2];
 #pragma unroll
         for (int k = 0; k < Y; ++k)
 #pragma unroll
-            for (int j = 0; j < N; ++j) sum[k][j] = 0.f;
+            for (int j = 0; j < N / 2; ++j) sum[k][j] = pair_of(0.f);
         uint4 v[Y + 2 * R][2 * R + 1], mid[Y];                   // the strip's input: all loads at once
 #pragma unroll
         for (int r = 0; r < Y + 2 * R; ++r)
@@ -458,22 +482,22 @@ __global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, 
             }
 #pragma unroll
         for (int r = 0; r < Y + 2 * R; ++r) {
-            float row[N];
+            float2 row[N / 2];
 #pragma unroll
-            for (int j = 0; j < N; ++j) row[j] = 0.f;
+            for (int j = 0; j < N / 2; ++j) row[j] = pair_of(0.f);
 #pragma unroll
             for (int dx = 0; dx <= 2 * R; ++dx) {
                 float f[N];
                 Unpack<T>::get(v[r][dx], f);
 #pragma unroll
-                for (int j = 0; j < N; ++j) row[j] = fmaf(f[j], f[j], row[j]);
+                for (int j = 0; j < N / 2; ++j) { const float2 g = make_float2(f[2 * j], f[2 * j + 1]); row[j] = fma2(g, g, row[j]); }
             }
             if (r >= R && r < Y + R) mid[r - R] = v[r][R];
 #pragma unroll
             for (int k = 0; k < Y; ++k)
                 if (r - R - k >= -R && r - R - k <= R) {
 #pragma unroll
-                    for (int j = 0; j < N; ++j) sum[k][j] += row[j];
+                    for (int j = 0; j < N / 2; ++j) sum[k][j] = add2(sum[k][j], row[j]);
                 }
         }
 #pragma unroll
@@ -481,15 +505,21 @@ __global__ void __launch_bounds__(256) k_lrn_vec(const uint4* in, int H, int W, 
             if (!((todo >> k) & 1u)) continue;
             float f[N];
             Unpack<T>::get(mid[k], f);
-            bool plain = beta == 0.75f;
+            float least = INFINITY, most = -INFINITY;                // NaN if one is
 #pragma unroll
-            for (int j = 0; j < N; ++j) { sum[k][j] = fmaf(alpha_n2, sum[k][j], kappa); plain = plain && sum[k][j] > 1e-30f && sum[k][j] < 1e30f; }
-            if (plain) {
+            for (int j = 0; j < N / 2; ++j) {
+                sum[k][j] = fma2(pair_of(alpha_n2), sum[k][j], pair_of(kappa));
+                least = min3_nan(least, sum[k][j].x, sum[k][j].y); most = max3_nan(most, sum[k][j].x, sum[k][j].y);
+            }
+            if (beta == 0.75f && least > 1e-30f && most < 1e30f) {
 #pragma unroll
-                for (int j = 0; j < N; ++j) f[j] *= inverse_3_4(sum[k][j]);
+                for (int j = 0; j < N / 2; ++j) {
+                    const float2 o = mul2(make_float2(f[2 * j], f[2 * j + 1]), inverse_3_4(sum[k][j]));
+                    f[2 * j] = o.x; f[2 * j + 1] = o.y;
+                }
             } else {
 #pragma unroll
-                for (int j = 0; j < N; ++j) f[j] *= powf(sum[k][j], -beta);
+                for (int j = 0; j < N / 2; ++j) { f[2 * j] *= powf(sum[k][j].x, -beta); f[2 * j + 1] *= powf(sum[k][j].y, -beta); }
             }
             out[(at + (size_t)k * W) * cv + c] = Unpack<T>::put(f);
         }
