@@ -640,7 +640,9 @@ static int ensure_lookahead_stream(dc_cache* c)
     DC_CUDA(cudaEventCreateWithFlags(&c->ev_key, cudaEventDisableTiming));
     DC_CUDA(cudaEventCreateWithFlags(&c->ev_match, cudaEventDisableTiming));
     DC_CUDA(cudaEventRecord(c->ev_key, c->stream));     // first use: everything enqueued so far
-    // tables of their own for the announced frame's rectangles; without the memory for them propagation stays with the inference
+    // tables of their own for the announced frame's rectangles; without the memory for them propagation stays with the inference, as it does
+    // where the matcher is large
+    if (matcher_is_large(c)) return DC_OK;
     const size_t before = c->bytes;
     dc_match_set m = c->mset[1];
     m.table = m.live = nullptr; m.dirty_count = m.reuse_px = nullptr; m.classify_table = nullptr;
@@ -683,7 +685,7 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
         // The rectangles through the layers too, unless the matcher is large: the walk wants much of an SM's shared memory and would wait
         // between the convolutions for it.  A pass in us, propagated by the inference and so: ResNet-50, one stream, 336 and 326; VGG, 6 streams of
         // 720p from host memory, 417 and 410; small CNN, 4 streams, 174 and 171; 24 streams of ResNet-50 and more the same.
-        c->la_propagated = rc == DC_OK && own_tables(c) && !matcher_is_large(c);
+        c->la_propagated = rc == DC_OK && own_tables(c);
         if (c->la_propagated) rc = dc_launch_propagate(c, c->regions0, c->n_regions, c->n_layers, true, nullptr, 0, nullptr);
         dc_use_match_set(c, main_set);
     } else {

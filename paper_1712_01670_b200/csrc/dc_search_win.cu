@@ -83,7 +83,7 @@ __device__ __forceinline__ void stage_window(const dc_win_args& a, const Tile& t
         if (x + 4 <= 0 || x >= a.W) continue;
         uint32_t* dst = win + (first_row - y0) * a.win_pitch + c;
         const uint8_t* p = prev + (ptrdiff_t)first_row * (ptrdiff_t)a.prev_pitch + (ptrdiff_t)x * 3;
-        if (p - 3 >= a.prev && prev + (ptrdiff_t)y_hi * (ptrdiff_t)a.prev_pitch + (ptrdiff_t)x * 3 + 16 <= a.prev_end) {
+        if ((const uint8_t*)((uintptr_t)p & ~(uintptr_t)3) >= a.prev && prev + (ptrdiff_t)y_hi * (ptrdiff_t)a.prev_pitch + (ptrdiff_t)x * 3 + 16 <= a.prev_end) {
 #pragma unroll 3
             for (int y = first_row; y <= y_hi; y += row_step, p += row_step * a.prev_pitch, dst += row_step * a.win_pitch) {
                 const uint32_t* q = (const uint32_t*)((uintptr_t)p & ~(uintptr_t)3);
