@@ -640,14 +640,30 @@ static int ensure_lookahead_stream(dc_cache* c)
     DC_CUDA(cudaEventCreateWithFlags(&c->ev_key, cudaEventDisableTiming));
     DC_CUDA(cudaEventCreateWithFlags(&c->ev_match, cudaEventDisableTiming));
     DC_CUDA(cudaEventRecord(c->ev_key, c->stream));     // first use: everything enqueued so far
-    // tables of their own for the announced frame's rectangles; without the memory for them propagation stays with the inference, as it does
-    // where the matcher is large
-    if (matcher_is_large(c)) return DC_OK;
+    return DC_OK;
+}
+
+static bool captured(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) { cudaGetLastError(); return true; }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// Tables of their own for the announced frame's rectangles.  Without the memory for them, and in calls that a capture records (which must not
+// allocate), propagation stays with the inference, as it does where the matcher is large.  While the second set is the current one, the
+// inference in flight may read the tables that both share: they part when the first is.  Another thread's capture is none of this call's.
+static void ensure_lookahead_tables(dc_cache* c)
+{
+    if (c->la_tables_tried || c->mset_cur != 0 || matcher_is_large(c) || captured(c->stream) || captured(c->la_stream)) return;
+    c->la_tables_tried = true;
     const size_t before = c->bytes;
     dc_match_set m = c->mset[1];
     m.table = m.live = nullptr; m.dirty_count = m.reuse_px = nullptr; m.classify_table = nullptr;
     cudaStream_t main_stream = c->stream;
-    c->stream = c->la_stream;                           // zeroed there, where they are written first
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    c->stream = c->la_stream;                           // written there, where they are first used
     const bool ok = alloc_tables(c, m) == DC_OK && dc_build_classify_table(c, m) == DC_OK;
     c->stream = main_stream;
     if (ok) {
@@ -657,7 +673,7 @@ static int ensure_lookahead_stream(dc_cache* c)
         free_tables(m);
         c->bytes = before;
     }
-    return DC_OK;
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
@@ -666,6 +682,7 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     if (!c->executable || !c->key_valid) return DC_ERR_STATE;       // needs a frame to match against
     DC_TRY(ensure_lookahead_stream(c));
     DC_TRY(cancel_lookahead(c));
+    ensure_lookahead_tables(c);
     // Everything the side stream touches is free once the main stream has passed the frame copy of the last
     // dc_infer_frame, dc_match_blocks or dc_cache_set_key (mark_key): the third key buffer was last read two frames ago, and the
     // match set that the current inference does not read was last read by the frame before it.  Waiting for

@@ -102,7 +102,7 @@ struct dc_cache {
     int mset_cur;
     cudaStream_t la_stream;         // dc_lookahead_frame: matcher of the next frame beside the current inference
     cudaEvent_t ev_key, ev_match;   // main stream: frame copied in; side stream: lookahead finished
-    const uint8_t* la_frame; size_t la_pitch; bool la_matched, la_propagated;
+    const uint8_t* la_frame; size_t la_pitch; bool la_matched, la_propagated, la_tables_tried;
     bool last_refreshed;
     bool overlap_mode;              // the last frame was looked ahead: the next one's matching will run beside this inference
     void* classify_table; int n_cached, classify_warps;   // all cached layers' classification in one launch (dc_regions.cu)

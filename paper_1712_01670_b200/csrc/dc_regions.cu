@@ -615,7 +615,7 @@ int dc_build_classify_table(dc_cache* c, dc_match_set& m)
     int rc = DC_OK;
     if (k > 0) {
         if (cudaMalloc(&m.classify_table, sizeof(ClassifyLayer) * k) != cudaSuccess) { cudaGetLastError(); rc = DC_ERR_ALLOC; }
-        else if (cudaMemcpy(m.classify_table, h, sizeof(ClassifyLayer) * k, cudaMemcpyHostToDevice) != cudaSuccess) rc = DC_ERR_CUDA;
+        else if (cudaMemcpyAsync(m.classify_table, h, sizeof(ClassifyLayer) * k, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) rc = DC_ERR_CUDA;
         else c->bytes += sizeof(ClassifyLayer) * k;
     }
     free(h);

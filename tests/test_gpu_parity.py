@@ -1424,6 +1424,43 @@ def test_lookahead_gives_identical_results():
         dc.close()
 
 
+@pytest.mark.parametrize("recorded", [1, 2])
+def test_first_lookahead_in_a_graph(recorded):
+    """The first announced frames of a cache recorded in a capture, where nothing may be allocated, and launched from there; then announced by
+    plain calls, with the match sets standing either way round.  Outputs are those of frames that were not announced."""
+    w = configs.WORKLOADS[3]()
+    sb = w.streams(1, 7)
+    frames = [torch.from_numpy(np.ascontiguousarray(sb.frame(i))).cuda() for i in range(7)]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        dc = DeepCache.from_workload(w)
+        pitch = w.width * 3
+        want = [dc.infer_frame(f).clone() for f in frames]
+        dc.reset()
+        got = [dc.infer_frame(frames[0]).clone()]
+        outs = [torch.empty_like(got[0]) for _ in range(recorded)]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        for k in range(recorded):
+            B.dc_lookahead_frame(dc.handle, frames[1 + k], pitch)
+            B.dc_infer_frame(dc.handle, frames[1 + k], pitch, outs[k], None)
+    with torch.cuda.stream(stream):
+        graph.replay()
+        stream.synchronize()
+        got += outs
+        for i in range(1 + recorded, 7):
+            if i > 1 + recorded:            # behind a capture a frame that is not announced comes first
+                B.dc_lookahead_frame(dc.handle, frames[i], pitch)
+            got.append(dc.infer_frame(frames[i]).clone())
+        stream.synchronize()
+        assert dc.status() == B.DC_OK
+    for i, (x, y) in enumerate(zip(want, got)):
+        assert torch.equal(x, y), f"frame {i}"
+    del graph
+    dc.close()
+
+
 @pytest.mark.parametrize("search,R", [(B.DC_SEARCH_DIAMOND, 12), (B.DC_SEARCH_THREE_STEP, 9)])
 @pytest.mark.parametrize("W,H,S", [(64, 48, 2), (144, 70, 3), (64, 37, 160)])
 def test_frames_matched_where_they_lie(search, R, W, H, S):
