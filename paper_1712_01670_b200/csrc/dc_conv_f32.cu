@@ -589,8 +589,8 @@ __global__ void k_pack_f32_fma(const float* w, int taps, int Cig, int Cog, int c
     }
 }
 
-// An MMA takes some 40 clocks for its pixels whatever its width: a step of 16 channels measured 240 clocks for 32 output channels and 310 for
-// 64.  Wide blocks, then, unless they leave SMs without an item: whichever takes fewer clocks with every tile dirty.
+// The pixels are read from shared memory again for every block of channels: a step of 16 channels measured 240 clocks for 32 output channels and 310
+// for 64.  Wide blocks, then, unless they leave SMs without an item: whichever takes fewer clocks with every tile dirty.
 int f32_bn(const dc_cache* c, const dc_layer_rt& L)
 {
     const int G = L.d.groups > 1 ? L.d.groups : 1, cog = L.d.cout / G;
