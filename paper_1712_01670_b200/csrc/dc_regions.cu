@@ -304,9 +304,9 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
     const int X0 = tx * DC_TILE_W, Y0 = ty * DC_TILE_H;
     const int X1 = min(X0 + DC_TILE_W, a.Wo), Y1 = min(Y0 + DC_TILE_H, a.Ho);
     const dc_region* regs = a.regions + (size_t)s * a.max_regions;
-    // the first rectangles travel with their number (the list has room for max_regions)
+    // the first rectangles of a frame travel with their number; of a caller's list no more is read than that says
     dc_region first = empty_region();
-    if (lane < a.max_regions) first = regs[lane];
+    if (a.alive && lane < a.max_regions) first = regs[lane];
     // every rectangle of this stream has eroded away before this layer: nothing to test or copy
     const int n = (a.alive && a.alive[s] == 0) ? 0 : min(a.n_regions[s], a.max_regions);
     const size_t map_base = (size_t)s * a.Ho * a.Wo * a.px_bytes;
@@ -316,7 +316,7 @@ __device__ __forceinline__ void classify_tile(const ClassifyArgs& a, const int t
         dc_region r = empty_region();
         int ix0 = 0, ix1 = 0, iy0 = 0, iy1 = 0;
         if (i < n) {
-            r = base == 0 ? first : regs[i];
+            r = a.alive && base == 0 ? first : regs[i];
             // Rectangles made by Step 5 and Table 2 lie inside the map on both sides.  One that does not (a caller's
             // own list) is not reused: neither side is ever addressed outside its map; the status word records it.
             const bool inside = r.x >= 0 && r.y >= 0 && r.sx >= 0 && r.sy >= 0 && r.w <= a.Wo && r.h <= a.Ho &&
