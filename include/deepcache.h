@@ -212,13 +212,14 @@ int dc_infer_frame(dc_cache* cache, const uint8_t* frame_dev, size_t pitch_bytes
                    void* out_map_dev, dc_frame_stats* stats_host);
 
 /* Announces the frame that the NEXT dc_infer_frame will get, so that its matching (Steps 1-5) runs on a
- * side stream while the convolutions of the current frame are still running: Section 7.6 points out that
- * matching one image and inferring another can proceed at the same time.  Call it after dc_infer_frame
+ * side stream while the convolutions of the current frame are still running, and its region propagation
+ * too unless the frames have so many blocks that matching is a large part of the step: Section 7.6 points out
+ * that matching one image and inferring another can proceed at the same time.  Call it after dc_infer_frame
  * for frame t, with frame t+1; the next dc_infer_frame must then be given the same frame_dev and
  * pitch_bytes (any other frame simply discards the lookahead).  frame_dev must stay unchanged until that
- * call.  Results are identical with and without it.  The side stream has the lowest priority; when the
- * stream given to dc_cache_create has a higher one, the convolution kernels get the SMs first and the
- * matcher fills what they leave, which shortens the overlapped step further.
+ * call.  Results are identical with and without it.  Allocates no device memory.  The side stream has the
+ * lowest priority; when the stream given to dc_cache_create has a higher one, the convolution kernels get
+ * the SMs first and the matcher fills what they leave, which shortens the overlapped step further.
  * Errors: DC_ERR_ARG, DC_ERR_STATE (no frame inferred yet, or layer table not executable), DC_ERR_CUDA. */
 int dc_lookahead_frame(dc_cache* cache, const uint8_t* frame_dev, size_t pitch_bytes);
 
@@ -242,7 +243,10 @@ int dc_prefetch_frame_host(dc_cache* cache, const uint8_t* frame_host, size_t pi
 int dc_cache_layer_map(dc_cache* cache, int layer, void** map_dev, size_t* bytes);
 
 /* Device address of the rectangles dc_infer_frame / dc_propagate_regions last computed for
- * `layer` ([S][max_regions]) and of their per-stream count ([S]). */
+ * `layer` ([S][max_regions]) and of their per-stream count ([S]).  A layer's address (layer >= 0) holds for the cache's
+ * life; the count's, and that of the rectangles on the frame (layer -1), until the next dc_infer_frame.  A program that
+ * has asked for a layer's address once finds the rectangles of every later frame there: their propagation then always
+ * runs with the inference (see dc_lookahead_frame).  May enqueue work on the cache's stream.  Errors: DC_ERR_ARG, DC_ERR_CUDA. */
 int dc_cache_layer_regions(dc_cache* cache, int layer, dc_region** regions_dev, int32_t** n_dev);
 
 /* Which kernel family runs convolution layer `layer` (chosen at creation): -1 not an executable convolution,

@@ -26,7 +26,7 @@ void dc_use_match_set(dc_cache* c, int k)
     c->mset_cur = k;
     c->blk_mv = m.blk_mv; c->blk_sse = m.blk_sse; c->matched = m.matched; c->run_end = m.run_end; c->mv_acc = m.mv_acc;
     c->long_list = m.long_list; c->gmv = m.gmv; c->regions0 = m.regions0; c->n_regions = m.n_regions;
-    c->table = m.table; c->live = m.live; c->dirty_count = m.dirty_count; c->reuse_px = m.reuse_px; c->alive = m.alive; c->classify_table = m.classify_table;
+    c->live = m.live; c->dirty_count = m.dirty_count; c->reuse_px = m.reuse_px; c->alive = m.alive; c->classify_table = m.classify_table;
 }
 
 bool dc_layer_cached(const dc_cache* c, int layer)
@@ -49,30 +49,51 @@ int dev_alloc(dc_cache* c, T** p, size_t count)
 }
 #define DC_TRY(expr) do { int rc__ = (expr); if (rc__ != DC_OK) return rc__; } while (0)
 
-// What region propagation writes, and the table that the reuse step reads it by (dc_build_classify_table).
-int alloc_tables(dc_cache* c, dc_match_set& m)
+// What the reuse step needs of region propagation, and the table that it reads it by (dc_build_classify_table).
+int alloc_lists(dc_cache* c, dc_match_set& m)
 {
     const size_t n = (size_t)c->n_layers, per_layer = (size_t)c->S * c->max_regions;
-    DC_TRY(dev_alloc(c, &m.table, n * per_layer));
     DC_TRY(dev_alloc(c, &m.live, n * per_layer));
     DC_TRY(dev_alloc(c, &m.dirty_count, n));
     DC_TRY(dev_alloc(c, &m.reuse_px, n * c->S * 2));
     m.alive = m.reuse_px + n * c->S;
-    DC_CUDA(cudaMemsetAsync(m.table, 0, sizeof(dc_region) * n * per_layer, c->stream));
     DC_CUDA(cudaMemsetAsync(m.reuse_px, 0, sizeof(int32_t) * n * c->S * 2, c->stream));
     return DC_OK;
 }
-void free_tables(dc_match_set& m)
+void free_lists(dc_match_set& m)
 {
-    cudaFree(m.table); cudaFree(m.live); cudaFree(m.dirty_count); cudaFree(m.reuse_px); cudaFree(m.classify_table);
-    m.table = m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = nullptr; m.classify_table = nullptr;
+    cudaFree(m.live); cudaFree(m.dirty_count); cudaFree(m.reuse_px); cudaFree(m.classify_table);
+    m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = nullptr; m.classify_table = nullptr;
 }
-void share_tables(dc_cache* c)
+void share_lists(dc_cache* c)
 {
     dc_match_set& m = c->mset[1]; const dc_match_set& o = c->mset[0];
-    m.table = o.table; m.live = o.live; m.dirty_count = o.dirty_count; m.reuse_px = o.reuse_px; m.alive = o.alive; m.classify_table = o.classify_table;
+    m.live = o.live; m.dirty_count = o.dirty_count; m.reuse_px = o.reuse_px; m.alive = o.alive; m.classify_table = o.classify_table;
 }
-bool own_tables(const dc_cache* c) { return c->mset[1].table != c->mset[0].table; }
+bool own_lists(const dc_cache* c) { return c->mset[1].live != c->mset[0].live; }
+
+// More blocks than the SMs hold warps, ten times over: matching a frame then takes about as long as a trunk's inference.  Measured
+// with the answer always no and always yes (VGG trunk, next frame announced, us a pass): full HD, 2 streams (110 blocks per SM) 248
+// and 308, 8 (441) 588 and 594, 10 (551) 711 both, 12 (662) 818 and 789, 32 (1764) 1891 and 1742; 720p, 16 (389) 808 and 807, 32 (778)
+// 1454 and 1381.
+bool matcher_is_large(const dc_cache* c) { return (long long)c->S * c->Gx * c->Gy > (long long)c->num_sms * 640; }
+
+// Lists of their own for the second match set, so that an announced frame's rectangles go through the layers beside the inference too.
+// Without the memory for them propagation stays with the inference, as it does where the matcher is large.
+int second_lists(dc_cache* c)
+{
+    share_lists(c);
+    if (!c->executable || matcher_is_large(c)) return DC_OK;
+    const size_t before = c->bytes;
+    dc_match_set m = c->mset[1];
+    m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = nullptr; m.classify_table = nullptr;
+    int rc = alloc_lists(c, m);
+    if (rc == DC_OK) rc = dc_build_classify_table(c, m);
+    if (rc == DC_OK) { c->mset[1] = m; return DC_OK; }
+    free_lists(m);
+    c->bytes = before;
+    return rc == DC_ERR_ALLOC ? DC_OK : rc;
+}
 
 // Can dc_infer_frame run this layer?  LRN needs its window stated consistently, a fully-connected layer must cover
 // its whole input map (it then runs as that convolution).
@@ -178,8 +199,10 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
         DC_TRY(dev_alloc(c, &m.n_regions, (size_t)S));
         DC_CUDA(cudaMemsetAsync(m.n_regions, 0, sizeof(int32_t) * S, c->stream));
     }
-    DC_TRY(alloc_tables(c, c->mset[0]));
-    share_tables(c);
+    DC_TRY(alloc_lists(c, c->mset[0]));
+    DC_TRY(dev_alloc(c, &c->table, (size_t)n * S * c->max_regions));
+    DC_CUDA(cudaMemsetAsync(c->table, 0, sizeof(dc_region) * n * S * c->max_regions, c->stream));
+    share_lists(c);
     dc_use_match_set(c, 0);
     DC_TRY(dc_build_propagate_table(c, layers));
     DC_TRY(dev_alloc(c, &c->all_count, (size_t)n * 2));
@@ -283,7 +306,7 @@ int build(dc_cache* c, const dc_layer_desc* layers, const void* const* weights_d
     }
     if (readers != 1) c->resize_feeds = -1;
     if (c->executable) DC_TRY(dc_build_classify_table(c, c->mset[0]));       // after the tuner: it decides each layer's tile geometry
-    share_tables(c);
+    DC_TRY(second_lists(c));
     dc_use_match_set(c, 0);
     DC_CUDA(cudaStreamSynchronize(c->stream));
     return DC_OK;
@@ -302,9 +325,9 @@ void release(dc_cache* c)
         cudaFree(m.blk_mv); cudaFree(m.blk_sse); cudaFree(m.matched); cudaFree(m.run_end); cudaFree(m.mv_acc);
         cudaFree(m.long_list); cudaFree(m.gmv); cudaFree(m.regions0); cudaFree(m.n_regions);
     }
-    if (own_tables(c)) free_tables(c->mset[1]);
-    free_tables(c->mset[0]);
-    cudaFree(c->prop_table); cudaFree(c->partial); cudaFree(c->all_count);
+    if (own_lists(c)) free_lists(c->mset[1]);
+    free_lists(c->mset[0]);
+    cudaFree(c->table); cudaFree(c->prop_table); cudaFree(c->partial); cudaFree(c->all_count);
     cudaFree(c->zero_masks); cudaFree(c->status); cudaFree(c->input_map);
     if (c->stats_pinned) cudaFreeHost(c->stats_pinned);
     for (int i = 0; i < c->n_layers; ++i) {
@@ -445,6 +468,14 @@ int dc_cache_set_key(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
     return mark_key(c);                                             // the key itself has changed
 }
 
+// The rectangles of the last frame at every layer, where its propagation ran beside an inference: from the frame's own, which are still there.
+static int settle_table(dc_cache* c)
+{
+    if (!c->table_stale) return DC_OK;
+    c->table_stale = false;
+    return dc_launch_propagate(c, c->regions0, c->n_regions, c->n_layers, false, c->table, nullptr, 0, nullptr);
+}
+
 int dc_match_blocks(dc_cache* c, const uint8_t* frame_dev, size_t pitch, int16_t* block_mv_dev,
                     uint32_t* block_sse_dev, uint8_t* matched_dev, int32_t* global_mv_dev,
                     dc_region* regions_dev, int32_t* n_regions_dev)
@@ -452,6 +483,7 @@ int dc_match_blocks(dc_cache* c, const uint8_t* frame_dev, size_t pitch, int16_t
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
     if (!c->key_valid) return DC_ERR_STATE;
     DC_TRY(cancel_lookahead(c));
+    DC_TRY(settle_table(c));
     const bool in_place = dc_match_in_place(c, frame_dev, pitch);
     uint8_t* scratch = in_place ? nullptr : c->key[(c->key_cur + 1) % 3];        // scratch copy; the cache key stays
     if (!in_place) DC_TRY(dc_launch_copy_frame(c, frame_dev, pitch, scratch, c->mv_acc));
@@ -470,7 +502,9 @@ int dc_propagate_regions(dc_cache* c, const dc_region* in_dev, const int32_t* n_
 {
     if (!c || !in_dev || !n_in_dev || !out_dev) return DC_ERR_ARG;
     if (layer_begin < 0 || layer_end > c->n_layers || layer_begin >= layer_end) return DC_ERR_ARG;
-    return dc_launch_propagate(c, in_dev, n_in_dev, layer_end, false, out_dev, layer_begin, n_out_dev);
+    if (layer_end < c->n_layers) DC_TRY(settle_table(c));
+    c->table_stale = false;
+    return dc_launch_propagate(c, in_dev, n_in_dev, layer_end, false, c->table, out_dev, layer_begin, n_out_dev);
 }
 
 int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* prev_out_dev,
@@ -493,12 +527,6 @@ int dc_conv_partial(dc_cache* c, int layer, const void* in_map_dev, const void* 
     }
     return dc_launch_conv(c, layer, in_map_dev, out_map_dev, L.all_list, dc_all_count(c, layer), c->zero_masks, tiles);
 }
-
-// More blocks than the SMs hold warps, ten times over: matching a frame then takes about as long as a trunk's inference.  Measured
-// with the answer always no and always yes (VGG trunk, next frame announced, us a pass): full HD, 2 streams (110 blocks per SM) 248
-// and 308, 8 (441) 588 and 594, 10 (551) 711 both, 12 (662) 818 and 789, 32 (1764) 1891 and 1742; 720p, 16 (389) 808 and 807, 32 (778)
-// 1454 and 1381.
-static bool matcher_is_large(const dc_cache* c) { return (long long)c->S * c->Gx * c->Gy > (long long)c->num_sms * 640; }
 
 static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void* out_map_dev, dc_frame_stats* stats)
 {
@@ -529,8 +557,8 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
         if (looked_ahead && c->la_matched) dc_use_match_set(c, c->mset_cur ^ 1);              // results are waiting there
         else DC_TRY(dc_launch_match(c, frame_copy, c->key[c->key_cur], nullptr, in_place, pitch));
         if (in_place) DC_TRY(mark_key(c));                                                    // the search has made the copy
-        if (!looked_ahead || !c->la_propagated)
-            DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n, true, nullptr, 0, nullptr));
+        c->table_stale = looked_ahead && c->la_propagated;
+        if (!c->table_stale) DC_TRY(dc_launch_propagate(c, c->regions0, c->n_regions, n, true, c->table, nullptr, 0, nullptr));
     }
     if (c->input_map && !c->fused_input) DC_TRY(dc_launch_input_map(c, frame_copy, c->key_pitch));
     const size_t per_layer = (size_t)S * c->max_regions;
@@ -556,7 +584,7 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             if (L.d.in0 < 0 && c->fused_input) { DC_TRY(dc_launch_frame_operand(c, i, frame_copy, c->key_pitch)); in = nullptr; }
             else if (i == c->resize_feeds) in = nullptr;              // its operand copy is filled already
             if (!refresh && !classified)
-                DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
+                DC_TRY(dc_launch_classify_copy(c, i, c->live + per_layer * i, c->alive + (size_t)i * S, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
             if (L.fuse_add >= 0) {                                    // every tile: the add is due for reused pixels too
                 dc_layer_rt& A = c->L[L.fuse_add];
                 c->add_in = layer_input(c, A.d.in0 == i ? A.d.in1 : A.d.in0); c->add_out = A.map[0]; c->add_relu = A.d.relu;
@@ -575,7 +603,7 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_maxpool(c, i, in, L.map[0], nullptr, also)); copied = also != nullptr; break; }
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
             if (!refresh) {           // Section 5's three steps on a pooling layer: copy, mark, compute the rest
-                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
+                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->live + per_layer * i, c->alive + (size_t)i * S, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
                 DC_TRY(dc_launch_maxpool(c, i, in, out, L.masks, nullptr));
             } else {
                 DC_TRY(dc_launch_maxpool(c, i, in, out, nullptr, nullptr));
@@ -595,7 +623,7 @@ static int infer_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch, void
             if (!dc_layer_cached(c, i)) { DC_TRY(dc_launch_lrn(c, i, in, L.map[0], nullptr)); break; }
             void* prev = L.map[L.cur]; void* out = L.map[L.cur ^ 1];
             if (!refresh) {
-                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->table + per_layer * i, c->n_regions, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
+                if (!classified) DC_TRY(dc_launch_classify_copy(c, i, c->live + per_layer * i, c->alive + (size_t)i * S, prev, out, c->dirty_count + i, c->reuse_px + (size_t)i * S, nullptr));
                 DC_TRY(dc_launch_lrn(c, i, in, out, L.masks));
             } else {
                 DC_TRY(dc_launch_lrn(c, i, in, out, nullptr));
@@ -650,39 +678,12 @@ static bool captured(cudaStream_t s)
     return st != cudaStreamCaptureStatusNone;
 }
 
-// Tables of their own for the announced frame's rectangles.  Without the memory for them, and in calls that a capture records (which must not
-// allocate), propagation stays with the inference, as it does where the matcher is large.  While the second set is the current one, the
-// inference in flight may read the tables that both share: they part when the first is.  Another thread's capture is none of this call's.
-static void ensure_lookahead_tables(dc_cache* c)
-{
-    if (c->la_tables_tried || c->mset_cur != 0 || matcher_is_large(c) || captured(c->stream) || captured(c->la_stream)) return;
-    c->la_tables_tried = true;
-    const size_t before = c->bytes;
-    dc_match_set m = c->mset[1];
-    m.table = m.live = nullptr; m.dirty_count = m.reuse_px = nullptr; m.classify_table = nullptr;
-    cudaStream_t main_stream = c->stream;
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    c->stream = c->la_stream;                           // written there, where they are first used
-    const bool ok = alloc_tables(c, m) == DC_OK && dc_build_classify_table(c, m) == DC_OK;
-    c->stream = main_stream;
-    if (ok) {
-        c->mset[1] = m;
-    } else {
-        cudaGetLastError();
-        free_tables(m);
-        c->bytes = before;
-    }
-    cudaThreadExchangeStreamCaptureMode(&mode);
-}
-
 int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
 {
     if (!c || !frame_dev || pitch < (size_t)c->cfg.width * 3) return DC_ERR_ARG;
     if (!c->executable || !c->key_valid) return DC_ERR_STATE;       // needs a frame to match against
     DC_TRY(ensure_lookahead_stream(c));
     DC_TRY(cancel_lookahead(c));
-    ensure_lookahead_tables(c);
     // Everything the side stream touches is free once the main stream has passed the frame copy of the last
     // dc_infer_frame, dc_match_blocks or dc_cache_set_key (mark_key): the third key buffer was last read two frames ago, and the
     // match set that the current inference does not read was last read by the frame before it.  Waiting for
@@ -702,8 +703,10 @@ int dc_lookahead_frame(dc_cache* c, const uint8_t* frame_dev, size_t pitch)
         // The rectangles through the layers too, unless the matcher is large: the walk wants much of an SM's shared memory and would wait
         // between the convolutions for it.  A pass in us, propagated by the inference and so: ResNet-50, one stream, 336 and 326; VGG, 6 streams of
         // 720p from host memory, 417 and 410; small CNN, 4 streams, 174 and 171; 24 streams of ResNet-50 and more the same.
-        c->la_propagated = rc == DC_OK && own_tables(c);
-        if (c->la_propagated) rc = dc_launch_propagate(c, c->regions0, c->n_regions, c->n_layers, true, nullptr, 0, nullptr);
+        // Not once the program has asked where each layer's rectangles are, nor in a graph that may be launched after it has: there the
+        // inference brings the table up to date, which the walk on the side does not write.
+        c->la_propagated = rc == DC_OK && own_lists(c) && !c->table_shown && !captured(c->la_stream);
+        if (c->la_propagated) rc = dc_launch_propagate(c, c->regions0, c->n_regions, c->n_layers, true, nullptr, nullptr, 0, nullptr);
         dc_use_match_set(c, main_set);
     } else {
         c->la_propagated = false;
@@ -805,6 +808,7 @@ int dc_cache_layer_conv_scheme(const dc_cache* c, int layer, int32_t* scheme)
 int dc_cache_layer_regions(dc_cache* c, int layer, dc_region** regions_dev, int32_t** n_dev)
 {
     if (!c || layer < -1 || layer >= c->n_layers || !regions_dev) return DC_ERR_ARG;
+    if (layer >= 0) { c->table_shown = true; DC_TRY(settle_table(c)); }
     *regions_dev = layer < 0 ? c->regions0 : c->table + (size_t)c->S * c->max_regions * layer;
     if (n_dev) *n_dev = c->n_regions;
     return DC_OK;

@@ -73,13 +73,13 @@ struct dc_layer_rt {
     int tm_next;                    // which of tm_a[] a new input base replaces
 };
 
-// Everything one run of the matcher and of region propagation writes.  Two sets exist so that both may already work on the
-// next frame (dc_lookahead_frame) while inference of the current frame still reads its own set.  What propagation writes is there
-// once, in both sets, until a frame has been announced.
+// Everything one run of the matcher writes, and what the reuse step needs of region propagation.  Two sets exist so that both may already
+// work on the next frame (dc_lookahead_frame) while inference of the current frame still reads its own set.  The last line is there once, in
+// both sets, where the matcher is large or memory short.
 struct dc_match_set {
     int16_t* blk_mv; uint32_t* blk_sse; uint8_t* matched; uint16_t* run_end; int32_t* mv_acc; uint4* long_list;
     int32_t* gmv; dc_region* regions0; int32_t* n_regions;
-    dc_region* table; dc_region* live; int32_t* dirty_count; int32_t* reuse_px; int32_t* alive; void* classify_table;
+    dc_region* live; int32_t* dirty_count; int32_t* reuse_px; int32_t* alive; void* classify_table;
 };
 
 struct dc_cache {
@@ -98,11 +98,11 @@ struct dc_cache {
 
     uint8_t* key[3];                // key frames [S][H][key_pitch]: key[key_cur] is the cached previous frame,
     int key_cur;                    // key[(key_cur + 1) % 3] receives the frame being processed or looked ahead
-    dc_match_set mset[2];           // the members blk_mv ... alive below, and classify_table, alias mset[mset_cur]
+    dc_match_set mset[2];           // the members blk_mv ... alive below (not table), and classify_table, alias mset[mset_cur]
     int mset_cur;
     cudaStream_t la_stream;         // dc_lookahead_frame: matcher of the next frame beside the current inference
     cudaEvent_t ev_key, ev_match;   // main stream: frame copied in; side stream: lookahead finished
-    const uint8_t* la_frame; size_t la_pitch; bool la_matched, la_propagated, la_tables_tried;
+    const uint8_t* la_frame; size_t la_pitch; bool la_matched, la_propagated;
     bool last_refreshed;
     bool overlap_mode;              // the last frame was looked ahead: the next one's matching will run beside this inference
     void* classify_table; int n_cached, classify_warps;   // all cached layers' classification in one launch (dc_regions.cu)
@@ -126,7 +126,8 @@ struct dc_cache {
     int32_t* gmv;                   // [S][3]: Mx, My, K
     dc_region* regions0;            // [S][max_regions] rectangles on the frame
     int32_t* n_regions;             // [S]
-    dc_region* table;               // [n_layers][S][max_regions]
+    dc_region* table;               // [n_layers][S][max_regions] every slot at every layer, at one address for the cache's life
+    bool table_shown, table_stale;  // the program has asked for its address; the last frame's rectangles are not in it yet (settle_table)
     dc_region* live;                // [n_layers][S][max_regions] per layer the rectangles that have not eroded away, closed up
     void* prop_table;               // [n_layers] the layer table as region propagation reads it (dc_regions.cu)
     int32_t* dirty_count;           // [n_layers]
@@ -220,7 +221,7 @@ int dc_launch_match(dc_cache* c, uint8_t* cur_key, const uint8_t* prev_key, cons
 bool dc_match_in_place(const dc_cache* c, const uint8_t* frame, size_t pitch);
 void dc_use_match_set(dc_cache* c, int k);
 int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers);
-int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out);
+int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* table, dc_region* out, int out_begin, int32_t* n_out);
 int dc_launch_classify_copy(dc_cache* c, int layer, const dc_region* regions, const int32_t* n_regions,
                             const void* prev_out, void* out, int32_t* count, int32_t* px, unsigned long long* running);
 int dc_launch_conv(dc_cache* c, int layer, const void* in, void* out, const int32_t* tile_list,

@@ -99,7 +99,7 @@ __device__ Span general_rule(const PropLayer& L, int lane, Span a, Span b)
 // by layer 26, so 11.
 // alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most of a
 // frame's erode within a few layers, and the reuse step tests every tile against all it is given.
-// out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): the lists are wanted, and the
+// table: every slot at every layer, or NULL.  out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): the lists are wanted, and the
 // counters of the reuse step are zeroed.
 // walkers: threads that walk (a multiple of 32); dynamic shared memory: 8 * layer_end * walkers bytes.
 __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions, int walkers,
@@ -179,8 +179,10 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
                     len = *(const int2*)(len_all + l * walkers + k * kLanes);
                 }
                 if (k < here) {
-                    int2* t = (int2*)(table + row + first + k);      // the tables are 8-byte aligned
-                    t[0] = at; t[1] = len; t[2] = src;
+                    if (table) {
+                        int2* t = (int2*)(table + row + first + k);  // the tables are 8-byte aligned
+                        t[0] = at; t[1] = len; t[2] = src;
+                    }
                     if (out && l >= out_begin) out[row - out_begin * layer_stride + first + k] = dc_region{at.x, at.y, len.x, len.y, src.x, src.y};
                 }
                 if (!alive) continue;
@@ -683,7 +685,7 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
 
 // for_frame: the rectangles of the frame being inferred (counts what is alive, zeroes the reuse step's counters);
 // otherwise a caller's, returned in out / n_out for layers out_begin .. layer_end - 1.
-int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* out, int out_begin, int32_t* n_out)
+int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* table, dc_region* out, int out_begin, int32_t* n_out)
 {
     dc_prof_scope ps(c, DC_ST_PROPAGATE);
     // as many walkers as the rectangles need and shared memory has room for, and at least eight warps for the writing
@@ -695,7 +697,7 @@ int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, i
     if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_propagate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
     const dim3 grid((unsigned)c->S, for_frame ? 1u : (unsigned)dc_div_up(c->max_regions, walkers / kLanes));
     DC_CUDA(dc_launch_pdl(k_propagate, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, walkers, in, n_in,
-                          c->table, c->live, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
+                          table, c->live, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
     c->launches += 1;
     return DC_OK;
 }

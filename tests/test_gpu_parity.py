@@ -1461,6 +1461,93 @@ def test_first_lookahead_in_a_graph(recorded):
     dc.close()
 
 
+@pytest.mark.parametrize("asked", ["first", "late", "behind other calls"])
+def test_rectangles_of_announced_frames_stay_where_the_program_found_them(asked):
+    """dc_cache_layer_regions names one address of a layer's rectangles for the cache's life.  Asked for once, before or after frames have been
+    announced, it holds those of each frame that follows, announced or not; announcing frames takes no memory."""
+    w = configs.WORKLOADS[3]()
+    sb = w.streams(1, 9)
+    frames = [torch.from_numpy(np.ascontiguousarray(sb.frame(i))).cuda() for i in range(9)]
+    dc = DeepCache.from_workload(w)
+    try:
+        n_layers, pitch = len(w.layers), w.width * 3
+
+        def tables(ptrs, n):
+            torch.cuda.synchronize()
+            return [device_view(p, (dc.max_regions, 6), torch.int32, dc.device)[:n].clone() for p in ptrs]
+
+        def ask():
+            return [B.dc_cache_layer_regions(dc.handle, l)[0] for l in range(n_layers)]
+
+        want = []
+        for f in frames:                                            # one after the other, in a cache of its own
+            if not want:
+                plain = DeepCache.from_workload(w)
+            _, st = plain.infer_frame(f, want_stats=True)
+            want.append([plain.layer_regions(l)[0][0, :st[0].n_regions] for l in range(n_layers)])
+        plain.close()
+        assert sum(int((r[0][:, 2] > 0).sum()) for r in want[1:]) > 8
+        size = dc.bytes()
+        ptrs = ask() if asked == "first" else None
+        for i, f in enumerate(frames):
+            _, st = dc.infer_frame(f, want_stats=True)
+            if i not in (5, len(frames) - 1):
+                B.dc_lookahead_frame(dc.handle, frames[i + 1], pitch)
+            if i < 3 and asked != "first":
+                continue
+            if ptrs is None and asked == "behind other calls":      # what writes the frame's rectangles, and some layers' tables, anew
+                other = dc.match_blocks(frames[0])
+                out, _ = dc.propagate_regions(other["regions"], other["n_regions"], 0, 2)
+                ptrs = ask()
+                got = tables(ptrs, st[0].n_regions)
+                for l in range(n_layers):
+                    assert torch.equal(got[l], out[l, 0, :st[0].n_regions] if l < 2 else want[i][l]), f"frame {i} layer {l}"
+                continue
+            ptrs = ptrs or ask()
+            assert ask() == ptrs
+            if not st[0].refreshed:
+                for l, (x, y) in enumerate(zip(tables(ptrs, st[0].n_regions), want[i])):
+                    assert torch.equal(x, y), f"frame {i} layer {l}"
+        assert dc.bytes() == size and dc.status() == B.DC_OK
+    finally:
+        dc.close()
+
+
+def test_rectangles_of_announced_frames_in_a_graph():
+    """A graph of an announced frame, recorded before the program asks for the address of a layer's rectangles, leaves them there when it is
+    launched again behind that, over the frame its buffer then holds."""
+    w = configs.WORKLOADS[3]()
+    sb = w.streams(1, 3)
+    frames = [torch.from_numpy(np.ascontiguousarray(sb.frame(i))).cuda() for i in range(3)]
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        dc = DeepCache.from_workload(w)
+        dc.infer_frame(frames[0])
+        _, st = dc.infer_frame(frames[2], want_stats=True)          # the frame of the second launch, behind frame 0
+        n, want = st[0].n_regions, [dc.layer_regions(l)[0][0, :st[0].n_regions] for l in range(len(w.layers))]
+        dc.close()
+        dc = DeepCache.from_workload(w)
+        dc.infer_frame(frames[0])
+        buf = frames[1].clone()
+        stream.synchronize()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        B.dc_lookahead_frame(dc.handle, buf, w.width * 3)
+        B.dc_infer_frame(dc.handle, buf, w.width * 3, None, None)
+    with torch.cuda.stream(stream):
+        graph.replay()
+        ptrs = [B.dc_cache_layer_regions(dc.handle, l)[0] for l in range(len(w.layers))]
+        buf.copy_(frames[2])
+        graph.replay()
+        stream.synchronize()
+        assert n > 0 and dc.status() == B.DC_OK
+        for l, p in enumerate(ptrs):
+            assert torch.equal(device_view(p, (dc.max_regions, 6), torch.int32, dc.device)[:n], want[l]), f"layer {l}"
+    del graph
+    dc.close()
+
+
 @pytest.mark.parametrize("search,R", [(B.DC_SEARCH_DIAMOND, 12), (B.DC_SEARCH_THREE_STEP, 9)])
 @pytest.mark.parametrize("W,H,S", [(64, 48, 2), (144, 70, 3), (64, 37, 160)])
 def test_frames_matched_where_they_lie(search, R, W, H, S):
