@@ -982,7 +982,7 @@ __global__ void __launch_bounds__(P_WARPS * 32, AHEAD ? 2 : 4) k_search_dsw_long
     const bool direct = long_list == nullptr;
     const int sgx = (a.Gx + a.skip_k - 1) / a.skip_k, sgy = (a.Gy + a.skip_k - 1) / a.skip_k;       // searched columns, rows
     const int n = direct ? a.S * sgx * sgy : *long_count;
-    const int max_rounds = 4 * a.R + 8;                               // each re-staging moves the centre by more than 4 px
+    const int max_rounds = (2 * a.R + 1) * (2 * a.R + 1);             // a window is staged for a move, and every move strictly lowers the key
 #pragma unroll 1
     for (;;) {
         int idx = 0;

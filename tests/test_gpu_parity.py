@@ -561,6 +561,54 @@ def test_propagate_strides_that_are_no_power_of_two():
     check_propagation(b.layers, 140, 120, 3)
 
 
+def winding_pair(R):
+    """A frame and its predecessor in which the walk of one block winds through its whole search range, and the walk's centres.  The block is grey
+    but for its first pixel, so that a candidate's SSE falls with the previous frame's pixel there along one direction of colour space; all
+    pixels of the previous frame lie on one sphere around grey, so that nothing else changes it.  Their colours get better along the path, whose
+    centres' diamonds hold no later centre but the next."""
+    path = [(0, 0)]
+
+    def go(dx, dy):
+        path.append((path[-1][0] + dx, path[-1][1] + dy))
+
+    E = R - 2
+    while path[-1][0] > -E and path[-1][1] < E - 4:                  # to a corner, then row by row through the rest
+        go(-1, 1)
+    go(0, 2), go(1, 1)
+    sx = 1
+    while True:
+        left = -E if path[-1][1] <= -8 else max(-E, 9 - path[-1][1])
+        while path[-1][0] + 2 <= E if sx > 0 else path[-1][0] - 2 >= left:
+            go(2 * sx, 0)
+        if path[-1][1] - 3 < -E:
+            break
+        go(0, -2), go(-sx, -1)
+        sx = -sx
+    v = np.arange(-127, 128)
+    sphere = np.stack([c.ravel() for c in np.meshgrid(v, v, v, indexing="ij")], 1)
+    sphere = sphere[(sphere ** 2).sum(1) == 15461]
+    towards = np.array([127, 101, 83])
+    _, first = np.unique(sphere @ towards, return_index=True)        # by how far they lie in that direction
+    colours = sphere[first]
+    assert len(colours) > len(path)
+    size = 16 + 2 * R
+    cur = np.full((size, size, 3), 128, np.uint8)
+    cur[R, R] += towards.astype(np.uint8)
+    prev = np.broadcast_to(128 + colours[0], (size, size, 3)).astype(np.uint8)
+    for i, (x, y) in enumerate(path):
+        prev[R + y, R + x] = 128 + colours[len(colours) - len(path) + i]
+    return prev, cur, path
+
+
+def test_match_winding_walk():
+    """A walk of two thousand moves through several hundred windows: every one of them is made, to the last."""
+    R = 64
+    prev, cur, path = winding_pair(R)
+    m = orc.match_blocks(cur, prev, 16, R, B.DC_SEARCH_DIAMOND, 20.0)
+    assert tuple(np.asarray(m["mv"])[4, 4]) == path[-1] and len(path) > 2000
+    check_pairs([(prev, cur)], 16, R, B.DC_SEARCH_DIAMOND)
+
+
 def test_propagate_more_rectangles_than_a_batch_holds():
     """A frame's rectangles in several batches (a deep network leaves room for few of them at once): table, lists and counts of every layer."""
     b = nets.NetBuilder(128, 128)
