@@ -763,7 +763,7 @@ int dc_infer_frame_host(dc_cache* c, const uint8_t* frame_host, size_t pitch, vo
         for (int k = 0; k < 2; ++k) if (!c->prefetched[k]) { slot = k; break; }
         if (slot < 0) {                                           // both buffers hold prefetches of other frames: drop one
             DC_CUDA(cudaStreamSynchronize(c->copy_stream));
-            DC_TRY(cancel_lookahead(c));                          // it may be matching that frame where it lies
+            DC_TRY(cancel_lookahead(c));                          // it may still be copying that frame, and its match is not the new one's
             slot = 0;
         }
         DC_CUDA(cudaMemcpyAsync(c->staging[slot], frame_host, bytes, cudaMemcpyHostToDevice, c->stream));

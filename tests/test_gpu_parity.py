@@ -1011,6 +1011,36 @@ def test_infer_host_buffers_with_and_without_prefetch():
         ref.close(); dc.close()
 
 
+def test_infer_host_drops_a_prefetch_that_is_announced():
+    """A frame that was not prefetched while both buffers hold prefetches, the first of them announced already: the dropped one's copy and match are
+    not taken for it, and the frames behind it, prefetched and not, come out as from device buffers."""
+    w = configs.WORKLOADS[2]()
+    sb = w.streams(1, 6)
+    frames = [torch.from_numpy(np.ascontiguousarray(sb.frame(i))).pin_memory() for i in range(6)]
+    ref, dc = DeepCache.from_workload(w), DeepCache.from_workload(w)
+    try:
+        out = torch.empty(ref.out_shape(-1), dtype=torch.float32).pin_memory()
+
+        def prefetch(i):
+            B.dc_prefetch_frame_host(dc.handle, frames[i].data_ptr(), w.width * 3)
+
+        def infer(i):
+            want = ref.infer_frame(frames[i].cuda())
+            B.dc_infer_frame_host(dc.handle, frames[i].data_ptr(), w.width * 3, out.data_ptr())
+            assert torch.equal(out, want.cpu()), f"frame {i}"
+
+        infer(5)
+        prefetch(0)
+        infer(1)                                      # announces frame 0
+        prefetch(2)
+        infer(3)                                      # takes frame 0's buffer, announces frame 2
+        infer(2)
+        infer(4)
+        assert dc.status() == B.DC_OK
+    finally:
+        ref.close(); dc.close()
+
+
 def test_region_overflow_sets_the_status_word():
     """More rectangles than max_regions: the extra ones are dropped and the device status word says so."""
     prev = rng(2).integers(0, 256, size=(64, 64, 3), dtype=np.uint8)
