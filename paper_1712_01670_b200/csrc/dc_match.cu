@@ -123,42 +123,82 @@ __device__ __forceinline__ uint32_t row_sse(const MatchArgs& a, int s, int b, in
     return acc;
 }
 
+// The same of a whole block, for blocks of more than 16 pixels, by a warp: a lane has a word of a row, of every second row where a row has at
+// most 16 words, so that the lanes of a load lie side by side; eight rows in flight.
+__device__ __forceinline__ uint32_t wide_sse(const MatchArgs& a, int s, int b, int Mx, int My, int lane)
+{
+    const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * a.B, y0 = by * a.B, bw = min(a.B, a.W - x0), bh = min(a.B, a.H - y0);
+    const uint8_t* c = a.cur + (size_t)s * a.cur_stream + (size_t)y0 * a.cur_pitch + (size_t)x0 * 3;
+    // the pitches of key frames are multiples of 16: every row starts at the same place in its word
+    const int skip = (int)((uintptr_t)c & 3u), words = (skip + bw * 3 + 3) >> 2, tail = skip + bw * 3 - 4 * (words - 1);     // 1 to 4 bytes of the last word
+    const uint8_t* p = a.prev + (size_t)s * a.prev_stream + (size_t)(y0 + My) * a.prev_pitch + (size_t)(x0 + Mx) * 3 - skip;
+    const uint32_t sh = ((uint32_t)(uintptr_t)p & 3u) * 8u;
+    const bool two = words <= 16;
+    const int j = two ? lane & 15 : lane, first = two ? lane >> 4 : 0, step = two ? 2 : 1;
+    uint32_t m = j < words ? 0xffffffffu : 0u;
+    if (j == words - 1) m >>= 8 * (4 - tail);
+    if (j == 0) m &= 0xffffffffu << (8 * skip);
+    const uint8_t* cq = c - skip + 4 * j;
+    const uint8_t* pq = (const uint8_t*)((uintptr_t)p & ~(uintptr_t)3) + 4 * j;
+    uint32_t acc = 0;
+    for (int r0 = first; r0 < bh; r0 += 8 * step) {
+        uint32_t cw[8], lo[8], hi[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int r = r0 + k * step;
+            const bool in = r < bh && j < words;
+            const uint32_t* q = (const uint32_t*)(pq + (size_t)r * a.prev_pitch);
+            cw[k] = in ? dc_ld((const uint32_t*)(cq + (size_t)r * a.cur_pitch)) : 0u;
+            lo[k] = in && (const uint8_t*)q >= a.prev ? dc_ld(q) : 0u;           // bytes before the row are masked; none lie before the buffer
+            hi[k] = in ? dc_ld(q + 1) : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t d = __vabsdiffu4(cw[k], __funnelshift_r(lo[k], hi[k], sh)) & m;
+            acc = __dp4a(d, d, acc);
+        }
+    }
+    return __reduce_add_sync(0xffffffffu, acc);
+}
+
 // Steps 3-4 for any block size (16-pixel blocks have kernels of their own).  A warp takes `share` blocks: a lane settles one from its own
-// vector where that is M, or where M leaves the frame or the range, then LPB lanes, one per row, score each of the others.
-// What bounds it: the latency of a row's loads; so few blocks per warp, two where the frame has few.  720p, 4 streams, 10-pixel blocks:
-// 29 us with a warp per block that fetched every block byte by byte, 12.5 so.
-template <int LPB>
+// vector where that is M, or where M leaves the frame or the range, then the warp scores the others: two at a time, 16 lanes each, one per row,
+// or (WIDE: more than 16 pixels) one at a time.
+// What bounds it: the latency of a row's loads.  us with a warp per block that fetched every block byte by byte, with a lane per row also of large
+// blocks, and so: 720p, 4 streams, 10 pixels, 29, 12.5, 12.5; 1080p, 2 streams, 20 pixels, 30, 210 (a load's rows in as many lines), 22.
+template <bool WIDE>
 __global__ void __launch_bounds__(256) k_verify(MatchArgs a, int share)
 {
     dc_pdl_wait();
     dc_pdl_release();
     const unsigned all = 0xffffffffu;
-    const int lane = threadIdx.x & 31, r = lane % LPB, half = lane / LPB, per = a.Gx * a.Gy;
+    const int lane = threadIdx.x & 31, r = lane & 15, half = lane >> 4, per = a.Gx * a.Gy;
     const unsigned gi = (blockIdx.x * 8u + (threadIdx.x >> 5)) * (unsigned)share + (unsigned)lane;
     const bool in_grid = lane < share && gi < (unsigned)(per * a.S);
     const int s = in_grid ? (int)(gi / (unsigned)per) : a.S - 1, b = in_grid ? (int)(gi - (unsigned)s * per) : 0;
     const Step4 v = settle(a, a.B, gi, s, b, in_grid);
     int ok = v.ok;
     if (in_grid && b == 0) { a.gmv[3 * s] = v.Mx; a.gmv[3 * s + 1] = v.My; a.gmv[3 * s + 2] = v.K; }
+    const int by = b / a.Gx, bx = b - by * a.Gx;
+    const uint32_t limit = a.limit[limit_index(a, min(a.B, a.W - bx * a.B), min(a.B, a.H - by * a.B))];
     unsigned todo = __ballot_sync(all, in_grid && !v.settled);
     while (todo) {                                                               // the same in all lanes
-        int i = __ffs(todo) - 1; bool on = true;
+        const int mine = __ffs(todo) - 1;
         todo &= todo - 1;
-        const int mine = i;
-        int second = -1;
-        if (LPB == 16) {
-            if (todo) { second = __ffs(todo) - 1; todo &= todo - 1; }
-            if (half) { on = second >= 0; i = on ? second : i; }
-        }
-        const int Mx = __shfl_sync(all, v.Mx, i), My = __shfl_sync(all, v.My, i), si = __shfl_sync(all, s, i), bi = __shfl_sync(all, b, i);
-        uint32_t sse = row_sse(a, si, bi, Mx, My, r, on);
+        if constexpr (WIDE) {
+            const uint32_t sse = wide_sse(a, __shfl_sync(all, s, mine), __shfl_sync(all, b, mine), __shfl_sync(all, v.Mx, mine), __shfl_sync(all, v.My, mine), lane);
+            if (lane == mine) ok = sse <= limit;
+        } else {
+            const int second = todo ? __ffs(todo) - 1 : -1, i = half && second >= 0 ? second : mine;
+            todo &= todo - 1;
+            const bool on = !half || second >= 0;
+            const int Mx = __shfl_sync(all, v.Mx, i), My = __shfl_sync(all, v.My, i), si = __shfl_sync(all, s, i), bi = __shfl_sync(all, b, i);
+            uint32_t sse = row_sse(a, si, bi, Mx, My, r, on);
 #pragma unroll
-        for (int o = LPB / 2; o > 0; o >>= 1) sse += __shfl_xor_sync(all, sse, o);
-        const uint32_t other = LPB == 16 ? __shfl_xor_sync(all, sse, 16) : 0u;   // every lane knows both halves' sums
-        const uint32_t first_sse = half ? other : sse, second_sse = half ? sse : other;
-        if (lane == mine || lane == second) {
-            const int by = b / a.Gx, bx = b - by * a.Gx;
-            ok = (lane == mine ? first_sse : second_sse) <= a.limit[limit_index(a, min(a.B, a.W - bx * a.B), min(a.B, a.H - by * a.B))];
+            for (int o = 8; o > 0; o >>= 1) sse += __shfl_xor_sync(all, sse, o);
+            const uint32_t other = __shfl_xor_sync(all, sse, 16);                // every lane knows both halves' sums
+            if (lane == mine) ok = (half ? other : sse) <= limit;
+            if (lane == second) ok = (half ? sse : other) <= limit;
         }
     }
     if (in_grid) a.matched[gi] = (uint8_t)ok;
@@ -1347,13 +1387,14 @@ __global__ void __launch_bounds__(256) k_copy_frame(const uint8_t* src, const ui
     }
 }
 
+// Few blocks per warp where the frames have few.  us with 2, 4 and 8 (from launch to end): 640 x 360, 6 streams, 24 pixels (16 blocks per SM) 38, 43,
+// 49; 227 x 227, 64 streams, 12 pixels (156) 18.6, 19.9, 24.7; 1080p, 2 streams, 10 pixels (280) 40, 26, 25, 8 pixels (438) 56, 33, 23.
 void launch_verify(dc_cache* c, const MatchArgs& a)
 {
     dc_prof_scope ps(c, DC_ST_VERIFY);
-    const int blocks = a.S * a.Gx * a.Gy, share = blocks <= c->num_sms * 64 ? 2 : 8;
+    const int blocks = a.S * a.Gx * a.Gy, share = blocks <= c->num_sms * 64 ? 2 : blocks <= c->num_sms * 280 ? 4 : 8;
     const dim3 grid((unsigned)dc_div_up(blocks, 8 * share));
-    if (a.B <= 16) dc_launch_pdl(k_verify<16>, grid, 256, 0, c->stream, a, share);       // errors: cudaGetLastError below
-    else dc_launch_pdl(k_verify<32>, grid, 256, 0, c->stream, a, share);
+    dc_launch_pdl(a.B <= 16 ? k_verify<false> : k_verify<true>, grid, 256, 0, c->stream, a, share);       // errors: cudaGetLastError below
 }
 
 // Step 2 over staged windows: every block, or (only_clipped, see dc_win_args) those that the 16-pixel kernels leave out

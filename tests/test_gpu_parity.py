@@ -240,6 +240,21 @@ def test_match_many_tiles(search, R, block):
     check_pairs(pairs, block, R, search)
 
 
+@pytest.mark.parametrize("S", [2, 40])
+@pytest.mark.parametrize("block,W,H", [(17, 100, 87), (20, 81, 100), (21, 150, 64), (24, 97, 98), (31, 94, 125), (32, 67, 100)])
+def test_match_verify_large_blocks(block, W, H, S):
+    """Step 4 of blocks of more than 16 pixels, a warp per block: rows of 13 to 25 words, two and one to a load, cut on either side, at every place of a
+    row in its words, most blocks with a vector that is not the mean."""
+    g = rng(block + S)
+    pairs = []
+    for s in range(S):
+        prev = g.integers(0, 256, size=(H, W, 3), dtype=np.uint8)
+        cur = np.roll(prev, (s % 5 - 2, s % 7 - 3), axis=(0, 1))
+        cur = np.clip(cur.astype(int) + g.normal(0, 14, size=cur.shape) * (g.random((H, 1, 1)) < 0.7), 0, 255).astype(np.uint8)
+        pairs.append((prev, cur))
+    check_pairs(pairs, block, 5, B.DC_SEARCH_DIAMOND)
+
+
 @pytest.mark.parametrize("h,w,k,st,p", [(33, 41, 3, 2, 1), (32, 32, 7, 2, 3), (47, 35, 5, 3, 2), (30, 31, 7, 3, 0), (39, 227, 11, 4, 0), (41, 43, 11, 4, 5)])
 def test_frame_into_block_map(h, w, k, st, p):
     """A frame goes straight into a strided first layer's block map: blocks of 2, 3 and 4, padding on every side, rows that
