@@ -131,8 +131,8 @@ __device__ __forceinline__ void flush_sums(const dc_win_args& a, const Tile& t, 
 
 // ---- walks -----------------------------------------------------------------------------------------------------------
 // FAR: the window holds fewer than R pixels around the tile.  BT, PT: block edge and window pitch where they are known at compile time
-// (walk_pitch), else 0.
-template <int ITERS, bool FAR, int BT, int PT>
+// (walk_pitch), else 0.  EDGE: no room for points beyond the range; rounds that the range or the frame cuts have a path of their own.
+template <int ITERS, bool FAR, int BT, int PT, bool EDGE>
 struct Walk {
     uint32_t base;                  // shared-memory byte address of displacement (0, 0)
     int pitch4_;                    // window row in bytes
@@ -193,7 +193,7 @@ struct Walk {
     }
     __device__ __forceinline__ uint32_t score(int dx, int dy) const
     {
-        if (FAR && !staged(dx, dy, 0)) return far(dx, dy);
+        if constexpr (FAR) { if (!staged(dx, dy, 0)) return far(dx, dy); }
         const uint32_t p = base + (uint32_t)(dy * pitch4() + dx * 4);
         uint32_t acc = 0;
 #pragma unroll
@@ -262,7 +262,7 @@ struct Walk {
             const int cx = disp_x(at), cy = disp_y(at), d = at + point;
             const bool ok = lane < 13 && within(d, valid);
             uint32_t mine = 0xffffffffu;
-            if (whole && staged(cx, cy, 2)) {
+            if (whole && staged(cx, cy, 2) && (!EDGE || (within(at - pair(2, 2), valid) && within(at + pair(2, 2), valid)))) {
                 const uint32_t pc = base + (uint32_t)(cy * pitch4() + cx * 4);
                 switch (kind) {
                 case 0: fast_set<kind_mask(0)>(pc, lane, mine); break;
@@ -340,7 +340,7 @@ __host__ __device__ constexpr int walk_pitch(int B) { return 8 * B + 36 + ((B - 
 // What it spends its instructions on (720p, 4 streams, 10 pixels, 1430 per block before): the candidates a third, so addresses known at compile
 // time, window rows by addition and whole blocks without a test per pixel: 80 us with run-time addresses and a path of their own for cut
 // rounds, 65 without these two, 57 so.
-template <int ITERS, bool FAR, int BT, bool AHEAD>
+template <int ITERS, bool FAR, int BT, bool AHEAD, bool EDGE = false>
 __global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 && !FAR && !AHEAD ? 3 : ITERS <= 8 ? 2 : 1) k_win_walk(const __grid_constant__ dc_win_args a)
 {
     extern __shared__ __align__(16) uint32_t win[];
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, ITERS <= 4 && !FAR && !AHEAD ?
     if (!any_mine(a, t)) return;
     const int ly = warp * a.inv_TX >> 16, lx = warp - ly * a.TX, bx = t.bx0 + lx, by = t.by0 + ly;
     const bool block = ly < a.TY && lx < t.nbx && ly < t.nby && mine(a, bx, by), walk = block && searched(a, bx, by);
-    Walk<ITERS, FAR, BT, PT> w;
+    Walk<ITERS, FAR, BT, PT, EDGE> w;
     const int x0 = bx * B, y0 = by * B, bw = min(B, a.W - x0), bh = min(B, a.H - y0);
     w.on = 0;
     w.whole = walk && bw == B && bh == B;
@@ -505,23 +505,22 @@ int launch(K kernel, const dc_win_args& a, int threads, size_t smem, int device,
 int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t stream)
 {
     const bool all = a.search == DC_SEARCH_EXHAUSTIVE;
+    const int iters = dc_div_up(a.B * a.B, 32);                       // pixels a lane owns
     size_t smem = 0;
-    bool known = false;                                               // block edge and pitch fit an instance that knows them
+    bool known = false;                                               // the instance that knows block edge and pitch
     auto shape = [&](int TX, int TY) {
         a.TX = TX; a.TY = TY; a.inv_TX = (65536 + TX - 1) / TX;
         a.tiles_x = dc_div_up(a.Gx, TX); a.tiles_y = dc_div_up(a.Gy, TY);
         a.win_cols = ((TX * a.B + 2 * (a.Rw - a.margin) + 3) & ~3) + 2 * a.margin;   // staged in groups of four
         a.win_rows = TY * a.B + 2 * a.Rw + (all ? E_ROWS - 1 : 0);    // rows only touched by displacements beyond R (scored, never compared)
-        a.win_pitch = a.win_cols + ((a.B - a.win_cols) % 32 + 32) % 32;   // = B modulo 32
-        known = !all && a.margin && a.B <= 16 && a.win_cols <= walk_pitch(a.B);
-        if (known) a.win_pitch = walk_pitch(a.B);
+        a.win_pitch = known ? walk_pitch(a.B) : a.win_cols + ((a.B - a.win_cols) % 32 + 32) % 32;   // = B modulo 32
         smem = (size_t)a.win_rows * a.win_pitch * 4 + (all ? (size_t)TX * TY * a.B * a.B * 4 : 0);
     };
     // Wide tiles stage fewer window pixels per block; they shrink while the window is too large for three CTAs per SM, and
     // while the frames have fewer tiles than the machine has SMs (down to two blocks, one for the exhaustive search).
     int TX = 0, TY = 0;
-    auto fit = [&](int Rw, int margin) {                              // returns the window pixels staged per block
-        a.Rw = Rw + margin; a.margin = margin;
+    auto fit = [&](int Rw) {                                          // returns the window pixels staged per block
+        a.Rw = Rw; a.margin = 0;
         TX = a.Gx < 8 ? a.Gx : 8; TY = TX < 4 ? 4 : 2;
         if (TY > a.Gy) TY = a.Gy;
         shape(TX, TY);
@@ -535,19 +534,34 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     // Walks over a long range: a window of kWalkReach where that stages less than a fifth per block.  (Match calls with the whole
     // window and with the capped one, range 64, diamond: 1080p, 16 streams, 8-pixel blocks, 13 times the pixels: 13456 and 1610 us;
     // 20 pixels, 6.6 times: 4145 and 2184; 227 x 227, 24 pixels, 2.7 times: 72 and 125.  Range 40, 1.4 to 1.8 times: 513 and 571.)
-    // The points around a centre at the end of the range lie up to two pixels beyond it: room for them, not staged.
-    const int beyond = a.search == DC_SEARCH_DIAMOND ? 2 : 0, whole = fit(a.R, beyond);
+    const int whole = fit(a.R);
     bool far = !all && a.R > kWalkReach;
-    if (far && whole <= 5 * fit(kWalkReach, 0)) { far = false; fit(a.R, beyond); }
+    if (far && whole <= 5 * fit(kWalkReach)) { far = false; fit(a.R); }
     // exhaustive: as many warps as there are groups of 32 items, up to 16
     const int n_d = 2 * a.R + 1, groups = (n_d * dc_div_up(n_d, E_ROWS) + 31) / 32;
     int warps = TX * TY < 8 ? 8 : TX * TY;                            // walks: a warp per block; spare ones help to stage the window
     if (all) { const long long units = (long long)TX * TY * groups; warps = units < 4 ? 4 : units > kMaxWarps ? kMaxWarps : (int)units; }
+    const bool few = (long long)a.tiles_x * a.tiles_y * a.S <= 2 * num_sms;
+    // The points around a centre at the end of the range lie up to two pixels beyond it: room for them (not staged), and the pitch of an instance
+    // that knows it, where the tile keeps its CTAs per SM.  (1080p, 4 streams, diamond, 16 pixels, range 48: 577 us with tiles shrunk to make that
+    // room, 282 with a known pitch whatever it costs, 262 so.)  Large blocks of a short range have no use for it: so many of a round's points
+    // are no candidates that a path of their own is cheaper (32 pixels, range 8: 239 and 209 us; 24 pixels, range 24, 278 and 284).
+    bool edge = false;
+    if (a.search == DC_SEARCH_DIAMOND && !far) {
+        const int threads = iters > 8 ? 512 : iters <= 4 && !few ? 1536 : 1024;   // an SM's, by the registers of the instance (launch bounds of k_win_walk)
+        auto ctas = [&] { const int by_smem = (int)(228 * 1024 / (smem + 1024 + 64)), by_regs = threads / (warps * 32); return by_smem < by_regs ? by_smem : by_regs; };
+        const int most = ctas();
+        a.Rw += 2; a.margin = 2;
+        known = a.B <= 16 && ((TX * a.B + 2 * a.R + 3) & ~3) + 4 <= walk_pitch(a.B);
+        shape(TX, TY);
+        if (known && ctas() < most) { known = false; shape(TX, TY); }
+        edge = iters > 8 && (a.R <= (iters <= 16 ? 6 : 12) || ctas() < most);
+        if (edge) { a.Rw -= 2; a.margin = 0; shape(TX, TY); }
+    }
     if (all) { static dc_once_per_device set; return launch(k_win_all, a, warps * 32, smem, device, set, stream); }
     // one instance per block edge up to 16, for ranges whose window fits its pitch (three step search: addresses with run-time steps gain
     // nothing from it), and one per number of pixels a lane owns
-#define DC_WALK_(n, f, b, ah) { static dc_once_per_device set; return launch(k_win_walk<n, f, b, ah>, a, warps * 32, smem, device, set, stream); }
-    const bool few = (long long)a.tiles_x * a.tiles_y * a.S <= 2 * num_sms;
+#define DC_WALK_(n, ...) { static dc_once_per_device set; return launch(k_win_walk<n, __VA_ARGS__>, a, warps * 32, smem, device, set, stream); }
     if (known) switch (a.B) {
 #define DC_WALK(b) case b: if (few) DC_WALK_((b * b + 31) / 32, false, b, true) DC_WALK_((b * b + 31) / 32, false, b, false)
         DC_WALK(4) DC_WALK(5) DC_WALK(6) DC_WALK(7) DC_WALK(8) DC_WALK(9) DC_WALK(10) DC_WALK(11)
@@ -556,8 +570,9 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
         DC_WALK(12) DC_WALK(13) DC_WALK(14) DC_WALK(15) DC_WALK(16)
 #undef DC_WALK
     }
+    if (edge) { if (iters <= 16) DC_WALK_(16, false, 0, false, true) DC_WALK_(32, false, 0, false, true) }
 #define DC_WALK(n) { if (far) DC_WALK_(n, true, 0, false) DC_WALK_(n, false, 0, false) }
-    switch (dc_div_up(a.B * a.B, 32)) {
+    switch (iters) {
     case 1: DC_WALK(1)
     case 2: DC_WALK(2)
     case 3: DC_WALK(3)
@@ -566,7 +581,7 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     case 6: DC_WALK(6)
     case 7: DC_WALK(7)
     case 8: DC_WALK(8)
-    default: if (a.B * a.B <= 512) DC_WALK(16) DC_WALK(32)
+    default: if (iters <= 16) DC_WALK(16) DC_WALK(32)
     }
 #undef DC_WALK
 #undef DC_WALK_

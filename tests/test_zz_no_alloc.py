@@ -120,3 +120,36 @@ def test_noalloc_rejects_sizes_beyond_its_scratch():
     with pytest.raises(B.DeepCacheError) as e:
         B.dc_search_blocks_noalloc(f, f, 48, 16, 16, B.DC_NOALLOC_MAX_STREAMS + 1, 16, 4, 1, 20.0, mv, sse, gmv)
     assert e.value.status == B.DC_ERR_LIMIT and "limit" in str(e.value)
+
+
+@pytest.mark.parametrize("block,R,S", [(16, 40, 30), (16, 48, 2), (14, 40, 30), (10, 30, 40), (11, 64, 3), (4, 16, 2), (20, 4, 20), (20, 8, 20), (24, 64, 6), (28, 8, 20), (32, 16, 20), (32, 32, 1)])
+def test_noalloc_search_windows(block, R, S):
+    """Ranges and block edges on either side of what the searches' instances and windows are made for: pitches that are known and are not, room for points
+    beyond the range and none, walks that end at the range's limit."""
+    g = np.random.Generator(np.random.PCG64(block + R))
+    W, H = 8 * block + 37, 2 * block + 30
+    size = (H + 2 * R) // 6 + 2, (W + 2 * R) // 6 + 2
+    prev, cur = np.empty((S, H, W, 3), np.uint8), np.empty((S, H, W, 3), np.uint8)
+    for s in range(S):
+        lat = np.clip(np.cumsum(g.normal(0, 30, size=(*size, 3)), axis=s % 2) + 128, 0, 255)
+        tex = np.repeat(np.repeat(lat, 6, 0), 6, 1)
+        tex = ((tex + np.roll(tex, 3, 0) + np.roll(tex, 3, 1) + np.roll(tex, 3, (0, 1))) / 4).astype(np.uint8)
+        dy, dx = (R // 2, -R) if s % 3 == 0 else (-(R - 1), R // 3) if s % 3 == 1 else (1, 0)
+        prev[s] = tex[R:R + H, R:R + W]
+        cur[s] = tex[R + dy:R + dy + H, R + dx:R + dx + W]
+        if s % 4 == 3:
+            cur[s] = g.integers(0, 256, (H, W, 3))
+    Gx, Gy = -(-W // block), -(-H // block)
+    mv = torch.empty((S, Gy, Gx, 2), dtype=torch.int16, device="cuda")
+    sse = torch.empty((S, Gy, Gx), dtype=torch.int32, device="cuda")
+    gmv = torch.empty((S, 3), dtype=torch.int32, device="cuda")
+    B.dc_search_blocks_noalloc(torch.from_numpy(cur).cuda(), torch.from_numpy(prev).cuda(), W * 3, W, H, S, block, R, B.DC_SEARCH_DIAMOND, 20.0, mv, sse, gmv)
+    torch.cuda.synchronize()
+    far = 0
+    for s in range(S):
+        o_mv, o_sse = orc.search(cur[s], prev[s], block, R, B.DC_SEARCH_DIAMOND)
+        far = max(far, int(np.abs(o_mv).max()))
+        assert np.array_equal(mv[s].cpu().numpy(), o_mv)
+        assert np.array_equal(sse[s].cpu().numpy().view(np.uint32), o_sse)
+        assert tuple(gmv[s].tolist()) == orc.mean_mv(o_mv, o_sse, W, H, block, 20.0)
+    assert far >= min(R, 12)
