@@ -93,15 +93,16 @@ __device__ Span general_rule(const PropLayer& L, int lane, Span a, Span b)
 // One CTA per stream (more for a caller's lists, which count nothing), batches of as many rectangles as have room in shared memory at all
 // layers.  First the walk, four lanes per rectangle: the two axes of the rectangle and of its cached image, which only meet where their
 // lengths are compared.  It leaves its rectangles in shared memory and does nothing else, because what bounds it is the chain of a lane's
-// instructions from layer to layer.  A warp whose rectangles have all vanished, those that later layers read too, stops.  Then all warps,
-// a layer at a time each, write the table and the lists.
+// instructions from layer to layer.  A warp whose rectangles have all vanished, those that later layers read too, stops.  Then all warps write
+// the table and the lists.
 // us for ResNet-50's 71 layers, one stream: a thread per rectangle that also wrote the table and asked for its places in the lists layer
 // by layer 26, so 11.
 // alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most of a
 // frame's erode within a few layers, and the reuse step tests every tile against all it is given.
-// table: every slot at every layer, or NULL.  out, n_out: a caller's copies of layers out_begin .. layer_end - 1 and of the counts.  alive (or NULL): the lists are wanted, and the
-// counters of the reuse step are zeroed.
+// FRAME: the rectangles of a frame: lists and counts are wanted, the counters of the reuse step are zeroed; table (every slot at every layer) or
+// NULL.  Else a caller's list: out, n_out, or NULL: copies of layers out_begin .. layer_end - 1 and of the counts.
 // walkers: threads that walk (a multiple of 32); dynamic shared memory: 8 * layer_end * walkers bytes.
+template <bool FRAME>
 __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions, int walkers,
                                                    const dc_region* in, const int32_t* n_in, dc_region* table, dc_region* live, int32_t* alive, int32_t* reuse_px,
                                                    int32_t* dirty_count, dc_region* out, int out_begin, int32_t* n_out)
@@ -118,8 +119,9 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
     dc_pdl_release();
     const int n = min(n_in[s], max_regions);              // a caller's count beyond the table is cut, never written
     // a caller's list has zeros behind its rectangles
-    const int rows = out ? max_regions : n;
+    const int rows = !FRAME && out ? max_regions : n;
     const size_t layer_stride = (size_t)S * max_regions;
+    const bool out_aligned = (uintptr_t)out % 8 == 0;     // a caller's array may lie at any word
     for (int first = blockIdx.y * per_batch; first < rows; first += gridDim.y * per_batch) {
         const int i = first + tid / kLanes;
         Span r0 = {0, 0};
@@ -165,39 +167,52 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
             if (lane == 0) end_of[warp] = l;
         }
         __syncthreads();
-        // a layer per warp, a rectangle per lane
-        const int here = min(per_batch, rows - first);
-        for (int l = warp; l < layer_end; l += nt >> 5) {
-            int listed = count[l];
-            const size_t row = l * layer_stride + (size_t)s * max_regions;
-            for (int k0 = 0; k0 < here; k0 += 32) {
-                const int k = k0 + lane;
-                int2 at = {0, 0}, len = {0, 0}, src = {0, 0};
-                if (k < here && l < end_of[k >> 3]) {
-                    const int32_t* p = at_all + l * walkers + k * kLanes;
-                    at = *(const int2*)p; src = *(const int2*)(p + 2);
-                    len = *(const int2*)(len_all + l * walkers + k * kLanes);
-                }
-                if (k < here) {
-                    if (table) {
-                        int2* t = (int2*)(table + row + first + k);  // the tables are 8-byte aligned
-                        t[0] = at; t[1] = len; t[2] = src;
-                    }
-                    if (out && l >= out_begin) out[row - out_begin * layer_stride + first + k] = dc_region{at.x, at.y, len.x, len.y, src.x, src.y};
-                }
-                if (!alive) continue;
-                const unsigned m = __ballot_sync(all, len.x > 0);
-                if (len.x > 0) {
-                    int2* t = (int2*)(live + row + listed + __popc(m & ((1u << lane) - 1u)));
-                    t[0] = at; t[1] = len; t[2] = src;
-                }
-                listed += __popc(m);
+        const int here = min(per_batch, rows - first), runs = (here + 31) >> 5;
+        // rectangle k of the batch at layer l
+        auto fetch = [&](int l, int k, int2& at, int2& len, int2& src) {
+            at = len = src = make_int2(0, 0);
+            if (k < here && l < end_of[k >> 3]) {
+                const int32_t* p = at_all + l * walkers + k * kLanes;
+                at = *(const int2*)p; src = *(const int2*)(p + 2);
+                len = *(const int2*)(len_all + l * walkers + k * kLanes);
             }
-            if (lane == 0) count[l] = listed;
+        };
+        auto put = [](dc_region* to, int2 at, int2 len, int2 src) { int2* t = (int2*)to; t[0] = at; t[1] = len; t[2] = src; };    // 8-byte aligned
+        if constexpr (FRAME) {
+            // a layer per warp, a rectangle per lane
+            for (int l = warp; l < layer_end; l += nt >> 5) {
+                const size_t row = l * layer_stride + (size_t)s * max_regions;
+                int listed = count[l];
+                for (int k0 = 0; k0 < here; k0 += 32) {
+                    const int k = k0 + lane;
+                    int2 at, len, src;
+                    fetch(l, k, at, len, src);
+                    if (table && k < here) put(table + row + first + k, at, len, src);
+                    const unsigned m = __ballot_sync(all, len.x > 0);
+                    if (len.x > 0) put(live + row + listed + __popc(m & ((1u << lane) - 1u)), at, len, src);
+                    listed += __popc(m);
+                }
+                if (lane == 0) count[l] = listed;
+            }
+        } else {
+            // 32 rectangles of a layer per warp, a rectangle per lane
+#pragma unroll 1
+            for (int u = warp; u < layer_end * runs; u += nt >> 5) {
+                const int l = u / runs, k = (u - l * runs) * 32 + lane;
+                const size_t row = l * layer_stride + (size_t)s * max_regions;
+                int2 at, len, src;
+                fetch(l, k, at, len, src);
+                if (k >= here) continue;
+                put(table + row + first + k, at, len, src);
+                if (!out || l < out_begin) continue;
+                dc_region* o = out + (row - out_begin * layer_stride + first + k);
+                if (out_aligned) put(o, at, len, src);
+                else *o = dc_region{at.x, at.y, len.x, len.y, src.x, src.y};
+            }
         }
     }
-    if (n_out && blockIdx.y == 0) for (int l = out_begin + tid; l < layer_end; l += nt) n_out[(l - out_begin) * S + s] = n_in[s];
-    if (alive) {
+    if (!FRAME && n_out && blockIdx.y == 0) for (int l = out_begin + tid; l < layer_end; l += nt) n_out[(l - out_begin) * S + s] = n_in[s];
+    if (FRAME) {
         __syncthreads();
         for (int l = tid; l < n_layers; l += nt) {
             alive[l * S + s] = l < layer_end ? count[l] : 0;
@@ -688,16 +703,23 @@ int dc_build_propagate_table(dc_cache* c, const dc_layer_desc* layers)
 int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, int layer_end, bool for_frame, dc_region* table, dc_region* out, int out_begin, int32_t* n_out)
 {
     dc_prof_scope ps(c, DC_ST_PROPAGATE);
-    // as many walkers as the rectangles need and shared memory has room for, and at least eight warps for the writing
+    // As many walkers as the rectangles need and shared memory has room for, and at least eight warps for the writing.  A caller's lists, whose
+    // every slot is written, go to CTAs of 32 rectangles, or of 64 where those are more than the SMs.  us with 1024 walkers, 256 and 128: 12 layers of
+    // 320 slots, 1 stream 8.8, 3.8, 3.6, 64 streams 10.0, 5.7, 6.3; 71 layers of 784 slots, 1 stream 8.2, 6.7, 4.9, 8 streams 8.3, 7.3, 10.4.
     const int room = (int)(kWalkBytes / (8 * (size_t)layer_end)) / 32 * 32, most = room > 1024 ? 1024 : room;
-    const int walkers = c->max_regions >= most / kLanes ? most : dc_div_up(c->max_regions * kLanes, 32) * 32;
+    const int lists = c->S * dc_div_up(c->max_regions, 32) <= c->num_sms ? 128 : 256;
+    const int cap = for_frame || lists > most ? most : lists;
+    const int walkers = c->max_regions >= cap / kLanes ? cap : dc_div_up(c->max_regions * kLanes, 32) * 32;
     const int threads = walkers < 256 ? 256 : walkers;
     const size_t smem = 8 * (size_t)layer_end * walkers;
     static dc_once_per_device attr_set;
-    if (attr_set.first(c->device)) DC_CUDA(cudaFuncSetAttribute(k_propagate, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+    if (attr_set.first(c->device)) {
+        DC_CUDA(cudaFuncSetAttribute(k_propagate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+        DC_CUDA(cudaFuncSetAttribute(k_propagate<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+    }
     const dim3 grid((unsigned)c->S, for_frame ? 1u : (unsigned)dc_div_up(c->max_regions, walkers / kLanes));
-    DC_CUDA(dc_launch_pdl(k_propagate, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, walkers, in, n_in,
-                          table, c->live, for_frame ? c->alive : nullptr, c->reuse_px, c->dirty_count, out, out_begin, n_out));
+    DC_CUDA(dc_launch_pdl(for_frame ? k_propagate<true> : k_propagate<false>, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, walkers, in, n_in,
+                          table, c->live, c->alive, c->reuse_px, c->dirty_count, out, out_begin, n_out));
     c->launches += 1;
     return DC_OK;
 }

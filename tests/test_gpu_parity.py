@@ -533,6 +533,35 @@ def test_propagate_networks(net, W, H):
     check_propagation(layers, W, H, 3)
 
 
+@pytest.mark.parametrize("S,slots,odd", [(4, 37 * 32, 0), (5, 37 * 32 - 1, 1), (1, 1, 0), (1, 33, 1), (3, 65, 0)])
+def test_propagate_lists_of_any_length(S, slots, odd):
+    """A caller's lists in CTAs of 32 and of 64 rectangles, with last ones that are not full, written to arrays that start at any word."""
+    layers = nets.inception_lrn_net(96, 128)
+    ws, bs = nets.random_weights(layers, 3)
+    dc = DeepCache(128, 96, layers, ws, bs, n_streams=S, block=16, search_range=2, dtype=B.DC_BF16, max_regions=slots)
+    try:
+        g = rng(slots)
+        n = [slots - min(s, slots - 1) for s in range(S)]
+        regs = np.zeros((S, slots, 6), np.int32)
+        for s in range(S):
+            w, h = g.integers(1, 90, n[s]), g.integers(1, 70, n[s])
+            x, y = g.integers(0, 128 - w + 1), g.integers(0, 96 - h + 1)
+            regs[s, :n[s]] = np.stack([x, y, w, h, g.integers(0, 128 - w + 1), g.integers(0, 96 - h + 1)], 1)
+        buf = torch.full((odd + len(layers) * S * slots * 6,), -7, dtype=torch.int32, device="cuda")
+        out = buf[odd:].view(len(layers), S, slots, 6)
+        n_out = torch.zeros((len(layers), S), dtype=torch.int32, device="cuda")
+        B.dc_propagate_regions(dc.handle, torch.from_numpy(regs).cuda(), torch.tensor(n, dtype=torch.int32, device="cuda"), 0, len(layers), out, n_out)
+        torch.cuda.synchronize()
+        assert not odd or int(buf[0]) == -7
+        for s in range(S):
+            want = orc.propagate(layers, (96, 128), U.regions_np(torch.from_numpy(regs[s, :n[s]])))
+            for l in range(len(layers)):
+                U.assert_regions_equal(U.regions_np(out[l, s, :n[s]]), want[l], f"stream {s} layer {l}")
+                assert not out[l, s, n[s]:].any() and int(n_out[l, s]) == n[s]
+    finally:
+        dc.close()
+
+
 def test_propagate_table2_rows():
     """Layer kinds that only region propagation knows (LRN, concat, fully connected)."""
     b = nets.NetBuilder(96, 96)
