@@ -26,7 +26,8 @@ void dc_use_match_set(dc_cache* c, int k)
     c->mset_cur = k;
     c->blk_mv = m.blk_mv; c->blk_sse = m.blk_sse; c->matched = m.matched; c->run_end = m.run_end; c->mv_acc = m.mv_acc;
     c->long_list = m.long_list; c->gmv = m.gmv; c->regions0 = m.regions0; c->n_regions = m.n_regions;
-    c->live = m.live; c->dirty_count = m.dirty_count; c->reuse_px = m.reuse_px; c->alive = m.alive; c->classify_table = m.classify_table;
+    c->live = m.live; c->dirty_count = m.dirty_count; c->reuse_px = m.reuse_px; c->alive = m.alive; c->places = m.places;
+    c->classify_table = m.classify_table;
 }
 
 bool dc_layer_cached(const dc_cache* c, int layer)
@@ -55,20 +56,20 @@ int alloc_lists(dc_cache* c, dc_match_set& m)
     const size_t n = (size_t)c->n_layers, per_layer = (size_t)c->S * c->max_regions;
     DC_TRY(dev_alloc(c, &m.live, n * per_layer));
     DC_TRY(dev_alloc(c, &m.dirty_count, n));
-    DC_TRY(dev_alloc(c, &m.reuse_px, n * c->S * 2));
-    m.alive = m.reuse_px + n * c->S;
-    DC_CUDA(cudaMemsetAsync(m.reuse_px, 0, sizeof(int32_t) * n * c->S * 2, c->stream));
+    DC_TRY(dev_alloc(c, &m.reuse_px, (n * 3 + 1) * c->S));
+    m.alive = m.reuse_px + n * c->S; m.places = m.alive + n * c->S;
+    DC_CUDA(cudaMemsetAsync(m.reuse_px, 0, sizeof(int32_t) * (n * 3 + 1) * c->S, c->stream));
     return DC_OK;
 }
 void free_lists(dc_match_set& m)
 {
     cudaFree(m.live); cudaFree(m.dirty_count); cudaFree(m.reuse_px); cudaFree(m.classify_table);
-    m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = nullptr; m.classify_table = nullptr;
+    m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = m.places = nullptr; m.classify_table = nullptr;
 }
 void share_lists(dc_cache* c)
 {
     dc_match_set& m = c->mset[1]; const dc_match_set& o = c->mset[0];
-    m.live = o.live; m.dirty_count = o.dirty_count; m.reuse_px = o.reuse_px; m.alive = o.alive; m.classify_table = o.classify_table;
+    m.live = o.live; m.dirty_count = o.dirty_count; m.reuse_px = o.reuse_px; m.alive = o.alive; m.places = o.places; m.classify_table = o.classify_table;
 }
 bool own_lists(const dc_cache* c) { return c->mset[1].live != c->mset[0].live; }
 
@@ -86,7 +87,7 @@ int second_lists(dc_cache* c)
     if (!c->executable || matcher_is_large(c)) return DC_OK;
     const size_t before = c->bytes;
     dc_match_set m = c->mset[1];
-    m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = nullptr; m.classify_table = nullptr;
+    m.live = nullptr; m.dirty_count = m.reuse_px = m.alive = m.places = nullptr; m.classify_table = nullptr;
     int rc = alloc_lists(c, m);
     if (rc == DC_OK) rc = dc_build_classify_table(c, m);
     if (rc == DC_OK) { c->mset[1] = m; return DC_OK; }

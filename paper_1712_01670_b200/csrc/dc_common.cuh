@@ -79,7 +79,7 @@ struct dc_layer_rt {
 struct dc_match_set {
     int16_t* blk_mv; uint32_t* blk_sse; uint8_t* matched; uint16_t* run_end; int32_t* mv_acc; uint4* long_list;
     int32_t* gmv; dc_region* regions0; int32_t* n_regions;
-    dc_region* live; int32_t* dirty_count; int32_t* reuse_px; int32_t* alive; void* classify_table;
+    dc_region* live; int32_t* dirty_count; int32_t* reuse_px; int32_t* alive; int32_t* places; void* classify_table;
 };
 
 struct dc_cache {
@@ -135,6 +135,7 @@ struct dc_cache {
     int32_t* all_count;             // [n_layers]
     int32_t* reuse_px;              // [n_layers][S]
     int32_t* alive;                 // [n_layers][S] rectangles not yet eroded away
+    int32_t* places;                // [n_layers + 1][S] region propagation's counters, zero between launches
     uint32_t* zero_masks;           // all-zero reuse bitmap shared by full frames
     int32_t* status;                // device status word
     void* input_map;                // frame / 255 as a map, [S][H][W][3]

@@ -1546,6 +1546,49 @@ def test_lookahead_gives_identical_results():
         dc.close()
 
 
+@pytest.mark.parametrize("S,W,H", [(1, 400, 240), (60, 400, 240), (80, 160, 96)])
+def test_propagate_frames_of_many_rectangles(S, W, H):
+    """A frame's rectangles shared by four CTAs, by two, and by none, in batches that the frame fills and does not: table, counts and reuse, frame
+    after frame, announced and not."""
+    nb = nets.NetBuilder(H, W)
+    x = nb.conv(-1, 16, 3, 1, 1)
+    for k in (1, 1, 3, 1, 1):
+        x = nb.conv(x, 16, k, 1, k // 2)
+    ws, bs = nets.random_weights(nb.layers, 2)
+    g = rng(S)
+    base = g.integers(0, 256, (S, H, W, 3), dtype=np.uint8)
+    frames = []
+    for t in range(5):
+        f = base.copy()
+        for s in range(S):
+            share = (0.0, 0.45, 0.1, 0.02, 0.5)[(t + s) % 5]
+            for y, x0 in np.argwhere(g.random((H // 8, W // 8)) < share):
+                f[s, 8 * y:8 * y + 8, 8 * x0:8 * x0 + 8] = g.integers(0, 256, (8, 8, 3))
+        frames.append(torch.from_numpy(f).cuda())
+    kw = dict(n_streams=S, block=8, search_range=0, dtype=B.DC_BF16, max_regions=W // 8 * (H // 8))
+    dc, ahead = DeepCache(W, H, nb.layers, ws, bs, **kw), DeepCache(W, H, nb.layers, ws, bs, **kw)
+    try:
+        for t, f in enumerate(frames):
+            _, st = dc.infer_frame(f, want_stats=True)
+            _, st2 = ahead.infer_frame(f, want_stats=True)
+            if t + 1 < len(frames):
+                B.dc_lookahead_frame(ahead.handle, frames[t + 1], W * 3)
+            if st[0].refreshed:
+                continue
+            regs0 = dc.layer_regions(-1)[0].cpu()
+            tables = [dc.layer_regions(l)[0].cpu() for l in range(len(nb.layers))]
+            for s in range(S):
+                n = st[s].n_regions
+                assert list(st[s].reuse_ratio[:len(nb.layers)]) == list(st2[s].reuse_ratio[:len(nb.layers)])
+                want = orc.propagate(nb.layers, (H, W), U.regions_np(regs0[s, :n]))
+                for l in range(len(nb.layers)):
+                    U.assert_regions_equal(U.regions_np(tables[l][s, :n]), want[l], f"frame {t} stream {s} layer {l}")
+                    assert abs(st[s].reuse_ratio[l] - float((want[l]["w"] * want[l]["h"]).sum()) / (W * H)) < 1e-6
+        assert max(x.n_regions for x in st) > (256 if W == 400 else 40) and dc.status() == B.DC_OK and ahead.status() == B.DC_OK
+    finally:
+        dc.close(); ahead.close()
+
+
 @pytest.mark.parametrize("recorded", [1, 2])
 def test_first_lookahead_in_a_graph(recorded):
     """The first announced frames of a cache recorded in a capture, where nothing may be allocated, and launched from there; then announced by
