@@ -16,7 +16,7 @@
 //   0      weights: one bulk copy per (32 channels, kernel row), packed as the MMA reads them
 //   1      MMA issue
 //   2-9    the sums: tensor memory -> registers after every kernel row; bias, ReLU, store of the pixels not reused.  A warp has 32 pixels and
-//          half of the channels, or (TURNS: more items than SMs) all of them of every other item: four warps empty the accumulators of one
+//          half of the channels, or (TURNS: several items per CTA) all of them of every other item: four warps empty the accumulators of one
 //          item while the other four finish the one before.
 //   10-15  input: the (16 + kh - 1) x (8 + kw - 1) patch of 32 channels, split into pieces on its way to shared memory (planes of
 //          8 channels, 16 bytes a pixel: every tap is a shifted view of it, as in the patch scheme of the bf16 kernels)
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
     auto k_steps = [&](int cc) { return cc + 1 < a.chunks ? kChF / 16 : a.ks_last; };
     // All of a layer's weights in the ring: they stay there, sent once.  Shared memory's bandwidth is what bounds a kernel row, and a fifth of
     // that went into weights that were there before (32 -> 32 at 227 x 227, 24 streams: 133 us so, 129 resident).
-    const bool resident = a.NB == 1 && a.chunks * KW <= a.stages;
+    const bool resident = TURNS && a.NB == 1 && a.chunks * KW <= a.stages;
 
     if (warp == 0) {
         // ---------------- weights ----------------
@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
         if (a.early) { dc_pdl_wait(); dc_pdl_release(); }
         const uint32_t stage = smem_u32(ctl + 1) + (warp - 2) * f32_stage_bytes(BN, KW);
         const uint32_t t_full = t_full0 + (TURNS ? 16u * group : 0u);
-        uint32_t phases = 0;                                               // bit s: of set s, for this group
+        uint32_t next_set = 0, phases = 0;                                 // phases: TURNS: bit s: of set s, for this group; else of both
         int seq = first;
         for (int item = blockIdx.x + first * gridDim.x; item < n_items; item += every * gridDim.x, seq += every) {
             const int tile = next;
@@ -391,11 +391,11 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
 #pragma unroll
             for (int j = 0; j < CH; ++j) sum[j] = 0.f;
             bool ok = true;
-            uint32_t set = (uint32_t)(seq * drains) & 1u;
+            uint32_t set = TURNS ? (uint32_t)(seq * drains) & 1u : next_set;
             for (int u = 0; u < drains; ++u, set ^= 1u) {
-                ok = f_wait_warp(t_full + 8u * set, (phases >> set) & 1u, lane, ctl, a.status);
+                ok = f_wait_warp(t_full + 8u * set, TURNS ? (phases >> set) & 1u : phases, lane, ctl, a.status);
                 if (!ok) break;
-                phases ^= 1u << set;
+                if (TURNS) phases ^= 1u << set;
                 tc_fence_after();
                 const uint32_t d = tmem_base + lanes + set * kSet + half * CH;
 #pragma unroll
@@ -414,11 +414,15 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl->t_empty[set]);
+                if (!TURNS && set == 1) phases ^= 1u;
             }
+            if (!TURNS) next_set = set;
             if (!ok) break;
             const int s = tile / per_stream, t = tile - s * per_stream, ty = t / a.tiles_x, tx = t - ty * a.tiles_x;
             const int y = ty * DC_TILE_H + row, x = tx * DC_TILE_W + col;
-            const bool active = y < a.Ho && x < a.Wo && !((word >> (8 * (row & 3) + col)) & 1u), odd = ctl->odd[seq % kTileFlags] == seq + 1;
+            const bool active = y < a.Ho && x < a.Wo && !((word >> (8 * (row & 3) + col)) & 1u);
+            auto odd_item = [&] { return ctl->odd[seq % kTileFlags] == seq + 1; };
+            const bool odd_early = TURNS && odd_item();
             const int nb = item % a.NB, grp = nb / a.nb_g;
 #pragma unroll
             for (int h = 0; h < CH; h += HALF) {
@@ -433,7 +437,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
 #pragma unroll
                     for (int j = 0; j < HALF; ++j) small = small || (fabsf(sum[h + j]) < kSmallSum && sum[h + j] != 0.f);
                 }
-                const bool redo = active && (!(most < INFINITY) || small || odd);
+                const bool redo = active && (!(most < INFINITY) || small || (TURNS ? odd_early : odd_item()));
                 // through shared memory, so that lanes side by side store side by side (a lane's own 32-byte pieces of its pixel: each store of a
                 // warp touched 32 lines, and the stores took as long as the MMAs)
                 const uint32_t todo = __ballot_sync(0xffffffffu, active && !redo);
@@ -696,10 +700,13 @@ int dc_launch_conv_f32(dc_cache* c, int layer, const void* in, void* out, const 
     const int grid = items > c->num_sms ? c->num_sms : (int)items;
     dc_prof_scope ps(c, DC_ST_CONV);
     c->launches += 1;
-    // Several items of 32 channels per CTA: TURNS.  With one each its eight warps finish it sooner together; sums of 64 channels are more than a
-    // thread's registers hold beside the rest (32 -> 32 at 227 x 227, 24 streams, 129 us without and 121 with it; 64-channel blocks 85.6 and 88).
-    const bool turns = BN == 32 && items > c->num_sms;
-#define DC_F32(kw) return turns ? launch_f32<32, kw, true>(c, a, grid) : BN == 64 ? launch_f32<64, kw, false>(c, a, grid) : launch_f32<32, kw, false>(c, a, grid)
+    // TURNS for 3 x 3 kernels where a CTA has several items of 32 channels; with few each the eight warps finish one sooner together, 5 x 5 kernels take 5%
+    // longer in turns whatever their number, 1 x 1 kernels up to 5%; sums of 64 channels are more than a thread's registers hold beside the rest.
+    // us without and with it, every tile dirty, by items: 32 -> 32, 250 11.1 and 11.8, 400 14.1 and 14.4, 450 16.3 and 16.2, 1000 26.1 and 24.2;
+    // 16 -> 32, 1000 21.7 and 19.3; 64 -> 32, 1000 41.1 and 39.2; 1 x 1, 32 -> 32, 5220 73 and 77.
+    const bool turns = BN == 32 && L.d.kw == 3 && items > 3ll * c->num_sms;
+#define DC_F32(kw) return BN == 64 ? launch_f32<64, kw, false>(c, a, grid) : launch_f32<32, kw, false>(c, a, grid)
+    if (turns) return launch_f32<32, 3, true>(c, a, grid);
     if (L.d.kw == 1) DC_F32(1);
     if (L.d.kw == 3) DC_F32(3);
     DC_F32(5);

@@ -1990,7 +1990,7 @@ def test_conv_fp32_on_tensor_cores_with_values_that_do_not_split():
         dc.close()
 
 
-@pytest.mark.parametrize("cin,k,S", [(32, 3, 24), (32, 3, 10), (96, 3, 24), (16, 5, 24), (32, 1, 24), (200, 1, 11)])
+@pytest.mark.parametrize("cin,k,S", [(32, 3, 24), (32, 3, 10), (96, 3, 24), (16, 5, 24), (32, 1, 24), (200, 1, 11), (32, 3, 40), (96, 3, 31)])
 def test_conv_fp32_items_in_turns(cin, k, S):
     """Layers with several items per CTA, finished by two groups of warps in turn, with weights that stay in shared memory (one patch of channels)
     and that do not: stream by stream the bits of one stream alone, where every item has an SM, also where pixels are left to FMAs or reused."""
