@@ -825,8 +825,9 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, AHEAD ? 2 : 3) k_search_dsw(Mat
 // two of the scores that matter are equal the exact order (SSE, |dx| + |dy|, dy, dx) picks from the same scores.
 // What bounds it: issue slots - 8 differences, 8 multiply-adds and a warp sum per point and block, and the loads, which the points of a
 // row share where the step is 8 or less.  Measured on 8 full-HD frames, range 16: 140 us with 4 lanes per block and byte-aligned rows (a
-// bank conflict and a realignment per word), 126 with 8 loads per point and two CTAs per SM, 114 so.  AHEAD (up to a tile per SM): the
-// loads of a step travel together; two 640 x 360 streams 9.9 -> 5.8 us.
+// bank conflict and a realignment per word), 126 with 8 loads per point and two CTAs per SM, 114 so.  AHEAD (up to two tiles per SM):
+// the loads of a step travel together; two 640 x 360 streams 9.9 -> 5.8 us, eight of 300 x 200 (1.1 tiles per SM) 8.4 -> 7.7, and 11.6
+// without it and with the points of blocks that the right edge cuts one by one.
 constexpr int TSS_VS = 2;
 struct TssShape { int s0, wr, side, pitch; };
 static TssShape tss_shape(int R)
@@ -841,9 +842,10 @@ static TssShape tss_shape(int R)
 }
 static size_t tss_window_bytes(const TssShape& t) { return (size_t)(16 * TSS_VS + 2 * t.wr) * t.pitch * sizeof(uint32_t); }
 
-// The eight points of a step of compile-time length, row by row (the middle of the centre's row is the best point so far).
-template <int STEP, bool AHEAD, int Y = -1>
-__device__ __forceinline__ void tss_score(uint32_t pc, uint32_t row_bytes, const uint32_t (&cw)[8], bool row_on, int lane, uint32_t& mine)
+// The eight points of a step of compile-time length, row by row (the middle of the centre's row is the best point so far).  CLIP: blocks that
+// the frame's right edge cuts; n_px: how many of the lane's eight pixels lie inside.
+template <int STEP, bool CLIP, bool AHEAD, int Y = -1>
+__device__ __forceinline__ void tss_score(uint32_t pc, uint32_t row_bytes, const uint32_t (&cw)[8], bool row_on, int n_px, int lane, uint32_t& mine)
 {
     if constexpr (Y <= 1) {
         const uint32_t p = pc + (uint32_t)Y * row_bytes;
@@ -853,17 +855,17 @@ __device__ __forceinline__ void tss_score(uint32_t pc, uint32_t row_bytes, const
             RowWords<0, 1ull> middle;
             sides.load(p);
             if constexpr (Y != 0) middle.load(p);
-            if constexpr (AHEAD) tss_score<STEP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, lane, mine);
-            sides.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == G + 2 * m ? v : mine; });
-            if constexpr (Y != 0) middle.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == G + 1 ? v : mine; });
+            if constexpr (AHEAD) tss_score<STEP, CLIP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, n_px, lane, mine);
+            sides.template score<CLIP>(cw, row_on, n_px, [&](int m, uint32_t v) { mine = lane == G + 2 * m ? v : mine; });
+            if constexpr (Y != 0) middle.template score<CLIP>(cw, row_on, n_px, [&](int m, uint32_t v) { mine = lane == G + 1 ? v : mine; });
         } else {
             constexpr unsigned long long DXS = 1ull | (Y != 0 ? 1ull << (STEP / 2) : 0ull) | 1ull << STEP;
             RowWords<-STEP, DXS> row;
             row.load(p);
-            if constexpr (AHEAD) tss_score<STEP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, lane, mine);
-            row.template score<false>(cw, row_on, 8, [&](int m, uint32_t v) { mine = lane == G + 2 * m / STEP ? v : mine; });
+            if constexpr (AHEAD) tss_score<STEP, CLIP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, n_px, lane, mine);
+            row.template score<CLIP>(cw, row_on, n_px, [&](int m, uint32_t v) { mine = lane == G + 2 * m / STEP ? v : mine; });
         }
-        if constexpr (!AHEAD) tss_score<STEP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, lane, mine);
+        if constexpr (!AHEAD) tss_score<STEP, CLIP, AHEAD, Y + 1>(pc, row_bytes, cw, row_on, n_px, lane, mine);
     }
 }
 
@@ -873,7 +875,6 @@ template <bool CLIP, bool AHEAD>
 __device__ __forceinline__ void tss_walk(uint32_t lane_base, int pitch, int s0, const uint32_t (&cw)[8], bool row_on, int n_px,
                                          Within valid, int& at, uint32_t& bs)
 {
-    const unsigned all = 0xffffffffu;
     const int lane = threadIdx.x & 31, point = pair(lane % 3 - 1, lane / 3 - 1);
     {   // the zero vector
         RowWords<0, 1ull> zero;
@@ -886,31 +887,13 @@ __device__ __forceinline__ void tss_walk(uint32_t lane_base, int pitch, int s0, 
     for (int step = s0; step > 0; step >>= 1) {
         const uint32_t row_bytes = (uint32_t)(step * pitch) * 4u;
         uint32_t mine = lane == 4 ? bs : 0xffffffffu;
-        if (!CLIP) {
-            switch (step) {
-            case 1: tss_score<1, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
-            case 2: tss_score<2, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
-            case 4: tss_score<4, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
-            case 8: tss_score<8, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
-            case 16: tss_score<16, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
-            default: tss_score<32, AHEAD>(pc, row_bytes, cw, row_on, lane, mine); break;
-            }
-        } else {
-            constexpr int BATCH = AHEAD ? 4 : 1;                  // blocks that the frame's right edge cuts
-#pragma unroll 1
-            for (int k0 = 0; k0 < 8; k0 += BATCH) {
-                RowWords<0, 1ull> one[BATCH];
-#pragma unroll
-                for (int k = 0; k < BATCH; ++k) {
-                    const int q = k0 + k + (k0 + k >= 4);
-                    one[k].load(pc + (uint32_t)(q / 3 - 1) * row_bytes + (uint32_t)((q % 3 - 1) * step * 4));
-                }
-#pragma unroll
-                for (int k = 0; k < BATCH; ++k) {
-                    const int q = k0 + k + (k0 + k >= 4);
-                    one[k].template score<true>(cw, row_on, n_px, [&](int, uint32_t v) { mine = lane == q ? v : mine; });
-                }
-            }
+        switch (step) {
+        case 1: tss_score<1, CLIP, AHEAD>(pc, row_bytes, cw, row_on, n_px, lane, mine); break;
+        case 2: tss_score<2, CLIP, AHEAD>(pc, row_bytes, cw, row_on, n_px, lane, mine); break;
+        case 4: tss_score<4, CLIP, AHEAD>(pc, row_bytes, cw, row_on, n_px, lane, mine); break;
+        case 8: tss_score<8, CLIP, AHEAD>(pc, row_bytes, cw, row_on, n_px, lane, mine); break;
+        case 16: tss_score<16, CLIP, AHEAD>(pc, row_bytes, cw, row_on, n_px, lane, mine); break;
+        default: tss_score<32, CLIP, AHEAD>(pc, row_bytes, cw, row_on, n_px, lane, mine); break;
         }
         const int d = at + step * point;
         if (!within(d, valid)) mine = 0xffffffffu;
@@ -921,7 +904,7 @@ __device__ __forceinline__ void tss_walk(uint32_t lane_base, int pitch, int s0, 
 }
 
 template <bool AHEAD>
-__global__ void __launch_bounds__(TSS_VS * 8 * 32, AHEAD ? 1 : 3) k_search_tss16(MatchArgs a, TssShape t)
+__global__ void __launch_bounds__(TSS_VS * 8 * 32, AHEAD ? 2 : 3) k_search_tss16(MatchArgs a, TssShape t)
 {
     dc_pdl_wait();
     dc_pdl_release();
@@ -1490,7 +1473,7 @@ int dc_launch_match(dc_cache* c, uint8_t* cur_key, const uint8_t* prev_key, cons
         }
         dc_prof_scope ps(c, DC_ST_SEARCH);
         const dim3 tiles((unsigned)((a.Gx + 7) / 8), (unsigned)((a.Gy + TSS_VS - 1) / TSS_VS), (unsigned)a.S);
-        DC_CUDA(dc_launch_pdl((long long)tiles.x * tiles.y * tiles.z <= c->num_sms ? k_search_tss16<true> : k_search_tss16<false>, tiles, TSS_VS * 8 * 32,
+        DC_CUDA(dc_launch_pdl((long long)tiles.x * tiles.y * tiles.z <= 2 * c->num_sms ? k_search_tss16<true> : k_search_tss16<false>, tiles, TSS_VS * 8 * 32,
                               tss_window_bytes(t), c->stream, a, t));
     } else if (a.B == 16 && a.search == DC_SEARCH_EXHAUSTIVE && a.R <= E_MAXR && a.W >= 16 && a.H >= 16) {
         const int chunks = (2 * a.R + 1 + E_DY - 1) / E_DY;
