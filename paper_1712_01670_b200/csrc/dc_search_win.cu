@@ -545,17 +545,18 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
     // The points around a centre at the end of the range lie up to two pixels beyond it: room for them (not staged), and the pitch of an instance
     // that knows it, where the tile keeps its CTAs per SM.  (1080p, 4 streams, diamond, 16 pixels, range 48: 577 us with tiles shrunk to make that
     // room, 282 with a known pitch whatever it costs, 262 so.)  Large blocks of a short range have no use for it: so many of a round's points
-    // are no candidates that a path of their own is cheaper (32 pixels, range 8: 239 and 209 us; 24 pixels, range 24, 278 and 284).
+    // are no candidates that a path of their own is cheaper (32 pixels, range 8: 239 and 209 us, range 16 335 and 318; 24 pixels, range 24, 278 and
+    // 284; four streams of 640 x 360, two tiles per SM, 32 pixels, range 16, 27.9 and 28.8).
     bool edge = false;
     if (a.search == DC_SEARCH_DIAMOND && !far) {
         const int threads = iters > 8 ? 512 : iters <= 4 && !few ? 1536 : 1024;   // an SM's, by the registers of the instance (launch bounds of k_win_walk)
         auto ctas = [&] { const int by_smem = (int)(228 * 1024 / (smem + 1024 + 64)), by_regs = threads / (warps * 32); return by_smem < by_regs ? by_smem : by_regs; };
-        const int most = ctas();
+        const int most = few && ctas() > 2 ? 2 : ctas();
         a.Rw += 2; a.margin = 2;
         known = a.B <= 16 && ((TX * a.B + 2 * a.R + 3) & ~3) + 4 <= walk_pitch(a.B);
         shape(TX, TY);
         if (known && ctas() < most) { known = false; shape(TX, TY); }
-        edge = iters > 8 && (a.R <= (iters <= 16 ? 6 : 12) || ctas() < most);
+        edge = ctas() < most || (iters > 8 && a.R <= (iters <= 16 ? 6 : few ? 8 : 16));
         if (edge) { a.Rw -= 2; a.margin = 0; shape(TX, TY); }
     }
     if (all) { static dc_once_per_device set; return launch(k_win_all, a, warps * 32, smem, device, set, stream); }
@@ -570,8 +571,7 @@ int dc_launch_search_win(dc_win_args a, int num_sms, int device, cudaStream_t st
         DC_WALK(12) DC_WALK(13) DC_WALK(14) DC_WALK(15) DC_WALK(16)
 #undef DC_WALK
     }
-    if (edge) { if (iters <= 16) DC_WALK_(16, false, 0, false, true) DC_WALK_(32, false, 0, false, true) }
-#define DC_WALK(n) { if (far) DC_WALK_(n, true, 0, false) DC_WALK_(n, false, 0, false) }
+#define DC_WALK(n) { if (far) DC_WALK_(n, true, 0, false) if (edge) DC_WALK_(n, false, 0, false, true) DC_WALK_(n, false, 0, false) }
     switch (iters) {
     case 1: DC_WALK(1)
     case 2: DC_WALK(2)
