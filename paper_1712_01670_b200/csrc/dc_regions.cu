@@ -100,10 +100,10 @@ __device__ Span general_rule(const PropLayer& L, int lane, Span a, Span b)
 // alive, live: how many rectangles are left at each layer and stream, and these alone, in any order (they are disjoint): most of a
 // frame's erode within a few layers, and the reuse step tests every tile against all it is given.
 // FRAME: the rectangles of a frame: lists and counts are wanted, the counters of the reuse step are zeroed; table (every slot at every layer) or
-// NULL.  Where its rectangles are more than a batch, the CTAs ask for their places in the lists in `places` ([n_layers][S], then a ticket per
+// NULL.  SHARED: several CTAs per stream; where a frame's rectangles are more than a batch, they ask for their places in the lists in `places` ([n_layers][S], then a ticket per
 // stream), and the last of them moves the counts to `alive` and leaves zeros behind.  Else a caller's list: out, n_out, or NULL: copies of layers out_begin .. layer_end - 1 and of the counts.
 // walkers: threads that walk (a multiple of 32); dynamic shared memory: 8 * layer_end * walkers bytes.
-template <bool FRAME>
+template <bool FRAME, bool SHARED>
 __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int layer_end, int n_layers, int S, int max_regions, int walkers,
                                                    const dc_region* in, const int32_t* n_in, dc_region* table, dc_region* live, int32_t* alive, int32_t* reuse_px,
                                                    int32_t* dirty_count, int32_t* places, dc_region* out, int out_begin, int32_t* n_out)
@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
     const int rows = !FRAME && out ? max_regions : n;
     const size_t layer_stride = (size_t)S * max_regions;
     const bool out_aligned = (uintptr_t)out % 8 == 0;     // a caller's array may lie at any word
-    const bool shared_lists = FRAME && gridDim.y > 1 && n > per_batch;
-    if (FRAME && blockIdx.y > 0 && (int)blockIdx.y * per_batch >= n) return;
+    const bool shared_lists = SHARED && n > per_batch;
+    if (SHARED && blockIdx.y > 0 && (int)blockIdx.y * per_batch >= n) return;
     for (int first = blockIdx.y * per_batch; first < rows; first += gridDim.y * per_batch) {
         const int i = first + tid / kLanes;
         Span r0 = {0, 0};
@@ -221,13 +221,15 @@ __global__ void __launch_bounds__(1024) k_propagate(const PropLayer* layers, int
         }
     }
     if (shared_lists) {
-        __threadfence();
         __syncthreads();
-        const int sharers = min((n + per_batch - 1) / per_batch, (int)gridDim.y);        // CTAs that have rectangles
-        if (tid == 0) last = atomicAdd(&places[n_layers * S + s], 1) == sharers - 1;
+        if (tid == 0) {
+            const int sharers = min((n + per_batch - 1) / per_batch, (int)gridDim.y);    // CTAs that have rectangles
+            __threadfence();                               // behind the barrier: for what all warps have added
+            last = atomicAdd(&places[n_layers * S + s], 1) == sharers - 1;
+            __threadfence();
+        }
         __syncthreads();
         if (!last) return;
-        __threadfence();
         if (tid < layer_end) { count[tid] = __ldcg(&places[tid * S + s]); places[tid * S + s] = 0; }
         if (tid == 0) places[n_layers * S + s] = 0;
     }
@@ -734,16 +736,17 @@ int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, i
     const size_t smem = 8 * (size_t)layer_end * walkers;
     static dc_once_per_device attr_set;
     if (attr_set.first(c->device)) {
-        DC_CUDA(cudaFuncSetAttribute(k_propagate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
-        DC_CUDA(cudaFuncSetAttribute(k_propagate<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+        DC_CUDA(cudaFuncSetAttribute(k_propagate<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+        DC_CUDA(cudaFuncSetAttribute(k_propagate<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
+        DC_CUDA(cudaFuncSetAttribute(k_propagate<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWalkBytes));
     }
-    // A frame whose slots are more than a batch's gets two or four CTAs per stream, as long as the SMs take them; those without a rectangle return at
+    // A frame whose slots are more than two batches' gets two or four CTAs per stream, as long as the SMs take them; those without a rectangle return at
     // once.  us with a thread per rectangle and no table in shared memory, with one CTA, and so: 19 layers, two full-HD streams, 8-pixel blocks, 9.5,
     // 14.3, 10.5, with their blocks' own vectors 28.5, 50.5, 21.7; 71 layers, one stream of 224 x 224, likewise 22.3, 17.0, 14.5.
     const int batches = dc_div_up(c->max_regions, walkers / kLanes), side = c->num_sms / c->S;
-    const int ctas = !for_frame ? batches : side < 2 || batches < 2 ? 1 : side < 4 || batches < 4 ? 2 : 4;
+    const int ctas = !for_frame ? batches : side < 2 || batches < 3 ? 1 : side < 4 || batches < 4 ? 2 : 4;
     const dim3 grid((unsigned)c->S, (unsigned)ctas);
-    DC_CUDA(dc_launch_pdl(for_frame ? k_propagate<true> : k_propagate<false>, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, walkers, in, n_in,
+    DC_CUDA(dc_launch_pdl(!for_frame ? k_propagate<false, false> : ctas > 1 ? k_propagate<true, true> : k_propagate<true, false>, grid, threads, smem, c->stream, (const PropLayer*)c->prop_table, layer_end, c->n_layers, c->S, c->max_regions, walkers, in, n_in,
                           table, c->live, c->alive, c->reuse_px, c->dirty_count, c->places, out, out_begin, n_out));
     c->launches += 1;
     return DC_OK;
