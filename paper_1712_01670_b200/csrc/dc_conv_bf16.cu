@@ -1869,7 +1869,10 @@ int dc_conv_bf16_autotune(dc_cache* c, int layer, const void* in)
     // wherever it can (1, 2 tap by tap; 3, 4 patch; 5, 6 column slabs; the second of each pair with two tiles per item;
     // 7 column slabs on CTA pairs; 8, 9 tap by tap on flat tiles; 10 tap by tap on clusters)
     const int only = getenv("DC_CONV_SCHEME") ? atoi(getenv("DC_CONV_SCHEME")) : 0;
+    // DC_CONV_BLOCK=<channels> likewise: only candidates with blocks of so many output channels
+    const int only_bn = getenv("DC_CONV_BLOCK") ? atoi(getenv("DC_CONV_BLOCK")) : 0;
     auto trial = [&](const char* what) {
+        if (only_bn > 0 && generic && L.tc_bn != only_bn) return;
         if (only > 0 && generic && (L.tc_cs > 0 ? 10 : L.flat ? L.tc_mt + 7 : L.tc_mt) != only) return;
         int rc = DC_OK;
         for (int rep = 0; rep < kTuneReps + 1 && rc == DC_OK; ++rep) {

@@ -1130,6 +1130,43 @@ def test_conv_on_clusters(hi, wi, cin, cout, k, st, p, S, monkeypatch):
     _one_layer_full_and_partial(hi, wi, cin, cout, k, st, p, S, 10)
 
 
+@pytest.mark.parametrize("what", ["add", "groups", "last block filled up", "strided"])
+def test_conv_narrow_blocks(what, monkeypatch, capfd):
+    """Tap-by-tap layers in blocks of 32 and of 64 output channels: the bits of the widest blocks, full and partial."""
+    nb = nets.NetBuilder(28, 30)
+    x = nb.conv(-1, 256, 3, 1, 1)
+    if what == "add":                                                # taken along by the convolution before it
+        nb.add(nb.conv(nb.conv(x, 64, 1, 1, 0), 256, 1, 1, 0, relu=0), x)
+    elif what == "groups":
+        nb.conv(x, 512, 3, 1, 1, groups=2)
+    elif what == "strided":
+        nb.conv(x, 256, 3, 2, 1)
+    else:
+        nb.conv(x, 248, 3, 1, 1)
+    ws, bs = nets.random_weights(nb.layers, 7)
+    g = rng(3)
+    f0 = g.integers(0, 256, (1, 28, 30, 3), dtype=np.uint8)
+    f1 = f0.copy()
+    f1[:, 9:17, 4:12] ^= 0x5A
+    monkeypatch.setenv("DC_VERBOSE", "1")
+    monkeypatch.setenv("DC_CONV_SCHEME", "1")
+    outs = {}
+    for width in (0, 32, 64):
+        monkeypatch.setenv("DC_CONV_BLOCK", str(width))
+        capfd.readouterr()
+        dc = DeepCache(30, 28, nb.layers, ws, bs, block=4, search_range=2, dtype=B.DC_BF16)
+        try:
+            chosen = [l for l in capfd.readouterr().err.splitlines() if ": chose code 1, " in l]
+            assert width == 0 or any(f" {width} channels per block" in l for l in chosen), chosen
+            outs[width] = [dc.infer_frame(f).clone() for f in (f0, f1)] + [dc.layer_map(l) for l in range(len(nb.layers))]
+            assert dc.status() == B.DC_OK
+        finally:
+            dc.close()
+    for width in (32, 64):
+        for a, b in zip(outs[0], outs[width]):
+            assert torch.equal(a, b), f"{width} channels per block"
+
+
 @pytest.mark.parametrize("scheme", [1, 2, 3, 4, 5, 6])
 @pytest.mark.parametrize("hi,wi,cin,cout,k,st,p,S", [
     (33, 18, 32, 16, 3, 1, 1, 3),        # half of the only block
