@@ -213,6 +213,7 @@ static inline cudaError_t dc_launch_pdl(void (*kernel)(KArgs...), dim3 grid, int
 }
 
 // ---- kernels' host-side launchers (each returns DC_OK or DC_ERR_CUDA) ----
+int dc_launch_clear(int32_t* p, int n, cudaStream_t stream);
 int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst, int32_t* zero);
 // arrays of a caller of dc_match_blocks that the kernels write themselves (NULL: not wanted)
 struct dc_match_out { int16_t* mv; uint32_t* sse; uint8_t* matched; int32_t* gmv; dc_region* regions; int32_t* n_regions; };

@@ -31,9 +31,9 @@ struct MatchArgs {
     int32_t* status;                     // device status word: a walk ended by its step limit records DC_ERR_TIMEOUT
 };
 
+// (SSE, |dx| + |dy|, dy, dx) packed into one integer: tie_key behind the SSE, in 64-bit steps, which the exhaustive search is 2% faster with.
 __device__ __forceinline__ unsigned long long cand_key(uint32_t sse, int dx, int dy)
 {
-    // lexicographic (SSE, |dx|+|dy|, dy, dx) packed into one integer
     return ((unsigned long long)sse << 32) | ((unsigned long long)(abs(dx) + abs(dy)) << 16) |
            ((unsigned long long)(dy + 128) << 8) | (unsigned long long)(dx + 128);
 }
@@ -404,76 +404,6 @@ __global__ void __launch_bounds__(1024) k_merge_large(const MergeArgs a)
 // Fast Steps 2 and 4: 16-pixel blocks, diamond search
 // ---------------------------------------------------------------------------------------------
 
-// NR rows (48 bytes each) of the current block per lane, masked for clipped edge blocks.
-template <int NR>
-struct RowCtx {
-    uint32_t cw[NR][12];
-    int row_bytes;                                                 // bw * 3: bytes of a block row (48 unless clipped)
-    // mask of the valid bytes of word j of a clipped row
-    __device__ __forceinline__ uint32_t word_mask(int j) const
-    {
-        const int nb = row_bytes - 4 * j;
-        return nb >= 4 ? 0xffffffffu : (nb <= 0 ? 0u : ((1u << (8 * nb)) - 1u));
-    }
-    bool clipped, row_on[NR];
-    // cur_rows[k]: address of row k of this lane (16-byte aligned in the library's frame copy)
-    __device__ __forceinline__ void load(const uint8_t* const* cur_rows, int bw, const bool* on)
-    {
-        clipped = bw < 16;
-        row_bytes = bw * 3;
-#pragma unroll
-        for (int k = 0; k < NR; ++k) {
-            row_on[k] = on[k];
-            const uint4* p = (const uint4*)cur_rows[k];
-            uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0, v2 = v0;
-            if (on[k]) { v0 = dc_ld(p); v1 = dc_ld(p + 1); v2 = dc_ld(p + 2); }
-            cw[k][0] = v0.x; cw[k][1] = v0.y; cw[k][2] = v0.z; cw[k][3] = v0.w; cw[k][4] = v1.x; cw[k][5] = v1.y;
-            cw[k][6] = v1.z; cw[k][7] = v1.w; cw[k][8] = v2.x; cw[k][9] = v2.y; cw[k][10] = v2.z; cw[k][11] = v2.w;
-            if (clipped) {
-#pragma unroll
-                for (int j = 0; j < 12; ++j) cw[k][j] &= word_mask(j);
-            }
-        }
-    }
-    // rows r, r + step, ... of the block whose top-left byte is `base`
-    __device__ __forceinline__ void load_block(const uint8_t* base, size_t pitch, int r, int step, int bw, int bh)
-    {
-        const uint8_t* rows[NR]; bool on[NR];
-#pragma unroll
-        for (int k = 0; k < NR; ++k) { rows[k] = base + (size_t)(r + k * step) * pitch; on[k] = r + k * step < bh; }
-        load(rows, bw, on);
-    }
-    // partial SSE of row k against 13 consecutive words at q, the row starting sh bits into q[0]
-    template <bool CLIP = true, typename P>
-    __device__ __forceinline__ uint32_t sse(int k, P q, uint32_t sh) const
-    {
-        uint32_t w[13];
-#pragma unroll
-        for (int j = 0; j < 13; ++j) w[j] = q[j];
-        return sse_words<CLIP>(k, w, sh);
-    }
-    // the same on 13 words already in registers
-    template <bool CLIP = true>
-    __device__ __forceinline__ uint32_t sse_words(int k, const uint32_t (&w)[13], uint32_t sh) const
-    {
-        uint32_t acc[3] = {0, 0, 0};                            // three chains hide the dp4a latency
-        if (!CLIP || !clipped) {
-#pragma unroll
-            for (int j = 0; j < 12; ++j) {
-                uint32_t d = __vabsdiffu4(cw[k][j], __funnelshift_r(w[j], w[j + 1], sh));
-                acc[j % 3] = __dp4a(d, d, acc[j % 3]);
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < 12; ++j) {
-                uint32_t d = __vabsdiffu4(cw[k][j], __funnelshift_r(w[j], w[j + 1], sh) & word_mask(j));
-                acc[j % 3] = __dp4a(d, d, acc[j % 3]);
-            }
-        }
-        return acc[0] + acc[1] + acc[2];
-    }
-};
-
 __device__ __forceinline__ void publish_block(const MatchArgs& a, int s, size_t g, int bw, int bh, unsigned long long bk)
 {
     const int fx = (int)(bk & 0xff) - 128, fy = (int)((bk >> 8) & 0xff) - 128;
@@ -634,6 +564,7 @@ __device__ __forceinline__ Within walk_range(const WalkBounds& b) { return Withi
 struct WalkW {
     int at, kind;               // centre, and how it was reached
     uint32_t bs;                // SSE of the best point so far (the centre, after the first round)
+    int left;                   // moves left; every one strictly lowers the key, so (2 R + 1)^2 are never used up
     int next, nk; uint32_t ns;  // on return 2: the centre the walk has chosen and not yet moved to, the kind of that move, and its SSE
 };
 
@@ -687,7 +618,7 @@ __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base,
     const int lane = threadIdx.x & 31, point = lane_point(lane);
     uint32_t pc = lane_base + bytes_of<PITCH>(w.at - disp(0, 0));
 #pragma unroll 1
-    for (int moves_left = (2 * a.R + 1) * (2 * a.R + 1);; --moves_left) {      // every move strictly lowers the key: never used up
+    for (;; --w.left) {
         uint32_t mine = 0xffffffffu;
         if (!clipped) {
             switch (w.kind) {
@@ -713,12 +644,12 @@ __device__ __forceinline__ int warp_walk(const MatchArgs& a, uint32_t lane_base,
         const int next = __shfl_sync(all, d, g);
         if (w.kind == KIND_SMALL) { w.at = next; w.bs = ns; return 1; }                // the small diamond's best is the result
         if (g == 8) { w.bs = ns; w.kind = KIND_SMALL; continue; }                      // centre won: small diamond, then done
-        if (moves_left <= 0) {                                    // a walk cut here is not valid: say so
+        if (w.left <= 0) {                                        // a walk cut here is not valid: say so
             if (lane == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
             w.bs = ns;
             return 1;
         }
-        if (!within(next, reach)) { w.next = next; w.nk = g; w.ns = ns; return 2; }
+        if (!within(next, reach)) { w.next = next; w.nk = g; w.ns = ns; --w.left; return 2; }
         pc += bytes_of<PITCH>(next - w.at);
         w.kind = g; w.at = next; w.bs = ns;
     }
@@ -792,7 +723,7 @@ __global__ void __launch_bounds__(W_VS * 8 * 32, AHEAD ? 2 : 3) k_search_dsw(Mat
         const WalkBounds wb = walk_bounds(a, x0, y0, bw, bh);
         const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(win) +
                                    (uint32_t)((((warp >> 3) * 16 + r + W_WRY) * W_PITCH + (x0 - xs + W_SIDE) + h) * 4);
-        WalkW w = {disp(0, 0), KIND_FIRST, 0xffffffffu, 0, 0, 0u};
+        WalkW w = {disp(0, 0), KIND_FIRST, 0xffffffffu, (2 * a.R + 1) * (2 * a.R + 1), 0, 0, 0u};
         const Within reach = {disp(2 - W_SIDE, 2 - W_WRY), disp(W_SIDE - 2, W_WRY - 2)};
         const int st = warp_walk<W_PITCH, AHEAD>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, walk_range(wb), w, reach);
         if (lane == 0) {
@@ -1005,25 +936,24 @@ __global__ void __launch_bounds__(P_WARPS * 32, AHEAD ? 2 : 4) k_search_dsw_long
     const bool direct = long_list == nullptr;
     const int sgx = (a.Gx + a.skip_k - 1) / a.skip_k, sgy = (a.Gy + a.skip_k - 1) / a.skip_k;       // searched columns, rows
     const int n = direct ? a.S * sgx * sgy : *long_count;
-    const int max_rounds = (2 * a.R + 1) * (2 * a.R + 1);             // a window is staged for a move, and every move strictly lowers the key
 #pragma unroll 1
     for (;;) {
         int idx = 0;
         if (lane == 0) idx = atomicAdd(cursor, 1);
         idx = __shfl_sync(0xffffffffu, idx, 0);
         if (idx >= n) break;
-        size_t g;
-        WalkW w = {disp(0, 0), KIND_FIRST, 0xffffffffu, 0, 0, 0u};
+        unsigned g;                                               // S * Gx * Gy < 2^31
+        WalkW w = {disp(0, 0), KIND_FIRST, 0xffffffffu, (2 * a.R + 1) * (2 * a.R + 1), 0, 0, 0u};
         if (direct) {
             const int ss = idx / (sgx * sgy), q = idx - ss * sgx * sgy, sby = q / sgx, sbx = q - sby * sgx;
-            g = (size_t)ss * per + (size_t)(sby * a.skip_k) * a.Gx + sbx * a.skip_k;
+            g = (unsigned)(ss * per + sby * a.skip_k * a.Gx + sbx * a.skip_k);
         } else {
             const uint4 e = long_list[idx];
             g = e.x; w.bs = e.z;
             w.at = (int)e.y;                                                                  // the move it had chosen: make it
             w.kind = (int)e.w;
         }
-        const int s = (int)(g / per), b = (int)(g - (size_t)s * per), by = b / a.Gx, bx = b - by * a.Gx;
+        const int s = (int)(g / (unsigned)per), b = (int)g - s * per, by = b / a.Gx, bx = b - by * a.Gx;
         const int x0 = bx * 16, y0 = by * 16, bh = min(16, a.H - y0), bw = min(16, a.W - x0);
         const bool row_on = r < bh;
         uint32_t cw[8];
@@ -1031,7 +961,7 @@ __global__ void __launch_bounds__(P_WARPS * 32, AHEAD ? 2 : 4) k_search_dsw_long
         const uint8_t* prev = a.prev + (size_t)s * a.prev_stream;
         const Within valid = walk_range(walk_bounds(a, x0, y0, bw, bh));
 #pragma unroll 1
-        for (int round = 0;; ++round) {
+        for (;;) {                                                       // ends: every window takes a move, of which warp_walk counts the rest
             // the window for the centre that is scored next
             constexpr int AROUND = P_REACH - 2;
             const int centre = w.at + 2 * lane_point(w.kind);
@@ -1068,10 +998,6 @@ __global__ void __launch_bounds__(P_WARPS * 32, AHEAD ? 2 : 4) k_search_dsw_long
             const uint32_t lane_base = (uint32_t)__cvta_generic_to_shared(win) + (uint32_t)(((r + y0 - wy0) * P_PITCH + (x0 - wx0) + h) * 4);
             const int st = warp_walk<P_PITCH, AHEAD>(a, lane_base, cw, row_on, lane_pixel_count(bw, h), bw < 16, valid, w, reach);
             if (st == 1) break;
-            if (round >= max_rounds) {                                   // never reached; a walk cut here is not valid
-                if (lane == 0) atomicExch(a.status, (int)DC_ERR_TIMEOUT);
-                break;
-            }
             // make the chosen move; the next round scores its new points in a window around the new centre
             w.kind = w.nk;
             w.at = w.next; w.bs = w.ns;
@@ -1092,8 +1018,15 @@ __device__ __forceinline__ uint32_t score16(const MatchArgs& a, int s, int b, in
 {
     const int by = b / a.Gx, bx = b - by * a.Gx, x0 = bx * 16, y0 = by * 16, bw = min(16, a.W - x0), bh = min(16, a.H - y0);
     if (!on || r >= bh) return 0;
-    RowCtx<1> rc;
-    rc.load_block(a.cur + (size_t)s * a.cur_stream + (size_t)y0 * a.cur_pitch + (size_t)x0 * 3, a.cur_pitch, r, 16, bw, bh);
+    const uint4* c16 = (const uint4*)(a.cur + (size_t)s * a.cur_stream + (size_t)(y0 + r) * a.cur_pitch + (size_t)x0 * 3);   // 16-byte aligned
+    const uint4 v0 = dc_ld(c16), v1 = dc_ld(c16 + 1), v2 = dc_ld(c16 + 2);
+    uint32_t cw[12] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w, v2.x, v2.y, v2.z, v2.w};
+    // the bytes of word j inside a block that the frame's right edge cuts
+    auto inside = [&](int j) { const int nb = bw * 3 - 4 * j; return nb >= 4 ? 0xffffffffu : nb <= 0 ? 0u : (1u << (8 * nb)) - 1u; };
+    if (bw < 16) {
+#pragma unroll
+        for (int j = 0; j < 12; ++j) cw[j] &= inside(j);
+    }
     // the 48 bytes of the displaced row lie in four aligned 16-byte chunks (rows of the frame copy are padded):
     // four wide loads instead of thirteen narrow ones, then a word offset that is the same for a whole stream
     const uint8_t* p = a.prev + (size_t)s * a.prev_stream + (size_t)(y0 + My + r) * a.prev_pitch + (size_t)(x0 + Mx) * 3;
@@ -1120,7 +1053,21 @@ __device__ __forceinline__ uint32_t score16(const MatchArgs& a, int s, int b, in
         for (int j = 0; j < 13; ++j) w[j] = ww[j + 3];
         break;
     }
-    return rc.sse_words(0, w, sh);
+    uint32_t acc[3] = {0, 0, 0};                                // three chains hide the dp4a latency
+    if (bw == 16) {
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+            const uint32_t d = __vabsdiffu4(cw[j], __funnelshift_r(w[j], w[j + 1], sh));
+            acc[j % 3] = __dp4a(d, d, acc[j % 3]);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+            const uint32_t d = __vabsdiffu4(cw[j], __funnelshift_r(w[j], w[j + 1], sh) & inside(j));
+            acc[j % 3] = __dp4a(d, d, acc[j % 3]);
+        }
+    }
+    return acc[0] + acc[1] + acc[2];
 }
 
 __global__ void __launch_bounds__(256) k_verify16_prep(MatchArgs a, uint32_t* list, int32_t* list_count)
@@ -1325,7 +1272,8 @@ __global__ void __launch_bounds__(256, 3) k_search_es16(MatchArgs a)
     if (lane == 0) publish_block(a, s, g, 16, 16, bk);            // the zero vector is always valid, so bk is set
 }
 
-// Step 3's sums and the list counters of a search that no frame copy precedes.
+// Step 3's sums and the list counters of a search that no frame copy precedes.  A kernel, not a memset: the search behind it is launched while it
+// runs (the search without a cache, 720p, 85 -> 82 us a call).
 __global__ void k_clear(int32_t* p, int n)
 {
     dc_pdl_wait();
@@ -1399,6 +1347,12 @@ int search_win(dc_cache* c, const MatchArgs& a, int only_clipped)
 }  // namespace
 
 // zero: the Step 3 sums of the match set that the search after this copy will use, or NULL
+int dc_launch_clear(int32_t* p, int n, cudaStream_t stream)
+{
+    DC_CUDA(dc_launch_pdl(k_clear, dim3(1), 256, 0, stream, p, n));
+    return DC_OK;
+}
+
 int dc_launch_copy_frame(dc_cache* c, const uint8_t* frame, size_t pitch, uint8_t* dst, int32_t* zero)
 {
     const int row_bytes = c->cfg.width * 3, rows = c->cfg.height * c->S, chunks = (row_bytes + 15) / 16;
@@ -1434,7 +1388,8 @@ int dc_launch_match(dc_cache* c, uint8_t* cur_key, const uint8_t* prev_key, cons
         a.copy = cur_key;
         a.cur = frame; a.cur_pitch = pitch; a.cur_stream = pitch * (size_t)c->cfg.height;
         dc_prof_scope ps(c, DC_ST_KEY_UPDATE);
-        DC_CUDA(dc_launch_pdl(k_clear, dim3(1), 256, 0, c->stream, c->mv_acc, 4 * c->S + 4));
+        const int rc = dc_launch_clear(c->mv_acc, 4 * c->S + 4, c->stream);
+        if (rc != DC_OK) return rc;
         c->launches += 1;
     }
     a.prev = prev_key; a.prev_pitch = c->key_pitch; a.prev_stream = c->key_pitch * (size_t)c->cfg.height;

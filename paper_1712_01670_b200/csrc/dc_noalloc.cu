@@ -24,14 +24,6 @@ constexpr int kMaxDevices = 64;
 // Step 3 accumulators: per stream sum dx, sum dy, K, unused
 static __device__ __align__(256) int32_t g_noalloc_acc[4 * DC_NOALLOC_MAX_STREAMS];
 
-// Clears the sums that a call uses.  A kernel, not a memset: the search behind it is launched while it runs (85 -> 82 us a call, 720p).
-__global__ void k_clear_noalloc(int32_t* acc, int n)
-{
-    dc_pdl_wait();
-    dc_pdl_release();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc[i] = 0;
-}
-
 // Step 3: mean vector, rounded to nearest with halves away from zero
 __global__ void k_mean_noalloc(const int32_t* acc, int S, int32_t* gmv)
 {
@@ -90,8 +82,9 @@ extern "C" int dc_search_blocks_noalloc(const uint8_t* frame_dev, const uint8_t*
     }
     a.mv = block_mv_dev; a.sse = block_sse_dev; a.acc = g_scratch_ptr[dev]; a.status = nullptr;
     // the array keeps the previous call's sums: clear this call's part first
-    DC_CUDA(dc_launch_pdl(k_clear_noalloc, dim3(1), 64, 0, stream, a.acc, 4 * (int)n_streams));
-    const int rc = dc_launch_search_win(a, g_sms[dev], dev, stream);
+    int rc = dc_launch_clear(a.acc, 4 * (int)n_streams, stream);
+    if (rc != DC_OK) return rc;
+    rc = dc_launch_search_win(a, g_sms[dev], dev, stream);
     if (rc != DC_OK) return rc;
     DC_CUDA(dc_launch_pdl(k_mean_noalloc, dim3((unsigned)dc_div_up(n_streams, 64)), 64, 0, stream, (const int32_t*)a.acc, (int)n_streams, global_mv_dev));
     return DC_OK;
