@@ -74,9 +74,9 @@ void share_lists(dc_cache* c)
 bool own_lists(const dc_cache* c) { return c->mset[1].live != c->mset[0].live; }
 
 // More blocks than the SMs hold warps, ten times over: matching a frame then takes about as long as a trunk's inference.  Measured
-// with the answer always no and always yes (VGG trunk, next frame announced, us a pass): full HD, 2 streams (110 blocks per SM) 248
-// and 308, 8 (441) 588 and 594, 10 (551) 711 both, 12 (662) 818 and 789, 32 (1764) 1891 and 1742; 720p, 16 (389) 808 and 807, 32 (778)
-// 1454 and 1381.
+// with the answer always no and always yes, and frames not announced (VGG trunk, us a pass): full HD, 2 streams (110 blocks per SM) 224, 296
+// and 269, 8 (441) 536, 563, 551, 10 (551) 657, 680, 672, 12 (662) 759, 761, 767, 16 (882) 951, 901, 939, 32 (1764) 1784, 1685, 1743;
+// 720p, 16 (389) 768, 768, 762, 24 (584) 1061, 1085, 1068, 32 (778) 1435, 1407, 1428, 64 (1557) 2767, 2714, 2766.
 bool matcher_is_large(const dc_cache* c) { return (long long)c->S * c->Gx * c->Gy > (long long)c->num_sms * 640; }
 
 // Lists of their own for the second match set, so that an announced frame's rectangles go through the layers beside the inference too.

@@ -20,9 +20,11 @@
 //          item while the other four finish the one before.
 //   10-15  input: the (16 + kh - 1) x (8 + kw - 1) patch of 32 channels, split into pieces on its way to shared memory (planes of
 //          8 channels, 16 bytes a pixel: every tap is a shifted view of it, as in the patch scheme of the bf16 kernels)
-// What bounds it: the tensor pipe (see f32_bn), and beside it the sums' way out: without MMAs 0.8 of the time, without the stores 0.9.
-// Measured, 24 streams, all tiles, us (CUDA cores, here): 32 -> 32 at 227 x 227 451, 203; 32 -> 64 at 113 x 113 246, 80; 64 -> 64 461, 134;
-// 64 -> 128 at 56 x 56 213, 71.  One stream: 29.4, 14.6; 19.8, 8.9; 32.5, 13.1; 17.3, 11.0.
+// What bounds it: no unit by itself.  MMAs run 52% of the clocks, as long as reading their operands takes (64-channel blocks; blocks of 32: 55%, a
+// half longer than their arithmetic); loads and stores of the other warps take the shared-memory pipe for 37 to 56% of the clocks, half of that bank
+// conflicts.  The rest is hand-overs around the kernel rows: without loads, drains and stores 0.78 of the time, without MMAs 0.8.
+// Measured, 24 streams, all tiles, us (CUDA cores, here): 32 -> 32 at 227 x 227 451, 178; 32 -> 64 at 113 x 113 246, 82; 64 -> 64 461, 133;
+// 64 -> 128 at 56 x 56 213, 69.  One stream: 29.0, 14.3; 19.5, 8.8; 32.2, 12.7; 17.0, 10.9.
 //
 // Infinities, NaN and magnitudes that no bf16 holds do not split (inf - inf), nor do most floats below 2^-110, whose last bits lie
 // under the smallest bf16 of 2^-133: whatever leaves a remainder behind its third piece.  The warps that split a tile mark it if it
@@ -268,8 +270,8 @@ __global__ void __launch_bounds__(kThreadsF, 1) k_conv_f32(const __grid_constant
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), a_full0 = smem_u32(&ctl->a_full[0]), a_empty0 = smem_u32(&ctl->a_empty[0]);
     const uint32_t t_full0 = smem_u32(&ctl->t_full[0]), t_empty0 = smem_u32(&ctl->t_empty[0]);
     auto k_steps = [&](int cc) { return cc + 1 < a.chunks ? kChF / 16 : a.ks_last; };
-    // All of a layer's weights in the ring: they stay there, sent once.  Shared memory's bandwidth is what bounds a kernel row, and a fifth of
-    // that went into weights that were there before (32 -> 32 at 227 x 227, 24 streams: 133 us so, 129 resident).
+    // All of a layer's weights in the ring: they stay there, sent once.  A fifth of what moves through shared memory in a kernel row were weights that
+    // were there before (32 -> 32 at 227 x 227, 24 streams, all tiles: 203 us without this and without turns, 205 with turns alone, 178 with both).
     const bool resident = TURNS && a.NB == 1 && a.chunks * KW <= a.stages;
 
     if (warp == 0) {
@@ -594,7 +596,9 @@ __global__ void k_pack_f32_fma(const float* w, int taps, int Cig, int Cog, int c
 }
 
 // The pixels are read from shared memory again for every block of channels: a step of 16 channels measured 240 clocks for 32 output channels and 310
-// for 64.  Wide blocks, then, unless they leave SMs without an item: whichever takes fewer clocks with every tile dirty.
+// for 64 (272 and 364 where a CTA has dozens of items: the same ratio).  Wide blocks, then, unless they leave SMs without an item: whichever takes
+// fewer clocks with every tile dirty.  us in blocks of 32 and 64, 3 x 3: 64 -> 128 at 56 x 56, 1 stream 10.8 and 11.8, 2 15.8 and 12.7, 24 95.7 and 69.0;
+// 64 -> 96 at 113 x 113 (three narrow blocks or two wide ones), 1 stream 20.9 and 19.0, 2 31.1 and 31.8, 4 54.1 and 51.3, 24 291 and 264.
 int f32_bn(const dc_cache* c, const dc_layer_rt& L)
 {
     const int G = L.d.groups > 1 ? L.d.groups : 1, cog = L.d.cout / G;

@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kCopyWarps * 32) k_classify_copy_all(const Cla
 {
     extern __shared__ uint8_t copy_smem[];
     CopyLane cl = copy_lane_setup(copy_smem);
-    // The table was complete when the cache was created: a warp finds its layer and tile while the kernel before still runs (half a dozen
+    // Both match sets' tables were complete when the cache was created (dc_cache_create waits for them): a warp finds its layer and tile while the kernel before still runs (half a dozen
     // loads one behind another; a pass in us before and so: small CNN, one
     // stream, 86.4 and 85.8; every layer kind, 16 streams, 162.2 and 160.6).
     const int w = blockIdx.x * kCopyWarps + (threadIdx.x >> 5);
@@ -742,7 +742,8 @@ int dc_launch_propagate(dc_cache* c, const dc_region* in, const int32_t* n_in, i
     }
     // A frame whose slots are more than two batches' gets two or four CTAs per stream, as long as the SMs take them; those without a rectangle return at
     // once.  us with a thread per rectangle and no table in shared memory, with one CTA, and so: 19 layers, two full-HD streams, 8-pixel blocks, 9.5,
-    // 14.3, 10.5, with their blocks' own vectors 28.5, 50.5, 21.7; 71 layers, one stream of 224 x 224, likewise 22.3, 17.0, 14.5.
+    // 14.3, 10.5, with their blocks' own vectors 28.5, 50.5, 21.7; 71 layers, one stream of 224 x 224, likewise 22.3, 17.0, 14.5.  With 32
+    // full-HD streams (launch to end, 19 layers), where hardly more rectangles than a batch turn up, 14.8, 16.6, 16.9, with own vectors 25.1, 39.3, 22.3.
     const int batches = dc_div_up(c->max_regions, walkers / kLanes), side = c->num_sms / c->S;
     const int ctas = !for_frame ? batches : side < 2 || batches < 3 ? 1 : side < 4 || batches < 4 ? 2 : 4;
     const dim3 grid((unsigned)c->S, (unsigned)ctas);
