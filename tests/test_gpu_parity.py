@@ -2027,7 +2027,7 @@ def test_conv_fp32_on_tensor_cores_with_values_that_do_not_split():
         dc.close()
 
 
-@pytest.mark.parametrize("cin,k,S", [(32, 3, 24), (32, 3, 10), (96, 3, 24), (16, 5, 24), (32, 1, 24), (200, 1, 11), (32, 3, 40), (96, 3, 31)])
+@pytest.mark.parametrize("cin,k,S", [(32, 3, 24), (32, 3, 10), (96, 3, 24), (16, 5, 24), (32, 1, 24), (200, 1, 11)])
 def test_conv_fp32_items_in_turns(cin, k, S):
     """Layers with several items per CTA, finished by two groups of warps in turn, with weights that stay in shared memory (one patch of channels)
     and that do not: stream by stream the bits of one stream alone, where every item has an SM, also where pixels are left to FMAs or reused."""
@@ -2059,6 +2059,12 @@ def test_conv_fp32_items_in_turns(cin, k, S):
     for s in range(S):
         one_full, one_part = run(s, s + 1)
         assert torch.allclose(full[s], one_full[0], rtol=0, atol=0, equal_nan=True) and torch.allclose(part[s], one_part[0], rtol=0, atol=0, equal_nan=True)
+
+
+@pytest.mark.parametrize("cin,S", [(32, 40), (96, 31)])
+def test_conv_fp32_many_items_in_turns(cin, S):
+    """The same of 3 x 3 layers with more than three items per SM, which alone are finished in turns."""
+    test_conv_fp32_items_in_turns(cin, 3, S)
 
 
 @pytest.mark.parametrize("relu", [0, 1])
